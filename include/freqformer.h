@@ -255,8 +255,8 @@ ff_status_t ff_get_tap(const ff_plan_t *plan, int32_t which, const void **dev_pt
  * tensor-core kernel, 2 = generic SIMT transform instead of the tensor-core passes, 4 = the three
  * axes of the tensor-core transform as separate passes (instead of two of them fused in one launch
  * with the intermediate kept in shared memory).  For tests and benchmarks.
- * The tensor-core kernels cover bf16 storage with head_dim 128 or 64, axis lengths 16, 32, 64 or 128
- * and mid block sizes that tile 128 ranks; the pooled low band joins the tensor-core attention launch
+ * The tensor-core kernels cover bf16 storage with head_dim 128 or 64 and mid block sizes that tile
+ * 128 ranks (any axis lengths; two axes share a launch where both are 16, 32, 64 or 128); the pooled low band joins the tensor-core attention launch
  * from 128 pooled tokens on.  Every other configuration runs on the generic fp32 kernels. */
 ff_status_t ff_plan_set_attention_impl(ff_plan_t *plan, int32_t impl);
 

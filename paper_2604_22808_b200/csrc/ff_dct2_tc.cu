@@ -723,15 +723,17 @@ bool ffk_dct2_supported(const FFDims& dm, int* axis2, int* cs) {
 // Matrix image of one axis and direction as the tensor-memory A operand: row j = output position
 // of a tile, cell c = the bf16 pair (A[j][2c], A[j][2c+1]); hi part [128][64], then lo part.
 // w axis: lines follow one another, A = I kron Mat (index = line*n + a); h, t: A = Mat kron I
-// (index = a*kf + line).  `mat` is the host matrix [n][n], out[a] = sum_b mat[a][b] in[b].
+// (index = a*kf + line); rows and columns past the tile's kf*n positions are zero.  `mat` is the host matrix
+// [n][n], out[a] = sum_b mat[a][b] in[b].
 bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat, int n) {
   const size_t per = (size_t)2 * ROWS * IMG_CELLS;      // cells of one image (hi + lo)
   if (!p->dct2_images && cudaMalloc((void**)&p->dct2_images, 6 * per * sizeof(uint32_t)) != cudaSuccess) return false;
-  const int kf = ROWS / n;
+  const FFPassShape g = ff_pass_shape(p->dm, axis);
+  const int kf = g.kf;
   const bool seq = axis == 2;
   std::vector<uint32_t> img(per);
-  for (int j = 0; j < ROWS; ++j)
-    for (int r = 0; r < ROWS; ++r) {
+  for (int j = 0; j < g.rows; ++j)
+    for (int r = 0; r < g.rows; ++r) {
       float v;
       if (seq) v = (j / n == r / n) ? mat[(j % n) * n + (r % n)] : 0.f;
       else v = (j % kf == r % kf) ? mat[(j / kf) * n + (r / kf)] : 0.f;

@@ -28,6 +28,12 @@
 // pass 0.38 -> 0.42 ms with byte-form input.  So the band-split pass always reads a bf16 pair (the second
 // forward pass writes one), and the fused two-axis launches keep bf16 pairs on both sides.
 //
+// Ragged grids.  A line of any length up to 128 fits a tile, so the passes run on every grid: floor(128 / n) lines
+// per tile, the left-over rows zero in the matrix and in shared memory, partial last tiles filled with zeros and
+// clipped by the copies (template parameter RAG).  21 x 45 x 80 tokens, 16 heads: forward transform 11.1 -> 1.63 ms
+// and inverse 5.8 -> 0.78 ms against the fp32 kernels these grids ran on before (the same 6.5 TB/s-bound traffic
+// per token as a power-of-two grid plus 6 - 37% of unused tile rows).
+//
 // Order of the tiles.  A pass that reads what the previous launch wrote walks its tiles from the last to the
 // first (P.reverse), the next one forward again: the end of the previous launch's output is still in L2.
 //
@@ -83,7 +89,9 @@ enum { MODE_FIRST = 0, MODE_MIDDLE = 1, MODE_SPLIT = 2, MODE_LAST = 3 };
 struct DctTcParams {
   FFDims dm;
   const uint32_t* image;   // matrix image as the tensor-memory A operand: hi [128][64] cells, then lo
-  int n;                   // axis length
+  FFPassShape g;           // lines and tiles of the pass
+  FFFastDiv by_tiles, by_inner;   // tiles of a tensor-head; tiles along the inner extent
+  FFFastDiv by_line;       // (SPLIT) unravels a line index: by W for the t axis, by H for the w axis
   int axis;                // 0 = t, 1 = h, 2 = w
   int mode;
   int group;               // tensor-heads in this launch
@@ -102,6 +110,7 @@ constexpr int STG_PITCH = 64;                       // bytes per staged row piec
 
 struct DctShared {
   uint64_t full[MAX_STAGE], empty[MAX_STAGE], acc_full[NACC], acc_empty[NACC], conv[MAX_STAGE];
+  uint64_t stg_full[2], stg_free[2];       // (ragged tiles) staging area of four epilogue warps: written / read by its store
   uint32_t tmem_base;
   int abort_flag;
   // per epilogue warp: 32 rows x 64 bytes of hi and of lo, to turn one-row-per-thread registers
@@ -109,14 +118,10 @@ struct DctShared {
   alignas(1024) uint8_t stage[8][2][32 * STG_PITCH];
 };
 
-// Grid coordinates (w, h, t) of the first position of tile `u` of a tensor-head.  A tile holds
-// kf = 128/n lines: kf consecutive h for the w axis, kf consecutive w for the h and t axes.
-// (all lengths are powers of two here: lq = log2 of the tiles per row of tiles, H / kf or W / kf)
-__device__ __forceinline__ void tile_origin(int axis, int lkf, int lq, int u, int& w, int& h, int& t) {
-  const int lo = (u & ((1 << lq) - 1)) << lkf, hi = u >> lq;
-  if (axis == 2) { w = 0; h = lo; t = hi; }
-  else if (axis == 1) { h = 0; w = lo; t = hi; }
-  else { t = 0; w = lo; h = hi; }
+// First line of tile `u` of a tensor-head: index along the inner extent and along the outer one.
+__device__ __forceinline__ void tile_origin(const DctTcParams& P, unsigned u, int& i0, int& o0) {
+  if (P.g.seq) { i0 = 0; o0 = (int)u * P.g.kf; }
+  else { const unsigned o = ff_div(u, P.by_inner); o0 = (int)o; i0 = (int)(u - o * (unsigned)P.g.tiles_inner) * P.g.kf; }
 }
 
 __device__ __forceinline__ void tma_load_5d(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2,
@@ -140,7 +145,11 @@ __device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_
 // Three source maps (Q, K, V) in MODE_FIRST; otherwise map0 (= hi) and, for split input, map1 (= lo).
 // map_oh / map_ol: destination hi / lo grids with the box of one epilogue warp (32 positions x 32
 // channels), all modes but SPLIT; MODE_LAST has no lo grid.
-template <int CH, bool LO8>
+// RAG: tiles of kf * n < 128 rows, or a last tile that is not full.  The rows past kf * n are zero in shared memory
+// (cleared once, no copy writes them) and zero in the matrix; lines past the end of the grid arrive as zeros and
+// are clipped by the stores.  32 rows are then no box of the grid, so the four warps of a channel half stage a
+// whole tile (32 channels) and one thread stores it.
+template <int CH, bool LO8, bool RAG>
 __global__ void __launch_bounds__(LO8 ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS, 1)
 dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
               const __grid_constant__ CUtensorMap map2, const __grid_constant__ CUtensorMap map_oh,
@@ -148,31 +157,33 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const FFDims& dm = P.dm;
-  const int n = P.n;
-  const int kf = TILE_ROWS / n;                           // lines per tile
-  const int lkf = 31 - __clz(kf);
-  const int ln = 31 - __clz(n);
-  const bool seq = P.axis == 2;                           // lines follow one another (w axis) or interleave
+  const int n = P.g.n, kf = P.g.kf;                       // axis length, lines per tile
+  const bool seq = P.g.seq;                               // lines follow one another (w axis) or interleave
+  const int rows = RAG ? P.g.rows : TILE_ROWS;
   const int NSTAGE = P.nstage;
-  const bool tma_out = P.mode != MODE_SPLIT;
+  const bool split = !LO8 && P.mode == MODE_SPLIT;        // (the band-split pass never reads the byte form)
+  const bool tma_out = !split;
   constexpr int TB = TILE_ROWS * CH * 2;                  // bytes of one data tile (16 KB for 64 channels)
   constexpr int LO8_OFF = CH == 128 ? TB : 2 * TB;         // where a stage takes the lo bytes
   const int STAGE_BYTES = LO8 ? LO8_OFF + TB / 2 + (CH == 128 ? TB / 2 : 0) : (P.in_split ? 2 * TB : TB);   // hi tile, lo tile
   uint8_t* sData = smem;                                  // NSTAGE x STAGE_BYTES
   DctShared& sh = *(DctShared*)(smem + NSTAGE * STAGE_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tiles_per_th = (int)(dm.N / TILE_ROWS);
-  const int ltpt = 31 - __clz(tiles_per_th);              // (a power of two)
-  const int lq = 31 - __clz((P.axis == 2 ? dm.H : dm.W) >> lkf);
-  const int total_tiles = P.group * tiles_per_th;
+  const unsigned tiles_per_th = (unsigned)P.g.tiles;
+  const int total_tiles = P.group * P.g.tiles;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NSTAGE; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 1); mbar_init(&sh.conv[i], 128); }
     for (int i = 0; i < NACC; ++i) { mbar_init(&sh.acc_full[i], 1); mbar_init(&sh.acc_empty[i], 256); }
+    if (RAG) for (int i = 0; i < 2; ++i) { mbar_init(&sh.stg_full[i], 128); mbar_init(&sh.stg_free[i], 1); }
     sh.abort_flag = 0;
     fence_mbar_init();
   }
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
+  if (RAG) {                                              // rows that no copy writes must not hold NaN patterns
+    for (int i = threadIdx.x * 16; i < NSTAGE * STAGE_BYTES; i += blockDim.x * 16) *(uint4*)(sData + i) = make_uint4(0, 0, 0, 0);
+    fence_proxy_async();
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -217,8 +228,8 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
         PROF_ADD(6, pt);
         if (!ok) break;
         uint8_t* dst = sData + slot * STAGE_BYTES;
-        const int gi = s >> ltpt, u = s & (tiles_per_th - 1);
-        int w, h, t; tile_origin(P.axis, lkf, lq, u, w, h, t);
+        const int gi = (int)ff_div((unsigned)s, P.by_tiles);
+        int i0, o0; tile_origin(P, (unsigned)s - (unsigned)gi * tiles_per_th, i0, o0);
         const CUtensorMap* map = &map0;
         int slice = gi;
         if (P.mode == MODE_FIRST) {
@@ -227,14 +238,14 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
           map = tensor == 0 ? &map0 : (tensor == 1 ? &map1 : &map2);
           slice = th - tensor * dm.BH;
         }
-        mbar_arrive_expect_tx(&sh.full[slot], LO8 ? TB + TB / 2 : STAGE_BYTES);
-        tma_load_5d(dst, map, &sh.full[slot], 0, w, h, t, slice);
-        if (CH == 128) tma_load_5d(dst + HALF_BYTES, map, &sh.full[slot], 64, w, h, t, slice);
+        mbar_arrive_expect_tx(&sh.full[slot], (uint32_t)(rows * CH) * (LO8 ? 3u : (P.in_split ? 4u : 2u)));
+        tma_load_5d(dst, map, &sh.full[slot], 0, i0, 0, o0, slice);
+        if (CH == 128) tma_load_5d(dst + HALF_BYTES, map, &sh.full[slot], 64, i0, 0, o0, slice);
         if (LO8) {
-          tma_load_5d(dst + LO8_OFF, &map1, &sh.full[slot], 0, w, h, t, slice);     // the lo bytes: rows of CH bytes
+          tma_load_5d(dst + LO8_OFF, &map1, &sh.full[slot], 0, i0, 0, o0, slice);     // the lo bytes: rows of CH bytes
         } else if (P.in_split) {
-          tma_load_5d(dst + TB, &map1, &sh.full[slot], 0, w, h, t, slice);
-          if (CH == 128) tma_load_5d(dst + TB + HALF_BYTES, &map1, &sh.full[slot], 64, w, h, t, slice);
+          tma_load_5d(dst + TB, &map1, &sh.full[slot], 0, i0, 0, o0, slice);
+          if (CH == 128) tma_load_5d(dst + TB + HALF_BYTES, &map1, &sh.full[slot], 64, i0, 0, o0, slice);
         }
       }
     }
@@ -256,8 +267,10 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
         const uint32_t dbase = smem_u32(sData + slot * STAGE_BYTES);
         const uint32_t d_tm = tm + COL_ACC + ab * 128;
         const uint64_t xh0 = smem_desc_sw128(dbase, HALF_BYTES, 1024), xl0 = smem_desc_sw128(dbase + TB, HALF_BYTES, 1024);
+        const int ksteps = (rows + 15) >> 4;               // (the rows behind them are zero)
 #pragma unroll
         for (int ks = 0; ks < TILE_ROWS / 16; ++ks) {
+          if (RAG && ks >= ksteps) break;
           // (a descriptor advances by 2048 bytes = 128 in its address field per 16 rows of K)
           umma_ts(d_tm, tm + COL_IMG_HI + ks * 8, xh0 + (uint64_t)(ks * 128), idesc, ks > 0 ? 1u : 0u);
           umma_ts(d_tm, tm + COL_IMG_LO + ks * 8, xh0 + (uint64_t)(ks * 128), idesc, 1u);
@@ -321,17 +334,17 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
   } else {
     const int quarter = warp & 3;
     const int j = quarter * 32 + lane;                    // output position of this thread inside a tile
-    const int a = seq ? j & (n - 1) : j >> lkf;           // output index along the axis
-    const int l = seq ? j >> ln : j & (kf - 1);           // line of the tile
+    const int a = seq ? j % n : j / kf;                   // output index along the axis
+    const int l = seq ? j / n : j % kf;                   // line of the tile
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const int ew = warp - 2;                              // epilogue warp 0..7: warps 0-3 take channels 0..63, 4-7 channels 64..127
     constexpr int NQ = CH / 64;                           // 32-channel chunks per thread
     const int q_lo = (ew >> 2) * NQ;
-    // Grid offset of the warp's first row (tile row 32 quarter) from the tile origin: the warp's 32
-    // rows are the box [32 channels] x [these offsets .. + the extents the store map was built with]
+    // Position along the axis and line of the warp's first row (tile row 32 quarter): the warp's 32
+    // rows are the box [32 channels] x [from there .. + the extents the store map was built with]
     const int j0 = quarter * 32;
-    const int a0 = seq ? j0 & (n - 1) : j0 >> lkf, l0 = seq ? j0 >> ln : j0 & (kf - 1);
-    const int dw = P.axis == 2 ? a0 : l0, dh = P.axis == 2 ? l0 : (P.axis == 1 ? a0 : 0), dt = P.axis == 0 ? a0 : 0;
+    const int a0 = seq ? j0 % n : j0 / kf, l0 = seq ? j0 / n : j0 % kf;
+    unsigned nchunk = 0;                                  // (RAG) chunks this channel half has staged
     const int Lhw = dm.L[1] * dm.L[2], Mhw = dm.M[1] * dm.M[2];
     // (SPLIT) lane k of a warp accumulates the energies of channels 32 q + 2 (k % 16) + {0, 1} over the
     // warp's rows of parity k / 16: ea = mid + high rows, em = mid rows
@@ -340,7 +353,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     unsigned it = 0;
     bool ok = true;
     auto flush_energy = [&]() {
-      if (e_sample >= 0 && P.energy) {
+      if (!LO8 && e_sample >= 0 && P.energy) {
 #pragma unroll
         for (int qi = 0; qi < NQ; ++qi)
 #pragma unroll
@@ -361,30 +374,42 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       if (!ok) break;
       tc_fence_after();
       PROF_T0(pe1);
-      const int gi = s >> ltpt, u = s & (tiles_per_th - 1);
-      int w, h, t; tile_origin(P.axis, lkf, lq, u, w, h, t);
+      const int gi = (int)ff_div((unsigned)s, P.by_tiles);
+      int i0, o0; tile_origin(P, (unsigned)s - (unsigned)gi * tiles_per_th, i0, o0);
       const int th = P.group_start + gi;
       const int tensor = (th >= dm.BH) + (th >= 2 * dm.BH), bh = th - tensor * dm.BH;
       // where this thread's row goes
       __nv_bfloat16* row_hi = nullptr; float* row_f32 = nullptr;
       int band = -1;
-      if (P.mode == MODE_SPLIT) {
+      if (split) {
         if (th != sample_th) { sample_th = th; sample_of_th = bh / dm.heads; }
         const int sample = sample_of_th;
         if (sample != e_sample) { flush_energy(); e_sample = sample; }
-        // Band and rank of this row's coefficient: the pass axis supplies index a, the tile origin the
-        // other two (lines of a tile are neighbours along w for the t and h passes, along h for the w
-        // pass).  The counts of box members below a coefficient are piecewise linear in the coordinates.
-        const int kt = P.axis == 0 ? a : t;
-        const int h_ = P.axis == 1 ? a : (P.axis == 2 ? h + l : h);
-        const int ww = P.axis == 2 ? a : w + l;
+        // Band and rank of this row's coefficient: the pass axis supplies index a, the line the other two.
+        // The counts of box members below a coefficient are piecewise linear in the coordinates.
+        int kt = a, h_ = a, ww = a;
+        bool inside = true;
+        if (P.axis == 0) {
+          const unsigned line = (unsigned)(i0 + l);
+          h_ = (int)ff_div(line, P.by_line); ww = (int)(line - (unsigned)h_ * P.by_line.d);
+          if (RAG) inside = j < rows && (int)line < P.g.inner;
+        } else if (P.axis == 1) {
+          kt = o0; ww = i0 + l;
+          if (RAG) inside = j < rows && ww < dm.W;
+        } else {
+          const unsigned line = (unsigned)(o0 + l);
+          kt = (int)ff_div(line, P.by_line); h_ = (int)(line - (unsigned)kt * P.by_line.d);
+          if (RAG) inside = j < rows && (int)line < P.g.outer;
+        }
         const bool hw_low = h_ < dm.L[1] && ww < dm.L[2], hw_mid = h_ < dm.M[1] && ww < dm.M[2];
         const int offM = (h_ < dm.M[1] ? h_ : dm.M[1]) * dm.M[2] + (h_ < dm.M[1] ? (ww < dm.M[2] ? ww : dm.M[2]) : 0);
         // (axis lengths are at most 128, so every count fits 32 bits)
         const int cm = kt < dm.M[0] ? kt * Mhw + offM : dm.M[0] * Mhw;
         const size_t th_slice = (size_t)tensor * dm.BH + bh;
-        long long rk, nband;                                                         // band-local rank, band length
-        if (kt < dm.L[0] && hw_low) {
+        long long rk = 0, nband = 1;                                                 // band-local rank, band length
+        if (RAG && !inside) {
+          kt = h_ = ww = 0;                                                          // no position of the grid: not stored
+        } else if (kt < dm.L[0] && hw_low) {
           band = 0;                                                                  // low band: fp32
           rk = (kt * dm.L[1] + h_) * dm.L[2] + ww; nband = dm.Nlow;
           row_f32 = P.spec_low + (th_slice * dm.Nlow + (unsigned)rk) * CH;
@@ -407,6 +432,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       }
       // (SPLIT) lane L stores for rows 8 i + L/4 of its warp: fetch those rows' destinations
       __nv_bfloat16* dst_hi[4];
+      if (split)
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int src = 8 * i + (lane >> 2);
@@ -427,7 +453,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       for (int qi = 0; qi < NQ; ++qi) {
         const int q = q_lo + qi;
         uint32_t (&r)[32] = rr2[qi];
-        if (row_f32) {
+        if (!LO8 && row_f32) {
 #pragma unroll
           for (int i = 0; i < 8; ++i)
             *(uint4*)(row_f32 + q * 32 + i * 4) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
@@ -460,9 +486,17 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
               lo[i] = *(const uint32_t*)&lp;
             }
           }
-          uint8_t* st_hi = sh.stage[ew][0];
-          uint8_t* st_lo = sh.stage[ew][1];
-          if (tma_out) {
+          const bool tile_out = RAG && tma_out;          // four warps stage one tile: 128 rows of hi, then of lo
+          const int grp = ew >> 2;
+          uint8_t* st_hi = tile_out ? sh.stage[grp * 4][0] + quarter * 32 * STG_PITCH : sh.stage[ew][0];
+          uint8_t* st_lo = tile_out ? sh.stage[grp * 4][0] + TILE_ROWS * STG_PITCH + quarter * 32 * (lo8 ? 32 : STG_PITCH) : sh.stage[ew][1];
+          if (tile_out) {
+            if (nchunk > 0) {
+              if (quarter == 0 && lane == 0) { bulk_wait_read0(); mbar_arrive(&sh.stg_free[grp]); }
+              ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_free[grp], (nchunk - 1) & 1, abort_flag));
+              if (!ok) break;
+            }
+          } else if (tma_out) {
             // the previous store of this warp must have read the staging area
             PROF_T0(pw);
             if (lane == 0) bulk_wait_read0();
@@ -480,17 +514,31 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
             *(uint4*)(st_lo + lane * 32) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             *(uint4*)(st_lo + lane * 32 + 16) = make_uint4(lo[4], lo[5], lo[6], lo[7]);
           }
-          if (tma_out) {
+          if (tile_out) {
+            fence_proxy_async();
+            mbar_arrive(&sh.stg_full[grp]);
+            if (quarter == 0) {
+              ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_full[grp], nchunk & 1, abort_flag));
+              if (!ok) break;
+              if (lane == 0) {
+                tma_store_5d(st_hi, &map_oh, q * 32, i0, 0, o0, out_slice);
+                if (want_lo) tma_store_5d(st_lo, &map_ol, q * 32, i0, 0, o0, out_slice);
+                bulk_commit();
+              }
+              __syncwarp();
+            }
+            ++nchunk;
+          } else if (tma_out) {
             PROF_T0(pf);
             fence_proxy_async();
             __syncwarp();
             if (threadIdx.x == 64) PROF_ADD(10, pf);
             if (lane == 0) {
-              tma_store_5d(st_hi, &map_oh, q * 32, w + dw, h + dh, t + dt, out_slice);
-              if (want_lo) tma_store_5d(st_lo, &map_ol, q * 32, w + dw, h + dh, t + dt, out_slice);
+              tma_store_5d(st_hi, &map_oh, q * 32, i0 + (seq ? 0 : l0), a0, o0 + (seq ? l0 : 0), out_slice);
+              if (want_lo) tma_store_5d(st_lo, &map_ol, q * 32, i0 + (seq ? 0 : l0), a0, o0 + (seq ? l0 : 0), out_slice);
               bulk_commit();
             }
-          } else {
+          } else if (!LO8) {
             __syncwarp();
             if (P.energy) {
               // Router statistics: channel energies of the staged (bf16) coefficients, summed down the
@@ -530,7 +578,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       }
       if (threadIdx.x == 64) PROF_ADD(5, pe1);
     }
-    if (P.mode == MODE_SPLIT) flush_energy();
+    if (split) flush_energy();
     if (tma_out && lane == 0) bulk_wait0();
   }
 
@@ -569,60 +617,46 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// 5-D map over a [slices][T][H][W][128] bf16 grid whose box is one tile of 128 positions for a pass
-// along `axis`: 128/n whole lines that are neighbours in memory.
-// `bytes`: the grid holds one byte per value (the lo part of the three-byte form); the box then spans all
-// channels of a row at once.
-bool encode_grid_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, bool bytes = false) {
+EncodeTiledFn encoder() {
   static EncodeTiledFn enc = nullptr;
   if (!enc) {
     cudaDriverEntryPointQueryResult qr;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", (void**)&enc, cudaEnableDefault, &qr) != cudaSuccess || !enc)
-      return false;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", (void**)&enc, cudaEnableDefault, &qr) != cudaSuccess) enc = nullptr;
   }
-  const cuuint64_t CH = (cuuint64_t)dm.d, eb = bytes ? 1 : 2;
-  cuuint64_t dims[5] = {CH, (cuuint64_t)dm.W, (cuuint64_t)dm.H, (cuuint64_t)dm.T, (cuuint64_t)slices};
-  cuuint64_t strides[4] = {CH * eb, (cuuint64_t)dm.W * CH * eb, (cuuint64_t)dm.H * dm.W * CH * eb,
-                           (cuuint64_t)dm.N * CH * eb};
-  const int n = axis == 2 ? dm.W : (axis == 1 ? dm.H : dm.T);
-  const int kf = TILE_ROWS / n;
-  cuuint32_t box[5] = {bytes ? (cuuint32_t)dm.d : 64u, 1, 1, 1, 1};
-  box[1 + (2 - axis)] = (cuuint32_t)n;
-  if (axis == 2) box[2] = (cuuint32_t)kf; else box[1] = (cuuint32_t)kf;
-  cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  return enc(map, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims,
-             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             bytes && dm.d == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return enc;
 }
 
-// Store map over the same kind of grid: the box is what one epilogue warp holds, 32 channels of the
-// 32 positions of a quarter tile (tile rows 32 q .. 32 q + 31 of a pass along `axis`), 64-byte swizzle.
-bool encode_store_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, bool bytes = false) {
-  static EncodeTiledFn enc = nullptr;
-  if (!enc) {
-    cudaDriverEntryPointQueryResult qr;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", (void**)&enc, cudaEnableDefault, &qr) != cudaSuccess || !enc)
-      return false;
-  }
+// 5-D map over a grid [slices][outer][n][inner][d] seen along `axis`.  Load map: the box is one tile, 64 channels of
+// kf whole lines.  Store map: 32 channels of what one epilogue warp holds (tile rows 32 q .. 32 q + 31), or of a
+// whole tile where the pass is ragged; 64-byte swizzle.  `bytes`: the grid holds one byte per value (the lo part
+// of the three-byte form); a load box then spans all channels of a row at once.
+bool encode_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, bool bytes, bool store) {
+  EncodeTiledFn enc = encoder();
+  if (!enc) return false;
+  const FFPassShape g = ff_pass_shape(dm, axis);
   const cuuint64_t CH = (cuuint64_t)dm.d, eb = bytes ? 1 : 2;
-  cuuint64_t dims[5] = {CH, (cuuint64_t)dm.W, (cuuint64_t)dm.H, (cuuint64_t)dm.T, (cuuint64_t)slices};
-  cuuint64_t strides[4] = {CH * eb, (cuuint64_t)dm.W * CH * eb, (cuuint64_t)dm.H * dm.W * CH * eb,
-                           (cuuint64_t)dm.N * CH * eb};
-  const int n = axis == 2 ? dm.W : (axis == 1 ? dm.H : dm.T);
-  const int kf = TILE_ROWS / n;
-  cuuint32_t box[5] = {32, 1, 1, 1, 1};
-  if (axis == 2) {                       // rows = line * n + a: 32 consecutive rows
-    box[1] = (cuuint32_t)(n < 32 ? n : 32);
-    box[2] = (cuuint32_t)(n < 32 ? 32 / n : 1);
-  } else {                               // rows = a * kf + line: 32 consecutive rows
-    box[1] = (cuuint32_t)(kf < 32 ? kf : 32);
-    box[1 + (2 - axis)] = (cuuint32_t)(kf < 32 ? 32 / kf : 1);
+  const cuuint64_t line = (cuuint64_t)g.inner * CH * eb;
+  cuuint64_t dims[5] = {CH, (cuuint64_t)g.inner, (cuuint64_t)g.n, (cuuint64_t)g.outer, (cuuint64_t)slices};
+  cuuint64_t strides[4] = {CH * eb, line, line * g.n, (cuuint64_t)dm.N * CH * eb};
+  cuuint32_t box[5] = {store ? 32u : (bytes ? (cuuint32_t)dm.d : 64u), (cuuint32_t)(g.seq ? 1 : g.kf), (cuuint32_t)g.n,
+                       (cuuint32_t)(g.seq ? g.kf : 1), 1};
+  if (store && !g.ragged) {                // 32 consecutive tile rows
+    if (g.seq) { box[2] = (cuuint32_t)(g.n < 32 ? g.n : 32); box[3] = (cuuint32_t)(g.n < 32 ? 32 / g.n : 1); }
+    else { box[1] = (cuuint32_t)(g.kf < 32 ? g.kf : 32); box[2] = (cuuint32_t)(g.kf < 32 ? 32 / g.kf : 1); }
   }
   cuuint32_t es[5] = {1, 1, 1, 1, 1};
+  const CUtensorMapSwizzle swz = store ? (bytes ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_64B)
+                                       : (bytes && dm.d == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
   return enc(map, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims,
-             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, bytes ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_64B,
-             CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
+             store ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+bool encode_grid_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, bool bytes = false) {
+  return encode_map(map, base, dm, slices, axis, bytes, false);
+}
+bool encode_store_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, bool bytes = false) {
+  return encode_map(map, base, dm, slices, axis, bytes, true);
 }
 
 // `in_lo8`: the input pair's lo grid is the byte form (m1 = its byte map).
@@ -636,16 +670,21 @@ cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1
   P.nstage = nstage;
   const size_t smem = nstage * stage + fixed;
   cudaError_t e = cudaSuccess;
-  const int stages = (int)(P.group * (P.dm.N / TILE_ROWS));
-  const int grid = stages < p->sm_count ? stages : p->sm_count;
-#define FF_DCT(D, L)                                                                                              \
-  do {                                                                                                            \
-    e = cudaFuncSetAttribute(dct_tc_kernel<D, L>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
-    if (e == cudaSuccess)                                                                                         \
-      dct_tc_kernel<D, L><<<grid, L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS, smem, st>>>(m0, m1, m2, moh, mol, P);  \
+  P.g = ff_pass_shape(P.dm, P.axis);
+  P.by_tiles = ff_fast_div((unsigned)P.g.tiles); P.by_inner = ff_fast_div((unsigned)P.g.tiles_inner);
+  P.by_line = ff_fast_div((unsigned)(P.axis == 2 ? P.dm.H : P.dm.W));
+  const int tiles = P.group * P.g.tiles;
+  const int grid = tiles < p->sm_count ? tiles : p->sm_count;
+#define FF_DCT(D, L, R)                                                                                              \
+  do {                                                                                                               \
+    e = cudaFuncSetAttribute(dct_tc_kernel<D, L, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
+    if (e == cudaSuccess)                                                                                            \
+      dct_tc_kernel<D, L, R><<<grid, L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS, smem, st>>>(m0, m1, m2, moh, mol, P);  \
   } while (0)
-  if (P.dm.d == 128) { if (in_lo8) FF_DCT(128, true); else FF_DCT(128, false); }
-  else { if (in_lo8) FF_DCT(64, true); else FF_DCT(64, false); }
+#define FF_DCT_R(D, L) do { if (P.g.ragged) FF_DCT(D, L, true); else FF_DCT(D, L, false); } while (0)
+  if (P.dm.d == 128) { if (in_lo8) FF_DCT_R(128, true); else FF_DCT_R(128, false); }
+  else { if (in_lo8) FF_DCT_R(64, true); else FF_DCT_R(64, false); }
+#undef FF_DCT_R
 #undef FF_DCT
   if (e != cudaSuccess) return e;
   p->launches += 1;
@@ -662,15 +701,14 @@ extern "C" void ff_debug_dct_prof(unsigned long long* out64, int reset) {
 namespace {
 #endif
 
-bool axis_ok(int n) { return n == 16 || n == 32 || n == 64 || n == 128; }
-
 }  // namespace
 
-// bf16, head_dim 128 or 64, power-of-two axis lengths 16..128.
+// bf16, head_dim 128 or 64; any axis lengths (at most 128: a line fits a tile).
 bool ffk_dct_tc_supported(const FFDims& dm) {
-  if (dm.fp32 || (dm.d != 128 && dm.d != 64) || !axis_ok(dm.T) || !axis_ok(dm.H) || !axis_ok(dm.W)) return false;
-  // a tile groups 128/n lines: consecutive h for the w pass, consecutive w for the h and t passes
-  return dm.H % (TILE_ROWS / dm.W) == 0 && dm.W % (TILE_ROWS / dm.H) == 0 && dm.W % (TILE_ROWS / dm.T) == 0;
+  if (dm.fp32 || (dm.d != 128 && dm.d != 64)) return false;
+  long long tiles = 0;
+  for (int a = 0; a < 3; ++a) { const FFPassShape g = ff_pass_shape(dm, a); if (g.tiles > tiles) tiles = g.tiles; }
+  return 3LL * dm.BH * tiles < (1LL << 31);              // tile numbers of a launch are 31-bit
 }
 
 // The matrix of axis `axis` (0 = t, 1 = h, 2 = w), forward or inverse, as the tensor-memory operand image the
@@ -707,7 +745,6 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
   // along the remaining axis.  Kernel-select bit 4: the three axes as separate passes w, h, t.
   const bool fused = p->dct2_ok && !(p->attn_impl & 4);
   const int last_axis = fused ? (p->dct2_axis2 == 1 ? 0 : 1) : 0;
-  const int last_n = last_axis == 0 ? dm.T : dm.H;
   // Between the launches the hi/lo pair has the three-byte form (the lo grids hold bytes).
   // mXh/mXl: load maps of a pass's input pair; oXh/oXl: store maps of a pass's output pair (the box
   // follows the axis of the pass that uses the map)
@@ -739,19 +776,19 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
       e = ffk_dct2_forward(p, Q, K, V, g0, g, sc.a_hi, sc.a_lo, st);
       if (e != cudaSuccess) return e;
       P.in_split = 1; P.out_lo8 = 0; P.reverse = 1;
-      P.mode = MODE_SPLIT; P.axis = last_axis; P.n = last_n; P.image = matrix_image(p, last_axis, 0);
+      P.mode = MODE_SPLIT; P.axis = last_axis; P.image = matrix_image(p, last_axis, 0);
       e = launch_pass(p, m3h, m3l, m3l, m3h, m3l, P, false, st);    // (no tensor stores in this mode)
       if (e != cudaSuccess) return e;
       continue;
     }
-    P.mode = MODE_FIRST; P.in_split = 0; P.out_lo8 = 1; P.reverse = 0; P.axis = 2; P.n = dm.W; P.image = matrix_image(p, 2, 0);
+    P.mode = MODE_FIRST; P.in_split = 0; P.out_lo8 = 1; P.reverse = 0; P.axis = 2; P.image = matrix_image(p, 2, 0);
     e = launch_pass(p, mq, mk, mv, o0h, o0l, P, false, st);
     if (e != cudaSuccess) return e;
-    P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = mid8 ? 1 : 0; P.reverse = 1; P.axis = 1; P.n = dm.H; P.image = matrix_image(p, 1, 0);
+    P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = mid8 ? 1 : 0; P.reverse = 1; P.axis = 1; P.image = matrix_image(p, 1, 0);
     e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, true, st);
     if (e != cudaSuccess) return e;
     P.in_split = 1; P.out_lo8 = 0; P.reverse = 0;
-    P.mode = MODE_SPLIT; P.axis = 0; P.n = dm.T; P.image = matrix_image(p, 0, 0);
+    P.mode = MODE_SPLIT; P.axis = 0; P.image = matrix_image(p, 0, 0);
     e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, mid8, st);    // (no tensor stores in this mode)
     if (e != cudaSuccess) return e;
   }
@@ -774,7 +811,6 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
   const Scratch sc = carve(p);
   const bool fused = p->dct2_ok && !(p->attn_impl & 4);
   const int first_axis = fused ? (p->dct2_axis2 == 1 ? 0 : 1) : 0;       // the axis the fused launch leaves out
-  const int first_n = first_axis == 0 ? dm.T : dm.H;
   // The first pass reads the exchange's output, which has the three-byte form.  With three passes the pairs
   // between them have it too; the fused launch takes a bf16 pair.
   const bool b8 = !fused;
@@ -789,14 +825,14 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
     return cudaErrorInvalidValue;
   DctTcParams P{};
   P.dm = dm; P.status = p->buf.status; P.group = g; P.group_start = h0;
-  P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = b8 ? 1 : 0; P.reverse = 1; P.axis = first_axis; P.n = first_n;
+  P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = b8 ? 1 : 0; P.reverse = 1; P.axis = first_axis;
   P.image = matrix_image(p, first_axis, 1);
   cudaError_t e = launch_pass(p, m_in, m_inl, m_inl, obh, obl, P, true, st);
   if (e != cudaSuccess) return e;
   if (fused) return ffk_dct2_inverse(p, sc.b_hi, sc.b_lo, h0, g, out, st);
-  P.in_split = 1; P.out_lo8 = inv8 ? 1 : 0; P.reverse = 0; P.axis = 1; P.n = dm.H; P.image = matrix_image(p, 1, 1);
+  P.in_split = 1; P.out_lo8 = inv8 ? 1 : 0; P.reverse = 0; P.axis = 1; P.image = matrix_image(p, 1, 1);
   e = launch_pass(p, mbh, mbl, mbl, oah, oal, P, true, st);
   if (e != cudaSuccess) return e;
-  P.mode = MODE_LAST; P.out_lo8 = 0; P.reverse = 1; P.axis = 2; P.n = dm.W; P.image = matrix_image(p, 2, 1);
+  P.mode = MODE_LAST; P.out_lo8 = 0; P.reverse = 1; P.axis = 2; P.image = matrix_image(p, 2, 1);
   return launch_pass(p, mah, mal, mal, mout, mout, P, inv8, st);
 }

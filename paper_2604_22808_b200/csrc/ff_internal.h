@@ -58,6 +58,46 @@ FF_HD int ff_band_rank_of(const FFDims& dm, int kt, int kh, int kw, long long* r
   return 2;
 }
 
+// Division of a 31-bit number by a number fixed on the host, as a multiply-high, an add and a shift (Granlund and
+// Montgomery, "Division by Invariant Integers using Multiplication", 1994).
+struct FFFastDiv { unsigned d, m, s; };
+inline FFFastDiv ff_fast_div(unsigned d) {
+  FFFastDiv f;
+  f.d = d; f.s = 0;
+  while ((1ull << f.s) < d) ++f.s;
+  f.m = (unsigned)(((((1ull << f.s) - d) << 32) / d) + 1);
+  return f;
+}
+#if defined(__CUDACC__)
+__device__ __forceinline__ unsigned ff_div(unsigned n, const FFFastDiv& f) { return (__umulhi(f.m, n) + n) >> f.s; }
+#endif
+
+// One axis of a tensor-core transform pass as a grid [outer][n][inner] of positions.  A tile is kf whole lines:
+// neighbours along `inner` (t and h axes: row = a * kf + line) or, where inner is 1 (w axis), along `outer`
+// (row = line * n + a).
+struct FFPassShape {
+  int n, kf, rows;          // axis length, lines per tile, rows in use (kf * n <= 128)
+  int inner, outer;
+  int seq;                  // w axis
+  int tiles_inner;          // tiles along `inner` (1 for the w axis)
+  int tiles;                // tiles of one tensor-head
+  int ragged;               // rows are left over, a last tile is not full, or 32 rows are not a box of the grid
+};
+inline FFPassShape ff_pass_shape(const FFDims& dm, int axis) {
+  FFPassShape g;
+  g.n = axis == 2 ? dm.W : (axis == 1 ? dm.H : dm.T);
+  g.inner = axis == 2 ? 1 : (axis == 1 ? dm.W : dm.H * dm.W);
+  g.outer = axis == 2 ? dm.T * dm.H : (axis == 1 ? dm.T : 1);
+  g.seq = axis == 2;
+  const int lines = g.seq ? g.outer : g.inner;
+  g.kf = 128 / g.n < lines ? 128 / g.n : lines;
+  g.rows = g.kf * g.n;
+  g.tiles_inner = g.seq ? 1 : (g.inner + g.kf - 1) / g.kf;
+  g.tiles = g.seq ? (g.outer + g.kf - 1) / g.kf : g.outer * g.tiles_inner;
+  g.ragged = g.rows != 128 || lines % g.kf != 0 || (g.n & (g.n - 1)) != 0;
+  return g;
+}
+
 // Device buffers inside the caller's workspace.
 struct FFBuffers {
   float* spec_low;   // [3][BH][Nlow][d]
