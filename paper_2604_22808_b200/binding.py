@@ -141,6 +141,11 @@ def _f32(a) -> Optional[np.ndarray]:
     return None if a is None else np.ascontiguousarray(a, dtype=np.float32)
 
 
+def _floats(values):
+    """A host float array for the call (None stays None)."""
+    return None if values is None else (C.c_float * len(values))(*values)
+
+
 def _ptr(a: Optional[np.ndarray]):
     return None if a is None else a.ctypes.data_as(C.c_void_p)
 
@@ -173,6 +178,9 @@ class Plan:
             self.workspace = torch.empty(nbytes, dtype=torch.uint8, device=self.device)
             _check(lib.ff_plan_set_workspace(self.handle, self.workspace.data_ptr(), nbytes), self.handle)
         self.workspace_bytes = nbytes
+        self._shape = torch.Size((cfg.batch, cfg.heads, cfg.T, cfg.H, cfg.W, cfg.head_dim))
+        self._dtype = torch.float32 if cfg.dtype == "fp32" else torch.bfloat16
+        self._raw_stream = torch._C._cuda_getCurrentRawStream      # (a Stream object per call costs more than a launch)
 
     # -- lifetime
     def destroy(self):
@@ -194,28 +202,28 @@ class Plan:
         return tuple(int(x) for x in out)
 
     def _stream(self):
-        return C.c_void_p(self._torch.cuda.current_stream(self.device).cuda_stream)
+        return self._raw_stream(self.device.index)
 
     @property
     def torch_dtype(self):
-        return self._torch.float32 if self.cfg.dtype == "fp32" else self._torch.bfloat16
+        return self._dtype
 
     def _check_io(self, *tensors):
-        shape = (self.cfg.batch, self.cfg.heads, self.cfg.T, self.cfg.H, self.cfg.W, self.cfg.head_dim)
+        shape, dtype, device = self._shape, self._dtype, self.device
         for t in tensors:
-            if tuple(t.shape) != shape or t.dtype != self.torch_dtype or not t.is_contiguous():
-                raise FFError(1, f"expected a contiguous {self.torch_dtype} tensor of shape {shape}")
-            if not t.is_cuda or t.device != self.device:
+            if t.shape != shape or t.dtype != dtype or not t.is_contiguous():
+                raise FFError(1, f"expected a contiguous {dtype} tensor of shape {tuple(shape)}")
+            if t.device != device:
                 raise FFError(1, f"expected a tensor on {self.device}, got one on {t.device}")
 
     # -- the path
     def route(self, Q, K, V, timesteps: Sequence[float], alloc_out=None, want_host: bool = True):
         self._check_io(Q, K, V)
-        ts = np.ascontiguousarray(timesteps, dtype=np.float32)
-        assert ts.shape == (self.cfg.batch,)
+        ts = _floats(timesteps)
+        assert len(timesteps) == self.cfg.batch
         alloc_h = np.zeros(self.cfg.batch * self.cfg.heads, np.uint8) if want_host else None
         pi_h = np.zeros((self.cfg.batch, 3), np.float32) if want_host else None
-        _check(library().ff_route(self.handle, Q.data_ptr(), K.data_ptr(), V.data_ptr(), _ptr(ts),
+        _check(library().ff_route(self.handle, Q.data_ptr(), K.data_ptr(), V.data_ptr(), ts,
                                   None if alloc_out is None else alloc_out.data_ptr(), _ptr(alloc_h), _ptr(pi_h),
                                   self._stream()), self.handle)
         return alloc_h, pi_h
@@ -223,18 +231,18 @@ class Plan:
     def forward(self, Q, K, V, out, alloc=None, timesteps: Optional[Sequence[float]] = None):
         """alloc: uint8 CUDA tensor [batch*heads] of band masks, or None to route from timesteps."""
         self._check_io(Q, K, V, out)
-        ts = None if timesteps is None else np.ascontiguousarray(timesteps, dtype=np.float32)
+        ts = _floats(timesteps)
         _check(library().ff_forward(self.handle, Q.data_ptr(), K.data_ptr(), V.data_ptr(),
-                                    None if alloc is None else alloc.data_ptr(), _ptr(ts), out.data_ptr(),
+                                    None if alloc is None else alloc.data_ptr(), ts, out.data_ptr(),
                                     self._stream()), self.handle)
         return out
 
     def forward_host(self, Qh, Kh, Vh, out_h, alloc_host: Optional[np.ndarray] = None,
                      timesteps: Optional[Sequence[float]] = None):
         """Host tensors (ideally pinned) in and out; the copies are part of the call."""
-        ts = None if timesteps is None else np.ascontiguousarray(timesteps, dtype=np.float32)
+        ts = _floats(timesteps)
         al = None if alloc_host is None else np.ascontiguousarray(alloc_host, dtype=np.uint8)
-        _check(library().ff_forward_host(self.handle, Qh.data_ptr(), Kh.data_ptr(), Vh.data_ptr(), _ptr(al), _ptr(ts),
+        _check(library().ff_forward_host(self.handle, Qh.data_ptr(), Kh.data_ptr(), Vh.data_ptr(), _ptr(al), ts,
                                          out_h.data_ptr(), self._stream()), self.handle)
         return out_h
 
@@ -248,9 +256,9 @@ class Plan:
             if (tuple(t.shape) != shape or t.dtype != torch.bfloat16 or not t.is_contiguous() or not t.is_cuda
                     or t.device != self.device):
                 raise FFError(1, f"expected a contiguous bf16 tensor of shape {shape} on {self.device}")
-        ts = None if timesteps is None else np.ascontiguousarray(timesteps, dtype=np.float32)
+        ts = _floats(timesteps)
         _check(library().ff_forward_projected(self.handle, X.data_ptr(), Wqkv.data_ptr(), Wo.data_ptr(),
-                                              None if alloc is None else alloc.data_ptr(), _ptr(ts), out.data_ptr(),
+                                              None if alloc is None else alloc.data_ptr(), ts, out.data_ptr(),
                                               self._stream()), self.handle)
         return out
 

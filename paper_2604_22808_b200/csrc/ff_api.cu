@@ -207,6 +207,17 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
     delete p;
     return FF_ERR_CUDA;
   }
+  ce = ffk_simt_init();
+  if (ce == cudaSuccess) ce = ffk_attention_tc_init();
+  if (ce == cudaSuccess) ce = ffk_exchange_tc_init();
+  if (ce == cudaSuccess) ce = ffk_dct_tc_init();
+  if (ce == cudaSuccess) ce = ffk_dct2_init();
+  if (ce == cudaSuccess) ce = ffk_proj_init();
+  if (ce != cudaSuccess) {
+    fail(nullptr, FF_ERR_CUDA, "could not prepare the kernels: %s", cudaGetErrorString(ce));
+    delete p;
+    return FF_ERR_CUDA;
+  }
   // The 1-D transform matrices C[k][i], evaluated in double: DCT-II, alpha_k cos(pi (2i+1) k / (2n)), or the
   // orthonormal Haar wavelets (row 0 constant; row 2^j + q is +-sqrt(2^j / n) on the halves of the q-th block of
   // n / 2^j positions), rows from the coarsest scale to the finest.

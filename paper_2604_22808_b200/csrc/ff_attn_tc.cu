@@ -78,6 +78,7 @@ __host__ __device__ __forceinline__ MidShape mid_shape(const FFDims& dm) {
 // Worklist: one unit per (head, mid band) and per (head, high band) that the allocation executes;
 // mid units first (their items are the long ones).  An item is a pair of query tiles.
 __global__ void build_worklist_kernel(TcParams P) {
+  ff_pdl_wait();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   const FFDims& dm = P.dm;
   int* offsets = P.work + 2;
@@ -285,16 +286,17 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
       mbar_init(&sh.o_full[i], 1); mbar_init(&sh.o_empty[i], 128 * NSPLIT);
     }
     sh.abort_flag = 0;
-    sh.n_units = P.work[0];
-    sh.total = P.work[1];
     sh.ms = mid_shape(dm);
     fence_mbar_init();
   }
-  __syncthreads();
   for (int i = threadIdx.x; i < 2 * 2 * NSPLIT * 128; i += TC_THREADS) {
     (&sh.xmax[0][0][0][0])[i] = 0ull;
     (&sh.xsum[0][0][0][0])[i] = 0ull;
   }
+  if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
+  ff_pdl_wait();
+  if (threadIdx.x == 0) { sh.n_units = P.work[0]; sh.total = P.work[1]; }
+  __syncthreads();
   for (int i = threadIdx.x; i <= sh.n_units; i += TC_THREADS) {
     sh.offsets[i] = P.work[2 + i];
     if (i < sh.n_units) {
@@ -302,7 +304,6 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
       sh.ntile[i] = P.work[2 + MAX_UNITS + 1 + MAX_UNITS + i];
     }
   }
-  if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -715,6 +716,16 @@ bool ffk_tc_supported(const FFDims& dm) {
   return true;
 }
 
+cudaError_t ffk_attention_tc_init() {
+  cudaError_t e = cudaSuccess;
+#define FF_ATT(D, LOW) \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(attention_tc_kernel<D, LOW>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                                                 (int)(6 * TILE_BYTES + sizeof(Shared) + 1024))
+  FF_ATT(128, true); FF_ATT(128, false); FF_ATT(64, true); FF_ATT(64, false);
+#undef FF_ATT
+  return e;
+}
+
 bool ffk_tc_prepare(ff_plan* p) {
   static_assert(sizeof(CUtensorMap) <= sizeof(p->tmap_mid), "tensor map storage too small");
   const FFDims& dm = p->dm;
@@ -738,24 +749,18 @@ cudaError_t ffk_attention_tc(ff_plan* p, cudaStream_t st) {
   P.y_mid = (__nv_bfloat16*)p->buf.y_mid; P.y_high = (__nv_bfloat16*)p->buf.y_high;
   P.y_low = p->buf.y_low; P.low_on = p->low_tc_ok ? 1 : 0;
   P.status = p->buf.status; P.rb_mid = dm.b < TILE ? dm.b : TILE;
-  build_worklist_kernel<<<1, 32, 0, st>>>(P);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = ff_launch(build_worklist_kernel, dim3(1), dim3(32), 0, st, P);
   if (e != cudaSuccess) return e;
   const size_t smem = 6 * TILE_BYTES + sizeof(Shared) + 1024;
   const CUtensorMap& mm = *(const CUtensorMap*)p->tmap_mid;
   const CUtensorMap& mh = *(const CUtensorMap*)p->tmap_high;
   const CUtensorMap& ml = p->low_tc_ok ? *(const CUtensorMap*)p->tmap_low : mh;
-#define FF_ATT(D, LOW)                                                                                             \
-  do {                                                                                                             \
-    e = cudaFuncSetAttribute(attention_tc_kernel<D, LOW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-    if (e == cudaSuccess) attention_tc_kernel<D, LOW><<<p->sm_count, TC_THREADS, smem, st>>>(mm, mh, ml, P);       \
-  } while (0)
-  if (dm.d == 128) { if (p->low_tc_ok) FF_ATT(128, true); else FF_ATT(128, false); }
-  else { if (p->low_tc_ok) FF_ATT(64, true); else FF_ATT(64, false); }
-#undef FF_ATT
-  if (e != cudaSuccess) return e;
   p->launches += 2;
-  return cudaGetLastError();
+#define FF_ATT(D, LOW) return ff_launch(attention_tc_kernel<D, LOW>, dim3(p->sm_count), dim3(TC_THREADS), smem, st, mm, mh, ml, P)
+  if (dm.d == 128) { if (p->low_tc_ok) FF_ATT(128, true); FF_ATT(128, false); }
+  if (p->low_tc_ok) FF_ATT(64, true);
+  FF_ATT(64, false);
+#undef FF_ATT
 }
 
 // ------------------------------------------------------------------------------------------------

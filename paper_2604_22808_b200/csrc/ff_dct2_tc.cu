@@ -279,6 +279,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     }
     tmem_wait_st();
   }
+  ff_pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -670,13 +671,14 @@ bool axis_ok(int n) { return n == 16 || n == 32 || n == 64 || n == 128; }
 
 cudaError_t launch(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, const CUtensorMap& m2, const CUtensorMap& moh,
                    const CUtensorMap& mol, Dct2Params& P, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(dct2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D2_SMEM);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   const int items = P.group * P.n3 * P.nchunk;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)P.cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
   cfg.blockDim = dim3(D2_THREADS); cfg.dynamicSmemBytes = D2_SMEM; cfg.stream = st;
   int clusters = p->dct2_clusters;
@@ -691,13 +693,26 @@ cudaError_t launch(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, con
   }
   if (clusters > items) clusters = items;
   cfg.gridDim = dim3((unsigned)(clusters * P.cs));
+  cfg.numAttrs = !P.in_split && p->pipe_in ? 1 : 2;      // (programmatic launch, except right after an event wait)
   e = cudaLaunchKernelEx(&cfg, dct2_tc_kernel, m0, m1, m2, moh, mol, P);
   if (e != cudaSuccess) return e;
   p->launches += 1;
-  return cudaGetLastError();
+  return cudaSuccess;
+}
+
+// (through the plan's cache)
+bool in_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis2) {
+  return p->maps.get(map, base, 16 | axis2, slices, [&] { return encode_in_map(map, base, p->dm, slices, axis2); });
+}
+bool out_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis2) {
+  return p->maps.get(map, base, 24 | axis2, slices, [&] { return encode_out_map(map, base, p->dm, slices, axis2); });
 }
 
 }  // namespace
+
+cudaError_t ffk_dct2_init() {
+  return cudaFuncSetAttribute(dct2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D2_SMEM);
+}
 
 // Which second axis the fused launch takes and how many CTAs share a plane: the shorter of h and t
 // (smaller planes need fewer CTAs), an even number of tiles per CTA.  The kernel runs clusters of up to
@@ -756,9 +771,9 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
   int axis2, cs;
   if (!ffk_dct2_supported(dm, &axis2, &cs)) return cudaErrorInvalidValue;
   CUtensorMap mq, mk, mv, oh, ol;
-  if (!encode_in_map(&mq, Q, dm, dm.BH, axis2) || !encode_in_map(&mk, K, dm, dm.BH, axis2) ||
-      !encode_in_map(&mv, V, dm, dm.BH, axis2) || !encode_out_map(&oh, out_hi, dm, G, axis2) ||
-      !encode_out_map(&ol, out_lo, dm, G, axis2))
+  if (!in_map(p, &mq, Q, dm.BH, axis2) || !in_map(p, &mk, K, dm.BH, axis2) ||
+      !in_map(p, &mv, V, dm.BH, axis2) || !out_map(p, &oh, out_hi, G, axis2) ||
+      !out_map(p, &ol, out_lo, G, axis2))
     return cudaErrorInvalidValue;
   const size_t per = (size_t)2 * ROWS * IMG_CELLS;
   Dct2Params P{};
@@ -777,8 +792,8 @@ cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, i
   int axis2, cs;
   if (!ffk_dct2_supported(dm, &axis2, &cs)) return cudaErrorInvalidValue;
   CUtensorMap mh, ml, mo;
-  if (!encode_in_map(&mh, in_hi, dm, G, axis2) || !encode_in_map(&ml, in_lo, dm, G, axis2) ||
-      !encode_out_map(&mo, out, dm, dm.BH, axis2))
+  if (!in_map(p, &mh, in_hi, G, axis2) || !in_map(p, &ml, in_lo, G, axis2) ||
+      !out_map(p, &mo, out, dm.BH, axis2))
     return cudaErrorInvalidValue;
   const size_t per = (size_t)2 * ROWS * IMG_CELLS;
   Dct2Params P{};

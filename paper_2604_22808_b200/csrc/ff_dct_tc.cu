@@ -211,6 +211,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     }
     tmem_wait_st();
   }
+  ff_pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -599,6 +600,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
 // Low-band energy for the router: sum of squares of the fp32 low-band coefficients per channel,
 // over Q~, K~, V~ and the heads of a sample.  grid = (row chunks, 3 BH); thread = channel.
 __global__ void low_energy_kernel(const float* spec_low, double* energy, FFDims dm) {
+  ff_pdl_wait();
   const int th = blockIdx.y, c = threadIdx.x;
   const long long per = (dm.Nlow + gridDim.x - 1) / gridDim.x;
   const long long r0 = (long long)blockIdx.x * per, r1 = r0 + per < dm.Nlow ? r0 + per : dm.Nlow;
@@ -652,11 +654,16 @@ bool encode_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices
              store ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-bool encode_grid_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, bool bytes = false) {
-  return encode_map(map, base, dm, slices, axis, bytes, false);
+// (through the plan's cache)
+bool map_for(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, bool bytes, bool store) {
+  return p->maps.get(map, base, axis | (bytes ? 4 : 0) | (store ? 8 : 0), slices,
+                     [&] { return encode_map(map, base, p->dm, slices, axis, bytes, store); });
 }
-bool encode_store_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, bool bytes = false) {
-  return encode_map(map, base, dm, slices, axis, bytes, true);
+bool grid_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, bool bytes = false) {
+  return map_for(p, map, base, slices, axis, bytes, false);
+}
+bool store_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, bool bytes = false) {
+  return map_for(p, map, base, slices, axis, bytes, true);
 }
 
 // `in_lo8`: the input pair's lo grid is the byte form (m1 = its byte map).
@@ -675,12 +682,11 @@ cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1
   P.by_line = ff_fast_div((unsigned)(P.axis == 2 ? P.dm.H : P.dm.W));
   const int tiles = P.group * P.g.tiles;
   const int grid = tiles < p->sm_count ? tiles : p->sm_count;
-#define FF_DCT(D, L, R)                                                                                              \
-  do {                                                                                                               \
-    e = cudaFuncSetAttribute(dct_tc_kernel<D, L, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);        \
-    if (e == cudaSuccess)                                                                                            \
-      dct_tc_kernel<D, L, R><<<grid, L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS, smem, st>>>(m0, m1, m2, moh, mol, P);  \
-  } while (0)
+#define FF_DCT(D, L, R)                                                                                                       \
+  e = P.mode == MODE_FIRST && p->pipe_in                                                                                       \
+          ? ff_launch_after_event(dct_tc_kernel<D, L, R>, dim3(grid), dim3(L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS), smem, st, \
+                                  m0, m1, m2, moh, mol, P)                                                                     \
+          : ff_launch(dct_tc_kernel<D, L, R>, dim3(grid), dim3(L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS), smem, st, m0, m1, m2, moh, mol, P)
 #define FF_DCT_R(D, L) do { if (P.g.ragged) FF_DCT(D, L, true); else FF_DCT(D, L, false); } while (0)
   if (P.dm.d == 128) { if (in_lo8) FF_DCT_R(128, true); else FF_DCT_R(128, false); }
   else { if (in_lo8) FF_DCT_R(64, true); else FF_DCT_R(64, false); }
@@ -688,7 +694,7 @@ cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1
 #undef FF_DCT
   if (e != cudaSuccess) return e;
   p->launches += 1;
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 #ifdef FF_DCT_PROF
@@ -702,6 +708,16 @@ namespace {
 #endif
 
 }  // namespace
+
+cudaError_t ffk_dct_tc_init() {
+  cudaError_t e = cudaSuccess;
+#define FF_DCT(D, L, R) \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(dct_tc_kernel<D, L, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 256)
+  FF_DCT(128, false, false); FF_DCT(128, true, false); FF_DCT(128, false, true); FF_DCT(128, true, true);
+  FF_DCT(64, false, false); FF_DCT(64, true, false); FF_DCT(64, false, true); FF_DCT(64, true, true);
+#undef FF_DCT
+  return e;
+}
 
 // bf16, head_dim 128 or 64; any axis lengths (at most 128: a line fits a tile).
 bool ffk_dct_tc_supported(const FFDims& dm) {
@@ -750,13 +766,12 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
   // follows the axis of the pass that uses the map)
   const bool mid8 = false;        // (measured: the band-split pass is slower with a byte-form input)
   CUtensorMap mq, mk, mv, m1h, m1l, m2h, m2l, o0h, o0l, o1h, o1l, m3h, m3l;
-  if (!encode_grid_map(&mq, Q, dm, dm.BH, 2) || !encode_grid_map(&mk, K, dm, dm.BH, 2) ||
-      !encode_grid_map(&mv, V, dm, dm.BH, 2) || !encode_grid_map(&m1h, sc.a_hi, dm, G, 1) ||
-      !encode_grid_map(&m1l, sc.a_lo, dm, G, 1, true) || !encode_grid_map(&m2h, sc.b_hi, dm, G, 0) ||
-      !encode_grid_map(&m2l, sc.b_lo, dm, G, 0, mid8) || !encode_store_map(&o0h, sc.a_hi, dm, G, 2) ||
-      !encode_store_map(&o0l, sc.a_lo, dm, G, 2, true) || !encode_store_map(&o1h, sc.b_hi, dm, G, 1) ||
-      !encode_store_map(&o1l, sc.b_lo, dm, G, 1, mid8) || !encode_grid_map(&m3h, sc.a_hi, dm, G, last_axis) ||
-      !encode_grid_map(&m3l, sc.a_lo, dm, G, last_axis))
+  if (fused ? !(grid_map(p, &m3h, sc.a_hi, G, last_axis) && grid_map(p, &m3l, sc.a_lo, G, last_axis))
+            : !(grid_map(p, &mq, Q, dm.BH, 2) && grid_map(p, &mk, K, dm.BH, 2) && grid_map(p, &mv, V, dm.BH, 2) &&
+                store_map(p, &o0h, sc.a_hi, G, 2) && store_map(p, &o0l, sc.a_lo, G, 2, true) &&
+                grid_map(p, &m1h, sc.a_hi, G, 1) && grid_map(p, &m1l, sc.a_lo, G, 1, true) &&
+                store_map(p, &o1h, sc.b_hi, G, 1) && store_map(p, &o1l, sc.b_lo, G, 1, mid8) &&
+                grid_map(p, &m2h, sc.b_hi, G, 0) && grid_map(p, &m2l, sc.b_lo, G, 0, mid8)))
     return cudaErrorInvalidValue;
   const int total = 3 * dm.BH;
   DctTcParams P{};
@@ -795,10 +810,8 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
   if (want_energy) {
     long long chunks = (dm.Nlow + 511) / 512;             // about 512 rows per block
     if (chunks > 256) chunks = 256;
-    low_energy_kernel<<<dim3((unsigned)chunks, (unsigned)total), dm.d, 0, st>>>(p->buf.spec_low, p->buf.energy, dm);
     p->launches += 1;
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    return ff_launch(low_energy_kernel, dim3((unsigned)chunks, (unsigned)total), dim3(dm.d), 0, st, p->buf.spec_low, p->buf.energy, dm);
   }
   return cudaSuccess;
 }
@@ -816,12 +829,13 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
   const bool b8 = !fused;
   const bool inv8 = true;
   CUtensorMap m_in, m_inl, mbh, mbl, mah, mal, obh, obl, oah, oal, mout;
-  if (!encode_grid_map(&m_in, sc.a_hi, dm, G, first_axis) || !encode_grid_map(&m_inl, sc.a_lo, dm, G, first_axis, true) ||
-      !encode_grid_map(&mbh, sc.b_hi, dm, G, 1) ||
-      !encode_grid_map(&mbl, sc.b_lo, dm, G, 1, true) || !encode_grid_map(&mah, sc.a_hi, dm, G, 2) ||
-      !encode_grid_map(&mal, sc.a_lo, dm, G, 2, inv8) || !encode_store_map(&obh, sc.b_hi, dm, G, first_axis) ||
-      !encode_store_map(&obl, sc.b_lo, dm, G, first_axis, b8) || !encode_store_map(&oah, sc.a_hi, dm, G, 1) ||
-      !encode_store_map(&oal, sc.a_lo, dm, G, 1, inv8) || !encode_store_map(&mout, out, dm, dm.BH, 2))
+  if (!grid_map(p, &m_in, sc.a_hi, G, first_axis) || !grid_map(p, &m_inl, sc.a_lo, G, first_axis, true) ||
+      !store_map(p, &obh, sc.b_hi, G, first_axis) || !store_map(p, &obl, sc.b_lo, G, first_axis, b8))
+    return cudaErrorInvalidValue;
+  if (!fused && (!grid_map(p, &mbh, sc.b_hi, G, 1) || !grid_map(p, &mbl, sc.b_lo, G, 1, true) ||
+                 !store_map(p, &oah, sc.a_hi, G, 1) || !store_map(p, &oal, sc.a_lo, G, 1, inv8) ||
+                 !grid_map(p, &mah, sc.a_hi, G, 2) || !grid_map(p, &mal, sc.a_lo, G, 2, inv8) ||
+                 !store_map(p, &mout, out, dm.BH, 2)))
     return cudaErrorInvalidValue;
   DctTcParams P{};
   P.dm = dm; P.status = p->buf.status; P.group = g; P.group_start = h0;

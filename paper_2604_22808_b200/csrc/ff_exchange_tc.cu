@@ -124,6 +124,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
     fence_mbar_init();
   }
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 256); tmem_relinquish(); }
+  ff_pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -483,6 +484,16 @@ bool ffk_exchange_tc_supported(const FFDims& dm) {
   return !dm.fp32 && (dm.d == 128 || dm.d == 64) && dm.m >= 1 && dm.m <= 32 && dm.N < (1LL << 31);
 }
 
+cudaError_t ffk_exchange_tc_init() {
+  cudaError_t e = cudaSuccess;
+  // (the largest: a token tile, 96 keys as hi and lo images)
+  const int most = 2 * X_TILE_BYTES + 4 * 96 * 128 + (int)sizeof(XShared) + 1024;
+#define FF_XCH(NK, D) if (e == cudaSuccess) e = cudaFuncSetAttribute(exchange_tc_kernel<NK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+  FF_XCH(1, 128); FF_XCH(2, 128); FF_XCH(3, 128); FF_XCH(1, 64); FF_XCH(2, 64); FF_XCH(3, 64);
+#undef FF_XCH
+  return e;
+}
+
 // Rank -> flat coefficient index tables of the mid and high bands (plan-owned device memory).
 bool ffk_exchange_tc_build_tables(ff_plan* p) {
   const FFDims& dm = p->dm;
@@ -533,19 +544,15 @@ cudaError_t ffk_exchange_tc(ff_plan* p, int h0, int g, void* grid_hi, void* grid
   const CUtensorMap& m1 = *(const CUtensorMap*)p->tmap_x[1];
   const CUtensorMap& m2 = *(const CUtensorMap*)p->tmap_x[2];
   const CUtensorMap& m3 = *(const CUtensorMap*)p->tmap_x[3];
-  cudaError_t e = cudaSuccess;
-#define FF_XCH(NK, D)                                                                                              \
-  do {                                                                                                             \
-    e = cudaFuncSetAttribute(exchange_tc_kernel<NK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);   \
-    if (e == cudaSuccess) exchange_tc_kernel<NK, D><<<grid, X_THREADS, smem, st>>>(m0, m1, m2, m3, P);             \
-  } while (0)
-  if (dm.d == 128) {
-    if (P.nkeys <= 32) FF_XCH(1, 128); else if (P.nkeys <= 64) FF_XCH(2, 128); else FF_XCH(3, 128);
-  } else {
-    if (P.nkeys <= 32) FF_XCH(1, 64); else if (P.nkeys <= 64) FF_XCH(2, 64); else FF_XCH(3, 64);
-  }
-#undef FF_XCH
-  if (e != cudaSuccess) return e;
   p->launches += 1;
-  return cudaGetLastError();
+#define FF_XCH(NK, D) return ff_launch(exchange_tc_kernel<NK, D>, dim3(grid), dim3(X_THREADS), smem, st, m0, m1, m2, m3, P)
+  if (dm.d == 128) {
+    if (P.nkeys <= 32) FF_XCH(1, 128);
+    if (P.nkeys <= 64) FF_XCH(2, 128);
+    FF_XCH(3, 128);
+  }
+  if (P.nkeys <= 32) FF_XCH(1, 64);
+  if (P.nkeys <= 64) FF_XCH(2, 64);
+  FF_XCH(3, 64);
+#undef FF_XCH
 }

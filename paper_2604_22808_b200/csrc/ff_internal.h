@@ -4,6 +4,9 @@
 #include <cuda_bf16.h>
 #include <stddef.h>
 #include <stdint.h>
+#include <string.h>
+
+#include <utility>
 
 #include "freqformer.h"
 
@@ -69,6 +72,32 @@ inline FFFastDiv ff_fast_div(unsigned d) {
   return f;
 }
 #if defined(__CUDACC__)
+// Programmatic dependent launch.  Every kernel of the path is launched with the attribute, does what does not
+// depend on earlier kernels (barriers, tensor memory, matrices of the plan), then waits here until the kernel
+// before it in the stream has finished and its writes are visible, and lets the next kernel start its own
+// prologue.  It reads or writes nothing another kernel touches before the wait.
+__device__ __forceinline__ void ff_pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// (a launch right after an event wait goes without the attribute: ff_launch_after_event)
+template <class... K, class... A>
+inline cudaError_t ff_launch_after_event(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  kernel<<<grid, block, smem, st>>>(std::forward<A>(args)...);
+  return cudaGetLastError();
+}
+template <class... K, class... A>
+inline cudaError_t ff_launch(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
 __device__ __forceinline__ unsigned ff_div(unsigned n, const FFFastDiv& f) { return (__umulhi(f.m, n) + n) >> f.s; }
 #endif
 
@@ -133,6 +162,28 @@ struct FFLayout {
 
 constexpr int FF_COPY_EVENTS = 64;
 
+// Tensor maps kept between calls (encoding two dozen of them took longer on the host than the launches they are
+// for).  An entry is known by the tensor's address, its number of slices and the encoder's own code for the rest,
+// which the plan's configuration determines; the oldest entry makes room for a new one.
+struct FFMapCache {
+  static constexpr int N = 48;
+  alignas(64) unsigned char map[N][128];
+  const void* base[N];
+  int code[N], slices[N];
+  int used, next;
+  template <class Encode>
+  bool get(void* out, const void* b, int c, int s, Encode encode) {
+    for (int i = 0; i < used; ++i)
+      if (base[i] == b && code[i] == c && slices[i] == s) { memcpy(out, map[i], 128); return true; }
+    if (!encode()) return false;
+    const int i = used < N ? used++ : next;
+    if (used == N) next = (i + 1) % N;
+    memcpy(map[i], out, 128);
+    base[i] = b; code[i] = c; slices[i] = s;
+    return true;
+  }
+};
+
 struct ff_plan {
   ff_config_t cfg;
   FFDims dm;
@@ -157,6 +208,7 @@ struct ff_plan {
   int* pos_table;                              // rank -> flat coefficient index of the mid, then the high band (plan-owned)
   alignas(64) unsigned char tmap_x[4][128];    // CUtensorMaps of the exchange kernel (Y / V~ of the mid and high bands)
   uint32_t* dct2_images;                       // 6 x (hi, lo) transform matrices as tensor-memory operand images (plan-owned)
+  FFMapCache maps;                             // tensor maps of the transform passes
   bool dct2_ok;                                // the fused two-axis launch covers this configuration
   int dct2_axis2;                              // its second axis (1 = h, 0 = t); the remaining axis gets a pass of its own
   int dct2_clusters;                           // clusters of that launch the device runs at once (0 = not yet asked)
@@ -184,6 +236,13 @@ void ff_set_thread_error(const char* msg);
 void ff_compute_layout(const FFDims& dm, bool with_staging, FFLayout* lay);
 
 // ---- kernel launchers (ff_simt.cu).  Each returns the cudaError_t of its launches. --------------
+// (..._init: kernel attributes on the current device, set at plan creation)
+cudaError_t ffk_simt_init();
+cudaError_t ffk_attention_tc_init();
+cudaError_t ffk_exchange_tc_init();
+cudaError_t ffk_dct_tc_init();
+cudaError_t ffk_dct2_init();
+cudaError_t ffk_proj_init();
 cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, const void* V, cudaStream_t st);
 cudaError_t ffk_band_energy(ff_plan* p, cudaStream_t st);
 cudaError_t ffk_router(ff_plan* p, uint8_t* alloc_out, cudaStream_t st);

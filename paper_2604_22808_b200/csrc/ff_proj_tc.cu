@@ -62,6 +62,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     fence_mbar_init();
   }
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
+  ff_pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -197,18 +198,20 @@ bool encode_map(CUtensorMap* map, const void* base, long long cols, long long ro
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+constexpr size_t P_SMEM = (size_t)P_NSTAGE * P_STAGE + sizeof(ProjShared) + 1024;
+
 cudaError_t launch_proj(ff_plan* p, const CUtensorMap& ma, const CUtensorMap& mb, const ProjParams& P, cudaStream_t st) {
-  const size_t smem = (size_t)P_NSTAGE * P_STAGE + sizeof(ProjShared) + 1024;
-  cudaError_t e = cudaFuncSetAttribute(proj_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const long long tiles = (long long)P.B * (P.N / PM) * (P.n_out / PN);
   const int grid = tiles < p->sm_count ? (int)tiles : p->sm_count;
-  proj_tc_kernel<<<grid, P_THREADS, smem, st>>>(ma, mb, P);
   p->launches += 1;
-  return cudaGetLastError();
+  return ff_launch(proj_tc_kernel, dim3(grid), dim3(P_THREADS), P_SMEM, st, ma, mb, P);
 }
 
 }  // namespace
+
+cudaError_t ffk_proj_init() {
+  return cudaFuncSetAttribute(proj_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P_SMEM);
+}
 
 // bf16 storage, head_dim 64 or 128, token count a multiple of 128, model width a multiple of 256.
 bool ffk_proj_supported(const FFDims& dm) {

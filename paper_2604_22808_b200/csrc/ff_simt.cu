@@ -46,6 +46,7 @@ struct DctPassParams {
 
 template <typename ST, int MODE>
 __global__ void __launch_bounds__(DCT_THREADS) dct_pass_kernel(const DctPassParams P) {
+  ff_pdl_wait();
   extern __shared__ float smem[];
   const int n = P.n;
   const int npad = (n + 7) & ~7;
@@ -136,12 +137,9 @@ template <typename ST, int MODE>
 cudaError_t launch_dct_pass(const DctPassParams& P, int group, cudaStream_t st) {
   const int npad = (P.n + 7) & ~7;
   const size_t smem = ((size_t)P.n * npad + (size_t)P.n * DCT_IC) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(dct_pass_kernel<ST, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
   const int chunks = (P.inner + DCT_IC - 1) / DCT_IC;
   dim3 grid((unsigned)((size_t)P.outer * chunks), (unsigned)group);
-  dct_pass_kernel<ST, MODE><<<grid, DCT_THREADS, smem, st>>>(P);
-  return cudaGetLastError();
+  return ff_launch(dct_pass_kernel<ST, MODE>, grid, dim3(DCT_THREADS), smem, st, P);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -153,6 +151,7 @@ constexpr int ENERGY_ROWS = 256;
 template <typename ST>
 __global__ void band_energy_kernel(const float* spec_low, const ST* spec_mid, const ST* spec_high, double* energy,
                                    FFDims dm) {
+  ff_pdl_wait();
   const int band = blockIdx.y;
   const int th = blockIdx.z;                 // tensor * BH + bh
   const long long nl = band == 0 ? dm.Nlow : (band == 1 ? dm.Nmid : dm.Nhigh);
@@ -181,6 +180,7 @@ __global__ void band_energy_kernel(const float* spec_low, const ST* spec_mid, co
 // z = W2 relu(W1 [g; e(t)] + b1) + b2, pi = softmax(z), largest-remainder quota, one-hot masks.
 __global__ void router_kernel(const double* energy, const float* timestep, const float* W1, const float* b1,
                               const float* W2, const float* b2, uint8_t* alloc, float* pi_out, FFDims dm) {
+  ff_pdl_wait();
   extern __shared__ float sm[];
   const int d = dm.d, nin = 3 * d + dm.dt, hid = dm.hid;
   float* x = sm;            // [nin]
@@ -246,6 +246,7 @@ __global__ void router_kernel(const double* energy, const float* timestep, const
 
 // Low-band compression: mean over groups of r consecutive low ranks, for Q~, K~ and V~.
 __global__ void pool_low_kernel(const float* spec_low, float* pooled, __nv_bfloat16* pooled_bf, FFDims dm) {
+  ff_pdl_wait();
   // block = (d channels) x (POOL_ROWS pooled tokens)
   const long long g = (long long)blockIdx.x * blockDim.y + threadIdx.y;
   const int th = blockIdx.y;
@@ -291,6 +292,7 @@ __device__ __forceinline__ void attend_range(const KT* __restrict__ Kp, const KT
 
 template <typename ST, int DPL>
 __global__ void __launch_bounds__(ATT_WARPS * 32) attention_simt_kernel(FFBuffers buf, FFDims dm, int band_bits) {
+  ff_pdl_wait();
   const int band = blockIdx.z, bh = blockIdx.y;
   if (!(buf.alloc[bh] & band_bits & (1 << band))) return;
   const long long n = band == 0 ? dm.Nbar : (band == 1 ? dm.Nmid : dm.Nhigh);
@@ -387,6 +389,7 @@ constexpr int SUM_THREADS = 256;
 
 template <typename ST>
 __global__ void __launch_bounds__(SUM_THREADS) summary_partial_kernel(FFBuffers buf, FFDims dm, int split) {
+  ff_pdl_wait();
   __shared__ float red[128];
   const int j = blockIdx.x / split, piece = blockIdx.x % split, band = blockIdx.y, bh = blockIdx.z;
   const int d = dm.d, vecs = d / 8;                // 8-channel vectors per row
@@ -456,6 +459,7 @@ __global__ void __launch_bounds__(SUM_THREADS) summary_partial_kernel(FFBuffers 
 
 template <typename ST>
 __global__ void summary_finalize_kernel(FFBuffers buf, const float* U, FFDims dm, int identity_u) {
+  ff_pdl_wait();
   __shared__ float pooled[128];
   const int j = blockIdx.x, band = blockIdx.y, bh = blockIdx.z;
   const int d = dm.d, c = threadIdx.x;
@@ -488,6 +492,7 @@ static int exc_rounds(long long tokens, int g, int sm_count) {
 template <typename ST, int DPL, typename OT>
 __global__ void __launch_bounds__(EXC_WARPS * 32) exchange_recombine_kernel(FFBuffers buf, FFDims dm, int bh0,
                                                                              OT* grid_out, void* grid_lo, int low_only, int rounds) {
+  ff_pdl_wait();
   extern __shared__ float S[];   // [3][m][d]
   const int gi = blockIdx.y, bh = bh0 + gi;
   const int d = dm.d, m = dm.m;
@@ -603,32 +608,28 @@ cudaError_t ffk_band_energy(ff_plan* p, cudaStream_t st) {
   if (dm.Nlow > nmax) nmax = dm.Nlow;
   dim3 grid((unsigned)((nmax + ENERGY_ROWS - 1) / ENERGY_ROWS), 3, (unsigned)(3 * dm.BH));
   const int threads = (256 / dm.d) * dm.d;
-  if (dm.fp32)
-    band_energy_kernel<float><<<grid, threads, 0, st>>>(p->buf.spec_low, (const float*)p->buf.spec_mid,
-                                                        (const float*)p->buf.spec_high, p->buf.energy, dm);
-  else
-    band_energy_kernel<__nv_bfloat16><<<grid, threads, 0, st>>>(p->buf.spec_low, (const __nv_bfloat16*)p->buf.spec_mid,
-                                                                (const __nv_bfloat16*)p->buf.spec_high, p->buf.energy, dm);
   p->launches += 1;
-  return cudaGetLastError();
+  if (dm.fp32)
+    return ff_launch(band_energy_kernel<float>, grid, dim3(threads), 0, st, p->buf.spec_low, (const float*)p->buf.spec_mid,
+                     (const float*)p->buf.spec_high, p->buf.energy, dm);
+  return ff_launch(band_energy_kernel<__nv_bfloat16>, grid, dim3(threads), 0, st, p->buf.spec_low, (const __nv_bfloat16*)p->buf.spec_mid,
+                   (const __nv_bfloat16*)p->buf.spec_high, p->buf.energy, dm);
 }
 
 cudaError_t ffk_router(ff_plan* p, uint8_t* alloc_out, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const size_t smem = (size_t)(3 * dm.d + dm.dt + dm.hid) * sizeof(float);
-  router_kernel<<<dm.B, 256, smem, st>>>(p->buf.energy, p->buf.timestep, p->W1, p->b1, p->W2, p->b2, alloc_out,
-                                         p->buf.pi, dm);
   p->launches += 1;
-  return cudaGetLastError();
+  return ff_launch(router_kernel, dim3(dm.B), dim3(256), smem, st, p->buf.energy, p->buf.timestep, p->W1, p->b1, p->W2, p->b2,
+                   alloc_out, p->buf.pi, dm);
 }
 
 cudaError_t ffk_pool_low(ff_plan* p, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int rows = dm.d <= 128 ? 512 / dm.d : 1;            // pooled tokens per CTA
   dim3 grid((unsigned)((dm.Nbar + rows - 1) / rows), (unsigned)(3 * dm.BH)), block((unsigned)dm.d, (unsigned)rows);
-  pool_low_kernel<<<grid, block, 0, st>>>(p->buf.spec_low, p->buf.pooled, p->low_tc_ok ? p->buf.pooled_bf : nullptr, dm);
   p->launches += 1;
-  return cudaGetLastError();
+  return ff_launch(pool_low_kernel, grid, block, 0, st, p->buf.spec_low, p->buf.pooled, p->low_tc_ok ? p->buf.pooled_bf : nullptr, dm);
 }
 
 template <typename ST>
@@ -641,14 +642,13 @@ static cudaError_t attention_simt_t(ff_plan* p, int band_bits, cudaStream_t st) 
   if (nmax == 0) return cudaSuccess;                 // (only an empty band was asked for)
   const int zdim = (band_bits & FF_BAND_HIGH) ? 3 : ((band_bits & FF_BAND_MID) ? 2 : 1);
   dim3 grid((unsigned)((nmax + ATT_WARPS - 1) / ATT_WARPS), (unsigned)dm.BH, zdim);
-  switch (dm.d / 32) {
-    case 1: attention_simt_kernel<ST, 1><<<grid, ATT_WARPS * 32, 0, st>>>(p->buf, dm, band_bits); break;
-    case 2: attention_simt_kernel<ST, 2><<<grid, ATT_WARPS * 32, 0, st>>>(p->buf, dm, band_bits); break;
-    case 3: attention_simt_kernel<ST, 3><<<grid, ATT_WARPS * 32, 0, st>>>(p->buf, dm, band_bits); break;
-    default: attention_simt_kernel<ST, 4><<<grid, ATT_WARPS * 32, 0, st>>>(p->buf, dm, band_bits); break;
-  }
   p->launches += 1;
-  return cudaGetLastError();
+  switch (dm.d / 32) {
+    case 1: return ff_launch(attention_simt_kernel<ST, 1>, grid, dim3(ATT_WARPS * 32), 0, st, p->buf, dm, band_bits);
+    case 2: return ff_launch(attention_simt_kernel<ST, 2>, grid, dim3(ATT_WARPS * 32), 0, st, p->buf, dm, band_bits);
+    case 3: return ff_launch(attention_simt_kernel<ST, 3>, grid, dim3(ATT_WARPS * 32), 0, st, p->buf, dm, band_bits);
+    default: return ff_launch(attention_simt_kernel<ST, 4>, grid, dim3(ATT_WARPS * 32), 0, st, p->buf, dm, band_bits);
+  }
 }
 
 cudaError_t ffk_attention_simt(ff_plan* p, int band_bits, cudaStream_t st) {
@@ -665,15 +665,15 @@ cudaError_t ffk_summaries(ff_plan* p, cudaStream_t st) {
   if (split < 1) split = 1;
   if (split > 64) split = 64;
   dim3 pgrid((unsigned)(dm.m * split), 3, (unsigned)dm.BH), fgrid((unsigned)dm.m, 3, (unsigned)dm.BH);
-  if (dm.fp32) {
-    summary_partial_kernel<float><<<pgrid, SUM_THREADS, 0, st>>>(p->buf, dm, split);
-    summary_finalize_kernel<float><<<fgrid, dm.d, 0, st>>>(p->buf, p->U, dm, p->identity_u);
-  } else {
-    summary_partial_kernel<__nv_bfloat16><<<pgrid, SUM_THREADS, 0, st>>>(p->buf, dm, split);
-    summary_finalize_kernel<__nv_bfloat16><<<fgrid, dm.d, 0, st>>>(p->buf, p->U, dm, p->identity_u);
-  }
   p->launches += 2;
-  return cudaGetLastError();
+  if (dm.fp32) {
+    e = ff_launch(summary_partial_kernel<float>, pgrid, dim3(SUM_THREADS), 0, st, p->buf, dm, split);
+    if (e == cudaSuccess) e = ff_launch(summary_finalize_kernel<float>, fgrid, dim3(dm.d), 0, st, p->buf, p->U, dm, p->identity_u);
+  } else {
+    e = ff_launch(summary_partial_kernel<__nv_bfloat16>, pgrid, dim3(SUM_THREADS), 0, st, p->buf, dm, split);
+    if (e == cudaSuccess) e = ff_launch(summary_finalize_kernel<__nv_bfloat16>, fgrid, dim3(dm.d), 0, st, p->buf, p->U, dm, p->identity_u);
+  }
+  return e;
 }
 
 __device__ __forceinline__ float exp2f_fast(float x) {
@@ -691,6 +691,7 @@ __device__ __forceinline__ float exp2f_fast(float x) {
 template <int DPL>
 __global__ void __launch_bounds__(EXC_WARPS * 32) exchange_low_kernel(FFBuffers buf, FFDims dm, int bh0, __nv_bfloat16* grid_hi,
                                                                        uint8_t* grid_lo, int rounds) {
+  ff_pdl_wait();
   extern __shared__ float S[];   // [3][m][d]
   const int gi = blockIdx.y, bh = bh0 + gi;
   const int d = dm.d, m = dm.m;
@@ -774,11 +775,8 @@ static cudaError_t exchange_to_grids(ff_plan* p, long long tokens, int g, size_t
   const int rounds = exc_rounds(tokens, g, p->sm_count);
   const long long per_block = (long long)EXC_WARPS * rounds;
   dim3 grid((unsigned)((tokens + per_block - 1) / per_block), (unsigned)g);
-  cudaError_t e = cudaFuncSetAttribute(exchange_recombine_kernel<__nv_bfloat16, DPL, __nv_bfloat16>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  exchange_recombine_kernel<__nv_bfloat16, DPL, __nv_bfloat16><<<grid, EXC_WARPS * 32, smem, st>>>(p->buf, p->dm, h0, ghi, glo, low_only, rounds);
-  return cudaGetLastError();
+  return ff_launch(exchange_recombine_kernel<__nv_bfloat16, DPL, __nv_bfloat16>, grid, dim3(EXC_WARPS * 32), smem, st, p->buf, p->dm,
+                   h0, ghi, (void*)glo, low_only, rounds);
 }
 
 // Tensor-core inverse: exchange + recombination into a bf16 grid, then the three axis passes.
@@ -798,14 +796,8 @@ static cudaError_t exchange_inverse_tc(ff_plan* p, void* out, cudaStream_t st) {
         const int rounds = exc_rounds(dm.Nlow, g, p->sm_count);
         const long long per_block = (long long)EXC_WARPS * rounds;
         dim3 grid((unsigned)((dm.Nlow + per_block - 1) / per_block), (unsigned)g);
-        if (dm.d == 128) {
-          e = cudaFuncSetAttribute(exchange_low_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-          if (e == cudaSuccess) exchange_low_kernel<4><<<grid, EXC_WARPS * 32, smem, st>>>(p->buf, dm, h0, ghi, (uint8_t*)glo, rounds);
-        } else {
-          e = cudaFuncSetAttribute(exchange_low_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-          if (e == cudaSuccess) exchange_low_kernel<2><<<grid, EXC_WARPS * 32, smem, st>>>(p->buf, dm, h0, ghi, (uint8_t*)glo, rounds);
-        }
-        if (e == cudaSuccess) e = cudaGetLastError();
+        e = ff_launch(dm.d == 128 ? exchange_low_kernel<4> : exchange_low_kernel<2>, grid, dim3(EXC_WARPS * 32), smem, st, p->buf, dm, h0,
+                      ghi, (uint8_t*)glo, rounds);
       }
       if (e == cudaSuccess) e = ffk_exchange_tc(p, h0, g, ghi, glo, st);
     } else {
@@ -840,18 +832,16 @@ static cudaError_t exchange_inverse_t(ff_plan* p, void* out, cudaStream_t st) {
     const int rounds = exc_rounds(dm.N, g, p->sm_count);
     dim3 grid((unsigned)((dm.N + (long long)EXC_WARPS * rounds - 1) / ((long long)EXC_WARPS * rounds)), (unsigned)g);
     cudaError_t e = cudaSuccess;
-#define FF_EXC(DPL)                                                                                                   \
-  e = cudaFuncSetAttribute(exchange_recombine_kernel<ST, DPL, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
-  if (e == cudaSuccess) exchange_recombine_kernel<ST, DPL, float><<<grid, EXC_WARPS * 32, smem, st>>>(p->buf, dm, h0, p->buf.scratchA, (float*)nullptr, 0, rounds);
+#define FF_EXC(DPL)                                                                                                     \
+  ff_launch(exchange_recombine_kernel<ST, DPL, float>, grid, dim3(EXC_WARPS * 32), smem, st, p->buf, dm, h0, p->buf.scratchA, \
+            (void*)nullptr, 0, rounds)
     switch (dm.d / 32) {
-      case 1: FF_EXC(1) break;
-      case 2: FF_EXC(2) break;
-      case 3: FF_EXC(3) break;
-      default: FF_EXC(4) break;
+      case 1: e = FF_EXC(1); break;
+      case 2: e = FF_EXC(2); break;
+      case 3: e = FF_EXC(3); break;
+      default: e = FF_EXC(4); break;
     }
 #undef FF_EXC
-    if (e != cudaSuccess) return e;
-    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     P.group_start = h0;
     // inverse along t, h, w with the transposed matrices
@@ -875,4 +865,20 @@ static cudaError_t exchange_inverse_t(ff_plan* p, void* out, cudaStream_t st) {
 cudaError_t ffk_exchange_inverse(ff_plan* p, void* out, cudaStream_t st) {
   if (p->dct_tc_ok && !(p->attn_impl & 2)) return exchange_inverse_tc(p, out, st);
   return p->dm.fp32 ? exchange_inverse_t<float>(p, out, st) : exchange_inverse_t<__nv_bfloat16>(p, out, st);
+}
+
+cudaError_t ffk_simt_init() {
+  cudaError_t e = cudaSuccess;
+  const int most = 3 * 64 * 128 * (int)sizeof(float);       // summaries of a head; a transform tile and its matrix need no more
+#define FF_SET(k) if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+#define FF_SET_T(T)                                                                                                    \
+  FF_SET((dct_pass_kernel<T, 0>)); FF_SET((dct_pass_kernel<T, 1>)); FF_SET((dct_pass_kernel<T, 2>)); FF_SET((dct_pass_kernel<T, 3>)); \
+  FF_SET((exchange_recombine_kernel<T, 1, float>)); FF_SET((exchange_recombine_kernel<T, 2, float>));                  \
+  FF_SET((exchange_recombine_kernel<T, 3, float>)); FF_SET((exchange_recombine_kernel<T, 4, float>))
+  FF_SET_T(float); FF_SET_T(__nv_bfloat16);
+  FF_SET((exchange_recombine_kernel<__nv_bfloat16, 2, __nv_bfloat16>)); FF_SET((exchange_recombine_kernel<__nv_bfloat16, 4, __nv_bfloat16>));
+  FF_SET(exchange_low_kernel<2>); FF_SET(exchange_low_kernel<4>);
+#undef FF_SET_T
+#undef FF_SET
+  return e;
 }
