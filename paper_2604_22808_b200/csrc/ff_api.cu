@@ -9,6 +9,7 @@
 #include <vector>
 
 #include "ff_internal.h"
+#include "ff_worklist.cuh"
 
 static thread_local char g_err[512] = "";
 
@@ -142,7 +143,7 @@ void ff_compute_layout(const FFDims& dm, bool with_staging, FFLayout* lay) {
       with_staging ? BH * (size_t)dm.N * d * e : 0,
       with_staging ? BH * (size_t)dm.N * d * e : 0,
       with_staging ? BH * (size_t)dm.N * d * e : 0,
-      ffk_tc_work_bytes(),                // 19 worklist
+      FF_WORK_INTS * sizeof(int),         // 19 worklist
       dm.fp32 ? 0 : 3 * BH * (size_t)dm.Nbar * d * 2,   // 20 pooled low band as bf16
   };
   size_t off = 0;
@@ -184,7 +185,7 @@ extern "C" ff_status_t ff_destroy(ff_plan_t* p) {
     for (int i = 0; i <= 2 * FF_COPY_EVENTS; ++i) cudaEventDestroy(p->ev_copy[i]);
     cudaStreamDestroy(p->copy_stream);
   }
-  cudaFree(p->dct2_images); cudaFree(p->pos_table);
+  cudaFree(p->dct2_images); cudaFree(p->pos_table); cudaFree(p->tickets);
   cudaFree(p->W1); cudaFree(p->b1); cudaFree(p->W2); cudaFree(p->b2); cudaFree(p->U);
   delete p;
   return FF_OK;
@@ -265,6 +266,8 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
     else for (size_t l = 0; l < 3; ++l) for (size_t i = 0; i < d; ++i) U[(l * d + i) * d + i] = 1.f;
     s = upload(p, &p->U, U.data(), U.size());
   }
+  if (s == FF_OK && (cudaMalloc((void**)&p->tickets, 256) != cudaSuccess || cudaMemset(p->tickets, 0, 256) != cudaSuccess))
+    s = fail(p, FF_ERR_CUDA, "could not allocate the ticket counters%s");
   if (s == FF_OK && ffk_exchange_tc_supported(p->dm) && !ffk_exchange_tc_build_tables(p))
     s = fail(p, FF_ERR_CUDA, "could not upload the band position tables%s");
   if (s != FF_OK) {
@@ -400,24 +403,23 @@ static cudaError_t mark(ff_plan* p, int boundary, cudaStream_t st) {
   return p->profiling ? cudaEventRecord(p->ev[boundary], st) : cudaSuccess;
 }
 
-// Transform, statistics and router: the part ff_route and an internally routed ff_forward share.
+// Transform, pooling, statistics and router (or the caller's masks): the part ff_route and ff_forward share.
 static ff_status_t transform_and_route(ff_plan* p, const void* Q, const void* K, const void* V, const float* timestep,
-                                       bool route, cudaStream_t st) {
+                                       const uint8_t* alloc_in, cudaStream_t st) {
   FF_CUDA(p, mark(p, 0, st));
+  const bool route = alloc_in == nullptr;
   if (route) {
     if (!p->has_router) return fail(p, FF_ERR_NOT_ROUTED, "the plan was created without router weights%s");
     if (!timestep) return fail(p, FF_ERR_NOT_ROUTED, "neither an allocation nor a timestep was given%s");
-    FF_CUDA(p, cudaMemcpyAsync(p->buf.timestep, timestep, sizeof(float) * p->dm.B, cudaMemcpyHostToDevice, st));
-    FF_CUDA(p, cudaMemsetAsync(p->buf.energy, 0, sizeof(double) * p->dm.B * 3 * p->dm.d, st));
+    if (p->dm.B > FF_TS_INLINE)
+      FF_CUDA(p, cudaMemcpyAsync(p->buf.timestep, timestep, sizeof(float) * p->dm.B, cudaMemcpyHostToDevice, st));
   }
   const bool tc_transform = p->dct_tc_ok && !(p->attn_impl & 2);
-  if (tc_transform) FF_CUDA(p, ffk_forward_transform_tc(p, Q, K, V, route, st));   // band energies come from its epilogue
-  else FF_CUDA(p, ffk_forward_transform(p, Q, K, V, st));
+  // (the transform's first launch clears the energies; the tensor-core passes sum those of the mid and high bands)
+  if (tc_transform) FF_CUDA(p, ffk_forward_transform_tc(p, Q, K, V, route, st));
+  else FF_CUDA(p, ffk_forward_transform(p, Q, K, V, route, st));
   FF_CUDA(p, mark(p, 1, st));
-  if (route) {
-    if (!tc_transform) FF_CUDA(p, ffk_band_energy(p, st));
-    FF_CUDA(p, ffk_router(p, p->buf.alloc, st));
-  }
+  FF_CUDA(p, ffk_band_stats(p, alloc_in, timestep, tc_transform, st));
   FF_CUDA(p, mark(p, 2, st));
   return FF_OK;
 }
@@ -429,7 +431,7 @@ extern "C" ff_status_t ff_route(ff_plan_t* p, const void* Q, const void* K, cons
   if (!timestep) return fail(p, FF_ERR_INVALID_ARG, "timestep is NULL%s");
   cudaStream_t st = (cudaStream_t)stream;
   p->launches = 0;
-  s = transform_and_route(p, Q, K, V, timestep, true, st);
+  s = transform_and_route(p, Q, K, V, timestep, nullptr, st);
   if (s != FF_OK) return s;
   if (alloc_dev) FF_CUDA(p, cudaMemcpyAsync(alloc_dev, p->buf.alloc, p->dm.BH, cudaMemcpyDeviceToDevice, st));
   if (alloc_host) FF_CUDA(p, cudaMemcpyAsync(alloc_host, p->buf.alloc, p->dm.BH, cudaMemcpyDeviceToHost, st));
@@ -447,10 +449,8 @@ extern "C" ff_status_t ff_forward(ff_plan_t* p, const void* Q, const void* K, co
   if (!alloc_dev && !timestep) return fail(p, FF_ERR_NOT_ROUTED, "neither an allocation nor a timestep was given%s");
   cudaStream_t st = (cudaStream_t)stream;
   p->launches = 0;
-  s = transform_and_route(p, Q, K, V, timestep, alloc_dev == nullptr, st);
+  s = transform_and_route(p, Q, K, V, timestep, alloc_dev, st);
   if (s != FF_OK) return s;
-  if (alloc_dev) FF_CUDA(p, cudaMemcpyAsync(p->buf.alloc, alloc_dev, p->dm.BH, cudaMemcpyDeviceToDevice, st));
-  FF_CUDA(p, ffk_pool_low(p, st));
   if (p->tc_ok && !(p->attn_impl & 1)) {
     // the tensor-core launch takes the high band, the strided mid band and a long pooled low band
     const int simt_bands = (p->low_tc_ok ? 0 : FF_BAND_LOW) | (p->dm.pattern == FF_MID_ANCHOR ? FF_BAND_MID : 0);

@@ -4,7 +4,7 @@
 // accumulation, head_dim 128 or 64 (template parameter HD).
 //
 // One persistent launch runs both branches from a worklist of (head, band, pair of query tiles)
-// items that is rebuilt from the head-to-band allocation before every launch.  A CTA owns every
+// items that is rebuilt whenever the head-to-band allocation is (ff_worklist.cuh).  A CTA owns every
 // gridDim-th item.  An item is two neighbouring 128-row query tiles ("streams" A and B) that walk
 // one sequence of 128-key tiles together: both streams of a mid-band item see every key tile of
 // their residue class; in the high band the union of the two windows is 2 + 2R/128 key tiles of
@@ -25,16 +25,17 @@
 
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
+#include "ff_worklist.cuh"
 
 using namespace sm100;
 
 namespace {
 
-constexpr int TILE = 128;            // query rows per stream = key rows per tile
+constexpr int TILE = FF_TILE;        // query rows per stream = key rows per tile
 constexpr int HD_MAX = 128;          // largest head_dim; the shared-memory slots are sized for it
 constexpr int TILE_BYTES = TILE * HD_MAX * 2;
 constexpr int HALF_BYTES = TILE_BYTES / 2;
-constexpr int MAX_UNITS = 1024;
+constexpr int MAX_UNITS = FF_MAX_UNITS;
 constexpr int NSPLIT = 2;                // softmax threads per query row
 constexpr int SCOLS = TILE / NSPLIT;     // key columns per softmax thread
 constexpr int TC_THREADS = 64 + 2 * 128 * NSPLIT;   // TMA warp, MMA warp, 2 streams x 4 NSPLIT softmax warps
@@ -43,7 +44,7 @@ constexpr float LAZY_LOG2 = 8.0f;    // rescale O only when the running max grow
 struct TcParams {
   FFDims dm;
   const uint8_t* alloc;
-  int* work;          // [0] = number of units, [1] = total items, then offsets[MAX_UNITS+1], desc[MAX_UNITS], tiles[MAX_UNITS]
+  int* work;          // the worklist (ff_worklist.cuh)
   __nv_bfloat16* y_mid;
   __nv_bfloat16* y_high;
   float* y_low;       // [BH][Nbar][d] fp32, written when low_on
@@ -52,64 +53,8 @@ struct TcParams {
   int rb_mid;         // rows per TMA box of the mid map = min(b, 128)
 };
 
-// The residue classes of the mid band come in two sizes: the first `rem` = nb mod s classes hold
-// one block more than the others.  Items of a (head, mid band) unit are numbered class by class.
-struct MidShape {
-  int rem;              // classes with the larger block count
-  int nclass;           // residue classes that exist: min(nb, s)
-  int nt_big, nt_small; // query (= key) tiles of a class of either size
-  int pairs_big, pairs_small;
-  int items;            // items of one head's mid band
-};
-
-__host__ __device__ __forceinline__ MidShape mid_shape(const FFDims& dm) {
-  MidShape m;
-  const long long q = dm.s > 0 ? dm.nb / dm.s : 0;
-  m.rem = dm.s > 0 ? (int)(dm.nb % dm.s) : 0;
-  m.nclass = (int)(dm.nb < dm.s ? dm.nb : dm.s);
-  m.nt_big = (int)(((q + 1) * dm.b + TILE - 1) / TILE);
-  m.nt_small = (int)((q * dm.b + TILE - 1) / TILE);
-  m.pairs_big = (m.nt_big + 1) / 2;
-  m.pairs_small = (m.nt_small + 1) / 2;
-  m.items = m.rem * m.pairs_big + (m.nclass - m.rem) * m.pairs_small;
-  return m;
-}
-
-// Worklist: one unit per (head, mid band) and per (head, high band) that the allocation executes;
-// mid units first (their items are the long ones).  An item is a pair of query tiles.
-__global__ void build_worklist_kernel(TcParams P) {
-  ff_pdl_wait();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const FFDims& dm = P.dm;
-  int* offsets = P.work + 2;
-  int* desc = offsets + MAX_UNITS + 1;
-  int* tiles = desc + MAX_UNITS;
-  int nu = 0, total = 0;
-  const MidShape ms = mid_shape(dm);
-  if (P.low_on) {
-    const int nt = (int)((dm.Nbar + TILE - 1) / TILE);
-    for (int bh = 0; bh < dm.BH && nu < MAX_UNITS; ++bh) {
-      if (!(P.alloc[bh] & FF_BAND_LOW)) continue;
-      offsets[nu] = total; desc[nu] = (bh << 12); tiles[nu] = nt;
-      total += (nt + 1) / 2; ++nu;
-    }
-  }
-  // (the anchor pattern of the mid band is not a union of dense classes: those heads run on the generic kernel)
-  for (int bh = 0; bh < dm.BH && nu < MAX_UNITS && dm.pattern == FF_MID_STRIDED; ++bh) {
-    if (!(P.alloc[bh] & FF_BAND_MID)) continue;
-    offsets[nu] = total; desc[nu] = (bh << 12) | (1 << 10); tiles[nu] = 0;
-    total += ms.items; ++nu;
-  }
-  for (int bh = 0; bh < dm.BH && nu < MAX_UNITS; ++bh) {
-    if (!(P.alloc[bh] & FF_BAND_HIGH)) continue;
-    const int nt = (int)((dm.Nhigh + TILE - 1) / TILE);
-    offsets[nu] = total; desc[nu] = (bh << 12) | (2 << 10); tiles[nu] = nt;
-    total += (nt + 1) / 2; ++nu;
-  }
-  offsets[nu] = total;
-  P.work[0] = nu;
-  P.work[1] = total;
-}
+// (ff_high_attention_noalloc only; the plan's worklist is built where its allocation is decided)
+__global__ void build_worklist_kernel(TcParams P) { build_worklist(P.dm, P.alloc, 0, P.work); }
 
 struct Item {
   int band, bh, c;
@@ -678,7 +623,7 @@ attention_tc_qkv_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_
 // Scratch of ff_high_attention_noalloc: the worklist, one band mask per head and a status word.
 // 13,824 bytes in every GPU context that loads this library, held until the process exits.
 constexpr int NOALLOC_MAX_HEADS = MAX_UNITS;
-constexpr size_t NOALLOC_WORK_BYTES = ((2 + 3 * MAX_UNITS + 1) * sizeof(int) + 255) / 256 * 256;
+constexpr size_t NOALLOC_WORK_BYTES = (FF_WORK_INTS * sizeof(int) + 255) / 256 * 256;
 constexpr size_t NOALLOC_BYTES = NOALLOC_WORK_BYTES + NOALLOC_MAX_HEADS + 256;
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
@@ -702,8 +647,6 @@ bool encode_band_map(CUtensorMap* map, void* base, long long rows, int slices, i
 }
 
 }  // namespace
-
-size_t ffk_tc_work_bytes() { return (size_t)(2 + 3 * MAX_UNITS + 1) * sizeof(int); }
 
 // The tensor-core kernel covers bf16, head_dim 128 or 64 and block sizes that tile 128 rows evenly.
 bool ffk_tc_supported(const FFDims& dm) {
@@ -749,13 +692,11 @@ cudaError_t ffk_attention_tc(ff_plan* p, cudaStream_t st) {
   P.y_mid = (__nv_bfloat16*)p->buf.y_mid; P.y_high = (__nv_bfloat16*)p->buf.y_high;
   P.y_low = p->buf.y_low; P.low_on = p->low_tc_ok ? 1 : 0;
   P.status = p->buf.status; P.rb_mid = dm.b < TILE ? dm.b : TILE;
-  cudaError_t e = ff_launch(build_worklist_kernel, dim3(1), dim3(32), 0, st, P);
-  if (e != cudaSuccess) return e;
   const size_t smem = 6 * TILE_BYTES + sizeof(Shared) + 1024;
   const CUtensorMap& mm = *(const CUtensorMap*)p->tmap_mid;
   const CUtensorMap& mh = *(const CUtensorMap*)p->tmap_high;
   const CUtensorMap& ml = p->low_tc_ok ? *(const CUtensorMap*)p->tmap_low : mh;
-  p->launches += 2;
+  p->launches += 1;
 #define FF_ATT(D, LOW) return ff_launch(attention_tc_kernel<D, LOW>, dim3(p->sm_count), dim3(TC_THREADS), smem, st, mm, mh, ml, P)
   if (dm.d == 128) { if (p->low_tc_ok) FF_ATT(128, true); FF_ATT(128, false); }
   if (p->low_tc_ok) FF_ATT(64, true);

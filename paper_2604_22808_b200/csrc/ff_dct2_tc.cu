@@ -63,6 +63,7 @@ struct Dct2Params {
   int nchunk;              // head_dim / 32
   int tpc;                 // tiles per CTA and item
   int cs;                  // CTAs per cluster
+  double* clear;           // band energies to clear for the sums that follow (first launch of a routed forward), or NULL
   int* status;
 };
 
@@ -280,6 +281,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     tmem_wait_st();
   }
   ff_pdl_wait();
+  if (P.clear && blockIdx.x == 0) for (int i = threadIdx.x; i < dm.B * 3 * dm.d; i += D2_THREADS) P.clear[i] = 0.0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -765,7 +767,7 @@ bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat, i
 
 // Forward: Q, K, V of tensor-heads [g0, g0 + g) -> w and second-axis transform -> hi/lo grids.
 cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
-                             cudaStream_t st) {
+                             bool clear_energy, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int G = p->dct_group;
   int axis2, cs;
@@ -780,6 +782,7 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
   P.dm = dm; P.status = p->buf.status;
   P.img1 = p->dct2_images + (size_t)(0 + 2) * per; P.img2 = p->dct2_images + (size_t)(0 + axis2) * per;
   P.axis2 = axis2; P.n1 = dm.W; P.n2 = axis2 == 1 ? dm.H : dm.T; P.n3 = axis2 == 1 ? dm.T : dm.H;
+  P.clear = clear_energy ? p->buf.energy : nullptr;
   P.in_split = 0; P.last = 0; P.group = g; P.group_start = g0; P.nchunk = dm.d / CHK;
   P.cs = cs; P.tpc = dm.W * P.n2 / ROWS / cs;
   return launch(p, mq, mk, mv, oh, ol, P, st);

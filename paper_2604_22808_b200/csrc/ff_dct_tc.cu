@@ -51,7 +51,7 @@
 //               high band in bf16, low band in fp32 straight from the accumulators (the hi/lo
 //               intermediates carry about 16 bits); the router's mid and high band energies are
 //               accumulated here from the stored bf16 coefficients (the low band's, few values per
-//               channel, by low_energy_kernel from the fp32 coefficients)
+//               channel, by the band-statistics kernel from the fp32 coefficients)
 //        LAST   intermediate -> the caller's out tensor
 #include <cuda.h>
 
@@ -102,7 +102,8 @@ struct DctTcParams {
   int reverse;             // walk the tiles from the last to the first (what the previous launch wrote last is still in L2)
   __nv_bfloat16* spec_mid; __nv_bfloat16* spec_high;
   float* spec_low;         // MODE_SPLIT: [3 BH][N_low][d] fp32
-  double* energy;          // [B][3][128]
+  double* energy;          // (SPLIT) [B][3][CH], or NULL
+  double* clear;           // (FIRST) band energies to clear for the sums that follow, or NULL
   int* status;
 };
 
@@ -113,6 +114,7 @@ struct DctShared {
   uint64_t stg_full[2], stg_free[2];       // (ragged tiles) staging area of four epilogue warps: written / read by its store
   uint32_t tmem_base;
   int abort_flag;
+  int e_sample;            // (SPLIT) sample of the CTA's last tile
   // per epilogue warp: 32 rows x 64 bytes of hi and of lo, to turn one-row-per-thread registers
   // into stores where four lanes cover a row's 64 contiguous bytes
   alignas(1024) uint8_t stage[8][2][32 * STG_PITCH];
@@ -212,6 +214,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     tmem_wait_st();
   }
   ff_pdl_wait();
+  if (!LO8 && P.clear && blockIdx.x == 0) for (int i = threadIdx.x; i < dm.B * 3 * CH; i += DCT_TC_THREADS) P.clear[i] = 0.0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -579,12 +582,32 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       }
       if (threadIdx.x == 64) PROF_ADD(5, pe1);
     }
-    if (split) flush_energy();
+    if (split && P.energy) {
+      // the CTA's last sample: the warp's sums into its staging area ([row parity][band][channel of the half]),
+      // added up below with one atomic per channel and CTA (1184 atomics per address took 40 us at the kernel's end)
+      if (lane == 0 && ew == 0) sh.e_sample = e_sample;
+      float* part = (float*)sh.stage[ew] + (lane >> 4) * CH;
+#pragma unroll
+      for (int qi = 0; qi < NQ; ++qi)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int c = qi * 32 + 2 * (lane & 15) + e;
+          part[c] = em[qi][e];
+          part[CH / 2 + c] = ea[qi][e] - em[qi][e];
+        }
+    }
     if (tma_out && lane == 0) bulk_wait0();
   }
 
   tc_fence_before();
   __syncthreads();
+  if (split && P.energy && threadIdx.x < 2 * CH && sh.e_sample >= 0) {
+    const int band = threadIdx.x / CH, half = threadIdx.x % CH / (CH / 2), c = threadIdx.x % (CH / 2);
+    double s = 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s += (double)((const float*)sh.stage[half * 4 + (i >> 1)])[(i & 1) * CH + band * (CH / 2) + c];
+    atomicAdd(P.energy + ((size_t)sh.e_sample * 3 + 1) * CH + threadIdx.x, s);     // mid band, then high band
+  }
   if (sh.abort_flag) {
     if (threadIdx.x == 0) atomicExch(P.status, FF_ERR_TIMEOUT | 0x200);   // low byte: status, next byte: which kernel
     const long long t0 = clock64();
@@ -595,24 +618,6 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     tc_fence_after();
     tmem_dealloc(tm, 512);
   }
-}
-
-// Low-band energy for the router: sum of squares of the fp32 low-band coefficients per channel,
-// over Q~, K~, V~ and the heads of a sample.  grid = (row chunks, 3 BH); thread = channel.
-__global__ void low_energy_kernel(const float* spec_low, double* energy, FFDims dm) {
-  ff_pdl_wait();
-  const int th = blockIdx.y, c = threadIdx.x;
-  const long long per = (dm.Nlow + gridDim.x - 1) / gridDim.x;
-  const long long r0 = (long long)blockIdx.x * per, r1 = r0 + per < dm.Nlow ? r0 + per : dm.Nlow;
-  const float* v = spec_low + ((size_t)th * dm.Nlow) * dm.d + c;
-  float e0 = 0.f, e1 = 0.f;
-  long long r = r0;
-  for (; r + 1 < r1; r += 2) {
-    const float x0 = v[(size_t)r * dm.d], x1 = v[(size_t)(r + 1) * dm.d];
-    e0 = fmaf(x0, x0, e0); e1 = fmaf(x1, x1, e1);
-  }
-  if (r < r1) { const float x0 = v[(size_t)r * dm.d]; e0 = fmaf(x0, x0, e0); }
-  if (r0 < r1) atomicAdd(energy + ((size_t)((th % dm.BH) / dm.heads) * 3) * dm.d + c, (double)(e0 + e1));
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -788,7 +793,7 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
       if (e != cudaSuccess) return e;
     }
     if (fused) {
-      e = ffk_dct2_forward(p, Q, K, V, g0, g, sc.a_hi, sc.a_lo, st);
+      e = ffk_dct2_forward(p, Q, K, V, g0, g, sc.a_hi, sc.a_lo, want_energy && g0 == 0, st);
       if (e != cudaSuccess) return e;
       P.in_split = 1; P.out_lo8 = 0; P.reverse = 1;
       P.mode = MODE_SPLIT; P.axis = last_axis; P.image = matrix_image(p, last_axis, 0);
@@ -796,9 +801,11 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
       if (e != cudaSuccess) return e;
       continue;
     }
+    P.clear = want_energy && g0 == 0 ? p->buf.energy : nullptr;
     P.mode = MODE_FIRST; P.in_split = 0; P.out_lo8 = 1; P.reverse = 0; P.axis = 2; P.image = matrix_image(p, 2, 0);
     e = launch_pass(p, mq, mk, mv, o0h, o0l, P, false, st);
     if (e != cudaSuccess) return e;
+    P.clear = nullptr;
     P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = mid8 ? 1 : 0; P.reverse = 1; P.axis = 1; P.image = matrix_image(p, 1, 0);
     e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, true, st);
     if (e != cudaSuccess) return e;
@@ -806,12 +813,6 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
     P.mode = MODE_SPLIT; P.axis = 0; P.image = matrix_image(p, 0, 0);
     e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, mid8, st);    // (no tensor stores in this mode)
     if (e != cudaSuccess) return e;
-  }
-  if (want_energy) {
-    long long chunks = (dm.Nlow + 511) / 512;             // about 512 rows per block
-    if (chunks > 256) chunks = 256;
-    p->launches += 1;
-    return ff_launch(low_energy_kernel, dim3((unsigned)chunks, (unsigned)total), dim3(dm.d), 0, st, p->buf.spec_low, p->buf.energy, dm);
   }
   return cudaSuccess;
 }

@@ -161,6 +161,7 @@ struct FFLayout {
 };
 
 constexpr int FF_COPY_EVENTS = 64;
+constexpr int FF_TS_INLINE = 32;     // timesteps of up to this many samples travel as kernel arguments
 
 // Tensor maps kept between calls (encoding two dozen of them took longer on the host than the launches they are
 // for).  An entry is known by the tensor's address, its number of slices and the encoder's own code for the rest,
@@ -205,6 +206,7 @@ struct ff_plan {
   bool dct_tc_ok;                              // tensor-core transform usable
   int dct_group;                               // tensor-heads per tensor-core transform launch
   bool xtc_ok;                                 // tensor-core exchange usable
+  unsigned* tickets;                           // "last block" counters, zero between launches (plan-owned)
   int* pos_table;                              // rank -> flat coefficient index of the mid, then the high band (plan-owned)
   alignas(64) unsigned char tmap_x[4][128];    // CUtensorMaps of the exchange kernel (Y / V~ of the mid and high bands)
   uint32_t* dct2_images;                       // 6 x (hi, lo) transform matrices as tensor-memory operand images (plan-owned)
@@ -243,13 +245,11 @@ cudaError_t ffk_exchange_tc_init();
 cudaError_t ffk_dct_tc_init();
 cudaError_t ffk_dct2_init();
 cudaError_t ffk_proj_init();
-cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, const void* V, cudaStream_t st);
-cudaError_t ffk_band_energy(ff_plan* p, cudaStream_t st);
-cudaError_t ffk_router(ff_plan* p, uint8_t* alloc_out, cudaStream_t st);
-cudaError_t ffk_pool_low(ff_plan* p, cudaStream_t st);
+cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy, cudaStream_t st);
+// ---- pooling, band statistics, router, worklist (ff_stats.cu) ---------------------------------------
+cudaError_t ffk_band_stats(ff_plan* p, const uint8_t* alloc_in, const float* timestep_host, bool bands_summed, cudaStream_t st);
 cudaError_t ffk_attention_simt(ff_plan* p, int band_bits, cudaStream_t st);   // band_bits: which bands to run
 // ---- tensor-core attention (ff_attn_tc.cu) -------------------------------------------------------
-size_t ffk_tc_work_bytes();
 bool ffk_tc_supported(const FFDims& dm);
 bool ffk_tc_prepare(ff_plan* p);               // builds the tensor maps over the workspace
 cudaError_t ffk_attention_tc(ff_plan* p, cudaStream_t st);
@@ -268,7 +268,7 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
 bool ffk_dct2_supported(const FFDims& dm, int* axis2, int* cs);
 bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat_host, int n);
 cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
-                             cudaStream_t st);
+                             bool clear_energy, cudaStream_t st);
 cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, int h0, int g, void* out, cudaStream_t st);
 // ---- projections around the path (ff_proj_tc.cu) -------------------------------------------------------
 bool ffk_proj_supported(const FFDims& dm);

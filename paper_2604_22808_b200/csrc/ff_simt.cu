@@ -42,12 +42,15 @@ struct DctPassParams {
   // MODE 2
   FFDims dm;
   float* spec_low; void* spec_mid; void* spec_high;
+  double* clear;        // MODE 0, first launch of a routed call: the band energies, cleared for the sums that follow
 };
 
 template <typename ST, int MODE>
 __global__ void __launch_bounds__(DCT_THREADS) dct_pass_kernel(const DctPassParams P) {
   ff_pdl_wait();
   extern __shared__ float smem[];
+  if (MODE == 0 && P.clear && blockIdx.x == 0 && blockIdx.y == 0)
+    for (int i = threadIdx.x; i < P.dm.B * 3 * P.dm.d; i += DCT_THREADS) P.clear[i] = 0.0;
   const int n = P.n;
   const int npad = (n + 7) & ~7;
   float* matT = smem;                       // [b][npad]: matT[b][a] = Mat[a][b]
@@ -140,125 +143,6 @@ cudaError_t launch_dct_pass(const DctPassParams& P, int group, cudaStream_t st) 
   const int chunks = (P.inner + DCT_IC - 1) / DCT_IC;
   dim3 grid((unsigned)((size_t)P.outer * chunks), (unsigned)group);
   return ff_launch(dct_pass_kernel<ST, MODE>, grid, dim3(DCT_THREADS), smem, st, P);
-}
-
-// ------------------------------------------------------------------------------------------------
-// Router statistics ("Spectral routing network"): sums of squared coefficients per sample, band
-// and channel, pooled over heads, band ranks and the three tensors.
-// ------------------------------------------------------------------------------------------------
-constexpr int ENERGY_ROWS = 256;
-
-template <typename ST>
-__global__ void band_energy_kernel(const float* spec_low, const ST* spec_mid, const ST* spec_high, double* energy,
-                                   FFDims dm) {
-  ff_pdl_wait();
-  const int band = blockIdx.y;
-  const int th = blockIdx.z;                 // tensor * BH + bh
-  const long long nl = band == 0 ? dm.Nlow : (band == 1 ? dm.Nmid : dm.Nhigh);
-  const long long r0 = (long long)blockIdx.x * ENERGY_ROWS;
-  if (r0 >= nl) return;
-  const long long r1 = (r0 + ENERGY_ROWS < nl) ? r0 + ENERGY_ROWS : nl;
-  const int d = dm.d;
-  const int c = threadIdx.x % d;
-  const int lane_rows = blockDim.x / d;
-  const int sub = threadIdx.x / d;
-  float acc = 0.f;
-  if (sub < lane_rows) {
-    for (long long r = r0 + sub; r < r1; r += lane_rows) {
-      float v;
-      if (band == 0) v = spec_low[((size_t)th * dm.Nlow + r) * d + c];
-      else if (band == 1) v = ldf<ST>(spec_mid + ((size_t)th * dm.Nmid + r) * d + c);
-      else v = ldf<ST>(spec_high + ((size_t)th * dm.Nhigh + r) * d + c);
-      acc = fmaf(v, v, acc);
-    }
-    const int bh = th % dm.BH;
-    const int sample = bh / dm.heads;
-    atomicAdd(energy + ((size_t)sample * 3 + band) * d + c, (double)acc);
-  }
-}
-
-// z = W2 relu(W1 [g; e(t)] + b1) + b2, pi = softmax(z), largest-remainder quota, one-hot masks.
-__global__ void router_kernel(const double* energy, const float* timestep, const float* W1, const float* b1,
-                              const float* W2, const float* b2, uint8_t* alloc, float* pi_out, FFDims dm) {
-  ff_pdl_wait();
-  extern __shared__ float sm[];
-  const int d = dm.d, nin = 3 * d + dm.dt, hid = dm.hid;
-  float* x = sm;            // [nin]
-  float* h = sm + nin;      // [hid]
-  __shared__ float z[3];
-  const int sample = blockIdx.x;
-  const long long cnt[3] = {dm.Nlow, dm.Nmid, dm.Nhigh};
-  for (int i = threadIdx.x; i < 3 * d; i += blockDim.x) {
-    const double terms = 3.0 * dm.heads * (double)(cnt[i / d] > 0 ? cnt[i / d] : 1);   // an empty band (two-band layer) has g = 0
-    x[i] = (float)log1p(energy[(size_t)sample * 3 * d + i] / terms);
-  }
-  const int half = dm.dt / 2;
-  const double t = (double)timestep[sample];
-  for (int i = threadIdx.x; i < half; i += blockDim.x) {
-    const double om = exp2(-(double)i / (double)half * 13.287712379549449);     // 10000^(-i/half); log2(10000)
-    double sn, cs;
-    sincos(t * om, &sn, &cs);
-    x[3 * d + i] = (float)sn;
-    x[3 * d + half + i] = (float)cs;
-  }
-  __syncthreads();
-  // hidden layer: one warp per unit, lanes stride over the inputs (coalesced rows of W1)
-  for (int j = threadIdx.x >> 5; j < hid; j += blockDim.x >> 5) {
-    float acc = 0.f;
-    for (int i = threadIdx.x & 31; i < nin; i += 32) acc = fmaf(W1[(size_t)j * nin + i], x[i], acc);
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) h[j] = fmaxf(acc + b1[j], 0.f);
-  }
-  __syncthreads();
-  if (threadIdx.x < 3) {
-    float acc = b2[threadIdx.x];
-    for (int j = 0; j < hid; ++j) acc = fmaf(W2[threadIdx.x * hid + j], h[j], acc);
-    z[threadIdx.x] = acc;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const float mx = fmaxf(z[0], fmaxf(z[1], z[2]));
-    float e[3], pi[3];
-    float sum = 0.f;
-    for (int l = 0; l < 3; ++l) { e[l] = expf(z[l] - mx); sum += e[l]; }
-    int base[3], total = 0;
-    float frac[3];
-    for (int l = 0; l < 3; ++l) {
-      pi[l] = e[l] / sum;
-      pi_out[sample * 3 + l] = pi[l];
-      const float q = pi[l] * (float)dm.heads;
-      base[l] = (int)floorf(q);
-      frac[l] = q - floorf(q);
-      total += base[l];
-    }
-    for (int left = dm.heads - total; left > 0; --left) {   // leftover heads: largest fraction, ties to the lower band
-      int best = 0;
-      for (int l = 1; l < 3; ++l) if (frac[l] > frac[best]) best = l;
-      base[best] += 1;
-      frac[best] = -1.f;
-    }
-    int hix = 0;
-    for (int l = 0; l < 3; ++l)
-      for (int k = 0; k < base[l] && hix < dm.heads; ++k) alloc[sample * dm.heads + hix++] = (uint8_t)(1 << l);
-    for (; hix < dm.heads; ++hix) alloc[sample * dm.heads + hix] = FF_BAND_HIGH;
-  }
-}
-
-// Low-band compression: mean over groups of r consecutive low ranks, for Q~, K~ and V~.
-__global__ void pool_low_kernel(const float* spec_low, float* pooled, __nv_bfloat16* pooled_bf, FFDims dm) {
-  ff_pdl_wait();
-  // block = (d channels) x (POOL_ROWS pooled tokens)
-  const long long g = (long long)blockIdx.x * blockDim.y + threadIdx.y;
-  const int th = blockIdx.y;
-  const int c = threadIdx.x;
-  if (c >= dm.d || g >= dm.Nbar) return;
-  const long long p0 = g * dm.r;
-  const long long p1 = (p0 + dm.r < dm.Nlow) ? p0 + dm.r : dm.Nlow;
-  float acc = 0.f;
-  for (long long p = p0; p < p1; ++p) acc += spec_low[((size_t)th * dm.Nlow + p) * dm.d + c];
-  const float v = acc / (float)(p1 - p0);
-  pooled[((size_t)th * dm.Nbar + g) * dm.d + c] = v;
-  if (pooled_bf) pooled_bf[((size_t)th * dm.Nbar + g) * dm.d + c] = __float2bfloat16_rn(v);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -569,7 +453,7 @@ __global__ void __launch_bounds__(EXC_WARPS * 32) exchange_recombine_kernel(FFBu
 // Launchers
 // ================================================================================================
 template <typename ST>
-static cudaError_t forward_transform_t(ff_plan* p, const void* Q, const void* K, const void* V, cudaStream_t st) {
+static cudaError_t forward_transform_t(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int total = 3 * dm.BH, G = p->lay.group;
   DctPassParams P{};
@@ -581,6 +465,7 @@ static cudaError_t forward_transform_t(ff_plan* p, const void* Q, const void* K,
     // w axis: lines of W elements with stride d
     P.src[0] = Q; P.src[1] = K; P.src[2] = V; P.dst = p->buf.scratchA; P.mat = p->basis[2];
     P.n = dm.W; P.inner = dm.d; P.outer = dm.T * dm.H;
+    P.clear = want_energy && g0 == 0 ? p->buf.energy : nullptr;
     cudaError_t e = launch_dct_pass<ST, 0>(P, g, st);
     if (e != cudaSuccess) return e;
     // h axis
@@ -598,38 +483,9 @@ static cudaError_t forward_transform_t(ff_plan* p, const void* Q, const void* K,
   return cudaSuccess;
 }
 
-cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, const void* V, cudaStream_t st) {
-  return p->dm.fp32 ? forward_transform_t<float>(p, Q, K, V, st) : forward_transform_t<__nv_bfloat16>(p, Q, K, V, st);
-}
-
-cudaError_t ffk_band_energy(ff_plan* p, cudaStream_t st) {
-  const FFDims& dm = p->dm;
-  long long nmax = dm.Nhigh > dm.Nmid ? dm.Nhigh : dm.Nmid;
-  if (dm.Nlow > nmax) nmax = dm.Nlow;
-  dim3 grid((unsigned)((nmax + ENERGY_ROWS - 1) / ENERGY_ROWS), 3, (unsigned)(3 * dm.BH));
-  const int threads = (256 / dm.d) * dm.d;
-  p->launches += 1;
-  if (dm.fp32)
-    return ff_launch(band_energy_kernel<float>, grid, dim3(threads), 0, st, p->buf.spec_low, (const float*)p->buf.spec_mid,
-                     (const float*)p->buf.spec_high, p->buf.energy, dm);
-  return ff_launch(band_energy_kernel<__nv_bfloat16>, grid, dim3(threads), 0, st, p->buf.spec_low, (const __nv_bfloat16*)p->buf.spec_mid,
-                   (const __nv_bfloat16*)p->buf.spec_high, p->buf.energy, dm);
-}
-
-cudaError_t ffk_router(ff_plan* p, uint8_t* alloc_out, cudaStream_t st) {
-  const FFDims& dm = p->dm;
-  const size_t smem = (size_t)(3 * dm.d + dm.dt + dm.hid) * sizeof(float);
-  p->launches += 1;
-  return ff_launch(router_kernel, dim3(dm.B), dim3(256), smem, st, p->buf.energy, p->buf.timestep, p->W1, p->b1, p->W2, p->b2,
-                   alloc_out, p->buf.pi, dm);
-}
-
-cudaError_t ffk_pool_low(ff_plan* p, cudaStream_t st) {
-  const FFDims& dm = p->dm;
-  const int rows = dm.d <= 128 ? 512 / dm.d : 1;            // pooled tokens per CTA
-  dim3 grid((unsigned)((dm.Nbar + rows - 1) / rows), (unsigned)(3 * dm.BH)), block((unsigned)dm.d, (unsigned)rows);
-  p->launches += 1;
-  return ff_launch(pool_low_kernel, grid, block, 0, st, p->buf.spec_low, p->buf.pooled, p->low_tc_ok ? p->buf.pooled_bf : nullptr, dm);
+cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy, cudaStream_t st) {
+  return p->dm.fp32 ? forward_transform_t<float>(p, Q, K, V, want_energy, st)
+                    : forward_transform_t<__nv_bfloat16>(p, Q, K, V, want_energy, st);
 }
 
 template <typename ST>

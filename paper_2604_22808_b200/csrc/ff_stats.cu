@@ -1,0 +1,231 @@
+// From the coefficients to the head-to-band allocation in one launch ("Low band: dense global attention on compressed
+// tokens", "Spectral routing network"): r:1 pooling of the low band, the channel energies the transform's epilogue has
+// not summed, the router MLP with its head quota, and the worklist of the attention launch.
+//
+// The router needs the energies of every block, so the block that finishes last (a ticket counter owned by the plan)
+// runs it.  What these steps cost is latency, not work: as five launches (low-band energy, router, pooling, worklist
+// and the fp32 path's energies) they took 53 us of a 16K-token layer, the router alone 29 us with its second layer
+// read by three threads.
+#include "ff_internal.h"
+#include "ff_worklist.cuh"
+
+namespace {
+
+constexpr int ST_THREADS = 512;
+constexpr int ST_STEPS = 8;              // rows per thread of a mid / high block
+
+struct StatsParams {
+  FFDims dm;
+  const float* spec_low; const void* spec_mid; const void* spec_high;
+  float* pooled; __nv_bfloat16* pooled_bf;
+  double* energy;                        // NULL: no statistics wanted (the caller gave the allocation)
+  const float* W1; const float* b1; const float* W2; const float* b2;
+  const float* timestep;                 // device, [B]; NULL: they are in ts
+  float ts[FF_TS_INLINE];
+  const uint8_t* alloc_in;               // the caller's masks, or NULL to route
+  uint8_t* alloc; float* pi;
+  int* work; int low_on;                 // attention worklist (NULL: the tensor-core kernel does not run)
+  unsigned* ticket;
+  int n_low, n_mid;                      // blocks of the low and of the mid band (the rest: high band); 0: not covered
+  int low_steps;                         // pooled tokens per thread of a low block
+};
+
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+__device__ __forceinline__ float4 load4(const float* p) { return *(const float4*)p; }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 w = *(const uint2*)p;
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                     __uint_as_float(w.y & 0xffff0000u));
+}
+__device__ __forceinline__ void add_squares(float4& e, const float4& x) {
+  e.x = fmaf(x.x, x.x, e.x); e.y = fmaf(x.y, x.y, e.y); e.z = fmaf(x.z, x.z, e.z); e.w = fmaf(x.w, x.w, e.w);
+}
+
+// z = W2 relu(W1 [g; e(t)] + b1) + b2, pi = softmax(z), largest-remainder quota, one-hot masks; a whole block.
+__device__ void route_sample(const StatsParams& P, int sample, float* sm) {
+  const FFDims& dm = P.dm;
+  const int d = dm.d, nin = 3 * d + dm.dt, hid = dm.hid, half = dm.dt / 2;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  float* x = sm;            // [nin]
+  float* h = sm + nin;      // [hid]
+  __shared__ float z[3];
+  __shared__ int first[4];  // first head of each band
+  const double t = (double)(P.timestep ? P.timestep[sample] : P.ts[sample]);
+  for (int i = tid; i < 3 * d + half; i += ST_THREADS) {
+    if (i < 3 * d) {
+      const int band = i / d;
+      const long long cnt = band == 0 ? dm.Nlow : (band == 1 ? dm.Nmid : dm.Nhigh);
+      const double terms = 3.0 * dm.heads * (double)(cnt > 0 ? cnt : 1);          // an empty band (two-band layer) has g = 0
+      x[i] = (float)log1p(__ldcg(P.energy + (size_t)sample * 3 * d + i) / terms);
+    } else {
+      const int k = i - 3 * d;
+      const double om = exp2(-(double)k / (double)half * 13.287712379549449);     // 10000^(-k/half); log2(10000)
+      double sn, cs;
+      sincos(t * om, &sn, &cs);
+      x[3 * d + k] = (float)sn;
+      x[3 * d + half + k] = (float)cs;
+    }
+  }
+  __syncthreads();
+  // hidden layer: four units per warp at a time, lanes stride over the inputs (coalesced rows of W1)
+  for (int j0 = warp * 4; j0 < hid; j0 += (ST_THREADS / 32) * 4) {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 4
+    for (int i = lane; i < nin; i += 32) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc[k] = fmaf(P.W1[(size_t)(j0 + k < hid ? j0 + k : j0) * nin + i], x[i], acc[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = warp_sum(acc[k]);
+    if (lane < 4 && j0 + lane < hid) {
+      const float v = lane == 0 ? acc[0] : (lane == 1 ? acc[1] : (lane == 2 ? acc[2] : acc[3]));
+      h[j0 + lane] = fmaxf(v + P.b1[j0 + lane], 0.f);
+    }
+  }
+  __syncthreads();
+  if (warp < 3) {
+    float acc = 0.f;
+    for (int j = lane; j < hid; j += 32) acc = fmaf(P.W2[warp * hid + j], h[j], acc);
+    acc = warp_sum(acc);
+    if (lane == 0) z[warp] = acc + P.b2[warp];
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const float mx = fmaxf(z[0], fmaxf(z[1], z[2]));
+    float e[3], frac[3], sum = 0.f;
+    int base[3], total = 0;
+    for (int l = 0; l < 3; ++l) { e[l] = expf(z[l] - mx); sum += e[l]; }
+    for (int l = 0; l < 3; ++l) {
+      const float p = e[l] / sum, q = p * (float)dm.heads;
+      P.pi[sample * 3 + l] = p;
+      base[l] = (int)floorf(q);
+      frac[l] = q - floorf(q);
+      total += base[l];
+    }
+    for (int left = dm.heads - total; left > 0; --left) {   // leftover heads: largest fraction, ties to the lower band
+      int best = 0;
+      for (int l = 1; l < 3; ++l) if (frac[l] > frac[best]) best = l;
+      base[best] += 1;
+      frac[best] = -1.f;
+    }
+    first[0] = 0; first[1] = base[0]; first[2] = base[0] + base[1]; first[3] = 0;
+  }
+  __syncthreads();
+  for (int hix = tid; hix < dm.heads; hix += ST_THREADS)
+    P.alloc[sample * dm.heads + hix] = hix < first[1] ? FF_BAND_LOW : (hix < first[2] ? FF_BAND_MID : FF_BAND_HIGH);
+  __syncthreads();                                          // (the next sample reuses the shared memory; the worklist reads the masks)
+}
+
+template <typename ST>
+__global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_constant__ StatsParams P) {
+  extern __shared__ float sm[];
+  __shared__ bool last;
+  ff_pdl_wait();
+  const FFDims& dm = P.dm;
+  const int d = dm.d, vecs = d / 4;                         // four channels per thread
+  const int vec = threadIdx.x % vecs, sub = threadIdx.x / vecs, nsub = ST_THREADS / vecs;
+  const int th = blockIdx.y;
+  float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
+  int band = 0;
+  if ((int)blockIdx.x < P.n_low) {
+    if (sub < nsub)
+      for (int k = 0; k < P.low_steps; ++k) {
+        const long long g = ((long long)blockIdx.x * P.low_steps + k) * nsub + sub;
+        if (g >= dm.Nbar) break;
+        const long long p0 = g * dm.r, p1 = p0 + dm.r < dm.Nlow ? p0 + dm.r : dm.Nlow;
+        const float* src = P.spec_low + ((size_t)th * dm.Nlow + p0) * d + vec * 4;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int n = (int)(p1 - p0);
+#pragma unroll 4
+        for (int i = 0; i < n; ++i) {
+          const float4 x = load4(src + (size_t)i * d);
+          acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
+          add_squares(e, x);
+        }
+        const float fn = (float)n;
+        acc = make_float4(acc.x / fn, acc.y / fn, acc.z / fn, acc.w / fn);
+        const size_t o = ((size_t)th * dm.Nbar + g) * d + vec * 4;
+        *(float4*)(P.pooled + o) = acc;
+        if (P.pooled_bf) {
+          __nv_bfloat162 a = __floats2bfloat162_rn(acc.x, acc.y), b = __floats2bfloat162_rn(acc.z, acc.w);
+          *(uint2*)(P.pooled_bf + o) = make_uint2(*(uint32_t*)&a, *(uint32_t*)&b);
+        }
+      }
+  } else {
+    const int bx = (int)blockIdx.x - P.n_low;
+    band = bx < P.n_mid ? 1 : 2;
+    const long long nl = band == 1 ? dm.Nmid : dm.Nhigh;
+    const long long r0 = (long long)(band == 1 ? bx : bx - P.n_mid) * nsub * ST_STEPS + sub;
+    const ST* src = (const ST*)(band == 1 ? P.spec_mid : P.spec_high) + (size_t)th * nl * d + vec * 4;
+    if (sub < nsub)
+#pragma unroll
+      for (int k = 0; k < ST_STEPS; ++k)
+        if (r0 + k * nsub < nl) add_squares(e, load4(src + (size_t)(r0 + k * nsub) * d));
+  }
+  if (P.energy) {
+    if (sub < nsub) *(float4*)(sm + sub * d + vec * 4) = e;
+    __syncthreads();
+    if ((int)threadIdx.x < d) {
+      double s = 0.0;
+      for (int i = 0; i < nsub; ++i) s += (double)sm[i * d + threadIdx.x];
+      atomicAdd(P.energy + ((size_t)((th % dm.BH) / dm.heads) * 3 + band) * d + threadIdx.x, s);
+    }
+  }
+  if (P.alloc_in) {                                          // nothing to wait for: one block copies the masks and lists the work
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+      for (int i = threadIdx.x; i < dm.BH; i += ST_THREADS) P.alloc[i] = P.alloc_in[i];
+      __syncthreads();
+      if (P.work && threadIdx.x < 32) build_worklist(dm, P.alloc, P.low_on, P.work);
+    }
+    return;
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(P.ticket, 1u) == gridDim.x * gridDim.y - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  if (threadIdx.x == 0) *P.ticket = 0;
+  for (int sample = 0; sample < dm.B; ++sample) route_sample(P, sample, sm);
+  if (P.work && threadIdx.x < 32) build_worklist(dm, P.alloc, P.low_on, P.work);
+}
+
+}  // namespace
+
+// Pooling, statistics, router or copy of the caller's masks, worklist.  `bands_summed`: the transform's epilogue has
+// summed the energies of the mid and high bands already.
+cudaError_t ffk_band_stats(ff_plan* p, const uint8_t* alloc_in, const float* timestep_host, bool bands_summed, cudaStream_t st) {
+  const FFDims& dm = p->dm;
+  StatsParams P{};
+  P.dm = dm;
+  P.spec_low = p->buf.spec_low; P.spec_mid = p->buf.spec_mid; P.spec_high = p->buf.spec_high;
+  P.pooled = p->buf.pooled; P.pooled_bf = p->low_tc_ok ? p->buf.pooled_bf : nullptr;
+  P.alloc_in = alloc_in; P.alloc = p->buf.alloc; P.pi = p->buf.pi;
+  P.ticket = p->tickets;
+  const bool tc = p->tc_ok && !(p->attn_impl & 1);
+  P.work = tc ? p->buf.work : nullptr; P.low_on = p->low_tc_ok ? 1 : 0;
+  if (!alloc_in) {
+    P.energy = p->buf.energy;
+    P.W1 = p->W1; P.b1 = p->b1; P.W2 = p->W2; P.b2 = p->b2;
+    if (dm.B <= FF_TS_INLINE) for (int i = 0; i < dm.B; ++i) P.ts[i] = timestep_host[i];
+    else P.timestep = p->buf.timestep;
+  }
+  const int nsub = ST_THREADS / (dm.d / 4);
+  // a low block takes one round of pooled tokens while the launch stays below eight blocks per SM, then up to 16
+  long long steps = dm.Nbar * 3 * dm.BH / ((long long)nsub * 8 * p->sm_count);
+  P.low_steps = (int)(steps < 1 ? 1 : (steps > 16 ? 16 : steps));
+  P.n_low = (int)((dm.Nbar + (long long)nsub * P.low_steps - 1) / ((long long)nsub * P.low_steps));
+  long long blocks = P.n_low;
+  if (!alloc_in && !bands_summed) {
+    P.n_mid = (int)((dm.Nmid + nsub * ST_STEPS - 1) / (nsub * ST_STEPS));
+    blocks += P.n_mid + (dm.Nhigh + nsub * ST_STEPS - 1) / (nsub * ST_STEPS);
+  }
+  const size_t red = (size_t)nsub * dm.d * sizeof(float), mlp = (size_t)(3 * dm.d + dm.dt + dm.hid) * sizeof(float);
+  p->launches += 1;
+  return ff_launch(dm.fp32 ? band_stats_kernel<float> : band_stats_kernel<__nv_bfloat16>, dim3((unsigned)blocks, (unsigned)(3 * dm.BH)),
+                   dim3(ST_THREADS), red > mlp ? red : mlp, st, P);
+}
