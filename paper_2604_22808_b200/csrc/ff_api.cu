@@ -123,7 +123,7 @@ void ff_compute_layout(const FFDims& dm, bool with_staging, FFLayout* lay) {
   if (Gp > Gt) Gp = Gt;
   lay->tc_group_pipe = (int)Gp;
   const size_t tc_scratch = ffk_dct_tc_supported(dm) ? ffk_dct_tc_scratch_bytes(dm, (int)Gt) : 0;
-  const size_t sizes[21] = {
+  const size_t sizes[23] = {
       3 * BH * (size_t)dm.Nlow * d * 4,   // 0 spec_low
       3 * BH * (size_t)dm.Nmid * d * e,   // 1 spec_mid
       3 * BH * (size_t)dm.Nhigh * d * e,  // 2 spec_high
@@ -145,9 +145,11 @@ void ff_compute_layout(const FFDims& dm, bool with_staging, FFLayout* lay) {
       with_staging ? BH * (size_t)dm.N * d * e : 0,
       FF_WORK_INTS * sizeof(int),         // 19 worklist
       dm.fp32 ? 0 : 3 * BH * (size_t)dm.Nbar * d * 2,   // 20 pooled low band as bf16
+      dm.fp32 ? 0 : BH * ff_zimg_bytes(dm.m),           // 21 operand images of the summaries
+      BH * 3 * (size_t)dm.m * ffk_summary_pieces(dm) * d * 4,   // 22 partial segment sums
   };
   size_t off = 0;
-  for (int i = 0; i < 21; ++i) { lay->off[i] = off; off += align_up(sizes[i], 256); }
+  for (int i = 0; i < 23; ++i) { lay->off[i] = off; off += align_up(sizes[i], 256); }
   lay->total = off;
 }
 
@@ -266,7 +268,8 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
     else for (size_t l = 0; l < 3; ++l) for (size_t i = 0; i < d; ++i) U[(l * d + i) * d + i] = 1.f;
     s = upload(p, &p->U, U.data(), U.size());
   }
-  if (s == FF_OK && (cudaMalloc((void**)&p->tickets, 256) != cudaSuccess || cudaMemset(p->tickets, 0, 256) != cudaSuccess))
+  const size_t ticket_bytes = (64 + (size_t)p->dm.BH * 3 * (p->dm.m > 0 ? p->dm.m : 1)) * sizeof(unsigned);   // band statistics; summaries
+  if (s == FF_OK && (cudaMalloc((void**)&p->tickets, ticket_bytes) != cudaSuccess || cudaMemset(p->tickets, 0, ticket_bytes) != cudaSuccess))
     s = fail(p, FF_ERR_CUDA, "could not allocate the ticket counters%s");
   if (s == FF_OK && ffk_exchange_tc_supported(p->dm) && !ffk_exchange_tc_build_tables(p))
     s = fail(p, FF_ERR_CUDA, "could not upload the band position tables%s");
@@ -316,6 +319,7 @@ extern "C" ff_status_t ff_plan_set_workspace(ff_plan_t* p, void* ptr, size_t byt
   b.stage_v = p->ws_has_staging ? base + o[17] : nullptr; b.stage_out = p->ws_has_staging ? base + o[18] : nullptr;
   b.work = (int*)(base + o[19]);
   b.pooled_bf = p->dm.fp32 ? nullptr : (__nv_bfloat16*)(base + o[20]);
+  b.zimg = (uint8_t*)(base + o[21]); b.sum_part = (float*)(base + o[22]);
   FF_CUDA(p, cudaMemset(b.status, 0, 256));
   p->tc_ok = ffk_tc_supported(p->dm) && ffk_tc_prepare(p);
   p->xtc_ok = p->pos_table && ffk_exchange_tc_supported(p->dm) && ffk_exchange_tc_prepare(p);
@@ -453,11 +457,11 @@ extern "C" ff_status_t ff_forward(ff_plan_t* p, const void* Q, const void* K, co
   if (s != FF_OK) return s;
   if (p->tc_ok && !(p->attn_impl & 1)) {
     // the tensor-core launch takes the high band, the strided mid band and a long pooled low band
-    const int simt_bands = (p->low_tc_ok ? 0 : FF_BAND_LOW) | (p->dm.pattern == FF_MID_ANCHOR ? FF_BAND_MID : 0);
+    const int simt_bands = (p->low_tc_ok || ffk_low_in_summary(p) ? 0 : FF_BAND_LOW) | (p->dm.pattern == FF_MID_ANCHOR ? FF_BAND_MID : 0);
     if (simt_bands) FF_CUDA(p, ffk_attention_simt(p, simt_bands, st));
     FF_CUDA(p, ffk_attention_tc(p, st));
   } else {
-    FF_CUDA(p, ffk_attention_simt(p, FF_BAND_LOW | FF_BAND_MID | FF_BAND_HIGH, st));
+    FF_CUDA(p, ffk_attention_simt(p, (ffk_low_in_summary(p) ? 0 : FF_BAND_LOW) | FF_BAND_MID | FF_BAND_HIGH, st));
   }
   FF_CUDA(p, mark(p, 3, st));
   if (p->dm.m > 0) FF_CUDA(p, ffk_summaries(p, st));

@@ -446,8 +446,8 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       const unsigned nonlow_rows = __ballot_sync(0xffffffffu, band > 0), mid_rows = __ballot_sync(0xffffffffu, band == 1);
       // both 32-channel chunks of the row at once; the accumulator buffer is free as soon as they are read
       uint32_t rr2[NQ][32];
-#pragma unroll
       PROF_T0(pl);
+#pragma unroll
       for (int qi = 0; qi < NQ; ++qi) tmem_ld32(tm + lane_addr + COL_ACC + ab * 128 + (q_lo + qi) * 32, rr2[qi]);
       tmem_wait_ld();
       if (threadIdx.x == 64) { PROF_ADD(8, pl); PROF_ADD(9, pe1); }

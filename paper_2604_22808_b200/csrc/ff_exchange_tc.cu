@@ -37,7 +37,7 @@ constexpr int X_THREADS = 320;           // TMA warp, MMA warp, 4 softmax warps,
 struct XParams {
   FFDims dm;
   const uint8_t* alloc;
-  const float* summary;       // [BH][3][m][d]
+  const uint8_t* zimg;        // [BH] operand images of the heads' summaries (hi, then lo; written by the summary launch)
   const int* pos_mid;         // [N_mid]  flat coefficient index of each band rank
   const int* pos_high;        // [N_high]
   __nv_bfloat16* grid_hi;     // [g][N][d]: upper 16 bits of the value rounded to 24 bits
@@ -65,7 +65,7 @@ __device__ unsigned long long g_x_prof[16];
 constexpr int X_STG_PITCH = 64;         // bytes per staged row piece (32 channels)
 
 struct XShared {
-  uint64_t y_full[2], y_empty[2], z_ready, s_full, p_full, d_full, d_empty;
+  uint64_t y_full[2], y_empty[2], z_ready, z_empty, s_full, p_full, d_full, d_empty;
   uint32_t tmem_base;
   int abort_flag;
   // per softmax warp: 32 rows x 64 bytes of hi and of lo (16-byte chunks XOR-swizzled with row / 2)
@@ -74,6 +74,12 @@ struct XShared {
 };
 
 struct XItem { int bh, band, tile; };
+
+__device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(smem_u32(smem_dst)), "l"((uint64_t)src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
 
 __device__ __forceinline__ float ex2f_approx(float x) {
   float y;
@@ -118,13 +124,15 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&sh.y_full[i], 1); mbar_init(&sh.y_empty[i], P.ybufs == 1 ? 1 : 128); }
-    mbar_init(&sh.z_ready, 128); mbar_init(&sh.s_full, 1); mbar_init(&sh.p_full, 128);
+    mbar_init(&sh.z_ready, 1); mbar_init(&sh.z_empty, 1); mbar_init(&sh.s_full, 1); mbar_init(&sh.p_full, 128);
     mbar_init(&sh.d_full, 1); mbar_init(&sh.d_empty, 128);
     sh.abort_flag = 0;
     fence_mbar_init();
   }
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 256); tmem_relinquish(); }
-  ff_pdl_wait();
+  // The launch before this one is the low band's part of the exchange, which writes other positions of the same
+  // grids: it let this launch start once the summaries were complete, and is waited for at the end only.
+  ff_pdl_trigger();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -136,7 +144,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
   if (warp == 0) {
     if (lane == 0) {
       bool ok = true;
-      int n = 0;
+      int n = 0, prev_bh = -1, zc = 0;
       for (int it = it0; it < it1 && ok; ++it, ++n) {
         const XItem x = x_decode(dm, P.h0, it, tm_tiles, th_tiles);
         const bool exec = P.alloc[x.bh] & (1 << x.band);
@@ -150,6 +158,17 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         mbar_arrive_expect_tx(&sh.y_full[slot], XT * XD * 2);
         tma_load_3d(sY + slot * X_TILE_BYTES, map, &sh.y_full[slot], 0, x.tile * XT, slice);
         if (XD == 128) tma_load_3d(sY + slot * X_TILE_BYTES + X_HALF, map, &sh.y_full[slot], 64, x.tile * XT, slice);
+        if (x.bh != prev_bh) {
+          // the head's summaries, once the MMAs of the previous head have read the old ones (staged and split by 128
+          // threads of every CTA before: 48 rounds of 2-byte stores at the start of every head)
+          prev_bh = x.bh;
+          if (zc > 0) ok = mbar_wait(&sh.z_empty, (zc - 1) & 1, abort_flag);
+          ++zc;
+          if (!ok) break;
+          const uint32_t bytes = 4u * (uint32_t)P.nkeys * 128u;
+          mbar_arrive_expect_tx(&sh.z_ready, bytes);
+          bulk_load(sZhi, P.zimg + (size_t)x.bh * bytes, bytes, &sh.z_ready);
+        }
       }
     }
   } else if (warp == 1) {
@@ -162,7 +181,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
       int n = 0, prev_bh = -1, zc = 0;
       for (int it = it0; it < it1 && ok; ++it, ++n) {
         const XItem x = x_decode(dm, P.h0, it, tm_tiles, th_tiles);
-        if (x.bh != prev_bh) {                            // the softmax warps re-staged Z for this head
+        if (x.bh != prev_bh) {                            // the head's summaries have arrived
           XPROF_T0(x4);
           ok = mbar_wait(&sh.z_ready, zc & 1, abort_flag); ++zc; prev_bh = x.bh;
           XPROF_ADD(4, x4);
@@ -200,6 +219,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
           umma_ts(tmem + 128, tmem + plo, bh_, idesc2, 1u);
         }
         umma_commit(&sh.d_full);
+        if (it + 1 < it1 && x_decode(dm, P.h0, it + 1, tm_tiles, th_tiles).bh != x.bh) umma_commit(&sh.z_empty);
       }
     }
   } else if (warp < 6) {
@@ -224,36 +244,9 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
       keys_mid[c3] = a; keys_high[c3] = b;
     }
     bool ok = true;
-    int n = 0, prev_bh = -1;
+    int n = 0;
     for (int it = it0; it < it1 && ok; ++it, ++n) {
       const XItem x = x_decode(dm, P.h0, it, tm_tiles, th_tiles);
-      if (x.bh != prev_bh) {
-        // Stage the head's 3m summaries as two bf16 images (hi, lo) in the operand layout: row = key,
-        // 64 channels per 128-byte row, 16-byte chunks XOR-swizzled with the row.  Rows >= 3m are zero.
-        // The MMAs of the previous tile, which read the old images, must have completed.
-        prev_bh = x.bh;
-        XPROF_T0(x8);
-        if (n >= 1) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&sh.d_full, (n - 1) & 1, abort_flag));
-          if (!ok) break;
-        }
-        if (tid == 0) XPROF_ADD(8, x8);
-        XPROF_T0(x5);
-        const float* S = P.summary + (size_t)x.bh * 3 * m * XD;
-        for (int idx = tid; idx < nk * XD; idx += 128) {
-          const int j = idx / XD, c = idx % XD;
-          const float v = j < 3 * m ? S[j * XD + c] : 0.f;
-          const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-          const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-          const int half = c >> 6, ck = c & 63;
-          const uint32_t off = half * (nk * 128) + j * 128 + ((((ck >> 3) ^ (j & 7)) << 4) | ((ck & 7) << 1));
-          *(__nv_bfloat16*)(sZhi + off) = hi;
-          *(__nv_bfloat16*)(sZlo + off) = lo;
-        }
-        fence_proxy_async();
-        mbar_arrive(&sh.z_ready);
-        if (tid == 0) XPROF_ADD(5, x5);
-      }
       // ---- softmax over the 2m summaries of the other bands
       XPROF_T0(x6);
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.s_full, n & 1, abort_flag));
@@ -445,6 +438,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
     while (clock64() - t0 < 2000000) { }
     __syncthreads();
   }
+  ff_pdl_join();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, 256);
@@ -528,10 +522,10 @@ bool ffk_exchange_tc_prepare(ff_plan* p) {
 cudaError_t ffk_exchange_tc(ff_plan* p, int h0, int g, void* grid_hi, void* grid_lo, cudaStream_t st) {
   const FFDims& dm = p->dm;
   XParams P;
-  P.dm = dm; P.alloc = p->buf.alloc; P.summary = p->buf.summary;
+  P.dm = dm; P.alloc = p->buf.alloc; P.zimg = p->buf.zimg;
   P.pos_mid = p->pos_table; P.pos_high = p->pos_table + dm.Nmid;
   P.grid_hi = (__nv_bfloat16*)grid_hi; P.grid_lo = (uint8_t*)grid_lo;
-  P.h0 = h0; P.g = g; P.nkeys = (3 * dm.m + 15) / 16 * 16; P.status = p->buf.status;
+  P.h0 = h0; P.g = g; P.nkeys = ff_exchange_keys(dm.m); P.status = p->buf.status;
   P.src[0] = (const __nv_bfloat16*)p->buf.y_mid; P.src[1] = (const __nv_bfloat16*)p->buf.spec_mid;
   P.src[2] = (const __nv_bfloat16*)p->buf.y_high; P.src[3] = (const __nv_bfloat16*)p->buf.spec_high;
   // Two CTAs per SM; the token tile is double-buffered if both still fit in shared memory

@@ -81,6 +81,11 @@ __device__ __forceinline__ void ff_pdl_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The two halves on their own, for a kernel that does not depend on the one before it (but on the ones before that):
+// it starts with the trigger and ends with the wait, so that whoever waits for it has waited for both.
+__device__ __forceinline__ void ff_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void ff_pdl_join() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // (a launch right after an event wait goes without the attribute: ff_launch_after_event)
 template <class... K, class... A>
 inline cudaError_t ff_launch_after_event(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
@@ -138,6 +143,8 @@ struct FFBuffers {
   void* y_mid;       // st [BH][Nmid][d]
   void* y_high;      // st [BH][Nhigh][d]
   float* summary;    // [BH][3][m][d]
+  uint8_t* zimg;     // [BH][hi, lo] summaries of a head as operand images of the tensor-core exchange
+  float* sum_part;   // [BH][3][m][pieces][d] partial segment sums
   double* energy;    // [B][3][d]
   uint8_t* alloc;    // [BH]
   float* pi;         // [B][3]
@@ -274,5 +281,13 @@ cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, i
 bool ffk_proj_supported(const FFDims& dm);
 cudaError_t ffk_project_qkv(ff_plan* p, const void* X, const void* Wqkv, void* Q, void* K, void* V, cudaStream_t st);
 cudaError_t ffk_project_out(ff_plan* p, const void* O, const void* Wo, void* out, cudaStream_t st);
+// ---- summary tokens and the low band's part of the exchange (ff_summary.cu) ----------------------------
+int ffk_summary_pieces(const FFDims& dm);
+bool ffk_low_in_summary(const ff_plan* p);     // the summary launch computes the (short) pooled low band's attention too
 cudaError_t ffk_summaries(ff_plan* p, cudaStream_t st);
+cudaError_t ffk_exchange_low(ff_plan* p, int h0, int g, void* grid_hi, void* grid_lo, cudaStream_t st);
+// Keys of the tensor-core exchange: the 3m summaries of a head, rounded up to a k-step; bytes of one operand image
+// pair (hi, lo; two 64-channel halves of 128-byte rows each).
+FF_HD int ff_exchange_keys(int m) { return (3 * m + 15) / 16 * 16; }
+FF_HD size_t ff_zimg_bytes(int m) { return (size_t)4 * ff_exchange_keys(m) * 128; }
 cudaError_t ffk_exchange_inverse(ff_plan* p, void* out, cudaStream_t st);

@@ -1,22 +1,10 @@
 // Generic FP32-arithmetic kernels of the FreqFormer forward.  They cover every configuration the
 // ABI accepts (any storage type, head_dim, block/stride/radius) and are the path of the fp32
 // workload; the bf16 workloads replace the attention step with the tensor-core kernel.
+#include "ff_bands.cuh"
 #include "ff_internal.h"
 
 namespace {
-
-template <typename T> __device__ __forceinline__ float ldf(const T* p);
-template <> __device__ __forceinline__ float ldf<float>(const float* p) { return *p; }
-template <> __device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16* p) { return __bfloat162float(*p); }
-template <typename T> __device__ __forceinline__ void stf(T* p, float v);
-template <> __device__ __forceinline__ void stf<float>(float* p, float v) { *p = v; }
-template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16* p, float v) { *p = __float2bfloat16_rn(v); }
-
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // ------------------------------------------------------------------------------------------------
 // One axis of the separable transform ("Separable spectral decomposition"):
@@ -233,135 +221,6 @@ __global__ void __launch_bounds__(ATT_WARPS * 32) attention_simt_kernel(FFBuffer
   }
 }
 
-// ------------------------------------------------------------------------------------------------
-// Working output of band `band` of head `bh` ("Cross-band residual exchange"): the operator's
-// output where the head's mask has the band, the value coefficients V~ otherwise.
-// ------------------------------------------------------------------------------------------------
-template <typename ST>
-struct BandView {
-  const float* f32;   // low band rows (pooled output or V~ low)
-  const ST* st;       // mid / high rows
-  long long n;        // working length
-  bool compressed;    // low band executed: row of rank p is p / r
-};
-
-template <typename ST>
-__device__ __forceinline__ BandView<ST> band_view(const FFBuffers& buf, const FFDims& dm, int bh, int band) {
-  BandView<ST> v;
-  const bool exec = buf.alloc[bh] & (1 << band);
-  const int d = dm.d;
-  v.f32 = nullptr; v.st = nullptr; v.compressed = false;
-  if (band == 0) {
-    if (exec) { v.f32 = buf.y_low + (size_t)bh * dm.Nbar * d; v.n = dm.Nbar; v.compressed = true; }
-    else { v.f32 = buf.spec_low + ((size_t)2 * dm.BH + bh) * dm.Nlow * d; v.n = dm.Nlow; }
-  } else if (band == 1) {
-    v.n = dm.Nmid;
-    v.st = exec ? (const ST*)buf.y_mid + (size_t)bh * dm.Nmid * d
-                : (const ST*)buf.spec_mid + ((size_t)2 * dm.BH + bh) * dm.Nmid * d;
-  } else {
-    v.n = dm.Nhigh;
-    v.st = exec ? (const ST*)buf.y_high + (size_t)bh * dm.Nhigh * d
-                : (const ST*)buf.spec_high + ((size_t)2 * dm.BH + bh) * dm.Nhigh * d;
-  }
-  return v;
-}
-
-// Summary tokens S = U_l Pool(Y^(l)): segment j covers [floor(j n/m), max(a+1, floor((j+1) n/m))).
-// Two steps: segment sums (each segment split over several CTAs, 16-byte loads, partial sums
-// added atomically into the summary buffer), then mean and projection in place.
-constexpr int SUM_THREADS = 256;
-
-template <typename ST>
-__global__ void __launch_bounds__(SUM_THREADS) summary_partial_kernel(FFBuffers buf, FFDims dm, int split) {
-  ff_pdl_wait();
-  __shared__ float red[128];
-  const int j = blockIdx.x / split, piece = blockIdx.x % split, band = blockIdx.y, bh = blockIdx.z;
-  const int d = dm.d, vecs = d / 8;                // 8-channel vectors per row
-  const BandView<ST> v = band_view<ST>(buf, dm, bh, band);
-  if (v.n == 0) return;                            // empty band (two-band layer): no summary tokens
-  const long long a = ((long long)j * v.n) / dm.m;
-  long long e = ((long long)(j + 1) * v.n) / dm.m;
-  if (e < a + 1) e = a + 1;
-  const long long chunk = (e - a + split - 1) / split;
-  const long long r0 = a + piece * chunk;
-  const long long r1 = r0 + chunk < e ? r0 + chunk : e;
-  const int vec = threadIdx.x % vecs, rsub = threadIdx.x / vecs, nrs = SUM_THREADS / vecs;
-  float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  if (rsub < nrs) {
-    long long p = r0 + rsub;
-    if (!v.f32 && sizeof(ST) == 2) {
-      // bf16 rows, eight rows in flight per thread
-      const __nv_bfloat16* base = (const __nv_bfloat16*)v.st + vec * 8;
-      for (; p + 7 * nrs < r1; p += 8 * nrs) {
-        uint4 x[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) x[u] = __ldcs((const uint4*)(base + (size_t)(p + u * nrs) * d));
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const uint32_t w[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            acc[2 * i] += __uint_as_float(w[i] << 16);
-            acc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
-          }
-        }
-      }
-    }
-    for (; p < r1; p += nrs) {
-      if (v.f32) {
-        const float4 x0 = *(const float4*)(v.f32 + (size_t)p * d + vec * 8);
-        const float4 x1 = *(const float4*)(v.f32 + (size_t)p * d + vec * 8 + 4);
-        acc[0] += x0.x; acc[1] += x0.y; acc[2] += x0.z; acc[3] += x0.w;
-        acc[4] += x1.x; acc[5] += x1.y; acc[6] += x1.z; acc[7] += x1.w;
-      } else if (sizeof(ST) == 4) {
-        const float4 x0 = *(const float4*)((const float*)v.st + (size_t)p * d + vec * 8);
-        const float4 x1 = *(const float4*)((const float*)v.st + (size_t)p * d + vec * 8 + 4);
-        acc[0] += x0.x; acc[1] += x0.y; acc[2] += x0.z; acc[3] += x0.w;
-        acc[4] += x1.x; acc[5] += x1.y; acc[6] += x1.z; acc[7] += x1.w;
-      } else {
-        const uint4 x = *(const uint4*)((const __nv_bfloat16*)v.st + (size_t)p * d + vec * 8);
-        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          acc[2 * i] += __uint_as_float(w[i] << 16);
-          acc[2 * i + 1] += __uint_as_float(w[i] & 0xffff0000u);
-        }
-      }
-    }
-  }
-  // combine the row groups: channel sums through shared-memory atomics, then one global atomic per channel
-  if (threadIdx.x < 128) red[threadIdx.x] = 0.f;
-  __syncthreads();
-  if (rsub < nrs) {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) atomicAdd(&red[vec * 8 + i], acc[i]);
-  }
-  __syncthreads();
-  if (threadIdx.x < d && r0 < r1)
-    atomicAdd(buf.summary + (((size_t)bh * 3 + band) * dm.m + j) * d + threadIdx.x, red[threadIdx.x]);
-}
-
-template <typename ST>
-__global__ void summary_finalize_kernel(FFBuffers buf, const float* U, FFDims dm, int identity_u) {
-  ff_pdl_wait();
-  __shared__ float pooled[128];
-  const int j = blockIdx.x, band = blockIdx.y, bh = blockIdx.z;
-  const int d = dm.d, c = threadIdx.x;
-  const BandView<ST> v = band_view<ST>(buf, dm, bh, band);
-  if (v.n == 0) return;                            // (its slots stay zero and are never attended)
-  const long long a = ((long long)j * v.n) / dm.m;
-  long long e = ((long long)(j + 1) * v.n) / dm.m;
-  if (e < a + 1) e = a + 1;
-  float* S = buf.summary + (((size_t)bh * 3 + band) * dm.m + j) * d;
-  pooled[c] = S[c] / (float)(e - a);
-  if (identity_u) { S[c] = pooled[c]; return; }
-  __syncthreads();
-  const float* Ul = U + ((size_t)band * d + c) * d;
-  float s = 0.f;
-  for (int i = 0; i < d; ++i) s = fmaf(Ul[i], pooled[i], s);
-  S[c] = s;
-}
-
 // Exchange + recombination ("Cross-band residual exchange", "Reconstruction"): for every
 // coefficient of the grid, fetch its band token, add softmax(y Z^T / sqrt(d)) Z over the 2m summary
 // tokens of the other two bands, and write the row at its coefficient position (fp32 grid).
@@ -511,119 +370,6 @@ cudaError_t ffk_attention_simt(ff_plan* p, int band_bits, cudaStream_t st) {
   return p->dm.fp32 ? attention_simt_t<float>(p, band_bits, st) : attention_simt_t<__nv_bfloat16>(p, band_bits, st);
 }
 
-cudaError_t ffk_summaries(ff_plan* p, cudaStream_t st) {
-  const FFDims& dm = p->dm;
-  cudaError_t e = cudaMemsetAsync(p->buf.summary, 0, (size_t)dm.BH * 3 * dm.m * dm.d * sizeof(float), st);
-  if (e != cudaSuccess) return e;
-  // split every segment so that each CTA reads about 1024 rows of the longest band
-  long long longest = dm.Nhigh > dm.Nmid ? dm.Nhigh : dm.Nmid;
-  int split = (int)((longest / dm.m + 1023) / 1024);
-  if (split < 1) split = 1;
-  if (split > 64) split = 64;
-  dim3 pgrid((unsigned)(dm.m * split), 3, (unsigned)dm.BH), fgrid((unsigned)dm.m, 3, (unsigned)dm.BH);
-  p->launches += 2;
-  if (dm.fp32) {
-    e = ff_launch(summary_partial_kernel<float>, pgrid, dim3(SUM_THREADS), 0, st, p->buf, dm, split);
-    if (e == cudaSuccess) e = ff_launch(summary_finalize_kernel<float>, fgrid, dim3(dm.d), 0, st, p->buf, p->U, dm, p->identity_u);
-  } else {
-    e = ff_launch(summary_partial_kernel<__nv_bfloat16>, pgrid, dim3(SUM_THREADS), 0, st, p->buf, dm, split);
-    if (e == cudaSuccess) e = ff_launch(summary_finalize_kernel<__nv_bfloat16>, fgrid, dim3(dm.d), 0, st, p->buf, p->U, dm, p->identity_u);
-  }
-  return e;
-}
-
-__device__ __forceinline__ float exp2f_fast(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// Low band of the tensor-core inverse ("Cross-band residual exchange", "Reconstruction"): exchange + recombination
-// of the low band's coefficients into the three-byte grids.  One warp per SOURCE row: a head that executes the
-// low band has one pooled output row for every r consecutive coefficient ranks, so its update is computed once
-// and written r times; other heads carry V~ low, one row per rank.  The scores of eight summaries at a time
-// are reduced side by side (independent shuffle trees) and merged into the running softmax as a group
-// (exponentials by ex2.approx on scores scaled to log2 units, like the tensor-core kernel's).  DPL = d / 32.
-template <int DPL>
-__global__ void __launch_bounds__(EXC_WARPS * 32) exchange_low_kernel(FFBuffers buf, FFDims dm, int bh0, __nv_bfloat16* grid_hi,
-                                                                       uint8_t* grid_lo, int rounds) {
-  ff_pdl_wait();
-  extern __shared__ float S[];   // [3][m][d]
-  const int gi = blockIdx.y, bh = bh0 + gi;
-  const int d = dm.d, m = dm.m;
-  for (int i = threadIdx.x; i < 3 * m * d; i += blockDim.x) S[i] = buf.summary[(size_t)bh * 3 * m * d + i];
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const bool exec = buf.alloc[bh] & FF_BAND_LOW;
-  const float* src = exec ? buf.y_low + (size_t)bh * dm.Nbar * d : buf.spec_low + ((size_t)2 * dm.BH + bh) * dm.Nlow * d;
-  const long long rows = exec ? dm.Nbar : dm.Nlow;
-  const int rep = exec ? dm.r : 1;
-  // the summaries of the other bands: the mid band's (none if it is empty), then the high band's
-  const int k_first = dm.Nmid == 0 ? 2 * m : m, nkeys = 3 * m - k_first;
-  const float scale = rsqrtf((float)d) * 1.4426950408889634f;      // scores in units of log2: exponentials by ex2
-  for (int round = 0; round < rounds; ++round) {
-    const long long row = ((long long)blockIdx.x * rounds + round) * EXC_WARPS + (threadIdx.x >> 5);
-    if (row >= rows) return;
-    float y[DPL], acc[DPL];
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) { y[j] = src[(size_t)row * d + lane + 32 * j]; acc[j] = 0.f; }
-    if (nkeys > 0) {
-      float mx = -INFINITY, den = 0.f;
-      for (int k0 = 0; k0 < nkeys; k0 += 8) {
-        float sc[8];
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const float* z = S + (size_t)(k_first + (k0 + kk < nkeys ? k0 + kk : 0)) * d;
-          float part = 0.f;
-#pragma unroll
-          for (int j = 0; j < DPL; ++j) part = fmaf(y[j], z[lane + 32 * j], part);
-          sc[kk] = part;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-          for (int kk = 0; kk < 8; ++kk) sc[kk] += __shfl_xor_sync(0xffffffffu, sc[kk], o);
-        float nm = mx;
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          sc[kk] = k0 + kk < nkeys ? sc[kk] * scale : -INFINITY;
-          nm = fmaxf(nm, sc[kk]);
-        }
-        const float corr = exp2f_fast(mx - nm);
-        den *= corr;
-#pragma unroll
-        for (int j = 0; j < DPL; ++j) acc[j] *= corr;
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const float pr = exp2f_fast(sc[kk] - nm);         // (0 for the keys past the end)
-          const float* z = S + (size_t)(k_first + (k0 + kk < nkeys ? k0 + kk : 0)) * d;
-          den += pr;
-#pragma unroll
-          for (int j = 0; j < DPL; ++j) acc[j] = fmaf(pr, z[lane + 32 * j], acc[j]);
-        }
-        mx = nm;
-      }
-#pragma unroll
-      for (int j = 0; j < DPL; ++j) acc[j] /= den;
-    }
-    // the value in three bytes (rounded to 24 bits: upper 16 bits and the next 8), at every rank the row stands for
-    uint32_t u[DPL];
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) u[j] = __float_as_uint(y[j] + acc[j]) + 0x80u;
-    for (int i = 0; i < rep; ++i) {
-      const long long p = row * rep + i;
-      if (p >= dm.Nlow) break;
-      const int kw = (int)(p % dm.L[2]), kh = (int)((p / dm.L[2]) % dm.L[1]), kt = (int)(p / ((long long)dm.L[2] * dm.L[1]));
-      const size_t o = ((size_t)gi * dm.N + ((size_t)kt * dm.H + kh) * dm.W + kw) * d;
-#pragma unroll
-      for (int j = 0; j < DPL; ++j) {
-        ((uint16_t*)grid_hi)[o + lane + 32 * j] = (uint16_t)(u[j] >> 16);
-        grid_lo[o + lane + 32 * j] = (uint8_t)(u[j] >> 8);
-      }
-    }
-  }
-}
-
 // Generic exchange + recombination into the hi/lo bf16 grids of the tensor-core inverse; DPL = d / 32.
 template <int DPL>
 static cudaError_t exchange_to_grids(ff_plan* p, long long tokens, int g, size_t smem, int h0, __nv_bfloat16* ghi,
@@ -631,6 +377,7 @@ static cudaError_t exchange_to_grids(ff_plan* p, long long tokens, int g, size_t
   const int rounds = exc_rounds(tokens, g, p->sm_count);
   const long long per_block = (long long)EXC_WARPS * rounds;
   dim3 grid((unsigned)((tokens + per_block - 1) / per_block), (unsigned)g);
+  p->launches += 1;
   return ff_launch(exchange_recombine_kernel<__nv_bfloat16, DPL, __nv_bfloat16>, grid, dim3(EXC_WARPS * 32), smem, st, p->buf, p->dm,
                    h0, ghi, (void*)glo, low_only, rounds);
 }
@@ -648,19 +395,12 @@ static cudaError_t exchange_inverse_tc(ff_plan* p, void* out, cudaStream_t st) {
     __nv_bfloat16* glo = (__nv_bfloat16*)((char*)p->buf.scratchA + grid_bytes);
     if (p->xtc_ok) {
       // mid and high bands on the tensor cores, the fp32 low band with its own kernel (one warp per source row)
-      {
-        const int rounds = exc_rounds(dm.Nlow, g, p->sm_count);
-        const long long per_block = (long long)EXC_WARPS * rounds;
-        dim3 grid((unsigned)((dm.Nlow + per_block - 1) / per_block), (unsigned)g);
-        e = ff_launch(dm.d == 128 ? exchange_low_kernel<4> : exchange_low_kernel<2>, grid, dim3(EXC_WARPS * 32), smem, st, p->buf, dm, h0,
-                      ghi, (uint8_t*)glo, rounds);
-      }
+      e = ffk_exchange_low(p, h0, g, ghi, glo, st);
       if (e == cudaSuccess) e = ffk_exchange_tc(p, h0, g, ghi, glo, st);
     } else {
       e = dm.d == 128 ? exchange_to_grids<4>(p, dm.N, g, smem, h0, ghi, glo, 0, st) : exchange_to_grids<2>(p, dm.N, g, smem, h0, ghi, glo, 0, st);
     }
     if (e != cudaSuccess) return e;
-    p->launches += 1;
     e = ffk_inverse_transform_tc(p, h0, g, out, st);
     if (e != cudaSuccess) return e;
     if (p->pipe_out) {                             // host-buffer entry point: hand this group of heads to the copy stream
@@ -733,7 +473,6 @@ cudaError_t ffk_simt_init() {
   FF_SET((exchange_recombine_kernel<T, 3, float>)); FF_SET((exchange_recombine_kernel<T, 4, float>))
   FF_SET_T(float); FF_SET_T(__nv_bfloat16);
   FF_SET((exchange_recombine_kernel<__nv_bfloat16, 2, __nv_bfloat16>)); FF_SET((exchange_recombine_kernel<__nv_bfloat16, 4, __nv_bfloat16>));
-  FF_SET(exchange_low_kernel<2>); FF_SET(exchange_low_kernel<4>);
 #undef FF_SET_T
 #undef FF_SET
   return e;
