@@ -1,10 +1,50 @@
 // Generic FP32-arithmetic kernels of the FreqFormer forward.  They cover every configuration the
 // ABI accepts (any storage type, head_dim, block/stride/radius) and are the path of the fp32
-// workload; the bf16 workloads replace the attention step with the tensor-core kernel.
+// workloads; the bf16 workloads replace them with the tensor-core kernels where those apply.
 #include "ff_bands.cuh"
 #include "ff_internal.h"
+#include "ff_worklist.cuh"
 
 namespace {
+
+__device__ __forceinline__ float4 ld4(const float* p) { return *(const float4*)p; }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
+  const uint2 w = *(const uint2*)p;
+  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                     __uint_as_float(w.y & 0xffff0000u));
+}
+__device__ __forceinline__ void st4(float* p, const float4& v) { *(float4*)p = v; }
+__device__ __forceinline__ void st4(__nv_bfloat16* p, const float4& v) {
+  const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+  *(uint2*)p = make_uint2(*(const uint32_t*)&a, *(const uint32_t*)&b);
+}
+__device__ __forceinline__ void fma4(float4& acc, float m, const float4& x) {
+  acc.x = fmaf(m, x.x, acc.x); acc.y = fmaf(m, x.y, acc.y); acc.z = fmaf(m, x.z, acc.z); acc.w = fmaf(m, x.w, acc.w);
+}
+
+// ff_band_rank_of in 32 bits (axis lengths are at most 128).
+__device__ __forceinline__ int band_rank(const FFDims& dm, int kt, int kh, int kw, int& rank) {
+  auto below = [&](const int (&A)[3]) {
+    if (kt >= A[0]) return A[0] * A[1] * A[2];
+    return kt * A[1] * A[2] + min(kh, A[1]) * A[2] + (kh < A[1] ? min(kw, A[2]) : 0);
+  };
+  const int cl = below(dm.L), cm = below(dm.M);
+  if (kt < dm.L[0] && kh < dm.L[1] && kw < dm.L[2]) { rank = cl; return 0; }
+  if (kt < dm.M[0] && kh < dm.M[1] && kw < dm.M[2]) { rank = cm - cl; return 1; }
+  rank = (kt * dm.H + kh) * dm.W + kw - cm;
+  return 2;
+}
+
+// Where coefficient (kt, kh, kw) of tensor-head th goes: four channels from `ch` on.
+template <typename ST>
+__device__ __forceinline__ void store_coefficient(const FFDims& dm, float* spec_low, void* spec_mid, void* spec_high, int th, int kt,
+                                                  int kh, int kw, int ch, const float4& v) {
+  int rank;
+  const int band = band_rank(dm, kt, kh, kw, rank);
+  if (band == 0) st4(spec_low + ((size_t)th * dm.Nlow + rank) * dm.d + ch, v);
+  else if (band == 1) st4((ST*)spec_mid + ((size_t)th * dm.Nmid + rank) * dm.d + ch, v);
+  else st4((ST*)spec_high + ((size_t)th * dm.Nhigh + rank) * dm.d + ch, v);
+}
 
 // ------------------------------------------------------------------------------------------------
 // One axis of the separable transform ("Separable spectral decomposition"):
@@ -12,298 +52,491 @@ namespace {
 // with the tensor-head as the slowest index.  Mat is C (forward) or C^T (inverse).
 // MODE 0: `in` is the caller's Q/K/V (storage type), `out` an fp32 scratch grid.
 // MODE 1: fp32 scratch -> fp32 scratch.
-// MODE 2: fp32 scratch -> band-major coefficient buffers (forward, last axis = t): the rank of
-//         every coefficient is evaluated in registers from the nested-box closed form.
+// MODE 2: fp32 scratch -> band-major coefficient buffers (forward, last axis = t).
 // MODE 3: fp32 scratch -> the caller's `out` tensor (storage type).
+//
+// A warp takes 128 neighbouring columns (o, c) and eight outputs along the axis: 32 accumulators per thread against
+// one 16-byte load of the line and two broadcast reads of the matrix in shared memory per step.  The warps of a block
+// that share a column tile find its lines in L1, so no tile is staged, and any n keeps all lanes busy (a block used to
+// own 64 columns, of which a 9-long axis kept 32 threads busy: 134 us for the t pass of 12 x 9 x 30 x 40 x 64 floats).
 // ------------------------------------------------------------------------------------------------
-constexpr int DCT_IC = 64;       // columns per CTA tile
 constexpr int DCT_THREADS = 256;
+constexpr int DCT_COLS = 128;    // columns of a warp's item
 
 struct DctPassParams {
   const void* src[3];   // MODE 0: Q, K, V; otherwise src[0] = scratch
   void* dst;            // MODE 0/1: scratch; MODE 3: out tensor
-  const float* mat;     // [n][n]
+  const float* mat_t;   // [b][a] = Mat[a][b]
   int n, inner, outer;
   int group_start;      // first tensor-head index of this launch
   int BH;
+  int tiles;            // column tiles of a tensor-head
   long long N_d;        // elements per tensor-head
-  // MODE 2
   FFDims dm;
+  // MODE 2
   float* spec_low; void* spec_mid; void* spec_high;
   double* clear;        // MODE 0, first launch of a routed call: the band energies, cleared for the sums that follow
 };
 
+// The matrix, rows padded to a multiple of eight outputs.
+__device__ __forceinline__ void stage_matrix(float* mt, const float* mat_t, int n, int npad) {
+  for (int idx = threadIdx.x; idx < n * npad; idx += blockDim.x) {
+    const int b = idx / npad, a = idx - b * npad;
+    mt[idx] = a < n ? mat_t[b * n + a] : 0.f;
+  }
+}
+
 template <typename ST, int MODE>
-__global__ void __launch_bounds__(DCT_THREADS) dct_pass_kernel(const DctPassParams P) {
+__global__ void __launch_bounds__(DCT_THREADS) dct_pass_kernel(const __grid_constant__ DctPassParams P) {
+  extern __shared__ float mt[];
+  const int n = P.n, npad = (n + 7) & ~7, groups = npad / 8;
+  stage_matrix(mt, P.mat_t, n, npad);
   ff_pdl_wait();
-  extern __shared__ float smem[];
   if (MODE == 0 && P.clear && blockIdx.x == 0 && blockIdx.y == 0)
     for (int i = threadIdx.x; i < P.dm.B * 3 * P.dm.d; i += DCT_THREADS) P.clear[i] = 0.0;
-  const int n = P.n;
-  const int npad = (n + 7) & ~7;
-  float* matT = smem;                       // [b][npad]: matT[b][a] = Mat[a][b]
-  float* tile = smem + (size_t)n * npad;    // [b][DCT_IC]
-  const int chunks = (P.inner + DCT_IC - 1) / DCT_IC;
-  const int o = blockIdx.x / chunks;
-  const int c0 = (blockIdx.x % chunks) * DCT_IC;
+  __syncthreads();
   const int gi = blockIdx.y;                // tensor-head inside the group
   const int th = P.group_start + gi;        // global tensor-head index: tensor * BH + bh
-  const int tid = threadIdx.x;
-
-  for (int idx = tid; idx < n * npad; idx += DCT_THREADS) {
-    const int b = idx / npad, a = idx % npad;
-    matT[idx] = (a < n) ? P.mat[(size_t)a * n + b] : 0.f;
-  }
-  const size_t line0 = ((size_t)o * n) * P.inner + c0;
-  if (MODE == 0) {
-    const ST* src = (const ST*)P.src[th / P.BH] + (size_t)(th % P.BH) * P.N_d + line0;
-    for (int idx = tid; idx < n * DCT_IC; idx += DCT_THREADS) {
-      const int b = idx / DCT_IC, c = idx % DCT_IC;
-      tile[idx] = (c0 + c < P.inner) ? ldf<ST>(src + (size_t)b * P.inner + c) : 0.f;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned inner = (unsigned)P.inner, cols = inner * (unsigned)P.outer;
+  const unsigned items = (unsigned)P.tiles * (unsigned)groups;
+  for (unsigned item = blockIdx.x * (DCT_THREADS / 32) + warp; item < items; item += gridDim.x * (DCT_THREADS / 32)) {
+    const unsigned tile = item / (unsigned)groups;
+    const int g = (int)(item - tile * (unsigned)groups);
+    const unsigned col = tile * DCT_COLS + lane * 4;
+    if (col >= cols) continue;
+    const unsigned o = col / inner, c = col - o * inner;
+    const size_t line = (size_t)o * n * inner + c;
+    float4 acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto sum_line = [&](auto* src) {
+      const float* m = mt + g * 8;
+#pragma unroll 4
+      for (int b = 0; b < n; ++b) {
+        const float4 x = ld4(src + (size_t)b * inner);
+        const float4 m0 = *(const float4*)(m + b * npad), m1 = *(const float4*)(m + b * npad + 4);
+        fma4(acc[0], m0.x, x); fma4(acc[1], m0.y, x); fma4(acc[2], m0.z, x); fma4(acc[3], m0.w, x);
+        fma4(acc[4], m1.x, x); fma4(acc[5], m1.y, x); fma4(acc[6], m1.z, x); fma4(acc[7], m1.w, x);
+      }
+    };
+    if (MODE == 0) sum_line((const ST*)P.src[th / P.BH] + (size_t)(th % P.BH) * P.N_d + line);
+    else sum_line((const float*)P.src[0] + (size_t)gi * P.N_d + line);
+    int ch = 0, kw = 0, kh = 0;
+    if (MODE == 2) {                        // a = k_t, column = (k_h, k_w, channel)
+      const unsigned p = c / (unsigned)P.dm.d;
+      ch = (int)(c - p * (unsigned)P.dm.d);
+      kh = (int)(p / (unsigned)P.dm.W); kw = (int)(p - (unsigned)kh * (unsigned)P.dm.W);
     }
-  } else {
-    const float* src = (const float*)P.src[0] + (size_t)gi * P.N_d + line0;
-    for (int idx = tid; idx < n * DCT_IC; idx += DCT_THREADS) {
-      const int b = idx / DCT_IC, c = idx % DCT_IC;
-      tile[idx] = (c0 + c < P.inner) ? src[(size_t)b * P.inner + c] : 0.f;
-    }
-  }
-  __syncthreads();
-
-  const int agroups = npad / 8;
-  for (int w = tid; w < agroups * (DCT_IC / 4); w += DCT_THREADS) {
-    const int ag = w / (DCT_IC / 4), cg = w % (DCT_IC / 4);
-    float acc[8][4];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    for (int b = 0; b < n; ++b) {
-      const float4 x = *(const float4*)(tile + b * DCT_IC + cg * 4);
-      const float4 m0 = *(const float4*)(matT + b * npad + ag * 8);
-      const float4 m1 = *(const float4*)(matT + b * npad + ag * 8 + 4);
-      const float mm[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
-      const float xx[4] = {x.x, x.y, x.z, x.w};
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(mm[i], xx[j], acc[i][j]);
-    }
-    const int c = c0 + cg * 4;
-    if (c >= P.inner) continue;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int a = ag * 8 + i;
+      const int a = g * 8 + i;
       if (a >= n) break;
-      if (MODE == 0 || MODE == 1) {
-        float* dst = (float*)P.dst + (size_t)gi * P.N_d + ((size_t)o * n + a) * P.inner + c;
-        *(float4*)dst = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-      } else if (MODE == 3) {
-        ST* dst = (ST*)P.dst + (size_t)th * P.N_d + ((size_t)o * n + a) * P.inner + c;
+      if (MODE <= 1) st4((float*)P.dst + (size_t)gi * P.N_d + line + (size_t)a * inner, acc[i]);
+      else if (MODE == 3) st4((ST*)P.dst + (size_t)th * P.N_d + line + (size_t)a * inner, acc[i]);
+      else store_coefficient<ST>(P.dm, P.spec_low, P.spec_mid, P.spec_high, th, a, kh, kw, ch, acc[i]);
+    }
+  }
+}
+
+template <typename ST, int MODE>
+cudaError_t launch_dct_pass(ff_plan* p, DctPassParams& P, int group, cudaStream_t st) {
+  const int npad = (P.n + 7) & ~7;
+  P.tiles = (int)(((long long)P.inner * P.outer + DCT_COLS - 1) / DCT_COLS);
+  // blocks stage the matrix once: about eight per SM, each with as many items as that leaves
+  const long long items = (long long)P.tiles * (npad / 8), want = (items + DCT_THREADS / 32 - 1) / (DCT_THREADS / 32);
+  long long blocks = 8LL * p->sm_count / group;
+  if (blocks < 1) blocks = 1;
+  if (blocks > want) blocks = want;
+  p->launches += 1;
+  return ff_launch(dct_pass_kernel<ST, MODE>, dim3((unsigned)blocks, (unsigned)group), dim3(DCT_THREADS),
+                   (size_t)P.n * npad * sizeof(float), st, P);
+}
+
+// ------------------------------------------------------------------------------------------------
+// All three axes of a small grid in one launch: a block holds eight channels of a tensor-head's whole grid in shared
+// memory and transforms it in place, axis by axis (lines are handled in rounds: everything a round reads is in
+// registers before any of it is overwritten).  Small grids are bound by launches and latency: 4 x 8 x 8 tokens take
+// one launch of 6 us instead of three of 5.
+// ------------------------------------------------------------------------------------------------
+constexpr int VOL_CH = 8, VOL_THREADS = 256;
+constexpr int VOL_MAX = 2304;            // positions: 72 KB, so that three blocks share an SM
+
+struct VolParams {
+  const void* src[3];      // forward: Q, K, V; inverse: src[0] = fp32 grids [g][N][d]
+  void* out;               // inverse: the caller's tensor
+  const float* mat_t[3];   // per axis (t, h, w): [b][a]
+  int group_start;
+  FFDims dm;
+  float* spec_low; void* spec_mid; void* spec_high;
+  double* clear;
+};
+
+template <typename ST, bool INVERSE>
+__global__ void __launch_bounds__(VOL_THREADS) dct_volume_kernel(const __grid_constant__ VolParams P) {
+  extern __shared__ float4 vol[];                      // [N][2]
+  const FFDims& dm = P.dm;
+  const int N = (int)dm.N, tid = threadIdx.x;
+  float* mt = (float*)(vol + 2 * N);
+  ff_pdl_wait();
+  if (!INVERSE && P.clear && blockIdx.x == 0 && blockIdx.y == 0)
+    for (int i = tid; i < dm.B * 3 * dm.d; i += VOL_THREADS) P.clear[i] = 0.0;
+  const int th = P.group_start + blockIdx.y, c0 = blockIdx.x * VOL_CH;
+  const size_t per = (size_t)N * dm.d;
+  for (int i = tid; i < 2 * N; i += VOL_THREADS) {
+    const size_t o = (size_t)(i >> 1) * dm.d + c0 + (i & 1) * 4;
+    vol[i] = INVERSE ? ld4((const float*)P.src[0] + (size_t)blockIdx.y * per + o)
+                     : ld4((const ST*)P.src[th / dm.BH] + (size_t)(th % dm.BH) * per + o);
+  }
+  for (int step = 0; step < 3; ++step) {
+    const int axis = INVERSE ? step : 2 - step;
+    const int n = axis == 2 ? dm.W : (axis == 1 ? dm.H : dm.T), stride = axis == 2 ? 1 : (axis == 1 ? dm.W : dm.H * dm.W);
+    const int npad = (n + 7) & ~7, groups = npad / 8;
+    stage_matrix(mt, P.mat_t[axis], n, npad);
+    __syncthreads();
+    const int upl = 2 * groups, lines = N / n;           // units (8 outputs x 4 channels) of a line
+    const int lpr = VOL_THREADS / upl;                   // lines per round
+    const int l = tid / upl, u = tid - l * upl, cg = u & 1, g = u >> 1;
+    for (int l0 = 0; l0 < lines; l0 += lpr) {
+      const int line = l0 + l;
+      const bool on = l < lpr && line < lines;
+      const int base = axis == 0 ? line : (line / stride) * stride * n + line % stride;
+      float4* x = vol + 2 * base + cg;
+      float4 acc[8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) stf<ST>(dst + j, acc[i][j]);
-      } else {  // MODE 2: a = k_t, column = (k_h, k_w, channel)
-        const int d = P.dm.d;
-        const int ch = c % d;
-        const int kw = (c / d) % P.dm.W;
-        const int kh = c / (d * P.dm.W);
-        long long rank;
-        const int band = ff_band_rank_of(P.dm, a, kh, kw, &rank);
-        const int tensor = th / P.BH, bh = th % P.BH;
-        if (band == 0) {
-          float* dst = P.spec_low + (((size_t)tensor * P.BH + bh) * P.dm.Nlow + rank) * d + ch;
-          *(float4*)dst = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-        } else {
-          const long long nl = (band == 1) ? P.dm.Nmid : P.dm.Nhigh;
-          ST* dst = (ST*)(band == 1 ? P.spec_mid : P.spec_high) + (((size_t)tensor * P.BH + bh) * nl + rank) * d + ch;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) stf<ST>(dst + j, acc[i][j]);
+      for (int i = 0; i < 8; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (on)
+#pragma unroll 4
+        for (int b = 0; b < n; ++b) {
+          const float4 v = x[2 * b * stride];
+          const float4 m0 = *(const float4*)(mt + b * npad + g * 8), m1 = *(const float4*)(mt + b * npad + g * 8 + 4);
+          fma4(acc[0], m0.x, v); fma4(acc[1], m0.y, v); fma4(acc[2], m0.z, v); fma4(acc[3], m0.w, v);
+          fma4(acc[4], m1.x, v); fma4(acc[5], m1.y, v); fma4(acc[6], m1.z, v); fma4(acc[7], m1.w, v);
         }
+      __syncthreads();
+      if (on)
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          if (g * 8 + i < n) x[2 * (g * 8 + i) * stride] = acc[i];
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < 2 * N; i += VOL_THREADS) {
+    const int f = i >> 1, ch = c0 + (i & 1) * 4;
+    if (INVERSE) st4((ST*)P.out + (size_t)th * per + (size_t)f * dm.d + ch, vol[i]);
+    else store_coefficient<ST>(dm, P.spec_low, P.spec_mid, P.spec_high, th, f / (dm.H * dm.W), f / dm.W % dm.H, f % dm.W, ch, vol[i]);
+  }
+}
+
+size_t vol_smem(const FFDims& dm) {
+  size_t m = 0;
+  const int n[3] = {dm.T, dm.H, dm.W};
+  for (int a = 0; a < 3; ++a) { const size_t x = (size_t)n[a] * ((n[a] + 7) & ~7); if (x > m) m = x; }
+  return (size_t)dm.N * VOL_CH * sizeof(float) + m * sizeof(float);
+}
+bool vol_fits(const FFDims& dm) { return dm.N <= VOL_MAX; }
+
+// ------------------------------------------------------------------------------------------------
+// Band operators ("Hierarchical frequency-domain attention") in fp32: a block takes 64 query rows of one (head, band)
+// and walks key tiles of 64 with an online softmax; Q and K tiles lie transposed in shared memory, P takes the place of
+// K between the two products.  A thread holds 4 x 4 scores (two 16-byte reads per 16 FMA) and 4 rows x d / 16 output
+// channels.  The key set of a row is generated from its rank: all pooled tokens (low), the blocks at block distance
+// 0 mod s (mid; query tiles then run along a residue class, so its keys are one dense range of class positions), own and
+// anchor blocks (mid, anchor pattern), the window |p - p'| <= R (high).
+// Bound by the FMA pipe and shared-memory reads; one warp per row with a five-shuffle reduction per score, as before,
+// took 1460 us where this takes about a tenth (9 x 30 x 40 tokens, 4 heads of 64 channels, all bands).
+// ------------------------------------------------------------------------------------------------
+constexpr int AT = 64, AT_THREADS = 256, AT_PITCH = AT + 4;
+
+template <int DPL> constexpr size_t at_smem() {
+  return (size_t)(DPL * 32 * AT_PITCH + (DPL >= 2 ? DPL * 32 : AT) * AT_PITCH + AT * DPL * 32) * sizeof(float);
+}
+
+template <typename KT, int DPL>
+__device__ __forceinline__ void attend_tile(const KT* Qp, const KT* Kp, const KT* Vp, KT* Yp, const FFDims& dm, int band, long long n,
+                                            int tile, float* sm) {
+  constexpr int d = DPL * 32;
+  float* Qt = sm;                                        // [d][AT_PITCH]
+  float* Kt = Qt + d * AT_PITCH;                         // [d][AT_PITCH], then P [key][AT_PITCH]
+  float* Vs = Kt + (d > AT ? d : AT) * AT_PITCH;         // [AT][d]
+  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  const float scale = rsqrtf((float)d);
+  const bool strided = band == 1 && dm.pattern == FF_MID_STRIDED;
+  const bool anchor = band == 1 && !strided;
+  // class-local (strided mid band) or band positions of the tile, and the range of key positions
+  int cls = 0;
+  long long q0 = (long long)tile * AT, len = n, ks = 0, ke = n;
+  if (strided) {
+    const int per = (int)(dm.nb / dm.s), rem = (int)(dm.nb % dm.s);                   // blocks of a class: per or per + 1
+    const int t_big = (int)(((long long)(per + 1) * dm.b + AT - 1) / AT), t_small = (int)(((long long)per * dm.b + AT - 1) / AT);
+    int t;
+    if (tile < rem * t_big) { cls = tile / t_big; t = tile % t_big; len = (long long)(per + 1) * dm.b; }
+    else {
+      const int rest = tile - rem * t_big;
+      if (t_small == 0 || rest >= (dm.s - rem) * t_small) return;
+      cls = rem + rest / t_small; t = rest % t_small; len = (long long)per * dm.b;
+    }
+    q0 = (long long)t * AT; ke = len;
+  } else {
+    if (q0 >= n) return;
+    if (band == 2) {
+      ks = q0 - dm.R > 0 ? q0 - dm.R : 0;
+      ke = q0 + AT + dm.R < n ? q0 + AT + dm.R : n;
+    }
+  }
+  auto rank_of = [&](long long u) -> long long {         // band rank of a position
+    if (!strided) return u;
+    const unsigned blk = (unsigned)u / (unsigned)dm.b;
+    return (long long)(((unsigned)cls + blk * (unsigned)dm.s) * (unsigned)dm.b + ((unsigned)u - blk * (unsigned)dm.b));
+  };
+  // a tile of rows, transposed: lanes along the rows, four channels per thread
+  auto load_t = [&](float* dst, const KT* src, long long u0, long long end) {
+    for (int i = tid; i < AT * (d / 4); i += AT_THREADS) {
+      const int row = i % AT, v = i / AT;
+      const long long u = u0 + row, rk = u < end ? rank_of(u) : n;
+      const float4 x = rk < n ? ld4(src + (size_t)rk * d + v * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+      dst[(v * 4) * AT_PITCH + row] = x.x; dst[(v * 4 + 1) * AT_PITCH + row] = x.y;
+      dst[(v * 4 + 2) * AT_PITCH + row] = x.z; dst[(v * 4 + 3) * AT_PITCH + row] = x.w;
+    }
+  };
+  load_t(Qt, Qp, q0, len);
+  long long pq[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) pq[i] = q0 + ty * 4 + i < len ? rank_of(q0 + ty * 4 + i) : n;
+  float mx[4], den[4], o[4][DPL][2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    mx[i] = -INFINITY; den[i] = 0.f;
+#pragma unroll
+    for (int j = 0; j < DPL; ++j) o[i][j][0] = o[i][j][1] = 0.f;
+  }
+  for (long long k0 = ks; k0 < ke; k0 += AT) {
+    if (anchor) {
+      // anchor blocks are s blocks apart: skip a key tile without one and without any of the rows' own blocks
+      const long long b0 = k0 / dm.b, b1 = ((k0 + AT < n ? k0 + AT : n) - 1) / dm.b;
+      const long long own0 = q0 / dm.b, own1 = ((q0 + AT < n ? q0 + AT : n) - 1) / dm.b;
+      const bool any = (b1 + 1) / dm.s > b0 / dm.s;      // some block J in [b0, b1] has J = s - 1 mod s
+      if (!any && (b1 < own0 || b0 > own1)) continue;
+    }
+    __syncthreads();                                     // the previous tile's P and V have been read
+    load_t(Kt, Kp, k0, ke);
+    for (int i = tid; i < AT * (d / 4); i += AT_THREADS) {
+      const int row = i / (d / 4), v = i % (d / 4);
+      const long long u = k0 + row, rk = u < ke ? rank_of(u) : n;
+      *(float4*)(Vs + row * d + v * 4) = rk < n ? ld4(Vp + (size_t)rk * d + v * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    float s[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
+#pragma unroll 8
+    for (int c = 0; c < d; ++c) {
+      const float4 q = *(const float4*)(Qt + c * AT_PITCH + ty * 4), k = *(const float4*)(Kt + c * AT_PITCH + tx * 4);
+      const float qq[4] = {q.x, q.y, q.z, q.w}, kk[4] = {k.x, k.y, k.z, k.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) s[i][j] = fmaf(qq[i], kk[j], s[i][j]);
+    }
+    // which of the thread's 4 x 4 pairs exist
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const long long u = k0 + tx * 4 + j, rk = u < ke ? rank_of(u) : n;
+      const bool in = rk < n;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        bool ok = in;
+        if (band == 2) ok = in && rk - pq[i] <= dm.R && pq[i] - rk <= dm.R;
+        else if (anchor) { const long long J = rk / dm.b; ok = in && (J == pq[i] / dm.b || J % dm.s == dm.s - 1); }
+        s[i][j] = ok ? s[i][j] * scale : -INFINITY;
+      }
+    }
+    __syncthreads();                                     // K has been read: P takes its place
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      float nm = fmaxf(fmaxf(s[i][0], s[i][1]), fmaxf(s[i][2], s[i][3]));
+#pragma unroll
+      for (int w = 8; w > 0; w >>= 1) nm = fmaxf(nm, __shfl_xor_sync(0xffffffffu, nm, w));
+      nm = fmaxf(nm, mx[i]);
+      const float ref = nm == -INFINITY ? 0.f : nm;      // (no key of the row so far)
+      const float corr = expf(mx[i] - ref);
+      float sum = 0.f;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) { s[i][j] = expf(s[i][j] - ref); sum += s[i][j]; }
+      den[i] = den[i] * corr + sum;                      // (this thread's share of the row sum)
+      mx[i] = nm;
+#pragma unroll
+      for (int j = 0; j < DPL; ++j) { o[i][j][0] *= corr; o[i][j][1] *= corr; }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) *(float4*)(Kt + (tx * 4 + j) * AT_PITCH + ty * 4) = make_float4(s[0][j], s[1][j], s[2][j], s[3][j]);
+    __syncthreads();
+    const int nk = ke - k0 < AT ? (int)(ke - k0) : AT;
+#pragma unroll 4
+    for (int k = 0; k < nk; ++k) {
+      const float4 p = *(const float4*)(Kt + k * AT_PITCH + ty * 4);
+      const float pp[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+      for (int j = 0; j < DPL; ++j) {
+        const float2 v = *(const float2*)(Vs + k * d + 32 * j + 2 * tx);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { o[i][j][0] = fmaf(pp[i], v.x, o[i][j][0]); o[i][j][1] = fmaf(pp[i], v.y, o[i][j][1]); }
       }
     }
   }
-}
-
-template <typename ST, int MODE>
-cudaError_t launch_dct_pass(const DctPassParams& P, int group, cudaStream_t st) {
-  const int npad = (P.n + 7) & ~7;
-  const size_t smem = ((size_t)P.n * npad + (size_t)P.n * DCT_IC) * sizeof(float);
-  const int chunks = (P.inner + DCT_IC - 1) / DCT_IC;
-  dim3 grid((unsigned)((size_t)P.outer * chunks), (unsigned)group);
-  return ff_launch(dct_pass_kernel<ST, MODE>, grid, dim3(DCT_THREADS), smem, st, P);
-}
-
-// ------------------------------------------------------------------------------------------------
-// Band operators ("Hierarchical frequency-domain attention"), one warp per query row, online
-// softmax with the score reduced by warp shuffles.  The key set of a row is generated from its
-// rank: all pooled tokens (low), the blocks at block distance 0 mod s (mid), the window
-// |p - p'| <= R (high).
-// ------------------------------------------------------------------------------------------------
-constexpr int ATT_WARPS = 8;
-
-template <typename KT, int DPL>   // DPL = d / 32 channels per lane
-__device__ __forceinline__ void attend_range(const KT* __restrict__ Kp, const KT* __restrict__ Vp, long long k0,
-                                             long long k1, int d, const float (&q)[DPL], float scale, float& mx,
-                                             float& den, float (&o)[DPL], int lane) {
-  for (long long k = k0; k < k1; ++k) {
-    const KT* kr = Kp + (size_t)k * d;
-    float part = 0.f;
 #pragma unroll
-    for (int j = 0; j < DPL; ++j) part = fmaf(q[j], ldf<KT>(kr + lane + 32 * j), part);
-    const float sc = warp_sum(part) * scale;
-    const float nm = fmaxf(mx, sc);
-    const float corr = expf(mx - nm);
-    const float pr = expf(sc - nm);
-    den = den * corr + pr;
-    const KT* vr = Vp + (size_t)k * d;
+  for (int i = 0; i < 4; ++i) {
 #pragma unroll
-    for (int j = 0; j < DPL; ++j) o[j] = fmaf(pr, ldf<KT>(vr + lane + 32 * j), o[j] * corr);
-    mx = nm;
+    for (int w = 8; w > 0; w >>= 1) den[i] += __shfl_xor_sync(0xffffffffu, den[i], w);
+    if (pq[i] >= n) continue;
+    KT* y = Yp + (size_t)pq[i] * d + 2 * tx;
+#pragma unroll
+    for (int j = 0; j < DPL; ++j) { stf<KT>(y + 32 * j, o[i][j][0] / den[i]); stf<KT>(y + 32 * j + 1, o[i][j][1] / den[i]); }
   }
 }
 
 template <typename ST, int DPL>
-__global__ void __launch_bounds__(ATT_WARPS * 32) attention_simt_kernel(FFBuffers buf, FFDims dm, int band_bits) {
+__global__ void __launch_bounds__(AT_THREADS, 2) attention_simt_kernel(FFBuffers buf, FFDims dm, int band_bits) {
+  extern __shared__ float sm[];
   ff_pdl_wait();
-  const int band = blockIdx.z, bh = blockIdx.y;
+  const int band = blockIdx.z == 0 ? 1 : (blockIdx.z == 1 ? 2 : 0);      // the mid band's items are the long ones
+  const int bh = blockIdx.y;
   if (!(buf.alloc[bh] & band_bits & (1 << band))) return;
   const long long n = band == 0 ? dm.Nbar : (band == 1 ? dm.Nmid : dm.Nhigh);
-  const long long p = (long long)blockIdx.x * ATT_WARPS + (threadIdx.x >> 5);
-  if (p >= n) return;
-  const int lane = threadIdx.x & 31;
-  const int d = dm.d;
-  const float scale = rsqrtf((float)d);
-  float q[DPL], o[DPL];
-  float mx = -INFINITY, den = 0.f;
-#pragma unroll
-  for (int j = 0; j < DPL; ++j) o[j] = 0.f;
-  const size_t BHn = (size_t)dm.BH * n * d;   // one tensor's extent in this band's buffer
+  if (n == 0) return;
+  const size_t one = (size_t)n * DPL * 32, tensor = (size_t)dm.BH * one;  // a head's, a tensor's extent in the band's buffer
   if (band == 0) {
-    const float* Qp = buf.pooled + (size_t)bh * n * d;
-    const float* Kp = Qp + BHn;
-    const float* Vp = Kp + BHn;
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) q[j] = Qp[(size_t)p * d + lane + 32 * j];
-    attend_range<float, DPL>(Kp, Vp, 0, n, d, q, scale, mx, den, o, lane);
-    float* y = buf.y_low + ((size_t)bh * n + p) * d;
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) y[lane + 32 * j] = o[j] / den;
+    const float* Q = buf.pooled + bh * one;
+    attend_tile<float, DPL>(Q, Q + tensor, Q + 2 * tensor, buf.y_low + bh * one, dm, band, n, blockIdx.x, sm);
   } else {
-    const ST* Qp = (const ST*)(band == 1 ? buf.spec_mid : buf.spec_high) + (size_t)bh * n * d;
-    const ST* Kp = Qp + BHn;
-    const ST* Vp = Kp + BHn;
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) q[j] = ldf<ST>(Qp + (size_t)p * d + lane + 32 * j);
-    if (band == 1 && dm.pattern == FF_MID_ANCHOR) {
-      // own block and every anchor block (block index = s-1 mod s)
-      const long long J = p / dm.b;
-      for (long long Jk = 0; Jk < dm.nb; ++Jk) {
-        if (Jk != J && Jk % dm.s != dm.s - 1) continue;
-        const long long k0 = Jk * dm.b;
-        const long long k1 = (k0 + dm.b < n) ? k0 + dm.b : n;
-        attend_range<ST, DPL>(Kp, Vp, k0, k1, d, q, scale, mx, den, o, lane);
-      }
-    } else if (band == 1) {
-      const long long J = p / dm.b;
-      for (long long Jk = J % dm.s; Jk < dm.nb; Jk += dm.s) {
-        const long long k0 = Jk * dm.b;
-        const long long k1 = (k0 + dm.b < n) ? k0 + dm.b : n;
-        attend_range<ST, DPL>(Kp, Vp, k0, k1, d, q, scale, mx, den, o, lane);
-      }
-    } else {
-      const long long k0 = (p - dm.R > 0) ? p - dm.R : 0;
-      const long long k1 = (p + dm.R + 1 < n) ? p + dm.R + 1 : n;
-      attend_range<ST, DPL>(Kp, Vp, k0, k1, d, q, scale, mx, den, o, lane);
-    }
-    ST* y = (ST*)(band == 1 ? buf.y_mid : buf.y_high) + ((size_t)bh * n + p) * d;
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) stf<ST>(y + lane + 32 * j, o[j] / den);
+    const ST* Q = (const ST*)(band == 1 ? buf.spec_mid : buf.spec_high) + bh * one;
+    attend_tile<ST, DPL>(Q, Q + tensor, Q + 2 * tensor, (ST*)(band == 1 ? buf.y_mid : buf.y_high) + bh * one, dm, band, n, blockIdx.x, sm);
   }
 }
 
 // Exchange + recombination ("Cross-band residual exchange", "Reconstruction"): for every
 // coefficient of the grid, fetch its band token, add softmax(y Z^T / sqrt(d)) Z over the 2m summary
-// tokens of the other two bands, and write the row at its coefficient position (fp32 grid).
+// tokens of the other two bands, and write the row at its coefficient position.
+// Eight lanes share a token (lane s holds channels 4 s + 32 i .. + 3): a score takes three shuffles for four tokens.
+// The four tokens of a warp may lie in different bands, so all 3m summaries are scored and a token's own band masked.
 constexpr int EXC_WARPS = 8;
+constexpr int EXC_TOKENS = EXC_WARPS * 4;      // per block and round
 
-// Coefficients per warp: up to 8, fewer when the launch would otherwise have too few blocks.
-static int exc_rounds(long long tokens, int g, int sm_count) {
-  long long r = tokens * g / ((long long)EXC_WARPS * 8 * sm_count);
+template <typename ST, int DPL, typename OT>
+__global__ void __launch_bounds__(EXC_WARPS * 32, 2) exchange_recombine_kernel(FFBuffers buf, FFDims dm, int bh0, OT* grid_out,
+                                                                               void* grid_lo, int rounds) {
+  extern __shared__ float4 Z[];                // [3 m][d]
+  constexpr int d = DPL * 32, KB = DPL >= 3 ? 4 : 8;       // keys scored side by side (registers)
+  ff_pdl_wait();
+  const int gi = blockIdx.y, bh = bh0 + gi, m = dm.m;
+  const float4* zsrc = (const float4*)(buf.summary + (size_t)bh * 3 * m * d);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < 3 * m * (d / 4); i += EXC_WARPS * 32) Z[i] = zsrc[i];
+  __syncthreads();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, s = lane & 7;
+  const float scale = rsqrtf((float)d);
+  const int N = (int)dm.N;
+  for (int round = 0; round < rounds; ++round) {
+    const int f0 = ((int)blockIdx.x * rounds + round) * EXC_TOKENS + warp * 4;
+    if (f0 >= N) return;
+    const int f = f0 + (lane >> 3) < N ? f0 + (lane >> 3) : N - 1;
+    const int row_w = f / dm.W, kw = f - row_w * dm.W, kt = row_w / dm.H, kh = row_w - kt * dm.H;
+    int rank;
+    const int band = band_rank(dm, kt, kh, kw, rank);
+    const BandView<ST> v = band_view<ST>(buf, dm, bh, band);
+    float4 y[DPL], acc[DPL];
+    const size_t at = (size_t)(v.compressed ? rank / dm.r : rank) * d + 4 * s;
+#pragma unroll
+    for (int i = 0; i < DPL; ++i) {
+      y[i] = v.f32 ? ld4(v.f32 + at + 32 * i) : ld4(v.st + at + 32 * i);
+      acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (m > 0) {
+      // keys of the token: not its own band's, and none of an empty mid band
+      const int skip0 = band * m, skip1 = dm.Nmid == 0 ? m : skip0;
+      float mx = -INFINITY, den = 0.f;
+      for (int k0 = 0; k0 < 3 * m; k0 += KB) {
+        float sc[KB];
+#pragma unroll
+        for (int k = 0; k < KB; ++k) {
+          const float4* z = Z + (k0 + k < 3 * m ? k0 + k : 0) * (d / 4) + s;
+          float part = 0.f;
+#pragma unroll
+          for (int i = 0; i < DPL; ++i) {
+            const float4 zz = z[8 * i];
+            part = fmaf(y[i].x, zz.x, part); part = fmaf(y[i].y, zz.y, part);
+            part = fmaf(y[i].z, zz.z, part); part = fmaf(y[i].w, zz.w, part);
+          }
+          sc[k] = part;
+        }
+#pragma unroll
+        for (int w = 4; w > 0; w >>= 1)
+#pragma unroll
+          for (int k = 0; k < KB; ++k) sc[k] += __shfl_xor_sync(0xffffffffu, sc[k], w);
+        float nm = mx;
+#pragma unroll
+        for (int k = 0; k < KB; ++k) {
+          const int key = k0 + k;
+          const bool on = key < 3 * m && !(key >= skip0 && key < skip0 + m) && !(key >= skip1 && key < skip1 + m);
+          sc[k] = on ? sc[k] * scale : -INFINITY;
+          nm = fmaxf(nm, sc[k]);
+        }
+        const float ref = nm == -INFINITY ? 0.f : nm;           // (no key so far)
+        const float corr = expf(mx - ref);
+        den *= corr;
+#pragma unroll
+        for (int i = 0; i < DPL; ++i) { acc[i].x *= corr; acc[i].y *= corr; acc[i].z *= corr; acc[i].w *= corr; }
+#pragma unroll
+        for (int k = 0; k < KB; ++k) {
+          const float pr = expf(sc[k] - ref);
+          const float4* z = Z + (k0 + k < 3 * m ? k0 + k : 0) * (d / 4) + s;
+          den += pr;
+#pragma unroll
+          for (int i = 0; i < DPL; ++i) fma4(acc[i], pr, z[8 * i]);
+        }
+        mx = nm;
+      }
+      if (den > 0.f)
+#pragma unroll
+        for (int i = 0; i < DPL; ++i) { acc[i].x /= den; acc[i].y /= den; acc[i].z /= den; acc[i].w /= den; }
+    }
+    if (f0 + (lane >> 3) >= N) continue;
+    // With a second grid (bf16 output) the value is stored in three bytes, rounded to 24 bits: its upper 16 bits
+    // in grid_out, the next 8 bits in the byte grid.  A band's tokens share almost the same exchange offset, so a
+    // single bf16 rounding would bias whole bands coherently and the inverse transform would focus that bias on a
+    // few tokens.
+    const size_t o = ((size_t)gi * N + f) * d + 4 * s;
+#pragma unroll
+    for (int i = 0; i < DPL; ++i) {
+      const float4 w = make_float4(y[i].x + acc[i].x, y[i].y + acc[i].y, y[i].z + acc[i].z, y[i].w + acc[i].w);
+      if (grid_lo) {
+        const uint32_t u0 = __float_as_uint(w.x) + 0x80u, u1 = __float_as_uint(w.y) + 0x80u;
+        const uint32_t u2 = __float_as_uint(w.z) + 0x80u, u3 = __float_as_uint(w.w) + 0x80u;
+        *(uint2*)((uint16_t*)grid_out + o + 32 * i) = make_uint2(__byte_perm(u0, u1, 0x7632), __byte_perm(u2, u3, 0x7632));
+        *(uint32_t*)((uint8_t*)grid_lo + o + 32 * i) = __byte_perm(__byte_perm(u0, u1, 0x0051), __byte_perm(u2, u3, 0x0051), 0x5410);
+      } else {
+        st4(grid_out + o + 32 * i, w);
+      }
+    }
+  }
+}
+
+// Rounds per block: up to 8, fewer when the launch would otherwise have too few blocks.
+int exc_rounds(long long tokens, int g, int sm_count) {
+  const long long r = tokens * g / ((long long)EXC_TOKENS * 8 * sm_count);
   return r < 1 ? 1 : (r > 8 ? 8 : (int)r);
 }
 
 template <typename ST, int DPL, typename OT>
-__global__ void __launch_bounds__(EXC_WARPS * 32) exchange_recombine_kernel(FFBuffers buf, FFDims dm, int bh0,
-                                                                             OT* grid_out, void* grid_lo, int low_only, int rounds) {
-  ff_pdl_wait();
-  extern __shared__ float S[];   // [3][m][d]
-  const int gi = blockIdx.y, bh = bh0 + gi;
-  const int d = dm.d, m = dm.m;
-  for (int i = threadIdx.x; i < 3 * m * d; i += blockDim.x) S[i] = buf.summary[(size_t)bh * 3 * m * d + i];
-  __syncthreads();
-  // low_only: the launch covers the low band's coefficients only (the other bands are exchanged
-  // by the tensor-core kernel); the index is then a low rank, unravelled inside the low box.
-  const int lane = threadIdx.x & 31;
-  // a block stages the summaries once and then works through rounds x EXC_WARPS coefficients
-  for (int round = 0; round < rounds; ++round) {
-  long long f = ((long long)blockIdx.x * rounds + round) * EXC_WARPS + (threadIdx.x >> 5);
-  if (f >= (low_only ? dm.Nlow : dm.N)) return;
-  int kw, kh, kt;
-  if (low_only) {
-    kw = (int)(f % dm.L[2]); kh = (int)((f / dm.L[2]) % dm.L[1]); kt = (int)(f / ((long long)dm.L[2] * dm.L[1]));
-    f = ((long long)kt * dm.H + kh) * dm.W + kw;
-  } else {
-    kw = (int)(f % dm.W); kh = (int)((f / dm.W) % dm.H); kt = (int)(f / ((long long)dm.W * dm.H));
-  }
-  long long rank;
-  const int band = ff_band_rank_of(dm, kt, kh, kw, &rank);
-  const BandView<ST> v = band_view<ST>(buf, dm, bh, band);
-  const long long row = v.compressed ? rank / dm.r : rank;
-  float y[DPL], acc[DPL];
-#pragma unroll
-  for (int j = 0; j < DPL; ++j) {
-    y[j] = v.f32 ? v.f32[(size_t)row * d + lane + 32 * j] : ldf<ST>(v.st + (size_t)row * d + lane + 32 * j);
-    acc[j] = 0.f;
-  }
-  if (m > 0) {
-    const float scale = rsqrtf((float)d);
-    float mx = -INFINITY, den = 0.f;
-    for (int ob = 0; ob < 3; ++ob) {
-      if (ob == band || (ob == 1 && dm.Nmid == 0)) continue;     // own band; an empty mid band has no summaries
-      for (int j2 = 0; j2 < m; ++j2) {
-        const float* z = S + ((size_t)ob * m + j2) * d;
-        float part = 0.f;
-#pragma unroll
-        for (int j = 0; j < DPL; ++j) part = fmaf(y[j], z[lane + 32 * j], part);
-        const float sc = warp_sum(part) * scale;
-        const float nm = fmaxf(mx, sc);
-        const float corr = expf(mx - nm), pr = expf(sc - nm);
-        den = den * corr + pr;
-#pragma unroll
-        for (int j = 0; j < DPL; ++j) acc[j] = fmaf(pr, z[lane + 32 * j], acc[j] * corr);
-        mx = nm;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < DPL; ++j) acc[j] /= den;
-  }
-  // With a second grid (bf16 output) the value is stored in three bytes, rounded to 24 bits: its upper 16 bits
-  // in grid_out, the next 8 bits in the byte grid.  A band's tokens share almost the same exchange offset, so a
-  // single bf16 rounding would bias whole bands coherently and the inverse transform would focus that bias on a
-  // few tokens.
-  OT* dst = grid_out + ((size_t)gi * dm.N + f) * d;
-#pragma unroll
-  for (int j = 0; j < DPL; ++j) {
-    const float v = y[j] + acc[j];
-    if (grid_lo) {
-      const uint32_t u = __float_as_uint(v) + 0x80u;
-      ((uint16_t*)dst)[lane + 32 * j] = (uint16_t)(u >> 16);
-      ((uint8_t*)grid_lo)[((size_t)gi * dm.N + f) * d + lane + 32 * j] = (uint8_t)(u >> 8);
-    } else {
-      stf<OT>(dst + lane + 32 * j, v);
-    }
-  }
-  }
+cudaError_t launch_exchange(ff_plan* p, int g, int h0, OT* grid_hi, void* grid_lo, cudaStream_t st) {
+  const FFDims& dm = p->dm;
+  const int rounds = exc_rounds(dm.N, g, p->sm_count);
+  const long long per_block = (long long)EXC_TOKENS * rounds;
+  p->launches += 1;
+  return ff_launch(exchange_recombine_kernel<ST, DPL, OT>, dim3((unsigned)((dm.N + per_block - 1) / per_block), (unsigned)g),
+                   dim3(EXC_WARPS * 32), (size_t)3 * dm.m * dm.d * sizeof(float), st, p->buf, dm, h0, grid_hi, grid_lo, rounds);
 }
 
 }  // namespace
@@ -314,6 +547,16 @@ __global__ void __launch_bounds__(EXC_WARPS * 32) exchange_recombine_kernel(FFBu
 template <typename ST>
 static cudaError_t forward_transform_t(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy, cudaStream_t st) {
   const FFDims& dm = p->dm;
+  if (vol_fits(dm)) {
+    VolParams P{};
+    P.src[0] = Q; P.src[1] = K; P.src[2] = V; P.dm = dm;
+    for (int a = 0; a < 3; ++a) P.mat_t[a] = p->basis_t[a];
+    P.spec_low = p->buf.spec_low; P.spec_mid = p->buf.spec_mid; P.spec_high = p->buf.spec_high;
+    P.clear = want_energy ? p->buf.energy : nullptr;
+    p->launches += 1;
+    return ff_launch(dct_volume_kernel<ST, false>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)(3 * dm.BH)), dim3(VOL_THREADS),
+                     vol_smem(dm), st, P);
+  }
   const int total = 3 * dm.BH, G = p->lay.group;
   DctPassParams P{};
   P.BH = dm.BH; P.N_d = dm.N * dm.d; P.dm = dm;
@@ -322,22 +565,21 @@ static cudaError_t forward_transform_t(ff_plan* p, const void* Q, const void* K,
     const int g = (total - g0 < G) ? total - g0 : G;
     P.group_start = g0;
     // w axis: lines of W elements with stride d
-    P.src[0] = Q; P.src[1] = K; P.src[2] = V; P.dst = p->buf.scratchA; P.mat = p->basis[2];
+    P.src[0] = Q; P.src[1] = K; P.src[2] = V; P.dst = p->buf.scratchA; P.mat_t = p->basis_t[2];
     P.n = dm.W; P.inner = dm.d; P.outer = dm.T * dm.H;
     P.clear = want_energy && g0 == 0 ? p->buf.energy : nullptr;
-    cudaError_t e = launch_dct_pass<ST, 0>(P, g, st);
+    cudaError_t e = launch_dct_pass<ST, 0>(p, P, g, st);
     if (e != cudaSuccess) return e;
     // h axis
-    P.src[0] = p->buf.scratchA; P.dst = p->buf.scratchB; P.mat = p->basis[1];
+    P.src[0] = p->buf.scratchA; P.dst = p->buf.scratchB; P.mat_t = p->basis_t[1];
     P.n = dm.H; P.inner = dm.W * dm.d; P.outer = dm.T;
-    e = launch_dct_pass<ST, 1>(P, g, st);
+    e = launch_dct_pass<ST, 1>(p, P, g, st);
     if (e != cudaSuccess) return e;
     // t axis + band split
-    P.src[0] = p->buf.scratchB; P.dst = nullptr; P.mat = p->basis[0];
+    P.src[0] = p->buf.scratchB; P.dst = nullptr; P.mat_t = p->basis_t[0];
     P.n = dm.T; P.inner = dm.H * dm.W * dm.d; P.outer = 1;
-    e = launch_dct_pass<ST, 2>(P, g, st);
+    e = launch_dct_pass<ST, 2>(p, P, g, st);
     if (e != cudaSuccess) return e;
-    p->launches += 3;
   }
   return cudaSuccess;
 }
@@ -350,19 +592,24 @@ cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, cons
 template <typename ST>
 static cudaError_t attention_simt_t(ff_plan* p, int band_bits, cudaStream_t st) {
   const FFDims& dm = p->dm;
-  long long nmax = 0;
-  if ((band_bits & FF_BAND_LOW) && dm.Nbar > nmax) nmax = dm.Nbar;
-  if ((band_bits & FF_BAND_MID) && dm.Nmid > nmax) nmax = dm.Nmid;
-  if ((band_bits & FF_BAND_HIGH) && dm.Nhigh > nmax) nmax = dm.Nhigh;
-  if (nmax == 0) return cudaSuccess;                 // (only an empty band was asked for)
-  const int zdim = (band_bits & FF_BAND_HIGH) ? 3 : ((band_bits & FF_BAND_MID) ? 2 : 1);
-  dim3 grid((unsigned)((nmax + ATT_WARPS - 1) / ATT_WARPS), (unsigned)dm.BH, zdim);
+  // the longest of the bands asked for, in tiles of 64 query rows (strided mid band: per residue class)
+  auto tiles = [](long long n) { return (n + AT - 1) / AT; };
+  long long most = 0;
+  if ((band_bits & FF_BAND_LOW) && tiles(dm.Nbar) > most) most = tiles(dm.Nbar);
+  if (band_bits & FF_BAND_MID) {
+    const long long per = dm.nb / dm.s, rem = dm.nb % dm.s;
+    const long long t = dm.pattern == FF_MID_STRIDED ? rem * tiles((per + 1) * dm.b) + (dm.s - rem) * tiles(per * dm.b) : tiles(dm.Nmid);
+    if (dm.Nmid > 0 && t > most) most = t;
+  }
+  if ((band_bits & FF_BAND_HIGH) && tiles(dm.Nhigh) > most) most = tiles(dm.Nhigh);
+  if (most == 0) return cudaSuccess;                 // (only an empty band was asked for)
+  const dim3 grid((unsigned)most, (unsigned)dm.BH, (band_bits & FF_BAND_LOW) ? 3 : ((band_bits & FF_BAND_HIGH) ? 2 : 1));
   p->launches += 1;
   switch (dm.d / 32) {
-    case 1: return ff_launch(attention_simt_kernel<ST, 1>, grid, dim3(ATT_WARPS * 32), 0, st, p->buf, dm, band_bits);
-    case 2: return ff_launch(attention_simt_kernel<ST, 2>, grid, dim3(ATT_WARPS * 32), 0, st, p->buf, dm, band_bits);
-    case 3: return ff_launch(attention_simt_kernel<ST, 3>, grid, dim3(ATT_WARPS * 32), 0, st, p->buf, dm, band_bits);
-    default: return ff_launch(attention_simt_kernel<ST, 4>, grid, dim3(ATT_WARPS * 32), 0, st, p->buf, dm, band_bits);
+    case 1: return ff_launch(attention_simt_kernel<ST, 1>, grid, dim3(AT_THREADS), at_smem<1>(), st, p->buf, dm, band_bits);
+    case 2: return ff_launch(attention_simt_kernel<ST, 2>, grid, dim3(AT_THREADS), at_smem<2>(), st, p->buf, dm, band_bits);
+    case 3: return ff_launch(attention_simt_kernel<ST, 3>, grid, dim3(AT_THREADS), at_smem<3>(), st, p->buf, dm, band_bits);
+    default: return ff_launch(attention_simt_kernel<ST, 4>, grid, dim3(AT_THREADS), at_smem<4>(), st, p->buf, dm, band_bits);
   }
 }
 
@@ -370,35 +617,22 @@ cudaError_t ffk_attention_simt(ff_plan* p, int band_bits, cudaStream_t st) {
   return p->dm.fp32 ? attention_simt_t<float>(p, band_bits, st) : attention_simt_t<__nv_bfloat16>(p, band_bits, st);
 }
 
-// Generic exchange + recombination into the hi/lo bf16 grids of the tensor-core inverse; DPL = d / 32.
-template <int DPL>
-static cudaError_t exchange_to_grids(ff_plan* p, long long tokens, int g, size_t smem, int h0, __nv_bfloat16* ghi,
-                                     __nv_bfloat16* glo, int low_only, cudaStream_t st) {
-  const int rounds = exc_rounds(tokens, g, p->sm_count);
-  const long long per_block = (long long)EXC_WARPS * rounds;
-  dim3 grid((unsigned)((tokens + per_block - 1) / per_block), (unsigned)g);
-  p->launches += 1;
-  return ff_launch(exchange_recombine_kernel<__nv_bfloat16, DPL, __nv_bfloat16>, grid, dim3(EXC_WARPS * 32), smem, st, p->buf, p->dm,
-                   h0, ghi, (void*)glo, low_only, rounds);
-}
-
-// Tensor-core inverse: exchange + recombination into a bf16 grid, then the three axis passes.
+// Tensor-core inverse: exchange + recombination into the three-byte grids, then the three axis passes.
 static cudaError_t exchange_inverse_tc(ff_plan* p, void* out, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int G = p->dct_group;
-  const size_t smem = (size_t)3 * dm.m * dm.d * sizeof(float);
   cudaError_t e = cudaSuccess;
   for (int h0 = 0; h0 < dm.BH; h0 += G) {
     const int g = (dm.BH - h0 < G) ? dm.BH - h0 : G;
     const size_t grid_bytes = ((size_t)G * dm.N * dm.d * 2 + 255) / 256 * 256;
     __nv_bfloat16* ghi = (__nv_bfloat16*)p->buf.scratchA;
-    __nv_bfloat16* glo = (__nv_bfloat16*)((char*)p->buf.scratchA + grid_bytes);
+    uint8_t* glo = (uint8_t*)p->buf.scratchA + grid_bytes;
     if (p->xtc_ok) {
-      // mid and high bands on the tensor cores, the fp32 low band with its own kernel (one warp per source row)
+      // mid and high bands on the tensor cores, the fp32 low band with its own kernel
       e = ffk_exchange_low(p, h0, g, ghi, glo, st);
       if (e == cudaSuccess) e = ffk_exchange_tc(p, h0, g, ghi, glo, st);
     } else {
-      e = dm.d == 128 ? exchange_to_grids<4>(p, dm.N, g, smem, h0, ghi, glo, 0, st) : exchange_to_grids<2>(p, dm.N, g, smem, h0, ghi, glo, 0, st);
+      e = dm.d == 128 ? launch_exchange<__nv_bfloat16, 4>(p, g, h0, ghi, glo, st) : launch_exchange<__nv_bfloat16, 2>(p, g, h0, ghi, glo, st);
     }
     if (e != cudaSuccess) return e;
     e = ffk_inverse_transform_tc(p, h0, g, out, st);
@@ -422,38 +656,39 @@ static cudaError_t exchange_inverse_t(ff_plan* p, void* out, cudaStream_t st) {
   const int G = p->lay.group;
   DctPassParams P{};
   P.BH = dm.BH; P.N_d = dm.N * dm.d; P.dm = dm;
-  const size_t smem = (size_t)3 * dm.m * dm.d * sizeof(float);
   for (int h0 = 0; h0 < dm.BH; h0 += G) {
     const int g = (dm.BH - h0 < G) ? dm.BH - h0 : G;
-    const int rounds = exc_rounds(dm.N, g, p->sm_count);
-    dim3 grid((unsigned)((dm.N + (long long)EXC_WARPS * rounds - 1) / ((long long)EXC_WARPS * rounds)), (unsigned)g);
-    cudaError_t e = cudaSuccess;
-#define FF_EXC(DPL)                                                                                                     \
-  ff_launch(exchange_recombine_kernel<ST, DPL, float>, grid, dim3(EXC_WARPS * 32), smem, st, p->buf, dm, h0, p->buf.scratchA, \
-            (void*)nullptr, 0, rounds)
+    cudaError_t e;
     switch (dm.d / 32) {
-      case 1: e = FF_EXC(1); break;
-      case 2: e = FF_EXC(2); break;
-      case 3: e = FF_EXC(3); break;
-      default: e = FF_EXC(4); break;
+      case 1: e = launch_exchange<ST, 1>(p, g, h0, p->buf.scratchA, nullptr, st); break;
+      case 2: e = launch_exchange<ST, 2>(p, g, h0, p->buf.scratchA, nullptr, st); break;
+      case 3: e = launch_exchange<ST, 3>(p, g, h0, p->buf.scratchA, nullptr, st); break;
+      default: e = launch_exchange<ST, 4>(p, g, h0, p->buf.scratchA, nullptr, st); break;
     }
-#undef FF_EXC
     if (e != cudaSuccess) return e;
-    P.group_start = h0;
     // inverse along t, h, w with the transposed matrices
-    P.src[0] = p->buf.scratchA; P.dst = p->buf.scratchB; P.mat = p->basis_t[0];
+    if (vol_fits(dm)) {
+      VolParams P{};
+      P.src[0] = p->buf.scratchA; P.out = out; P.dm = dm; P.group_start = h0;
+      for (int a = 0; a < 3; ++a) P.mat_t[a] = p->basis[a];
+      p->launches += 1;
+      e = ff_launch(dct_volume_kernel<ST, true>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)g), dim3(VOL_THREADS), vol_smem(dm), st, P);
+      if (e != cudaSuccess) return e;
+      continue;
+    }
+    P.group_start = h0;
+    P.src[0] = p->buf.scratchA; P.dst = p->buf.scratchB; P.mat_t = p->basis[0];
     P.n = dm.T; P.inner = dm.H * dm.W * dm.d; P.outer = 1;
-    e = launch_dct_pass<ST, 1>(P, g, st);
+    e = launch_dct_pass<ST, 1>(p, P, g, st);
     if (e != cudaSuccess) return e;
-    P.src[0] = p->buf.scratchB; P.dst = p->buf.scratchA; P.mat = p->basis_t[1];
+    P.src[0] = p->buf.scratchB; P.dst = p->buf.scratchA; P.mat_t = p->basis[1];
     P.n = dm.H; P.inner = dm.W * dm.d; P.outer = dm.T;
-    e = launch_dct_pass<ST, 1>(P, g, st);
+    e = launch_dct_pass<ST, 1>(p, P, g, st);
     if (e != cudaSuccess) return e;
-    P.src[0] = p->buf.scratchA; P.dst = out; P.mat = p->basis_t[2];
+    P.src[0] = p->buf.scratchA; P.dst = out; P.mat_t = p->basis[2];
     P.n = dm.W; P.inner = dm.d; P.outer = dm.T * dm.H;
-    e = launch_dct_pass<ST, 3>(P, g, st);
+    e = launch_dct_pass<ST, 3>(p, P, g, st);
     if (e != cudaSuccess) return e;
-    p->launches += 4;
   }
   return cudaSuccess;
 }
@@ -465,15 +700,18 @@ cudaError_t ffk_exchange_inverse(ff_plan* p, void* out, cudaStream_t st) {
 
 cudaError_t ffk_simt_init() {
   cudaError_t e = cudaSuccess;
-  const int most = 3 * 64 * 128 * (int)sizeof(float);       // summaries of a head; a transform tile and its matrix need no more
-#define FF_SET(k) if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
-#define FF_SET_T(T)                                                                                                    \
-  FF_SET((dct_pass_kernel<T, 0>)); FF_SET((dct_pass_kernel<T, 1>)); FF_SET((dct_pass_kernel<T, 2>)); FF_SET((dct_pass_kernel<T, 3>)); \
-  FF_SET((exchange_recombine_kernel<T, 1, float>)); FF_SET((exchange_recombine_kernel<T, 2, float>));                  \
-  FF_SET((exchange_recombine_kernel<T, 3, float>)); FF_SET((exchange_recombine_kernel<T, 4, float>))
+  const int most = 144 * 1024;       // the largest: a 72 KB volume and a 128 x 128 matrix
+#define FF_SET(...) if (e == cudaSuccess) e = cudaFuncSetAttribute(__VA_ARGS__, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+#define FF_SET_D(T, D)                                                                         \
+  FF_SET(attention_simt_kernel<T, D>); FF_SET(exchange_recombine_kernel<T, D, float>)
+#define FF_SET_T(T)                                                                            \
+  FF_SET(dct_pass_kernel<T, 0>); FF_SET(dct_pass_kernel<T, 1>); FF_SET(dct_pass_kernel<T, 2>); FF_SET(dct_pass_kernel<T, 3>); \
+  FF_SET(dct_volume_kernel<T, false>); FF_SET(dct_volume_kernel<T, true>);                     \
+  FF_SET_D(T, 1); FF_SET_D(T, 2); FF_SET_D(T, 3); FF_SET_D(T, 4)
   FF_SET_T(float); FF_SET_T(__nv_bfloat16);
-  FF_SET((exchange_recombine_kernel<__nv_bfloat16, 2, __nv_bfloat16>)); FF_SET((exchange_recombine_kernel<__nv_bfloat16, 4, __nv_bfloat16>));
+  FF_SET(exchange_recombine_kernel<__nv_bfloat16, 2, __nv_bfloat16>); FF_SET(exchange_recombine_kernel<__nv_bfloat16, 4, __nv_bfloat16>);
 #undef FF_SET_T
+#undef FF_SET_D
 #undef FF_SET
   return e;
 }
