@@ -716,13 +716,12 @@ cudaError_t ffk_dct2_init() {
   return cudaFuncSetAttribute(dct2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D2_SMEM);
 }
 
-// Which second axis the fused launch takes and how many CTAs share a plane: the shorter of h and t
-// (smaller planes need fewer CTAs), an even number of tiles per CTA.  The kernel runs clusters of up to
-// eight CTAs, but it is used only where one or two CTAs hold the plane (W x n2 <= 2048 positions):
-// measured on B200, the launch beats the separate passes by 23% at T=16, W=64 (one CTA per plane) and by
-// 6% at T=32 (two), and loses from four CTAs on (the remote stores of phase 1 and their cluster-scope
-// release cost more than the saved DRAM round trip).
-constexpr int MAX_CLUSTER_USED = 2;
+// Which second axis the fused launch takes: the shorter of h and t (smaller planes), an even number of tiles.  It is
+// used only where one CTA holds the plane (W x n2 <= 1024 positions): on B200 the launch beats the separate passes by
+// 23% at T = 16, W = 64 and loses from two CTAs per plane on (the remote stores of phase 1 and their cluster-scope
+// release cost more than the saved DRAM round trip: whole layer, T = 32, W = 64: 13.27 against 12.67 ms with three
+// passes, two samples of 24 heads; T = 16, W = 128: 1.32 against 1.18 ms).
+constexpr int MAX_CLUSTER_USED = 1;
 
 bool ffk_dct2_supported(const FFDims& dm, int* axis2, int* cs) {
   if (dm.fp32 || dm.d % CHK != 0 || (dm.d != 128 && dm.d != 64) || !axis_ok(dm.T) || !axis_ok(dm.H) || !axis_ok(dm.W)) return false;

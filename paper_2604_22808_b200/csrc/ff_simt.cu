@@ -87,7 +87,7 @@ __device__ __forceinline__ void stage_matrix(float* mt, const float* mat_t, int 
 }
 
 template <typename ST, int MODE>
-__global__ void __launch_bounds__(DCT_THREADS) dct_pass_kernel(const __grid_constant__ DctPassParams P) {
+__global__ void __launch_bounds__(DCT_THREADS, 3) dct_pass_kernel(const __grid_constant__ DctPassParams P) {
   extern __shared__ float mt[];
   const int n = P.n, npad = (n + 7) & ~7, groups = npad / 8;
   stage_matrix(mt, P.mat_t, n, npad);
@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(DCT_THREADS) dct_pass_kernel(const __grid_cons
     for (int i = 0; i < 8; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     auto sum_line = [&](auto* src) {
       const float* m = mt + g * 8;
-#pragma unroll 4
+#pragma unroll 8
       for (int b = 0; b < n; ++b) {
         const float4 x = ld4(src + (size_t)b * inner);
         const float4 m0 = *(const float4*)(m + b * npad), m1 = *(const float4*)(m + b * npad + 4);
@@ -143,9 +143,9 @@ template <typename ST, int MODE>
 cudaError_t launch_dct_pass(ff_plan* p, DctPassParams& P, int group, cudaStream_t st) {
   const int npad = (P.n + 7) & ~7;
   P.tiles = (int)(((long long)P.inner * P.outer + DCT_COLS - 1) / DCT_COLS);
-  // blocks stage the matrix once: about eight per SM, each with as many items as that leaves
+  // the three blocks an SM holds, each with as many items as that leaves (the matrix is staged once per block)
   const long long items = (long long)P.tiles * (npad / 8), want = (items + DCT_THREADS / 32 - 1) / (DCT_THREADS / 32);
-  long long blocks = 8LL * p->sm_count / group;
+  long long blocks = 3LL * p->sm_count / group;
   if (blocks < 1) blocks = 1;
   if (blocks > want) blocks = want;
   p->launches += 1;
@@ -249,7 +249,7 @@ bool vol_fits(const FFDims& dm) { return dm.N <= VOL_MAX; }
 constexpr int AT = 64, AT_THREADS = 256, AT_PITCH = AT + 4;
 
 template <int DPL> constexpr size_t at_smem() {
-  return (size_t)(DPL * 32 * AT_PITCH + (DPL >= 2 ? DPL * 32 : AT) * AT_PITCH + AT * DPL * 32) * sizeof(float);
+  return (size_t)(DPL * 32 * AT_PITCH + (DPL >= 2 ? DPL * 32 : AT) * AT_PITCH + AT * (DPL * 32 + 4)) * sizeof(float);
 }
 
 template <typename KT, int DPL>
@@ -258,7 +258,7 @@ __device__ __forceinline__ void attend_tile(const KT* Qp, const KT* Kp, const KT
   constexpr int d = DPL * 32;
   float* Qt = sm;                                        // [d][AT_PITCH]
   float* Kt = Qt + d * AT_PITCH;                         // [d][AT_PITCH], then P [key][AT_PITCH]
-  float* Vs = Kt + (d > AT ? d : AT) * AT_PITCH;         // [AT][d]
+  float* Vs = Kt + (d > AT ? d : AT) * AT_PITCH;         // [AT][d + 4]
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const float scale = rsqrtf((float)d);
   const bool strided = band == 1 && dm.pattern == FF_MID_STRIDED;
@@ -289,17 +289,19 @@ __device__ __forceinline__ void attend_tile(const KT* Qp, const KT* Kp, const KT
     const unsigned blk = (unsigned)u / (unsigned)dm.b;
     return (long long)(((unsigned)cls + blk * (unsigned)dm.s) * (unsigned)dm.b + ((unsigned)u - blk * (unsigned)dm.b));
   };
-  // a tile of rows, transposed: lanes along the rows, four channels per thread
-  auto load_t = [&](float* dst, const KT* src, long long u0, long long end) {
-    for (int i = tid; i < AT * (d / 4); i += AT_THREADS) {
-      const int row = i % AT, v = i / AT;
-      const long long u = u0 + row, rk = u < end ? rank_of(u) : n;
-      const float4 x = rk < n ? ld4(src + (size_t)rk * d + v * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-      dst[(v * 4) * AT_PITCH + row] = x.x; dst[(v * 4 + 1) * AT_PITCH + row] = x.y;
-      dst[(v * 4 + 2) * AT_PITCH + row] = x.z; dst[(v * 4 + 3) * AT_PITCH + row] = x.w;
-    }
+  // A thread loads row `lrow` of every tile, a quarter of its channels (lanes along the rows, so that the transposed
+  // stores meet no bank twice).
+  const int lrow = tid % AT, lv = tid / AT;
+  auto put_t = [&](float* dst, int v, const float4& x) {
+    dst[(v * 4) * AT_PITCH + lrow] = x.x; dst[(v * 4 + 1) * AT_PITCH + lrow] = x.y;
+    dst[(v * 4 + 2) * AT_PITCH + lrow] = x.z; dst[(v * 4 + 3) * AT_PITCH + lrow] = x.w;
   };
-  load_t(Qt, Qp, q0, len);
+  {
+    const long long rk = q0 + lrow < len ? rank_of(q0 + lrow) : n;
+    const KT* src = Qp + (size_t)(rk < n ? rk : 0) * d;
+#pragma unroll 2
+    for (int v = lv; v < d / 4; v += AT_THREADS / AT) put_t(Qt, v, rk < n ? ld4(src + v * 4) : make_float4(0.f, 0.f, 0.f, 0.f));
+  }
   long long pq[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) pq[i] = q0 + ty * 4 + i < len ? rank_of(q0 + ty * 4 + i) : n;
@@ -319,11 +321,16 @@ __device__ __forceinline__ void attend_tile(const KT* Qp, const KT* Kp, const KT
       if (!any && (b1 < own0 || b0 > own1)) continue;
     }
     __syncthreads();                                     // the previous tile's P and V have been read
-    load_t(Kt, Kp, k0, ke);
-    for (int i = tid; i < AT * (d / 4); i += AT_THREADS) {
-      const int row = i / (d / 4), v = i % (d / 4);
-      const long long u = k0 + row, rk = u < ke ? rank_of(u) : n;
-      *(float4*)(Vs + row * d + v * 4) = rk < n ? ld4(Vp + (size_t)rk * d + v * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+    {
+      const long long rk = k0 + lrow < ke ? rank_of(k0 + lrow) : n;
+      const size_t at = (size_t)(rk < n ? rk : 0) * d;
+#pragma unroll 2
+      for (int v = lv; v < d / 4; v += AT_THREADS / AT) {
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 kx = rk < n ? ld4(Kp + at + v * 4) : zero, vx = rk < n ? ld4(Vp + at + v * 4) : zero;
+        put_t(Kt, v, kx);
+        *(float4*)(Vs + lrow * (d + 4) + v * 4) = vx;
+      }
     }
     __syncthreads();
     float s[4][4];
@@ -331,7 +338,7 @@ __device__ __forceinline__ void attend_tile(const KT* Qp, const KT* Kp, const KT
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-#pragma unroll 8
+#pragma unroll 4
     for (int c = 0; c < d; ++c) {
       const float4 q = *(const float4*)(Qt + c * AT_PITCH + ty * 4), k = *(const float4*)(Kt + c * AT_PITCH + tx * 4);
       const float qq[4] = {q.x, q.y, q.z, q.w}, kk[4] = {k.x, k.y, k.z, k.w};
@@ -380,7 +387,7 @@ __device__ __forceinline__ void attend_tile(const KT* Qp, const KT* Kp, const KT
       const float pp[4] = {p.x, p.y, p.z, p.w};
 #pragma unroll
       for (int j = 0; j < DPL; ++j) {
-        const float2 v = *(const float2*)(Vs + k * d + 32 * j + 2 * tx);
+        const float2 v = *(const float2*)(Vs + k * (d + 4) + 32 * j + 2 * tx);
 #pragma unroll
         for (int i = 0; i < 4; ++i) { o[i][j][0] = fmaf(pp[i], v.x, o[i][j][0]); o[i][j][1] = fmaf(pp[i], v.y, o[i][j][1]); }
       }
@@ -407,7 +414,11 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attention_simt_kernel(FFBuffers
   const long long n = band == 0 ? dm.Nbar : (band == 1 ? dm.Nmid : dm.Nhigh);
   if (n == 0) return;
   const size_t one = (size_t)n * DPL * 32, tensor = (size_t)dm.BH * one;  // a head's, a tensor's extent in the band's buffer
-  if (band == 0) {
+  if (sizeof(ST) == 4) {                          // (one copy of the code: small launches are bound by fetching it)
+    const float* Q = (band == 0 ? buf.pooled : (const float*)(band == 1 ? buf.spec_mid : buf.spec_high)) + bh * one;
+    float* Y = (band == 0 ? buf.y_low : (float*)(band == 1 ? buf.y_mid : buf.y_high)) + bh * one;
+    attend_tile<float, DPL>(Q, Q + tensor, Q + 2 * tensor, Y, dm, band, n, blockIdx.x, sm);
+  } else if (band == 0) {
     const float* Q = buf.pooled + bh * one;
     attend_tile<float, DPL>(Q, Q + tensor, Q + 2 * tensor, buf.y_low + bh * one, dm, band, n, blockIdx.x, sm);
   } else {

@@ -231,7 +231,7 @@ __device__ __forceinline__ float exp2f_fast(float x) {
 // every r consecutive coefficient ranks, so its update is computed once and written r times; other heads carry V~ low,
 // one row per rank.  Eight lanes share a row (lane s holds channels 4 s + 32 i .. + 3), so that a score takes three
 // shuffles for four rows at once: with a whole warp per row the kernel was bound by its five shuffles per score and row
-// (131 072 rows of 64 channels, 16 keys: 106 us).  Scores of eight keys are reduced side by side and merged into the
+// (131 072 rows of 64 channels, 16 keys: 106 us).  Scores of four or eight keys are reduced side by side and merged into the
 // running softmax as a group, exponentials by ex2.approx on scores in log2 units, like the tensor-core kernel's.
 constexpr int XL_WARPS = 8;
 template <int DPL>
@@ -239,6 +239,7 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
                                                                       uint8_t* grid_lo, int rounds) {
   extern __shared__ float4 Z[];                 // the summaries of the other bands, [keys][d]
   constexpr int d = DPL * 32, V = DPL;          // float4 per lane and row
+  constexpr int KB = DPL >= 4 ? 4 : 8;          // keys scored side by side (registers)
   ff_pdl_wait();
   const int gi = blockIdx.y, bh = bh0 + gi, m = dm.m;
   // the summaries of the other bands: the mid band's (none if it is empty), then the high band's
@@ -263,10 +264,10 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
 #pragma unroll
     for (int i = 0; i < V; ++i) { y[i] = yr[8 * i]; acc[i] = make_float4(0.f, 0.f, 0.f, 0.f); }
     float mx = -INFINITY, den = 0.f;
-    for (int k0 = 0; k0 < nkeys; k0 += 8) {
-      float sc[8];
+    for (int k0 = 0; k0 < nkeys; k0 += KB) {
+      float sc[KB];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
+      for (int k = 0; k < KB; ++k) {
         const float4* z = Z + (size_t)(k0 + k < nkeys ? k0 + k : 0) * (d / 4) + s;
         float part = 0.f;
 #pragma unroll
@@ -280,16 +281,16 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
 #pragma unroll
       for (int o = 4; o > 0; o >>= 1)
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sc[k] += __shfl_xor_sync(0xffffffffu, sc[k], o);
+        for (int k = 0; k < KB; ++k) sc[k] += __shfl_xor_sync(0xffffffffu, sc[k], o);
       float nm = mx;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) { sc[k] = k0 + k < nkeys ? sc[k] * scale : -INFINITY; nm = fmaxf(nm, sc[k]); }
+      for (int k = 0; k < KB; ++k) { sc[k] = k0 + k < nkeys ? sc[k] * scale : -INFINITY; nm = fmaxf(nm, sc[k]); }
       const float corr = exp2f_fast(mx - nm);
       den *= corr;
 #pragma unroll
       for (int i = 0; i < V; ++i) { acc[i].x *= corr; acc[i].y *= corr; acc[i].z *= corr; acc[i].w *= corr; }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
+      for (int k = 0; k < KB; ++k) {
         const float p = exp2f_fast(sc[k] - nm);               // (0 for the keys past the end)
         const float4* z = Z + (size_t)(k0 + k < nkeys ? k0 + k : 0) * (d / 4) + s;
         den += p;
@@ -328,10 +329,10 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
   }
 }
 
-// Rows a piece of a segment should have: about six blocks per SM over all bands while that leaves 128 rows or more, at
-// most 1024 (256 KB of bf16 at head_dim 128).
+// Rows a piece of a segment should have: about the three blocks an SM holds over all bands while that leaves 128 rows or
+// more (a block's own latency is three to four microseconds), at most 1024 (256 KB of bf16 at head_dim 128).
 int piece_rows(const FFDims& dm) {
-  const long long rows = (long long)dm.BH * dm.N / (148 * 6);
+  const long long rows = (long long)dm.BH * dm.N / (148 * 3);
   return (int)(rows < 128 ? 128 : (rows > 1024 ? 1024 : rows));
 }
 
