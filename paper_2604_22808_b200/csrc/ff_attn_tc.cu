@@ -190,12 +190,6 @@ __device__ __forceinline__ bool row_exchange(unsigned long long* slots, int part
   return true;
 }
 
-// max of three (one instruction on sm_100)
-__device__ __forceinline__ float max3f(float a, float b, float c) {
-  float r;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

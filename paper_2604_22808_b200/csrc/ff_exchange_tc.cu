@@ -5,20 +5,27 @@
 // written to the coefficient grid at the position of band rank p (a table built at plan creation).
 //
 // A CTA owns a contiguous run of (head, band, 128-rank tile) items, so the summary tokens of a head
-// are re-staged only a few times per CTA.
-// Two CTAs share an SM (256 tensor-memory columns each).  Inside a CTA the softmax warps work on
-// tile n + 1 while the store warps finish tile n.  Per tile:
+// are loaded only a few times per CTA.  Two CTAs share an SM (256 tensor-memory columns each).  Per tile:
 //   TMA     the 128 band tokens (operator output where the head's mask has the band, V~ otherwise)
-//   MMA 1   S[128 x 3m] = Y Z^T against all 3m summaries of the head (own band masked in the softmax)
-//   softmax one token per thread (row = TMEM lane); P written back to TMEM as bf16 hi + lo (normalised
-//           for up to 32 keys, otherwise unnormalised with the row sum handed to the store warps)
+//   MMA 1   S[128 x 3m] = Y Z^T against all 3m summaries of the head; with up to 64 keys into one of two buffers, so
+//           that the next tile's scores are computed during this tile's softmax
+//   softmax one token per thread (row = TMEM lane), 16 keys at a time; chunks that are the band's own summaries are
+//           skipped; P (unnormalised) goes back to TMEM as bf16 hi + lo over the 16 scores it comes from, the row sum
+//           to the store warps
 //   MMA 2   D[128 x 128] = P Z  (A = P from tensor memory, B = the same Z image read MN-major)
-//   store   Y + D in the three-byte form the inverse passes read (the value rounded to 24 bits: a grid of its
-//           upper 16 bits and a grid of the next byte); a thread owns a token, the warp stages 32 channels of
-//           its 32 tokens in shared memory and four lanes then write a token's 64 + 32 contiguous bytes
+//   store   Y + D / row sum in the three-byte form the inverse passes read (the value rounded to 24 bits: a grid of its
+//           upper 16 bits and a grid of the next byte).  A warp has 32 tokens, one per lane; it turns 32 channels of
+//           them in shared memory, so that four lanes write 64 (hi) and 32 (lo) contiguous bytes of a token.  With more
+//           than 64 keys a second token tile no longer fits: the tile then goes back to the producer as soon as the
+//           scores are done, the update is turned as fp32 and the tokens are read again from global memory, four lanes
+//           64 contiguous bytes.
 // Z and P are split into bf16 hi + lo parts (Y is exact bf16), so the logits and the update carry
 // about 16 bits: the summary logits of a band with large low-frequency content reach O(100).
-// The low band (fp32, a few hundred tokens) is handled by the generic kernel.
+// The low band (fp32, a few hundred tokens) has a kernel of its own (ff_summary.cu).
+//
+// Bound by the chain of these steps between the warps of a tile and by its row-scattered stores (without them the launch
+// takes half the time); 64K tokens, 24 heads: 0.28 ms = 3.6 TB/s.  1M tokens (96 keys): 2.2 -> 1.55 ms per 8 heads since
+// the residual is read four lanes to a token (it was one lane to a token) and own-band chunks are skipped.
 #include <cuda.h>
 
 #include "ff_internal.h"
@@ -45,10 +52,6 @@ struct XParams {
   int h0, g;                  // heads [h0, h0+g)
   int nkeys;                  // 3m rounded up to a multiple of 16
   int ybufs;                  // token-tile buffers in shared memory (1 or 2)
-  // With one buffer (two CTAs with two buffers each no longer fit an SM: more than 64 summary keys) the tile is
-  // handed back to the producer as soon as the score MMAs have read it, and the store warps take the tokens for
-  // the residual add from global memory instead (they were just loaded: L2 hits), so that the next tile's load
-  // still overlaps this tile's softmax and stores.
   const __nv_bfloat16* src[4];   // y_mid, v~_mid, y_high, v~_high: bases of the buffers the four maps cover
   int* status;
 };
@@ -62,15 +65,17 @@ __device__ unsigned long long g_x_prof[16];
 #define XPROF_ADD(i, v)
 #endif
 
-constexpr int X_STG_PITCH = 64;         // bytes per staged row piece (32 channels)
+// per store warp: 32 channels of 32 tokens, 64 bytes of hi and 32 of lo each, or in fp32
+__host__ __device__ constexpr int x_stage_bytes(bool reread) { return reread ? 32 * 128 : 32 * 96; }
 
 struct XShared {
-  uint64_t y_full[2], y_empty[2], z_ready, z_empty, s_full, p_full, d_full, d_empty;
+  uint64_t y_full[2], y_empty[2], z_ready, z_empty, s_full[2], p_full[2], d_full, d_empty;
   uint32_t tmem_base;
   int abort_flag;
-  // per softmax warp: 32 rows x 64 bytes of hi and of lo (16-byte chunks XOR-swizzled with row / 2)
-  alignas(16) uint8_t stage[4][2][32 * X_STG_PITCH];
-  float inv[2][XT];          // (two-sweep variants) 1 / row sum of the tile, by tile parity
+  // keys a token attends to, as bit masks per band (mid, high) and 16-key chunk: the 3m summaries without the token's own
+  // band's and without those of an empty mid band
+  uint32_t keys[2][6];
+  float inv[4][XT];          // 1 / row sum of a tile (the softmax may be two tiles ahead of the store warps)
 };
 
 struct XItem { int bh, band, tile; };
@@ -87,22 +92,24 @@ __device__ __forceinline__ float ex2f_approx(float x) {
   return y;
 }
 
-__device__ __forceinline__ XItem x_decode(const FFDims& dm, int h0, int it, int tm, int th) {
+__device__ __forceinline__ XItem x_decode(int h0, int it, int tm, int th) {
   XItem x;
-  const int per = tm + th;
+  const int per = tm + th, rem = it % per;
   x.bh = h0 + it / per;
-  const int rem = it % per;
   x.band = rem < tm ? 1 : 2;
   x.tile = rem < tm ? rem : rem - tm;
   return x;
 }
+__device__ __forceinline__ void x_next(XItem& x, int tm, int th) {
+  if (++x.tile == (x.band == 1 ? tm : th)) {
+    x.tile = 0;
+    if (x.band == 1) x.band = 2;
+    else { ++x.bh; x.band = tm > 0 ? 1 : 2; }
+  }
+}
 
-// NK32 = 32-key chunks of the score row that are in use (3m <= 32 NK32).
-// With two or three chunks the score row does not fit the registers two resident CTAs leave a
-// thread: those variants sweep the scores twice (maximum, then exponentials chunk by chunk), write
-// P unnormalised and let the store warps scale the update by 1 / row sum.  Their P_lo chunks sit in
-// columns 96, 112 and 80, where no unread score can be overwritten.
-template <int NK32, int XD>
+// NK = 16-key chunks of the score row (3m rounded up).
+template <int NK, int XD>
 __global__ void __launch_bounds__(X_THREADS, 2)
 exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_constant__ CUtensorMap map_v_mid,
                    const __grid_constant__ CUtensorMap map_y_high, const __grid_constant__ CUtensorMap map_v_high,
@@ -112,10 +119,13 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
   uint8_t* sY = smem;                                    // ybufs x 32 KB
   uint8_t* sZhi = smem + P.ybufs * X_TILE_BYTES;         // [2 halves][nkeys rows][128 B]
   uint8_t* sZlo = sZhi + 2 * P.nkeys * 128;
-  XShared& sh = *(XShared*)(sZlo + 2 * P.nkeys * 128);
+  constexpr bool REREAD = NK > 4;                         // one token tile: the residual comes from global memory
+  uint8_t* sStage = sZlo + 2 * P.nkeys * 128;            // 4 x x_stage_bytes
+  XShared& sh = *(XShared*)(sStage + 4 * x_stage_bytes(REREAD));
   const FFDims& dm = P.dm;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m = dm.m, nk = P.nkeys;
+  constexpr int nk = NK * 16, SB = NK <= 4 ? 2 : 1;      // keys; score buffers (64 columns apart)
+  const int m = dm.m;
   const int tm_tiles = (int)((dm.Nmid + XT - 1) / XT), th_tiles = (int)((dm.Nhigh + XT - 1) / XT);
   const int total = P.g * (tm_tiles + th_tiles);
   const int chunk = (total + gridDim.x - 1) / gridDim.x;
@@ -123,11 +133,23 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
   const int it1 = it0 + chunk < total ? it0 + chunk : total;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < 2; ++i) { mbar_init(&sh.y_full[i], 1); mbar_init(&sh.y_empty[i], P.ybufs == 1 ? 1 : 128); }
-    mbar_init(&sh.z_ready, 1); mbar_init(&sh.z_empty, 1); mbar_init(&sh.s_full, 1); mbar_init(&sh.p_full, 128);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&sh.y_full[i], 1); mbar_init(&sh.y_empty[i], REREAD ? 1 : 128); mbar_init(&sh.s_full[i], 1); mbar_init(&sh.p_full[i], 128);
+    }
+    mbar_init(&sh.z_ready, 1); mbar_init(&sh.z_empty, 1);
     mbar_init(&sh.d_full, 1); mbar_init(&sh.d_empty, 128);
     sh.abort_flag = 0;
     fence_mbar_init();
+  }
+  if (threadIdx.x >= 64 && threadIdx.x < 64 + 2 * NK) {
+    const int band = (threadIdx.x - 64) / NK, c = (threadIdx.x - 64) % NK;
+    uint32_t a = 0;
+    for (int i = 0; i < 16; ++i) {
+      const int j = c * 16 + i;
+      const bool live = j < 3 * m && !(dm.Nmid == 0 && j >= m && j < 2 * m);
+      if (live && (band == 0 ? j < m || j >= 2 * m : j < 2 * m)) a |= 1u << i;
+    }
+    sh.keys[band][c] = a;
   }
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 256); tmem_relinquish(); }
   // The launch before this one is the low band's part of the exchange, which writes other positions of the same
@@ -138,15 +160,15 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
   tc_fence_after();
   const uint32_t tmem = sh.tmem_base;
   volatile int* abort_flag = &sh.abort_flag;
-  // tensor-memory columns: S [0,96), overwritten by P_hi [0,48) and P_lo [48,96);  D [128,256)
+  // tensor-memory columns: S [0,128): one buffer of up to 96 columns or two of 64; P over the scores;  D [128,256)
   const int YB = P.ybufs;
 
   if (warp == 0) {
     if (lane == 0) {
       bool ok = true;
       int n = 0, prev_bh = -1, zc = 0;
-      for (int it = it0; it < it1 && ok; ++it, ++n) {
-        const XItem x = x_decode(dm, P.h0, it, tm_tiles, th_tiles);
+      XItem x = x_decode(P.h0, it0, tm_tiles, th_tiles);
+      for (int it = it0; it < it1 && ok; ++it, ++n, x_next(x, tm_tiles, th_tiles)) {
         const bool exec = P.alloc[x.bh] & (1 << x.band);
         const CUtensorMap* map = x.band == 1 ? (exec ? &map_y_mid : &map_v_mid) : (exec ? &map_y_high : &map_v_high);
         const int slice = exec ? x.bh : 2 * dm.BH + x.bh;
@@ -178,48 +200,64 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
       const uint32_t zhi = smem_u32(sZhi), zlo = smem_u32(sZlo);
       const uint32_t zhalf = nk * 128;                    // bytes between the two 64-channel halves of a Z image
       bool ok = true;
-      int n = 0, prev_bh = -1, zc = 0;
-      for (int it = it0; it < it1 && ok; ++it, ++n) {
-        const XItem x = x_decode(dm, P.h0, it, tm_tiles, th_tiles);
+      int prev_bh = -1, zc = 0;
+      // S = Y (Zhi + Zlo)^T of the CTA's tile n, K = head_dim
+      auto scores = [&](int n, const XItem& x) -> bool {
         if (x.bh != prev_bh) {                            // the head's summaries have arrived
           XPROF_T0(x4);
-          ok = mbar_wait(&sh.z_ready, zc & 1, abort_flag); ++zc; prev_bh = x.bh;
+          if (!mbar_wait(&sh.z_ready, zc & 1, abort_flag)) return false;
           XPROF_ADD(4, x4);
-          if (!ok) break;
+          ++zc; prev_bh = x.bh;
         }
         const int slot = n % YB;
         XPROF_T0(x1);
-        ok = mbar_wait(&sh.y_full[slot], (n / YB) & 1, abort_flag);
+        if (!mbar_wait(&sh.y_full[slot], (n / YB) & 1, abort_flag)) return false;
         XPROF_ADD(1, x1);
-        if (!ok) break;
         tc_fence_after();
-        const uint32_t ybase = smem_u32(sY + slot * X_TILE_BYTES);
+        const uint32_t ybase = smem_u32(sY + slot * X_TILE_BYTES), s_tm = tmem + (SB == 2 ? (n & 1) * 64 : 0);
 #pragma unroll
-        for (int k = 0; k < XD / 16; ++k) {               // S = Y (Zhi + Zlo)^T, K = head_dim
+        for (int k = 0; k < XD / 16; ++k) {
           const uint64_t a = smem_desc_sw128(ybase + (k >> 2) * X_HALF + (k & 3) * 32, 16, 1024);
           const uint32_t zo = (k >> 2) * zhalf + (k & 3) * 32;
-          umma_ss(tmem, a, smem_desc_sw128(zhi + zo, 16, 1024), idesc1, k > 0 ? 1u : 0u);
-          umma_ss(tmem, a, smem_desc_sw128(zlo + zo, 16, 1024), idesc1, 1u);
+          umma_ss(s_tm, a, smem_desc_sw128(zhi + zo, 16, 1024), idesc1, k > 0 ? 1u : 0u);
+          umma_ss(s_tm, a, smem_desc_sw128(zlo + zo, 16, 1024), idesc1, 1u);
         }
-        umma_commit(&sh.s_full);
-        if (YB == 1) umma_commit(&sh.y_empty[slot]);      // single buffer: free for the next load once the scores are done
+        umma_commit(&sh.s_full[n & 1]);
+        if (REREAD) umma_commit(&sh.y_empty[slot]);       // the tile has been read
+        return true;
+      };
+      XItem x = x_decode(P.h0, it0, tm_tiles, th_tiles);
+      if (it0 < it1) ok = scores(0, x);
+      for (int it = it0, n = 0; it < it1 && ok; ++it, ++n) {
+        // the next tile's scores ahead of this tile's update: into the other buffer, and against the same summaries
+        const bool more = it + 1 < it1;
+        XItem next = x;
+        x_next(next, tm_tiles, th_tiles);
+        const bool ahead = SB == 2 && more && next.bh == x.bh;
+        if (ahead) ok = scores(n + 1, next);
         XPROF_T0(x2);
-        ok = mbar_wait(&sh.p_full, n & 1, abort_flag);
+        if (ok) ok = mbar_wait(&sh.p_full[n & 1], (n >> 1) & 1, abort_flag);
         XPROF_ADD(2, x2);
         XPROF_T0(x3);
         if (ok && n >= 1) ok = mbar_wait(&sh.d_empty, (n - 1) & 1, abort_flag);
         XPROF_ADD(3, x3);
         if (!ok) break;
         tc_fence_after();
-        for (int k = 0; k < nk / 16; ++k) {               // D = (Phi + Plo) (Zhi + Zlo) without lo*lo, K = keys
+        const uint32_t p_tm = tmem + (SB == 2 ? (n & 1) * 64 : 0);
+        uint32_t acc = 0;
+#pragma unroll
+        for (int k = 0; k < NK; ++k) {                    // D = (Phi + Plo) (Zhi + Zlo) without lo*lo, K = keys
+          if (sh.keys[x.band - 1][k] == 0) continue;
           const uint64_t bh_ = smem_desc_sw128(zhi + k * 2048, zhalf, 1024);
-          umma_ts(tmem + 128, tmem + k * 8, bh_, idesc2, k > 0 ? 1u : 0u);
-          umma_ts(tmem + 128, tmem + k * 8, smem_desc_sw128(zlo + k * 2048, zhalf, 1024), idesc2, 1u);
-          const uint32_t plo = NK32 >= 2 ? (k < 2 ? 96u : (k < 4 ? 112u : 80u)) + (k & 1) * 8 : 48u + k * 8;
-          umma_ts(tmem + 128, tmem + plo, bh_, idesc2, 1u);
+          umma_ts(tmem + 128, p_tm + k * 16, bh_, idesc2, acc);
+          umma_ts(tmem + 128, p_tm + k * 16, smem_desc_sw128(zlo + k * 2048, zhalf, 1024), idesc2, 1u);
+          umma_ts(tmem + 128, p_tm + k * 16 + 8, bh_, idesc2, 1u);
+          acc = 1;
         }
         umma_commit(&sh.d_full);
-        if (it + 1 < it1 && x_decode(dm, P.h0, it + 1, tm_tiles, th_tiles).bh != x.bh) umma_commit(&sh.z_empty);
+        if (more && next.bh != x.bh) umma_commit(&sh.z_empty);
+        if (more && !ahead) ok = scores(n + 1, next);
+        x = next;
       }
     }
   } else if (warp < 6) {
@@ -229,204 +267,223 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
     const int tid = row;                                  // 0..127 among the softmax threads
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const float sl2 = rsqrtf((float)XD) * 1.4426950408889634f;
-    // Keys a token attends to, as bit masks per 32-key chunk and band: the 3m summaries without the token's own
-    // band's and without those of an empty mid band.
-    uint32_t keys_mid[NK32], keys_high[NK32];
-#pragma unroll
-    for (int c3 = 0; c3 < NK32; ++c3) {
-      uint32_t a = 0, b = 0;
-      for (int i = 0; i < 32; ++i) {
-        const int j = c3 * 32 + i;
-        const bool live = j < 3 * m && !(dm.Nmid == 0 && j >= m && j < 2 * m);
-        if (live && (j < m || j >= 2 * m)) a |= 1u << i;
-        if (live && j < 2 * m) b |= 1u << i;
-      }
-      keys_mid[c3] = a; keys_high[c3] = b;
-    }
     bool ok = true;
     int n = 0;
-    for (int it = it0; it < it1 && ok; ++it, ++n) {
-      const XItem x = x_decode(dm, P.h0, it, tm_tiles, th_tiles);
+    XItem x = x_decode(P.h0, it0, tm_tiles, th_tiles);
+    for (int it = it0; it < it1 && ok; ++it, ++n, x_next(x, tm_tiles, th_tiles)) {
       // ---- softmax over the 2m summaries of the other bands
       XPROF_T0(x6);
-      ok = __all_sync(0xffffffffu, mbar_wait(&sh.s_full, n & 1, abort_flag));
+      ok = __all_sync(0xffffffffu, mbar_wait(&sh.s_full[n & 1], (n >> 1) & 1, abort_flag));
       if (tid == 0) XPROF_ADD(6, x6);
       if (!ok) break;
       XPROF_T0(x7);
       tc_fence_after();
-      uint32_t keys[NK32];
-#pragma unroll
-      for (int c3 = 0; c3 < NK32; ++c3) keys[c3] = x.band == 1 ? keys_mid[c3] : keys_high[c3];
-      if (NK32 >= 2) {
-        // first sweep: the row maximum
-        float mx = -INFINITY;
-#pragma unroll
-        for (int c3 = 0; c3 < NK32; ++c3) {
-          uint32_t r[32];
-          tmem_ld32(tmem + lane_addr + c3 * 32, r);
-          tmem_wait_ld();
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            if (keys[c3] & (1u << i)) mx = fmaxf(mx, __uint_as_float(r[i]));
-          }
-        }
-        const float mb = mx * sl2;
-        // second sweep: exponentials and their sum, P (unnormalised, bf16 hi + lo) chunk by chunk
-        float den0 = 0.f, den1 = 0.f;
-#pragma unroll
-        for (int c3 = 0; c3 < NK32; ++c3) {
-          uint32_t r[32];
-          tmem_ld32(tmem + lane_addr + c3 * 32, r);
-          tmem_wait_ld();
-          uint32_t ph[16], pl[16];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            float p0 = 0.f, p1 = 0.f;
-            if (keys[c3] & (1u << (2 * i))) p0 = ex2f_approx(fmaf(__uint_as_float(r[2 * i]), sl2, -mb));
-            if (keys[c3] & (2u << (2 * i))) p1 = ex2f_approx(fmaf(__uint_as_float(r[2 * i + 1]), sl2, -mb));
-            den0 += p0; den1 += p1;
-            const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
-            ph[i] = *(const uint32_t*)&h2;
-            const __nv_bfloat162 l2 = __floats2bfloat162_rn(p0 - __uint_as_float(ph[i] << 16), p1 - __uint_as_float(ph[i] & 0xffff0000u));
-            pl[i] = *(const uint32_t*)&l2;
-          }
-          tmem_st16(tmem + lane_addr + c3 * 16, ph);                              // over scores already read
-          tmem_st16(tmem + lane_addr + (c3 == 0 ? 96 : (c3 == 1 ? 112 : 80)), pl);
-        }
-        sh.inv[n & 1][row] = 1.f / (den0 + den1);
-      } else {
-      // all scores of the row into registers (they are overwritten by P below)
-        uint32_t sc[NK32 * 32];
-#pragma unroll
-        for (int c3 = 0; c3 < NK32; ++c3) {
-          uint32_t r[32];
-          tmem_ld32(tmem + lane_addr + c3 * 32, r);
-#pragma unroll
-          for (int i = 0; i < 32; ++i) sc[c3 * 32 + i] = r[i];
-        }
+      const uint32_t s_tm = tmem + lane_addr + (SB == 2 ? (n & 1) * 64 : 0);
+      const uint32_t* masks = sh.keys[x.band - 1];
+      // first sweep: the row maximum
+      float mx0 = -INFINITY, mx1 = -INFINITY;
+#pragma unroll 1
+      for (int c = 0; c < NK; ++c) {
+        const uint32_t keys = masks[c];
+        if (keys == 0) continue;
+        uint32_t r[16];
+        tmem_ld16(s_tm + c * 16, r);
         tmem_wait_ld();
-        float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+        if (keys == 0xffffu) {
 #pragma unroll
-        for (int j = 0; j < NK32 * 32; ++j)
-          if (keys[j >> 5] & (1u << (j & 31))) mx4[j & 3] = fmaxf(mx4[j & 3], __uint_as_float(sc[j]));
-        const float mb = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * sl2;
-        float den4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-        for (int j = 0; j < NK32 * 32; ++j) {
-          float pv = 0.f;
-          if (keys[j >> 5] & (1u << (j & 31))) pv = ex2f_approx(fmaf(__uint_as_float(sc[j]), sl2, -mb));
-          den4[j & 3] += pv;
-          sc[j] = __float_as_uint(pv);
-        }
-        const float inv = 1.f / ((den4[0] + den4[1]) + (den4[2] + den4[3]));
-#pragma unroll
-        for (int c3 = 0; c3 < NK32; ++c3) {
-          if (c3 * 32 < nk) {
-            uint32_t ph[16], pl[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float p0 = __uint_as_float(sc[c3 * 32 + 2 * i]) * inv, p1 = __uint_as_float(sc[c3 * 32 + 2 * i + 1]) * inv;
-              const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
-              ph[i] = *(const uint32_t*)&h2;
-              const __nv_bfloat162 l2 = __floats2bfloat162_rn(p0 - __uint_as_float(ph[i] << 16), p1 - __uint_as_float(ph[i] & 0xffff0000u));
-              pl[i] = *(const uint32_t*)&l2;
-            }
-            tmem_st16(tmem + lane_addr + c3 * 16, ph);
-            tmem_st16(tmem + lane_addr + 48 + c3 * 16, pl);
+          for (int i = 0; i < 16; i += 4) {
+            mx0 = max3f(mx0, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+            mx1 = max3f(mx1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
           }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (keys & (1u << i)) mx0 = fmaxf(mx0, __uint_as_float(r[i]));
         }
       }
+      const float mb = fmaxf(mx0, mx1) * sl2;
+      const float2 sl22 = make_float2(sl2, sl2), nmb2 = make_float2(-mb, -mb), minus = make_float2(-1.f, -1.f);
+      // second sweep: exponentials and their sum, P (unnormalised, bf16 hi + lo) over the chunk's own scores
+      float2 den = make_float2(0.f, 0.f);
+#pragma unroll 1
+      for (int c = 0; c < NK; ++c) {
+        const uint32_t keys = masks[c];
+        if (keys == 0) continue;
+        uint32_t r[16], ph[8], pl[8];
+        tmem_ld16(s_tm + c * 16, r);
+        tmem_wait_ld();
+        if (keys != 0xffffu) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            if (!(keys & (1u << i))) r[i] = 0xff800000u;       // (-inf: exponential 0)
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float2 arg = __ffma2_rn(make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), sl22, nmb2);
+          const float2 p = make_float2(ex2f_approx(arg.x), ex2f_approx(arg.y));
+          den = __fadd2_rn(den, p);
+          const __nv_bfloat162 h2 = __floats2bfloat162_rn(p.x, p.y);
+          ph[i] = *(const uint32_t*)&h2;
+          const float2 l = __ffma2_rn(make_float2(__uint_as_float(ph[i] << 16), __uint_as_float(ph[i] & 0xffff0000u)), minus, p);
+          const __nv_bfloat162 l2 = __floats2bfloat162_rn(l.x, l.y);
+          pl[i] = *(const uint32_t*)&l2;
+        }
+        tmem_st8(s_tm + c * 16, ph);
+        tmem_st8(s_tm + c * 16 + 8, pl);
+      }
+      sh.inv[n & 3][row] = 1.f / (den.x + den.y);
       tmem_wait_st();
       tc_fence_before();
-      mbar_arrive(&sh.p_full);
+      mbar_arrive(&sh.p_full[n & 1]);
       if (tid == 0) XPROF_ADD(7, x7);
     }
   } else {
     // ------------------------------------------------------------------ store warps
-    const int quarter = warp & 3;
-    const int row = quarter * 32 + lane;
+    const int quarter = warp & 3;                              // 32 tokens of the tile
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+    uint8_t* st = sStage + quarter * x_stage_bytes(REREAD);
     bool ok = true;
     int n = 0;
-    for (int it = it0; it < it1 && ok; ++it, ++n) {
-      const XItem x = x_decode(dm, P.h0, it, tm_tiles, th_tiles);
-      const int slot = n % YB;
+    XItem x = x_decode(P.h0, it0, tm_tiles, th_tiles);
+    for (int it = it0; it < it1 && ok; ++it, ++n, x_next(x, tm_tiles, th_tiles)) {
       const long long n_band = x.band == 1 ? dm.Nmid : dm.Nhigh;
-      const long long p = (long long)x.tile * XT + row;
-      // ---- residual add and store (where the rows go does not depend on the data: looked up before the wait)
-      const bool valid = p < n_band;
+      // ---- where the lane's tokens (8 i + r8 of the warp's) come from and go: looked up before the wait
       XPROF_T0(x14);
-      int f = valid ? (x.band == 1 ? P.pos_mid[p] : P.pos_high[p]) : -1;
-      if (valid && !FF_DBG_OK(f >= 0 && f < dm.N && x.bh >= P.h0 && x.bh < P.h0 + P.g, P.status, 3)) f = -1;   // (debug build)
-      // lane L stores for rows 8 i + L/4 of its warp: fetch those rows' grid positions
-      int fpos[4];
+      const int* pos = x.band == 1 ? P.pos_mid : P.pos_high;
+      if (!REREAD) {
+        const long long p = (long long)x.tile * XT + quarter * 32 + lane;
+        int f = p < n_band ? __ldg(pos + p) : -1;
+        if (f >= 0 && !FF_DBG_OK(f < dm.N && x.bh >= P.h0 && x.bh < P.h0 + P.g, P.status, 3)) f = -1;   // (debug build)
+        f *= XD;                                           // element offset of the token's row in the head's grid, or < 0
+        // the rows this lane stores pieces of: 8 i + lane / 4
+        int out[4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) fpos[i] = __shfl_sync(0xffffffffu, f, 8 * i + (lane >> 2));
-      const size_t obase = (size_t)(x.bh - P.h0) * dm.N * XD;
-      const uint8_t* yrow = sY + slot * X_TILE_BYTES + row * 128;
-      // (single buffer) this token's row in global memory; rows past the band end are never stored
-      const bool exec_g = P.alloc[x.bh] & (1 << x.band);
-      const __nv_bfloat16* grow = P.src[(x.band == 1 ? 0 : 2) + (exec_g ? 0 : 1)] +
-                                  ((size_t)(exec_g ? x.bh : 2 * dm.BH + x.bh) * n_band + (valid ? p : 0)) * XD;
-      uint8_t* st_hi = sh.stage[quarter][0];
-      uint8_t* st_lo = sh.stage[quarter][1];
-      if (row == 0) XPROF_ADD(14, x14);
+        for (int i = 0; i < 4; ++i) out[i] = __shfl_sync(0xffffffffu, f, 8 * i + (lane >> 2));
+        const size_t obase = (size_t)(x.bh - P.h0) * dm.N * XD;
+        __nv_bfloat16* const grid_hi = P.grid_hi + obase + (lane & 3) * 8;
+        uint8_t* const grid_lo = P.grid_lo + obase + (lane & 3) * 8;
+        const int slot = n % YB, row = quarter * 32 + lane;
+        const uint8_t* yrow = sY + slot * X_TILE_BYTES + row * 128;
+        if (threadIdx.x == 192) XPROF_ADD(14, x14);
+        XPROF_T0(x9);
+        ok = __all_sync(0xffffffffu, mbar_wait(&sh.d_full, n & 1, abort_flag));
+        if (threadIdx.x == 192) XPROF_ADD(9, x9);
+        if (!ok) break;
+        XPROF_T0(x10);
+        tc_fence_after();
+        const float2 s2 = make_float2(sh.inv[n & 3][row], sh.inv[n & 3][row]);
+#pragma unroll 4
+        for (int q = 0; q < XD / 32; ++q) {                // 32 channels
+          uint32_t r[32];
+          tmem_ld32(tmem + lane_addr + 128 + q * 32, r);
+          tmem_wait_ld();
+          if (q == XD / 32 - 1) {                          // D has been read
+            tc_fence_before();
+            mbar_arrive(&sh.d_empty);
+          }
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {                    // 8 channels: 16 bytes of the swizzled token row
+            const int c = q * 4 + v;
+            const uint4 yv = *(const uint4*)(yrow + (c >> 3) * X_HALF + (((c & 7) ^ (row & 7)) << 4));
+            const uint32_t yw[4] = {yv.x, yv.y, yv.z, yv.w};
+            uint32_t hi[4], u[8];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const float2 d = make_float2(__uint_as_float(r[8 * v + 2 * k]), __uint_as_float(r[8 * v + 2 * k + 1]));
+              const float2 w = __ffma2_rn(d, s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
+              u[2 * k] = __float_as_uint(w.x) + 0x80u;
+              u[2 * k + 1] = __float_as_uint(w.y) + 0x80u;
+              hi[k] = __byte_perm(u[2 * k], u[2 * k + 1], 0x7632);
+            }
+            *(uint4*)(st + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            // (lo: 32 bytes per row, 8-byte pieces XOR-swizzled with row / 4)
+            *(uint2*)(st + 2048 + lane * 32 + ((v ^ ((lane >> 2) & 3)) << 3)) =
+                make_uint2(__byte_perm(__byte_perm(u[0], u[1], 0x0051), __byte_perm(u[2], u[3], 0x0051), 0x5410),
+                           __byte_perm(__byte_perm(u[4], u[5], 0x0051), __byte_perm(u[6], u[7], 0x0051), 0x5410));
+          }
+          if (q == XD / 32 - 1) mbar_arrive(&sh.y_empty[slot]);
+          __syncwarp();
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int t = 8 * i + (lane >> 2), piece = lane & 3;
+            if (out[i] >= 0) {
+              *(uint4*)(grid_hi + out[i] + q * 32) = *(const uint4*)(st + t * 64 + ((piece ^ ((t >> 1) & 3)) << 4));
+              *(uint2*)(grid_lo + out[i] + q * 32) = *(const uint2*)(st + 2048 + t * 32 + ((piece ^ ((t >> 2) & 3)) << 3));
+            }
+          }
+          __syncwarp();
+        }
+        if (threadIdx.x == 192) XPROF_ADD(10, x10);
+        continue;
+      }
+      const int piece = lane & 3, r8 = lane >> 2;          // a lane's 8 channels of 32 and its token of eight, when storing
+      // 16-byte chunk v of token t at v ^ (t mod 8)
+      const uint8_t* st_rd0 = st + r8 * 128 + (((2 * piece) ^ r8) << 4);
+      const uint8_t* st_rd1 = st + r8 * 128 + (((2 * piece + 1) ^ r8) << 4);
+      const long long p0 = (long long)x.tile * XT + quarter * 32 + r8;
+      const bool exec = P.alloc[x.bh] & (1 << x.band);
+      const __nv_bfloat16* yrow = P.src[(x.band == 1 ? 0 : 2) + (exec ? 0 : 1)] +
+                                  ((size_t)(exec ? x.bh : 2 * dm.BH + x.bh) * n_band + p0) * XD + piece * 8;
+      const size_t obase = (size_t)(x.bh - P.h0) * dm.N * XD + piece * 8;
+      __nv_bfloat16* const grid_hi = P.grid_hi + obase;
+      uint8_t* const grid_lo = P.grid_lo + obase;
+      int out[4];                                              // element offset of the token's row in the head's grid, or -1
+      uint4 yv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        int f = p0 + 8 * i < n_band ? __ldg(pos + p0 + 8 * i) : -1;
+        if (f >= 0 && !FF_DBG_OK(f < dm.N && x.bh >= P.h0 && x.bh < P.h0 + P.g, P.status, 3)) f = -1;   // (debug build)
+        out[i] = f * XD;
+        yv[i] = f >= 0 ? __ldg((const uint4*)(yrow + 8 * i * XD)) : make_uint4(0, 0, 0, 0);
+      }
+      if (threadIdx.x == 192) XPROF_ADD(14, x14);
       XPROF_T0(x9);
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.d_full, n & 1, abort_flag));
-      if (row == 0) XPROF_ADD(9, x9);
+      if (threadIdx.x == 192) XPROF_ADD(9, x9);
       if (!ok) break;
       XPROF_T0(x10);
       tc_fence_after();
-      const float dscale = NK32 >= 2 ? sh.inv[n & 1][row] : 1.f;    // (two-sweep variants: P was left unnormalised)
-#pragma unroll
+      const float* inv = sh.inv[n & 3] + quarter * 32 + r8;
+#pragma unroll 1
       for (int q = 0; q < XD / 32; ++q) {
-        uint32_t r[32];
-        XPROF_T0(x11);
-        tmem_ld32(tmem + lane_addr + 128 + q * 32, r);
-        tmem_wait_ld();
-        if (row == 0) XPROF_ADD(11, x11);
-        XPROF_T0(x12);
+        {
+          uint32_t r[32];
+          tmem_ld32(tmem + lane_addr + 128 + q * 32, r);
+          tmem_wait_ld();
 #pragma unroll
-        for (int v4 = 0; v4 < 4; ++v4) {
-          // channels 32q + 8v4 .. +7 of this token: one 16-byte chunk of the swizzled Y tile
-          const int cch = q * 4 + v4;                    // 16-byte chunk index along the row, 0..15
-          const uint4 yv = YB == 1 ? __ldg((const uint4*)(grow + cch * 8))
-                                   : *(const uint4*)(yrow + (cch >> 3) * X_HALF + (((cch & 7) ^ (row & 7)) << 4));
-          const uint32_t yw[4] = {yv.x, yv.y, yv.z, yv.w};
-          // three-byte form: the value rounded to 24 bits; hi = its upper 16 bits, lo = the next byte
-          uint32_t hi[4], u[8];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            u[2 * i] = __float_as_uint(fmaf(__uint_as_float(r[v4 * 8 + 2 * i]), dscale, __uint_as_float(yw[i] << 16))) + 0x80u;
-            u[2 * i + 1] = __float_as_uint(fmaf(__uint_as_float(r[v4 * 8 + 2 * i + 1]), dscale, __uint_as_float(yw[i] & 0xffff0000u))) + 0x80u;
-            hi[i] = __byte_perm(u[2 * i], u[2 * i + 1], 0x7632);
-          }
-          const uint32_t lo0 = __byte_perm(__byte_perm(u[0], u[1], 0x0051), __byte_perm(u[2], u[3], 0x0051), 0x5410);
-          const uint32_t lo1 = __byte_perm(__byte_perm(u[4], u[5], 0x0051), __byte_perm(u[6], u[7], 0x0051), 0x5410);
-          *(uint4*)(st_hi + lane * X_STG_PITCH + ((v4 ^ ((lane >> 1) & 3)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          // (lo: 32 bytes per row, 8-byte pieces XOR-swizzled with row / 4)
-          *(uint2*)(st_lo + lane * 32 + ((v4 ^ ((lane >> 2) & 3)) << 3)) = make_uint2(lo0, lo1);
+          for (int v = 0; v < 8; ++v)
+            *(uint4*)(st + lane * 128 + ((v ^ (lane & 7)) << 4)) = make_uint4(r[4 * v], r[4 * v + 1], r[4 * v + 2], r[4 * v + 3]);
+        }
+        if (q == XD / 32 - 1) {                            // D has been read
+          tc_fence_before();
+          mbar_arrive(&sh.d_empty);
         }
         __syncwarp();
-        if (row == 0) XPROF_ADD(12, x12);
-        XPROF_T0(x13);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const int rr = 8 * i + (lane >> 2), piece = lane & 3;      // row of the warp, 16-byte piece of its 64 bytes
-          if (fpos[i] >= 0) {
-            const size_t o = obase + (size_t)fpos[i] * XD + q * 32 + piece * 8;
-            const int so = rr * X_STG_PITCH + ((piece ^ ((rr >> 1) & 3)) << 4);
-            *(uint4*)(P.grid_hi + o) = *(const uint4*)(st_hi + so);
-            *(uint2*)(P.grid_lo + o) = *(const uint2*)(st_lo + rr * 32 + ((piece ^ ((rr >> 2) & 3)) << 3));
+          const float4 d0 = *(const float4*)(st_rd0 + i * 1024), d1 = *(const float4*)(st_rd1 + i * 1024);
+          const float2 s2 = make_float2(inv[8 * i], inv[8 * i]);
+          const float2 dd[4] = {make_float2(d0.x, d0.y), make_float2(d0.z, d0.w), make_float2(d1.x, d1.y), make_float2(d1.z, d1.w)};
+          const uint32_t yw[4] = {yv[i].x, yv[i].y, yv[i].z, yv[i].w};
+          uint32_t hi[4], u[8];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float2 v = __ffma2_rn(dd[k], s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
+            u[2 * k] = __float_as_uint(v.x) + 0x80u;
+            u[2 * k + 1] = __float_as_uint(v.y) + 0x80u;
+            hi[k] = __byte_perm(u[2 * k], u[2 * k + 1], 0x7632);
+          }
+          if (q + 1 < XD / 32 && out[i] >= 0) yv[i] = __ldg((const uint4*)(yrow + 8 * i * XD + (q + 1) * 32));
+          if (out[i] >= 0) {
+            *(uint4*)(grid_hi + out[i] + q * 32) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *(uint2*)(grid_lo + out[i] + q * 32) =
+                make_uint2(__byte_perm(__byte_perm(u[0], u[1], 0x0051), __byte_perm(u[2], u[3], 0x0051), 0x5410),
+                           __byte_perm(__byte_perm(u[4], u[5], 0x0051), __byte_perm(u[6], u[7], 0x0051), 0x5410));
           }
         }
         __syncwarp();
-        if (row == 0) XPROF_ADD(13, x13);
       }
-      tc_fence_before();
-      mbar_arrive(&sh.d_empty);
-      if (YB > 1) mbar_arrive(&sh.y_empty[slot]);
-      if (row == 0) XPROF_ADD(10, x10);
+      if (threadIdx.x == 192) XPROF_ADD(10, x10);
     }
   }
 
@@ -480,10 +537,11 @@ bool ffk_exchange_tc_supported(const FFDims& dm) {
 
 cudaError_t ffk_exchange_tc_init() {
   cudaError_t e = cudaSuccess;
-  // (the largest: a token tile, 96 keys as hi and lo images)
-  const int most = 2 * X_TILE_BYTES + 4 * 96 * 128 + (int)sizeof(XShared) + 1024;
-#define FF_XCH(NK, D) if (e == cudaSuccess) e = cudaFuncSetAttribute(exchange_tc_kernel<NK, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
-  FF_XCH(1, 128); FF_XCH(2, 128); FF_XCH(3, 128); FF_XCH(1, 64); FF_XCH(2, 64); FF_XCH(3, 64);
+  const int most = 113 * 1024;
+#define FF_XCH(NK)                                                                                                                \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(exchange_tc_kernel<NK, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);  \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(exchange_tc_kernel<NK, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+  FF_XCH(1); FF_XCH(2); FF_XCH(3); FF_XCH(4); FF_XCH(5); FF_XCH(6);
 #undef FF_XCH
   return e;
 }
@@ -528,10 +586,11 @@ cudaError_t ffk_exchange_tc(ff_plan* p, int h0, int g, void* grid_hi, void* grid
   P.h0 = h0; P.g = g; P.nkeys = ff_exchange_keys(dm.m); P.status = p->buf.status;
   P.src[0] = (const __nv_bfloat16*)p->buf.y_mid; P.src[1] = (const __nv_bfloat16*)p->buf.spec_mid;
   P.src[2] = (const __nv_bfloat16*)p->buf.y_high; P.src[3] = (const __nv_bfloat16*)p->buf.spec_high;
-  // Two CTAs per SM; the token tile is double-buffered if both still fit in shared memory
+  // Two CTAs per SM, two token tiles each up to 64 keys
   const int per_sm = 2;
-  P.ybufs = (2 * X_TILE_BYTES + 4 * P.nkeys * 128 + sizeof(XShared) + 2048) * per_sm <= 227 * 1024 ? 2 : 1;
-  const size_t smem = P.ybufs * X_TILE_BYTES + 4 * P.nkeys * 128 + sizeof(XShared) + 1024;
+  const bool reread = P.nkeys > 64;
+  P.ybufs = reread ? 1 : 2;
+  const size_t smem = P.ybufs * X_TILE_BYTES + 4 * (size_t)P.nkeys * 128 + 4 * x_stage_bytes(reread) + sizeof(XShared) + 1024;
   const long long tiles = (long long)g * ((dm.Nmid + XT - 1) / XT + (dm.Nhigh + XT - 1) / XT);
   const int grid = tiles < per_sm * p->sm_count ? (int)tiles : per_sm * p->sm_count;
   const CUtensorMap& m0 = *(const CUtensorMap*)p->tmap_x[0];
@@ -540,13 +599,17 @@ cudaError_t ffk_exchange_tc(ff_plan* p, int h0, int g, void* grid_hi, void* grid
   const CUtensorMap& m3 = *(const CUtensorMap*)p->tmap_x[3];
   p->launches += 1;
 #define FF_XCH(NK, D) return ff_launch(exchange_tc_kernel<NK, D>, dim3(grid), dim3(X_THREADS), smem, st, m0, m1, m2, m3, P)
-  if (dm.d == 128) {
-    if (P.nkeys <= 32) FF_XCH(1, 128);
-    if (P.nkeys <= 64) FF_XCH(2, 128);
-    FF_XCH(3, 128);
+#define FF_XCH_D(D)                     \
+  switch (P.nkeys / 16) {               \
+    case 1: FF_XCH(1, D);               \
+    case 2: FF_XCH(2, D);               \
+    case 3: FF_XCH(3, D);               \
+    case 4: FF_XCH(4, D);               \
+    case 5: FF_XCH(5, D);               \
+    default: FF_XCH(6, D);              \
   }
-  if (P.nkeys <= 32) FF_XCH(1, 64);
-  if (P.nkeys <= 64) FF_XCH(2, 64);
-  FF_XCH(3, 64);
+  if (dm.d == 128) FF_XCH_D(128)
+  FF_XCH_D(64)
+#undef FF_XCH_D
 #undef FF_XCH
 }
