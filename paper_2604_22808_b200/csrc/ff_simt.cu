@@ -55,13 +55,13 @@ __device__ __forceinline__ void store_coefficient(const FFDims& dm, float* spec_
 // MODE 2: fp32 scratch -> band-major coefficient buffers (forward, last axis = t).
 // MODE 3: fp32 scratch -> the caller's `out` tensor (storage type).
 //
-// A warp takes 128 neighbouring columns (o, c) and eight outputs along the axis: 32 accumulators per thread against
-// one 16-byte load of the line and two broadcast reads of the matrix in shared memory per step.  The warps of a block
-// that share a column tile find its lines in L1, so no tile is staged, and any n keeps all lanes busy (a block used to
-// own 64 columns, of which a 9-long axis kept 32 threads busy: 134 us for the t pass of 12 x 9 x 30 x 40 x 64 floats).
+// A block stages tiles of n positions x V groups of four neighbouring columns (o, c) with asynchronous copies, the next
+// tile while it works on this one; a thread computes eight outputs of one group, V = 256 / (output groups), so any n
+// keeps the lanes busy.  Bound by the FMA pipe next to the shared-memory reads (one of the tile, two broadcasts of the
+// matrix per 32 FMA); straight from global memory, as before, it waited for loads two thirds of the time (w pass of
+// 12 x 9 x 30 x 40 x 64 floats 44 us).
 // ------------------------------------------------------------------------------------------------
 constexpr int DCT_THREADS = 256;
-constexpr int DCT_COLS = 128;    // columns of a warp's item
 
 struct DctPassParams {
   const void* src[3];   // MODE 0: Q, K, V; otherwise src[0] = scratch
@@ -70,7 +70,9 @@ struct DctPassParams {
   int n, inner, outer;
   int group_start;      // first tensor-head index of this launch
   int BH;
-  int tiles;            // column tiles of a tensor-head
+  int V, tiles;         // column groups per tile; tiles of a tensor-head
+  int nbuf;             // tile buffers: 2, or 1 where two would leave an SM with a single block
+  int group;            // tensor-heads of the launch
   long long N_d;        // elements per tensor-head
   FFDims dm;
   // MODE 2
@@ -86,71 +88,106 @@ __device__ __forceinline__ void stage_matrix(float* mt, const float* mat_t, int 
   }
 }
 
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool on) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+               ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
 template <typename ST, int MODE>
 __global__ void __launch_bounds__(DCT_THREADS, 3) dct_pass_kernel(const __grid_constant__ DctPassParams P) {
   extern __shared__ float mt[];
-  const int n = P.n, npad = (n + 7) & ~7, groups = npad / 8;
+  const int n = P.n, npad = (n + 7) & ~7, groups = npad / 8, V = P.V;
+  float* buf = mt + n * npad;               // nbuf x [n][4 V]
   stage_matrix(mt, P.mat_t, n, npad);
   ff_pdl_wait();
-  if (MODE == 0 && P.clear && blockIdx.x == 0 && blockIdx.y == 0)
+  if (MODE == 0 && P.clear && blockIdx.x == 0)
     for (int i = threadIdx.x; i < P.dm.B * 3 * P.dm.d; i += DCT_THREADS) P.clear[i] = 0.0;
-  __syncthreads();
-  const int gi = blockIdx.y;                // tensor-head inside the group
-  const int th = P.group_start + gi;        // global tensor-head index: tensor * BH + bh
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned inner = (unsigned)P.inner, cols = inner * (unsigned)P.outer;
-  const unsigned items = (unsigned)P.tiles * (unsigned)groups;
-  for (unsigned item = blockIdx.x * (DCT_THREADS / 32) + warp; item < items; item += gridDim.x * (DCT_THREADS / 32)) {
-    const unsigned tile = item / (unsigned)groups;
-    const int g = (int)(item - tile * (unsigned)groups);
-    const unsigned col = tile * DCT_COLS + lane * 4;
-    if (col >= cols) continue;
-    const unsigned o = col / inner, c = col - o * inner;
-    const size_t line = (size_t)o * n * inner + c;
-    float4 acc[8];
+  const int total = P.tiles * P.group;
+  const int g = (int)threadIdx.x / V, v = (int)threadIdx.x - g * V, rstep = DCT_THREADS / V;
+  auto load = [&](int t, float* dst) {
+    if (t < total && g < rstep) {
+      const int gi = t / P.tiles, th = P.group_start + gi;     // tensor-head inside the group; tensor * BH + bh
+      const unsigned col = (unsigned)((t - gi * P.tiles) * V + v) * 4;
+      const bool on = col < cols;
+      const unsigned o = on ? col / inner : 0, c = on ? col - o * inner : 0;
+      const size_t line = (size_t)o * n * inner + c;
+      if (MODE == 0 && sizeof(ST) == 2) {
+        const ST* src = (const ST*)P.src[th / P.BH] + (size_t)(th % P.BH) * P.N_d + line;
+#pragma unroll 4
+        for (int b = g; b < n; b += rstep) *(float4*)(dst + (b * V + v) * 4) = ld4(src + (size_t)b * inner);
+      } else {
+        const float* src = (MODE == 0 ? (const float*)P.src[th / P.BH] + (size_t)(th % P.BH) * P.N_d : (const float*)P.src[0] + (size_t)gi * P.N_d) + line;
+#pragma unroll 4
+        for (int b = g; b < n; b += rstep) cp_async16(dst + (b * V + v) * 4, src + (size_t)b * inner, on);
+      }
+    }
+    cp_async_commit();
+  };
+  int cur = 0;
+  load(blockIdx.x, buf);
+  for (int t = blockIdx.x; t < total; t += gridDim.x) {
+    const float* tile = buf + (size_t)cur * n * V * 4;
+    if (P.nbuf == 2) {
+      load(t + gridDim.x, buf + (size_t)(cur ^ 1) * n * V * 4);
+      cp_async_wait<1>();
+    } else {
+      cp_async_wait<0>();
+    }
+    __syncthreads();
+    const int gi = t / P.tiles, th = P.group_start + gi;
+    const unsigned col = (unsigned)((t - gi * P.tiles) * V + v) * 4;
+    if (g < groups && col < cols) {
+      const unsigned o = col / inner, c = col - o * inner;
+      const size_t line = (size_t)o * n * inner + c;
+      float4 acc[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto sum_line = [&](auto* src) {
+      for (int i = 0; i < 8; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       const float* m = mt + g * 8;
-#pragma unroll 8
+      const float* xs = tile + v * 4;
+#pragma unroll 4
       for (int b = 0; b < n; ++b) {
-        const float4 x = ld4(src + (size_t)b * inner);
+        const float4 x = *(const float4*)(xs + b * V * 4);
         const float4 m0 = *(const float4*)(m + b * npad), m1 = *(const float4*)(m + b * npad + 4);
         fma4(acc[0], m0.x, x); fma4(acc[1], m0.y, x); fma4(acc[2], m0.z, x); fma4(acc[3], m0.w, x);
         fma4(acc[4], m1.x, x); fma4(acc[5], m1.y, x); fma4(acc[6], m1.z, x); fma4(acc[7], m1.w, x);
       }
-    };
-    if (MODE == 0) sum_line((const ST*)P.src[th / P.BH] + (size_t)(th % P.BH) * P.N_d + line);
-    else sum_line((const float*)P.src[0] + (size_t)gi * P.N_d + line);
-    int ch = 0, kw = 0, kh = 0;
-    if (MODE == 2) {                        // a = k_t, column = (k_h, k_w, channel)
-      const unsigned p = c / (unsigned)P.dm.d;
-      ch = (int)(c - p * (unsigned)P.dm.d);
-      kh = (int)(p / (unsigned)P.dm.W); kw = (int)(p - (unsigned)kh * (unsigned)P.dm.W);
-    }
+      int ch = 0, kw = 0, kh = 0;
+      if (MODE == 2) {                      // a = k_t, column = (k_h, k_w, channel)
+        const unsigned p = c / (unsigned)P.dm.d;
+        ch = (int)(c - p * (unsigned)P.dm.d);
+        kh = (int)(p / (unsigned)P.dm.W); kw = (int)(p - (unsigned)kh * (unsigned)P.dm.W);
+      }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int a = g * 8 + i;
-      if (a >= n) break;
-      if (MODE <= 1) st4((float*)P.dst + (size_t)gi * P.N_d + line + (size_t)a * inner, acc[i]);
-      else if (MODE == 3) st4((ST*)P.dst + (size_t)th * P.N_d + line + (size_t)a * inner, acc[i]);
-      else store_coefficient<ST>(P.dm, P.spec_low, P.spec_mid, P.spec_high, th, a, kh, kw, ch, acc[i]);
+      for (int i = 0; i < 8; ++i) {
+        const int a = g * 8 + i;
+        if (a >= n) break;
+        if (MODE <= 1) st4((float*)P.dst + (size_t)gi * P.N_d + line + (size_t)a * inner, acc[i]);
+        else if (MODE == 3) st4((ST*)P.dst + (size_t)th * P.N_d + line + (size_t)a * inner, acc[i]);
+        else store_coefficient<ST>(P.dm, P.spec_low, P.spec_mid, P.spec_high, th, a, kh, kw, ch, acc[i]);
+      }
     }
+    __syncthreads();
+    if (P.nbuf == 2) cur ^= 1; else load(t + gridDim.x, buf);
   }
+  cp_async_wait<0>();
 }
 
 template <typename ST, int MODE>
 cudaError_t launch_dct_pass(ff_plan* p, DctPassParams& P, int group, cudaStream_t st) {
   const int npad = (P.n + 7) & ~7;
-  P.tiles = (int)(((long long)P.inner * P.outer + DCT_COLS - 1) / DCT_COLS);
-  // the three blocks an SM holds, each with as many items as that leaves (the matrix is staged once per block)
-  const long long items = (long long)P.tiles * (npad / 8), want = (items + DCT_THREADS / 32 - 1) / (DCT_THREADS / 32);
-  long long blocks = 3LL * p->sm_count / group;
-  if (blocks < 1) blocks = 1;
-  if (blocks > want) blocks = want;
+  P.V = DCT_THREADS / (npad / 8);
+  P.tiles = (int)(((long long)P.inner * P.outer / 4 + P.V - 1) / P.V);
+  P.group = group;
+  const size_t mat = (size_t)P.n * npad * sizeof(float), tile = (size_t)P.n * P.V * 4 * sizeof(float);
+  P.nbuf = mat + 2 * tile <= 112 * 1024 ? 2 : 1;
+  const size_t smem = mat + P.nbuf * tile;
+  const int per_sm = smem <= 75 * 1024 ? 3 : 2;
+  const long long total = (long long)P.tiles * group, most = (long long)per_sm * p->sm_count;
   p->launches += 1;
-  return ff_launch(dct_pass_kernel<ST, MODE>, dim3((unsigned)blocks, (unsigned)group), dim3(DCT_THREADS),
-                   (size_t)P.n * npad * sizeof(float), st, P);
+  return ff_launch(dct_pass_kernel<ST, MODE>, dim3((unsigned)(total < most ? total : most)), dim3(DCT_THREADS), smem, st, P);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -177,7 +214,12 @@ __global__ void __launch_bounds__(VOL_THREADS) dct_volume_kernel(const __grid_co
   extern __shared__ float4 vol[];                      // [N][2]
   const FFDims& dm = P.dm;
   const int N = (int)dm.N, tid = threadIdx.x;
-  float* mt = (float*)(vol + 2 * N);
+  float* mats = (float*)(vol + 2 * N);                 // the matrices of the three axes, before anything is waited for
+  for (int axis = 0, at = 0; axis < 3; ++axis) {
+    const int n = axis == 2 ? dm.W : (axis == 1 ? dm.H : dm.T), npad = (n + 7) & ~7;
+    stage_matrix(mats + at, P.mat_t[axis], n, npad);
+    at += n * npad;
+  }
   ff_pdl_wait();
   if (!INVERSE && P.clear && blockIdx.x == 0 && blockIdx.y == 0)
     for (int i = tid; i < dm.B * 3 * dm.d; i += VOL_THREADS) P.clear[i] = 0.0;
@@ -188,12 +230,13 @@ __global__ void __launch_bounds__(VOL_THREADS) dct_volume_kernel(const __grid_co
     vol[i] = INVERSE ? ld4((const float*)P.src[0] + (size_t)blockIdx.y * per + o)
                      : ld4((const ST*)P.src[th / dm.BH] + (size_t)(th % dm.BH) * per + o);
   }
+  __syncthreads();
   for (int step = 0; step < 3; ++step) {
     const int axis = INVERSE ? step : 2 - step;
     const int n = axis == 2 ? dm.W : (axis == 1 ? dm.H : dm.T), stride = axis == 2 ? 1 : (axis == 1 ? dm.W : dm.H * dm.W);
     const int npad = (n + 7) & ~7, groups = npad / 8;
-    stage_matrix(mt, P.mat_t[axis], n, npad);
-    __syncthreads();
+    const int at = axis == 0 ? 0 : dm.T * ((dm.T + 7) & ~7) + (axis == 1 ? 0 : dm.H * ((dm.H + 7) & ~7));
+    const float* mt = mats + at;
     const int upl = 2 * groups, lines = N / n;           // units (8 outputs x 4 channels) of a line
     const int lpr = VOL_THREADS / upl;                   // lines per round
     const int l = tid / upl, u = tid - l * upl, cg = u & 1, g = u >> 1;
@@ -231,139 +274,158 @@ __global__ void __launch_bounds__(VOL_THREADS) dct_volume_kernel(const __grid_co
 size_t vol_smem(const FFDims& dm) {
   size_t m = 0;
   const int n[3] = {dm.T, dm.H, dm.W};
-  for (int a = 0; a < 3; ++a) { const size_t x = (size_t)n[a] * ((n[a] + 7) & ~7); if (x > m) m = x; }
+  for (int a = 0; a < 3; ++a) m += (size_t)n[a] * ((n[a] + 7) & ~7);
   return (size_t)dm.N * VOL_CH * sizeof(float) + m * sizeof(float);
 }
 bool vol_fits(const FFDims& dm) { return dm.N <= VOL_MAX; }
 
 // ------------------------------------------------------------------------------------------------
 // Band operators ("Hierarchical frequency-domain attention") in fp32: a block takes 64 query rows of one (head, band)
-// and walks key tiles of 64 with an online softmax; Q and K tiles lie transposed in shared memory, P takes the place of
-// K between the two products.  A thread holds 4 x 4 scores (two 16-byte reads per 16 FMA) and 4 rows x d / 16 output
-// channels.  The key set of a row is generated from its rank: all pooled tokens (low), the blocks at block distance
-// 0 mod s (mid; query tiles then run along a residue class, so its keys are one dense range of class positions), own and
-// anchor blocks (mid, anchor pattern), the window |p - p'| <= R (high).
-// Bound by the FMA pipe and shared-memory reads; one warp per row with a five-shuffle reduction per score, as before,
-// took 1460 us where this takes about a tenth (9 x 30 x 40 tokens, 4 heads of 64 channels, all bands).
+// and walks key tiles with an online softmax.  The key set of a row is generated from its rank: all pooled tokens
+// (low), the blocks at block distance 0 mod s (mid; query tiles then run along a residue class, so its keys are one
+// dense range of class positions), own and anchor blocks (mid, anchor pattern), the window |p - p'| <= R (high).
+//
+// Bound by the FMA pipe (5.3 GFLOP of tiles at 9 x 30 x 40 tokens, 4 heads of 64 channels, all bands: 78 us at full
+// rate).  A thread holds 8 rows x KT / 16 keys of scores, so that a step of four channels is 12 16-byte shared reads for
+// 128 FMA (4 x 4 scores per thread were bound by those reads: 233 us), then 8 rows x d / 16 output channels.  Rows lie
+// as they are in memory, padded by 16 bytes against bank conflicts, so copies are asynchronous: the next keys arrive
+// during the softmax and P V, the values during Q K.  P is only read by the half warp that wrote it.  64 keys a tile up
+// to head_dim 64, 32 above (three blocks, two blocks per SM).  Measured there: 196 us, 70% of the issue slots; packed
+// pairs of FMA gained nothing (204 us).
 // ------------------------------------------------------------------------------------------------
-constexpr int AT = 64, AT_THREADS = 256, AT_PITCH = AT + 4;
+constexpr int AT = 64, AT_THREADS = 128, AT_PITCH = AT + 4;
 
-template <int DPL> constexpr size_t at_smem() {
-  return (size_t)(DPL * 32 * AT_PITCH + (DPL >= 2 ? DPL * 32 : AT) * AT_PITCH + AT * (DPL * 32 + 4)) * sizeof(float);
-}
+template <int DPL> struct AtShape {
+  static constexpr int d = DPL * 32, KT = DPL <= 2 ? 64 : 32, KJ = KT / 16, PITCH = d + 4;
+  static constexpr size_t smem = (size_t)(AT * PITCH + 2 * KT * PITCH + KT * AT_PITCH) * sizeof(float);
+};
 
-template <typename KT, int DPL>
-__device__ __forceinline__ void attend_tile(const KT* Qp, const KT* Kp, const KT* Vp, KT* Yp, const FFDims& dm, int band, long long n,
-                                            int tile, float* sm) {
-  constexpr int d = DPL * 32;
-  float* Qt = sm;                                        // [d][AT_PITCH]
-  float* Kt = Qt + d * AT_PITCH;                         // [d][AT_PITCH], then P [key][AT_PITCH]
-  float* Vs = Kt + (d > AT ? d : AT) * AT_PITCH;         // [AT][d + 4]
+template <typename KT_, int DPL>
+__device__ __forceinline__ void attend_tile(const KT_* Qp, const KT_* Kp, const KT_* Vp, KT_* Yp, const FFDims& dm, int band, int n, int tile,
+                                            float* sm) {
+  using S = AtShape<DPL>;
+  constexpr int d = S::d, KT = S::KT, KJ = S::KJ, PITCH = S::PITCH, VEC = d / 4;
+  float* Qs = sm;                                        // [AT][PITCH]
+  float* Ks = Qs + AT * PITCH;                           // [KT][PITCH]
+  float* Vs = Ks + KT * PITCH;                           // [KT][PITCH]
+  float* Ps = Vs + KT * PITCH;                           // [KT][AT_PITCH]: P transposed
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
   const float scale = rsqrtf((float)d);
+  const int blk_rows = min(dm.b, n), R = min(dm.R, n);   // (so that sums of positions stay in 32 bits)
   const bool strided = band == 1 && dm.pattern == FF_MID_STRIDED;
   const bool anchor = band == 1 && !strided;
   // class-local (strided mid band) or band positions of the tile, and the range of key positions
-  int cls = 0;
-  long long q0 = (long long)tile * AT, len = n, ks = 0, ke = n;
+  int cls = 0, q0 = tile * AT, len = n, ks = 0, ke = n;
   if (strided) {
     const int per = (int)(dm.nb / dm.s), rem = (int)(dm.nb % dm.s);                   // blocks of a class: per or per + 1
-    const int t_big = (int)(((long long)(per + 1) * dm.b + AT - 1) / AT), t_small = (int)(((long long)per * dm.b + AT - 1) / AT);
+    const int t_big = ((per + 1) * blk_rows + AT - 1) / AT, t_small = (per * blk_rows + AT - 1) / AT;
     int t;
-    if (tile < rem * t_big) { cls = tile / t_big; t = tile % t_big; len = (long long)(per + 1) * dm.b; }
+    if (tile < rem * t_big) { cls = tile / t_big; t = tile % t_big; len = (per + 1) * blk_rows; }
     else {
       const int rest = tile - rem * t_big;
       if (t_small == 0 || rest >= (dm.s - rem) * t_small) return;
-      cls = rem + rest / t_small; t = rest % t_small; len = (long long)per * dm.b;
+      cls = rem + rest / t_small; t = rest % t_small; len = per * blk_rows;
     }
-    q0 = (long long)t * AT; ke = len;
+    q0 = t * AT; ke = len;
   } else {
     if (q0 >= n) return;
     if (band == 2) {
-      ks = q0 - dm.R > 0 ? q0 - dm.R : 0;
-      ke = q0 + AT + dm.R < n ? q0 + AT + dm.R : n;
+      ks = q0 > R ? q0 - R : 0;
+      ke = n - q0 - AT < R ? n : q0 + AT + R;
     }
   }
-  auto rank_of = [&](long long u) -> long long {         // band rank of a position
+  auto rank_of = [&](int u) -> int {                     // band rank of a position
     if (!strided) return u;
-    const unsigned blk = (unsigned)u / (unsigned)dm.b;
-    return (long long)(((unsigned)cls + blk * (unsigned)dm.s) * (unsigned)dm.b + ((unsigned)u - blk * (unsigned)dm.b));
+    const unsigned blk = (unsigned)u / (unsigned)blk_rows;
+    return (int)(((unsigned)cls + blk * (unsigned)dm.s) * (unsigned)blk_rows + ((unsigned)u - blk * (unsigned)blk_rows));
   };
-  // A thread loads row `lrow` of every tile, a quarter of its channels (lanes along the rows, so that the transposed
-  // stores meet no bank twice).
-  const int lrow = tid % AT, lv = tid / AT;
-  auto put_t = [&](float* dst, int v, const float4& x) {
-    dst[(v * 4) * AT_PITCH + lrow] = x.x; dst[(v * 4 + 1) * AT_PITCH + lrow] = x.y;
-    dst[(v * 4 + 2) * AT_PITCH + lrow] = x.z; dst[(v * 4 + 3) * AT_PITCH + lrow] = x.w;
+  // rows u0 .. u0 + ROWS of the positions below `end`, zeros past them
+  auto load = [&](float* dst, const KT_* src, int rows, int u0, int end) {
+#pragma unroll 4
+    for (int i = tid; i < rows * VEC; i += AT_THREADS) {
+      const int r = i / VEC, v = i - r * VEC, rk = u0 + r < end ? rank_of(u0 + r) : n;
+      const bool on = rk < n;
+      const KT_* from = src + (size_t)(on ? rk : 0) * d + v * 4;
+      float* to = dst + r * PITCH + v * 4;
+      if (sizeof(KT_) == 4) cp_async16(to, (const float*)from, on);
+      else *(float4*)to = on ? ld4(from) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    cp_async_commit();
   };
-  {
-    const long long rk = q0 + lrow < len ? rank_of(q0 + lrow) : n;
-    const KT* src = Qp + (size_t)(rk < n ? rk : 0) * d;
-#pragma unroll 2
-    for (int v = lv; v < d / 4; v += AT_THREADS / AT) put_t(Qt, v, rk < n ? ld4(src + v * 4) : make_float4(0.f, 0.f, 0.f, 0.f));
-  }
-  long long pq[4];
+  // (anchor) anchor blocks are s blocks apart: skip key tiles without one and without any of the rows' own blocks
+  auto next_tile = [&](int k0) {
+    for (; anchor && k0 < ke; k0 += KT) {
+      const int b0 = k0 / blk_rows, b1 = (min(k0 + KT, n) - 1) / blk_rows;
+      const bool any = (b1 + 1) / dm.s > b0 / dm.s;      // some block J in [b0, b1] has J = s - 1 mod s
+      if (any || !(b1 < q0 / blk_rows || b0 > (min(q0 + AT, n) - 1) / blk_rows)) break;
+    }
+    return k0;
+  };
+  int k0 = next_tile(ks);
+  load(Qs, Qp, AT, q0, len);
+  load(Ks, Kp, KT, k0, ke);
+  int pq[8];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) pq[i] = q0 + ty * 4 + i < len ? rank_of(q0 + ty * 4 + i) : n;
-  float mx[4], den[4], o[4][DPL][2];
+  for (int i = 0; i < 8; ++i) pq[i] = q0 + ty * 8 + i < len ? rank_of(q0 + ty * 8 + i) : n;
+  float mx[8], den[8], o[8][DPL][2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < 8; ++i) {
     mx[i] = -INFINITY; den[i] = 0.f;
 #pragma unroll
     for (int j = 0; j < DPL; ++j) o[i][j][0] = o[i][j][1] = 0.f;
   }
-  for (long long k0 = ks; k0 < ke; k0 += AT) {
-    if (anchor) {
-      // anchor blocks are s blocks apart: skip a key tile without one and without any of the rows' own blocks
-      const long long b0 = k0 / dm.b, b1 = ((k0 + AT < n ? k0 + AT : n) - 1) / dm.b;
-      const long long own0 = q0 / dm.b, own1 = ((q0 + AT < n ? q0 + AT : n) - 1) / dm.b;
-      const bool any = (b1 + 1) / dm.s > b0 / dm.s;      // some block J in [b0, b1] has J = s - 1 mod s
-      if (!any && (b1 < own0 || b0 > own1)) continue;
-    }
-    __syncthreads();                                     // the previous tile's P and V have been read
-    {
-      const long long rk = k0 + lrow < ke ? rank_of(k0 + lrow) : n;
-      const size_t at = (size_t)(rk < n ? rk : 0) * d;
-#pragma unroll 2
-      for (int v = lv; v < d / 4; v += AT_THREADS / AT) {
-        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-        const float4 kx = rk < n ? ld4(Kp + at + v * 4) : zero, vx = rk < n ? ld4(Vp + at + v * 4) : zero;
-        put_t(Kt, v, kx);
-        *(float4*)(Vs + lrow * (d + 4) + v * 4) = vx;
-      }
-    }
+  while (k0 < ke) {
+    load(Vs, Vp, KT, k0, ke);                            // (P V of the previous tile has been read: barrier below)
+    cp_async_wait<1>();
     __syncthreads();
-    float s[4][4];
+    float s[8][KJ];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-#pragma unroll 4
-    for (int c = 0; c < d; ++c) {
-      const float4 q = *(const float4*)(Qt + c * AT_PITCH + ty * 4), k = *(const float4*)(Kt + c * AT_PITCH + tx * 4);
-      const float qq[4] = {q.x, q.y, q.z, q.w}, kk[4] = {k.x, k.y, k.z, k.w};
+      for (int j = 0; j < KJ; ++j) s[i][j] = 0.f;
+#pragma unroll 2
+    for (int c = 0; c < d; c += 4) {
+      float4 k[KJ];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int j = 0; j < KJ; ++j) k[j] = *(const float4*)(Ks + (tx + 16 * j) * PITCH + c);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) s[i][j] = fmaf(qq[i], kk[j], s[i][j]);
-    }
-    // which of the thread's 4 x 4 pairs exist
+      for (int i = 0; i < 8; ++i) {
+        const float4 q = *(const float4*)(Qs + (ty * 8 + i) * PITCH + c);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const long long u = k0 + tx * 4 + j, rk = u < ke ? rank_of(u) : n;
-      const bool in = rk < n;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        bool ok = in;
-        if (band == 2) ok = in && rk - pq[i] <= dm.R && pq[i] - rk <= dm.R;
-        else if (anchor) { const long long J = rk / dm.b; ok = in && (J == pq[i] / dm.b || J % dm.s == dm.s - 1); }
-        s[i][j] = ok ? s[i][j] * scale : -INFINITY;
+        for (int j = 0; j < KJ; ++j)
+          s[i][j] = fmaf(q.x, k[j].x, fmaf(q.y, k[j].y, fmaf(q.z, k[j].z, fmaf(q.w, k[j].w, s[i][j]))));
       }
     }
-    __syncthreads();                                     // K has been read: P takes its place
+    __syncthreads();                                     // K has been read
+    const int k1 = next_tile(k0 + KT);
+    if (k1 < ke) load(Ks, Kp, KT, k1, ke);
+    // which pairs exist: all of them, except in edge tiles
+    bool full = k0 + KT <= ke && !anchor;
+    if (band == 2) full = full && k0 >= q0 + AT - 1 - R && k0 + KT - 1 <= q0 + R;
+    else if (strided) full = full && rank_of(k0 + KT - 1) < n;
+    if (full) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float nm = fmaxf(fmaxf(s[i][0], s[i][1]), fmaxf(s[i][2], s[i][3]));
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int j = 0; j < KJ; ++j) s[i][j] *= scale;
+    } else {
+#pragma unroll
+      for (int j = 0; j < KJ; ++j) {
+        const int u = k0 + tx + 16 * j, rk = u < ke ? rank_of(u) : n;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          bool ok = rk < n;
+          if (band == 2) ok = ok && rk - pq[i] <= R && pq[i] - rk <= R;
+          else if (anchor) { const int J = rk / blk_rows; ok = ok && (J == pq[i] / blk_rows || J % dm.s == dm.s - 1); }
+          s[i][j] = ok ? s[i][j] * scale : -INFINITY;
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float nm = s[i][0];
+#pragma unroll
+      for (int j = 1; j < KJ; ++j) nm = fmaxf(nm, s[i][j]);
 #pragma unroll
       for (int w = 8; w > 0; w >>= 1) nm = fmaxf(nm, __shfl_xor_sync(0xffffffffu, nm, w));
       nm = fmaxf(nm, mx[i]);
@@ -371,47 +433,53 @@ __device__ __forceinline__ void attend_tile(const KT* Qp, const KT* Kp, const KT
       const float corr = expf(mx[i] - ref);
       float sum = 0.f;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) { s[i][j] = expf(s[i][j] - ref); sum += s[i][j]; }
+      for (int j = 0; j < KJ; ++j) { s[i][j] = expf(s[i][j] - ref); sum += s[i][j]; }
       den[i] = den[i] * corr + sum;                      // (this thread's share of the row sum)
       mx[i] = nm;
 #pragma unroll
       for (int j = 0; j < DPL; ++j) { o[i][j][0] *= corr; o[i][j][1] *= corr; }
     }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) *(float4*)(Kt + (tx * 4 + j) * AT_PITCH + ty * 4) = make_float4(s[0][j], s[1][j], s[2][j], s[3][j]);
+    for (int j = 0; j < KJ; ++j) {
+      float* p = Ps + (tx + 16 * j) * AT_PITCH + ty * 8;
+      *(float4*)p = make_float4(s[0][j], s[1][j], s[2][j], s[3][j]);
+      *(float4*)(p + 4) = make_float4(s[4][j], s[5][j], s[6][j], s[7][j]);
+    }
+    if (k1 < ke) cp_async_wait<1>(); else cp_async_wait<0>();      // V has arrived (the next K may still be on its way)
     __syncthreads();
-    const int nk = ke - k0 < AT ? (int)(ke - k0) : AT;
 #pragma unroll 4
-    for (int k = 0; k < nk; ++k) {
-      const float4 p = *(const float4*)(Kt + k * AT_PITCH + ty * 4);
-      const float pp[4] = {p.x, p.y, p.z, p.w};
+    for (int k = 0; k < KT; ++k) {
+      const float4 p0 = *(const float4*)(Ps + k * AT_PITCH + ty * 8), p1 = *(const float4*)(Ps + k * AT_PITCH + ty * 8 + 4);
+      const float pp[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
 #pragma unroll
       for (int j = 0; j < DPL; ++j) {
-        const float2 v = *(const float2*)(Vs + k * (d + 4) + 32 * j + 2 * tx);
+        const float2 v = *(const float2*)(Vs + k * PITCH + 32 * j + 2 * tx);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { o[i][j][0] = fmaf(pp[i], v.x, o[i][j][0]); o[i][j][1] = fmaf(pp[i], v.y, o[i][j][1]); }
+        for (int i = 0; i < 8; ++i) { o[i][j][0] = fmaf(pp[i], v.x, o[i][j][0]); o[i][j][1] = fmaf(pp[i], v.y, o[i][j][1]); }
       }
     }
+    __syncthreads();                                     // V has been read
+    k0 = k1;
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < 8; ++i) {
 #pragma unroll
     for (int w = 8; w > 0; w >>= 1) den[i] += __shfl_xor_sync(0xffffffffu, den[i], w);
     if (pq[i] >= n) continue;
-    KT* y = Yp + (size_t)pq[i] * d + 2 * tx;
+    KT_* y = Yp + (size_t)pq[i] * d + 2 * tx;
 #pragma unroll
-    for (int j = 0; j < DPL; ++j) { stf<KT>(y + 32 * j, o[i][j][0] / den[i]); stf<KT>(y + 32 * j + 1, o[i][j][1] / den[i]); }
+    for (int j = 0; j < DPL; ++j) { stf<KT_>(y + 32 * j, o[i][j][0] / den[i]); stf<KT_>(y + 32 * j + 1, o[i][j][1] / den[i]); }
   }
 }
 
 template <typename ST, int DPL>
-__global__ void __launch_bounds__(AT_THREADS, 2) attention_simt_kernel(FFBuffers buf, FFDims dm, int band_bits) {
+__global__ void __launch_bounds__(AT_THREADS, DPL <= 2 ? 3 : 2) attention_simt_kernel(FFBuffers buf, FFDims dm, int band_bits) {
   extern __shared__ float sm[];
   ff_pdl_wait();
   const int band = blockIdx.z == 0 ? 1 : (blockIdx.z == 1 ? 2 : 0);      // the mid band's items are the long ones
   const int bh = blockIdx.y;
   if (!(buf.alloc[bh] & band_bits & (1 << band))) return;
-  const long long n = band == 0 ? dm.Nbar : (band == 1 ? dm.Nmid : dm.Nhigh);
+  const int n = (int)(band == 0 ? dm.Nbar : (band == 1 ? dm.Nmid : dm.Nhigh));
   if (n == 0) return;
   const size_t one = (size_t)n * DPL * 32, tensor = (size_t)dm.BH * one;  // a head's, a tensor's extent in the band's buffer
   if (sizeof(ST) == 4) {                          // (one copy of the code: small launches are bound by fetching it)
@@ -424,6 +492,89 @@ __global__ void __launch_bounds__(AT_THREADS, 2) attention_simt_kernel(FFBuffers
   } else {
     const ST* Q = (const ST*)(band == 1 ? buf.spec_mid : buf.spec_high) + bh * one;
     attend_tile<ST, DPL>(Q, Q + tensor, Q + 2 * tensor, (ST*)(band == 1 ? buf.y_mid : buf.y_high) + bh * one, dm, band, n, blockIdx.x, sm);
+  }
+}
+
+// Small launches (up to ROW_PAIRS scored pairs): one warp per query row, eight keys side by side, merged into the running
+// softmax as a group.  Little code and as many warps as rows; the tiled kernel above spends most of its 17 us there on
+// fetching its instructions (256 tokens, 2 heads of 32 channels).
+constexpr int ROW_WARPS = 4;
+constexpr long long ROW_PAIRS = 1 << 18;
+
+template <typename KT_, int DPL>
+__device__ __forceinline__ void attend_row(const KT_* Qp, const KT_* Kp, const KT_* Vp, KT_* Yp, const FFDims& dm, int band, int n, int p) {
+  const int lane = threadIdx.x & 31, d = DPL * 32;
+  const int b = min(dm.b, n), R = min(dm.R, n);
+  const bool strided = band == 1;
+  // keys: positions of the row's residue class, or a range of ranks
+  int cls = 0, k_lo = 0, k_hi = n;
+  if (strided) { cls = (int)((p / b) % dm.s); k_hi = (int)((dm.nb - cls + dm.s - 1) / dm.s) * b; }
+  else if (band == 2) { k_lo = max(p - R, 0); k_hi = min(p + R + 1, n); }
+  const float scale = rsqrtf((float)d);
+  float q[DPL], o[DPL], mx = -INFINITY, den = 0.f;
+#pragma unroll
+  for (int j = 0; j < DPL; ++j) { q[j] = ldf<KT_>(Qp + (size_t)p * d + lane + 32 * j); o[j] = 0.f; }
+#pragma unroll 1
+  for (int k0 = k_lo; k0 < k_hi; k0 += 8) {
+    float sc[8], v[8][DPL];
+    bool on[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int u = k0 + k;
+      int rk = u;
+      if (strided) { const unsigned blk = (unsigned)u / (unsigned)b; rk = (int)(((unsigned)cls + blk * (unsigned)dm.s) * (unsigned)b + ((unsigned)u - blk * (unsigned)b)); }
+      on[k] = u < k_hi && rk < n;
+      const size_t at = (size_t)(on[k] ? rk : p) * d + lane;
+      float part = 0.f;
+#pragma unroll
+      for (int j = 0; j < DPL; ++j) { part = fmaf(q[j], ldf<KT_>(Kp + at + 32 * j), part); v[k][j] = ldf<KT_>(Vp + at + 32 * j); }
+      sc[k] = part;
+    }
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1)
+#pragma unroll
+      for (int k = 0; k < 8; ++k) sc[k] += __shfl_xor_sync(0xffffffffu, sc[k], w);
+    float nm = mx;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) { sc[k] = on[k] ? sc[k] * scale : -INFINITY; nm = fmaxf(nm, sc[k]); }
+    const float ref = nm == -INFINITY ? 0.f : nm;        // (no key of the row so far)
+    const float corr = expf(mx - ref);
+    // (every lane has all eight scores: lane k takes the exponential of key k)
+    float mine = sc[0];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) mine = (lane & 7) == k ? sc[k] : mine;
+    mine = expf(mine - ref);
+    den *= corr;
+#pragma unroll
+    for (int j = 0; j < DPL; ++j) o[j] *= corr;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float pr = __shfl_sync(0xffffffffu, mine, k);
+      den += pr;
+#pragma unroll
+      for (int j = 0; j < DPL; ++j) o[j] = fmaf(pr, v[k][j], o[j]);
+    }
+    mx = nm;
+  }
+#pragma unroll
+  for (int j = 0; j < DPL; ++j) stf<KT_>(Yp + (size_t)p * d + lane + 32 * j, o[j] / den);
+}
+
+template <typename ST, int DPL>
+__global__ void __launch_bounds__(ROW_WARPS * 32) attention_row_kernel(FFBuffers buf, FFDims dm, int band_bits) {
+  ff_pdl_wait();
+  const int band = blockIdx.z == 0 ? 1 : (blockIdx.z == 1 ? 2 : 0), bh = blockIdx.y;
+  if (!(buf.alloc[bh] & band_bits & (1 << band))) return;
+  const int n = (int)(band == 0 ? dm.Nbar : (band == 1 ? dm.Nmid : dm.Nhigh)), p = blockIdx.x * ROW_WARPS + (threadIdx.x >> 5);
+  if (p >= n) return;
+  const size_t one = (size_t)n * DPL * 32, tensor = (size_t)dm.BH * one;
+  if (sizeof(ST) == 4 || band == 0) {
+    const float* Q = (band == 0 ? buf.pooled : (const float*)(band == 1 ? buf.spec_mid : buf.spec_high)) + bh * one;
+    float* Y = (band == 0 ? buf.y_low : (float*)(band == 1 ? buf.y_mid : buf.y_high)) + bh * one;
+    attend_row<float, DPL>(Q, Q + tensor, Q + 2 * tensor, Y, dm, band, n, p);
+  } else {
+    const ST* Q = (const ST*)(band == 1 ? buf.spec_mid : buf.spec_high) + bh * one;
+    attend_row<ST, DPL>(Q, Q + tensor, Q + 2 * tensor, (ST*)(band == 1 ? buf.y_mid : buf.y_high) + bh * one, dm, band, n, p);
   }
 }
 
@@ -609,18 +760,35 @@ static cudaError_t attention_simt_t(ff_plan* p, int band_bits, cudaStream_t st) 
   if ((band_bits & FF_BAND_LOW) && tiles(dm.Nbar) > most) most = tiles(dm.Nbar);
   if (band_bits & FF_BAND_MID) {
     const long long per = dm.nb / dm.s, rem = dm.nb % dm.s;
-    const long long t = dm.pattern == FF_MID_STRIDED ? rem * tiles((per + 1) * dm.b) + (dm.s - rem) * tiles(per * dm.b) : tiles(dm.Nmid);
+    const long long b = dm.b < dm.Nmid ? dm.b : dm.Nmid;
+    const long long t = dm.pattern == FF_MID_STRIDED ? rem * tiles((per + 1) * b) + (dm.s - rem) * tiles(per * b) : tiles(dm.Nmid);
     if (dm.Nmid > 0 && t > most) most = t;
   }
   if ((band_bits & FF_BAND_HIGH) && tiles(dm.Nhigh) > most) most = tiles(dm.Nhigh);
   if (most == 0) return cudaSuccess;                 // (only an empty band was asked for)
-  const dim3 grid((unsigned)most, (unsigned)dm.BH, (band_bits & FF_BAND_LOW) ? 3 : ((band_bits & FF_BAND_HIGH) ? 2 : 1));
+  const unsigned bands = (band_bits & FF_BAND_LOW) ? 3 : ((band_bits & FF_BAND_HIGH) ? 2 : 1);
   p->launches += 1;
+  // scored pairs, if every head ran every band asked for
+  long long rows = 0, pairs = 0;
+  auto add = [&](long long n, long long keys) { rows = n > rows ? n : rows; pairs += dm.BH * n * (keys < n ? keys : n); };
+  if (band_bits & FF_BAND_LOW) add(dm.Nbar, dm.Nbar);
+  if (band_bits & FF_BAND_MID) add(dm.Nmid, (dm.nb + dm.s - 1) / dm.s * dm.b);
+  if (band_bits & FF_BAND_HIGH) add(dm.Nhigh, 2LL * dm.R + 1);
+  if (pairs <= ROW_PAIRS && !((band_bits & FF_BAND_MID) && dm.pattern == FF_MID_ANCHOR)) {
+    const dim3 grid((unsigned)((rows + ROW_WARPS - 1) / ROW_WARPS), (unsigned)dm.BH, bands);
+    switch (dm.d / 32) {
+      case 1: return ff_launch(attention_row_kernel<ST, 1>, grid, dim3(ROW_WARPS * 32), 0, st, p->buf, dm, band_bits);
+      case 2: return ff_launch(attention_row_kernel<ST, 2>, grid, dim3(ROW_WARPS * 32), 0, st, p->buf, dm, band_bits);
+      case 3: return ff_launch(attention_row_kernel<ST, 3>, grid, dim3(ROW_WARPS * 32), 0, st, p->buf, dm, band_bits);
+      default: return ff_launch(attention_row_kernel<ST, 4>, grid, dim3(ROW_WARPS * 32), 0, st, p->buf, dm, band_bits);
+    }
+  }
+  const dim3 grid((unsigned)most, (unsigned)dm.BH, bands);
   switch (dm.d / 32) {
-    case 1: return ff_launch(attention_simt_kernel<ST, 1>, grid, dim3(AT_THREADS), at_smem<1>(), st, p->buf, dm, band_bits);
-    case 2: return ff_launch(attention_simt_kernel<ST, 2>, grid, dim3(AT_THREADS), at_smem<2>(), st, p->buf, dm, band_bits);
-    case 3: return ff_launch(attention_simt_kernel<ST, 3>, grid, dim3(AT_THREADS), at_smem<3>(), st, p->buf, dm, band_bits);
-    default: return ff_launch(attention_simt_kernel<ST, 4>, grid, dim3(AT_THREADS), at_smem<4>(), st, p->buf, dm, band_bits);
+    case 1: return ff_launch(attention_simt_kernel<ST, 1>, grid, dim3(AT_THREADS), AtShape<1>::smem, st, p->buf, dm, band_bits);
+    case 2: return ff_launch(attention_simt_kernel<ST, 2>, grid, dim3(AT_THREADS), AtShape<2>::smem, st, p->buf, dm, band_bits);
+    case 3: return ff_launch(attention_simt_kernel<ST, 3>, grid, dim3(AT_THREADS), AtShape<3>::smem, st, p->buf, dm, band_bits);
+    default: return ff_launch(attention_simt_kernel<ST, 4>, grid, dim3(AT_THREADS), AtShape<4>::smem, st, p->buf, dm, band_bits);
   }
 }
 

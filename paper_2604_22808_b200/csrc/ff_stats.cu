@@ -45,36 +45,40 @@ __device__ __forceinline__ void add_squares(float4& e, const float4& x) {
   e.x = fmaf(x.x, x.x, e.x); e.y = fmaf(x.y, x.y, e.y); e.z = fmaf(x.z, x.z, e.z); e.w = fmaf(x.w, x.w, e.w);
 }
 
-// z = W2 relu(W1 [g; e(t)] + b1) + b2, pi = softmax(z), largest-remainder quota, one-hot masks; a whole block.
+// Sinusoidal embedding of the sample's timestep into et[dt]: double-precision sines that depend on no other kernel.
+__device__ void embed_timestep(const StatsParams& P, int sample, float* et) {
+  const int half = P.dm.dt / 2;
+  for (int k = threadIdx.x; k < half; k += ST_THREADS) {
+    const double t = (double)(P.timestep ? P.timestep[sample] : P.ts[sample]);
+    const double om = exp2(-(double)k / (double)half * 13.287712379549449);     // 10000^(-k/half); log2(10000)
+    double sn, cs;
+    sincos(t * om, &sn, &cs);
+    et[k] = (float)sn;
+    et[half + k] = (float)cs;
+  }
+}
+
+// z = W2 relu(W1 [g; e(t)] + b1) + b2, pi = softmax(z), largest-remainder quota, one-hot masks; a whole block.  e(t) is
+// in place already.
 __device__ void route_sample(const StatsParams& P, int sample, float* sm) {
   const FFDims& dm = P.dm;
-  const int d = dm.d, nin = 3 * d + dm.dt, hid = dm.hid, half = dm.dt / 2;
+  const int d = dm.d, nin = 3 * d + dm.dt, hid = dm.hid;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* x = sm;            // [nin]
   float* h = sm + nin;      // [hid]
   __shared__ float z[3];
   __shared__ int first[4];  // first head of each band
-  const double t = (double)(P.timestep ? P.timestep[sample] : P.ts[sample]);
-  for (int i = tid; i < 3 * d + half; i += ST_THREADS) {
-    if (i < 3 * d) {
-      const int band = i / d;
-      const long long cnt = band == 0 ? dm.Nlow : (band == 1 ? dm.Nmid : dm.Nhigh);
-      const double terms = 3.0 * dm.heads * (double)(cnt > 0 ? cnt : 1);          // an empty band (two-band layer) has g = 0
-      x[i] = (float)log1p(__ldcg(P.energy + (size_t)sample * 3 * d + i) / terms);
-    } else {
-      const int k = i - 3 * d;
-      const double om = exp2(-(double)k / (double)half * 13.287712379549449);     // 10000^(-k/half); log2(10000)
-      double sn, cs;
-      sincos(t * om, &sn, &cs);
-      x[3 * d + k] = (float)sn;
-      x[3 * d + half + k] = (float)cs;
-    }
+  for (int i = tid; i < 3 * d; i += ST_THREADS) {
+    const int band = i / d;
+    const long long cnt = band == 0 ? dm.Nlow : (band == 1 ? dm.Nmid : dm.Nhigh);
+    const double terms = 3.0 * dm.heads * (double)(cnt > 0 ? cnt : 1);          // an empty band (two-band layer) has g = 0
+    x[i] = (float)log1p(__ldcg(P.energy + (size_t)sample * 3 * d + i) / terms);
   }
   __syncthreads();
   // hidden layer: four units per warp at a time, lanes stride over the inputs (coalesced rows of W1)
   for (int j0 = warp * 4; j0 < hid; j0 += (ST_THREADS / 32) * 4) {
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
+#pragma unroll 8
     for (int i = lane; i < nin; i += 32) {
 #pragma unroll
       for (int k = 0; k < 4; ++k) acc[k] = fmaf(P.W1[(size_t)(j0 + k < hid ? j0 + k : j0) * nin + i], x[i], acc[k]);
@@ -124,8 +128,11 @@ template <typename ST>
 __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_constant__ StatsParams P) {
   extern __shared__ float sm[];
   __shared__ bool last;
-  ff_pdl_wait();
   const FFDims& dm = P.dm;
+  // (any block may turn out to be the one that routes; the sums below use other shared memory)
+  float* mlp = sm + (ST_THREADS / (dm.d / 4)) * dm.d;
+  if (!P.alloc_in && !P.timestep) embed_timestep(P, 0, mlp + 3 * dm.d);
+  ff_pdl_wait();
   const int d = dm.d, vecs = d / 4;                         // four channels per thread
   const int vec = threadIdx.x % vecs, sub = threadIdx.x / vecs, nsub = ST_THREADS / vecs;
   const int th = blockIdx.y;
@@ -190,7 +197,10 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
   if (!last) return;
   __threadfence();
   if (threadIdx.x == 0) *P.ticket = 0;
-  for (int sample = 0; sample < dm.B; ++sample) route_sample(P, sample, sm);
+  for (int sample = 0; sample < dm.B; ++sample) {
+    if (sample > 0 || P.timestep) embed_timestep(P, sample, mlp + 3 * d);
+    route_sample(P, sample, mlp);
+  }
   if (P.work && threadIdx.x < 32) build_worklist(dm, P.alloc, P.low_on, P.work);
 }
 
@@ -227,5 +237,5 @@ cudaError_t ffk_band_stats(ff_plan* p, const uint8_t* alloc_in, const float* tim
   const size_t red = (size_t)nsub * dm.d * sizeof(float), mlp = (size_t)(3 * dm.d + dm.dt + dm.hid) * sizeof(float);
   p->launches += 1;
   return ff_launch(dm.fp32 ? band_stats_kernel<float> : band_stats_kernel<__nv_bfloat16>, dim3((unsigned)blocks, (unsigned)(3 * dm.BH)),
-                   dim3(ST_THREADS), red > mlp ? red : mlp, st, P);
+                   dim3(ST_THREADS), red + mlp, st, P);
 }

@@ -16,6 +16,9 @@ CASES = [
     dict(grid=(1, 2, 128), d=96, dtype="fp32", b=7, s=40, R=1000, m=1),     # more classes than blocks
     dict(grid=(7, 9, 10), d=32, dtype="bf16", b=16, s=4, R=8, m=40),        # bf16 storage, 120 summaries
     dict(grid=(6, 20, 24), d=96, dtype="bf16", b=32, s=2, R=33, m=5),
+    dict(grid=(3, 10, 16), d=96, dtype="bf16", b=16, s=3, R=20, m=2),       # small enough for one warp per query row
+    dict(grid=(4, 8, 20), d=128, dtype="fp32", b=5, s=2, R=0, m=2),         # ... with a window of one key
+    dict(grid=(5, 16, 24), d=128, dtype="fp32", b=10 ** 9, s=1, R=2 ** 31 - 1, m=2),     # one block, a window of everything
     dict(grid=(6, 20, 24), d=64, dtype="fp32", b=24, s=3, R=16, m=6, mid_pattern="anchor"),
 ]
 
