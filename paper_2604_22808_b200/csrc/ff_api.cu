@@ -113,13 +113,15 @@ void ff_compute_layout(const FFDims& dm, bool with_staging, FFLayout* lay) {
   // Tensor-core transform: as many tensor-heads per launch as fit ~8 GiB of scratch (at least 3): every launch
   // pays a ramp-up and a tail, and fewer, longer launches measured faster (64K tokens, 72 tensor-heads: one group against
   // 32 + 32 + 8, 1.58 against 1.66 ms for the forward transform).  The host-buffer entry point
-  // works in groups of a quarter of that, so that the transform of one group overlaps the copy of the next.
+  // works in smaller groups, a sixth of the tensor-heads or 2 GiB of scratch, so that the transform of one group overlaps
+  // the copy of the next (six heads of 16K tokens in one group: 2190 us, of which 1850 are the copies).
   size_t Gt = ((size_t)8 << 30) / (4 * (size_t)dm.N * d * 2);
   if (Gt < 3) Gt = 3;
   if (Gt > 3 * BH) Gt = 3 * BH;
   lay->tc_group = (int)Gt;
   size_t Gp = ((size_t)2 << 30) / (4 * (size_t)dm.N * d * 2);
   if (Gp < 3) Gp = 3;
+  if (Gp > (3 * BH + 5) / 6) Gp = (3 * BH + 5) / 6;
   if (Gp > Gt) Gp = Gt;
   lay->tc_group_pipe = (int)Gp;
   const size_t tc_scratch = ffk_dct_tc_supported(dm) ? ffk_dct_tc_scratch_bytes(dm, (int)Gt) : 0;
