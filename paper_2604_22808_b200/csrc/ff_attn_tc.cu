@@ -14,10 +14,13 @@
 //   warp 1       tcgen05.mma issuer: S_x = Q_x K^T (operands from shared memory), O_x += P_x V
 //                (A = P from tensor memory, B = V as an MN-major operand), issue order
 //                PV_A[j], QK_A[j+1], PV_B[j], QK_B[j+1]; owns the tensor-memory allocation
-//   warps 2..17  softmax: per stream two threads per query row (row = TMEM lane, 64 key columns
-//                each); scores read with tcgen05.ld, key masks generated in registers from the row's
-//                band rank, P written back to tensor memory as bf16 over the thread's own scores; O
-//                accumulates in tensor memory and is rescaled only when a row maximum grows by > 2^8
+//   warps 4..11  softmax: per stream one thread per query row (row = TMEM lane); the row's 128 scores are read into
+//                registers once, key masks are generated from the row's band rank, P is written back to tensor memory
+//                as bf16 over the scores; O accumulates in tensor memory and is rescaled only when a row maximum grows
+//                by > 2^8.  The registers of the first warpgroup (120 are left of 168 a thread) go to these two
+//                (192): 128 x 120 + 256 x 192 = 384 x 168.  With two threads a row, a shared-memory hand-shake for the
+//                maximum and a second read of the scores the launch took 1.37 instead of 1.17 ms (64K tokens, 24 heads,
+//                all bands)
 // Tensor memory (512 columns): S/P of stream A, S/P of stream B, O of stream A, O of stream B.
 // Every wait is bounded; when one runs out the CTA raises FF_ERR_TIMEOUT in the plan's status
 // word, stops taking work, lets its copies drain, frees its tensor memory and returns.
@@ -36,9 +39,7 @@ constexpr int HD_MAX = 128;          // largest head_dim; the shared-memory slot
 constexpr int TILE_BYTES = TILE * HD_MAX * 2;
 constexpr int HALF_BYTES = TILE_BYTES / 2;
 constexpr int MAX_UNITS = FF_MAX_UNITS;
-constexpr int NSPLIT = 2;                // softmax threads per query row
-constexpr int SCOLS = TILE / NSPLIT;     // key columns per softmax thread
-constexpr int TC_THREADS = 64 + 2 * 128 * NSPLIT;   // TMA warp, MMA warp, 2 streams x 4 NSPLIT softmax warps
+constexpr int TC_THREADS = 128 + 2 * 128;            // warpgroups: TMA and MMA warp (and two idle ones), softmax of streams A and B
 constexpr float LAZY_LOG2 = 8.0f;    // rescale O only when the running max grows by more than this (log2 units)
 
 struct TcParams {
@@ -75,9 +76,6 @@ struct Shared {
   int offsets[MAX_UNITS + 1];
   int desc[MAX_UNITS];
   int ntile[MAX_UNITS];
-  // hand-shake slots of the threads of a row: (sequence number << 32) | float bits
-  unsigned long long xmax[2][2][NSPLIT][128];     // [parity][stream][part][row]
-  unsigned long long xsum[2][2][NSPLIT][128];
 };
 
 template <bool HAS_LOW>
@@ -163,33 +161,6 @@ __device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* map, 
   }
 }
 
-// The NSPLIT softmax threads of a row share one float each: a thread publishes (seq, value) in its
-// slot and reads the others' slots, waiting (bounded) until they carry the same sequence number.
-// `slots` points at [NSPLIT][128] entries; MAX selects max, otherwise sum.
-template <bool MAX>
-__device__ __forceinline__ bool row_exchange(unsigned long long* slots, int part, int row, unsigned seq, float& v,
-                                             volatile int* abort_flag) {
-  *(volatile unsigned long long*)(slots + part * 128 + row) = ((unsigned long long)seq << 32) | __float_as_uint(v);
-  float acc = v;
-#pragma unroll
-  for (int o = 1; o < NSPLIT; ++o) {
-    const volatile unsigned long long* theirs = slots + ((part + o) % NSPLIT) * 128 + row;
-    const long long t0 = clock64();
-    while (true) {
-      const unsigned long long w = *theirs;
-      if ((unsigned)(w >> 32) == seq) {
-        const float xv = __uint_as_float((unsigned)w);
-        acc = MAX ? fmaxf(acc, xv) : acc + xv;
-        break;
-      }
-      if (*abort_flag) return false;
-      if (clock64() - t0 > kWaitLimitCycles) { *abort_flag = 1; return false; }
-    }
-  }
-  v = acc;
-  return true;
-}
-
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -214,23 +185,18 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int HALVES = HD / 64;                  // 64-channel halves of a row
   constexpr int TB = TILE * HD * 2;                // bytes of one tile
-  constexpr int OCOLS = HD / NSPLIT;               // output columns per softmax thread
 
   if (threadIdx.x == 0) {
     mbar_init(&sh.q_full, 1); mbar_init(&sh.q_empty, 1);
     for (int i = 0; i < 2; ++i) {
       mbar_init(&sh.k_full[i], 1); mbar_init(&sh.k_empty[i], 1);
       mbar_init(&sh.v_full[i], 1); mbar_init(&sh.v_empty[i], 1);
-      mbar_init(&sh.s_full[i], 1); mbar_init(&sh.p_full[i], 128 * NSPLIT);
-      mbar_init(&sh.o_full[i], 1); mbar_init(&sh.o_empty[i], 128 * NSPLIT);
+      mbar_init(&sh.s_full[i], 1); mbar_init(&sh.p_full[i], 128);
+      mbar_init(&sh.o_full[i], 1); mbar_init(&sh.o_empty[i], 128);
     }
     sh.abort_flag = 0;
     sh.ms = mid_shape(dm);
     fence_mbar_init();
-  }
-  for (int i = threadIdx.x; i < 2 * 2 * NSPLIT * 128; i += TC_THREADS) {
-    (&sh.xmax[0][0][0][0])[i] = 0ull;
-    (&sh.xsum[0][0][0][0])[i] = 0ull;
   }
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
   ff_pdl_wait();
@@ -250,6 +216,8 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
   const int total = sh.total;
   volatile int* abort_flag = &sh.abort_flag;
 
+  if (warp < 4) {
+  reg_dec<120>();
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -292,15 +260,20 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
       unsigned cp[2] = {0, 0};          // P phases consumed per stream
       unsigned ce[2] = {0, 0};          // items seen per stream (for the O buffer hand-back)
       bool ok = true;
+      // Operand descriptors of the first slots, once: an instruction then takes an add each (a step inside a slot or a
+      // slot is a constant in the address field).  Assembled anew for every instruction they made the issuing
+      // thread the limit, 135 cycles an instruction where the tensor core takes 64.
+      const uint64_t q_desc = smem_desc_sw128(smem_u32(sQ), 16, 1024), k_desc = smem_desc_sw128(smem_u32(sK), 16, 1024);
+      const uint64_t v_desc = smem_desc_sw128(smem_u32(sV), HALF_BYTES, 1024);
       // S_x = Q_x K[tile]^T; `last` = no further QK uses this K stage
       auto issue_qk = [&](int sx, unsigned gt, bool last, bool release_q) {
         const int st = gt & 1;
-        const uint32_t qbase = smem_u32(sQ + sx * TILE_BYTES), kbase = smem_u32(sK + st * TILE_BYTES);
+        const uint64_t qd = q_desc + (uint64_t)(sx * (TILE_BYTES >> 4)), kd = k_desc + (uint64_t)(st * (TILE_BYTES >> 4));
+        const uint32_t d_tm = tm + sx * 128;
 #pragma unroll
         for (int k = 0; k < HD / 16; ++k) {
-          const uint32_t off = (k >> 2) * HALF_BYTES + (k & 3) * 32;
-          umma_ss(tm + sx * 128, smem_desc_sw128(qbase + off, 16, 1024), smem_desc_sw128(kbase + off, 16, 1024),
-                  idesc_qk, k > 0 ? 1u : 0u);
+          const uint64_t off = (uint64_t)(((k >> 2) * HALF_BYTES + (k & 3) * 32) >> 4);
+          umma_ss(d_tm, qd + off, kd + off, idesc_qk, k > 0 ? 1u : 0u);
         }
         umma_commit(&sh.s_full[sx]);
         if (last) umma_commit(&sh.k_empty[st]);
@@ -313,13 +286,12 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         ++cp[sx];
         if (first_of_item && ce[sx] >= 1 && !mbar_wait(&sh.o_empty[sx], (ce[sx] - 1) & 1, abort_flag)) return false;
         tc_fence_after();
-        const uint32_t vbase = smem_u32(sV + st * TILE_BYTES);
+        const uint64_t vd = v_desc + (uint64_t)(st * (TILE_BYTES >> 4));
+        const uint32_t p_tm = tm + sx * 128, d_tm = p_tm + 256, first = first_of_item ? 0u : 1u;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          // P of keys 16k..16k+15 sits at the start of the score columns of the thread that owns them
-          const uint32_t pcol = ((16 * k) / SCOLS) * SCOLS + ((16 * k) % SCOLS) / 2;
-          umma_ts(tm + 256 + sx * 128, tm + sx * 128 + pcol, smem_desc_sw128(vbase + k * 2048, HALF_BYTES, 1024),
-                  idesc_pv, (first_of_item && k == 0) ? 0u : 1u);
+          umma_ts(d_tm, p_tm + k * 8,                      // (P of keys 16 k .. 16 k + 15: eight columns)
+                  vd + (uint64_t)(k * (2048 >> 4)), idesc_pv, k == 0 ? first : 1u);
         }
         umma_commit(&sh.o_full[sx]);
         if (last) umma_commit(&sh.v_empty[st]);
@@ -367,25 +339,20 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         if (x.has_b) ce[1] += 1;
       }
     }
+  }
   } else {
+    reg_inc<192>();
     // ------------------------------------------------------------------ softmax
-    // Warps 2..9 serve stream A, 10..17 stream B.  Inside a stream the first four warps take key
-    // columns 0..63 of their 32 rows, the next four columns 64..127 (a warp reaches the TMEM lanes
-    // 32*(warp%4)..+31).  The threads of a row agree on the row maximum through a bounded
-    // hand-shake in shared memory; each keeps the partial row sum of its own columns.
+    // Warps 4..7 serve stream A, 8..11 stream B (a warp reaches the TMEM lanes 32*(warp%4)..+31).
     const int quarter = warp & 3;
-    const int sx = (warp - 2) / (4 * NSPLIT);
-    const int part = ((warp - 2) >> 2) % NSPLIT;
+    const int sx = (warp - 4) >> 2;
     const int row = quarter * 32 + lane;
-    const int col0 = part * SCOLS;                      // first key column of this thread
-    const int ocol0 = part * OCOLS;                     // first output column of this thread
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const uint32_t s_addr = tm + lane_addr + sx * 128;
-    const uint32_t o_addr = tm + lane_addr + 256 + sx * 128 + ocol0;     // this thread's output columns
+    const uint32_t o_addr = tm + lane_addr + 256 + sx * 128;
     const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
     unsigned cs = 0;                  // key tiles this stream has processed (phases of s_full / p_full)
     unsigned co = 0;                  // phases of o_full consumed
-    unsigned ci = 0;                  // items this stream has processed
     bool ok = true;
     for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
       const Item x = decode_item<HAS_LOW>(sh, dm, it);
@@ -425,47 +392,35 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
             chi = hi < TILE - 1 ? (int)(hi < -1 ? -1 : hi) : TILE - 1;
           }
         }
-        // (edge tiles) the valid columns of this thread's 32-column chunks as bit masks
-        uint32_t vmask[SCOLS / 32];
-#pragma unroll
-        for (int c = 0; c < SCOLS / 32; ++c) {
-          const int a = clo - (col0 + c * 32), b = chi - (col0 + c * 32);      // valid bits [a, b] of the chunk
-          const uint32_t lo_m = a <= 0 ? 0xffffffffu : (a >= 32 ? 0u : 0xffffffffu << a);
-          const uint32_t hi_m = b >= 31 ? 0xffffffffu : (b < 0 ? 0u : 0xffffffffu >> (31 - b));
-          vmask[c] = lo_m & hi_m;
-        }
         ok = __all_sync(0xffffffffu, mbar_wait(&sh.s_full[sx], cs & 1, abort_flag));
         if (!ok) break;
         tc_fence_after();
-        // first sweep over this thread's raw scores: the row maximum of its columns
-        float tmax = -INFINITY;
-        {
-          // (both 32-column chunks are requested before the first is used: one tensor-memory latency instead of two)
-          static_assert(SCOLS == 64, "the first sweep reads two chunks");
-          uint32_t r0[32], r1[32];
-          tmem_ld32(s_addr + col0, r0);
-          tmem_ld32(s_addr + col0 + 32, r1);
-          tmem_wait_ld();
-          if (full) {
-            float t1 = -INFINITY;                          // two chains
+        // the row's scores, and their maximum in four chains
+        uint32_t r[4][32];
 #pragma unroll
-            for (int i = 0; i < 32; i += 2) {
-              tmax = max3f(tmax, __uint_as_float(r0[i]), __uint_as_float(r0[i + 1]));
-              t1 = max3f(t1, __uint_as_float(r1[i]), __uint_as_float(r1[i + 1]));
-            }
-            tmax = fmaxf(tmax, t1);
-          } else {
+        for (int c = 0; c < 4; ++c) tmem_ld32(s_addr + c * 32, r[c]);
+        tmem_wait_ld();
+        if (!full) {
+          // (edge tiles) columns outside [clo, chi] count as -inf
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              if (vmask[0] & (1u << i)) tmax = fmaxf(tmax, __uint_as_float(r0[i]));
-              if (vmask[1] & (1u << i)) tmax = fmaxf(tmax, __uint_as_float(r1[i]));
-            }
+          for (int c = 0; c < 4; ++c) {
+            const int a = clo - c * 32, b = chi - c * 32;                        // valid bits [a, b] of the chunk
+            const uint32_t lo_m = a <= 0 ? 0xffffffffu : (a >= 32 ? 0u : 0xffffffffu << a);
+            const uint32_t hi_m = b >= 31 ? 0xffffffffu : (b < 0 ? 0u : 0xffffffffu >> (31 - b));
+            const uint32_t valid = lo_m & hi_m;
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if (!(valid & (1u << i))) r[c][i] = 0xff800000u;
           }
         }
-        // row maximum over the row's threads (slots alternate with the tile parity, so a partner's
-        // read of this tile cannot meet this thread's write of the next)
-        ok = __all_sync(0xffffffffu, row_exchange<true>(&sh.xmax[cs & 1][sx][0][0], part, row, cs + 1, tmax, abort_flag));
-        if (!ok) break;
+        float t4[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) t4[c] = fmaxf(__uint_as_float(r[c][0]), __uint_as_float(r[c][1]));
+#pragma unroll
+        for (int i = 2; i < 32; i += 2)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) t4[c] = max3f(t4[c], __uint_as_float(r[c][i]), __uint_as_float(r[c][i + 1]));
+        const float tmax = fmaxf(max3f(t4[0], t4[1], t4[2]), t4[3]);
         const float m_new = fmaxf(m_ref, tmax);
         const bool need = (m_new - m_ref) * sl2 > LAZY_LOG2;
         const float alpha = need ? ex2((m_ref - m_new) * sl2) : 1.f;
@@ -473,7 +428,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         // just before P is published, when it has long completed; only a row maximum that grew past
         // the lazy threshold needs it now, because O is then rescaled in place.  Every phase of the
         // barrier is awaited exactly once, in order (parity waits must not skip phases), and before
-        // the arrival that lets the next PV be issued.  All threads of a row see the same `need`.
+        // the arrival that lets the next PV be issued.
         bool waited_prev = false;
         if (!first && __any_sync(0xffffffffu, need)) {
           ok = __all_sync(0xffffffffu, mbar_wait(&sh.o_full[sx], co & 1, abort_flag));
@@ -482,13 +437,13 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
           if (!ok) break;
           tc_fence_after();
 #pragma unroll
-          for (int c = 0; c < OCOLS / 32; ++c) {
-            uint32_t r[32];
-            tmem_ld32(o_addr + c * 32, r);
+          for (int c = 0; c < HD / 16; ++c) {               // (16 columns at a time: the scores stay in registers)
+            uint32_t v[16];
+            tmem_ld16(o_addr + c * 16, v);
             tmem_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * alpha);
-            tmem_st32(o_addr + c * 32, r);
+            for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) * alpha);
+            tmem_st16(o_addr + c * 16, v);
           }
           tmem_wait_st();
         }
@@ -498,36 +453,17 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         float2 sum2 = make_float2(0.f, 0.f);              // (two scores per FMA / add: packed fp32 instructions)
         const float2 sl22 = make_float2(sl2, sl2), nmb2 = make_float2(-mb, -mb);
 #pragma unroll
-        for (int c = 0; c < SCOLS / 32; ++c) {
-          // second sweep: the scores again (tensor-memory reads are cheap; keeping them in registers
-          // is not, with 576 threads per CTA), P written over them
-          uint32_t r[32];
-          tmem_ld32(s_addr + col0 + c * 32, r);
-          tmem_wait_ld();
+        for (int c = 0; c < 4; ++c) {
           uint32_t pk[16];
-          if (full) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float2 arg = __ffma2_rn(make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), sl22, nmb2);
-              const float2 pp = make_float2(ex2(arg.x), ex2(arg.y));
-              sum2 = __fadd2_rn(sum2, pp);
-              const __nv_bfloat162 v = __floats2bfloat162_rn(pp.x, pp.y);
-              pk[i] = *(const uint32_t*)&v;
-            }
-          } else {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float2 arg = __ffma2_rn(make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), sl22, nmb2);
-              float p0 = ex2(arg.x);
-              float p1 = ex2(arg.y);
-              if (!(vmask[c] & (1u << (2 * i)))) p0 = 0.f;
-              if (!(vmask[c] & (2u << (2 * i)))) p1 = 0.f;
-              sum2 = __fadd2_rn(sum2, make_float2(p0, p1));
-              const __nv_bfloat162 v = __floats2bfloat162_rn(p0, p1);
-              pk[i] = *(const uint32_t*)&v;
-            }
+          for (int i = 0; i < 16; ++i) {
+            const float2 arg = __ffma2_rn(make_float2(__uint_as_float(r[c][2 * i]), __uint_as_float(r[c][2 * i + 1])), sl22, nmb2);
+            const float2 pp = make_float2(ex2(arg.x), ex2(arg.y));
+            sum2 = __fadd2_rn(sum2, pp);
+            const __nv_bfloat162 v = __floats2bfloat162_rn(pp.x, pp.y);
+            pk[i] = *(const uint32_t*)&v;
           }
-          tmem_st16(s_addr + col0 + c * 16, pk);      // inside this thread's own score columns
+          tmem_st16(s_addr + c * 16, pk);
         }
         l += sum2.x + sum2.y;
         tmem_wait_st();
@@ -542,19 +478,17 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         ++cs;
       }
       if (!ok) break;
-      // epilogue: O / l -> Y, once the item's last PV has landed; l = the partial row sums together
-      ok = __all_sync(0xffffffffu, row_exchange<false>(&sh.xsum[ci & 1][sx][0][0], part, row, ci + 1, l, abort_flag));
-      if (!ok) break;
+      // epilogue: O / l -> Y, once the item's last PV has landed
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.o_full[sx], co & 1, abort_flag));
       ++co;
       if (!ok) break;
       tc_fence_after();
       const float inv = 1.f / l;
       const bool store = p < x.n && FF_DBG_OK(p >= 0 && x.bh >= 0 && x.bh < dm.BH, P.status, 1);
-      __nv_bfloat16* y = (x.band == 1 ? P.y_mid : P.y_high) + ((size_t)x.bh * x.n + (store ? p : 0)) * HD + ocol0;
-      float* yl = HAS_LOW && x.band == 0 ? P.y_low + ((size_t)x.bh * x.n + (store ? p : 0)) * HD + ocol0 : nullptr;   // low band: fp32
+      __nv_bfloat16* y = (x.band == 1 ? P.y_mid : P.y_high) + ((size_t)x.bh * x.n + (store ? p : 0)) * HD;
+      float* yl = HAS_LOW && x.band == 0 ? P.y_low + ((size_t)x.bh * x.n + (store ? p : 0)) * HD : nullptr;   // low band: fp32
 #pragma unroll
-      for (int c = 0; c < OCOLS / 32; ++c) {
+      for (int c = 0; c < HD / 32; ++c) {
         uint32_t r[32];
         tmem_ld32(o_addr + c * 32, r);
         tmem_wait_ld();
@@ -579,7 +513,6 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
       }
       tc_fence_before();
       mbar_arrive(&sh.o_empty[sx]);
-      ++ci;
     }
   }
 

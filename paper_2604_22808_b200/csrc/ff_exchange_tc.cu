@@ -197,8 +197,10 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
     if (lane == 0) {
       const uint32_t idesc1 = idesc_bf16_f32(XT, nk, false, false);
       const uint32_t idesc2 = idesc_bf16_f32(XT, XD, false, true);
-      const uint32_t zhi = smem_u32(sZhi), zlo = smem_u32(sZlo);
-      const uint32_t zhalf = nk * 128;                    // bytes between the two 64-channel halves of a Z image
+      // operand descriptors, once (assembling them for every instruction is slower than the instruction): token tiles, Z
+      // as the K-major and as the MN-major operand (halves of 64 channels nk * 128 bytes apart), its lo image behind
+      const uint64_t y_desc = smem_desc_sw128(smem_u32(sY), 16, 1024), zk_desc = smem_desc_sw128(smem_u32(sZhi), 16, 1024);
+      const uint64_t zmn_desc = smem_desc_sw128(smem_u32(sZhi), nk * 128, 1024), zlo_step = (uint64_t)(2 * nk * 128 >> 4);
       bool ok = true;
       int prev_bh = -1, zc = 0;
       // S = Y (Zhi + Zlo)^T of the CTA's tile n, K = head_dim
@@ -214,13 +216,14 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         if (!mbar_wait(&sh.y_full[slot], (n / YB) & 1, abort_flag)) return false;
         XPROF_ADD(1, x1);
         tc_fence_after();
-        const uint32_t ybase = smem_u32(sY + slot * X_TILE_BYTES), s_tm = tmem + (SB == 2 ? (n & 1) * 64 : 0);
+        const uint64_t y = y_desc + (uint64_t)(slot * (X_TILE_BYTES >> 4));
+        const uint32_t s_tm = tmem + (SB == 2 ? (n & 1) * 64 : 0);
 #pragma unroll
         for (int k = 0; k < XD / 16; ++k) {
-          const uint64_t a = smem_desc_sw128(ybase + (k >> 2) * X_HALF + (k & 3) * 32, 16, 1024);
-          const uint32_t zo = (k >> 2) * zhalf + (k & 3) * 32;
-          umma_ss(s_tm, a, smem_desc_sw128(zhi + zo, 16, 1024), idesc1, k > 0 ? 1u : 0u);
-          umma_ss(s_tm, a, smem_desc_sw128(zlo + zo, 16, 1024), idesc1, 1u);
+          const uint64_t a = y + (uint64_t)(((k >> 2) * X_HALF + (k & 3) * 32) >> 4);
+          const uint64_t zo = (uint64_t)(((k >> 2) * nk * 128 + (k & 3) * 32) >> 4);
+          umma_ss(s_tm, a, zk_desc + zo, idesc1, k > 0 ? 1u : 0u);
+          umma_ss(s_tm, a, zk_desc + zlo_step + zo, idesc1, 1u);
         }
         umma_commit(&sh.s_full[n & 1]);
         if (REREAD) umma_commit(&sh.y_empty[slot]);       // the tile has been read
@@ -248,9 +251,9 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
 #pragma unroll
         for (int k = 0; k < NK; ++k) {                    // D = (Phi + Plo) (Zhi + Zlo) without lo*lo, K = keys
           if (sh.keys[x.band - 1][k] == 0) continue;
-          const uint64_t bh_ = smem_desc_sw128(zhi + k * 2048, zhalf, 1024);
+          const uint64_t bh_ = zmn_desc + (uint64_t)(k * (2048 >> 4));
           umma_ts(tmem + 128, p_tm + k * 16, bh_, idesc2, acc);
-          umma_ts(tmem + 128, p_tm + k * 16, smem_desc_sw128(zlo + k * 2048, zhalf, 1024), idesc2, 1u);
+          umma_ts(tmem + 128, p_tm + k * 16, bh_ + zlo_step, idesc2, 1u);
           umma_ts(tmem + 128, p_tm + k * 16 + 8, bh_, idesc2, 1u);
           acc = 1;
         }

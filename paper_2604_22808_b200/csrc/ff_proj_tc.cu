@@ -96,6 +96,8 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(PM, PN, /*a_mn_major=*/false, /*b_mn_major=*/true);
+      // (operand descriptors once: a slot or a step inside one is a constant in the address field)
+      const uint64_t a0 = smem_desc_sw128(smem_u32(smem), 16, 1024), b0 = smem_desc_sw128(smem_u32(smem) + A_BYTES, B_PIECE, 1024);
       unsigned n = 0, nt = 0;
       bool ok = true;
       for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++nt) {
@@ -108,11 +110,10 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
           ok = mbar_wait(&sh.full[slot], (n / P_NSTAGE) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t abase = smem_u32(smem + slot * P_STAGE), bbase = abase + A_BYTES;
+          const uint64_t step = (uint64_t)(slot * (P_STAGE >> 4));
 #pragma unroll
           for (int ks = 0; ks < PK / 16; ++ks)
-            umma_ss(tm + ab * PN, smem_desc_sw128(abase + ks * 32, 16, 1024), smem_desc_sw128(bbase + ks * 2048, B_PIECE, 1024),
-                    idesc, (kc > 0 || ks > 0) ? 1u : 0u);
+            umma_ss(tm + ab * PN, a0 + step + (uint64_t)(ks * 2), b0 + step + (uint64_t)(ks * 128), idesc, ks > 0 ? 1u : (kc > 0 ? 1u : 0u));
           umma_commit(&sh.empty[slot]);
         }
         umma_commit(&sh.acc_full[ab]);

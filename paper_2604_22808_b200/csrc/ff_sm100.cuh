@@ -10,6 +10,10 @@ namespace sm100 {
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// Moves registers between the warpgroups of a block (whole warpgroup; the shares add up to the launch's total).
+template <int N> __device__ __forceinline__ void reg_inc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void reg_dec() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
+
 // max of three (one instruction on sm_100)
 __device__ __forceinline__ float max3f(float a, float b, float c) {
   float r;
