@@ -17,8 +17,8 @@
 //   warps 4..11  softmax: per stream one thread per query row (row = TMEM lane); the row's 128 scores are read into
 //                registers once, key masks are generated from the row's band rank, P is written back to tensor memory
 //                as bf16 over the scores; O accumulates in tensor memory and is rescaled only when a row maximum grows
-//                by > 2^8.  The registers of the first warpgroup (120 are left of 168 a thread) go to these two
-//                (192): 128 x 120 + 256 x 192 = 384 x 168.  With two threads a row, a shared-memory hand-shake for the
+//                by > 2^8.  The registers of the first warpgroup (104 are left of 168 a thread) go to these two
+//                (200): 128 x 104 + 256 x 200 = 384 x 168.  With two threads a row, a shared-memory hand-shake for the
 //                maximum and a second read of the scores the launch took 1.37 instead of 1.17 ms (64K tokens, 24 heads,
 //                all bands)
 // Tensor memory (512 columns): S/P of stream A, S/P of stream B, O of stream A, O of stream B.
@@ -64,11 +64,12 @@ struct Item {
   int nk;             // key tiles of the item
   long long n;        // band length
   long long ks;       // high: first key rank of key tile 0
+  int lo[2], hi[2];   // key tiles lo .. hi that streams A and B take part in
 };
 
 struct Shared {
   uint64_t q_full, q_empty, k_full[2], k_empty[2], v_full[2], v_empty[2];
-  uint64_t s_full[2], p_full[2], o_full[2], o_empty[2];      // per stream
+  uint64_t s_full[2], p_half[2], p_full[2], o_full[2], o_empty[2];      // per stream
   uint32_t tmem_base;
   int abort_flag;
   int n_units, total;
@@ -118,18 +119,22 @@ __device__ __forceinline__ Item decode_item(const Shared& sh, const FFDims& dm, 
     if (ke > x.n) ke = x.n;
     x.nk = (int)((ke - x.ks + TILE - 1) / TILE);
   }
+  // Mid and low band: every tile.  High band: the tiles that meet the window of the stream's 128 query rows.
+#pragma unroll
+  for (int sx = 0; sx < 2; ++sx) {
+    x.lo[sx] = 0; x.hi[sx] = x.nk - 1;
+    if (x.band == 2) {
+      const long long q0 = (long long)(x.tile_a + sx) * TILE, q1 = q0 + TILE - 1 + dm.R < x.n - 1 ? q0 + TILE - 1 + dm.R : x.n - 1;
+      const long long first = q0 - dm.R - x.ks;             // (tile 0 holds it or what is left of it)
+      x.lo[sx] = first > 0 ? (int)(first / TILE) : 0;
+      x.hi[sx] = (int)((q1 - x.ks) / TILE);
+    }
+    if (sx == 1 && !x.has_b) { x.lo[1] = 1; x.hi[1] = 0; }
+  }
   return x;
 }
 
-// Does stream `sx` (0 = A, 1 = B) take part in key tile j of the item?  Mid band: always.  High
-// band: when the tile meets the window of the stream's 128 query rows.
-__device__ __forceinline__ bool stream_active(const Item& x, const FFDims& dm, int sx, int j) {
-  if (sx == 1 && !x.has_b) return false;
-  if (x.band != 2) return true;
-  const long long t0 = x.ks + (long long)j * TILE;
-  const long long q0 = (long long)(x.tile_a + sx) * TILE;
-  return t0 <= q0 + TILE - 1 + dm.R && t0 + TILE - 1 >= q0 - dm.R && t0 < x.n;
-}
+__device__ __forceinline__ bool stream_active(const Item& x, int sx, int j) { return j >= x.lo[sx] && j <= x.hi[sx]; }
 
 // Band rank of class-local position u of residue class c (mid band).
 // (32-bit arithmetic: positions and ranks stay below 2^32 for every supported size.)
@@ -191,7 +196,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
     for (int i = 0; i < 2; ++i) {
       mbar_init(&sh.k_full[i], 1); mbar_init(&sh.k_empty[i], 1);
       mbar_init(&sh.v_full[i], 1); mbar_init(&sh.v_empty[i], 1);
-      mbar_init(&sh.s_full[i], 1); mbar_init(&sh.p_full[i], 128);
+      mbar_init(&sh.s_full[i], 1); mbar_init(&sh.p_half[i], 128); mbar_init(&sh.p_full[i], 128);
       mbar_init(&sh.o_full[i], 1); mbar_init(&sh.o_empty[i], 128);
     }
     sh.abort_flag = 0;
@@ -217,7 +222,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
   volatile int* abort_flag = &sh.abort_flag;
 
   if (warp < 4) {
-  reg_dec<120>();
+  reg_dec<104>();
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
@@ -253,7 +258,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    {
       const uint32_t idesc_qk = idesc_bf16_f32(TILE, TILE, false, false);
       const uint32_t idesc_pv = idesc_bf16_f32(TILE, HD, false, true);
       int iter = 0; unsigned g = 0;
@@ -279,56 +284,62 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         if (last) umma_commit(&sh.k_empty[st]);
         if (release_q) umma_commit(&sh.q_empty);
       };
-      // O_x (+)= P_x V[tile]
-      auto issue_pv = [&](int sx, unsigned gt, bool first_of_item, bool last) -> bool {
+      // O_x (+)= P_x V[tile]: the first 64 keys while the softmax works on the others
+      auto issue_pv = [&](int sx, unsigned gt, bool first_of_item, bool last, bool last_of_item) -> bool {
         const int st = gt & 1;
-        if (!mbar_wait(&sh.p_full[sx], cp[sx] & 1, abort_flag)) return false;
-        ++cp[sx];
-        if (first_of_item && ce[sx] >= 1 && !mbar_wait(&sh.o_empty[sx], (ce[sx] - 1) & 1, abort_flag)) return false;
+        if (!mbar_wait_warp(&sh.p_half[sx], cp[sx] & 1, abort_flag)) return false;
+        if (first_of_item && ce[sx] >= 1 && !mbar_wait_warp(&sh.o_empty[sx], (ce[sx] - 1) & 1, abort_flag)) return false;
         tc_fence_after();
         const uint64_t vd = v_desc + (uint64_t)(st * (TILE_BYTES >> 4));
         const uint32_t p_tm = tm + sx * 128, d_tm = p_tm + 256, first = first_of_item ? 0u : 1u;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
+          if (k == 4) {
+            if (!mbar_wait_warp(&sh.p_full[sx], cp[sx] & 1, abort_flag)) return false;
+            ++cp[sx];
+            tc_fence_after();
+          }
           umma_ts(d_tm, p_tm + k * 8,                      // (P of keys 16 k .. 16 k + 15: eight columns)
                   vd + (uint64_t)(k * (2048 >> 4)), idesc_pv, k == 0 ? first : 1u);
         }
-        umma_commit(&sh.o_full[sx]);
+        if (last_of_item) umma_commit(&sh.o_full[sx]);
         if (last) umma_commit(&sh.v_empty[st]);
         return true;
       };
       for (int it = blockIdx.x; it < total && ok; it += gridDim.x, ++iter) {
         const Item x = decode_item<HAS_LOW>(sh, dm, it);
-        ok = mbar_wait(&sh.q_full, iter & 1, abort_flag);
+        ok = mbar_wait_warp(&sh.q_full, iter & 1, abort_flag);
         if (!ok) break;
         const unsigned g0 = g;
         bool started[2] = {false, false};
         // key tile 0: QK of both streams
-        ok = mbar_wait(&sh.k_full[g0 & 1], (g0 >> 1) & 1, abort_flag);
+        ok = mbar_wait_warp(&sh.k_full[g0 & 1], (g0 >> 1) & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
         {
-          const bool a0 = stream_active(x, dm, 0, 0), b0 = stream_active(x, dm, 1, 0);
+          const bool a0 = stream_active(x, 0, 0), b0 = stream_active(x, 1, 0);
           if (a0) issue_qk(0, g0, !b0, x.nk == 1 && !b0);
           if (b0) issue_qk(1, g0, true, x.nk == 1);
         }
         for (int j = 0; j < x.nk && ok; ++j) {
           const unsigned gt = g0 + j;
-          const bool aj = stream_active(x, dm, 0, j), bj = stream_active(x, dm, 1, j);
+          const bool aj = stream_active(x, 0, j), bj = stream_active(x, 1, j);
           const bool more = j + 1 < x.nk;
-          const bool an = more && stream_active(x, dm, 0, j + 1), bn = more && stream_active(x, dm, 1, j + 1);
+          const bool an = more && stream_active(x, 0, j + 1), bn = more && stream_active(x, 1, j + 1);
           bool v_ready = false, k_ready = false;
-          for (int sx = 0; sx < 2 && ok; ++sx) {
+#pragma unroll
+          for (int sx = 0; sx < 2; ++sx) {
+            if (!ok) break;
             const bool act = sx ? bj : aj, nxt = sx ? bn : an;
             if (act) {
-              if (!v_ready) { ok = mbar_wait(&sh.v_full[gt & 1], (gt >> 1) & 1, abort_flag); v_ready = true; if (!ok) break; }
+              if (!v_ready) { ok = mbar_wait_warp(&sh.v_full[gt & 1], (gt >> 1) & 1, abort_flag); v_ready = true; if (!ok) break; }
               const bool last_pv = sx == 1 || !bj;
-              ok = issue_pv(sx, gt, !started[sx], last_pv);
+              ok = issue_pv(sx, gt, !started[sx], last_pv, !nxt);
               started[sx] = true;
               if (!ok) break;
             }
             if (nxt) {
-              if (!k_ready) { ok = mbar_wait(&sh.k_full[(gt + 1) & 1], ((gt + 1) >> 1) & 1, abort_flag); k_ready = true; if (!ok) break; tc_fence_after(); }
+              if (!k_ready) { ok = mbar_wait_warp(&sh.k_full[(gt + 1) & 1], ((gt + 1) >> 1) & 1, abort_flag); k_ready = true; if (!ok) break; tc_fence_after(); }
               const bool last_qk = sx == 1 || !bn;
               issue_qk(sx, gt + 1, last_qk, last_qk && j + 2 == x.nk);
             }
@@ -341,7 +352,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
     }
   }
   } else {
-    reg_inc<192>();
+    reg_inc<200>();
     // ------------------------------------------------------------------ softmax
     // Warps 4..7 serve stream A, 8..11 stream B (a warp reaches the TMEM lanes 32*(warp%4)..+31).
     const int quarter = warp & 3;
@@ -352,7 +363,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
     const uint32_t o_addr = tm + lane_addr + 256 + sx * 128;
     const float sl2 = rsqrtf((float)HD) * 1.4426950408889634f;
     unsigned cs = 0;                  // key tiles this stream has processed (phases of s_full / p_full)
-    unsigned co = 0;                  // phases of o_full consumed
+    unsigned co = 0;                  // phases of o_full consumed: one per item
     bool ok = true;
     for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
       const Item x = decode_item<HAS_LOW>(sh, dm, it);
@@ -363,8 +374,8 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
       const long long p = x.band == 1 ? mid_rank(dm, x.c, u_q) : u_q;
       float m_ref = -1e30f, l = 0.f;
       bool first = true;
-      for (int j = 0; j < x.nk && ok; ++j) {
-        if (!stream_active(x, dm, sx, j)) continue;
+      const int j_lo = sx ? x.lo[1] : x.lo[0], j_hi = sx ? x.hi[1] : x.hi[0];
+      for (int j = j_lo; j <= j_hi && ok; ++j) {
         // valid key columns [clo, chi] of this row in this tile
         int clo = 0, chi = TILE - 1;
         bool full;
@@ -424,18 +435,9 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         const float m_new = fmaxf(m_ref, tmax);
         const bool need = (m_new - m_ref) * sl2 > LAZY_LOG2;
         const float alpha = need ? ex2((m_ref - m_new) * sl2) : 1.f;
-        // The phase of the previous PV of this stream is normally consumed at the end of this tile,
-        // just before P is published, when it has long completed; only a row maximum that grew past
-        // the lazy threshold needs it now, because O is then rescaled in place.  Every phase of the
-        // barrier is awaited exactly once, in order (parity waits must not skip phases), and before
-        // the arrival that lets the next PV be issued.
-        bool waited_prev = false;
+        // The previous PV of this stream has completed: the scores of this tile, which s_full announces, were issued
+        // behind it by the same thread.  So O may be rescaled in place.
         if (!first && __any_sync(0xffffffffu, need)) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&sh.o_full[sx], co & 1, abort_flag));
-          ++co;
-          waited_prev = true;
-          if (!ok) break;
-          tc_fence_after();
 #pragma unroll
           for (int c = 0; c < HD / 16; ++c) {               // (16 columns at a time: the scores stay in registers)
             uint32_t v[16];
@@ -464,16 +466,13 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
             pk[i] = *(const uint32_t*)&v;
           }
           tmem_st16(s_addr + c * 16, pk);
+          if (c & 1) {                                    // 64 keys are there
+            tmem_wait_st();
+            tc_fence_before();
+            mbar_arrive(c == 1 ? &sh.p_half[sx] : &sh.p_full[sx]);
+          }
         }
         l += sum2.x + sum2.y;
-        tmem_wait_st();
-        if (!first && !waited_prev) {
-          ok = __all_sync(0xffffffffu, mbar_wait(&sh.o_full[sx], co & 1, abort_flag));
-          ++co;
-          if (!ok) break;
-        }
-        tc_fence_before();
-        mbar_arrive(&sh.p_full[sx]);
         first = false;
         ++cs;
       }

@@ -325,7 +325,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     // ------------------------------------------------------------------ MMA issuer, phase 1
     // batches of bt input tiles (neighbouring slots of the ring), N = 32 bt.  A descriptor advances by
     // 1024 bytes (64 in its address field) per 16 rows of K.
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(ROWS, bt * CHK, /*a_mn_major=*/false, /*b_mn_major=*/true);
       const uint32_t in_base = smem_u32(sIn);
       unsigned n1b = 0;
@@ -335,10 +335,10 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           const int ab = n1b % NA1;
           const unsigned nt = bt * n1b;                            // index of the batch's first tile in the ring sequence
           PROF_T0(tm0);
-          for (int i = 0; i < bt && ok; ++i) ok = mbar_wait(&sh.in_full[(nt + i) % nslot], ((nt + i) / nslot) & 1, abort_flag);
+          for (int i = 0; i < bt && ok; ++i) ok = mbar_wait_warp(&sh.in_full[(nt + i) % nslot], ((nt + i) / nslot) & 1, abort_flag);
           PROF_ADD(7, tm0);
           PROF_T0(tm1);
-          if (ok && n1b >= (unsigned)NA1) ok = mbar_wait(&sh.acc1_empty[ab], ((n1b / NA1) - 1) & 1, abort_flag);
+          if (ok && n1b >= (unsigned)NA1) ok = mbar_wait_warp(&sh.acc1_empty[ab], ((n1b / NA1) - 1) & 1, abort_flag);
           PROF_ADD(8, tm1);
           if (!ok) break;
           tc_fence_after();
@@ -367,7 +367,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   } else if (warp == 3) {
     // ------------------------------------------------------------------ MMA issuer, phase 2
     // (a thread of its own: phase 2 of an item waits for the whole cluster, phase 1 of the next item does not)
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(ROWS, bt * CHK, /*a_mn_major=*/false, /*b_mn_major=*/true);
       const uint32_t buf_base = smem_u32(sBuf);
       unsigned n2b = 0, ni = 0;
@@ -376,15 +376,15 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         // the plane's rows have landed in this CTA's buffer
         PROF_T0(tm2);
         const int sl = (int)(ni % nsl);                             // the item's slot of the plane buffer
-        ok = half_start ? mbar_wait(&sh.buf_half[sl], (ni / nsl) & 1, abort_flag)
-                        : mbar_wait_cluster(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
+        ok = half_start ? mbar_wait_warp(&sh.buf_half[sl], (ni / nsl) & 1, abort_flag)
+                        : __all_sync(0xffffffffu, mbar_wait_cluster(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag));
         PROF_ADD(9, tm2);
         if (!ok) break;
         fence_proxy_async_all();
         for (int kb = 0; kb < nb && ok; ++kb, ++n2b) {
           const int ab = n2b % NA2;
           PROF_T0(tm3);
-          if (n2b >= (unsigned)NA2) ok = mbar_wait(&sh.acc2_empty[ab], ((n2b / NA2) - 1) & 1, abort_flag);
+          if (n2b >= (unsigned)NA2) ok = mbar_wait_warp(&sh.acc2_empty[ab], ((n2b / NA2) - 1) & 1, abort_flag);
           PROF_ADD(10, tm3);
           if (!ok) break;
           tc_fence_after();
@@ -395,7 +395,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           for (int ks = 0; ks < ROWS / 16; ++ks) {
             if (ks == ROWS / 32 && kb == 0 && half_start) {          // the second half of the rows
               PROF_T0(tm4);
-              ok = mbar_wait_cluster(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
+              ok = __all_sync(0xffffffffu, mbar_wait_cluster(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag));
               PROF_ADD(11, tm4);
               if (!ok) break;
               fence_proxy_async_all();

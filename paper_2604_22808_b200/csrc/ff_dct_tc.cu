@@ -254,17 +254,17 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(TILE_ROWS, CH, /*a_mn_major=*/false, /*b_mn_major=*/true);
       unsigned it = 0;
       bool ok = true;
       for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
         const int slot = it % NSTAGE, ab = it % NACC;
         PROF_T0(pm);
-        ok = mbar_wait(LO8 ? &sh.conv[slot] : &sh.full[slot], (it / NSTAGE) & 1, abort_flag);
+        ok = mbar_wait_warp(LO8 ? &sh.conv[slot] : &sh.full[slot], (it / NSTAGE) & 1, abort_flag);
         PROF_ADD(2, pm);
         PROF_T0(pm2);
-        if (ok && it >= NACC) ok = mbar_wait(&sh.acc_empty[ab], ((it / NACC) - 1) & 1, abort_flag);
+        if (ok && it >= NACC) ok = mbar_wait_warp(&sh.acc_empty[ab], ((it / NACC) - 1) & 1, abort_flag);
         PROF_ADD(3, pm2);
         if (!ok) break;
         tc_fence_after();

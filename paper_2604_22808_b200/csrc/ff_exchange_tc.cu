@@ -194,7 +194,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint32_t idesc1 = idesc_bf16_f32(XT, nk, false, false);
       const uint32_t idesc2 = idesc_bf16_f32(XT, XD, false, true);
       // operand descriptors, once (assembling them for every instruction is slower than the instruction): token tiles, Z
@@ -207,13 +207,13 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
       auto scores = [&](int n, const XItem& x) -> bool {
         if (x.bh != prev_bh) {                            // the head's summaries have arrived
           XPROF_T0(x4);
-          if (!mbar_wait(&sh.z_ready, zc & 1, abort_flag)) return false;
+          if (!mbar_wait_warp(&sh.z_ready, zc & 1, abort_flag)) return false;
           XPROF_ADD(4, x4);
           ++zc; prev_bh = x.bh;
         }
         const int slot = n % YB;
         XPROF_T0(x1);
-        if (!mbar_wait(&sh.y_full[slot], (n / YB) & 1, abort_flag)) return false;
+        if (!mbar_wait_warp(&sh.y_full[slot], (n / YB) & 1, abort_flag)) return false;
         XPROF_ADD(1, x1);
         tc_fence_after();
         const uint64_t y = y_desc + (uint64_t)(slot * (X_TILE_BYTES >> 4));
@@ -239,10 +239,10 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         const bool ahead = SB == 2 && more && next.bh == x.bh;
         if (ahead) ok = scores(n + 1, next);
         XPROF_T0(x2);
-        if (ok) ok = mbar_wait(&sh.p_full[n & 1], (n >> 1) & 1, abort_flag);
+        if (ok) ok = mbar_wait_warp(&sh.p_full[n & 1], (n >> 1) & 1, abort_flag);
         XPROF_ADD(2, x2);
         XPROF_T0(x3);
-        if (ok && n >= 1) ok = mbar_wait(&sh.d_empty, (n - 1) & 1, abort_flag);
+        if (ok && n >= 1) ok = mbar_wait_warp(&sh.d_empty, (n - 1) & 1, abort_flag);
         XPROF_ADD(3, x3);
         if (!ok) break;
         tc_fence_after();

@@ -94,7 +94,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16_f32(PM, PN, /*a_mn_major=*/false, /*b_mn_major=*/true);
       // (operand descriptors once: a slot or a step inside one is a constant in the address field)
       const uint64_t a0 = smem_desc_sw128(smem_u32(smem), 16, 1024), b0 = smem_desc_sw128(smem_u32(smem) + A_BYTES, B_PIECE, 1024);
@@ -102,12 +102,12 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
       bool ok = true;
       for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++nt) {
         const int ab = nt & 1;
-        if (nt >= 2) ok = mbar_wait(&sh.acc_empty[ab], ((nt >> 1) - 1) & 1, abort_flag);
+        if (nt >= 2) ok = mbar_wait_warp(&sh.acc_empty[ab], ((nt >> 1) - 1) & 1, abort_flag);
         if (!ok) break;
         tc_fence_after();
         for (int kc = 0; kc < kchunks && ok; ++kc, ++n) {
           const int slot = n % P_NSTAGE;
-          ok = mbar_wait(&sh.full[slot], (n / P_NSTAGE) & 1, abort_flag);
+          ok = mbar_wait_warp(&sh.full[slot], (n / P_NSTAGE) & 1, abort_flag);
           if (!ok) break;
           tc_fence_after();
           const uint64_t step = (uint64_t)(slot * (P_STAGE >> 4));
