@@ -286,10 +286,13 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     }
   } else if (LO8 && warp >= 10) {
     // ------------------------------------------------------------------ lo bytes -> bf16 lo operand
-    // A thread owns a row of the tile.  For every value: v24 = (hi << 16) | (byte << 8) as fp32; lo = v24 - hi,
-    // exact in bf16.  The bytes arrive as rows of CH bytes (128-byte swizzle for 128 channels, 64-byte for 64),
+    // A thread owns a row of the tile.  For every value v24 = (hi << 16) | (byte << 8) as fp32: lo = v24 - hi =
+    // +-byte 2^(E-15) with hi's sign and exponent E, exact in bf16.  A byte in the low half of a bf16 is byte 2^-133
+    // (below 128 as a subnormal number), so two packed multiplications give two values: by 2^118, and by hi without
+    // its mantissa (+-2^E).  Four instructions a pair; as two fp32 differences and a conversion it took eight.  The bytes arrive as rows of CH bytes (128-byte swizzle for 128 channels, 64-byte for 64),
     // the bf16 tiles as 64-channel halves of 128-byte rows (128-byte swizzle).
     const int r0 = threadIdx.x - 320;
+    const __nv_bfloat162 up = __float2bfloat162_rn(0x1p118f);
     unsigned it = 0;
     bool ok = true;
     for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
@@ -321,11 +324,9 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
         uint32_t ow[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const uint32_t by = lw[2 * c8 + (i >> 1)] >> (16 * (i & 1));              // bytes of channels 2i, 2i+1 in the low half
-          const uint32_t h0 = hw[i] << 16, h1 = hw[i] & 0xffff0000u;
-          const float l0 = __uint_as_float(h0 | ((by & 0xffu) << 8)) - __uint_as_float(h0);
-          const float l1 = __uint_as_float(h1 | (by & 0xff00u)) - __uint_as_float(h1);
-          const __nv_bfloat162 lp = __floats2bfloat162_rn(l0, l1);
+          const uint32_t b2 = __byte_perm(lw[2 * c8 + (i >> 1)], 0u, (i & 1) ? 0x4342 : 0x4140);     // 0x00b1'00b0
+          const uint32_t e2 = hw[i] & 0xff80ff80u;
+          const __nv_bfloat162 lp = __hmul2(__hmul2(*(const __nv_bfloat162*)&b2, up), *(const __nv_bfloat162*)&e2);
           ow[i] = *(const uint32_t*)&lp;
         }
         *(uint4*)(base + TB + off) = make_uint4(ow[0], ow[1], ow[2], ow[3]);
