@@ -3,16 +3,14 @@
 // intermediate between them kept in shared memory.  bf16 storage, 32 channels per work item.
 //
 // A work item is one plane of the grid (all positions of the two axes at one coordinate of the third
-// axis) of one tensor-head, for one chunk of 32 channels.  A thread-block cluster of CS CTAs owns the
-// item: the plane's intermediate (hi/lo bf16, 4 bytes per value) is spread over the CTAs' shared
-// memory, 128 KB or less each.
-//   phase 1  every CTA transforms its share of the plane's w lines (tiles of 128 positions = 128/W
-//            lines, fetched by TMA) and scatters each result row, as a hi/lo bf16 pair, into the
-//            shared memory of the CTA that owns the row's w coefficient (st.shared::cluster); the
-//            rows land in the operand layout of phase 2
-//   phase 2  every CTA transforms the second axis for its share of the w coefficients (tiles of
-//            128/n2 neighbouring coefficients x all n2 positions), straight from its part of the
-//            buffer, and stores the result with tensor stores (hi/lo grids, or the caller's tensor)
+// axis) of one tensor-head, for one chunk of 32 channels.  A CTA owns the item: the plane's
+// intermediate (hi/lo bf16, 4 bytes per value) takes 128 KB or less of its shared memory.
+//   phase 1  transforms the plane's w lines (tiles of 128 positions = 128/W lines, fetched by TMA) and
+//            scatters each result row, as a hi/lo bf16 pair, into the plane buffer; the rows land in
+//            the operand layout of phase 2
+//   phase 2  transforms the second axis (tiles of 128/n2 neighbouring w coefficients x all n2
+//            positions), straight from the buffer, and stores the result with tensor stores (hi/lo
+//            grids, or the caller's tensor)
 // Both contractions are D[j][c] = sum_r A[j][r] X[r][c] over tiles of 128 positions x 32 channels
 // with the matrix A = I kron Mat (w lines follow one another) or Mat kron I (lines of the second
 // axis interleave) held in TENSOR MEMORY as the A operand (hi and lo bf16 parts, 64 columns each),
@@ -22,13 +20,13 @@
 //
 //   warp 0        TMA producer (ring of 8 tiles, or 4 hi/lo pairs)
 //   warp 1        tcgen05.mma issuer of phase 1; owns the tensor-memory allocation
-//   warp 2        tells the cluster when this CTA has finished reading its part of the buffer
+//   warp 2        idle
 //   warp 3        tcgen05.mma issuer of phase 2
 //   warps 4..11   phase-1 epilogue (a thread owns one position of a tile; the first four warps take
 //                 the first tile of a pair, the next four the second)
 //   warps 12..19  phase-2 epilogue
 // so that phase 1 of the next item runs while phase 2 of the current one drains.
-// Hand-shakes across the cluster use mbarriers with remote arrivals; every wait is bounded.
+// Every wait is bounded.
 #include <cuda.h>
 
 #include <vector>
@@ -45,8 +43,8 @@ constexpr int ROWS = 128;                     // positions per tile
 constexpr int TILE_B = ROWS * CHK * 2;        // 8 KB: one bf16 tile
 constexpr int NSTG = 8;                       // input ring: at most 8 tiles (64 KB: 8 bf16 tiles or 4 hi/lo pairs)
 constexpr int RING_B = NSTG * TILE_B;
-constexpr int MAX_TPC = 8;                    // tiles per CTA and item (128 KB of hi/lo buffer)
-constexpr int D2_THREADS = 640;                 // TMA, MMA 1, release, MMA 2, 8 phase-1 and 8 phase-2 epilogue warps
+constexpr int MAX_TPC = 8;                    // tiles of a plane (128 KB of hi/lo buffer)
+constexpr int D2_THREADS = 640;                 // TMA, MMA 1, idle, MMA 2, 8 phase-1 and 8 phase-2 epilogue warps
 constexpr int NA1 = 1, NA2 = 1;               // accumulator buffers (batches of 128 columns) of the two phases
 constexpr int IMG_CELLS = 64;                 // 32-bit tensor-memory cells per matrix row: two bf16 K elements each
 constexpr int STG_ROW = 64;                   // bytes per staged row (32 channels)
@@ -61,8 +59,7 @@ struct Dct2Params {
   int last;                // output is the caller's tensor (bf16, no lo part)
   int group, group_start;
   int nchunk;              // head_dim / 32
-  int tpc;                 // tiles per CTA and item
-  int cs;                  // CTAs per cluster
+  int tpc;                 // tiles of a plane
   double* clear;           // band energies to clear for the sums that follow (first launch of a routed forward), or NULL
   int* status;
 };
@@ -80,11 +77,10 @@ struct D2Shared {
   uint64_t in_full[NSTG], in_empty[NSTG], acc1_full[NA1], acc1_empty[NA1], acc2_full[NA2], acc2_empty[NA2];
   // The plane buffer has one slot of 8 tiles or two of 4 (items alternate): phase 1 of the next item fills one
   // slot while phase 2 of the current item reads the other.
-  uint64_t buf_full[2];    // all rows of the item have landed in this CTA's slot (arrivals from every CTA's warps)
-  uint64_t buf_half[2];    // (one CTA per plane) the rows of the first half of the second axis have landed
-  uint64_t half_free[2];   // (one CTA per plane) phase 2 has finished reading those rows (its k-steps 0..3 of every batch)
-  uint64_t buf_free[2];    // every CTA of the cluster has finished reading the slot (phase 2 of the item)
-  uint64_t mma2_done[2];   // this CTA's phase-2 instructions of the item (by slot) have completed
+  uint64_t buf_full[2];    // all rows of the item have landed in the slot
+  uint64_t buf_half[2];    // the rows of the first half of the second axis have landed
+  uint64_t half_free[2];   // phase 2 has finished reading those rows (its k-steps 0..3 of every batch)
+  uint64_t buf_free[2];    // phase 2 of the item has finished reading the slot
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -101,62 +97,9 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t smem_addr, uint32_t 
   return d;
 }
 
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_id_x() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_count_x() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
-  return r;
-}
-// Address of the same shared-memory location in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint4 v) {
-  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-               : "memory");
-}
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar_addr) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait on a barrier whose arrivals come from other CTAs of the cluster.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait_cluster(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (true) {
-    if (mbar_try_wait_cluster(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if (clock64() - t0 > kWaitLimitCycles) { *abort_flag = 1; return false; }
-  }
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
-
 __device__ __forceinline__ void tma_load_5d(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2,
                                             int c3, int c4) {
   asm volatile(
@@ -174,7 +117,7 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
-// Item `it` of the launch: chunk fastest (clusters that run side by side read neighbouring 64-byte
+// Item `it` of the launch: chunk fastest (CTAs that run side by side read neighbouring 64-byte
 // pieces of the same rows), then the coordinate of the remaining axis, then the tensor-head.
 __device__ __forceinline__ void decode_item(const Dct2Params& P, int it, int& gi, int& a3, int& chunk) {
   chunk = it % P.nchunk;
@@ -217,21 +160,18 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   D2Shared& sh = *(D2Shared*)(sIn + RING_B);
   const int nslot = RING_B / STAGE_B;                              // ring slots: 8 tiles, or 4 hi/lo pairs
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();
-  const int cs = P.cs;
   const int n1 = P.n1, n2 = P.n2;
   const int ln1 = 31 - __clz(n1);
   const int kf1 = ROWS / n1, kf2 = ROWS / n2;
   const int lkf2 = 31 - __clz(kf2);
-  const int ltpc = 31 - __clz(tpc);
   const int total = P.group * P.n3 * P.nchunk;
   const int nsl = tpc <= MAX_TPC / 2 ? 2 : 1;                      // slots of the plane buffer
   const int bt = tpc < 4 ? tpc : 4;                                // tiles per instruction batch (N = 32 bt columns): an
   const int nb = tpc / bt;                                         // instruction costs the same for any N up to 128
-  // One CTA per plane and an even number of batches: the first half of the phase-1 batches holds the first half
+  // With an even number of batches the first half of the phase-1 batches holds the first half
   // of the second axis, i.e. rows 0..63 of every phase-2 tile = its k-steps 0..3.  Phase 2 of the item's first
   // batch starts on those while phase 1 still works on the second half.
-  const bool half_start = cs == 1 && nb >= 2 && (nb & 1) == 0;
+  const bool half_start = nb >= 2 && (nb & 1) == 0;
   // ... and phase 1 of the next item may overwrite those rows as soon as phase 2 has read them (forward launch:
   // measured slower for the inverse, whose phase 1 issues half as many instructions again)
   const bool half_release = half_start && !P.in_split;
@@ -240,8 +180,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     for (int i = 0; i < NSTG; ++i) { mbar_init(&sh.in_full[i], 1); mbar_init(&sh.in_empty[i], 1); }
     for (int i = 0; i < NA1; ++i) { mbar_init(&sh.acc1_full[i], 1); mbar_init(&sh.acc1_empty[i], 256); }
     for (int i = 0; i < NA2; ++i) { mbar_init(&sh.acc2_full[i], 1); mbar_init(&sh.acc2_empty[i], 256); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&sh.buf_full[i], 8 * cs); mbar_init(&sh.buf_free[i], cs); mbar_init(&sh.buf_half[i], 8); }
-    mbar_init(&sh.mma2_done[0], 1); mbar_init(&sh.mma2_done[1], 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(&sh.buf_full[i], 8); mbar_init(&sh.buf_free[i], 1); mbar_init(&sh.buf_half[i], 8); }
     mbar_init(&sh.half_free[0], 1); mbar_init(&sh.half_free[1], 1);
     sh.abort_flag = 0;
     fence_mbar_init();
@@ -249,9 +188,6 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
-  // every CTA's barriers exist before any peer arrives at them
-  cluster_arrive();
-  cluster_wait();
   tc_fence_after();
   const uint32_t tm = sh.tmem_base;
   volatile int* abort_flag = &sh.abort_flag;
@@ -286,7 +222,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   __syncthreads();
   tc_fence_after();
 
-  const int cid = (int)cluster_id_x(), ncl = (int)cluster_count_x();
+  const int cid = (int)blockIdx.x, ncl = (int)gridDim.x;
   PROF_T0(t_all);
 
   if (warp == 0) {
@@ -312,7 +248,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           PROF_ADD(12, tp0);
           if (!ok) break;
           uint8_t* dst = sIn + slot * STAGE_B;
-          const int u1 = (int)rank * tpc + k;                      // tile of the plane: lines u1 kf1 .. + kf1
+          const int u1 = k;                                        // tile of the plane: lines u1 kf1 .. + kf1
           const int b0 = u1 * kf1;
           const int ch = P.axis2 == 1 ? b0 : a3, ct = P.axis2 == 1 ? a3 : b0;
           mbar_arrive_expect_tx(&sh.in_full[slot], STAGE_B);
@@ -366,7 +302,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     }
   } else if (warp == 3) {
     // ------------------------------------------------------------------ MMA issuer, phase 2
-    // (a thread of its own: phase 2 of an item waits for the whole cluster, phase 1 of the next item does not)
+    // (a thread of its own: phase 2 of an item waits for all of its phase 1, phase 1 of the next item does not)
     {
       const uint32_t idesc = idesc_bf16_f32(ROWS, bt * CHK, /*a_mn_major=*/false, /*b_mn_major=*/true);
       const uint32_t buf_base = smem_u32(sBuf);
@@ -377,10 +313,10 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         PROF_T0(tm2);
         const int sl = (int)(ni % nsl);                             // the item's slot of the plane buffer
         ok = half_start ? mbar_wait_warp(&sh.buf_half[sl], (ni / nsl) & 1, abort_flag)
-                        : __all_sync(0xffffffffu, mbar_wait_cluster(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag));
+                        : mbar_wait_warp(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
         PROF_ADD(9, tm2);
         if (!ok) break;
-        fence_proxy_async_all();
+        fence_proxy_async();
         for (int kb = 0; kb < nb && ok; ++kb, ++n2b) {
           const int ab = n2b % NA2;
           PROF_T0(tm3);
@@ -395,10 +331,10 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           for (int ks = 0; ks < ROWS / 16; ++ks) {
             if (ks == ROWS / 32 && kb == 0 && half_start) {          // the second half of the rows
               PROF_T0(tm4);
-              ok = __all_sync(0xffffffffu, mbar_wait_cluster(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag));
+              ok = mbar_wait_warp(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
               PROF_ADD(11, tm4);
               if (!ok) break;
-              fence_proxy_async_all();
+              fence_proxy_async();
               tc_fence_after();
             }
             umma_ts(d_tm, tm + COL_A2H + ks * 8, xh + (uint64_t)(ks * 64), idesc, ks > 0 ? 1u : 0u);
@@ -411,23 +347,12 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           if (!ok) break;
           umma_commit(&sh.acc2_full[ab]);
         }
-        umma_commit(&sh.mma2_done[sl]);
-      }
-    }
-  } else if (warp == 2) {
-    // ------------------------------------------------------------------ buffer release
-    if (lane == 0) {
-      unsigned ni = 0;
-      bool ok = true;
-      for (int it = cid; it < total && ok; it += ncl, ++ni) {
-        ok = mbar_wait(&sh.mma2_done[ni % nsl], (ni / nsl) & 1, abort_flag);
-        if (!ok) break;
-        for (int rk = 0; rk < cs; ++rk) mbar_arrive_cluster(mapa(smem_u32(&sh.buf_free[ni % nsl]), (uint32_t)rk));
+        umma_commit(&sh.buf_free[sl]);
       }
     }
   } else if (warp >= 4 && warp < 12) {
     // ------------------------------------------------------------------ phase-1 epilogue
-    // accumulators -> hi/lo rows in the owners' buffers.  A thread owns row (line l1, w coefficient a1)
+    // accumulators -> hi/lo rows in the plane buffer.  A thread owns row (line l1, w coefficient a1)
     // of its tile and sends it as four 16-byte pieces of hi and four of lo, straight from registers.
     const int ew = warp - 4;                               // 0..7
     const int half = ew >> 2;                              // which tile of a pair
@@ -437,8 +362,6 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     const uint32_t buf_base = smem_u32(sBuf);
     const int l1 = j >> ln1, a1 = j & (n1 - 1);
     const int u2 = a1 >> lkf2;                             // phase-2 tile of the plane that takes coefficient a1
-    const uint32_t owner = (uint32_t)(u2 >> ltpc);
-    const int u2l = u2 & (tpc - 1);
     // Eight neighbouring lanes store at once; their rows are kf2 per tile, and rows of different tiles
     // that share (row / 2) % 4 would meet in the same banks: the lanes of tile t of the eight start
     // their four pieces at piece `rot` instead of 0, which spreads them over the banks.
@@ -451,13 +374,13 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       if (ni >= (unsigned)nsl) {
         // (half_release: the first half of the batches writes rows phase 2 releases earlier; the rest waits below)
         ok = half_release ? __all_sync(0xffffffffu, mbar_wait(&sh.half_free[sl], ((ni / nsl) - 1) & 1, abort_flag))
-                        : __all_sync(0xffffffffu, mbar_wait_cluster(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag));
+                        : mbar_wait_warp(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag);
         if (!ok) break;
       }
       if (threadIdx.x == 128) PROF_ADD(1, te0);
       for (int kb = 0; kb < nb && ok; ++kb, ++n1b) {
         if (half_release && kb == nb / 2 && ni >= (unsigned)nsl) {
-          ok = __all_sync(0xffffffffu, mbar_wait_cluster(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag));
+          ok = mbar_wait_warp(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag);
           if (!ok) break;
         }
         const int ab = n1b % NA1;
@@ -477,15 +400,14 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         }
         uint32_t hi[16], lo[16];
         split_hi_lo(r, hi, lo, true);
-        // where the row goes: position b of the second axis, row b kf2 + (a1 mod kf2) of tile u2l of `owner`
-        const int u1 = (int)rank * tpc + bt * kb + tb;
+        // where the row goes: position b of the second axis, row b kf2 + (a1 mod kf2) of tile u2
+        const int u1 = bt * kb + tb;
         const int b = u1 * kf1 + l1;
         const int drow = (b << lkf2) | (a1 & (kf2 - 1));
-        const uint32_t laddr = buf_base + (uint32_t)(sl * tpc + u2l) * 2 * TILE_B + (uint32_t)drow * STG_ROW;
-        const uint32_t daddr = cs == 1 ? laddr : mapa(laddr, owner);
+        const uint32_t daddr = buf_base + (uint32_t)(sl * tpc + u2) * 2 * TILE_B + (uint32_t)drow * STG_ROW;
         const int swz = (drow >> 1) & 3;
-        // (debug build) the row lies inside a tile of the owner's buffer
-        if (!FF_DBG_OK(drow >= 0 && drow < ROWS && u2l >= 0 && u2l < tpc && owner < (uint32_t)cs && b < n2, P.status, 4)) continue;
+        // (debug build) the row lies inside a tile of the buffer
+        if (!FF_DBG_OK(drow >= 0 && drow < ROWS && u2 >= 0 && u2 < tpc && b < n2, P.status, 4)) continue;
         // rotate the pieces by `rot` (two conditional swaps), then piece i of the registers is piece (i + rot) % 4 of the row
         if (rot & 1) {
 #pragma unroll
@@ -506,13 +428,8 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const uint32_t dst = daddr + (uint32_t)((((i + rot) & 3) ^ swz) << 4);
-          if (cs == 1) {                                    // the whole plane is this CTA's: plain shared-memory stores
-            st_shared_v4(dst, make_uint4(hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]));
-            st_shared_v4(dst + TILE_B, make_uint4(lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]));
-          } else {
-            st_cluster_v4(dst, make_uint4(hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]));
-            st_cluster_v4(dst + TILE_B, make_uint4(lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]));
-          }
+          st_shared_v4(dst, make_uint4(hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]));
+          st_shared_v4(dst + TILE_B, make_uint4(lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]));
         }
         }
         if (threadIdx.x == 128) PROF_ADD(2, te2);
@@ -523,17 +440,11 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         }
       }
       if (!ok) break;
-      // this warp's rows of the item are written: tell every CTA of the cluster
+      // this warp's rows of the item are written
       PROF_T0(te4);
-      if (cs == 1) {
-        fence_proxy_async();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.buf_full[sl]);
-      } else {
-        fence_proxy_async_all();
-        __syncwarp();
-        if (lane < cs) mbar_arrive_cluster(mapa(smem_u32(&sh.buf_full[sl]), (uint32_t)lane));
-      }
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.buf_full[sl]);
       if (threadIdx.x == 128) PROF_ADD(6, te4);
     }
   } else if (warp >= 12) {
@@ -586,7 +497,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) {
-          const int u2g = (int)rank * tpc + bt * kb + tb;        // tile of the plane: w coefficients u2g kf2 .. + kf2
+          const int u2g = bt * kb + tb;        // tile of the plane: w coefficients u2g kf2 .. + kf2
           const int cw = u2g * kf2 + l0;
           const int ch = P.axis2 == 1 ? a0 : a3, ct = P.axis2 == 1 ? a3 : a0;
           tma_store_5d(st_hi, &map_oh, chunk * CHK, cw, ch, ct, out_slice);
@@ -610,9 +521,6 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     while (clock64() - t0 < 2000000) { }
     __syncthreads();
   }
-  // no CTA leaves while a peer may still write into its shared memory or arrive at its barriers
-  cluster_arrive();
-  cluster_wait();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tm, 512);
@@ -673,30 +581,11 @@ bool axis_ok(int n) { return n == 16 || n == 32 || n == 64 || n == 128; }
 
 cudaError_t launch(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, const CUtensorMap& m2, const CUtensorMap& moh,
                    const CUtensorMap& mol, Dct2Params& P, cudaStream_t st) {
-  cudaError_t e = cudaSuccess;
   const int items = P.group * P.n3 * P.nchunk;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)P.cs; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  cfg.blockDim = dim3(D2_THREADS); cfg.dynamicSmemBytes = D2_SMEM; cfg.stream = st;
-  int clusters = p->dct2_clusters;
-  if (clusters <= 0) {
-    // how many clusters of this size the device runs at once
-    cfg.gridDim = dim3((unsigned)(p->sm_count / P.cs * P.cs));
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, dct2_tc_kernel, &cfg);
-    if (e != cudaSuccess || n < 1) { (void)cudaGetLastError(); n = P.cs == 1 ? p->sm_count : p->sm_count / P.cs / 2; }
-    if (n < 1) n = 1;
-    clusters = p->dct2_clusters = n;
-  }
-  if (clusters > items) clusters = items;
-  cfg.gridDim = dim3((unsigned)(clusters * P.cs));
-  cfg.numAttrs = !P.in_split && p->pipe_in ? 1 : 2;      // (programmatic launch, except right after an event wait)
-  e = cudaLaunchKernelEx(&cfg, dct2_tc_kernel, m0, m1, m2, moh, mol, P);
+  const dim3 grid((unsigned)(items < p->sm_count ? items : p->sm_count));
+  const cudaError_t e = !P.in_split && p->pipe_in
+      ? ff_launch_after_event(dct2_tc_kernel, grid, dim3(D2_THREADS), D2_SMEM, st, m0, m1, m2, moh, mol, P)
+      : ff_launch(dct2_tc_kernel, grid, dim3(D2_THREADS), D2_SMEM, st, m0, m1, m2, moh, mol, P);
   if (e != cudaSuccess) return e;
   p->launches += 1;
   return cudaSuccess;
@@ -717,22 +606,17 @@ cudaError_t ffk_dct2_init() {
 }
 
 // Which second axis the fused launch takes: the shorter of h and t (smaller planes), an even number of tiles.  It is
-// used only where one CTA holds the plane (W x n2 <= 1024 positions): on B200 the launch beats the separate passes by
-// 23% at T = 16, W = 64 and loses from two CTAs per plane on (the remote stores of phase 1 and their cluster-scope
-// release cost more than the saved DRAM round trip: whole layer, T = 32, W = 64: 13.27 against 12.67 ms with three
-// passes, two samples of 24 heads; T = 16, W = 128: 1.32 against 1.18 ms).
-constexpr int MAX_CLUSTER_USED = 1;
-
-bool ffk_dct2_supported(const FFDims& dm, int* axis2, int* cs) {
+// used only where one CTA holds the plane (W x n2 <= 1024 positions): there the launch beats the separate passes by 23%
+// (T = 16, W = 64).  With the plane spread over a cluster of two CTAs it lost to them (the remote stores of phase 1 and
+// their cluster-scope release cost more than the saved DRAM round trip: whole layer, T = 32, W = 64: 13.27 against 12.67
+// ms with three passes, two samples of 24 heads; T = 16, W = 128: 1.32 against 1.18 ms).
+bool ffk_dct2_supported(const FFDims& dm, int* axis2) {
   if (dm.fp32 || dm.d % CHK != 0 || (dm.d != 128 && dm.d != 64) || !axis_ok(dm.T) || !axis_ok(dm.H) || !axis_ok(dm.W)) return false;
   const int a2 = dm.T < dm.H ? 0 : 1;
   const int n2 = a2 == 1 ? dm.H : dm.T;
   const int tiles = dm.W * n2 / ROWS;
-  int c = 1;
-  while (tiles / c > MAX_TPC) c *= 2;
-  if (c > MAX_CLUSTER_USED || tiles % c != 0 || (tiles / c) % 2 != 0) return false;
+  if (tiles > MAX_TPC || tiles % 2 != 0) return false;
   if (axis2) *axis2 = a2;
-  if (cs) *cs = c;
   return true;
 }
 
@@ -769,8 +653,8 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
                              bool clear_energy, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int G = p->dct_group;
-  int axis2, cs;
-  if (!ffk_dct2_supported(dm, &axis2, &cs)) return cudaErrorInvalidValue;
+  int axis2;
+  if (!ffk_dct2_supported(dm, &axis2)) return cudaErrorInvalidValue;
   CUtensorMap mq, mk, mv, oh, ol;
   if (!in_map(p, &mq, Q, dm.BH, axis2) || !in_map(p, &mk, K, dm.BH, axis2) ||
       !in_map(p, &mv, V, dm.BH, axis2) || !out_map(p, &oh, out_hi, G, axis2) ||
@@ -783,7 +667,7 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
   P.axis2 = axis2; P.n1 = dm.W; P.n2 = axis2 == 1 ? dm.H : dm.T; P.n3 = axis2 == 1 ? dm.T : dm.H;
   P.clear = clear_energy ? p->buf.energy : nullptr;
   P.in_split = 0; P.last = 0; P.group = g; P.group_start = g0; P.nchunk = dm.d / CHK;
-  P.cs = cs; P.tpc = dm.W * P.n2 / ROWS / cs;
+  P.tpc = dm.W * P.n2 / ROWS;
   return launch(p, mq, mk, mv, oh, ol, P, st);
 }
 
@@ -791,8 +675,8 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
 cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, int h0, int g, void* out, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int G = p->dct_group;
-  int axis2, cs;
-  if (!ffk_dct2_supported(dm, &axis2, &cs)) return cudaErrorInvalidValue;
+  int axis2;
+  if (!ffk_dct2_supported(dm, &axis2)) return cudaErrorInvalidValue;
   CUtensorMap mh, ml, mo;
   if (!in_map(p, &mh, in_hi, G, axis2) || !in_map(p, &ml, in_lo, G, axis2) ||
       !out_map(p, &mo, out, dm.BH, axis2))
@@ -803,7 +687,7 @@ cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, i
   P.img1 = p->dct2_images + (size_t)(3 + 2) * per; P.img2 = p->dct2_images + (size_t)(3 + axis2) * per;
   P.axis2 = axis2; P.n1 = dm.W; P.n2 = axis2 == 1 ? dm.H : dm.T; P.n3 = axis2 == 1 ? dm.T : dm.H;
   P.in_split = 1; P.last = 1; P.group = g; P.group_start = h0; P.nchunk = dm.d / CHK;
-  P.cs = cs; P.tpc = dm.W * P.n2 / ROWS / cs;
+  P.tpc = dm.W * P.n2 / ROWS;
   return launch(p, mh, ml, ml, mo, mo, P, st);
 }
 

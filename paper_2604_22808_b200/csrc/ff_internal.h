@@ -220,7 +220,6 @@ struct ff_plan {
   FFMapCache maps;                             // tensor maps of the transform passes
   bool dct2_ok;                                // the fused two-axis launch covers this configuration
   int dct2_axis2;                              // its second axis (1 = h, 0 = t); the remaining axis gets a pass of its own
-  int dct2_clusters;                           // clusters of that launch the device runs at once (0 = not yet asked)
   alignas(64) unsigned char tmap_mid[128];     // CUtensorMap over the mid-band / high-band coefficient buffers
   alignas(64) unsigned char tmap_high[128];
   alignas(64) unsigned char tmap_low[128];     // ... over the pooled low band (bf16 copy), when low_tc_ok
@@ -272,7 +271,7 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
                                      cudaStream_t st);
 cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaStream_t st);
 // ---- two axis passes in one launch, intermediate in shared memory (ff_dct2_tc.cu) --------------------
-bool ffk_dct2_supported(const FFDims& dm, int* axis2, int* cs);
+bool ffk_dct2_supported(const FFDims& dm, int* axis2);
 bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat_host, int n);
 cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
                              bool clear_energy, cudaStream_t st);
