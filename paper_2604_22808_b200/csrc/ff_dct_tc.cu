@@ -59,6 +59,7 @@
 
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
+#include "ff_three_byte.cuh"
 
 using namespace sm100;
 
@@ -468,14 +469,12 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
           const bool lo8 = want_lo && P.out_lo8;
           uint32_t hi[16], lo[16];
           if (lo8) {
-            // three-byte form: the value rounded to 24 bits; hi = its upper 16 bits, lo = the next byte
 #pragma unroll
-            for (int i = 0; i < 32; ++i) r[i] += 0x80u;
+            for (int i = 0; i < 32; ++i) r[i] = ff_round24(r[i]);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) hi[i] = __byte_perm(r[2 * i], r[2 * i + 1], 0x7632);
+            for (int i = 0; i < 16; ++i) hi[i] = ff_hi2(r[2 * i], r[2 * i + 1]);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-              lo[i] = __byte_perm(__byte_perm(r[4 * i], r[4 * i + 1], 0x0051), __byte_perm(r[4 * i + 2], r[4 * i + 3], 0x0051), 0x5410);
+            for (int i = 0; i < 8; ++i) lo[i] = ff_lo4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
           } else {
 #pragma unroll
           for (int i = 0; i < 16; ++i) {

@@ -30,6 +30,7 @@
 
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
+#include "ff_three_byte.cuh"
 
 using namespace sm100;
 
@@ -375,6 +376,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         XPROF_T0(x10);
         tc_fence_after();
         const float2 s2 = make_float2(sh.inv[n & 3][row], sh.inv[n & 3][row]);
+        const uint32_t half = s2.x != s2.x ? 0u : FF_HALF24;   // (a NaN in a token or in a summary is in every score of the row)
 #pragma unroll 4
         for (int q = 0; q < XD / 32; ++q) {                // 32 channels
           uint32_t r[32];
@@ -394,15 +396,14 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
             for (int k = 0; k < 4; ++k) {
               const float2 d = make_float2(__uint_as_float(r[8 * v + 2 * k]), __uint_as_float(r[8 * v + 2 * k + 1]));
               const float2 w = __ffma2_rn(d, s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
-              u[2 * k] = __float_as_uint(w.x) + 0x80u;
-              u[2 * k + 1] = __float_as_uint(w.y) + 0x80u;
-              hi[k] = __byte_perm(u[2 * k], u[2 * k + 1], 0x7632);
+              u[2 * k] = __float_as_uint(w.x) + half;
+              u[2 * k + 1] = __float_as_uint(w.y) + half;
+              hi[k] = ff_hi2(u[2 * k], u[2 * k + 1]);
             }
             *(uint4*)(st + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
             // (lo: 32 bytes per row, 8-byte pieces XOR-swizzled with row / 4)
             *(uint2*)(st + 2048 + lane * 32 + ((v ^ ((lane >> 2) & 3)) << 3)) =
-                make_uint2(__byte_perm(__byte_perm(u[0], u[1], 0x0051), __byte_perm(u[2], u[3], 0x0051), 0x5410),
-                           __byte_perm(__byte_perm(u[4], u[5], 0x0051), __byte_perm(u[6], u[7], 0x0051), 0x5410));
+                make_uint2(ff_lo4(u[0], u[1], u[2], u[3]), ff_lo4(u[4], u[5], u[6], u[7]));
           }
           if (q == XD / 32 - 1) mbar_arrive(&sh.y_empty[slot]);
           __syncwarp();
@@ -466,22 +467,22 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         for (int i = 0; i < 4; ++i) {
           const float4 d0 = *(const float4*)(st_rd0 + i * 1024), d1 = *(const float4*)(st_rd1 + i * 1024);
           const float2 s2 = make_float2(inv[8 * i], inv[8 * i]);
+          const uint32_t half = s2.x != s2.x ? 0u : FF_HALF24;
           const float2 dd[4] = {make_float2(d0.x, d0.y), make_float2(d0.z, d0.w), make_float2(d1.x, d1.y), make_float2(d1.z, d1.w)};
           const uint32_t yw[4] = {yv[i].x, yv[i].y, yv[i].z, yv[i].w};
           uint32_t hi[4], u[8];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             const float2 v = __ffma2_rn(dd[k], s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
-            u[2 * k] = __float_as_uint(v.x) + 0x80u;
-            u[2 * k + 1] = __float_as_uint(v.y) + 0x80u;
-            hi[k] = __byte_perm(u[2 * k], u[2 * k + 1], 0x7632);
+            u[2 * k] = __float_as_uint(v.x) + half;
+            u[2 * k + 1] = __float_as_uint(v.y) + half;
+            hi[k] = ff_hi2(u[2 * k], u[2 * k + 1]);
           }
           if (q + 1 < XD / 32 && out[i] >= 0) yv[i] = __ldg((const uint4*)(yrow + 8 * i * XD + (q + 1) * 32));
           if (out[i] >= 0) {
             *(uint4*)(grid_hi + out[i] + q * 32) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
             *(uint2*)(grid_lo + out[i] + q * 32) =
-                make_uint2(__byte_perm(__byte_perm(u[0], u[1], 0x0051), __byte_perm(u[2], u[3], 0x0051), 0x5410),
-                           __byte_perm(__byte_perm(u[4], u[5], 0x0051), __byte_perm(u[6], u[7], 0x0051), 0x5410));
+                make_uint2(ff_lo4(u[0], u[1], u[2], u[3]), ff_lo4(u[4], u[5], u[6], u[7]));
           }
         }
         __syncwarp();

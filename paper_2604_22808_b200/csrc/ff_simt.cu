@@ -3,6 +3,7 @@
 // workloads; the bf16 workloads replace them with the tensor-core kernels where those apply.
 #include "ff_bands.cuh"
 #include "ff_internal.h"
+#include "ff_three_byte.cuh"
 #include "ff_worklist.cuh"
 
 namespace {
@@ -665,19 +666,17 @@ __global__ void __launch_bounds__(EXC_WARPS * 32, 2) exchange_recombine_kernel(F
         for (int i = 0; i < DPL; ++i) { acc[i].x /= den; acc[i].y /= den; acc[i].z /= den; acc[i].w /= den; }
     }
     if (f0 + (lane >> 3) >= N) continue;
-    // With a second grid (bf16 output) the value is stored in three bytes, rounded to 24 bits: its upper 16 bits
-    // in grid_out, the next 8 bits in the byte grid.  A band's tokens share almost the same exchange offset, so a
-    // single bf16 rounding would bias whole bands coherently and the inverse transform would focus that bias on a
-    // few tokens.
+    // With a second grid (bf16 output) the value is stored in three bytes.  A band's tokens share almost the same
+    // exchange offset, so a single bf16 rounding would bias whole bands coherently and the inverse transform would
+    // focus that bias on a few tokens.
     const size_t o = ((size_t)gi * N + f) * d + 4 * s;
 #pragma unroll
     for (int i = 0; i < DPL; ++i) {
       const float4 w = make_float4(y[i].x + acc[i].x, y[i].y + acc[i].y, y[i].z + acc[i].z, y[i].w + acc[i].w);
       if (grid_lo) {
-        const uint32_t u0 = __float_as_uint(w.x) + 0x80u, u1 = __float_as_uint(w.y) + 0x80u;
-        const uint32_t u2 = __float_as_uint(w.z) + 0x80u, u3 = __float_as_uint(w.w) + 0x80u;
-        *(uint2*)((uint16_t*)grid_out + o + 32 * i) = make_uint2(__byte_perm(u0, u1, 0x7632), __byte_perm(u2, u3, 0x7632));
-        *(uint32_t*)((uint8_t*)grid_lo + o + 32 * i) = __byte_perm(__byte_perm(u0, u1, 0x0051), __byte_perm(u2, u3, 0x0051), 0x5410);
+        const uint32_t u0 = ff_round24(w.x), u1 = ff_round24(w.y), u2 = ff_round24(w.z), u3 = ff_round24(w.w);
+        *(uint2*)((uint16_t*)grid_out + o + 32 * i) = make_uint2(ff_hi2(u0, u1), ff_hi2(u2, u3));
+        *(uint32_t*)((uint8_t*)grid_lo + o + 32 * i) = ff_lo4(u0, u1, u2, u3);
       } else {
         st4(grid_out + o + 32 * i, w);
       }

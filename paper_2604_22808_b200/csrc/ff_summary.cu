@@ -12,6 +12,7 @@
 // its own in front of the tensor-core kernel it cost 6 - 27 us of the step for microseconds of work.
 #include "ff_bands.cuh"
 #include "ff_internal.h"
+#include "ff_three_byte.cuh"
 
 namespace {
 
@@ -304,14 +305,14 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
       mx = nm;
     }
     const float inv = nkeys > 0 ? 1.f / den : 0.f;
-    // the value in three bytes (rounded to 24 bits: upper 16 bits and the next 8), at every rank the row stands for
+    // the value in three bytes, at every rank the row stands for
     uint2 hi[V]; uint32_t lo[V];
 #pragma unroll
     for (int i = 0; i < V; ++i) {
-      const uint32_t u0 = __float_as_uint(fmaf(acc[i].x, inv, y[i].x)) + 0x80u, u1 = __float_as_uint(fmaf(acc[i].y, inv, y[i].y)) + 0x80u;
-      const uint32_t u2 = __float_as_uint(fmaf(acc[i].z, inv, y[i].z)) + 0x80u, u3 = __float_as_uint(fmaf(acc[i].w, inv, y[i].w)) + 0x80u;
-      hi[i] = make_uint2(__byte_perm(u0, u1, 0x7632), __byte_perm(u2, u3, 0x7632));
-      lo[i] = __byte_perm(__byte_perm(u0, u1, 0x0051), __byte_perm(u2, u3, 0x0051), 0x5410);
+      const uint32_t u0 = ff_round24(fmaf(acc[i].x, inv, y[i].x)), u1 = ff_round24(fmaf(acc[i].y, inv, y[i].y));
+      const uint32_t u2 = ff_round24(fmaf(acc[i].z, inv, y[i].z)), u3 = ff_round24(fmaf(acc[i].w, inv, y[i].w));
+      hi[i] = make_uint2(ff_hi2(u0, u1), ff_hi2(u2, u3));
+      lo[i] = ff_lo4(u0, u1, u2, u3);
     }
     if (!live) continue;
     unsigned p = (unsigned)row * (unsigned)rep;
