@@ -141,9 +141,20 @@ def _f32(a) -> Optional[np.ndarray]:
     return None if a is None else np.ascontiguousarray(a, dtype=np.float32)
 
 
-def _floats(values):
-    """A host float array for the call (None stays None)."""
-    return None if values is None else (C.c_float * len(values))(*values)
+def _floats(values, count: int):
+    """A host float array for a call that reads `count` of them: a sequence of numbers, or one number (None stays None)."""
+    if values is None:
+        return None
+    if isinstance(values, np.ndarray):
+        values = values.ravel()
+    try:
+        out = (C.c_float * len(values))(*values)
+    except TypeError:                                    # a number, a nested sequence
+        flat = np.ascontiguousarray(values, dtype=np.float32).ravel()
+        out = (C.c_float * flat.size)(*flat)
+    if len(out) < count:
+        raise FFError(1, f"expected {count} timesteps (one per sample), got {len(out)}")
+    return out
 
 
 def _ptr(a: Optional[np.ndarray]):
@@ -216,32 +227,49 @@ class Plan:
             if t.device != device:
                 raise FFError(1, f"expected a tensor on {self.device}, got one on {t.device}")
 
+    def _check_masks(self, masks):
+        """The device pointer of a tensor of batch * heads band masks, one byte each (None stays None)."""
+        if masks is None:
+            return None
+        n = self.cfg.batch * self.cfg.heads
+        if masks.element_size() != 1 or masks.numel() < n or not masks.is_contiguous() or masks.device != self.device:
+            raise FFError(1, f"expected a contiguous uint8 tensor of {n} band masks on {self.device}")
+        return masks.data_ptr()
+
+    def _check_host(self, *tensors):
+        n = self._shape.numel() * self._dtype.itemsize
+        for t in tensors:
+            if t.numel() * t.element_size() < n or not t.is_contiguous():
+                raise FFError(1, f"expected a contiguous {self._dtype} tensor of shape {tuple(self._shape)}")
+
     # -- the path
     def route(self, Q, K, V, timesteps: Sequence[float], alloc_out=None, want_host: bool = True):
         self._check_io(Q, K, V)
-        ts = _floats(timesteps)
-        assert len(timesteps) == self.cfg.batch
+        ts = _floats(timesteps, self.cfg.batch)
+        assert len(ts) == self.cfg.batch
         alloc_h = np.zeros(self.cfg.batch * self.cfg.heads, np.uint8) if want_host else None
         pi_h = np.zeros((self.cfg.batch, 3), np.float32) if want_host else None
         _check(library().ff_route(self.handle, Q.data_ptr(), K.data_ptr(), V.data_ptr(), ts,
-                                  None if alloc_out is None else alloc_out.data_ptr(), _ptr(alloc_h), _ptr(pi_h),
+                                  self._check_masks(alloc_out), _ptr(alloc_h), _ptr(pi_h),
                                   self._stream()), self.handle)
         return alloc_h, pi_h
 
     def forward(self, Q, K, V, out, alloc=None, timesteps: Optional[Sequence[float]] = None):
         """alloc: uint8 CUDA tensor [batch*heads] of band masks, or None to route from timesteps."""
         self._check_io(Q, K, V, out)
-        ts = _floats(timesteps)
-        _check(library().ff_forward(self.handle, Q.data_ptr(), K.data_ptr(), V.data_ptr(),
-                                    None if alloc is None else alloc.data_ptr(), ts, out.data_ptr(),
-                                    self._stream()), self.handle)
+        ts = _floats(timesteps, self.cfg.batch)
+        _check(library().ff_forward(self.handle, Q.data_ptr(), K.data_ptr(), V.data_ptr(), self._check_masks(alloc), ts,
+                                    out.data_ptr(), self._stream()), self.handle)
         return out
 
     def forward_host(self, Qh, Kh, Vh, out_h, alloc_host: Optional[np.ndarray] = None,
                      timesteps: Optional[Sequence[float]] = None):
         """Host tensors (ideally pinned) in and out; the copies are part of the call."""
-        ts = _floats(timesteps)
+        self._check_host(Qh, Kh, Vh, out_h)
+        ts = _floats(timesteps, self.cfg.batch)
         al = None if alloc_host is None else np.ascontiguousarray(alloc_host, dtype=np.uint8)
+        if al is not None and al.size < self.cfg.batch * self.cfg.heads:
+            raise FFError(1, f"expected {self.cfg.batch * self.cfg.heads} band masks, got {al.size}")
         _check(library().ff_forward_host(self.handle, Qh.data_ptr(), Kh.data_ptr(), Vh.data_ptr(), _ptr(al), ts,
                                          out_h.data_ptr(), self._stream()), self.handle)
         return out_h
@@ -256,10 +284,9 @@ class Plan:
             if (tuple(t.shape) != shape or t.dtype != torch.bfloat16 or not t.is_contiguous() or not t.is_cuda
                     or t.device != self.device):
                 raise FFError(1, f"expected a contiguous bf16 tensor of shape {shape} on {self.device}")
-        ts = _floats(timesteps)
+        ts = _floats(timesteps, self.cfg.batch)
         _check(library().ff_forward_projected(self.handle, X.data_ptr(), Wqkv.data_ptr(), Wo.data_ptr(),
-                                              None if alloc is None else alloc.data_ptr(), ts, out.data_ptr(),
-                                              self._stream()), self.handle)
+                                              self._check_masks(alloc), ts, out.data_ptr(), self._stream()), self.handle)
         return out
 
     def device_status(self) -> int:
