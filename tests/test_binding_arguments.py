@@ -1,5 +1,7 @@
-"""The binding's own checks, on the CPU: what may stand for the timesteps, and that nothing shorter than what the library
-reads reaches it."""
+"""The binding's own checks, on the CPU: what may stand for the timesteps, that nothing shorter than what the library
+reads reaches it, and where the stream handle comes from."""
+from types import SimpleNamespace
+
 import numpy as np
 import pytest
 import torch
@@ -88,3 +90,10 @@ def test_short_arguments_of_the_projected_layer(plan):
         plan.forward_projected(*args, alloc=torch.zeros(1, dtype=torch.uint8))
     with pytest.raises(B.FFError, match="plan is NULL"):
         plan.forward_projected(*args, timesteps=[1.0, 2.0])
+
+
+def test_stream_handle_with_and_without_the_private_name():
+    public = SimpleNamespace(current_stream=lambda index: SimpleNamespace(cuda_stream=100 + index))
+    assert B._stream_getter(SimpleNamespace(_C=SimpleNamespace(), cuda=public))(3) == 103
+    private = SimpleNamespace(_cuda_getCurrentRawStream=lambda index: 200 + index)
+    assert B._stream_getter(SimpleNamespace(_C=private, cuda=public))(3) == 203
