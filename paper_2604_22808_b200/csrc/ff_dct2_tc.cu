@@ -583,9 +583,7 @@ cudaError_t launch(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, con
                    const CUtensorMap& mol, Dct2Params& P, cudaStream_t st) {
   const int items = P.group * P.n3 * P.nchunk;
   const dim3 grid((unsigned)(items < p->sm_count ? items : p->sm_count));
-  const cudaError_t e = !P.in_split && p->pipe_in
-      ? ff_launch_after_event(dct2_tc_kernel, grid, dim3(D2_THREADS), D2_SMEM, st, m0, m1, m2, moh, mol, P)
-      : ff_launch(dct2_tc_kernel, grid, dim3(D2_THREADS), D2_SMEM, st, m0, m1, m2, moh, mol, P);
+  const cudaError_t e = ff_launch(dct2_tc_kernel, grid, dim3(D2_THREADS), D2_SMEM, st, m0, m1, m2, moh, mol, P);
   if (e != cudaSuccess) return e;
   p->launches += 1;
   return cudaSuccess;

@@ -688,10 +688,7 @@ cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1
   const int tiles = P.group * P.g.tiles;
   const int grid = tiles < p->sm_count ? tiles : p->sm_count;
 #define FF_DCT(D, L, R)                                                                                                       \
-  e = P.mode == MODE_FIRST && p->pipe_in                                                                                       \
-          ? ff_launch_after_event(dct_tc_kernel<D, L, R>, dim3(grid), dim3(L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS), smem, st, \
-                                  m0, m1, m2, moh, mol, P)                                                                     \
-          : ff_launch(dct_tc_kernel<D, L, R>, dim3(grid), dim3(L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS), smem, st, m0, m1, m2, moh, mol, P)
+  e = ff_launch(dct_tc_kernel<D, L, R>, dim3(grid), dim3(L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS), smem, st, m0, m1, m2, moh, mol, P)
 #define FF_DCT_R(D, L) do { if (P.g.ragged) FF_DCT(D, L, true); else FF_DCT(D, L, false); } while (0)
   if (P.dm.d == 128) { if (in_lo8) FF_DCT_R(128, true); else FF_DCT_R(128, false); }
   else { if (in_lo8) FF_DCT_R(64, true); else FF_DCT_R(64, false); }

@@ -86,12 +86,7 @@ __device__ __forceinline__ void ff_pdl_wait() {
 __device__ __forceinline__ void ff_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void ff_pdl_join() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// (a launch right after an event wait goes without the attribute: ff_launch_after_event)
-template <class... K, class... A>
-inline cudaError_t ff_launch_after_event(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
-  kernel<<<grid, block, smem, st>>>(std::forward<A>(args)...);
-  return cudaGetLastError();
-}
+// (an event wait in the stream before the launch, the library's own or the caller's, holds the whole kernel back)
 template <class... K, class... A>
 inline cudaError_t ff_launch(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
