@@ -17,10 +17,10 @@
 // single bf16 rounding between passes would not meet the output tolerance.
 //
 // Three-byte intermediates.  Where the three axes run as separate passes, the pair written by the first forward
-// pass and the pairs between the inverse passes are stored as the fp32 value rounded to 24 bits: the upper 16
-// bits (a bf16 by truncation) in the hi grid and the next 8 bits in a byte grid.  hi and (value - hi) are both
-// exact bf16 operands, together they carry 16 significant bits like the bf16 hi/lo pair, and a pass moves 3
-// instead of 4 bytes per value.  A launch whose input has the byte form (template parameter LO8) runs four more
+// pass and the pairs between the inverse passes are stored (large planes, see pairs_between_passes) as the fp32 value
+// rounded to 24 bits: the upper 16 bits (a bf16 by truncation) in the hi grid and the next 8 bits in a byte grid.  hi
+// and (value - hi) are both exact bf16 operands, together they carry 16 significant bits, one less than a bf16 hi/lo
+// pair, and a pass moves 3 instead of 4 bytes per value.  A launch whose input has the byte form (template parameter LO8) runs four more
 // warps that expand the bytes of every arriving tile to the bf16 lo operand in shared memory before the MMAs
 // read it (128 channels: in place, the bytes of a row arrive inside the row's own bf16 space).  The expansion
 // competes with the epilogue for issue slots; measured per launch at 1M tokens (3 tensor-heads): a middle pass
@@ -752,6 +752,16 @@ Scratch carve(ff_plan* p) {
   s.b_hi = (__nv_bfloat16*)(base + 2 * grid_bytes); s.b_lo = (__nv_bfloat16*)(base + 3 * grid_bytes);
   return s;
 }
+// Form of the values between three separate passes.  The byte form is a rounding to 2^-17, a bf16 pair one to 2^-18: the
+// transform's error on N(0,1) input is 1.5 times that of pairs (low coefficients 9.6e-6 against 6.3e-6).  Planes of 2048
+// positions have pairs like the smaller ones, whose two axes share a launch (two samples of 32 x 64 x 64 tokens 13.50 ms,
+// with bytes 12.16).  Larger planes have bytes: 17.9 against 19.2 ms at 64 x 64 x 64, 40.0 against 43.0 at 64 x 128 x 128.
+bool pairs_between_passes(const ff_plan* p) {
+  auto ok = [](int n) { return n == 16 || n == 32 || n == 64 || n == 128; };
+  const FFDims& dm = p->dm;
+  const int plane = dm.W * (dm.T < dm.H ? dm.T : dm.H);
+  return ok(dm.T) && ok(dm.H) && ok(dm.W) && plane > 1024 && plane <= 2048;
+}
 }  // namespace
 
 cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy,
@@ -763,17 +773,17 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
   // along the remaining axis.  Kernel-select bit 4: the three axes as separate passes w, h, t.
   const bool fused = p->dct2_ok && !(p->attn_impl & 4);
   const int last_axis = fused ? (p->dct2_axis2 == 1 ? 0 : 1) : 0;
-  // Between the launches the hi/lo pair has the three-byte form (the lo grids hold bytes).
   // mXh/mXl: load maps of a pass's input pair; oXh/oXl: store maps of a pass's output pair (the box
   // follows the axis of the pass that uses the map)
-  const bool mid8 = false;        // (measured: the band-split pass is slower with a byte-form input)
+  const bool w8 = !pairs_between_passes(p);   // the first pass writes the byte form; the second one always a pair
+                                              // (measured: the band-split pass is slower with a byte-form input)
   CUtensorMap mq, mk, mv, m1h, m1l, m2h, m2l, o0h, o0l, o1h, o1l, m3h, m3l;
   if (fused ? !(grid_map(p, &m3h, sc.a_hi, G, last_axis) && grid_map(p, &m3l, sc.a_lo, G, last_axis))
             : !(grid_map(p, &mq, Q, dm.BH, 2) && grid_map(p, &mk, K, dm.BH, 2) && grid_map(p, &mv, V, dm.BH, 2) &&
-                store_map(p, &o0h, sc.a_hi, G, 2) && store_map(p, &o0l, sc.a_lo, G, 2, true) &&
-                grid_map(p, &m1h, sc.a_hi, G, 1) && grid_map(p, &m1l, sc.a_lo, G, 1, true) &&
-                store_map(p, &o1h, sc.b_hi, G, 1) && store_map(p, &o1l, sc.b_lo, G, 1, mid8) &&
-                grid_map(p, &m2h, sc.b_hi, G, 0) && grid_map(p, &m2l, sc.b_lo, G, 0, mid8)))
+                store_map(p, &o0h, sc.a_hi, G, 2) && store_map(p, &o0l, sc.a_lo, G, 2, w8) &&
+                grid_map(p, &m1h, sc.a_hi, G, 1) && grid_map(p, &m1l, sc.a_lo, G, 1, w8) &&
+                store_map(p, &o1h, sc.b_hi, G, 1) && store_map(p, &o1l, sc.b_lo, G, 1) &&
+                grid_map(p, &m2h, sc.b_hi, G, 0) && grid_map(p, &m2l, sc.b_lo, G, 0)))
     return cudaErrorInvalidValue;
   const int total = 3 * dm.BH;
   DctTcParams P{};
@@ -799,16 +809,16 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
       continue;
     }
     P.clear = want_energy && g0 == 0 ? p->buf.energy : nullptr;
-    P.mode = MODE_FIRST; P.in_split = 0; P.out_lo8 = 1; P.reverse = 0; P.axis = 2; P.image = matrix_image(p, 2, 0);
+    P.mode = MODE_FIRST; P.in_split = 0; P.out_lo8 = w8 ? 1 : 0; P.reverse = 0; P.axis = 2; P.image = matrix_image(p, 2, 0);
     e = launch_pass(p, mq, mk, mv, o0h, o0l, P, false, st);
     if (e != cudaSuccess) return e;
     P.clear = nullptr;
-    P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = mid8 ? 1 : 0; P.reverse = 1; P.axis = 1; P.image = matrix_image(p, 1, 0);
-    e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, true, st);
+    P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = 0; P.reverse = 1; P.axis = 1; P.image = matrix_image(p, 1, 0);
+    e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, w8, st);
     if (e != cudaSuccess) return e;
     P.in_split = 1; P.out_lo8 = 0; P.reverse = 0;
     P.mode = MODE_SPLIT; P.axis = 0; P.image = matrix_image(p, 0, 0);
-    e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, mid8, st);    // (no tensor stores in this mode)
+    e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, false, st);    // (no tensor stores in this mode)
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -822,17 +832,15 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
   const Scratch sc = carve(p);
   const bool fused = p->dct2_ok && !(p->attn_impl & 4);
   const int first_axis = fused ? (p->dct2_axis2 == 1 ? 0 : 1) : 0;       // the axis the fused launch leaves out
-  // The first pass reads the exchange's output, which has the three-byte form.  With three passes the pairs
-  // between them have it too; the fused launch takes a bf16 pair.
-  const bool b8 = !fused;
-  const bool inv8 = true;
+  // The first pass reads the exchange's output, which has the three-byte form.
+  const bool b8 = !fused && !pairs_between_passes(p);                    // what the passes hand on has it too
   CUtensorMap m_in, m_inl, mbh, mbl, mah, mal, obh, obl, oah, oal, mout;
   if (!grid_map(p, &m_in, sc.a_hi, G, first_axis) || !grid_map(p, &m_inl, sc.a_lo, G, first_axis, true) ||
       !store_map(p, &obh, sc.b_hi, G, first_axis) || !store_map(p, &obl, sc.b_lo, G, first_axis, b8))
     return cudaErrorInvalidValue;
-  if (!fused && (!grid_map(p, &mbh, sc.b_hi, G, 1) || !grid_map(p, &mbl, sc.b_lo, G, 1, true) ||
-                 !store_map(p, &oah, sc.a_hi, G, 1) || !store_map(p, &oal, sc.a_lo, G, 1, inv8) ||
-                 !grid_map(p, &mah, sc.a_hi, G, 2) || !grid_map(p, &mal, sc.a_lo, G, 2, inv8) ||
+  if (!fused && (!grid_map(p, &mbh, sc.b_hi, G, 1) || !grid_map(p, &mbl, sc.b_lo, G, 1, b8) ||
+                 !store_map(p, &oah, sc.a_hi, G, 1) || !store_map(p, &oal, sc.a_lo, G, 1, b8) ||
+                 !grid_map(p, &mah, sc.a_hi, G, 2) || !grid_map(p, &mal, sc.a_lo, G, 2, b8) ||
                  !store_map(p, &mout, out, dm.BH, 2)))
     return cudaErrorInvalidValue;
   DctTcParams P{};
@@ -842,9 +850,9 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
   cudaError_t e = launch_pass(p, m_in, m_inl, m_inl, obh, obl, P, true, st);
   if (e != cudaSuccess) return e;
   if (fused) return ffk_dct2_inverse(p, sc.b_hi, sc.b_lo, h0, g, out, st);
-  P.in_split = 1; P.out_lo8 = inv8 ? 1 : 0; P.reverse = 0; P.axis = 1; P.image = matrix_image(p, 1, 1);
-  e = launch_pass(p, mbh, mbl, mbl, oah, oal, P, true, st);
+  P.in_split = 1; P.reverse = 0; P.axis = 1; P.image = matrix_image(p, 1, 1);
+  e = launch_pass(p, mbh, mbl, mbl, oah, oal, P, b8, st);
   if (e != cudaSuccess) return e;
   P.mode = MODE_LAST; P.out_lo8 = 0; P.reverse = 1; P.axis = 2; P.image = matrix_image(p, 2, 1);
-  return launch_pass(p, mah, mal, mal, mout, mout, P, inv8, st);
+  return launch_pass(p, mah, mal, mal, mout, mout, P, b8, st);
 }
