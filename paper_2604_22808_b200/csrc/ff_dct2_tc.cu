@@ -202,7 +202,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
 #pragma unroll 1
     for (int im = 0; im < 4; ++im) {
-      const uint32_t* src = (im < 2 ? P.img1 : P.img2) + (size_t)(im & 1) * ROWS * IMG_CELLS + (size_t)row * IMG_CELLS;
+      const uint32_t* src = (im < 2 ? P.img1 : P.img2) + (size_t)(im & 1) * FF_IMAGE_PART + (size_t)row * IMG_CELLS;
 #pragma unroll
       for (int c0 = 0; c0 < IMG_CELLS; c0 += 32) {
         uint32_t r[32];
@@ -577,8 +577,6 @@ bool encode_out_map(CUtensorMap* map, const void* base, const FFDims& dm, int sl
 // (the staging areas of the tensor stores sit 1024-byte aligned: their 64-byte swizzle is a function of the address)
 constexpr size_t D2_SMEM = 1024 + (size_t)MAX_TPC * 2 * TILE_B + (size_t)8 * 2 * 32 * STG_ROW + (size_t)RING_B + sizeof(D2Shared) + 64;
 
-bool axis_ok(int n) { return n == 16 || n == 32 || n == 64 || n == 128; }
-
 cudaError_t launch(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, const CUtensorMap& m2, const CUtensorMap& moh,
                    const CUtensorMap& mol, Dct2Params& P, cudaStream_t st) {
   const int items = P.group * P.n3 * P.nchunk;
@@ -591,10 +589,10 @@ cudaError_t launch(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, con
 
 // (through the plan's cache)
 bool in_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis2) {
-  return p->maps.get(map, base, 16 | axis2, slices, [&] { return encode_in_map(map, base, p->dm, slices, axis2); });
+  return p->maps.get(map, base, 32 | axis2, slices, [&] { return encode_in_map(map, base, p->dm, slices, axis2); });
 }
 bool out_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis2) {
-  return p->maps.get(map, base, 24 | axis2, slices, [&] { return encode_out_map(map, base, p->dm, slices, axis2); });
+  return p->maps.get(map, base, 40 | axis2, slices, [&] { return encode_out_map(map, base, p->dm, slices, axis2); });
 }
 
 }  // namespace
@@ -609,7 +607,7 @@ cudaError_t ffk_dct2_init() {
 // their cluster-scope release cost more than the saved DRAM round trip: whole layer, T = 32, W = 64: 13.27 against 12.67
 // ms with three passes, two samples of 24 heads; T = 16, W = 128: 1.32 against 1.18 ms).
 bool ffk_dct2_supported(const FFDims& dm, int* axis2) {
-  if (dm.fp32 || dm.d % CHK != 0 || (dm.d != 128 && dm.d != 64) || !axis_ok(dm.T) || !axis_ok(dm.H) || !axis_ok(dm.W)) return false;
+  if (dm.fp32 || dm.d % CHK != 0 || (dm.d != 128 && dm.d != 64) || ff_fp32_grid(dm)) return false;
   const int a2 = dm.T < dm.H ? 0 : 1;
   const int n2 = a2 == 1 ? dm.H : dm.T;
   const int tiles = dm.W * n2 / ROWS;
@@ -619,12 +617,13 @@ bool ffk_dct2_supported(const FFDims& dm, int* axis2) {
 }
 
 // Matrix image of one axis and direction as the tensor-memory A operand: row j = output position
-// of a tile, cell c = the bf16 pair (A[j][2c], A[j][2c+1]); hi part [128][64], then lo part.
+// of a tile, cell c = the bf16 pair (A[j][2c], A[j][2c+1]); three parts [128][64], each the bf16 next to what the parts
+// before it leave.
 // w axis: lines follow one another, A = I kron Mat (index = line*n + a); h, t: A = Mat kron I
 // (index = a*kf + line); rows and columns past the tile's kf*n positions are zero.  `mat` is the host matrix
 // [n][n], out[a] = sum_b mat[a][b] in[b].
 bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat, int n) {
-  const size_t per = (size_t)2 * ROWS * IMG_CELLS;      // cells of one image (hi + lo)
+  const size_t per = FF_IMAGE_CELLS;
   if (!p->dct2_images && cudaMalloc((void**)&p->dct2_images, 6 * per * sizeof(uint32_t)) != cudaSuccess) return false;
   const FFPassShape g = ff_pass_shape(p->dm, axis);
   const int kf = g.kf;
@@ -635,12 +634,13 @@ bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat, i
       float v;
       if (seq) v = (j / n == r / n) ? mat[(j % n) * n + (r % n)] : 0.f;
       else v = (j % kf == r % kf) ? mat[(j / kf) * n + (r / kf)] : 0.f;
-      const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-      const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-      const uint32_t hb = *(const uint16_t*)&hi, lb = *(const uint16_t*)&lo;
-      const size_t cell = (size_t)j * IMG_CELLS + (r >> 1);
-      if (r & 1) { img[cell] |= hb << 16; img[(size_t)ROWS * IMG_CELLS + cell] |= lb << 16; }
-      else { img[cell] = hb; img[(size_t)ROWS * IMG_CELLS + cell] = lb; }
+      size_t cell = (size_t)j * IMG_CELLS + (r >> 1);
+      for (int part = 0; part < 3; ++part, cell += FF_IMAGE_PART) {
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        const uint32_t hb = *(const uint16_t*)&h;
+        img[cell] |= (r & 1) ? hb << 16 : hb;
+        v -= __bfloat162float(h);
+      }
     }
   const int slot = (inverse ? 3 : 0) + axis;
   return cudaMemcpy(p->dct2_images + slot * per, img.data(), per * sizeof(uint32_t), cudaMemcpyHostToDevice) == cudaSuccess;
@@ -658,7 +658,7 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
       !in_map(p, &mv, V, dm.BH, axis2) || !out_map(p, &oh, out_hi, G, axis2) ||
       !out_map(p, &ol, out_lo, G, axis2))
     return cudaErrorInvalidValue;
-  const size_t per = (size_t)2 * ROWS * IMG_CELLS;
+  const size_t per = FF_IMAGE_CELLS;
   Dct2Params P{};
   P.dm = dm; P.status = p->buf.status;
   P.img1 = p->dct2_images + (size_t)(0 + 2) * per; P.img2 = p->dct2_images + (size_t)(0 + axis2) * per;
@@ -679,7 +679,7 @@ cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, i
   if (!in_map(p, &mh, in_hi, G, axis2) || !in_map(p, &ml, in_lo, G, axis2) ||
       !out_map(p, &mo, out, dm.BH, axis2))
     return cudaErrorInvalidValue;
-  const size_t per = (size_t)2 * ROWS * IMG_CELLS;
+  const size_t per = FF_IMAGE_CELLS;
   Dct2Params P{};
   P.dm = dm; P.status = p->buf.status;
   P.img1 = p->dct2_images + (size_t)(3 + 2) * per; P.img2 = p->dct2_images + (size_t)(3 + axis2) * per;

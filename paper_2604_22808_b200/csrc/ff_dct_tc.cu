@@ -28,11 +28,16 @@
 // pass 0.38 -> 0.42 ms with byte-form input.  So the band-split pass always reads a bf16 pair (the second
 // forward pass writes one), and the fused two-axis launches keep bf16 pairs on both sides.
 //
-// Ragged grids.  A line of any length up to 128 fits a tile, so the passes run on every grid: floor(128 / n) lines
+// Any grid.  A line of any length up to 128 fits a tile, so the passes run on every grid: floor(128 / n) lines
 // per tile, the left-over rows zero in the matrix and in shared memory, partial last tiles filled with zeros and
-// clipped by the copies (template parameter RAG).  21 x 45 x 80 tokens, 16 heads: forward transform 11.1 -> 1.63 ms
-// and inverse 5.8 -> 0.78 ms against the fp32 kernels these grids ran on before (the same 6.5 TB/s-bound traffic
-// per token as a power-of-two grid plus 6 - 37% of unused tile rows).
+// clipped by the copies.  Grids with an axis other than 16, 32, 64 or 128 ran on fp32 kernels, and the precision stays
+// that of fp32 numbers: the passes hand on fp32 grids (forms EXACT1 and EXACT), matrix and data are three bf16 parts
+// each, which hold all 24 bits, and six of their nine products are summed, the small ones first (the others are below
+// 2^-24).  The parts of the data are made by the four warps that expand bytes in form BYTES: truncations, so that they
+// add up to the value.  A pass moves 4 bytes per value like a bf16 pair, and 48 instructions a tile keep the tensor core
+// below the copies' time.  21 x 45 x 80 tokens, 16 heads: forward transform 1.94 ms and inverse with the exchange 0.94
+// (fp32 kernels: 4.46 and 2.83; 16-bit intermediates: 1.54 and 0.67); the passes run at 4.1 - 5.9 TB/s, the later ones
+// below the first because two stages of 96 KB are all that fit.
 //
 // Order of the tiles.  A pass that reads what the previous launch wrote walks its tiles from the last to the
 // first (P.reverse), the next one forward again: the end of the previous launch's output is still in L2.
@@ -79,17 +84,31 @@ __device__ unsigned long long g_dct_prof[128];
 #define PROF_T0(v)
 #define PROF_ADD(i, v)
 #endif
-constexpr int NACC = 3;                     // accumulator buffers of 128 tensor-memory columns, behind the matrix (128 columns)
+constexpr int NACC_MAX = 3;
 constexpr int IMG_CELLS = 64;               // 32-bit tensor-memory cells per matrix row: two bf16 K elements each
-constexpr uint32_t COL_IMG_HI = 0, COL_IMG_LO = 64, COL_ACC = 128;
-constexpr int DCT_TC_THREADS = 320;        // TMA warp, MMA warp, 8 epilogue warps
-constexpr int DCT_TC_THREADS_LO8 = 448;    // ... and 4 warps that expand a one-byte lo part to the bf16 operand
+
+// What a pass reads and, with it, the parts of its operands.
+enum {
+  FORM_PAIR,      // bf16: the caller's tensor, or a hi/lo pair of grids
+  FORM_BYTES,     // a pair in the three-byte form
+  FORM_EXACT1,    // any grid: the caller's bf16 tensor, handed on as fp32
+  FORM_EXACT      // any grid: an fp32 grid
+};
+template <int FORM> struct Shape {
+  static constexpr bool any_grid = FORM >= FORM_EXACT1;
+  static constexpr bool convert = FORM == FORM_BYTES || FORM == FORM_EXACT;
+  static constexpr int threads = convert ? 448 : 320;      // TMA warp, MMA warp, 8 epilogue warps; 4 that make operands of the data
+  static constexpr int parts = any_grid ? 3 : 2;           // of the matrix, 64 tensor-memory columns each
+  static constexpr uint32_t col_acc = parts * 64;          // accumulator buffers of 128 columns behind them
+  static constexpr int nacc = any_grid ? 2 : NACC_MAX;
+  static_assert(col_acc + nacc * 128 <= 512, "tensor memory has 512 columns");
+};
 
 enum { MODE_FIRST = 0, MODE_MIDDLE = 1, MODE_SPLIT = 2, MODE_LAST = 3 };
 
 struct DctTcParams {
   FFDims dm;
-  const uint32_t* image;   // matrix image as the tensor-memory A operand: hi [128][64] cells, then lo
+  const uint32_t* image;   // matrix image as the tensor-memory A operand: parts of [128][64] cells
   FFPassShape g;           // lines and tiles of the pass
   FFFastDiv by_tiles, by_inner;   // tiles of a tensor-head; tiles along the inner extent
   FFFastDiv by_line;       // (SPLIT) unravels a line index: by W for the t axis, by H for the w axis
@@ -111,8 +130,8 @@ struct DctTcParams {
 constexpr int STG_PITCH = 64;                       // bytes per staged row piece; the 16-byte chunks are rotated by row/2 against bank conflicts
 
 struct DctShared {
-  uint64_t full[MAX_STAGE], empty[MAX_STAGE], acc_full[NACC], acc_empty[NACC], conv[MAX_STAGE];
-  uint64_t stg_full[2], stg_free[2];       // (ragged tiles) staging area of four epilogue warps: written / read by its store
+  uint64_t full[MAX_STAGE], empty[MAX_STAGE], acc_full[NACC_MAX], acc_empty[NACC_MAX], conv[MAX_STAGE];
+  uint64_t stg_full[2], stg_free[2];       // (any grid) staging area of four epilogue warps: written / read by its store
   uint32_t tmem_base;
   int abort_flag;
   int e_sample;            // (SPLIT) sample of the CTA's last tile
@@ -145,30 +164,38 @@ __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.comm
 __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
+__device__ __forceinline__ uint32_t bf16_pair(uint32_t a, uint32_t b) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(__uint_as_float(a), __uint_as_float(b));
+  return *(const uint32_t*)&v;
+}
+
 // Three source maps (Q, K, V) in MODE_FIRST; otherwise map0 (= hi) and, for split input, map1 (= lo).
 // map_oh / map_ol: destination hi / lo grids with the box of one epilogue warp (32 positions x 32
-// channels), all modes but SPLIT; MODE_LAST has no lo grid.
-// RAG: tiles of kf * n < 128 rows, or a last tile that is not full.  The rows past kf * n are zero in shared memory
-// (cleared once, no copy writes them) and zero in the matrix; lines past the end of the grid arrive as zeros and
+// channels), all modes but SPLIT; MODE_LAST and the EXACT forms have no lo grid.
+// RAG (any grid): tiles of kf * n < 128 rows, or a last tile that is not full.  The rows past kf * n are zero in shared
+// memory (cleared once, no copy writes them) and zero in the matrix; lines past the end of the grid arrive as zeros and
 // are clipped by the stores.  32 rows are then no box of the grid, so the four warps of a channel half stage a
 // whole tile (32 channels) and one thread stores it.
-template <int CH, bool LO8, bool RAG>
-__global__ void __launch_bounds__(LO8 ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS, 1)
+template <int CH, int FORM>
+__global__ void __launch_bounds__(Shape<FORM>::threads, 1)
 dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
               const __grid_constant__ CUtensorMap map2, const __grid_constant__ CUtensorMap map_oh,
               const __grid_constant__ CUtensorMap map_ol, const DctTcParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  constexpr bool LO8 = FORM == FORM_BYTES, F32 = FORM == FORM_EXACT, RAG = Shape<FORM>::any_grid, CONVERT = Shape<FORM>::convert;
+  constexpr int NACC = Shape<FORM>::nacc, THREADS = Shape<FORM>::threads;
+  constexpr uint32_t COL_ACC = Shape<FORM>::col_acc;
   const FFDims& dm = P.dm;
   const int n = P.g.n, kf = P.g.kf;                       // axis length, lines per tile
   const bool seq = P.g.seq;                               // lines follow one another (w axis) or interleave
   const int rows = RAG ? P.g.rows : TILE_ROWS;
   const int NSTAGE = P.nstage;
-  const bool split = !LO8 && P.mode == MODE_SPLIT;        // (the band-split pass never reads the byte form)
+  const bool split = !LO8 && FORM != FORM_EXACT1 && P.mode == MODE_SPLIT;     // (the band-split pass never reads the byte form)
   const bool tma_out = !split;
   constexpr int TB = TILE_ROWS * CH * 2;                  // bytes of one data tile (16 KB for 64 channels)
   constexpr int LO8_OFF = CH == 128 ? TB : 2 * TB;         // where a stage takes the lo bytes
-  const int STAGE_BYTES = LO8 ? LO8_OFF + TB / 2 + (CH == 128 ? TB / 2 : 0) : (P.in_split ? 2 * TB : TB);   // hi tile, lo tile
+  const int STAGE_BYTES = LO8 ? LO8_OFF + TB / 2 + (CH == 128 ? TB / 2 : 0) : (F32 ? 3 * TB : (P.in_split ? 2 * TB : TB));   // hi tile, lo tile
   uint8_t* sData = smem;                                  // NSTAGE x STAGE_BYTES
   DctShared& sh = *(DctShared*)(smem + NSTAGE * STAGE_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -194,13 +221,13 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
   volatile int* abort_flag = &sh.abort_flag;
 
   if (warp >= 2 && warp < 6) {
-    // The matrix (hi and lo bf16 parts) into tensor memory, where it is the A operand of every tile: a thread
+    // The matrix (its bf16 parts) into tensor memory, where it is the A operand of every tile: a thread
     // loads the row of its lane (prepared at plan creation as pairs of bf16 K elements per 32-bit cell).
     const int quarter = warp & 3, row = quarter * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
 #pragma unroll 1
-    for (int im = 0; im < 2; ++im) {
-      const uint32_t* src = P.image + (size_t)im * TILE_ROWS * IMG_CELLS + (size_t)row * IMG_CELLS;
+    for (int im = 0; im < Shape<FORM>::parts; ++im) {
+      const uint32_t* src = P.image + (size_t)im * FF_IMAGE_PART + (size_t)row * IMG_CELLS;
 #pragma unroll
       for (int c0 = 0; c0 < IMG_CELLS; c0 += 32) {
         uint32_t r[32];
@@ -215,7 +242,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     tmem_wait_st();
   }
   ff_pdl_wait();
-  if (!LO8 && P.clear && blockIdx.x == 0) for (int i = threadIdx.x; i < dm.B * 3 * CH; i += DCT_TC_THREADS) P.clear[i] = 0.0;
+  if (!CONVERT && P.clear && blockIdx.x == 0) for (int i = threadIdx.x; i < dm.B * 3 * CH; i += THREADS) P.clear[i] = 0.0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -243,7 +270,12 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
           map = tensor == 0 ? &map0 : (tensor == 1 ? &map1 : &map2);
           slice = th - tensor * dm.BH;
         }
-        mbar_arrive_expect_tx(&sh.full[slot], (uint32_t)(rows * CH) * (LO8 ? 3u : (P.in_split ? 4u : 2u)));
+        mbar_arrive_expect_tx(&sh.full[slot], (uint32_t)(rows * CH) * (LO8 ? 3u : (F32 || P.in_split ? 4u : 2u)));
+        if (F32) {                                         // blocks of 32 channels: rows of 128 bytes
+#pragma unroll
+          for (int b = 0; b < CH / 32; ++b) tma_load_5d(dst + b * HALF_BYTES, map, &sh.full[slot], 32 * b, i0, 0, o0, slice);
+          continue;
+        }
         tma_load_5d(dst, map, &sh.full[slot], 0, i0, 0, o0, slice);
         if (CH == 128) tma_load_5d(dst + HALF_BYTES, map, &sh.full[slot], 64, i0, 0, o0, slice);
         if (LO8) {
@@ -262,7 +294,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
         const int slot = it % NSTAGE, ab = it % NACC;
         PROF_T0(pm);
-        ok = mbar_wait_warp(LO8 ? &sh.conv[slot] : &sh.full[slot], (it / NSTAGE) & 1, abort_flag);
+        ok = mbar_wait_warp(CONVERT ? &sh.conv[slot] : &sh.full[slot], (it / NSTAGE) & 1, abort_flag);
         PROF_ADD(2, pm);
         PROF_T0(pm2);
         if (ok && it >= NACC) ok = mbar_wait_warp(&sh.acc_empty[ab], ((it / NACC) - 1) & 1, abort_flag);
@@ -271,19 +303,88 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
         tc_fence_after();
         const uint32_t dbase = smem_u32(sData + slot * STAGE_BYTES);
         const uint32_t d_tm = tm + COL_ACC + ab * 128;
-        const uint64_t xh0 = smem_desc_sw128(dbase, HALF_BYTES, 1024), xl0 = smem_desc_sw128(dbase + TB, HALF_BYTES, 1024);
         const int ksteps = (rows + 15) >> 4;               // (the rows behind them are zero)
+        // k-steps of matrix part `part` times the operand at `x` (a descriptor advances by 2048 bytes = 128 in its address
+        // field per 16 rows of K)
+        auto product = [&](int part, uint64_t x, bool first) {
 #pragma unroll
-        for (int ks = 0; ks < TILE_ROWS / 16; ++ks) {
-          if (RAG && ks >= ksteps) break;
-          // (a descriptor advances by 2048 bytes = 128 in its address field per 16 rows of K)
-          umma_ts(d_tm, tm + COL_IMG_HI + ks * 8, xh0 + (uint64_t)(ks * 128), idesc, ks > 0 ? 1u : 0u);
-          umma_ts(d_tm, tm + COL_IMG_LO + ks * 8, xh0 + (uint64_t)(ks * 128), idesc, 1u);
-          if (P.in_split) umma_ts(d_tm, tm + COL_IMG_HI + ks * 8, xl0 + (uint64_t)(ks * 128), idesc, 1u);
+          for (int ks = 0; ks < TILE_ROWS / 16; ++ks)
+            if (ks < ksteps) umma_ts(d_tm, tm + part * 64 + ks * 8, x + (uint64_t)(ks * 128), idesc, first && ks == 0 ? 0u : 1u);
+        };
+        if (F32) {
+          // (the halves of 64 channels of the first two parts alternate, those of the third follow one another)
+          const uint64_t x0 = smem_desc_sw128(dbase, 2 * HALF_BYTES, 1024), x1 = smem_desc_sw128(dbase + HALF_BYTES, 2 * HALF_BYTES, 1024);
+          const uint64_t x2 = smem_desc_sw128(dbase + 2 * TB, HALF_BYTES, 1024);
+          product(2, x0, true);
+          product(1, x1, false);
+          product(0, x2, false);
+          product(1, x0, false);
+          product(0, x1, false);
+          product(0, x0, false);
+        } else if (RAG) {
+          const uint64_t x = smem_desc_sw128(dbase, HALF_BYTES, 1024);
+          product(2, x, true);
+          product(1, x, false);
+          product(0, x, false);
+        } else {
+          const uint64_t xh0 = smem_desc_sw128(dbase, HALF_BYTES, 1024), xl0 = smem_desc_sw128(dbase + TB, HALF_BYTES, 1024);
+#pragma unroll
+          for (int ks = 0; ks < TILE_ROWS / 16; ++ks) {
+            umma_ts(d_tm, tm + ks * 8, xh0 + (uint64_t)(ks * 128), idesc, ks > 0 ? 1u : 0u);
+            umma_ts(d_tm, tm + 64 + ks * 8, xh0 + (uint64_t)(ks * 128), idesc, 1u);
+            if (P.in_split) umma_ts(d_tm, tm + ks * 8, xl0 + (uint64_t)(ks * 128), idesc, 1u);
+          }
         }
         umma_commit(&sh.empty[slot]);
         umma_commit(&sh.acc_full[ab]);
       }
+    }
+  } else if (F32 && warp >= 10) {
+    // ------------------------------------------------------------------ fp32 -> three bf16 parts, in place
+    // A thread owns a row of the tile.  64 channels at a time: they arrive in two blocks of 32 channels, the first and the
+    // second part go where they were (64 channels a block), the third part behind the tile; all with the 128-byte swizzle.
+    const int r0 = threadIdx.x - 320;
+    unsigned it = 0;
+    bool ok = true;
+    for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
+      const int slot = it % NSTAGE;
+      PROF_T0(pc0);
+      ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[slot], (it / NSTAGE) & 1, abort_flag));
+      if (threadIdx.x == 320) PROF_ADD(0, pc0);
+      if (!ok) break;
+      PROF_T0(pc1);
+      if (r0 < rows) {
+#pragma unroll 1
+        for (int h = 0; h < CH / 64; ++h) {
+          uint8_t* b0 = sData + slot * STAGE_BYTES + h * 2 * HALF_BYTES + r0 * 128;
+          uint8_t* b2 = sData + slot * STAGE_BYTES + 2 * TB + h * HALF_BYTES + r0 * 128;
+          uint4 x[16];                                     // four channels each
+#pragma unroll
+          for (int c = 0; c < 16; ++c) x[c] = *(const uint4*)(b0 + (c >> 3) * HALF_BYTES + (((c & 7) ^ (r0 & 7)) << 4));
+#pragma unroll
+          for (int c = 0; c < 8; ++c) {                    // eight channels: a 16-byte chunk of each part
+            const uint32_t v[8] = {x[2 * c].x, x[2 * c].y, x[2 * c].z, x[2 * c].w, x[2 * c + 1].x, x[2 * c + 1].y, x[2 * c + 1].z, x[2 * c + 1].w};
+            uint32_t p0[4], p1[4], p2[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const uint32_t va = v[2 * i], vb = v[2 * i + 1];
+              const uint32_t ra = __float_as_uint(__uint_as_float(va) - __uint_as_float(va & 0xffff0000u));
+              const uint32_t rb = __float_as_uint(__uint_as_float(vb) - __uint_as_float(vb & 0xffff0000u));
+              const float ta = __uint_as_float(ra) - __uint_as_float(ra & 0xffff0000u), tb = __uint_as_float(rb) - __uint_as_float(rb & 0xffff0000u);
+              p0[i] = __byte_perm(va, vb, 0x7632);
+              p1[i] = __byte_perm(ra, rb, 0x7632);
+              p2[i] = __byte_perm(__float_as_uint(ta), __float_as_uint(tb), 0x7632);
+            }
+            const uint32_t off = (uint32_t)((c ^ (r0 & 7)) << 4);
+            *(uint4*)(b0 + off) = make_uint4(p0[0], p0[1], p0[2], p0[3]);
+            *(uint4*)(b0 + HALF_BYTES + off) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
+            *(uint4*)(b2 + off) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
+          }
+        }
+      }
+      fence_proxy_async();
+      mbar_arrive(&sh.conv[slot]);
+      if (threadIdx.x == 320) PROF_ADD(1, pc1);
     }
   } else if (LO8 && warp >= 10) {
     // ------------------------------------------------------------------ lo bytes -> bf16 lo operand
@@ -350,7 +451,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     // rows are the box [32 channels] x [from there .. + the extents the store map was built with]
     const int j0 = quarter * 32;
     const int a0 = seq ? j0 % n : j0 / kf, l0 = seq ? j0 / n : j0 % kf;
-    unsigned nchunk = 0;                                  // (RAG) chunks this channel half has staged
+    unsigned nchunk = 0;                                  // (any grid) chunks this channel half has staged
     const int Lhw = dm.L[1] * dm.L[2], Mhw = dm.M[1] * dm.M[2];
     // (SPLIT) lane k of a warp accumulates the energies of channels 32 q + 2 (k % 16) + {0, 1} over the
     // warp's rows of parity k / 16: ea = mid + high rows, em = mid rows
@@ -464,8 +565,44 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
           for (int i = 0; i < 8; ++i)
             *(uint4*)(row_f32 + q * 32 + i * 4) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
         }
-        {
-          const bool want_lo = P.mode == MODE_FIRST || P.mode == MODE_MIDDLE;
+        if (RAG && tma_out) {
+          // four warps stage one tile, 32 channels of 128 rows: fp32 in rows of 128 bytes (128-byte swizzle), or the caller's
+          // bf16 in rows of 64 (64-byte swizzle).  (Two areas of half the size in turn: 3470 against 3300 us for the
+          // 76K-token layer.)
+          const int grp = ew >> 2;
+          uint8_t* area = sh.stage[grp * 4][0];
+          if (nchunk > 0) {
+            if (quarter == 0 && lane == 0) { bulk_wait_read0(); mbar_arrive(&sh.stg_free[grp]); }
+            ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_free[grp], (nchunk - 1) & 1, abort_flag));
+            if (!ok) break;
+          }
+          if (FORM == FORM_EXACT1 || P.mode == MODE_MIDDLE) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              *(uint4*)(area + j * 128 + ((i ^ (j & 7)) << 4)) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              uint32_t w[4];
+#pragma unroll
+              for (int k = 0; k < 4; ++k) w[k] = bf16_pair(r[8 * i + 2 * k], r[8 * i + 2 * k + 1]);
+              *(uint4*)(area + j * STG_PITCH + ((i ^ ((j >> 1) & 3)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+          }
+          fence_proxy_async();
+          mbar_arrive(&sh.stg_full[grp]);
+          if (quarter == 0) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_full[grp], nchunk & 1, abort_flag));
+            if (!ok) break;
+            if (lane == 0) {
+              tma_store_5d(area, &map_oh, q * 32, i0, 0, o0, out_slice);
+              bulk_commit();
+            }
+            __syncwarp();
+          }
+          ++nchunk;
+        } else {
+          const bool want_lo = !RAG && (P.mode == MODE_FIRST || P.mode == MODE_MIDDLE);
           const bool lo8 = want_lo && P.out_lo8;
           uint32_t hi[16], lo[16];
           if (lo8) {
@@ -477,10 +614,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
             for (int i = 0; i < 8; ++i) lo[i] = ff_lo4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
           } else {
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const __nv_bfloat162 hp = __floats2bfloat162_rn(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1]));
-            hi[i] = *(const uint32_t*)&hp;
-          }
+            for (int i = 0; i < 16; ++i) hi[i] = bf16_pair(r[2 * i], r[2 * i + 1]);
           }
           if (want_lo && !lo8) {
 #pragma unroll
@@ -490,17 +624,9 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
               lo[i] = *(const uint32_t*)&lp;
             }
           }
-          const bool tile_out = RAG && tma_out;          // four warps stage one tile: 128 rows of hi, then of lo
-          const int grp = ew >> 2;
-          uint8_t* st_hi = tile_out ? sh.stage[grp * 4][0] + quarter * 32 * STG_PITCH : sh.stage[ew][0];
-          uint8_t* st_lo = tile_out ? sh.stage[grp * 4][0] + TILE_ROWS * STG_PITCH + quarter * 32 * (lo8 ? 32 : STG_PITCH) : sh.stage[ew][1];
-          if (tile_out) {
-            if (nchunk > 0) {
-              if (quarter == 0 && lane == 0) { bulk_wait_read0(); mbar_arrive(&sh.stg_free[grp]); }
-              ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_free[grp], (nchunk - 1) & 1, abort_flag));
-              if (!ok) break;
-            }
-          } else if (tma_out) {
+          uint8_t* st_hi = sh.stage[ew][0];
+          uint8_t* st_lo = sh.stage[ew][1];
+          if (tma_out) {
             // the previous store of this warp must have read the staging area
             PROF_T0(pw);
             if (lane == 0) bulk_wait_read0();
@@ -518,21 +644,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
             *(uint4*)(st_lo + lane * 32) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
             *(uint4*)(st_lo + lane * 32 + 16) = make_uint4(lo[4], lo[5], lo[6], lo[7]);
           }
-          if (tile_out) {
-            fence_proxy_async();
-            mbar_arrive(&sh.stg_full[grp]);
-            if (quarter == 0) {
-              ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_full[grp], nchunk & 1, abort_flag));
-              if (!ok) break;
-              if (lane == 0) {
-                tma_store_5d(st_hi, &map_oh, q * 32, i0, 0, o0, out_slice);
-                if (want_lo) tma_store_5d(st_lo, &map_ol, q * 32, i0, 0, o0, out_slice);
-                bulk_commit();
-              }
-              __syncwarp();
-            }
-            ++nchunk;
-          } else if (tma_out) {
+          if (tma_out) {
             PROF_T0(pf);
             fence_proxy_async();
             __syncwarp();
@@ -633,66 +745,70 @@ EncodeTiledFn encoder() {
   return enc;
 }
 
-// 5-D map over a grid [slices][outer][n][inner][d] seen along `axis`.  Load map: the box is one tile, 64 channels of
-// kf whole lines.  Store map: 32 channels of what one epilogue warp holds (tile rows 32 q .. 32 q + 31), or of a
-// whole tile where the pass is ragged; 64-byte swizzle.  `bytes`: the grid holds one byte per value (the lo part
-// of the three-byte form); a load box then spans all channels of a row at once.
-bool encode_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, bool bytes, bool store) {
+enum { T_BF16, T_BYTE, T_F32 };
+// 5-D map over a grid [slices][outer][n][inner][d] seen along `axis`.  Load map: the box is one tile, kf whole lines of
+// 64 (bf16), 32 (fp32) or all channels (bytes: the lo part of the three-byte form), 128-byte rows but for the 64 bytes of
+// head_dim 64.  Store map: 32 channels of what one epilogue warp holds (tile rows 32 q .. 32 q + 31), or of a whole tile
+// where 32 rows are not a box of the grid.
+bool encode_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, int type, bool store) {
   EncodeTiledFn enc = encoder();
   if (!enc) return false;
   const FFPassShape g = ff_pass_shape(dm, axis);
-  const cuuint64_t CH = (cuuint64_t)dm.d, eb = bytes ? 1 : 2;
+  const cuuint64_t CH = (cuuint64_t)dm.d, eb = type == T_BYTE ? 1 : (type == T_BF16 ? 2 : 4);
   const cuuint64_t line = (cuuint64_t)g.inner * CH * eb;
   cuuint64_t dims[5] = {CH, (cuuint64_t)g.inner, (cuuint64_t)g.n, (cuuint64_t)g.outer, (cuuint64_t)slices};
   cuuint64_t strides[4] = {CH * eb, line, line * g.n, (cuuint64_t)dm.N * CH * eb};
-  cuuint32_t box[5] = {store ? 32u : (bytes ? (cuuint32_t)dm.d : 64u), (cuuint32_t)(g.seq ? 1 : g.kf), (cuuint32_t)g.n,
+  cuuint32_t box[5] = {store || type == T_F32 ? 32u : (type == T_BYTE ? (cuuint32_t)dm.d : 64u), (cuuint32_t)(g.seq ? 1 : g.kf), (cuuint32_t)g.n,
                        (cuuint32_t)(g.seq ? g.kf : 1), 1};
-  if (store && !g.ragged) {                // 32 consecutive tile rows
+  if (store && !ff_fp32_grid(dm)) {        // 32 consecutive tile rows
     if (g.seq) { box[2] = (cuuint32_t)(g.n < 32 ? g.n : 32); box[3] = (cuuint32_t)(g.n < 32 ? 32 / g.n : 1); }
     else { box[1] = (cuuint32_t)(g.kf < 32 ? g.kf : 32); box[2] = (cuuint32_t)(g.kf < 32 ? 32 / g.kf : 1); }
   }
   cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  const CUtensorMapSwizzle swz = store ? (bytes ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_64B)
-                                       : (bytes && dm.d == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B);
-  return enc(map, bytes ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims,
-             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
+  const cuuint32_t row = box[0] * (cuuint32_t)eb;      // bytes of a row in shared memory
+  const CUtensorMapSwizzle swz = row == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (row == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE);
+  return enc(map, type == T_BYTE ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : (type == T_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32),
+             5, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
              store ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 // (through the plan's cache)
-bool map_for(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, bool bytes, bool store) {
-  return p->maps.get(map, base, axis | (bytes ? 4 : 0) | (store ? 8 : 0), slices,
-                     [&] { return encode_map(map, base, p->dm, slices, axis, bytes, store); });
+bool map_for(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, int type, bool store) {
+  return p->maps.get(map, base, axis | (type << 2) | (store ? 16 : 0), slices,
+                     [&] { return encode_map(map, base, p->dm, slices, axis, type, store); });
 }
-bool grid_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, bool bytes = false) {
-  return map_for(p, map, base, slices, axis, bytes, false);
+bool grid_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, int type = T_BF16) {
+  return map_for(p, map, base, slices, axis, type, false);
 }
-bool store_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, bool bytes = false) {
-  return map_for(p, map, base, slices, axis, bytes, true);
+bool store_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, int type = T_BF16) {
+  return map_for(p, map, base, slices, axis, type, true);
 }
 
-// `in_lo8`: the input pair's lo grid is the byte form (m1 = its byte map).
+// `form`: what the pass reads.
 cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, const CUtensorMap& m2,
-                        const CUtensorMap& moh, const CUtensorMap& mol, DctTcParams& P, bool in_lo8, cudaStream_t st) {
+                        const CUtensorMap& moh, const CUtensorMap& mol, DctTcParams& P, int form, cudaStream_t st) {
   const size_t tile = (size_t)TILE_ROWS * P.dm.d * 2;
-  const size_t stage = in_lo8 ? (P.dm.d == 128 ? 2 * tile : 2 * tile + tile / 2) : (size_t)(P.in_split ? 2 : 1) * tile;
+  const size_t stage = form == FORM_EXACT ? 3 * tile : (form == FORM_BYTES ? (P.dm.d == 128 ? 2 * tile : 2 * tile + tile / 2) : (size_t)(P.in_split ? 2 : 1) * tile);
   const size_t fixed = sizeof(DctShared) + 1024;
   int nstage = (int)((232448 - 256 - fixed) / stage);   // 227 KB of shared memory per CTA
   if (nstage > MAX_STAGE) nstage = MAX_STAGE;
   P.nstage = nstage;
   const size_t smem = nstage * stage + fixed;
-  cudaError_t e = cudaSuccess;
   P.g = ff_pass_shape(P.dm, P.axis);
   P.by_tiles = ff_fast_div((unsigned)P.g.tiles); P.by_inner = ff_fast_div((unsigned)P.g.tiles_inner);
   P.by_line = ff_fast_div((unsigned)(P.axis == 2 ? P.dm.H : P.dm.W));
   const int tiles = P.group * P.g.tiles;
   const int grid = tiles < p->sm_count ? tiles : p->sm_count;
-#define FF_DCT(D, L, R)                                                                                                       \
-  e = ff_launch(dct_tc_kernel<D, L, R>, dim3(grid), dim3(L ? DCT_TC_THREADS_LO8 : DCT_TC_THREADS), smem, st, m0, m1, m2, moh, mol, P)
-#define FF_DCT_R(D, L) do { if (P.g.ragged) FF_DCT(D, L, true); else FF_DCT(D, L, false); } while (0)
-  if (P.dm.d == 128) { if (in_lo8) FF_DCT_R(128, true); else FF_DCT_R(128, false); }
-  else { if (in_lo8) FF_DCT_R(64, true); else FF_DCT_R(64, false); }
-#undef FF_DCT_R
+  cudaError_t e;
+#define FF_DCT(D, F) e = ff_launch(dct_tc_kernel<D, F>, dim3(grid), dim3(Shape<F>::threads), smem, st, m0, m1, m2, moh, mol, P)
+#define FF_DCT_D(F) do { if (P.dm.d == 128) FF_DCT(128, F); else FF_DCT(64, F); } while (0)
+  switch (form) {
+    case FORM_PAIR: FF_DCT_D(FORM_PAIR); break;
+    case FORM_BYTES: FF_DCT_D(FORM_BYTES); break;
+    case FORM_EXACT1: FF_DCT_D(FORM_EXACT1); break;
+    default: FF_DCT_D(FORM_EXACT);
+  }
+#undef FF_DCT_D
 #undef FF_DCT
   if (e != cudaSuccess) return e;
   p->launches += 1;
@@ -713,10 +829,10 @@ namespace {
 
 cudaError_t ffk_dct_tc_init() {
   cudaError_t e = cudaSuccess;
-#define FF_DCT(D, L, R) \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(dct_tc_kernel<D, L, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 256)
-  FF_DCT(128, false, false); FF_DCT(128, true, false); FF_DCT(128, false, true); FF_DCT(128, true, true);
-  FF_DCT(64, false, false); FF_DCT(64, true, false); FF_DCT(64, false, true); FF_DCT(64, true, true);
+#define FF_DCT(D, F) \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(dct_tc_kernel<D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 256)
+  FF_DCT(128, FORM_PAIR); FF_DCT(128, FORM_BYTES); FF_DCT(128, FORM_EXACT1); FF_DCT(128, FORM_EXACT);
+  FF_DCT(64, FORM_PAIR); FF_DCT(64, FORM_BYTES); FF_DCT(64, FORM_EXACT1); FF_DCT(64, FORM_EXACT);
 #undef FF_DCT
   return e;
 }
@@ -733,10 +849,10 @@ bool ffk_dct_tc_supported(const FFDims& dm) {
 // plan holds (built at plan creation by ffk_dct2_build_image: w lines follow one another, A = I kron Mat;
 // h and t lines interleave, A = Mat kron I).
 static const uint32_t* matrix_image(const ff_plan* p, int axis, int inverse) {
-  return p->dct2_images + (size_t)((inverse ? 3 : 0) + axis) * 2 * TILE_ROWS * IMG_CELLS;
+  return p->dct2_images + (size_t)((inverse ? 3 : 0) + axis) * FF_IMAGE_CELLS;
 }
 
-// Scratch: two hi/lo pairs of bf16 grids for `group` tensor-heads.
+// Scratch: two hi/lo pairs of bf16 grids for `group` tensor-heads, or two fp32 grids.
 size_t ffk_dct_tc_scratch_bytes(const FFDims& dm, int group) {
   const size_t grid = (size_t)group * dm.N * dm.d * 2;
   return 4 * ((grid + 255) / 256 * 256);
@@ -757,10 +873,8 @@ Scratch carve(ff_plan* p) {
 // positions have pairs like the smaller ones, whose two axes share a launch (two samples of 32 x 64 x 64 tokens 13.50 ms,
 // with bytes 12.16).  Larger planes have bytes: 17.9 against 19.2 ms at 64 x 64 x 64, 40.0 against 43.0 at 64 x 128 x 128.
 bool pairs_between_passes(const ff_plan* p) {
-  auto ok = [](int n) { return n == 16 || n == 32 || n == 64 || n == 128; };
-  const FFDims& dm = p->dm;
-  const int plane = dm.W * (dm.T < dm.H ? dm.T : dm.H);
-  return ok(dm.T) && ok(dm.H) && ok(dm.W) && plane > 1024 && plane <= 2048;
+  const int plane = p->dm.W * (p->dm.T < p->dm.H ? p->dm.T : p->dm.H);
+  return plane > 1024 && plane <= 2048;
 }
 }  // namespace
 
@@ -775,16 +889,21 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
   const int last_axis = fused ? (p->dct2_axis2 == 1 ? 0 : 1) : 0;
   // mXh/mXl: load maps of a pass's input pair; oXh/oXl: store maps of a pass's output pair (the box
   // follows the axis of the pass that uses the map)
+  const bool exact = ff_fp32_grid(dm);        // fp32 grids between the passes (in the place of a pair)
   const bool w8 = !pairs_between_passes(p);   // the first pass writes the byte form; the second one always a pair
                                               // (measured: the band-split pass is slower with a byte-form input)
   CUtensorMap mq, mk, mv, m1h, m1l, m2h, m2l, o0h, o0l, o1h, o1l, m3h, m3l;
-  if (fused ? !(grid_map(p, &m3h, sc.a_hi, G, last_axis) && grid_map(p, &m3l, sc.a_lo, G, last_axis))
-            : !(grid_map(p, &mq, Q, dm.BH, 2) && grid_map(p, &mk, K, dm.BH, 2) && grid_map(p, &mv, V, dm.BH, 2) &&
-                store_map(p, &o0h, sc.a_hi, G, 2) && store_map(p, &o0l, sc.a_lo, G, 2, w8) &&
-                grid_map(p, &m1h, sc.a_hi, G, 1) && grid_map(p, &m1l, sc.a_lo, G, 1, w8) &&
-                store_map(p, &o1h, sc.b_hi, G, 1) && store_map(p, &o1l, sc.b_lo, G, 1) &&
-                grid_map(p, &m2h, sc.b_hi, G, 0) && grid_map(p, &m2l, sc.b_lo, G, 0)))
+  const int lo = w8 ? T_BYTE : T_BF16;
+  if (!fused && !(grid_map(p, &mq, Q, dm.BH, 2) && grid_map(p, &mk, K, dm.BH, 2) && grid_map(p, &mv, V, dm.BH, 2))) return cudaErrorInvalidValue;
+  if (fused   ? !(grid_map(p, &m3h, sc.a_hi, G, last_axis) && grid_map(p, &m3l, sc.a_lo, G, last_axis))
+      : exact ? !(store_map(p, &o0h, sc.a_hi, G, 2, T_F32) && grid_map(p, &m1h, sc.a_hi, G, 1, T_F32) &&
+                  store_map(p, &o1h, sc.b_hi, G, 1, T_F32) && grid_map(p, &m2h, sc.b_hi, G, 0, T_F32))
+              : !(store_map(p, &o0h, sc.a_hi, G, 2) && store_map(p, &o0l, sc.a_lo, G, 2, lo) &&
+                  grid_map(p, &m1h, sc.a_hi, G, 1) && grid_map(p, &m1l, sc.a_lo, G, 1, lo) &&
+                  store_map(p, &o1h, sc.b_hi, G, 1) && store_map(p, &o1l, sc.b_lo, G, 1) &&
+                  grid_map(p, &m2h, sc.b_hi, G, 0) && grid_map(p, &m2l, sc.b_lo, G, 0)))
     return cudaErrorInvalidValue;
+  if (exact) { o0l = o0h; m1l = m1h; o1l = o1h; m2l = m2h; }     // (not used)
   const int total = 3 * dm.BH;
   DctTcParams P{};
   P.dm = dm; P.status = p->buf.status;
@@ -804,55 +923,57 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
       if (e != cudaSuccess) return e;
       P.in_split = 1; P.out_lo8 = 0; P.reverse = 1;
       P.mode = MODE_SPLIT; P.axis = last_axis; P.image = matrix_image(p, last_axis, 0);
-      e = launch_pass(p, m3h, m3l, m3l, m3h, m3l, P, false, st);    // (no tensor stores in this mode)
+      e = launch_pass(p, m3h, m3l, m3l, m3h, m3l, P, FORM_PAIR, st);    // (no tensor stores in this mode)
       if (e != cudaSuccess) return e;
       continue;
     }
     P.clear = want_energy && g0 == 0 ? p->buf.energy : nullptr;
     P.mode = MODE_FIRST; P.in_split = 0; P.out_lo8 = w8 ? 1 : 0; P.reverse = 0; P.axis = 2; P.image = matrix_image(p, 2, 0);
-    e = launch_pass(p, mq, mk, mv, o0h, o0l, P, false, st);
+    e = launch_pass(p, mq, mk, mv, o0h, o0l, P, exact ? FORM_EXACT1 : FORM_PAIR, st);
     if (e != cudaSuccess) return e;
     P.clear = nullptr;
     P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = 0; P.reverse = 1; P.axis = 1; P.image = matrix_image(p, 1, 0);
-    e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, w8, st);
+    e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, exact ? FORM_EXACT : (w8 ? FORM_BYTES : FORM_PAIR), st);
     if (e != cudaSuccess) return e;
     P.in_split = 1; P.out_lo8 = 0; P.reverse = 0;
     P.mode = MODE_SPLIT; P.axis = 0; P.image = matrix_image(p, 0, 0);
-    e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, false, st);    // (no tensor stores in this mode)
+    e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, exact ? FORM_EXACT : FORM_PAIR, st);    // (no tensor stores in this mode)
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-// Inverse transform of `g` recombined grids (three-byte form in the first scratch pair, written by the
-// exchange) into out[h0 .. h0+g).
+// Inverse transform of `g` recombined grids (in the first scratch pair, written by the exchange: three-byte form or
+// fp32) into out[h0 .. h0+g).
 cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int G = p->dct_group;
   const Scratch sc = carve(p);
-  const bool fused = p->dct2_ok && !(p->attn_impl & 4);
+  const bool fused = p->dct2_ok && !(p->attn_impl & 4), exact = ff_fp32_grid(dm);
   const int first_axis = fused ? (p->dct2_axis2 == 1 ? 0 : 1) : 0;       // the axis the fused launch leaves out
-  // The first pass reads the exchange's output, which has the three-byte form.
-  const bool b8 = !fused && !pairs_between_passes(p);                    // what the passes hand on has it too
+  const bool b8 = !fused && !pairs_between_passes(p);                    // the passes hand on the three-byte form
+  const int hi = exact ? T_F32 : T_BF16, lo = b8 ? T_BYTE : T_BF16;
+  const int form = exact ? FORM_EXACT : (b8 ? FORM_BYTES : FORM_PAIR);
   CUtensorMap m_in, m_inl, mbh, mbl, mah, mal, obh, obl, oah, oal, mout;
-  if (!grid_map(p, &m_in, sc.a_hi, G, first_axis) || !grid_map(p, &m_inl, sc.a_lo, G, first_axis, true) ||
-      !store_map(p, &obh, sc.b_hi, G, first_axis) || !store_map(p, &obl, sc.b_lo, G, first_axis, b8))
+  if (!grid_map(p, &m_in, sc.a_hi, G, first_axis, hi) || !store_map(p, &obh, sc.b_hi, G, first_axis, hi) ||
+      (!fused && (!grid_map(p, &mbh, sc.b_hi, G, 1, hi) || !store_map(p, &oah, sc.a_hi, G, 1, hi) ||
+                  !grid_map(p, &mah, sc.a_hi, G, 2, hi) || !store_map(p, &mout, out, dm.BH, 2))))
     return cudaErrorInvalidValue;
-  if (!fused && (!grid_map(p, &mbh, sc.b_hi, G, 1) || !grid_map(p, &mbl, sc.b_lo, G, 1, b8) ||
-                 !store_map(p, &oah, sc.a_hi, G, 1) || !store_map(p, &oal, sc.a_lo, G, 1, b8) ||
-                 !grid_map(p, &mah, sc.a_hi, G, 2) || !grid_map(p, &mal, sc.a_lo, G, 2, b8) ||
-                 !store_map(p, &mout, out, dm.BH, 2)))
+  if (exact) { m_inl = m_in; obl = obh; mbl = mbh; oal = oah; mal = mah; }     // (not used)
+  else if (!grid_map(p, &m_inl, sc.a_lo, G, first_axis, T_BYTE) || !store_map(p, &obl, sc.b_lo, G, first_axis, lo) ||
+           (!fused && (!grid_map(p, &mbl, sc.b_lo, G, 1, lo) || !store_map(p, &oal, sc.a_lo, G, 1, lo) ||
+                       !grid_map(p, &mal, sc.a_lo, G, 2, lo))))
     return cudaErrorInvalidValue;
   DctTcParams P{};
   P.dm = dm; P.status = p->buf.status; P.group = g; P.group_start = h0;
   P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = b8 ? 1 : 0; P.reverse = 1; P.axis = first_axis;
   P.image = matrix_image(p, first_axis, 1);
-  cudaError_t e = launch_pass(p, m_in, m_inl, m_inl, obh, obl, P, true, st);
+  cudaError_t e = launch_pass(p, m_in, m_inl, m_inl, obh, obl, P, exact ? FORM_EXACT : FORM_BYTES, st);
   if (e != cudaSuccess) return e;
   if (fused) return ffk_dct2_inverse(p, sc.b_hi, sc.b_lo, h0, g, out, st);
-  P.in_split = 1; P.reverse = 0; P.axis = 1; P.image = matrix_image(p, 1, 1);
-  e = launch_pass(p, mbh, mbl, mbl, oah, oal, P, b8, st);
+  P.reverse = 0; P.axis = 1; P.image = matrix_image(p, 1, 1);
+  e = launch_pass(p, mbh, mbl, mbl, oah, oal, P, form, st);
   if (e != cudaSuccess) return e;
   P.mode = MODE_LAST; P.out_lo8 = 0; P.reverse = 1; P.axis = 2; P.image = matrix_image(p, 2, 1);
-  return launch_pass(p, mah, mal, mal, mout, mout, P, b8, st);
+  return launch_pass(p, mah, mal, mal, mout, mout, P, form, st);
 }

@@ -50,6 +50,7 @@ struct XParams {
   const int* pos_high;        // [N_high]
   __nv_bfloat16* grid_hi;     // [g][N][d]: upper 16 bits of the value rounded to 24 bits
   uint8_t* grid_lo;           // [g][N][d]: the next 8 bits (the three-byte form the inverse passes read)
+  float* grid_f32;            // [g][N][d] instead of the two (template parameter F32: grids whose inverse passes read fp32)
   int h0, g;                  // heads [h0, h0+g)
   int nkeys;                  // 3m rounded up to a multiple of 16
   int ybufs;                  // token-tile buffers in shared memory (1 or 2)
@@ -110,7 +111,7 @@ __device__ __forceinline__ void x_next(XItem& x, int tm, int th) {
 }
 
 // NK = 16-key chunks of the score row (3m rounded up).
-template <int NK, int XD>
+template <int NK, int XD, bool F32>
 __global__ void __launch_bounds__(X_THREADS, 2)
 exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_constant__ CUtensorMap map_v_mid,
                    const __grid_constant__ CUtensorMap map_y_high, const __grid_constant__ CUtensorMap map_v_high,
@@ -366,6 +367,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         const size_t obase = (size_t)(x.bh - P.h0) * dm.N * XD;
         __nv_bfloat16* const grid_hi = P.grid_hi + obase + (lane & 3) * 8;
         uint8_t* const grid_lo = P.grid_lo + obase + (lane & 3) * 8;
+        float* const grid_f32 = P.grid_f32 + obase + (lane & 3) * 4;
         const int slot = n % YB, row = quarter * 32 + lane;
         const uint8_t* yrow = sY + slot * X_TILE_BYTES + row * 128;
         if (threadIdx.x == 192) XPROF_ADD(14, x14);
@@ -385,6 +387,34 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
           if (q == XD / 32 - 1) {                          // D has been read
             tc_fence_before();
             mbar_arrive(&sh.d_empty);
+          }
+          if (F32) {
+            // 16 channels at a time: four lanes store 64 bytes of a token
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+#pragma unroll
+              for (int v = 0; v < 2; ++v) {                // 8 channels: 16 bytes of the swizzled token row
+                const int c = q * 4 + half * 2 + v, r0 = half * 16 + v * 8;
+                const uint4 yv = *(const uint4*)(yrow + (c >> 3) * X_HALF + (((c & 7) ^ (row & 7)) << 4));
+                const uint32_t yw[4] = {yv.x, yv.y, yv.z, yv.w};
+                float2 w[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                  w[k] = __ffma2_rn(make_float2(__uint_as_float(r[r0 + 2 * k]), __uint_as_float(r[r0 + 2 * k + 1])), s2,
+                                    make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
+                *(float4*)(st + lane * 64 + (((2 * v) ^ ((lane >> 1) & 3)) << 4)) = make_float4(w[0].x, w[0].y, w[1].x, w[1].y);
+                *(float4*)(st + lane * 64 + (((2 * v + 1) ^ ((lane >> 1) & 3)) << 4)) = make_float4(w[2].x, w[2].y, w[3].x, w[3].y);
+              }
+              if (q == XD / 32 - 1 && half == 1) mbar_arrive(&sh.y_empty[slot]);
+              __syncwarp();
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int t = 8 * i + (lane >> 2), piece = lane & 3;
+                if (out[i] >= 0) *(float4*)(grid_f32 + out[i] + q * 32 + half * 16) = *(const float4*)(st + t * 64 + ((piece ^ ((t >> 1) & 3)) << 4));
+              }
+              __syncwarp();
+            }
+            continue;
           }
 #pragma unroll
           for (int v = 0; v < 4; ++v) {                    // 8 channels: 16 bytes of the swizzled token row
@@ -431,6 +461,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
       const size_t obase = (size_t)(x.bh - P.h0) * dm.N * XD + piece * 8;
       __nv_bfloat16* const grid_hi = P.grid_hi + obase;
       uint8_t* const grid_lo = P.grid_lo + obase;
+      float* const grid_f32 = P.grid_f32 + obase;
       int out[4];                                              // element offset of the token's row in the head's grid, or -1
       uint4 yv[4];
 #pragma unroll
@@ -471,15 +502,21 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
           const float2 dd[4] = {make_float2(d0.x, d0.y), make_float2(d0.z, d0.w), make_float2(d1.x, d1.y), make_float2(d1.z, d1.w)};
           const uint32_t yw[4] = {yv[i].x, yv[i].y, yv[i].z, yv[i].w};
           uint32_t hi[4], u[8];
+          float2 w[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const float2 v = __ffma2_rn(dd[k], s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
+            const float2 v = w[k] = __ffma2_rn(dd[k], s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
             u[2 * k] = __float_as_uint(v.x) + half;
             u[2 * k + 1] = __float_as_uint(v.y) + half;
             hi[k] = ff_hi2(u[2 * k], u[2 * k + 1]);
           }
           if (q + 1 < XD / 32 && out[i] >= 0) yv[i] = __ldg((const uint4*)(yrow + 8 * i * XD + (q + 1) * 32));
-          if (out[i] >= 0) {
+          if (F32) {
+            if (out[i] >= 0) {
+              *(float4*)(grid_f32 + out[i] + q * 32) = make_float4(w[0].x, w[0].y, w[1].x, w[1].y);
+              *(float4*)(grid_f32 + out[i] + q * 32 + 4) = make_float4(w[2].x, w[2].y, w[3].x, w[3].y);
+            }
+          } else if (out[i] >= 0) {
             *(uint4*)(grid_hi + out[i] + q * 32) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
             *(uint2*)(grid_lo + out[i] + q * 32) =
                 make_uint2(ff_lo4(u[0], u[1], u[2], u[3]), ff_lo4(u[4], u[5], u[6], u[7]));
@@ -542,11 +579,12 @@ bool ffk_exchange_tc_supported(const FFDims& dm) {
 cudaError_t ffk_exchange_tc_init() {
   cudaError_t e = cudaSuccess;
   const int most = 113 * 1024;
-#define FF_XCH(NK)                                                                                                                \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(exchange_tc_kernel<NK, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);  \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(exchange_tc_kernel<NK, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+#define FF_XCH_D(NK, D, F) \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(exchange_tc_kernel<NK, D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
+#define FF_XCH(NK) FF_XCH_D(NK, 128, false); FF_XCH_D(NK, 64, false); FF_XCH_D(NK, 128, true); FF_XCH_D(NK, 64, true)
   FF_XCH(1); FF_XCH(2); FF_XCH(3); FF_XCH(4); FF_XCH(5); FF_XCH(6);
 #undef FF_XCH
+#undef FF_XCH_D
   return e;
 }
 
@@ -580,13 +618,13 @@ bool ffk_exchange_tc_prepare(ff_plan* p) {
          encode_rows_map((CUtensorMap*)p->tmap_x[3], p->buf.spec_high, dm.Nhigh, 3 * dm.BH, dm.d);
 }
 
-// Exchange + recombination of the mid and high bands of heads [h0, h0+g) into the hi/lo grids.
+// Exchange + recombination of the mid and high bands of heads [h0, h0+g) into the hi/lo grids (no lo grid: one of fp32).
 cudaError_t ffk_exchange_tc(ff_plan* p, int h0, int g, void* grid_hi, void* grid_lo, cudaStream_t st) {
   const FFDims& dm = p->dm;
   XParams P;
   P.dm = dm; P.alloc = p->buf.alloc; P.zimg = p->buf.zimg;
   P.pos_mid = p->pos_table; P.pos_high = p->pos_table + dm.Nmid;
-  P.grid_hi = (__nv_bfloat16*)grid_hi; P.grid_lo = (uint8_t*)grid_lo;
+  P.grid_hi = (__nv_bfloat16*)grid_hi; P.grid_lo = (uint8_t*)grid_lo; P.grid_f32 = (float*)grid_hi;
   P.h0 = h0; P.g = g; P.nkeys = ff_exchange_keys(dm.m); P.status = p->buf.status;
   P.src[0] = (const __nv_bfloat16*)p->buf.y_mid; P.src[1] = (const __nv_bfloat16*)p->buf.spec_mid;
   P.src[2] = (const __nv_bfloat16*)p->buf.y_high; P.src[3] = (const __nv_bfloat16*)p->buf.spec_high;
@@ -602,18 +640,19 @@ cudaError_t ffk_exchange_tc(ff_plan* p, int h0, int g, void* grid_hi, void* grid
   const CUtensorMap& m2 = *(const CUtensorMap*)p->tmap_x[2];
   const CUtensorMap& m3 = *(const CUtensorMap*)p->tmap_x[3];
   p->launches += 1;
-#define FF_XCH(NK, D) return ff_launch(exchange_tc_kernel<NK, D>, dim3(grid), dim3(X_THREADS), smem, st, m0, m1, m2, m3, P)
-#define FF_XCH_D(D)                     \
+#define FF_XCH(NK, D, F) return ff_launch(exchange_tc_kernel<NK, D, F>, dim3(grid), dim3(X_THREADS), smem, st, m0, m1, m2, m3, P)
+#define FF_XCH_D(D, F)                  \
   switch (P.nkeys / 16) {               \
-    case 1: FF_XCH(1, D);               \
-    case 2: FF_XCH(2, D);               \
-    case 3: FF_XCH(3, D);               \
-    case 4: FF_XCH(4, D);               \
-    case 5: FF_XCH(5, D);               \
-    default: FF_XCH(6, D);              \
+    case 1: FF_XCH(1, D, F);            \
+    case 2: FF_XCH(2, D, F);            \
+    case 3: FF_XCH(3, D, F);            \
+    case 4: FF_XCH(4, D, F);            \
+    case 5: FF_XCH(5, D, F);            \
+    default: FF_XCH(6, D, F);           \
   }
-  if (dm.d == 128) FF_XCH_D(128)
-  FF_XCH_D(64)
+  if (grid_lo) { if (dm.d == 128) FF_XCH_D(128, false) FF_XCH_D(64, false) }
+  if (dm.d == 128) FF_XCH_D(128, true)
+  FF_XCH_D(64, true)
 #undef FF_XCH_D
 #undef FF_XCH
 }

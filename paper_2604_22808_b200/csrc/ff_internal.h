@@ -110,7 +110,6 @@ struct FFPassShape {
   int seq;                  // w axis
   int tiles_inner;          // tiles along `inner` (1 for the w axis)
   int tiles;                // tiles of one tensor-head
-  int ragged;               // rows are left over, a last tile is not full, or 32 rows are not a box of the grid
 };
 inline FFPassShape ff_pass_shape(const FFDims& dm, int axis) {
   FFPassShape g;
@@ -123,9 +122,16 @@ inline FFPassShape ff_pass_shape(const FFDims& dm, int axis) {
   g.rows = g.kf * g.n;
   g.tiles_inner = g.seq ? 1 : (g.inner + g.kf - 1) / g.kf;
   g.tiles = g.seq ? (g.outer + g.kf - 1) / g.kf : g.outer * g.tiles_inner;
-  g.ragged = g.rows != 128 || lines % g.kf != 0 || (g.n & (g.n - 1)) != 0;
   return g;
 }
+// Axes that divide a tile of 128 rows into boxes of whole lines.  With any other axis the values between the passes of
+// the tensor-core transform are fp32 numbers, and its operands three bf16 parts (ff_dct_tc.cu).
+FF_HD bool ff_tile_axis(int n) { return n == 16 || n == 32 || n == 64 || n == 128; }
+FF_HD bool ff_fp32_grid(const FFDims& dm) { return !(ff_tile_axis(dm.T) && ff_tile_axis(dm.H) && ff_tile_axis(dm.W)); }
+
+// Transform matrix of an axis as tensor-memory operand images: [3 parts][128 rows][64 cells of two bf16]; the first two
+// parts are the bf16 pair, all three the fp32 value.
+constexpr size_t FF_IMAGE_PART = (size_t)128 * 64, FF_IMAGE_CELLS = 3 * FF_IMAGE_PART;
 
 // Device buffers inside the caller's workspace.
 struct FFBuffers {
@@ -211,7 +217,7 @@ struct ff_plan {
   unsigned* tickets;                           // "last block" counters, zero between launches (plan-owned)
   int* pos_table;                              // rank -> flat coefficient index of the mid, then the high band (plan-owned)
   alignas(64) unsigned char tmap_x[4][128];    // CUtensorMaps of the exchange kernel (Y / V~ of the mid and high bands)
-  uint32_t* dct2_images;                       // 6 x (hi, lo) transform matrices as tensor-memory operand images (plan-owned)
+  uint32_t* dct2_images;                       // 6 transform matrices as tensor-memory operand images (plan-owned)
   FFMapCache maps;                             // tensor maps of the transform passes
   bool dct2_ok;                                // the fused two-axis launch covers this configuration
   int dct2_axis2;                              // its second axis (1 = h, 0 = t); the remaining axis gets a pass of its own

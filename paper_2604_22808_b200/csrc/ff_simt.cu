@@ -795,7 +795,7 @@ cudaError_t ffk_attention_simt(ff_plan* p, int band_bits, cudaStream_t st) {
   return p->dm.fp32 ? attention_simt_t<float>(p, band_bits, st) : attention_simt_t<__nv_bfloat16>(p, band_bits, st);
 }
 
-// Tensor-core inverse: exchange + recombination into the three-byte grids, then the three axis passes.
+// Tensor-core inverse: exchange + recombination into the three-byte grids (or one of fp32, ff_fp32_grid), then the axis passes.
 static cudaError_t exchange_inverse_tc(ff_plan* p, void* out, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int G = p->dct_group;
@@ -804,13 +804,16 @@ static cudaError_t exchange_inverse_tc(ff_plan* p, void* out, cudaStream_t st) {
     const int g = (dm.BH - h0 < G) ? dm.BH - h0 : G;
     const size_t grid_bytes = ((size_t)G * dm.N * dm.d * 2 + 255) / 256 * 256;
     __nv_bfloat16* ghi = (__nv_bfloat16*)p->buf.scratchA;
-    uint8_t* glo = (uint8_t*)p->buf.scratchA + grid_bytes;
+    uint8_t* glo = ff_fp32_grid(dm) ? nullptr : (uint8_t*)p->buf.scratchA + grid_bytes;
     if (p->xtc_ok) {
       // mid and high bands on the tensor cores, the fp32 low band with its own kernel
       e = ffk_exchange_low(p, h0, g, ghi, glo, st);
       if (e == cudaSuccess) e = ffk_exchange_tc(p, h0, g, ghi, glo, st);
-    } else {
+    } else if (glo) {
       e = dm.d == 128 ? launch_exchange<__nv_bfloat16, 4>(p, g, h0, ghi, glo, st) : launch_exchange<__nv_bfloat16, 2>(p, g, h0, ghi, glo, st);
+    } else {
+      e = dm.d == 128 ? launch_exchange<__nv_bfloat16, 4>(p, g, h0, p->buf.scratchA, nullptr, st)
+                      : launch_exchange<__nv_bfloat16, 2>(p, g, h0, p->buf.scratchA, nullptr, st);
     }
     if (e != cudaSuccess) return e;
     e = ffk_inverse_transform_tc(p, h0, g, out, st);

@@ -228,16 +228,16 @@ __device__ __forceinline__ float exp2f_fast(float x) {
 }
 
 // Low band of the tensor-core inverse ("Cross-band residual exchange", "Reconstruction"): exchange + recombination of the
-// low band's coefficients into the three-byte grids.  A head that executes the low band has one pooled output row for
+// low band's coefficients into the three-byte grids (F32: into one of fp32).  A head that executes the low band has one pooled output row for
 // every r consecutive coefficient ranks, so its update is computed once and written r times; other heads carry V~ low,
 // one row per rank.  Eight lanes share a row (lane s holds channels 4 s + 32 i .. + 3), so that a score takes three
 // shuffles for four rows at once: with a whole warp per row the kernel was bound by its five shuffles per score and row
 // (131 072 rows of 64 channels, 16 keys: 106 us).  Scores of four or eight keys are reduced side by side and merged into the
 // running softmax as a group, exponentials by ex2.approx on scores in log2 units, like the tensor-core kernel's.
 constexpr int XL_WARPS = 8;
-template <int DPL>
+template <int DPL, bool F32>
 __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffers buf, FFDims dm, int bh0, __nv_bfloat16* grid_hi,
-                                                                      uint8_t* grid_lo, int rounds) {
+                                                                      uint8_t* grid_lo, float* grid_f32, int rounds) {
   extern __shared__ float4 Z[];                 // the summaries of the other bands, [keys][d]
   constexpr int d = DPL * 32, V = DPL;          // float4 per lane and row
   constexpr int KB = DPL >= 4 ? 4 : 8;          // keys scored side by side (registers)
@@ -305,10 +305,14 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
       mx = nm;
     }
     const float inv = nkeys > 0 ? 1.f / den : 0.f;
-    // the value in three bytes, at every rank the row stands for
+    // the value, in three bytes or as it is, at every rank the row stands for
     uint2 hi[V]; uint32_t lo[V];
 #pragma unroll
     for (int i = 0; i < V; ++i) {
+      if (F32) {
+        y[i] = make_float4(fmaf(acc[i].x, inv, y[i].x), fmaf(acc[i].y, inv, y[i].y), fmaf(acc[i].z, inv, y[i].z), fmaf(acc[i].w, inv, y[i].w));
+        continue;
+      }
       const uint32_t u0 = ff_round24(fmaf(acc[i].x, inv, y[i].x)), u1 = ff_round24(fmaf(acc[i].y, inv, y[i].y));
       const uint32_t u2 = ff_round24(fmaf(acc[i].z, inv, y[i].z)), u3 = ff_round24(fmaf(acc[i].w, inv, y[i].w));
       hi[i] = make_uint2(ff_hi2(u0, u1), ff_hi2(u2, u3));
@@ -322,6 +326,7 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
       const size_t o = ((size_t)gi * dm.N + ((size_t)kt * dm.H + kh) * dm.W + kw) * d + 4 * s;
 #pragma unroll
       for (int q = 0; q < V; ++q) {
+        if (F32) { *(float4*)(grid_f32 + o + 32 * q) = y[q]; continue; }
         *(uint2*)(grid_hi + o + 32 * q) = hi[q];
         *(uint32_t*)(grid_lo + o + 32 * q) = lo[q];
       }
@@ -382,6 +387,8 @@ cudaError_t ffk_exchange_low(ff_plan* p, int h0, int g, void* grid_hi, void* gri
   rounds = rounds < 1 ? 1 : (rounds > 8 ? 8 : rounds);
   const dim3 grid((unsigned)((dm.Nlow + per_round * rounds - 1) / (per_round * rounds)), (unsigned)g);
   p->launches += 1;
-  return ff_launch(dm.d == 128 ? exchange_low_kernel<4> : exchange_low_kernel<2>, grid, dim3(XL_WARPS * 32), smem, st, p->buf, dm, h0,
-                   (__nv_bfloat16*)grid_hi, (uint8_t*)grid_lo, (int)rounds);
+  auto* kernel = grid_lo ? (dm.d == 128 ? exchange_low_kernel<4, false> : exchange_low_kernel<2, false>)
+                         : (dm.d == 128 ? exchange_low_kernel<4, true> : exchange_low_kernel<2, true>);
+  return ff_launch(kernel, grid, dim3(XL_WARPS * 32), smem, st, p->buf, dm, h0, (__nv_bfloat16*)grid_hi, (uint8_t*)grid_lo, (float*)grid_hi,
+                   (int)rounds);
 }

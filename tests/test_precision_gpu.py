@@ -32,3 +32,13 @@ def _low_band_error(grid, d, impl=0):
 @pytest.mark.parametrize("d", [64, 128])
 def test_pairs_between_the_axes(grid, d):
     assert _low_band_error(grid, d) < 2.0 ** -17
+
+
+# fp32 grids between the axes, three bf16 parts of matrix and data: as far from fp64 as fp32 arithmetic (which the generic
+# kernels do on the same grid: 1.6e-7 to 2.7e-7), a few 2^-24 per axis.
+@pytest.mark.parametrize("grid", [(21, 45, 80), (13, 33, 50), (8, 64, 64), (16, 32, 48), (7, 90, 127), (128, 3, 31)],
+                         ids=lambda g: "x".join(map(str, g)))
+@pytest.mark.parametrize("d", [64, 128])
+def test_fp32_between_the_axes_of_any_other_grid(grid, d):
+    assert _low_band_error(grid, d) < 4.0 * 2.0 ** -23
+    assert _low_band_error(grid, d, impl=2) < 4.0 * 2.0 ** -23
