@@ -4,7 +4,10 @@
 //
 // A work item is one plane of the grid (all positions of the two axes at one coordinate of the third
 // axis) of one tensor-head, for one chunk of 32 channels.  A CTA owns the item: the plane's
-// intermediate (hi/lo bf16, 4 bytes per value) takes 128 KB or less of its shared memory.
+// intermediate (hi/lo bf16, 4 bytes per value) takes 128 KB or less of its shared memory.  A plane of twice that
+// belongs to a cluster of two CTAs (template parameter PAIR): each transforms half of its lines in phase 1, sends a
+// result row to the CTA that owns the row's w coefficient (st.shared::cluster), and takes half of the w coefficients in
+// phase 2; the buffer is handed over with barriers that the other CTA arrives at.
 //   phase 1  transforms the plane's w lines (tiles of 128 positions = 128/W lines, fetched by TMA) and
 //            scatters each result row, as a hi/lo bf16 pair, into the plane buffer; the rows land in
 //            the operand layout of phase 2
@@ -20,7 +23,7 @@
 //
 //   warp 0        TMA producer (ring of 8 tiles, or 4 hi/lo pairs)
 //   warp 1        tcgen05.mma issuer of phase 1; owns the tensor-memory allocation
-//   warp 2        idle
+//   warp 2        idle (PAIR: tells both CTAs when this one has finished reading its part of the buffer)
 //   warp 3        tcgen05.mma issuer of phase 2
 //   warps 4..11   phase-1 epilogue (a thread owns one position of a tile; the first four warps take
 //                 the first tile of a pair, the next four the second)
@@ -43,8 +46,8 @@ constexpr int ROWS = 128;                     // positions per tile
 constexpr int TILE_B = ROWS * CHK * 2;        // 8 KB: one bf16 tile
 constexpr int NSTG = 8;                       // input ring: at most 8 tiles (64 KB: 8 bf16 tiles or 4 hi/lo pairs)
 constexpr int RING_B = NSTG * TILE_B;
-constexpr int MAX_TPC = 8;                    // tiles of a plane (128 KB of hi/lo buffer)
-constexpr int D2_THREADS = 640;                 // TMA, MMA 1, idle, MMA 2, 8 phase-1 and 8 phase-2 epilogue warps
+constexpr int MAX_TPC = 8;                    // tiles per CTA and item (128 KB of hi/lo buffer)
+constexpr int D2_THREADS = 640;                 // TMA, MMA 1, release, MMA 2, 8 phase-1 and 8 phase-2 epilogue warps
 constexpr int NA1 = 1, NA2 = 1;               // accumulator buffers (batches of 128 columns) of the two phases
 constexpr int IMG_CELLS = 64;                 // 32-bit tensor-memory cells per matrix row: two bf16 K elements each
 constexpr int STG_ROW = 64;                   // bytes per staged row (32 channels)
@@ -59,7 +62,7 @@ struct Dct2Params {
   int last;                // output is the caller's tensor (bf16, no lo part)
   int group, group_start;
   int nchunk;              // head_dim / 32
-  int tpc;                 // tiles of a plane
+  int tpc;                 // tiles per CTA and item
   double* clear;           // band energies to clear for the sums that follow (first launch of a routed forward), or NULL
   int* status;
 };
@@ -80,7 +83,8 @@ struct D2Shared {
   uint64_t buf_full[2];    // all rows of the item have landed in the slot
   uint64_t buf_half[2];    // the rows of the first half of the second axis have landed
   uint64_t half_free[2];   // phase 2 has finished reading those rows (its k-steps 0..3 of every batch)
-  uint64_t buf_free[2];    // phase 2 of the item has finished reading the slot
+  uint64_t buf_free[2];    // phase 2 of the item has finished reading the slot (PAIR: in both CTAs)
+  uint64_t mma2_done[2];   // (PAIR) this CTA's phase-2 instructions of the item (by slot) have completed
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -97,6 +101,56 @@ __device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t smem_addr, uint32_t 
   return d;
 }
 
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Address of the same shared-memory location in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint4 v) {
+  asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar_addr) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bounded wait of a whole warp on a barrier of the plane buffer; with PAIR its arrivals come from both CTAs.
+template <bool PAIR>
+__device__ __forceinline__ bool wait_buffer(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  if (!PAIR) return mbar_wait_warp(bar, parity, abort_flag);
+  bool ok = mbar_try_wait_cluster(bar, parity);
+  const long long t0 = clock64();
+  while (!ok && !*abort_flag) {
+    ok = mbar_try_wait_cluster(bar, parity);
+    if (!ok && clock64() - t0 > kWaitLimitCycles) *abort_flag = 1;
+  }
+  return __all_sync(0xffffffffu, ok);
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// (rows that the other CTA wrote, or that go there)
+template <bool PAIR> __device__ __forceinline__ void fence_buffer() {
+  if (PAIR) asm volatile("fence.proxy.async;" ::: "memory");
+  else fence_proxy_async();
+}
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
@@ -145,6 +199,7 @@ __device__ __forceinline__ void split_hi_lo(const uint32_t (&r)[32], uint32_t (&
 
 // map0..map2: sources (Q, K, V; or hi, lo, -).  map_oh / map_ol: destinations (hi / lo grids, or the
 // caller's tensor in map_oh), box = the 32 positions x 32 channels an epilogue warp holds.
+template <bool PAIR>
 __global__ void __launch_bounds__(D2_THREADS, 1)
 dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
                const __grid_constant__ CUtensorMap map2, const __grid_constant__ CUtensorMap map_oh,
@@ -160,18 +215,20 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   D2Shared& sh = *(D2Shared*)(sIn + RING_B);
   const int nslot = RING_B / STAGE_B;                              // ring slots: 8 tiles, or 4 hi/lo pairs
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int cs = PAIR ? 2 : 1;                                 // CTAs of a plane
+  const int rank = PAIR ? (int)cluster_ctarank() : 0;
   const int n1 = P.n1, n2 = P.n2;
   const int ln1 = 31 - __clz(n1);
   const int kf1 = ROWS / n1, kf2 = ROWS / n2;
   const int lkf2 = 31 - __clz(kf2);
   const int total = P.group * P.n3 * P.nchunk;
-  const int nsl = tpc <= MAX_TPC / 2 ? 2 : 1;                      // slots of the plane buffer
+  const int nsl = !PAIR && tpc <= MAX_TPC / 2 ? 2 : 1;             // slots of the plane buffer
   const int bt = tpc < 4 ? tpc : 4;                                // tiles per instruction batch (N = 32 bt columns): an
   const int nb = tpc / bt;                                         // instruction costs the same for any N up to 128
-  // With an even number of batches the first half of the phase-1 batches holds the first half
+  // One CTA per plane and an even number of batches: the first half of the phase-1 batches holds the first half
   // of the second axis, i.e. rows 0..63 of every phase-2 tile = its k-steps 0..3.  Phase 2 of the item's first
   // batch starts on those while phase 1 still works on the second half.
-  const bool half_start = nb >= 2 && (nb & 1) == 0;
+  const bool half_start = !PAIR && nb >= 2 && (nb & 1) == 0;
   // ... and phase 1 of the next item may overwrite those rows as soon as phase 2 has read them (forward launch:
   // measured slower for the inverse, whose phase 1 issues half as many instructions again)
   const bool half_release = half_start && !P.in_split;
@@ -180,7 +237,8 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     for (int i = 0; i < NSTG; ++i) { mbar_init(&sh.in_full[i], 1); mbar_init(&sh.in_empty[i], 1); }
     for (int i = 0; i < NA1; ++i) { mbar_init(&sh.acc1_full[i], 1); mbar_init(&sh.acc1_empty[i], 256); }
     for (int i = 0; i < NA2; ++i) { mbar_init(&sh.acc2_full[i], 1); mbar_init(&sh.acc2_empty[i], 256); }
-    for (int i = 0; i < 2; ++i) { mbar_init(&sh.buf_full[i], 8); mbar_init(&sh.buf_free[i], 1); mbar_init(&sh.buf_half[i], 8); }
+    for (int i = 0; i < 2; ++i) { mbar_init(&sh.buf_full[i], 8 * cs); mbar_init(&sh.buf_free[i], cs); mbar_init(&sh.buf_half[i], 8); }
+    if (PAIR) { mbar_init(&sh.mma2_done[0], 1); mbar_init(&sh.mma2_done[1], 1); }
     mbar_init(&sh.half_free[0], 1); mbar_init(&sh.half_free[1], 1);
     sh.abort_flag = 0;
     fence_mbar_init();
@@ -188,6 +246,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_barrier();                                     // the other CTA's barriers exist before anyone arrives there
   tc_fence_after();
   const uint32_t tm = sh.tmem_base;
   volatile int* abort_flag = &sh.abort_flag;
@@ -222,7 +281,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   __syncthreads();
   tc_fence_after();
 
-  const int cid = (int)blockIdx.x, ncl = (int)gridDim.x;
+  const int cid = (int)blockIdx.x / cs, ncl = (int)gridDim.x / cs;
   PROF_T0(t_all);
 
   if (warp == 0) {
@@ -248,7 +307,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           PROF_ADD(12, tp0);
           if (!ok) break;
           uint8_t* dst = sIn + slot * STAGE_B;
-          const int u1 = k;                                        // tile of the plane: lines u1 kf1 .. + kf1
+          const int u1 = rank * tpc + k;                           // tile of the plane: lines u1 kf1 .. + kf1
           const int b0 = u1 * kf1;
           const int ch = P.axis2 == 1 ? b0 : a3, ct = P.axis2 == 1 ? a3 : b0;
           mbar_arrive_expect_tx(&sh.in_full[slot], STAGE_B);
@@ -302,7 +361,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     }
   } else if (warp == 3) {
     // ------------------------------------------------------------------ MMA issuer, phase 2
-    // (a thread of its own: phase 2 of an item waits for all of its phase 1, phase 1 of the next item does not)
+    // (a warp of its own: phase 2 of an item waits for all of its phase 1, phase 1 of the next item does not)
     {
       const uint32_t idesc = idesc_bf16_f32(ROWS, bt * CHK, /*a_mn_major=*/false, /*b_mn_major=*/true);
       const uint32_t buf_base = smem_u32(sBuf);
@@ -313,10 +372,10 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         PROF_T0(tm2);
         const int sl = (int)(ni % nsl);                             // the item's slot of the plane buffer
         ok = half_start ? mbar_wait_warp(&sh.buf_half[sl], (ni / nsl) & 1, abort_flag)
-                        : mbar_wait_warp(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
+                        : wait_buffer<PAIR>(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
         PROF_ADD(9, tm2);
         if (!ok) break;
-        fence_proxy_async();
+        fence_buffer<PAIR>();
         for (int kb = 0; kb < nb && ok; ++kb, ++n2b) {
           const int ab = n2b % NA2;
           PROF_T0(tm3);
@@ -347,7 +406,18 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           if (!ok) break;
           umma_commit(&sh.acc2_full[ab]);
         }
-        umma_commit(&sh.buf_free[sl]);
+        umma_commit(PAIR ? &sh.mma2_done[sl] : &sh.buf_free[sl]);
+      }
+    }
+  } else if (PAIR && warp == 2) {
+    // ------------------------------------------------------------------ buffer release, to both CTAs
+    if (lane == 0) {
+      unsigned ni = 0;
+      bool ok = true;
+      for (int it = cid; it < total && ok; it += ncl, ++ni) {
+        ok = mbar_wait(&sh.mma2_done[ni % nsl], (ni / nsl) & 1, abort_flag);
+        if (!ok) break;
+        for (int rk = 0; rk < cs; ++rk) mbar_arrive_cluster(mapa(smem_u32(&sh.buf_free[ni % nsl]), (uint32_t)rk));
       }
     }
   } else if (warp >= 4 && warp < 12) {
@@ -361,7 +431,8 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const uint32_t buf_base = smem_u32(sBuf);
     const int l1 = j >> ln1, a1 = j & (n1 - 1);
-    const int u2 = a1 >> lkf2;                             // phase-2 tile of the plane that takes coefficient a1
+    const int u2g = a1 >> lkf2;                            // phase-2 tile of the plane that takes coefficient a1
+    const int owner = PAIR ? u2g / tpc : 0, u2 = u2g - owner * tpc;      // its CTA, its tile there
     // Eight neighbouring lanes store at once; their rows are kf2 per tile, and rows of different tiles
     // that share (row / 2) % 4 would meet in the same banks: the lanes of tile t of the eight start
     // their four pieces at piece `rot` instead of 0, which spreads them over the banks.
@@ -374,7 +445,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       if (ni >= (unsigned)nsl) {
         // (half_release: the first half of the batches writes rows phase 2 releases earlier; the rest waits below)
         ok = half_release ? __all_sync(0xffffffffu, mbar_wait(&sh.half_free[sl], ((ni / nsl) - 1) & 1, abort_flag))
-                        : mbar_wait_warp(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag);
+                        : wait_buffer<PAIR>(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag);
         if (!ok) break;
       }
       if (threadIdx.x == 128) PROF_ADD(1, te0);
@@ -401,13 +472,14 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         uint32_t hi[16], lo[16];
         split_hi_lo(r, hi, lo, true);
         // where the row goes: position b of the second axis, row b kf2 + (a1 mod kf2) of tile u2
-        const int u1 = bt * kb + tb;
+        const int u1 = rank * tpc + bt * kb + tb;
         const int b = u1 * kf1 + l1;
         const int drow = (b << lkf2) | (a1 & (kf2 - 1));
-        const uint32_t daddr = buf_base + (uint32_t)(sl * tpc + u2) * 2 * TILE_B + (uint32_t)drow * STG_ROW;
+        uint32_t daddr = buf_base + (uint32_t)(sl * tpc + u2) * 2 * TILE_B + (uint32_t)drow * STG_ROW;
+        if (PAIR) daddr = mapa(daddr, (uint32_t)owner);
         const int swz = (drow >> 1) & 3;
         // (debug build) the row lies inside a tile of the buffer
-        if (!FF_DBG_OK(drow >= 0 && drow < ROWS && u2 >= 0 && u2 < tpc && b < n2, P.status, 4)) continue;
+        if (!FF_DBG_OK(drow >= 0 && drow < ROWS && u2 >= 0 && u2 < tpc && owner < cs && b < n2, P.status, 4)) continue;
         // rotate the pieces by `rot` (two conditional swaps), then piece i of the registers is piece (i + rot) % 4 of the row
         if (rot & 1) {
 #pragma unroll
@@ -428,8 +500,10 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const uint32_t dst = daddr + (uint32_t)((((i + rot) & 3) ^ swz) << 4);
-          st_shared_v4(dst, make_uint4(hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]));
-          st_shared_v4(dst + TILE_B, make_uint4(lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]));
+          const uint4 vh = make_uint4(hi[4 * i], hi[4 * i + 1], hi[4 * i + 2], hi[4 * i + 3]);
+          const uint4 vl = make_uint4(lo[4 * i], lo[4 * i + 1], lo[4 * i + 2], lo[4 * i + 3]);
+          if (PAIR) { st_cluster_v4(dst, vh); st_cluster_v4(dst + TILE_B, vl); }
+          else { st_shared_v4(dst, vh); st_shared_v4(dst + TILE_B, vl); }
         }
         }
         if (threadIdx.x == 128) PROF_ADD(2, te2);
@@ -442,9 +516,10 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       if (!ok) break;
       // this warp's rows of the item are written
       PROF_T0(te4);
-      fence_proxy_async();
+      fence_buffer<PAIR>();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.buf_full[sl]);
+      if (PAIR) { if (lane < cs) mbar_arrive_cluster(mapa(smem_u32(&sh.buf_full[sl]), (uint32_t)lane)); }
+      else if (lane == 0) mbar_arrive(&sh.buf_full[sl]);
       if (threadIdx.x == 128) PROF_ADD(6, te4);
     }
   } else if (warp >= 12) {
@@ -497,7 +572,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) {
-          const int u2g = bt * kb + tb;        // tile of the plane: w coefficients u2g kf2 .. + kf2
+          const int u2g = rank * tpc + bt * kb + tb;        // tile of the plane: w coefficients u2g kf2 .. + kf2
           const int cw = u2g * kf2 + l0;
           const int ch = P.axis2 == 1 ? a0 : a3, ct = P.axis2 == 1 ? a3 : a0;
           tma_store_5d(st_hi, &map_oh, chunk * CHK, cw, ch, ct, out_slice);
@@ -521,6 +596,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     while (clock64() - t0 < 2000000) { }
     __syncthreads();
   }
+  if (PAIR) cluster_barrier();      // no CTA leaves while the other may still write into its shared memory or arrive at its barriers
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tm, 512);
@@ -579,9 +655,12 @@ constexpr size_t D2_SMEM = 1024 + (size_t)MAX_TPC * 2 * TILE_B + (size_t)8 * 2 *
 
 cudaError_t launch(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, const CUtensorMap& m2, const CUtensorMap& moh,
                    const CUtensorMap& mol, Dct2Params& P, cudaStream_t st) {
-  const int items = P.group * P.n3 * P.nchunk;
-  const dim3 grid((unsigned)(items < p->sm_count ? items : p->sm_count));
-  const cudaError_t e = ff_launch(dct2_tc_kernel, grid, dim3(D2_THREADS), D2_SMEM, st, m0, m1, m2, moh, mol, P);
+  const int items = P.group * P.n3 * P.nchunk, cs = p->dct2_pair ? 2 : 1;
+  const int most = p->sm_count / cs, ncl = items < most ? items : most;
+  const dim3 grid((unsigned)(ncl * cs));
+  const cudaError_t e = p->dct2_pair
+      ? ff_launch_cluster(dct2_tc_kernel<true>, cs, grid, dim3(D2_THREADS), D2_SMEM, st, m0, m1, m2, moh, mol, P)
+      : ff_launch(dct2_tc_kernel<false>, grid, dim3(D2_THREADS), D2_SMEM, st, m0, m1, m2, moh, mol, P);
   if (e != cudaSuccess) return e;
   p->launches += 1;
   return cudaSuccess;
@@ -598,21 +677,25 @@ bool out_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axi
 }  // namespace
 
 cudaError_t ffk_dct2_init() {
-  return cudaFuncSetAttribute(dct2_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D2_SMEM);
+  const cudaError_t e = cudaFuncSetAttribute(dct2_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D2_SMEM);
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(dct2_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)D2_SMEM);
 }
 
-// Which second axis the fused launch takes: the shorter of h and t (smaller planes), an even number of tiles.  It is
-// used only where one CTA holds the plane (W x n2 <= 1024 positions): there the launch beats the separate passes by 23%
-// (T = 16, W = 64).  With the plane spread over a cluster of two CTAs it lost to them (the remote stores of phase 1 and
-// their cluster-scope release cost more than the saved DRAM round trip: whole layer, T = 32, W = 64: 13.27 against 12.67
-// ms with three passes, two samples of 24 heads; T = 16, W = 128: 1.32 against 1.18 ms).
-bool ffk_dct2_supported(const FFDims& dm, int* axis2) {
+// Which second axis the fused launch takes, and whether two CTAs share a plane: the shorter of h and t (smaller planes),
+// an even number of tiles a CTA, up to 2048 positions (W x n2).  One CTA a plane (up to 1024): 23% faster than the separate
+// passes (T = 16, W = 64).  Two CTAs: two samples of 32 x 64 x 64 tokens, 24 heads, 12.91 ms against 13.88 with passes that
+// hand on bf16 pairs.  (With byte-form intermediates those take 12.52 ms, but lose a bit: low coefficients 9.6e-6 instead
+// of 6.3e-6 from fp64.)  From four CTAs on the launch loses to the passes with bytes, which the
+// larger planes take (64 x 64 x 64: 10.9 against 8.7 ms for the transform): the remote stores of phase 1 and their
+// cluster-scope release cost more than the saved round trip.
+bool ffk_dct2_supported(const FFDims& dm, int* axis2, bool* pair) {
   if (dm.fp32 || dm.d % CHK != 0 || (dm.d != 128 && dm.d != 64) || ff_fp32_grid(dm)) return false;
   const int a2 = dm.T < dm.H ? 0 : 1;
   const int n2 = a2 == 1 ? dm.H : dm.T;
-  const int tiles = dm.W * n2 / ROWS;
-  if (tiles > MAX_TPC || tiles % 2 != 0) return false;
-  if (axis2) *axis2 = a2;
+  const int tiles = dm.W * n2 / ROWS, cs = tiles > MAX_TPC ? 2 : 1;
+  if (tiles / cs > MAX_TPC || tiles / cs % 2 != 0) return false;
+  *axis2 = a2;
+  *pair = cs == 2;
   return true;
 }
 
@@ -651,8 +734,7 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
                              bool clear_energy, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int G = p->dct_group;
-  int axis2;
-  if (!ffk_dct2_supported(dm, &axis2)) return cudaErrorInvalidValue;
+  const int axis2 = p->dct2_axis2;
   CUtensorMap mq, mk, mv, oh, ol;
   if (!in_map(p, &mq, Q, dm.BH, axis2) || !in_map(p, &mk, K, dm.BH, axis2) ||
       !in_map(p, &mv, V, dm.BH, axis2) || !out_map(p, &oh, out_hi, G, axis2) ||
@@ -665,7 +747,7 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
   P.axis2 = axis2; P.n1 = dm.W; P.n2 = axis2 == 1 ? dm.H : dm.T; P.n3 = axis2 == 1 ? dm.T : dm.H;
   P.clear = clear_energy ? p->buf.energy : nullptr;
   P.in_split = 0; P.last = 0; P.group = g; P.group_start = g0; P.nchunk = dm.d / CHK;
-  P.tpc = dm.W * P.n2 / ROWS;
+  P.tpc = dm.W * P.n2 / ROWS / (p->dct2_pair ? 2 : 1);
   return launch(p, mq, mk, mv, oh, ol, P, st);
 }
 
@@ -673,8 +755,7 @@ cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const voi
 cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, int h0, int g, void* out, cudaStream_t st) {
   const FFDims& dm = p->dm;
   const int G = p->dct_group;
-  int axis2;
-  if (!ffk_dct2_supported(dm, &axis2)) return cudaErrorInvalidValue;
+  const int axis2 = p->dct2_axis2;
   CUtensorMap mh, ml, mo;
   if (!in_map(p, &mh, in_hi, G, axis2) || !in_map(p, &ml, in_lo, G, axis2) ||
       !out_map(p, &mo, out, dm.BH, axis2))
@@ -685,7 +766,7 @@ cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, i
   P.img1 = p->dct2_images + (size_t)(3 + 2) * per; P.img2 = p->dct2_images + (size_t)(3 + axis2) * per;
   P.axis2 = axis2; P.n1 = dm.W; P.n2 = axis2 == 1 ? dm.H : dm.T; P.n3 = axis2 == 1 ? dm.T : dm.H;
   P.in_split = 1; P.last = 1; P.group = g; P.group_start = h0; P.nchunk = dm.d / CHK;
-  P.tpc = dm.W * P.n2 / ROWS;
+  P.tpc = dm.W * P.n2 / ROWS / (p->dct2_pair ? 2 : 1);
   return launch(p, mh, ml, ml, mo, mo, P, st);
 }
 

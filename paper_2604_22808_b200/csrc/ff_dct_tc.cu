@@ -17,7 +17,7 @@
 // single bf16 rounding between passes would not meet the output tolerance.
 //
 // Three-byte intermediates.  Where the three axes run as separate passes, the pair written by the first forward
-// pass and the pairs between the inverse passes are stored (large planes, see pairs_between_passes) as the fp32 value
+// pass and the pairs between the inverse passes are stored (planes above 2048 positions) as the fp32 value
 // rounded to 24 bits: the upper 16 bits (a bf16 by truncation) in the hi grid and the next 8 bits in a byte grid.  hi
 // and (value - hi) are both exact bf16 operands, together they carry 16 significant bits, one less than a bf16 hi/lo
 // pair, and a pass moves 3 instead of 4 bytes per value.  A launch whose input has the byte form (template parameter LO8) runs four more
@@ -868,14 +868,6 @@ Scratch carve(ff_plan* p) {
   s.b_hi = (__nv_bfloat16*)(base + 2 * grid_bytes); s.b_lo = (__nv_bfloat16*)(base + 3 * grid_bytes);
   return s;
 }
-// Form of the values between three separate passes.  The byte form is a rounding to 2^-17, a bf16 pair one to 2^-18: the
-// transform's error on N(0,1) input is 1.5 times that of pairs (low coefficients 9.6e-6 against 6.3e-6).  Planes of 2048
-// positions have pairs like the smaller ones, whose two axes share a launch (two samples of 32 x 64 x 64 tokens 13.50 ms,
-// with bytes 12.16).  Larger planes have bytes: 17.9 against 19.2 ms at 64 x 64 x 64, 40.0 against 43.0 at 64 x 128 x 128.
-bool pairs_between_passes(const ff_plan* p) {
-  const int plane = p->dm.W * (p->dm.T < p->dm.H ? p->dm.T : p->dm.H);
-  return plane > 1024 && plane <= 2048;
-}
 }  // namespace
 
 cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy,
@@ -890,16 +882,15 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
   // mXh/mXl: load maps of a pass's input pair; oXh/oXl: store maps of a pass's output pair (the box
   // follows the axis of the pass that uses the map)
   const bool exact = ff_fp32_grid(dm);        // fp32 grids between the passes (in the place of a pair)
-  const bool w8 = !pairs_between_passes(p);   // the first pass writes the byte form; the second one always a pair
-                                              // (measured: the band-split pass is slower with a byte-form input)
   CUtensorMap mq, mk, mv, m1h, m1l, m2h, m2l, o0h, o0l, o1h, o1l, m3h, m3l;
-  const int lo = w8 ? T_BYTE : T_BF16;
+  // (otherwise the first pass writes the byte form; the second one a pair, measured: the band-split pass is slower with a
+  // byte-form input)
   if (!fused && !(grid_map(p, &mq, Q, dm.BH, 2) && grid_map(p, &mk, K, dm.BH, 2) && grid_map(p, &mv, V, dm.BH, 2))) return cudaErrorInvalidValue;
   if (fused   ? !(grid_map(p, &m3h, sc.a_hi, G, last_axis) && grid_map(p, &m3l, sc.a_lo, G, last_axis))
       : exact ? !(store_map(p, &o0h, sc.a_hi, G, 2, T_F32) && grid_map(p, &m1h, sc.a_hi, G, 1, T_F32) &&
                   store_map(p, &o1h, sc.b_hi, G, 1, T_F32) && grid_map(p, &m2h, sc.b_hi, G, 0, T_F32))
-              : !(store_map(p, &o0h, sc.a_hi, G, 2) && store_map(p, &o0l, sc.a_lo, G, 2, lo) &&
-                  grid_map(p, &m1h, sc.a_hi, G, 1) && grid_map(p, &m1l, sc.a_lo, G, 1, lo) &&
+              : !(store_map(p, &o0h, sc.a_hi, G, 2) && store_map(p, &o0l, sc.a_lo, G, 2, T_BYTE) &&
+                  grid_map(p, &m1h, sc.a_hi, G, 1) && grid_map(p, &m1l, sc.a_lo, G, 1, T_BYTE) &&
                   store_map(p, &o1h, sc.b_hi, G, 1) && store_map(p, &o1l, sc.b_lo, G, 1) &&
                   grid_map(p, &m2h, sc.b_hi, G, 0) && grid_map(p, &m2l, sc.b_lo, G, 0)))
     return cudaErrorInvalidValue;
@@ -928,12 +919,12 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
       continue;
     }
     P.clear = want_energy && g0 == 0 ? p->buf.energy : nullptr;
-    P.mode = MODE_FIRST; P.in_split = 0; P.out_lo8 = w8 ? 1 : 0; P.reverse = 0; P.axis = 2; P.image = matrix_image(p, 2, 0);
+    P.mode = MODE_FIRST; P.in_split = 0; P.out_lo8 = 1; P.reverse = 0; P.axis = 2; P.image = matrix_image(p, 2, 0);
     e = launch_pass(p, mq, mk, mv, o0h, o0l, P, exact ? FORM_EXACT1 : FORM_PAIR, st);
     if (e != cudaSuccess) return e;
     P.clear = nullptr;
     P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = 0; P.reverse = 1; P.axis = 1; P.image = matrix_image(p, 1, 0);
-    e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, exact ? FORM_EXACT : (w8 ? FORM_BYTES : FORM_PAIR), st);
+    e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, exact ? FORM_EXACT : FORM_BYTES, st);
     if (e != cudaSuccess) return e;
     P.in_split = 1; P.out_lo8 = 0; P.reverse = 0;
     P.mode = MODE_SPLIT; P.axis = 0; P.image = matrix_image(p, 0, 0);
@@ -951,9 +942,9 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
   const Scratch sc = carve(p);
   const bool fused = p->dct2_ok && !(p->attn_impl & 4), exact = ff_fp32_grid(dm);
   const int first_axis = fused ? (p->dct2_axis2 == 1 ? 0 : 1) : 0;       // the axis the fused launch leaves out
-  const bool b8 = !fused && !pairs_between_passes(p);                    // the passes hand on the three-byte form
-  const int hi = exact ? T_F32 : T_BF16, lo = b8 ? T_BYTE : T_BF16;
-  const int form = exact ? FORM_EXACT : (b8 ? FORM_BYTES : FORM_PAIR);
+  // (the exchange writes the three-byte form; three passes hand it on, the fused launch takes a bf16 pair)
+  const int hi = exact ? T_F32 : T_BF16, lo = fused ? T_BF16 : T_BYTE;
+  const int form = exact ? FORM_EXACT : FORM_BYTES;
   CUtensorMap m_in, m_inl, mbh, mbl, mah, mal, obh, obl, oah, oal, mout;
   if (!grid_map(p, &m_in, sc.a_hi, G, first_axis, hi) || !store_map(p, &obh, sc.b_hi, G, first_axis, hi) ||
       (!fused && (!grid_map(p, &mbh, sc.b_hi, G, 1, hi) || !store_map(p, &oah, sc.a_hi, G, 1, hi) ||
@@ -966,9 +957,9 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
     return cudaErrorInvalidValue;
   DctTcParams P{};
   P.dm = dm; P.status = p->buf.status; P.group = g; P.group_start = h0;
-  P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = b8 ? 1 : 0; P.reverse = 1; P.axis = first_axis;
+  P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = fused ? 0 : 1; P.reverse = 1; P.axis = first_axis;
   P.image = matrix_image(p, first_axis, 1);
-  cudaError_t e = launch_pass(p, m_in, m_inl, m_inl, obh, obl, P, exact ? FORM_EXACT : FORM_BYTES, st);
+  cudaError_t e = launch_pass(p, m_in, m_inl, m_inl, obh, obl, P, form, st);
   if (e != cudaSuccess) return e;
   if (fused) return ffk_dct2_inverse(p, sc.b_hi, sc.b_lo, h0, g, out, st);
   P.reverse = 0; P.axis = 1; P.image = matrix_image(p, 1, 1);
