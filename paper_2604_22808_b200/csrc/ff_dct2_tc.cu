@@ -36,6 +36,7 @@
 
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
+#include "ff_tensor_map.h"
 
 using namespace sm100;
 
@@ -603,40 +604,21 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encoder() {
-  static EncodeTiledFn enc = nullptr;
-  if (!enc) {
-    cudaDriverEntryPointQueryResult qr;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", (void**)&enc, cudaEnableDefault, &qr) != cudaSuccess) enc = nullptr;
-  }
-  return enc;
-}
-
 // 5-D map over a [slices][T][H][W][d] bf16 grid.  Load box: one phase-1 tile, 32 channels of 128/W
 // whole w lines that are neighbours along the second axis.
 bool encode_in_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis2) {
-  EncodeTiledFn enc = encoder();
-  if (!enc) return false;
   const cuuint64_t CH = (cuuint64_t)dm.d;
   cuuint64_t dims[5] = {CH, (cuuint64_t)dm.W, (cuuint64_t)dm.H, (cuuint64_t)dm.T, (cuuint64_t)slices};
   cuuint64_t strides[4] = {CH * 2, (cuuint64_t)dm.W * CH * 2, (cuuint64_t)dm.H * dm.W * CH * 2, (cuuint64_t)dm.N * CH * 2};
   cuuint32_t box[5] = {CHK, (cuuint32_t)dm.W, 1, 1, 1};
   box[axis2 == 1 ? 2 : 3] = (cuuint32_t)(ROWS / dm.W);
-  cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return ff_encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B,
+                       CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 
 // Store box: what one epilogue warp holds after phase 2, 32 channels of tile rows 32 q .. 32 q + 31,
 // row = (position along the second axis) * kf2 + (w coefficient inside the tile).
 bool encode_out_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis2) {
-  EncodeTiledFn enc = encoder();
-  if (!enc) return false;
   const cuuint64_t CH = (cuuint64_t)dm.d;
   cuuint64_t dims[5] = {CH, (cuuint64_t)dm.W, (cuuint64_t)dm.H, (cuuint64_t)dm.T, (cuuint64_t)slices};
   cuuint64_t strides[4] = {CH * 2, (cuuint64_t)dm.W * CH * 2, (cuuint64_t)dm.H * dm.W * CH * 2, (cuuint64_t)dm.N * CH * 2};
@@ -644,10 +626,8 @@ bool encode_out_map(CUtensorMap* map, const void* base, const FFDims& dm, int sl
   const int kf2 = ROWS / n2;                       // at most 8
   cuuint32_t box[5] = {CHK, (cuuint32_t)kf2, 1, 1, 1};
   box[axis2 == 1 ? 2 : 3] = (cuuint32_t)(32 / kf2);
-  cuuint32_t es[5] = {1, 1, 1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base), dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return ff_encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B,
+                       CU_TENSOR_MAP_L2_PROMOTION_NONE);
 }
 
 // (the staging areas of the tensor stores sit 1024-byte aligned: their 64-byte swizzle is a function of the address)

@@ -64,6 +64,7 @@
 
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
+#include "ff_tensor_map.h"
 #include "ff_three_byte.cuh"
 
 using namespace sm100;
@@ -732,27 +733,12 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
   }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encoder() {
-  static EncodeTiledFn enc = nullptr;
-  if (!enc) {
-    cudaDriverEntryPointQueryResult qr;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", (void**)&enc, cudaEnableDefault, &qr) != cudaSuccess) enc = nullptr;
-  }
-  return enc;
-}
-
 enum { T_BF16, T_BYTE, T_F32 };
 // 5-D map over a grid [slices][outer][n][inner][d] seen along `axis`.  Load map: the box is one tile, kf whole lines of
 // 64 (bf16), 32 (fp32) or all channels (bytes: the lo part of the three-byte form), 128-byte rows but for the 64 bytes of
 // head_dim 64.  Store map: 32 channels of what one epilogue warp holds (tile rows 32 q .. 32 q + 31), or of a whole tile
 // where 32 rows are not a box of the grid.
 bool encode_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices, int axis, int type, bool store) {
-  EncodeTiledFn enc = encoder();
-  if (!enc) return false;
   const FFPassShape g = ff_pass_shape(dm, axis);
   const cuuint64_t CH = (cuuint64_t)dm.d, eb = type == T_BYTE ? 1 : (type == T_BF16 ? 2 : 4);
   const cuuint64_t line = (cuuint64_t)g.inner * CH * eb;
@@ -764,13 +750,12 @@ bool encode_map(CUtensorMap* map, const void* base, const FFDims& dm, int slices
     if (g.seq) { box[2] = (cuuint32_t)(g.n < 32 ? g.n : 32); box[3] = (cuuint32_t)(g.n < 32 ? 32 / g.n : 1); }
     else { box[1] = (cuuint32_t)(g.kf < 32 ? g.kf : 32); box[2] = (cuuint32_t)(g.kf < 32 ? 32 / g.kf : 1); }
   }
-  cuuint32_t es[5] = {1, 1, 1, 1, 1};
   const cuuint32_t row = box[0] * (cuuint32_t)eb;      // bytes of a row in shared memory
   const CUtensorMapSwizzle swz = row == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : (row == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE);
-  return enc(map, type == T_BYTE ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : (type == T_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32),
-             5, const_cast<void*>(base), dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-             store ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const CUtensorMapDataType element = type == T_BYTE ? CU_TENSOR_MAP_DATA_TYPE_UINT8
+                                      : type == T_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  return ff_encode_map(map, element, 5, base, dims, strides, box, swz,
+                       store ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
 }
 // (through the plan's cache)
 bool map_for(ff_plan* p, CUtensorMap* map, const void* base, int slices, int axis, int type, bool store) {
