@@ -28,7 +28,6 @@
 
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
-#include "ff_tensor_map.h"
 #include "ff_worklist.cuh"
 
 using namespace sm100;

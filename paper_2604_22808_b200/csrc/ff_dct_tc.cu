@@ -64,7 +64,6 @@
 
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
-#include "ff_tensor_map.h"
 #include "ff_three_byte.cuh"
 
 using namespace sm100;

@@ -8,6 +8,7 @@
 
 #include <utility>
 
+#include "ff_tensor_map.h"
 #include "freqformer.h"
 
 #if defined(__CUDACC__)
@@ -177,28 +178,6 @@ struct FFLayout {
 constexpr int FF_COPY_EVENTS = 64;
 constexpr int FF_TS_INLINE = 32;     // timesteps of up to this many samples travel as kernel arguments
 
-// Tensor maps kept between calls (encoding two dozen of them took longer on the host than the launches they are
-// for).  An entry is known by the tensor's address, its number of slices and the encoder's own code for the rest,
-// which the plan's configuration determines; the oldest entry makes room for a new one.
-struct FFMapCache {
-  static constexpr int N = 48;
-  alignas(64) unsigned char map[N][128];
-  const void* base[N];
-  int code[N], slices[N];
-  int used, next;
-  template <class Encode>
-  bool get(void* out, const void* b, int c, int s, Encode encode) {
-    for (int i = 0; i < used; ++i)
-      if (base[i] == b && code[i] == c && slices[i] == s) { memcpy(out, map[i], 128); return true; }
-    if (!encode()) return false;
-    const int i = used < N ? used++ : next;
-    if (used == N) next = (i + 1) % N;
-    memcpy(map[i], out, 128);
-    base[i] = b; code[i] = c; slices[i] = s;
-    return true;
-  }
-};
-
 struct ff_plan {
   ff_config_t cfg;
   FFDims dm;
@@ -224,7 +203,7 @@ struct ff_plan {
   int* pos_table;                              // rank -> flat coefficient index of the mid, then the high band (plan-owned)
   alignas(64) unsigned char tmap_x[4][128];    // CUtensorMaps of the exchange kernel (Y / V~ of the mid and high bands)
   uint32_t* dct2_images;                       // 6 transform matrices as tensor-memory operand images (plan-owned)
-  FFMapCache maps;                             // tensor maps of the transform passes
+  FFMapCache maps;                             // tensor maps of the transform passes, by shape
   bool dct2_ok;                                // the fused two-axis launch covers this configuration
   int dct2_axis2;                              // its second axis (1 = h, 0 = t); the remaining axis gets a pass of its own
   bool dct2_pair;                              // two CTAs share a plane there

@@ -15,7 +15,6 @@
 
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
-#include "ff_tensor_map.h"
 
 using namespace sm100;
 

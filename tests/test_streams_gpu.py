@@ -1,5 +1,6 @@
 """Streams: a forward right behind an event wait reads what the event stands for, whoever waits (the caller, or the
 host-buffer call for its own copies), eagerly and in a captured graph."""
+import numpy as np
 import pytest
 
 from paper_2604_22808_b200 import configs as C
@@ -80,4 +81,38 @@ def test_host_call_equals_the_device_call(cfg):
             plan.forward_host(x.cpu(), x.cpu(), x.cpu(), torch.empty_like(host[0]), alloc_host=alloc.numpy())
         plan.forward_host(*host, out, alloc_host=alloc.numpy())
         assert torch.equal(out, want)
+    plan.destroy()
+
+
+@pytest.mark.parametrize("cfg", CONFIGS[1:], ids=lambda c: c.name)
+def test_new_buffers_in_every_call(cfg):
+    """The plan's tensor maps are known by their shape: each call puts in its own addresses, in any order, also those of
+    other tensors of an earlier call."""
+    import torch
+    from paper_2604_22808_b200 import binding as B
+    plan = B.Plan(cfg, I.router_weights(cfg), host_staging=True)
+    alloc = torch.full((cfg.batch * cfg.heads,), 7, dtype=torch.uint8, device="cuda")
+    src = [Hn.to_device(x, cfg) for x in Hn.host_inputs(cfg)]
+    want = {}
+    n = src[0].numel()
+    pool = torch.empty(8 * n, dtype=src[0].dtype, device="cuda")
+    gen = np.random.default_rng(5)
+    for k in range(12):
+        slots = gen.permutation(8)[:4]
+        order = tuple(gen.integers(0, 3, 3))
+        q, kk, v, out = (pool[s * n:(s + 1) * n].view(src[0].shape) for s in slots)
+        for dst, i in zip((q, kk, v), order):
+            dst.copy_(src[i])
+        plan.set_attention_impl(4 if k % 3 == 2 else 0)
+        plan.forward(q, kk, v, out, alloc=alloc)
+        key = (order, k % 3 == 2)
+        if key not in want:
+            fresh = B.Plan(cfg, I.router_weights(cfg))
+            fresh.set_attention_impl(4 if k % 3 == 2 else 0)
+            want[key] = fresh.forward(*(src[i].clone() for i in order), torch.empty_like(src[0]), alloc=alloc).clone()
+            fresh.destroy()
+        assert torch.equal(out, want[key])
+        if k == 6:                                              # (other launch groups, other maps over the same workspace)
+            host = [src[i].cpu() for i in order]
+            plan.forward_host(*host, torch.empty_like(host[0]), alloc_host=alloc.cpu().numpy())
     plan.destroy()
