@@ -686,18 +686,19 @@ bool ffk_dct2_supported(const FFDims& dm, int* axis2, bool* pair) {
 // [n][n], out[a] = sum_b mat[a][b] in[b].
 bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat, int n) {
   const size_t per = FF_IMAGE_CELLS;
+  const int parts = ff_fp32_grid(p->dm) ? 3 : 2;        // (the third is read on those grids only)
   if (!p->dct2_images && cudaMalloc((void**)&p->dct2_images, 6 * per * sizeof(uint32_t)) != cudaSuccess) return false;
   const FFPassShape g = ff_pass_shape(p->dm, axis);
   const int kf = g.kf;
   const bool seq = axis == 2;
-  std::vector<uint32_t> img(per);
+  std::vector<uint32_t> img(parts * FF_IMAGE_PART);
   for (int j = 0; j < g.rows; ++j)
     for (int r = 0; r < g.rows; ++r) {
       float v;
       if (seq) v = (j / n == r / n) ? mat[(j % n) * n + (r % n)] : 0.f;
       else v = (j % kf == r % kf) ? mat[(j / kf) * n + (r / kf)] : 0.f;
       size_t cell = (size_t)j * IMG_CELLS + (r >> 1);
-      for (int part = 0; part < 3; ++part, cell += FF_IMAGE_PART) {
+      for (int part = 0; part < parts; ++part, cell += FF_IMAGE_PART) {
         const __nv_bfloat16 h = __float2bfloat16_rn(v);
         const uint32_t hb = *(const uint16_t*)&h;
         img[cell] |= (r & 1) ? hb << 16 : hb;
@@ -705,7 +706,7 @@ bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat, i
       }
     }
   const int slot = (inverse ? 3 : 0) + axis;
-  return cudaMemcpy(p->dct2_images + slot * per, img.data(), per * sizeof(uint32_t), cudaMemcpyHostToDevice) == cudaSuccess;
+  return cudaMemcpy(p->dct2_images + slot * per, img.data(), img.size() * sizeof(uint32_t), cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
 // Forward: Q, K, V of tensor-heads [g0, g0 + g) -> w and second-axis transform -> hi/lo grids.

@@ -811,12 +811,13 @@ namespace {
 
 }  // namespace
 
-cudaError_t ffk_dct_tc_init() {
+cudaError_t ffk_dct_tc_init(const FFDims& dm) {
   cudaError_t e = cudaSuccess;
 #define FF_DCT(D, F) \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(dct_tc_kernel<D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 256)
-  FF_DCT(128, FORM_PAIR); FF_DCT(128, FORM_BYTES); FF_DCT(128, FORM_EXACT1); FF_DCT(128, FORM_EXACT);
-  FF_DCT(64, FORM_PAIR); FF_DCT(64, FORM_BYTES); FF_DCT(64, FORM_EXACT1); FF_DCT(64, FORM_EXACT);
+  if (e == cudaSuccess && dm.d == D) e = cudaFuncSetAttribute(dct_tc_kernel<D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 256)
+  if (!ffk_dct_tc_supported(dm)) return e;
+  if (ff_fp32_grid(dm)) { FF_DCT(128, FORM_EXACT1); FF_DCT(128, FORM_EXACT); FF_DCT(64, FORM_EXACT1); FF_DCT(64, FORM_EXACT); }
+  else { FF_DCT(128, FORM_PAIR); FF_DCT(128, FORM_BYTES); FF_DCT(64, FORM_PAIR); FF_DCT(64, FORM_BYTES); }
 #undef FF_DCT
   return e;
 }

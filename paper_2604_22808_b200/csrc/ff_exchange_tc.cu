@@ -378,7 +378,6 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         XPROF_T0(x10);
         tc_fence_after();
         const float2 s2 = make_float2(sh.inv[n & 3][row], sh.inv[n & 3][row]);
-        const uint32_t half = s2.x != s2.x ? 0u : FF_HALF24;   // (a NaN in a token or in a summary is in every score of the row)
 #pragma unroll 4
         for (int q = 0; q < XD / 32; ++q) {                // 32 channels
           uint32_t r[32];
@@ -426,8 +425,8 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
             for (int k = 0; k < 4; ++k) {
               const float2 d = make_float2(__uint_as_float(r[8 * v + 2 * k]), __uint_as_float(r[8 * v + 2 * k + 1]));
               const float2 w = __ffma2_rn(d, s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
-              u[2 * k] = __float_as_uint(w.x) + half;
-              u[2 * k + 1] = __float_as_uint(w.y) + half;
+              u[2 * k] = __float_as_uint(w.x) + FF_HALF24;
+              u[2 * k + 1] = __float_as_uint(w.y) + FF_HALF24;
               hi[k] = ff_hi2(u[2 * k], u[2 * k + 1]);
             }
             *(uint4*)(st + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
@@ -435,6 +434,10 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
             *(uint2*)(st + 2048 + lane * 32 + ((v ^ ((lane >> 2) & 3)) << 3)) =
                 make_uint2(ff_lo4(u[0], u[1], u[2], u[3]), ff_lo4(u[4], u[5], u[6], u[7]));
           }
+          // a NaN in the token or in a summary is in every score of the row: all of it is NaN (a branch, because a register
+          // for the half that is added above spills)
+          if (s2.x != s2.x)
+            for (int v = 0; v < 4; ++v) *(uint4*)(st + lane * 64 + v * 16) = make_uint4(0x7fff7fff, 0x7fff7fff, 0x7fff7fff, 0x7fff7fff);
           if (q == XD / 32 - 1) mbar_arrive(&sh.y_empty[slot]);
           __syncwarp();
 #pragma unroll
@@ -498,7 +501,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         for (int i = 0; i < 4; ++i) {
           const float4 d0 = *(const float4*)(st_rd0 + i * 1024), d1 = *(const float4*)(st_rd1 + i * 1024);
           const float2 s2 = make_float2(inv[8 * i], inv[8 * i]);
-          const uint32_t half = s2.x != s2.x ? 0u : FF_HALF24;
+          const uint32_t half = s2.x != s2.x ? 0u : FF_HALF24;     // (a row of NaN)
           const float2 dd[4] = {make_float2(d0.x, d0.y), make_float2(d0.z, d0.w), make_float2(d1.x, d1.y), make_float2(d1.z, d1.w)};
           const uint32_t yw[4] = {yv[i].x, yv[i].y, yv[i].z, yv[i].w};
           uint32_t hi[4], u[8];
@@ -565,16 +568,27 @@ bool ffk_exchange_tc_supported(const FFDims& dm) {
   return !dm.fp32 && (dm.d == 128 || dm.d == 64) && dm.m >= 1 && dm.m <= 32 && dm.N < (1LL << 31);
 }
 
-cudaError_t ffk_exchange_tc_init() {
-  cudaError_t e = cudaSuccess;
-  const int most = 113 * 1024;
-#define FF_XCH_D(NK, D, F) \
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(exchange_tc_kernel<NK, D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, most)
-#define FF_XCH(NK) FF_XCH_D(NK, 128, false); FF_XCH_D(NK, 64, false); FF_XCH_D(NK, 128, true); FF_XCH_D(NK, 64, true)
-  FF_XCH(1); FF_XCH(2); FF_XCH(3); FF_XCH(4); FF_XCH(5); FF_XCH(6);
-#undef FF_XCH
-#undef FF_XCH_D
-  return e;
+// The form of the kernel a configuration uses.
+typedef void (*XKernel)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, XParams);
+template <int D, bool F> static XKernel x_kernel_of(int nkeys) {
+  switch (nkeys / 16) {
+    case 1: return exchange_tc_kernel<1, D, F>;
+    case 2: return exchange_tc_kernel<2, D, F>;
+    case 3: return exchange_tc_kernel<3, D, F>;
+    case 4: return exchange_tc_kernel<4, D, F>;
+    case 5: return exchange_tc_kernel<5, D, F>;
+    default: return exchange_tc_kernel<6, D, F>;
+  }
+}
+static XKernel x_kernel(const FFDims& dm) {
+  const int nkeys = ff_exchange_keys(dm.m);
+  if (ff_fp32_grid(dm)) return dm.d == 128 ? x_kernel_of<128, true>(nkeys) : x_kernel_of<64, true>(nkeys);
+  return dm.d == 128 ? x_kernel_of<128, false>(nkeys) : x_kernel_of<64, false>(nkeys);
+}
+
+cudaError_t ffk_exchange_tc_init(const FFDims& dm) {
+  if (!ffk_exchange_tc_supported(dm)) return cudaSuccess;
+  return cudaFuncSetAttribute(x_kernel(dm), cudaFuncAttributeMaxDynamicSharedMemorySize, 113 * 1024);
 }
 
 // Rank -> flat coefficient index tables of the mid and high bands (plan-owned device memory).
@@ -629,19 +643,5 @@ cudaError_t ffk_exchange_tc(ff_plan* p, int h0, int g, void* grid_hi, void* grid
   const CUtensorMap& m2 = *(const CUtensorMap*)p->tmap_x[2];
   const CUtensorMap& m3 = *(const CUtensorMap*)p->tmap_x[3];
   p->launches += 1;
-#define FF_XCH(NK, D, F) return ff_launch(exchange_tc_kernel<NK, D, F>, dim3(grid), dim3(X_THREADS), smem, st, m0, m1, m2, m3, P)
-#define FF_XCH_D(D, F)                  \
-  switch (P.nkeys / 16) {               \
-    case 1: FF_XCH(1, D, F);            \
-    case 2: FF_XCH(2, D, F);            \
-    case 3: FF_XCH(3, D, F);            \
-    case 4: FF_XCH(4, D, F);            \
-    case 5: FF_XCH(5, D, F);            \
-    default: FF_XCH(6, D, F);           \
-  }
-  if (grid_lo) { if (dm.d == 128) FF_XCH_D(128, false) FF_XCH_D(64, false) }
-  if (dm.d == 128) FF_XCH_D(128, true)
-  FF_XCH_D(64, true)
-#undef FF_XCH_D
-#undef FF_XCH
+  return ff_launch(x_kernel(dm), dim3(grid), dim3(X_THREADS), smem, st, m0, m1, m2, m3, P);
 }

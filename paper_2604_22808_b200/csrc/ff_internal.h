@@ -231,11 +231,12 @@ void ff_set_thread_error(const char* msg);
 void ff_compute_layout(const FFDims& dm, bool with_staging, FFLayout* lay);
 
 // ---- kernel launchers (ff_simt.cu).  Each returns the cudaError_t of its launches. --------------
-// (..._init: kernel attributes on the current device, set at plan creation)
+// (..._init: kernel attributes on the current device, set at plan creation; of the forms the configuration uses where
+// there are many: the first look at a kernel loads it)
 cudaError_t ffk_simt_init();
 cudaError_t ffk_attention_tc_init();
-cudaError_t ffk_exchange_tc_init();
-cudaError_t ffk_dct_tc_init();
+cudaError_t ffk_exchange_tc_init(const FFDims& dm);
+cudaError_t ffk_dct_tc_init(const FFDims& dm);
 cudaError_t ffk_dct2_init();
 cudaError_t ffk_proj_init();
 cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy, cudaStream_t st);
