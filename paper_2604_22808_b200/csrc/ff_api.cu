@@ -218,6 +218,7 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
   if (ce == cudaSuccess) ce = ffk_dct_tc_init(p->dm);
   if (ce == cudaSuccess) ce = ffk_dct2_init();
   if (ce == cudaSuccess) ce = ffk_proj_init();
+  if (ce == cudaSuccess) ce = ffk_stats_init(p->dm);
   if (ce != cudaSuccess) {
     fail(nullptr, FF_ERR_CUDA, "could not prepare the kernels: %s", cudaGetErrorString(ce));
     delete p;

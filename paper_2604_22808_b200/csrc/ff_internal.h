@@ -239,6 +239,7 @@ cudaError_t ffk_exchange_tc_init(const FFDims& dm);
 cudaError_t ffk_dct_tc_init(const FFDims& dm);
 cudaError_t ffk_dct2_init();
 cudaError_t ffk_proj_init();
+cudaError_t ffk_stats_init(const FFDims& dm);
 cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy, cudaStream_t st);
 // ---- pooling, band statistics, router, worklist (ff_stats.cu) ---------------------------------------
 cudaError_t ffk_band_stats(ff_plan* p, const uint8_t* alloc_in, const float* timestep_host, bool bands_summed, cudaStream_t st);

@@ -218,7 +218,18 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
   if (P.work && threadIdx.x < 32) build_worklist(dm, P.alloc, P.low_on, P.work);
 }
 
+// Shared memory of a block: a row of channels per thread group for the sums, and the router's input and hidden layer.
+size_t sums_bytes(const FFDims& dm) { return (size_t)(ST_THREADS / (dm.d / 4)) * dm.d * sizeof(float); }
+size_t router_bytes(const FFDims& dm) { return (size_t)(3 * dm.d + dm.dt + dm.hid) * sizeof(float); }
+
 }  // namespace
+
+// (routers up to what a block can have; a wider one fails where it is used, with the launch's error)
+cudaError_t ffk_stats_init(const FFDims& dm) {
+  const size_t most = 226 * 1024, need = sums_bytes(dm) + router_bytes(dm);
+  return cudaFuncSetAttribute(dm.fp32 ? band_stats_kernel<float> : band_stats_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(need < most ? need : most));
+}
 
 // Pooling, statistics, router or copy of the caller's masks, worklist.  `bands_summed`: the transform's epilogue has
 // summed the energies of the mid and high bands already.
@@ -250,8 +261,7 @@ cudaError_t ffk_band_stats(ff_plan* p, const uint8_t* alloc_in, const float* tim
     P.n_mid = (int)((dm.Nmid + nsub * ST_STEPS - 1) / (nsub * ST_STEPS));
     blocks += P.n_mid + (dm.Nhigh + nsub * ST_STEPS - 1) / (nsub * ST_STEPS);
   }
-  const size_t red = (size_t)nsub * dm.d * sizeof(float), mlp = (size_t)(3 * dm.d + dm.dt + dm.hid) * sizeof(float);
   p->launches += 1;
   return ff_launch(dm.fp32 ? band_stats_kernel<float> : band_stats_kernel<__nv_bfloat16>, dim3((unsigned)blocks, (unsigned)(3 * dm.BH)),
-                   dim3(ST_THREADS), red + mlp, st, P);
+                   dim3(ST_THREADS), sums_bytes(dm) + (alloc_in ? 0 : router_bytes(dm)), st, P);
 }
