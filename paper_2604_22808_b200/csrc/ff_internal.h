@@ -140,6 +140,10 @@ FF_HD bool ff_fp32_grid(const FFDims& dm) { return !(ff_tile_axis(dm.T) && ff_ti
 // parts are the bf16 pair, all three the fp32 value.
 constexpr size_t FF_IMAGE_PART = (size_t)128 * 64, FF_IMAGE_CELLS = 3 * FF_IMAGE_PART;
 
+// SMs for the rules that shape the workspace: its size is a function of the configuration alone (it is asked for without
+// a device).  Rules that shape only a launch take the device's count.
+constexpr int FF_B200_SMS = 148;
+
 // Device buffers inside the caller's workspace.
 struct FFBuffers {
   float* spec_low;   // [3][BH][Nlow][d]

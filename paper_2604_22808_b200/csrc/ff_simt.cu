@@ -496,11 +496,14 @@ __global__ void __launch_bounds__(AT_THREADS, DPL <= 2 ? 3 : 2) attention_simt_k
   }
 }
 
-// Small launches (up to ROW_PAIRS scored pairs): one warp per query row, eight keys side by side, merged into the running
-// softmax as a group.  Little code and as many warps as rows; the tiled kernel above spends most of its 17 us there on
-// fetching its instructions (256 tokens, 2 heads of 32 channels).
+// Small launches (up to ROW_PAIRS scored pairs, if every head ran every band): one warp per query row, eight keys side by
+// side, merged into the running softmax as a group.  Little code and as many warps as rows; the tiled kernel above spends
+// most of its 17 us there on fetching its instructions (256 tokens, 2 heads of 32 channels).  Whole layer with the tiled
+// kernel / with this one, us, all bands: 23K pairs 42.2 / 32.3 (head_dim 64) and 48.5 / 31.1 (128), 73K 44.0 / 45.8 and
+// 51.0 / 43.8, 90K 46.4 / 50.3 and 58.4 / 50.5, 103K 42.5 / 47.4 (32), 227K 52.7 / 77.3 and 66.7 / 82.8, 492K 58.5 / 99.9
+// and 79.6 / 101.3.  (head_dim 96: 206K 74.8 / 58.4, 492K 83.6 / 89.7.)
 constexpr int ROW_WARPS = 4;
-constexpr long long ROW_PAIRS = 1 << 18;
+constexpr long long ROW_PAIRS = 3 << 15;
 
 template <typename KT_, int DPL>
 __device__ __forceinline__ void attend_row(const KT_* Qp, const KT_* Kp, const KT_* Vp, KT_* Yp, const FFDims& dm, int band, int n, int p) {

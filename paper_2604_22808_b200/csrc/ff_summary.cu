@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
 // Rows a piece of a segment should have: about the three blocks an SM holds over all bands while that leaves 128 rows or
 // more (a block's own latency is three to four microseconds), at most 1024 (256 KB of bf16 at head_dim 128).
 int piece_rows(const FFDims& dm) {
-  const long long rows = (long long)dm.BH * dm.N / (148 * 3);
+  const long long rows = (long long)dm.BH * dm.N / (FF_B200_SMS * 3);
   return (int)(rows < 128 ? 128 : (rows > 1024 ? 1024 : rows));
 }
 
