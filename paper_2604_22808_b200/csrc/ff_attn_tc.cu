@@ -166,12 +166,6 @@ __device__ __forceinline__ void load_tile(uint8_t* dst, const CUtensorMap* map, 
   }
 }
 
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // The kernel body.  QKV_MAPS = false: map_a / map_b cover the plan's mid / high coefficient buffers,
 // which hold Q~, K~ and V~ of head bh in slices bh, BH + bh and 2 BH + bh.  QKV_MAPS = true (the entry
 // point that allocates nothing): map_a, map_b, map_c are the caller's separate Q, K, V tensors of one

@@ -88,12 +88,6 @@ __device__ __forceinline__ void bulk_load(void* smem_dst, const void* src, uint3
                : "memory");
 }
 
-__device__ __forceinline__ float ex2f_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 __device__ __forceinline__ XItem x_decode(int h0, int it, int tm, int th) {
   XItem x;
   const int per = tm + th, rem = it % per;
@@ -325,7 +319,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
           const float2 arg = __ffma2_rn(make_float2(__uint_as_float(r[2 * i]), __uint_as_float(r[2 * i + 1])), sl22, nmb2);
-          const float2 p = make_float2(ex2f_approx(arg.x), ex2f_approx(arg.y));
+          const float2 p = make_float2(ex2(arg.x), ex2(arg.y));
           den = __fadd2_rn(den, p);
           const __nv_bfloat162 h2 = __floats2bfloat162_rn(p.x, p.y);
           ph[i] = *(const uint32_t*)&h2;

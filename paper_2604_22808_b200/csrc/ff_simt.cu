@@ -8,17 +8,6 @@
 
 namespace {
 
-__device__ __forceinline__ float4 ld4(const float* p) { return *(const float4*)p; }
-__device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
-  const uint2 w = *(const uint2*)p;
-  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
-                     __uint_as_float(w.y & 0xffff0000u));
-}
-__device__ __forceinline__ void st4(float* p, const float4& v) { *(float4*)p = v; }
-__device__ __forceinline__ void st4(__nv_bfloat16* p, const float4& v) {
-  const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-  *(uint2*)p = make_uint2(*(const uint32_t*)&a, *(const uint32_t*)&b);
-}
 __device__ __forceinline__ void fma4(float4& acc, float m, const float4& x) {
   acc.x = fmaf(m, x.x, acc.x); acc.y = fmaf(m, x.y, acc.y); acc.z = fmaf(m, x.z, acc.z); acc.w = fmaf(m, x.w, acc.w);
 }

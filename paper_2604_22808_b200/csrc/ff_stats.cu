@@ -6,6 +6,7 @@
 // runs it.  What these steps cost is latency, not work: as five launches (low-band energy, router, pooling, worklist
 // and the fp32 path's energies) they took 53 us of a 16K-token layer, the router alone 29 us with its second layer
 // read by three threads.
+#include "ff_bands.cuh"
 #include "ff_internal.h"
 #include "ff_worklist.cuh"
 
@@ -30,17 +31,6 @@ struct StatsParams {
   int low_steps;                         // pooled tokens per thread of a low block
 };
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-__device__ __forceinline__ float4 load4(const float* p) { return *(const float4*)p; }
-__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
-  const uint2 w = *(const uint2*)p;
-  return make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
-                     __uint_as_float(w.y & 0xffff0000u));
-}
 __device__ __forceinline__ void add_squares(float4& e, const float4& x) {
   e.x = fmaf(x.x, x.x, e.x); e.y = fmaf(x.y, x.y, e.y); e.z = fmaf(x.z, x.z, e.z); e.w = fmaf(x.w, x.w, e.w);
 }
@@ -163,7 +153,7 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
         const int n = (int)(p1 - p0);
 #pragma unroll 4
         for (int i = 0; i < n; ++i) {
-          const float4 x = load4(src + (size_t)i * d);
+          const float4 x = ld4(src + (size_t)i * d);
           acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
           add_squares(e, x);
         }
@@ -185,7 +175,7 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
     if (sub < nsub)
 #pragma unroll
       for (int k = 0; k < ST_STEPS; ++k)
-        if (r0 + k * nsub < nl) add_squares(e, load4(src + (size_t)(r0 + k * nsub) * d));
+        if (r0 + k * nsub < nl) add_squares(e, ld4(src + (size_t)(r0 + k * nsub) * d));
   }
   if (P.energy) {
     if (sub < nsub) *(float4*)(sm + sub * d + vec * 4) = e;

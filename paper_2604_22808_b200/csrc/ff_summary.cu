@@ -12,6 +12,7 @@
 // its own in front of the tensor-core kernel it cost 6 - 27 us of the step for microseconds of work.
 #include "ff_bands.cuh"
 #include "ff_internal.h"
+#include "ff_sm100.cuh"
 #include "ff_three_byte.cuh"
 
 namespace {
@@ -221,12 +222,6 @@ __global__ void __launch_bounds__(SUM_THREADS) summary_kernel(const __grid_const
     for (int i = tid; i < (P.nkeys - 3 * m) * d; i += SUM_THREADS) store_image(P, bh, 3 * m + i / d, i % d, 0.f);
 }
 
-__device__ __forceinline__ float exp2f_fast(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Low band of the tensor-core inverse ("Cross-band residual exchange", "Reconstruction"): exchange + recombination of the
 // low band's coefficients into the three-byte grids (F32: into one of fp32).  A head that executes the low band has one pooled output row for
 // every r consecutive coefficient ranks, so its update is computed once and written r times; other heads carry V~ low,
@@ -286,13 +281,13 @@ __global__ void __launch_bounds__(XL_WARPS * 32, 2) exchange_low_kernel(FFBuffer
       float nm = mx;
 #pragma unroll
       for (int k = 0; k < KB; ++k) { sc[k] = k0 + k < nkeys ? sc[k] * scale : -INFINITY; nm = fmaxf(nm, sc[k]); }
-      const float corr = exp2f_fast(mx - nm);
+      const float corr = sm100::ex2(mx - nm);
       den *= corr;
 #pragma unroll
       for (int i = 0; i < V; ++i) { acc[i].x *= corr; acc[i].y *= corr; acc[i].z *= corr; acc[i].w *= corr; }
 #pragma unroll
       for (int k = 0; k < KB; ++k) {
-        const float p = exp2f_fast(sc[k] - nm);               // (0 for the keys past the end)
+        const float p = sm100::ex2(sc[k] - nm);               // (0 for the keys past the end)
         const float4* z = Z + (size_t)(k0 + k < nkeys ? k0 + k : 0) * (d / 4) + s;
         den += p;
 #pragma unroll
