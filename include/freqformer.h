@@ -256,8 +256,9 @@ ff_status_t ff_get_tap(const ff_plan_t *plan, int32_t which, const void **dev_pt
  * axes of the tensor-core transform as separate passes (instead of two of them fused in one launch
  * with the intermediate kept in shared memory).  For tests and benchmarks.
  * The tensor-core kernels cover bf16 storage with head_dim 128 or 64 and mid block sizes that tile
- * 128 ranks (any axis lengths; two axes share a launch where both are 16, 32, 64 or 128); the pooled low band joins the tensor-core attention launch
- * from 128 pooled tokens on.  Every other configuration runs on the generic fp32 kernels. */
+ * 128 ranks, and any axis lengths: with axes of 16, 32, 64 or 128 two of them share a launch where the plane has at
+ * most 2048 positions, with any other axis the values between the axes are fp32.  The pooled low band joins the
+ * tensor-core attention launch from 128 pooled tokens on.  Every other configuration runs on the generic fp32 kernels. */
 ff_status_t ff_plan_set_attention_impl(ff_plan_t *plan, int32_t impl);
 
 /* ---- for callers that cannot allocate device memory ---------------------------------------------

@@ -14,9 +14,10 @@ import numpy as np
 
 from .configs import FFConfig
 
-# FF_LIBRARY_VARIANT=debug loads the build with device-side range checks (python -m paper_2604_22808_b200.build --debug)
-_LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)),
-                         "libfreqformer_debug.so" if os.environ.get("FF_LIBRARY_VARIANT") == "debug" else "libfreqformer.so")
+# FF_LIBRARY_VARIANT=debug loads the build with device-side range checks (python -m paper_2604_22808_b200.build --debug),
+# =clocks the one with cycle sums (--clocks)
+_LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), {
+    "debug": "libfreqformer_debug.so", "clocks": "libfreqformer_clocks.so"}.get(os.environ.get("FF_LIBRARY_VARIANT"), "libfreqformer.so"))
 _lib = None
 
 FF_OK = 0

@@ -11,6 +11,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 LIB = os.path.join(PKG, "libfreqformer.so")
 LIB_DEBUG = os.path.join(PKG, "libfreqformer_debug.so")     # the same sources with -DFF_DEBUG (device-side range checks)
+LIB_CLOCKS = os.path.join(PKG, "libfreqformer_clocks.so")   # ... with -DFF_CLOCKS (cycle sums, see clocks.py)
 
 
 def _nvcc() -> str:
@@ -33,14 +34,14 @@ def needs_build(lib: str = LIB) -> bool:
     return any(os.path.getmtime(f) > t for f in deps)
 
 
-def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
-    lib = LIB_DEBUG if debug else LIB
+def build(force: bool = False, verbose: bool = False, debug: bool = False, clocks: bool = False) -> str:
+    lib = LIB_CLOCKS if clocks else (LIB_DEBUG if debug else LIB)
     if not force and not needs_build(lib):
         return lib
     cmd = [_nvcc(), "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
            "-shared", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", os.path.join(PKG, "csrc"),
-           "-o", lib] + (["-DFF_DEBUG"] if debug else []) + sources()
-    cmd[1:1] = os.environ.get("FF_NVCC_FLAGS", "").split()      # e.g. -DFF_DEBUG: the build with device-side range checks
+           "-o", lib] + (["-DFF_CLOCKS"] if clocks else ["-DFF_DEBUG"] if debug else []) + sources()
+    cmd[1:1] = os.environ.get("FF_NVCC_FLAGS", "").split()      # e.g. --threads 8
     if verbose:
         cmd.insert(1, "-Xptxas")
         cmd.insert(2, "-v")
@@ -53,4 +54,5 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
 
 
 if __name__ == "__main__":
-    print(build(force="--force" in sys.argv, verbose="-v" in sys.argv, debug="--debug" in sys.argv))
+    print(build(force="--force" in sys.argv, verbose="-v" in sys.argv, debug="--debug" in sys.argv,
+                clocks="--clocks" in sys.argv))

@@ -102,8 +102,7 @@ BY_NAME.update({c.name: c for c in REPLICAS})
 # experiments"): d_k = 64, band fractions 0.125 / 0.375 / 0.5 (low box = half of every axis, mid box
 # = the box of about 0.794 of every axis), r = 4 so that N_low_bar = N / 32, window w = 64 (R = 32),
 # m = 8, and a mid pattern of constant degree k_mid = 256: blocks of 32 ranks with stride
-# s = N_mid / 256 rounded, so that a residue class holds 8 blocks.  head_dim 64 is outside the
-# tensor-core exchange kernel (head_dim 128 only), which the generic kernel replaces here.
+# s = N_mid / 256 rounded, so that a residue class holds 8 blocks.
 PAPER_REF_64K = FFConfig(name="paper_ref_64k", batch=1, T=16, H=64, W=64, heads=16, head_dim=64, dtype="bf16",
                          low_cut=(8, 32, 32), mid_cut=(13, 51, 51), r=4, b=32, s=100, R=32, m=8, seed=5,
                          timesteps=(500.0,))

@@ -26,6 +26,7 @@
 // word, stops taking work, lets its copies drain, frees its tensor memory and returns.
 #include <cuda.h>
 
+#include "ff_clocks.cuh"
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
 #include "ff_worklist.cuh"
@@ -269,27 +270,34 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         const int st = gt & 1;
         const uint64_t qd = q_desc + (uint64_t)(sx * (TILE_BYTES >> 4)), kd = k_desc + (uint64_t)(st * (TILE_BYTES >> 4));
         const uint32_t d_tm = tm + sx * 128;
+        FF_CLOCK(c_qk);
 #pragma unroll
         for (int k = 0; k < HD / 16; ++k) {
           const uint64_t off = (uint64_t)(((k >> 2) * HALF_BYTES + (k & 3) * 32) >> 4);
           umma_ss(d_tm, qd + off, kd + off, idesc_qk, k > 0 ? 1u : 0u);
         }
         umma_commit(&sh.s_full[sx]);
+        FF_CLOCK_ADD(lane == 0, 0, c_qk);
         if (last) umma_commit(&sh.k_empty[st]);
         if (release_q) umma_commit(&sh.q_empty);
       };
       // O_x (+)= P_x V[tile]: the first 64 keys while the softmax works on the others
       auto issue_pv = [&](int sx, unsigned gt, bool first_of_item, bool last, bool last_of_item) -> bool {
         const int st = gt & 1;
+        FF_CLOCK(c_half);
         if (!mbar_wait_warp(&sh.p_half[sx], cp[sx] & 1, abort_flag)) return false;
+        FF_CLOCK_ADD(lane == 0, 2, c_half);
         if (first_of_item && ce[sx] >= 1 && !mbar_wait_warp(&sh.o_empty[sx], (ce[sx] - 1) & 1, abort_flag)) return false;
         tc_fence_after();
         const uint64_t vd = v_desc + (uint64_t)(st * (TILE_BYTES >> 4));
         const uint32_t p_tm = tm + sx * 128, d_tm = p_tm + 256, first = first_of_item ? 0u : 1u;
+        FF_CLOCK(c_pv);                                    // (with the wait for the second half)
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           if (k == 4) {
+            FF_CLOCK(c_full);
             if (!mbar_wait_warp(&sh.p_full[sx], cp[sx] & 1, abort_flag)) return false;
+            FF_CLOCK_ADD(lane == 0, 3, c_full);
             ++cp[sx];
             tc_fence_after();
           }
@@ -298,6 +306,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         }
         if (last_of_item) umma_commit(&sh.o_full[sx]);
         if (last) umma_commit(&sh.v_empty[st]);
+        FF_CLOCK_ADD(lane == 0, 1, c_pv);
         return true;
       };
       for (int it = blockIdx.x; it < total && ok; it += gridDim.x, ++iter) {
@@ -316,6 +325,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
           if (b0) issue_qk(1, g0, true, x.nk == 1);
         }
         for (int j = 0; j < x.nk && ok; ++j) {
+          FF_CLOCK(c_tile);
           const unsigned gt = g0 + j;
           const bool aj = stream_active(x, 0, j), bj = stream_active(x, 1, j);
           const bool more = j + 1 < x.nk;
@@ -338,6 +348,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
               issue_qk(sx, gt + 1, last_qk, last_qk && j + 2 == x.nk);
             }
           }
+          FF_CLOCK_ADD(lane == 0, 4, c_tile);
         }
         g = g0 + x.nk;
         ce[0] += 1;
@@ -397,8 +408,11 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
             chi = hi < TILE - 1 ? (int)(hi < -1 ? -1 : hi) : TILE - 1;
           }
         }
+        FF_CLOCK(c_wait);
         ok = __all_sync(0xffffffffu, mbar_wait(&sh.s_full[sx], cs & 1, abort_flag));
         if (!ok) break;
+        FF_CLOCK_ADD((threadIdx.x & 127) == 0, 8, c_wait);
+        FF_CLOCK(c_max);
         tc_fence_after();
         // the row's scores, and their maximum in four chains
         uint32_t r[4][32];
@@ -429,6 +443,8 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
         const float m_new = fmaxf(m_ref, tmax);
         const bool need = (m_new - m_ref) * sl2 > LAZY_LOG2;
         const float alpha = need ? ex2((m_ref - m_new) * sl2) : 1.f;
+        FF_CLOCK_ADD((threadIdx.x & 127) == 0, 9, c_max);
+        FF_CLOCK(c_scale);
         // The previous PV of this stream has completed: the scores of this tile, which s_full announces, were issued
         // behind it by the same thread.  So O may be rescaled in place.
         if (!first && __any_sync(0xffffffffu, need)) {
@@ -444,6 +460,8 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
           tmem_wait_st();
         }
         if (need) { l *= alpha; m_ref = m_new; }
+        FF_CLOCK_ADD((threadIdx.x & 127) == 0, 10, c_scale);
+        FF_CLOCK(c_exp);
         // P = 2^(s*scale*log2e - m) as bf16 over the scores, partial row sum
         const float mb = m_ref * sl2;
         float2 sum2 = make_float2(0.f, 0.f);              // (two scores per FMA / add: packed fp32 instructions)
@@ -466,6 +484,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
             mbar_arrive(c == 1 ? &sh.p_half[sx] : &sh.p_full[sx]);
           }
         }
+        FF_CLOCK_ADD((threadIdx.x & 127) == 0, 11, c_exp);
         l += sum2.x + sum2.y;
         first = false;
         ++cs;
@@ -587,8 +606,8 @@ bool ffk_tc_prepare(ff_plan* p) {
                        3 * dm.BH, dm.Nmid > 0 ? rb : 1, dm.d) ||
       !encode_band_map((CUtensorMap*)p->tmap_high, p->buf.spec_high, dm.Nhigh, 3 * dm.BH, TILE, dm.d))
     return false;
-  // The low branch joins this launch when the pooled band is at least one tile long (shorter ones
-  // stay on the generic fp32 kernel, which is exact and costs microseconds there).
+  // The low branch joins this launch when the pooled band is at least one tile long (shorter ones are attended in fp32 by
+  // the summary launch, or by the generic kernel where there are no summaries).
   p->low_tc_ok = p->buf.pooled_bf && dm.Nbar >= TILE && dm.Nbar < (1LL << 31) - 256 && (long long)dm.BH * 3 <= MAX_UNITS &&
                  encode_band_map((CUtensorMap*)p->tmap_low, p->buf.pooled_bf, dm.Nbar, 3 * dm.BH, TILE, dm.d);
   return true;
@@ -697,3 +716,5 @@ extern "C" ff_status_t ff_high_attention_noalloc(const void* q, const void* k, c
   }
   return FF_OK;
 }
+
+FF_CLOCKS_READ(attention)

@@ -34,6 +34,7 @@
 
 #include <vector>
 
+#include "ff_clocks.cuh"
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
 
@@ -66,15 +67,6 @@ struct Dct2Params {
   double* clear;           // band energies to clear for the sums that follow (first launch of a routed forward), or NULL
   int* status;
 };
-
-#ifdef FF_D2_PROF
-__device__ unsigned long long g_d2_prof[32];
-#define PROF_T0(v) const long long v = clock64()
-#define PROF_ADD(i, v) atomicAdd(&g_d2_prof[i], (unsigned long long)(clock64() - (v)))
-#else
-#define PROF_T0(v)
-#define PROF_ADD(i, v)
-#endif
 
 struct D2Shared {
   uint64_t in_full[NSTG], in_empty[NSTG], acc1_full[NA1], acc1_empty[NA1], acc2_full[NA2], acc2_empty[NA2];
@@ -265,7 +257,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   tc_fence_after();
 
   const int cid = (int)blockIdx.x / cs, ncl = (int)gridDim.x / cs;
-  PROF_T0(t_all);
+  FF_CLOCK(t_all);
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -285,9 +277,9 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         }
         for (int k = 0; k < tpc && ok; ++k, ++n) {
           const int slot = n % nslot;
-          PROF_T0(tp0);
+          FF_CLOCK(tp0);
           if (n >= (unsigned)nslot) ok = mbar_wait(&sh.in_empty[slot], ((n / nslot) - 1) & 1, abort_flag);
-          PROF_ADD(12, tp0);
+          FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 12, tp0);
           if (!ok) break;
           uint8_t* dst = sIn + slot * STAGE_B;
           const int u1 = rank * tpc + k;                           // tile of the plane: lines u1 kf1 .. + kf1
@@ -312,12 +304,12 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         for (int kb = 0; kb < nb && ok; ++kb, ++n1b) {
           const int ab = n1b % NA1;
           const unsigned nt = bt * n1b;                            // index of the batch's first tile in the ring sequence
-          PROF_T0(tm0);
+          FF_CLOCK(tm0);
           for (int i = 0; i < bt && ok; ++i) ok = mbar_wait_warp(&sh.in_full[(nt + i) % nslot], ((nt + i) / nslot) & 1, abort_flag);
-          PROF_ADD(7, tm0);
-          PROF_T0(tm1);
+          FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 7, tm0);
+          FF_CLOCK(tm1);
           if (ok && n1b >= (unsigned)NA1) ok = mbar_wait_warp(&sh.acc1_empty[ab], ((n1b / NA1) - 1) & 1, abort_flag);
-          PROF_ADD(8, tm1);
+          FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 8, tm1);
           if (!ok) break;
           tc_fence_after();
           const uint32_t x0 = in_base + (uint32_t)(nt % nslot) * STAGE_B;
@@ -352,18 +344,18 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       bool ok = true;
       for (int it = cid; it < total && ok; it += ncl, ++ni) {
         // the plane's rows have landed in this CTA's buffer
-        PROF_T0(tm2);
+        FF_CLOCK(tm2);
         const int sl = (int)(ni % nsl);                             // the item's slot of the plane buffer
         ok = half_start ? mbar_wait_warp(&sh.buf_half[sl], (ni / nsl) & 1, abort_flag)
                         : wait_buffer<PAIR>(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
-        PROF_ADD(9, tm2);
+        FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 9, tm2);
         if (!ok) break;
         fence_buffer<PAIR>();
         for (int kb = 0; kb < nb && ok; ++kb, ++n2b) {
           const int ab = n2b % NA2;
-          PROF_T0(tm3);
+          FF_CLOCK(tm3);
           if (n2b >= (unsigned)NA2) ok = mbar_wait_warp(&sh.acc2_empty[ab], ((n2b / NA2) - 1) & 1, abort_flag);
-          PROF_ADD(10, tm3);
+          FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 10, tm3);
           if (!ok) break;
           tc_fence_after();
           const uint32_t x0 = buf_base + (uint32_t)(sl * tpc + bt * kb) * 2 * TILE_B;   // tiles bt kb ..: hi, lo of each in turn
@@ -372,9 +364,9 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
 #pragma unroll
           for (int ks = 0; ks < ROWS / 16; ++ks) {
             if (ks == ROWS / 32 && kb == 0 && half_start) {          // the second half of the rows
-              PROF_T0(tm4);
+              FF_CLOCK(tm4);
               ok = mbar_wait_warp(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
-              PROF_ADD(11, tm4);
+              FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 11, tm4);
               if (!ok) break;
               fence_proxy_async();
               tc_fence_after();
@@ -423,7 +415,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     unsigned n1b = 0, ni = 0;
     bool ok = true;
     for (int it = cid; it < total && ok; it += ncl, ++ni) {
-      PROF_T0(te0);
+      FF_CLOCK(te0);
       const int sl = (int)(ni % nsl);                         // the item's slot: free once phase 2 of item ni - nsl is done
       if (ni >= (unsigned)nsl) {
         // (half_release: the first half of the batches writes rows phase 2 releases earlier; the rest waits below)
@@ -431,18 +423,18 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
                         : wait_buffer<PAIR>(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag);
         if (!ok) break;
       }
-      if (threadIdx.x == 128) PROF_ADD(1, te0);
+      FF_CLOCK_ADD(threadIdx.x == 128, P.in_split * 16 + 1, te0);
       for (int kb = 0; kb < nb && ok; ++kb, ++n1b) {
         if (half_release && kb == nb / 2 && ni >= (unsigned)nsl) {
           ok = mbar_wait_warp(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag);
           if (!ok) break;
         }
         const int ab = n1b % NA1;
-        PROF_T0(te1);
+        FF_CLOCK(te1);
         ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc1_full[ab], (n1b / NA1) & 1, abort_flag));
         if (!ok) break;
-        if (threadIdx.x == 128) PROF_ADD(0, te1);
-        PROF_T0(te2);
+        FF_CLOCK_ADD(threadIdx.x == 128, P.in_split * 16 + 0, te1);
+        FF_CLOCK(te2);
         tc_fence_after();
         for (int tb = half; tb < bt; tb += 2) {            // this warp's tiles of the batch
         uint32_t r[32];
@@ -489,7 +481,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           else { st_shared_v4(dst, vh); st_shared_v4(dst + TILE_B, vl); }
         }
         }
-        if (threadIdx.x == 128) PROF_ADD(2, te2);
+        FF_CLOCK_ADD(threadIdx.x == 128, P.in_split * 16 + 2, te2);
         if (half_start && kb == nb / 2 - 1) {               // this warp's rows of the first half are written
           fence_proxy_async();
           __syncwarp();
@@ -498,12 +490,12 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       }
       if (!ok) break;
       // this warp's rows of the item are written
-      PROF_T0(te4);
+      FF_CLOCK(te4);
       fence_buffer<PAIR>();
       __syncwarp();
       if (PAIR) { if (lane < cs) mbar_arrive_cluster(mapa(smem_u32(&sh.buf_full[sl]), (uint32_t)lane)); }
       else if (lane == 0) mbar_arrive(&sh.buf_full[sl]);
-      if (threadIdx.x == 128) PROF_ADD(6, te4);
+      FF_CLOCK_ADD(threadIdx.x == 128, P.in_split * 16 + 6, te4);
     }
   } else if (warp >= 12) {
     // ------------------------------------------------------------------ phase-2 epilogue
@@ -524,11 +516,11 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       const int out_slice = P.last ? P.group_start + gi : gi;
       for (int kb = 0; kb < nb && ok; ++kb, ++n2b) {
         const int ab = n2b % NA2;
-        PROF_T0(te5);
+        FF_CLOCK(te5);
         ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc2_full[ab], (n2b / NA2) & 1, abort_flag));
         if (!ok) break;
-        if (threadIdx.x == 384) PROF_ADD(3, te5);
-        PROF_T0(te6);
+        FF_CLOCK_ADD(threadIdx.x == 384, P.in_split * 16 + 3, te5);
+        FF_CLOCK(te6);
         tc_fence_after();
         for (int tb = half; tb < bt; tb += 2) {            // this warp's tiles of the batch
         uint32_t r[32];
@@ -541,10 +533,10 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
         uint32_t hi[16], lo[16];
         split_hi_lo(r, hi, lo, !P.last);
         // the previous tensor store of this warp must have read the staging area
-        PROF_T0(te7);
+        FF_CLOCK(te7);
         if (lane == 0) bulk_wait_read0();
         __syncwarp();
-        if (threadIdx.x == 384) PROF_ADD(4, te7);
+        FF_CLOCK_ADD(threadIdx.x == 384, P.in_split * 16 + 4, te7);
         // 16-byte chunk i of row `lane` at chunk position i ^ (lane / 2 % 4): the 64-byte swizzle
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -563,14 +555,14 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           bulk_commit();
         }
         }
-        if (threadIdx.x == 384) PROF_ADD(5, te6);
+        FF_CLOCK_ADD(threadIdx.x == 384, P.in_split * 16 + 5, te6);
       }
     }
     if (lane == 0) bulk_wait0();
   }
 
   // ------------------------------------------------------------------ teardown
-  if (threadIdx.x == 128) PROF_ADD(15, t_all);
+  FF_CLOCK_ADD(threadIdx.x == 128, P.in_split * 16 + 15, t_all);
   tc_fence_before();
   __syncthreads();
   if (sh.abort_flag) {
@@ -733,10 +725,4 @@ cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, i
   return launch(p, mh, ml, ml, mo, mo, P, st);
 }
 
-#ifdef FF_D2_PROF
-extern "C" void ff_debug_d2_prof(unsigned long long* out32, int reset) {
-  cudaDeviceSynchronize();
-  cudaMemcpyFromSymbol(out32, g_d2_prof, sizeof(unsigned long long) * 32);
-  if (reset) { unsigned long long z[32] = {}; cudaMemcpyToSymbol(g_d2_prof, z, sizeof(z)); }
-}
-#endif
+FF_CLOCKS_READ(transform_plane)

@@ -62,6 +62,7 @@
 
 #include <vector>
 
+#include "ff_clocks.cuh"
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
 #include "ff_three_byte.cuh"
@@ -76,14 +77,6 @@ constexpr int TILE_BYTES = TILE_ROWS * CH_MAX * 2; // 32 KB: 128 rows of bf16
 constexpr int HALF_BYTES = TILE_BYTES / 2;
 constexpr int MAX_STAGE = 8;
 
-#ifdef FF_DCT_PROF
-__device__ unsigned long long g_dct_prof[128];
-#define PROF_T0(v) const long long v = clock64()
-#define PROF_ADD(i, v) atomicAdd(&g_dct_prof[(P.mode * 2 + (LO8 ? 1 : 0)) * 12 + (i)], (unsigned long long)(clock64() - (v)))
-#else
-#define PROF_T0(v)
-#define PROF_ADD(i, v)
-#endif
 constexpr int NACC_MAX = 3;
 constexpr int IMG_CELLS = 64;               // 32-bit tensor-memory cells per matrix row: two bf16 K elements each
 
@@ -232,9 +225,9 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
         const int s = P.reverse ? total_tiles - 1 - sl : sl;
         const int slot = it % NSTAGE;
-        PROF_T0(pt);
+        FF_CLOCK(pt);
         if (it >= (unsigned)NSTAGE) ok = mbar_wait(&sh.empty[slot], ((it / NSTAGE) - 1) & 1, abort_flag);
-        PROF_ADD(6, pt);
+        FF_CLOCK_ADD(lane == 0, P.mode * 16 + 6, pt);
         if (!ok) break;
         uint8_t* dst = sData + slot * STAGE_BYTES;
         const int gi = (int)ff_div((unsigned)s, P.by_tiles);
@@ -270,12 +263,12 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       bool ok = true;
       for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
         const int slot = it % NSTAGE, ab = it % NACC;
-        PROF_T0(pm);
+        FF_CLOCK(pm);
         ok = mbar_wait_warp(CONVERT ? &sh.conv[slot] : &sh.full[slot], (it / NSTAGE) & 1, abort_flag);
-        PROF_ADD(2, pm);
-        PROF_T0(pm2);
+        FF_CLOCK_ADD(lane == 0, P.mode * 16 + 2, pm);
+        FF_CLOCK(pm2);
         if (ok && it >= NACC) ok = mbar_wait_warp(&sh.acc_empty[ab], ((it / NACC) - 1) & 1, abort_flag);
-        PROF_ADD(3, pm2);
+        FF_CLOCK_ADD(lane == 0, P.mode * 16 + 3, pm2);
         if (!ok) break;
         tc_fence_after();
         const uint32_t dbase = smem_u32(sData + slot * STAGE_BYTES);
@@ -325,11 +318,11 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     bool ok = true;
     for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
       const int slot = it % NSTAGE;
-      PROF_T0(pc0);
+      FF_CLOCK(pc0);
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[slot], (it / NSTAGE) & 1, abort_flag));
-      if (threadIdx.x == 320) PROF_ADD(0, pc0);
+      FF_CLOCK_ADD(threadIdx.x == 320, P.mode * 16 + 0, pc0);
       if (!ok) break;
-      PROF_T0(pc1);
+      FF_CLOCK(pc1);
       if (r0 < rows) {
 #pragma unroll 1
         for (int h = 0; h < CH / 64; ++h) {
@@ -361,7 +354,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       }
       fence_proxy_async();
       mbar_arrive(&sh.conv[slot]);
-      if (threadIdx.x == 320) PROF_ADD(1, pc1);
+      FF_CLOCK_ADD(threadIdx.x == 320, P.mode * 16 + 1, pc1);
     }
   } else if (LO8 && warp >= 10) {
     // ------------------------------------------------------------------ lo bytes -> bf16 lo operand
@@ -376,11 +369,11 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     bool ok = true;
     for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
       const int slot = it % NSTAGE;
-      PROF_T0(pc0);
+      FF_CLOCK(pc0);
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[slot], (it / NSTAGE) & 1, abort_flag));
-      if (threadIdx.x == 320) PROF_ADD(0, pc0);
+      FF_CLOCK_ADD(threadIdx.x == 320, P.mode * 16 + 0, pc0);
       if (!ok) break;
-      PROF_T0(pc1);
+      FF_CLOCK(pc1);
       uint8_t* base = sData + slot * STAGE_BYTES;
 #pragma unroll 1
       for (int r = r0; r < TILE_ROWS; r += 128) {
@@ -413,7 +406,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       }
       fence_proxy_async();
       mbar_arrive(&sh.conv[slot]);
-      if (threadIdx.x == 320) PROF_ADD(1, pc1);
+      FF_CLOCK_ADD(threadIdx.x == 320, P.mode * 16 + 1, pc1);
     }
   } else {
     const int quarter = warp & 3;
@@ -452,12 +445,12 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
       const int s = P.reverse ? total_tiles - 1 - sl : sl;
       const int ab = it % NACC;
-      PROF_T0(pe0);
+      FF_CLOCK(pe0);
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc_full[ab], (it / NACC) & 1, abort_flag));
-      if (threadIdx.x == 64) PROF_ADD(4, pe0);
+      FF_CLOCK_ADD(threadIdx.x == 64, P.mode * 16 + 4, pe0);
       if (!ok) break;
       tc_fence_after();
-      PROF_T0(pe1);
+      FF_CLOCK(pe1);
       const int gi = (int)ff_div((unsigned)s, P.by_tiles);
       int i0, o0; tile_origin(P, (unsigned)s - (unsigned)gi * tiles_per_th, i0, o0);
       const int th = P.group_start + gi;
@@ -526,11 +519,11 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       const unsigned nonlow_rows = __ballot_sync(0xffffffffu, band > 0), mid_rows = __ballot_sync(0xffffffffu, band == 1);
       // both 32-channel chunks of the row at once; the accumulator buffer is free as soon as they are read
       uint32_t rr2[NQ][32];
-      PROF_T0(pl);
+      FF_CLOCK(pl);
 #pragma unroll
       for (int qi = 0; qi < NQ; ++qi) tmem_ld32(tm + lane_addr + COL_ACC + ab * 128 + (q_lo + qi) * 32, rr2[qi]);
       tmem_wait_ld();
-      if (threadIdx.x == 64) { PROF_ADD(8, pl); PROF_ADD(9, pe1); }
+      FF_CLOCK_ADD(threadIdx.x == 64, P.mode * 16 + 8, pl);
       tc_fence_before();
       mbar_arrive(&sh.acc_empty[ab]);
 #pragma unroll
@@ -605,10 +598,10 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
           uint8_t* st_lo = sh.stage[ew][1];
           if (tma_out) {
             // the previous store of this warp must have read the staging area
-            PROF_T0(pw);
+            FF_CLOCK(pw);
             if (lane == 0) bulk_wait_read0();
             __syncwarp();
-            if (threadIdx.x == 64) PROF_ADD(7, pw);
+            FF_CLOCK_ADD(threadIdx.x == 64, P.mode * 16 + 7, pw);
           }
           // 16-byte chunk i of row `lane` at chunk position i ^ (lane / 2 % 4): the 64-byte swizzle
 #pragma unroll
@@ -622,10 +615,10 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
             *(uint4*)(st_lo + lane * 32 + 16) = make_uint4(lo[4], lo[5], lo[6], lo[7]);
           }
           if (tma_out) {
-            PROF_T0(pf);
+            FF_CLOCK(pf);
             fence_proxy_async();
             __syncwarp();
-            if (threadIdx.x == 64) PROF_ADD(10, pf);
+            FF_CLOCK_ADD(threadIdx.x == 64, P.mode * 16 + 10, pf);
             if (lane == 0) {
               tma_store_5d(st_hi, &map_oh, q * 32, i0 + (seq ? 0 : l0), a0, o0 + (seq ? l0 : 0), out_slice);
               if (want_lo) tma_store_5d(st_lo, &map_ol, q * 32, i0 + (seq ? 0 : l0), a0, o0 + (seq ? l0 : 0), out_slice);
@@ -669,7 +662,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
           }
         }
       }
-      if (threadIdx.x == 64) PROF_ADD(5, pe1);
+      FF_CLOCK_ADD(threadIdx.x == 64, P.mode * 16 + 5, pe1);
     }
     if (split && P.energy) {
       // the CTA's last sample: the warp's sums into its staging area ([row parity][band][channel of the half]),
@@ -775,16 +768,6 @@ cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1
   p->launches += 1;
   return cudaSuccess;
 }
-
-#ifdef FF_DCT_PROF
-}  // namespace
-extern "C" void ff_debug_dct_prof(unsigned long long* out64, int reset) {
-  cudaDeviceSynchronize();
-  cudaMemcpyFromSymbol(out64, g_dct_prof, sizeof(unsigned long long) * 128);
-  if (reset) { unsigned long long z[128] = {}; cudaMemcpyToSymbol(g_dct_prof, z, sizeof(z)); }
-}
-namespace {
-#endif
 
 }  // namespace
 
@@ -930,3 +913,5 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
   P.mode = MODE_LAST; P.out_lo8 = 0; P.reverse = 1; P.axis = 2; P.image = matrix_image(p, 2, 1);
   return launch_pass(p, mah, mal, mal, mout, mout, P, form, st);
 }
+
+FF_CLOCKS_READ(transform_pass)

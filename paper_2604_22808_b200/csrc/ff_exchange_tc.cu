@@ -23,11 +23,12 @@
 // about 16 bits: the summary logits of a band with large low-frequency content reach O(100).
 // The low band (fp32, a few hundred tokens) has a kernel of its own (ff_summary.cu).
 //
-// Bound by the chain of these steps between the warps of a tile and by its row-scattered stores (without them the launch
-// takes half the time); 64K tokens, 24 heads: 0.28 ms = 3.6 TB/s.  1M tokens (96 keys): 2.2 -> 1.55 ms per 8 heads since
+// Bound by the store warps (5800 of 9700 cycles a tile; the rest they wait, the softmax takes 1500): 64K tokens, 24 heads
+// 248 us = 4.1 TB/s; without the row-scattered stores to global memory 181 us, without all of the store warps' work 105.  1M tokens (96 keys): 2.2 -> 1.55 ms per 8 heads since
 // the residual is read four lanes to a token (it was one lane to a token) and own-band chunks are skipped.
 #include <cuda.h>
 
+#include "ff_clocks.cuh"
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
 #include "ff_three_byte.cuh"
@@ -57,15 +58,6 @@ struct XParams {
   const __nv_bfloat16* src[4];   // y_mid, v~_mid, y_high, v~_high: bases of the buffers the four maps cover
   int* status;
 };
-
-#ifdef FF_X_PROF
-__device__ unsigned long long g_x_prof[16];
-#define XPROF_T0(v) const long long v = clock64()
-#define XPROF_ADD(i, v) atomicAdd(&g_x_prof[i], (unsigned long long)(clock64() - (v)))
-#else
-#define XPROF_T0(v)
-#define XPROF_ADD(i, v)
-#endif
 
 // per store warp: 32 channels of 32 tokens, 64 bytes of hi and 32 of lo each, or in fp32
 __host__ __device__ constexpr int x_stage_bytes(bool reread) { return reread ? 32 * 128 : 32 * 96; }
@@ -169,9 +161,9 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         const CUtensorMap* map = x.band == 1 ? (exec ? &map_y_mid : &map_v_mid) : (exec ? &map_y_high : &map_v_high);
         const int slice = exec ? x.bh : 2 * dm.BH + x.bh;
         const int slot = n % YB;
-        XPROF_T0(x0);
+        FF_CLOCK(x0);
         if (n >= YB) ok = mbar_wait(&sh.y_empty[slot], ((n / YB) - 1) & 1, abort_flag);
-        XPROF_ADD(0, x0);
+        FF_CLOCK_ADD(lane == 0, 0, x0);
         if (!ok) break;
         mbar_arrive_expect_tx(&sh.y_full[slot], XT * XD * 2);
         tma_load_3d(sY + slot * X_TILE_BYTES, map, &sh.y_full[slot], 0, x.tile * XT, slice);
@@ -202,15 +194,15 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
       // S = Y (Zhi + Zlo)^T of the CTA's tile n, K = head_dim
       auto scores = [&](int n, const XItem& x) -> bool {
         if (x.bh != prev_bh) {                            // the head's summaries have arrived
-          XPROF_T0(x4);
+          FF_CLOCK(x4);
           if (!mbar_wait_warp(&sh.z_ready, zc & 1, abort_flag)) return false;
-          XPROF_ADD(4, x4);
+          FF_CLOCK_ADD(lane == 0, 4, x4);
           ++zc; prev_bh = x.bh;
         }
         const int slot = n % YB;
-        XPROF_T0(x1);
+        FF_CLOCK(x1);
         if (!mbar_wait_warp(&sh.y_full[slot], (n / YB) & 1, abort_flag)) return false;
-        XPROF_ADD(1, x1);
+        FF_CLOCK_ADD(lane == 0, 1, x1);
         tc_fence_after();
         const uint64_t y = y_desc + (uint64_t)(slot * (X_TILE_BYTES >> 4));
         const uint32_t s_tm = tmem + (SB == 2 ? (n & 1) * 64 : 0);
@@ -234,12 +226,12 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         x_next(next, tm_tiles, th_tiles);
         const bool ahead = SB == 2 && more && next.bh == x.bh;
         if (ahead) ok = scores(n + 1, next);
-        XPROF_T0(x2);
+        FF_CLOCK(x2);
         if (ok) ok = mbar_wait_warp(&sh.p_full[n & 1], (n >> 1) & 1, abort_flag);
-        XPROF_ADD(2, x2);
-        XPROF_T0(x3);
+        FF_CLOCK_ADD(lane == 0, 2, x2);
+        FF_CLOCK(x3);
         if (ok && n >= 1) ok = mbar_wait_warp(&sh.d_empty, (n - 1) & 1, abort_flag);
-        XPROF_ADD(3, x3);
+        FF_CLOCK_ADD(lane == 0, 3, x3);
         if (!ok) break;
         tc_fence_after();
         const uint32_t p_tm = tmem + (SB == 2 ? (n & 1) * 64 : 0);
@@ -263,7 +255,6 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
     // ------------------------------------------------------------------ softmax warps
     const int quarter = warp & 3;
     const int row = quarter * 32 + lane;
-    const int tid = row;                                  // 0..127 among the softmax threads
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const float sl2 = rsqrtf((float)XD) * 1.4426950408889634f;
     bool ok = true;
@@ -271,11 +262,11 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
     XItem x = x_decode(P.h0, it0, tm_tiles, th_tiles);
     for (int it = it0; it < it1 && ok; ++it, ++n, x_next(x, tm_tiles, th_tiles)) {
       // ---- softmax over the 2m summaries of the other bands
-      XPROF_T0(x6);
+      FF_CLOCK(x6);
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.s_full[n & 1], (n >> 1) & 1, abort_flag));
-      if (tid == 0) XPROF_ADD(6, x6);
+      FF_CLOCK_ADD(row == 0, 6, x6);
       if (!ok) break;
-      XPROF_T0(x7);
+      FF_CLOCK(x7);
       tc_fence_after();
       const uint32_t s_tm = tmem + lane_addr + (SB == 2 ? (n & 1) * 64 : 0);
       const uint32_t* masks = sh.keys[x.band - 1];
@@ -334,7 +325,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
       tmem_wait_st();
       tc_fence_before();
       mbar_arrive(&sh.p_full[n & 1]);
-      if (tid == 0) XPROF_ADD(7, x7);
+      FF_CLOCK_ADD(row == 0, 7, x7);
     }
   } else {
     // ------------------------------------------------------------------ store warps
@@ -347,7 +338,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
     for (int it = it0; it < it1 && ok; ++it, ++n, x_next(x, tm_tiles, th_tiles)) {
       const long long n_band = x.band == 1 ? dm.Nmid : dm.Nhigh;
       // ---- where the lane's tokens (8 i + r8 of the warp's) come from and go: looked up before the wait
-      XPROF_T0(x14);
+      FF_CLOCK(x14);
       const int* pos = x.band == 1 ? P.pos_mid : P.pos_high;
       if (!REREAD) {
         const long long p = (long long)x.tile * XT + quarter * 32 + lane;
@@ -364,12 +355,12 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         float* const grid_f32 = P.grid_f32 + obase + (lane & 3) * 4;
         const int slot = n % YB, row = quarter * 32 + lane;
         const uint8_t* yrow = sY + slot * X_TILE_BYTES + row * 128;
-        if (threadIdx.x == 192) XPROF_ADD(14, x14);
-        XPROF_T0(x9);
+        FF_CLOCK_ADD(threadIdx.x == 192, 14, x14);
+        FF_CLOCK(x9);
         ok = __all_sync(0xffffffffu, mbar_wait(&sh.d_full, n & 1, abort_flag));
-        if (threadIdx.x == 192) XPROF_ADD(9, x9);
+        FF_CLOCK_ADD(threadIdx.x == 192, 9, x9);
         if (!ok) break;
-        XPROF_T0(x10);
+        FF_CLOCK(x10);
         tc_fence_after();
         const float2 s2 = make_float2(sh.inv[n & 3][row], sh.inv[n & 3][row]);
 #pragma unroll 4
@@ -407,44 +398,44 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
               }
               __syncwarp();
             }
-            continue;
-          }
+          } else {
 #pragma unroll
-          for (int v = 0; v < 4; ++v) {                    // 8 channels: 16 bytes of the swizzled token row
-            const int c = q * 4 + v;
-            const uint4 yv = *(const uint4*)(yrow + (c >> 3) * X_HALF + (((c & 7) ^ (row & 7)) << 4));
-            const uint32_t yw[4] = {yv.x, yv.y, yv.z, yv.w};
-            uint32_t hi[4], u[8];
+            for (int v = 0; v < 4; ++v) {                    // 8 channels: 16 bytes of the swizzled token row
+              const int c = q * 4 + v;
+              const uint4 yv = *(const uint4*)(yrow + (c >> 3) * X_HALF + (((c & 7) ^ (row & 7)) << 4));
+              const uint32_t yw[4] = {yv.x, yv.y, yv.z, yv.w};
+              uint32_t hi[4], u[8];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float2 d = make_float2(__uint_as_float(r[8 * v + 2 * k]), __uint_as_float(r[8 * v + 2 * k + 1]));
-              const float2 w = __ffma2_rn(d, s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
-              u[2 * k] = __float_as_uint(w.x) + FF_HALF24;
-              u[2 * k + 1] = __float_as_uint(w.y) + FF_HALF24;
-              hi[k] = ff_hi2(u[2 * k], u[2 * k + 1]);
+              for (int k = 0; k < 4; ++k) {
+                const float2 d = make_float2(__uint_as_float(r[8 * v + 2 * k]), __uint_as_float(r[8 * v + 2 * k + 1]));
+                const float2 w = __ffma2_rn(d, s2, make_float2(__uint_as_float(yw[k] << 16), __uint_as_float(yw[k] & 0xffff0000u)));
+                u[2 * k] = __float_as_uint(w.x) + FF_HALF24;
+                u[2 * k + 1] = __float_as_uint(w.y) + FF_HALF24;
+                hi[k] = ff_hi2(u[2 * k], u[2 * k + 1]);
+              }
+              *(uint4*)(st + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+              // (lo: 32 bytes per row, 8-byte pieces XOR-swizzled with row / 4)
+              *(uint2*)(st + 2048 + lane * 32 + ((v ^ ((lane >> 2) & 3)) << 3)) =
+                  make_uint2(ff_lo4(u[0], u[1], u[2], u[3]), ff_lo4(u[4], u[5], u[6], u[7]));
             }
-            *(uint4*)(st + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-            // (lo: 32 bytes per row, 8-byte pieces XOR-swizzled with row / 4)
-            *(uint2*)(st + 2048 + lane * 32 + ((v ^ ((lane >> 2) & 3)) << 3)) =
-                make_uint2(ff_lo4(u[0], u[1], u[2], u[3]), ff_lo4(u[4], u[5], u[6], u[7]));
-          }
-          // a NaN in the token or in a summary is in every score of the row: all of it is NaN (a branch, because a register
-          // for the half that is added above spills)
-          if (s2.x != s2.x)
-            for (int v = 0; v < 4; ++v) *(uint4*)(st + lane * 64 + v * 16) = make_uint4(0x7fff7fff, 0x7fff7fff, 0x7fff7fff, 0x7fff7fff);
-          if (q == XD / 32 - 1) mbar_arrive(&sh.y_empty[slot]);
-          __syncwarp();
+            // a NaN in the token or in a summary is in every score of the row: all of it is NaN (a branch, because a register
+            // for the half that is added above spills)
+            if (s2.x != s2.x)
+              for (int v = 0; v < 4; ++v) *(uint4*)(st + lane * 64 + v * 16) = make_uint4(0x7fff7fff, 0x7fff7fff, 0x7fff7fff, 0x7fff7fff);
+            if (q == XD / 32 - 1) mbar_arrive(&sh.y_empty[slot]);
+            __syncwarp();
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int t = 8 * i + (lane >> 2), piece = lane & 3;
-            if (out[i] >= 0) {
-              *(uint4*)(grid_hi + out[i] + q * 32) = *(const uint4*)(st + t * 64 + ((piece ^ ((t >> 1) & 3)) << 4));
-              *(uint2*)(grid_lo + out[i] + q * 32) = *(const uint2*)(st + 2048 + t * 32 + ((piece ^ ((t >> 2) & 3)) << 3));
+            for (int i = 0; i < 4; ++i) {
+              const int t = 8 * i + (lane >> 2), piece = lane & 3;
+              if (out[i] >= 0) {
+                *(uint4*)(grid_hi + out[i] + q * 32) = *(const uint4*)(st + t * 64 + ((piece ^ ((t >> 1) & 3)) << 4));
+                *(uint2*)(grid_lo + out[i] + q * 32) = *(const uint2*)(st + 2048 + t * 32 + ((piece ^ ((t >> 2) & 3)) << 3));
+              }
             }
+            __syncwarp();
           }
-          __syncwarp();
         }
-        if (threadIdx.x == 192) XPROF_ADD(10, x10);
+        FF_CLOCK_ADD(threadIdx.x == 192, 10, x10);
         continue;
       }
       const int piece = lane & 3, r8 = lane >> 2;          // a lane's 8 channels of 32 and its token of eight, when storing
@@ -468,12 +459,12 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         out[i] = f * XD;
         yv[i] = f >= 0 ? __ldg((const uint4*)(yrow + 8 * i * XD)) : make_uint4(0, 0, 0, 0);
       }
-      if (threadIdx.x == 192) XPROF_ADD(14, x14);
-      XPROF_T0(x9);
+      FF_CLOCK_ADD(threadIdx.x == 192, 14, x14);
+      FF_CLOCK(x9);
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.d_full, n & 1, abort_flag));
-      if (threadIdx.x == 192) XPROF_ADD(9, x9);
+      FF_CLOCK_ADD(threadIdx.x == 192, 9, x9);
       if (!ok) break;
-      XPROF_T0(x10);
+      FF_CLOCK(x10);
       tc_fence_after();
       const float* inv = sh.inv[n & 3] + quarter * 32 + r8;
 #pragma unroll 1
@@ -521,7 +512,7 @@ exchange_tc_kernel(const __grid_constant__ CUtensorMap map_y_mid, const __grid_c
         }
         __syncwarp();
       }
-      if (threadIdx.x == 192) XPROF_ADD(10, x10);
+      FF_CLOCK_ADD(threadIdx.x == 192, 10, x10);
     }
   }
 
@@ -549,14 +540,6 @@ bool encode_rows_map(CUtensorMap* map, void* base, long long rows, int slices, i
 }
 
 }  // namespace
-
-#ifdef FF_X_PROF
-extern "C" void ff_debug_x_prof(unsigned long long* out16, int reset) {
-  cudaDeviceSynchronize();
-  cudaMemcpyFromSymbol(out16, g_x_prof, sizeof(unsigned long long) * 16);
-  if (reset) { unsigned long long z[16] = {}; cudaMemcpyToSymbol(g_x_prof, z, sizeof(z)); }
-}
-#endif
 
 bool ffk_exchange_tc_supported(const FFDims& dm) {
   return !dm.fp32 && (dm.d == 128 || dm.d == 64) && dm.m >= 1 && dm.m <= 32 && dm.N < (1LL << 31);
@@ -639,3 +622,5 @@ cudaError_t ffk_exchange_tc(ff_plan* p, int h0, int g, void* grid_hi, void* grid
   p->launches += 1;
   return ff_launch(x_kernel(dm), dim3(grid), dim3(X_THREADS), smem, st, m0, m1, m2, m3, P);
 }
+
+FF_CLOCKS_READ(exchange)
