@@ -159,6 +159,7 @@ ff_status_t ff_route(ff_plan_t *plan, const void *Q, const void *K, const void *
 /* The attention forward ("Separable spectral decomposition" .. "Reconstruction").
  *   alloc_dev   device, [batch*heads] band masks (any subset of LOW|MID|HIGH per head), or
  *               NULL to route internally from `timestep` (host, [batch]) as ff_route does
+ *               (the values are taken during the call: a captured call keeps them in every replay)
  *   out         device, same shape and type as Q
  * Errors found on the host are returned at once; a device-side FF_ERR_TIMEOUT is reported by
  * ff_plan_device_status after a synchronisation. */

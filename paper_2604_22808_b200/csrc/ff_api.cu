@@ -417,8 +417,7 @@ static ff_status_t transform_and_route(ff_plan* p, const void* Q, const void* K,
   if (route) {
     if (!p->has_router) return fail(p, FF_ERR_NOT_ROUTED, "the plan was created without router weights%s");
     if (!timestep) return fail(p, FF_ERR_NOT_ROUTED, "neither an allocation nor a timestep was given%s");
-    if (p->dm.B > FF_TS_INLINE)
-      FF_CUDA(p, cudaMemcpyAsync(p->buf.timestep, timestep, sizeof(float) * p->dm.B, cudaMemcpyHostToDevice, st));
+    if (p->dm.B > FF_TS_INLINE) FF_CUDA(p, ffk_set_timesteps(p, timestep, st));
   }
   const bool tc_transform = p->dct_tc_ok && !(p->attn_impl & 2);
   // (the transform's first launch clears the energies; the tensor-core passes sum those of the mid and high bands)

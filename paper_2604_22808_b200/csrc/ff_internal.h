@@ -246,6 +246,7 @@ cudaError_t ffk_proj_init();
 cudaError_t ffk_stats_init(const FFDims& dm);
 cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, const void* V, bool want_energy, cudaStream_t st);
 // ---- pooling, band statistics, router, worklist (ff_stats.cu) ---------------------------------------
+cudaError_t ffk_set_timesteps(ff_plan* p, const float* host, cudaStream_t st);     // (more than FF_TS_INLINE samples)
 cudaError_t ffk_band_stats(ff_plan* p, const uint8_t* alloc_in, const float* timestep_host, bool bands_summed, cudaStream_t st);
 cudaError_t ffk_attention_simt(ff_plan* p, int band_bits, cudaStream_t st);   // band_bits: which bands to run
 // ---- tensor-core attention (ff_attn_tc.cu) -------------------------------------------------------

@@ -208,6 +208,14 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
   if (P.work && threadIdx.x < 32) build_worklist(dm, P.alloc, P.low_on, P.work);
 }
 
+// More timesteps than fit the statistics' arguments, in launches of their own: a copy from the caller's memory would be
+// read again when a captured call is replayed.
+struct TimestepChunk { float v[256]; };
+__global__ void set_timesteps_kernel(const __grid_constant__ TimestepChunk c, float* dst, int n) {
+  ff_pdl_wait();
+  if ((int)threadIdx.x < n) dst[threadIdx.x] = c.v[threadIdx.x];
+}
+
 // Shared memory of a block: a row of channels per thread group for the sums, and the router's input and hidden layer.
 size_t sums_bytes(const FFDims& dm) { return (size_t)(ST_THREADS / (dm.d / 4)) * dm.d * sizeof(float); }
 size_t router_bytes(const FFDims& dm) { return (size_t)(3 * dm.d + dm.dt + dm.hid) * sizeof(float); }
@@ -220,6 +228,18 @@ cudaError_t ffk_stats_init(const FFDims& dm) {
   if (need <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(dm.fp32 ? band_stats_kernel<float> : band_stats_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)(need < most ? need : most));
+}
+
+cudaError_t ffk_set_timesteps(ff_plan* p, const float* host, cudaStream_t st) {
+  for (int b0 = 0; b0 < p->dm.B; b0 += 256) {
+    TimestepChunk c;
+    const int n = p->dm.B - b0 < 256 ? p->dm.B - b0 : 256;
+    memcpy(c.v, host + b0, n * sizeof(float));
+    p->launches += 1;
+    const cudaError_t e = ff_launch(set_timesteps_kernel, dim3(1), dim3(256), 0, st, c, p->buf.timestep + b0, n);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // Pooling, statistics, router or copy of the caller's masks, worklist.  `bands_summed`: the transform's epilogue has

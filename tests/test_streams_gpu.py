@@ -11,6 +11,7 @@ import harness as Hn
 pytestmark = pytest.mark.gpu
 
 CONFIGS = [C.TINY, C.R64K.scaled("two_axes", heads=3),
+           C.R64K.scaled("cta_pairs", H=16, W=128, low_cut=(2, 2, 16), mid_cut=(10, 10, 80), heads=3),
            C.R64K.scaled("ragged", T=5, H=33, W=20, low_cut=(1, 4, 2), mid_cut=(3, 20, 12), heads=3)]
 
 
@@ -116,3 +117,35 @@ def test_new_buffers_in_every_call(cfg):
             host = [src[i].cpu() for i in order]
             plan.forward_host(*host, torch.empty_like(host[0]), alloc_host=alloc.cpu().numpy())
     plan.destroy()
+
+
+@pytest.mark.parametrize("batch", [32, 33, 300])
+def test_captured_call_keeps_its_timesteps(batch):
+    """Up to 32 timesteps travel as arguments of one launch, more in launches of their own; the caller's array may change or
+    go once the call has returned."""
+    import torch
+    from paper_2604_22808_b200 import binding as B
+    cfg = C.TINY.scaled("many", batch=batch)
+    weights = I.router_weights(cfg)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    q, k, v = (torch.randn((batch, cfg.heads, cfg.T, cfg.H, cfg.W, cfg.head_dim), generator=gen, device="cuda") for _ in range(3))
+    ts = np.linspace(0, 999, batch).astype(np.float32)
+    plan, one = B.Plan(cfg, weights), B.Plan(C.TINY, weights)
+    want = torch.cat([one.forward(*(x[i:i + 1] for x in (q, k, v)), torch.empty_like(q[:1]), timesteps=ts[i:i + 1]) for i in range(batch)])
+    out = torch.empty_like(q)
+    stream = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    gone = ts.copy()
+    with torch.cuda.graph(graph, stream=stream):
+        plan.forward(q, k, v, out, timesteps=gone)
+    gone[:] = -1.0
+    for _ in range(2):
+        out.zero_()
+        plan.tap(B.TAP_PI).zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert (out - want).abs().max() <= 1e-5 * want.abs().max()     # (energies are summed by atomics)
+    del graph
+    plan.destroy()
+    one.destroy()
