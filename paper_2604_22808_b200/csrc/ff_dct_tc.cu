@@ -16,11 +16,11 @@
 // values (low-frequency content, the constant offset the exchange adds to a whole band), so a
 // single bf16 rounding between passes would not meet the output tolerance.
 //
-// Three-byte intermediates.  Where the three axes run as separate passes, the pair written by the first forward
-// pass and the pairs between the inverse passes are stored (planes above 2048 positions) as the fp32 value
+// Three-byte intermediates.  Where the three axes run as separate passes (planes above 2048 positions, or asked for), the
+// pair written by the first forward pass and the pairs between the inverse passes are stored as the fp32 value
 // rounded to 24 bits: the upper 16 bits (a bf16 by truncation) in the hi grid and the next 8 bits in a byte grid.  hi
 // and (value - hi) are both exact bf16 operands, together they carry 16 significant bits, one less than a bf16 hi/lo
-// pair, and a pass moves 3 instead of 4 bytes per value.  A launch whose input has the byte form (template parameter LO8) runs four more
+// pair, and a pass moves 3 instead of 4 bytes per value.  A launch whose input has the byte form (FORM_BYTES) runs four more
 // warps that expand the bytes of every arriving tile to the bf16 lo operand in shared memory before the MMAs
 // read it (128 channels: in place, the bytes of a row arrive inside the row's own bf16 space).  The expansion
 // competes with the epilogue for issue slots; measured per launch at 1M tokens (3 tensor-heads): a middle pass
@@ -31,9 +31,9 @@
 // Any grid.  A line of any length up to 128 fits a tile, so the passes run on every grid: floor(128 / n) lines
 // per tile, the left-over rows zero in the matrix and in shared memory, partial last tiles filled with zeros and
 // clipped by the copies.  Grids with an axis other than 16, 32, 64 or 128 ran on fp32 kernels, and the precision stays
-// that of fp32 numbers: the passes hand on fp32 grids (forms EXACT1 and EXACT), matrix and data are three bf16 parts
+// that of fp32 numbers: the passes hand on fp32 grids (FORM_EXACT1 and FORM_EXACT), matrix and data are three bf16 parts
 // each, which hold all 24 bits, and six of their nine products are summed, the small ones first (the others are below
-// 2^-24).  The parts of the data are made by the four warps that expand bytes in form BYTES: truncations, so that they
+// 2^-24).  The parts of the data are made by the four warps that expand bytes in FORM_BYTES: truncations, so that they
 // add up to the value.  A pass moves 4 bytes per value like a bf16 pair, and 48 instructions a tile keep the tensor core
 // below the copies' time.  21 x 45 x 80 tokens, 16 heads: forward transform 1.94 ms and inverse with the exchange 0.94
 // (fp32 kernels: 4.46 and 2.83; 16-bit intermediates: 1.54 and 0.67); the passes run at 4.1 - 5.9 TB/s, the later ones
@@ -42,19 +42,21 @@
 // Order of the tiles.  A pass that reads what the previous launch wrote walks its tiles from the last to the
 // first (P.reverse), the next one forward again: the end of the previous launch's output is still in L2.
 //
-//   warp 0      TMA producer (ring of 3-7 stages)
-//   warp 1      tcgen05.mma issuer (A from tensor memory), 3 accumulator buffers of 128 TMEM columns
-//   warps 2..9  epilogue: tcgen05.ld, convert to hi/lo bf16, store; a thread owns one output position
+//   warp 0      TMA producer (ring of 2-8 stages)
+//   warp 1      tcgen05.mma issuer (A from tensor memory), 3 accumulator buffers of 128 TMEM columns (2 beside three
+//               matrix parts)
+//   warps 2..9  epilogue: tcgen05.ld, convert to the output's form, store; a thread owns one output position
+//   warps 10..13  (FORM_BYTES, FORM_EXACT) operands of an arriving tile
 // Output path (FIRST, MIDDLE, LAST): an epilogue warp's 32 rows are 32 grid positions that form a
 // box of the grid, so the warp writes 32 channels of them (64 bytes per row, 64-byte swizzle, no
 // bank conflicts) into its own staging area and one lane sends them out with a tensor store; the
 // area is reused when that store has read it.  SPLIT scatters rows to band positions: staged the
 // same way, then stored by all lanes with four lanes per 64-byte row piece.
-// Modes: FIRST  caller's Q/K/V -> hi/lo intermediate
-//        MIDDLE hi/lo intermediate -> hi/lo intermediate
+// Modes: FIRST  caller's Q/K/V -> intermediate
+//        MIDDLE intermediate -> intermediate
 //        SPLIT  intermediate -> band-major coefficient buffers (rank evaluated in registers): mid and
-//               high band in bf16, low band in fp32 straight from the accumulators (the hi/lo
-//               intermediates carry about 16 bits); the router's mid and high band energies are
+//               high band in bf16, low band in fp32 straight from the accumulators (hi/lo
+//               intermediates carry 16 or 17 bits); the router's mid and high band energies are
 //               accumulated here from the stored bf16 coefficients (the low band's, few values per
 //               channel, by the band-statistics kernel from the fp32 coefficients)
 //        LAST   intermediate -> the caller's out tensor

@@ -13,19 +13,21 @@
 //           skipped; P (unnormalised) goes back to TMEM as bf16 hi + lo over the 16 scores it comes from, the row sum
 //           to the store warps
 //   MMA 2   D[128 x 128] = P Z  (A = P from tensor memory, B = the same Z image read MN-major)
-//   store   Y + D / row sum in the three-byte form the inverse passes read (the value rounded to 24 bits: a grid of its
-//           upper 16 bits and a grid of the next byte).  A warp has 32 tokens, one per lane; it turns 32 channels of
-//           them in shared memory, so that four lanes write 64 (hi) and 32 (lo) contiguous bytes of a token.  With more
-//           than 64 keys a second token tile no longer fits: the tile then goes back to the producer as soon as the
-//           scores are done, the update is turned as fp32 and the tokens are read again from global memory, four lanes
-//           64 contiguous bytes.
+//   store   Y + D / row sum in the form the inverse passes read: three bytes (the value rounded to 24 bits: a grid of its
+//           upper 16 bits and a grid of the next byte), or fp32 (template parameter F32).  A warp has 32 tokens, one per
+//           lane; it turns 32 channels of them in shared memory, so that four lanes write 64 (hi) and 32 (lo) contiguous
+//           bytes of a token.  With more than 64 keys a second token tile no longer fits: the tile then goes back to the
+//           producer as soon as the scores are done, the update is turned as fp32 and the tokens are read again from
+//           global memory, four lanes 64 contiguous bytes.
 // Z and P are split into bf16 hi + lo parts (Y is exact bf16), so the logits and the update carry
-// about 16 bits: the summary logits of a band with large low-frequency content reach O(100).
+// about 16 bits: the summary logits of a band with large low-frequency content reach O(100).  (Grids whose values are fp32
+// up to here had an fp32 exchange before: the output's error against fp64 is the same to 2e-5 of itself, 1.660e-3.)
 // The low band (fp32, a few hundred tokens) has a kernel of its own (ff_summary.cu).
 //
 // Bound by the store warps (5800 of 9700 cycles a tile; the rest they wait, the softmax takes 1500): 64K tokens, 24 heads
-// 248 us = 4.1 TB/s; without the row-scattered stores to global memory 181 us, without all of the store warps' work 105.  1M tokens (96 keys): 2.2 -> 1.55 ms per 8 heads since
-// the residual is read four lanes to a token (it was one lane to a token) and own-band chunks are skipped.
+// 248 us = 4.1 TB/s; without the row-scattered stores to global memory 181 us, without all of the store warps' work 105.
+// 1M tokens (96 keys): 2.2 -> 1.55 ms per 8 heads since the residual is read four lanes to a token (it was one lane to a
+// token) and own-band chunks are skipped.
 #include <cuda.h>
 
 #include "ff_clocks.cuh"
