@@ -255,7 +255,7 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
         !(ffk_dct2_build_image(p, a, 0, C.data(), n[a]) && ffk_dct2_build_image(p, a, 1, Ct.data(), n[a])))
       s = fail(p, FF_ERR_CUDA, "could not upload the transform matrix images%s");
   }
-  p->dct2_ok = s == FF_OK && p->dct2_images && ffk_dct2_supported(p->dm, &p->dct2_axis2, &p->dct2_pair);
+  p->dct2_ok = s == FF_OK && p->dct2_images && ffk_dct2_supported(p->dm, &p->dct2_axis2, &p->dct2_chunk);
   const size_t d = c->head_dim, hid = c->router_hidden, nin = 3 * d + c->t_embed_dim;
   if (s == FF_OK && w && w->W1 && w->b1 && w->W2 && w->b2) {
     s = upload(p, &p->W1, w->W1, hid * nin);
@@ -348,7 +348,7 @@ extern "C" ff_status_t ff_plan_set_attention_impl(ff_plan_t* p, int32_t impl) {
 extern "C" ff_status_t ff_plan_kernel_info(const ff_plan_t* p, int32_t info[4]) {
   if (!p || !info) return fail(nullptr, FF_ERR_INVALID_ARG, "plan or info is NULL%s");
   const bool fused = p->dct_tc_ok && p->dct2_ok && !(p->attn_impl & 6);
-  info[0] = fused ? 1 : 0; info[1] = fused ? (p->dct2_pair ? 2 : 1) : 0;
+  info[0] = fused ? 1 : 0; info[1] = fused ? 1 : 0;
   info[2] = (p->tc_ok && !(p->attn_impl & 1)) ? 1 : 0; info[3] = (info[2] && p->low_tc_ok) ? 1 : 0;
   return FF_OK;
 }

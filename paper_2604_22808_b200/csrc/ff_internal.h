@@ -89,20 +89,14 @@ __device__ __forceinline__ void ff_pdl_join() { asm volatile("griddepcontrol.wai
 
 // (an event wait in the stream before the launch, the library's own or the caller's, holds the whole kernel back)
 template <class... K, class... A>
-inline cudaError_t ff_launch_cluster(void (*kernel)(K...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+inline cudaError_t ff_launch(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[2];
+  cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-  cfg.attrs = attr; cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
-}
-template <class... K, class... A>
-inline cudaError_t ff_launch(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
-  return ff_launch_cluster(kernel, 1, grid, block, smem, st, std::forward<A>(args)...);
 }
 
 __device__ __forceinline__ unsigned ff_div(unsigned n, const FFFastDiv& f) { return (__umulhi(f.m, n) + n) >> f.s; }
@@ -210,7 +204,7 @@ struct ff_plan {
   FFMapCache maps;                             // tensor maps of the transform passes, by shape
   bool dct2_ok;                                // the fused two-axis launch covers this configuration
   int dct2_axis2;                              // its second axis (1 = h, 0 = t); the remaining axis gets a pass of its own
-  bool dct2_pair;                              // two CTAs share a plane there
+  int dct2_chunk;                              // channels of its work items: 32, or 16 for the larger planes
   alignas(64) unsigned char tmap_mid[128];     // CUtensorMap over the mid-band / high-band coefficient buffers
   alignas(64) unsigned char tmap_high[128];
   alignas(64) unsigned char tmap_low[128];     // ... over the pooled low band (bf16 copy), when low_tc_ok
@@ -265,7 +259,7 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
                                      cudaStream_t st);
 cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaStream_t st);
 // ---- two axis passes in one launch, intermediate in shared memory (ff_dct2_tc.cu) --------------------
-bool ffk_dct2_supported(const FFDims& dm, int* axis2, bool* pair);
+bool ffk_dct2_supported(const FFDims& dm, int* axis2, int* chunk);
 bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat_host, int n);
 cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
                              bool clear_energy, cudaStream_t st);

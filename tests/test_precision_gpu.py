@@ -42,3 +42,28 @@ def test_pairs_between_the_axes(grid, d):
 def test_fp32_between_the_axes_of_any_other_grid(grid, d):
     assert _low_band_error(grid, d) < 4.0 * 2.0 ** -23
     assert _low_band_error(grid, d, impl=2) < 4.0 * 2.0 ** -23
+
+
+# Planes of 2048 positions go in chunks of 16 channels: every number of coefficients a phase-2 tile can hold (128 / n2 =
+# 1, 2, 4, 8), against fp64 and against the separate passes.  The latter hand on one byte-form intermediate (2^-16 of the low
+# coefficients' norm); the 16-bit taps differ where a value lies that close to the middle of two bf16 numbers, by a bf16
+# step: share 2^-8 of the values at most, 2^-8 sqrt(2^-8) = 2.5e-4 of the norm.
+@pytest.mark.parametrize("grid", [(128, 128, 16), (64, 64, 32), (32, 64, 64), (16, 32, 128)], ids=lambda g: "x".join(map(str, g)))
+@pytest.mark.parametrize("d", [64, 128])
+def test_planes_of_2048_positions(grid, d):
+    import torch
+    from paper_2604_22808_b200 import binding as B
+    low, mid = tuple(n // 8 for n in grid), tuple(n // 8 + n // 2 for n in grid)
+    cfg = C.FFConfig(name="plane", batch=1, T=grid[0], H=grid[1], W=grid[2], heads=1, head_dim=d, dtype="bf16", low_cut=low,
+                     mid_cut=mid, r=8, b=64, s=8, R=64, m=16, seed=83, timesteps=(500.0,))
+    qkv = Hn.host_inputs(cfg)
+    got = []
+    for impl in (0, 4):
+        out, plan = Hn.gpu_forward(cfg, *qkv, None, None, alloc=[7], attention_impl=impl)
+        assert plan.kernel_info()["transform_fused"] == (impl == 0)
+        got.append([plan.tap(w).double().clone() for w in (B.TAP_SPEC_LOW, B.TAP_SPEC_MID, B.TAP_SPEC_HIGH)] + [torch.as_tensor(np.asarray(out)).double()])
+        plan.destroy()
+    apart = [((a - b).norm() / b.norm()).item() for a, b in zip(*got)]
+    assert apart[0] < 2.0 ** -16 and apart[1] < 2.5e-4 and apart[2] < 2.5e-4, apart
+    assert apart[3] < 2.0 ** -8, apart
+    assert _low_band_error(grid, d) < 2.0 ** -17
