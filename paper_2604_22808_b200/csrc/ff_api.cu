@@ -217,6 +217,7 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
   if (ce == cudaSuccess) ce = ffk_exchange_tc_init(p->dm);
   if (ce == cudaSuccess) ce = ffk_dct_tc_init(p->dm);
   if (ce == cudaSuccess) ce = ffk_dct2_init();
+  if (ce == cudaSuccess) ce = ffk_dct_t16_init();
   if (ce == cudaSuccess) ce = ffk_proj_init();
   if (ce == cudaSuccess) ce = ffk_stats_init(p->dm);
   if (ce != cudaSuccess) {
@@ -249,6 +250,8 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
         C[(size_t)k * n[a] + i] = (float)v;
         Ct[(size_t)i * n[a] + k] = (float)v;
       }
+    if (a == 0 && c->T == 16)
+      for (int k = 0; k < 16; ++k) for (int i = 0; i < 8; ++i) p->t16_mat[k][i] = C[(size_t)k * 16 + i];
     s = upload(p, &p->basis[a], C.data(), C.size());
     if (s == FF_OK) s = upload(p, &p->basis_t[a], Ct.data(), Ct.size());
     if (s == FF_OK && ffk_dct_tc_supported(p->dm) &&
@@ -256,6 +259,7 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
       s = fail(p, FF_ERR_CUDA, "could not upload the transform matrix images%s");
   }
   p->dct2_ok = s == FF_OK && p->dct2_images && ffk_dct2_supported(p->dm, &p->dct2_axis2, &p->dct2_chunk);
+  p->t16 = ffk_dct_t16_supported(p);
   const size_t d = c->head_dim, hid = c->router_hidden, nin = 3 * d + c->t_embed_dim;
   if (s == FF_OK && w && w->W1 && w->b1 && w->W2 && w->b2) {
     s = upload(p, &p->W1, w->W1, hid * nin);

@@ -143,7 +143,8 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   uint8_t* sStage = smem + MAX_GPI * 2 * GROUP_B;                  // 8 phase-2 warps x (hi 2 KB, lo 2 KB), 1024-byte aligned
   uint8_t* sIn = sStage + 8 * 2 * STG_B;                           // ring: 8 groups, or 4 and behind them their lo parts
   D2Shared& sh = *(D2Shared*)(sIn + RING_B);
-  const int nslot = P.in_split ? NSTG / 2 : NSTG;
+  const int lslot = P.in_split ? 2 : 3, nslot = 1 << lslot;
+  static_assert(NSTG == 8, "ring slots");
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n1 = P.n1, n2 = P.n2;
   const int ln1 = 31 - __clz(n1);
@@ -151,8 +152,10 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
   const int lkf2 = 31 - __clz(kf2);
   const int total = P.group * P.n3 * P.nchunk;
   const int nsl = gpi <= MAX_GPI / 2 ? 2 : 1;                      // slots of the plane buffer
-  const int bt1 = P.bt1, nb1 = gpi / bt1, na1 = ACC_GROUPS / bt1;  // groups per instruction batch (N = 32 groups columns),
-  const int bt2 = P.bt2, nb2 = gpi / bt2, na2 = ACC_GROUPS / bt2;  // batches of an item, accumulator buffers
+  // groups per instruction batch (N = 32 groups columns), batches of an item, and the accumulator buffers: one, or two with
+  // batches of two (as logarithms: divisions by launch parameters would stand in front of every wait)
+  const int bt1 = P.bt1, nb1 = gpi / bt1, la1 = bt1 <= ACC_GROUPS / 2, m1 = (1 << la1) - 1;
+  const int bt2 = P.bt2, nb2 = gpi / bt2, la2 = bt2 <= ACC_GROUPS / 2, m2 = (1 << la2) - 1;
   // With an even number of batches, the first half of the phase-1 batches holds the first half
   // of the second axis, i.e. rows 0..63 of every phase-2 tile = its k-steps 0..3.  Phase 2 of the item's first
   // batch starts on those while phase 1 still works on the second half.
@@ -227,9 +230,9 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           slice = th % dm.BH;
         }
         for (int k = 0; k < gpi && ok; ++k, ++n) {
-          const int slot = n % nslot;
+          const int slot = n & (nslot - 1);
           FF_CLOCK(tp0);
-          if (n >= (unsigned)nslot) ok = mbar_wait(&sh.in_empty[slot], ((n / nslot) - 1) & 1, abort_flag);
+          if (n >= (unsigned)nslot) ok = mbar_wait(&sh.in_empty[slot], ((n >> lslot) - 1) & 1, abort_flag);
           FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 12, tp0);
           if (!ok) break;
           uint8_t* dst = sIn + slot * GROUP_B;
@@ -251,17 +254,17 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       bool ok = true;
       for (int it = cid; it < total && ok; it += ncta) {
         for (int kb = 0; kb < nb1 && ok; ++kb, ++n1b) {
-          const int ab = n1b % na1;
+          const int ab = n1b & m1;
           const unsigned nt = bt1 * n1b;                            // index of the batch's first group in the ring sequence
           FF_CLOCK(tm0);
-          for (int i = 0; i < bt1 && ok; ++i) ok = mbar_wait_warp(&sh.in_full[(nt + i) % nslot], ((nt + i) / nslot) & 1, abort_flag);
+          for (int i = 0; i < bt1 && ok; ++i) ok = mbar_wait_warp(&sh.in_full[(nt + i) & (nslot - 1)], ((nt + i) >> lslot) & 1, abort_flag);
           FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 7, tm0);
           FF_CLOCK(tm1);
-          if (ok && n1b >= (unsigned)na1) ok = mbar_wait_warp(&sh.acc1_empty[ab], ((n1b / na1) - 1) & 1, abort_flag);
+          if (ok && n1b > (unsigned)m1) ok = mbar_wait_warp(&sh.acc1_empty[ab], ((n1b >> la1) - 1) & 1, abort_flag);
           FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 8, tm1);
           if (!ok) break;
           tc_fence_after();
-          const uint32_t x0 = in_base + (uint32_t)(nt % nslot) * GROUP_B;
+          const uint32_t x0 = in_base + (uint32_t)(nt & (nslot - 1)) * GROUP_B;
           const uint64_t xh = smem_desc_rows<C>(x0, TILE_B), xl = smem_desc_rows<C>(x0 + RING_B / 2, TILE_B);
           const uint32_t d_tm = tm + COL_ACC1 + ab * bt1 * GCOLS;
           if (P.in_split) {
@@ -278,7 +281,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
               umma_ts(d_tm, tm + COL_A1L + ks * 8, xh + (uint64_t)(ks * KSTEP), idesc, 1u);
             }
           }
-          for (int i = 0; i < bt1; ++i) umma_commit(&sh.in_empty[(nt + i) % nslot]);
+          for (int i = 0; i < bt1; ++i) umma_commit(&sh.in_empty[(nt + i) & (nslot - 1)]);
           umma_commit(&sh.acc1_full[ab]);
         }
       }
@@ -294,15 +297,15 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       for (int it = cid; it < total && ok; it += ncta, ++ni) {
         // the plane's rows have landed in this CTA's buffer
         FF_CLOCK(tm2);
-        const int sl = (int)(ni % nsl);                             // the item's slot of the plane buffer
-        ok = mbar_wait_warp(half_start ? &sh.buf_half[sl] : &sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
+        const int sl = (int)(ni & (nsl - 1));                             // the item's slot of the plane buffer
+        ok = mbar_wait_warp(half_start ? &sh.buf_half[sl] : &sh.buf_full[sl], (ni >> (nsl - 1)) & 1, abort_flag);
         FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 9, tm2);
         if (!ok) break;
         fence_proxy_async();
         for (int kb = 0; kb < nb2 && ok; ++kb, ++n2b) {
-          const int ab = n2b % na2;
+          const int ab = n2b & m2;
           FF_CLOCK(tm3);
-          if (n2b >= (unsigned)na2) ok = mbar_wait_warp(&sh.acc2_empty[ab], ((n2b / na2) - 1) & 1, abort_flag);
+          if (n2b > (unsigned)m2) ok = mbar_wait_warp(&sh.acc2_empty[ab], ((n2b >> la2) - 1) & 1, abort_flag);
           FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 10, tm3);
           if (!ok) break;
           tc_fence_after();
@@ -313,7 +316,7 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
           for (int ks = 0; ks < ROWS / 16; ++ks) {
             if (ks == ROWS / 32 && kb == 0 && half_start) {          // the second half of the rows
               FF_CLOCK(tm4);
-              ok = mbar_wait_warp(&sh.buf_full[sl], (ni / nsl) & 1, abort_flag);
+              ok = mbar_wait_warp(&sh.buf_full[sl], (ni >> (nsl - 1)) & 1, abort_flag);
               FF_CLOCK_ADD(lane == 0, P.in_split * 16 + 11, tm4);
               if (!ok) break;
               fence_proxy_async();
@@ -353,21 +356,21 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
     bool ok = true;
     for (int it = cid; it < total && ok; it += ncta, ++ni) {
       FF_CLOCK(te0);
-      const int sl = (int)(ni % nsl);                         // the item's slot: free once phase 2 of item ni - nsl is done
+      const int sl = (int)(ni & (nsl - 1));                         // the item's slot: free once phase 2 of item ni - nsl is done
       if (ni >= (unsigned)nsl) {
         // (half_release: the first half of the batches writes rows phase 2 releases earlier; the rest waits below)
-        ok = mbar_wait_warp(half_release ? &sh.half_free[sl] : &sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag);
+        ok = mbar_wait_warp(half_release ? &sh.half_free[sl] : &sh.buf_free[sl], ((ni >> (nsl - 1)) - 1) & 1, abort_flag);
         if (!ok) break;
       }
       FF_CLOCK_ADD(threadIdx.x == 128, P.in_split * 16 + 1, te0);
       for (int kb = 0; kb < nb1 && ok; ++kb, ++n1b) {
         if (half_release && kb == nb1 / 2 && ni >= (unsigned)nsl) {
-          ok = mbar_wait_warp(&sh.buf_free[sl], ((ni / nsl) - 1) & 1, abort_flag);
+          ok = mbar_wait_warp(&sh.buf_free[sl], ((ni >> (nsl - 1)) - 1) & 1, abort_flag);
           if (!ok) break;
         }
-        const int ab = n1b % na1;
+        const int ab = n1b & m1;
         FF_CLOCK(te1);
-        ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc1_full[ab], (n1b / na1) & 1, abort_flag));
+        ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc1_full[ab], (n1b >> la1) & 1, abort_flag));
         if (!ok) break;
         FF_CLOCK_ADD(threadIdx.x == 128, P.in_split * 16 + 0, te1);
         FF_CLOCK(te2);
@@ -460,9 +463,9 @@ dct2_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__
       int gi, a3, chunk; decode_item(P, it, gi, a3, chunk);
       const int out_slice = P.last ? P.group_start + gi : gi;
       for (int kb = 0; kb < nb2 && ok; ++kb, ++n2b) {
-        const int ab = n2b % na2;
+        const int ab = n2b & m2;
         FF_CLOCK(te5);
-        ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc2_full[ab], (n2b / na2) & 1, abort_flag));
+        ok = __all_sync(0xffffffffu, mbar_wait(&sh.acc2_full[ab], (n2b >> la2) & 1, abort_flag));
         if (!ok) break;
         FF_CLOCK_ADD(threadIdx.x == 384, P.in_split * 16 + 3, te5);
         FF_CLOCK(te6);

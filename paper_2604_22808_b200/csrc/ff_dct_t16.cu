@@ -1,0 +1,305 @@
+// The last launch of the inverse transform ("Reconstruction") where the t axis has 16 positions: the w axis on the tensor
+// cores, t in fp32 registers.  bf16 storage, DCT-II.
+//
+// A 16 x 16 matrix is too small for the tensor core: as Mat kron I it fills an eighth of the 128 x 128 operand that
+// ff_dct2_tc.cu multiplies with, three times over for the hi/lo parts, and its input has to go from the accumulators through
+// registers and shared memory to become an operand.  Here a thread takes all 16 t coefficients of a (h, w) position and four
+// channels from the accumulators of the w axis and folds them (C[k][15 - i] = (-1)^k C[k][i]: even and odd k apart), eight
+// FMA and one addition a value, in fp32.  On long runs every launch of this path meets the board's power limit; three of six
+// tensor products and the plane's way through shared memory are energy, too.
+//
+// A work item is 16 t x 128 (h, w) positions (128/W neighbouring h) x 16 channels of a head.  A tile of 128 positions at
+// one t is the MN-major B operand (32-byte rows, 32-byte swizzle), the matrix I kron C_w the A operand in tensor memory
+// (hi and lo bf16 parts); eight tiles share one instruction (N = 128).  D holds a position per lane and (t, channel) in its
+// columns, so that nothing crosses lanes; 256 columns an item and 128 more for the first half of the next.
+//   warp 0       TMA producer (ring of twelve slots: two tiles as a hi/lo pair)
+//   warp 1       tcgen05.mma issuer; owns the tensor-memory allocation
+//   warps 2..17  epilogue: four warps per 32 lanes, four channels each; they stage rows of 16 channels together and one
+//                thread sends two t positions at a time out with tensor stores
+// Every wait is bounded.
+//
+// Bound by its rows of 32 bytes.  24 heads of 64K tokens, at 1.6 GHz under the power limit: 334 us with ff_dct2_tc.cu, 254
+// here (1.2 GB at 4.7 TB/s); six heads of 16K tokens 28 and 22 us.  The forward launch stays with ff_dct2_tc.cu: it writes a
+// hi/lo pair, and with twice as many 32-byte rows out as in it took 1130 to 1160 instead of 883 us.
+#include <cuda.h>
+
+#include "ff_clocks.cuh"
+#include "ff_internal.h"
+#include "ff_sm100.cuh"
+
+using namespace sm100;
+
+namespace {
+
+constexpr int T = 16, C = 16;                  // t positions, channels of an item
+constexpr int ROWS = 128;                      // positions of a tile
+constexpr int TILE_B = ROWS * C * 2;           // 4 KB as bf16
+constexpr int SLOT_B = 2 * TILE_B;             // two t positions
+constexpr int BATCH = 4;                       // slots of an instruction batch: N = 8 tiles of 16 channels
+constexpr int NSLOT = 12, LO_OFF = NSLOT * SLOT_B;     // ring: three batches, the hi parts, behind them their lo parts (192 KB)
+constexpr int NACC = 3;                        // accumulator buffers of 128 columns, behind the matrix (2 x 64)
+constexpr int EPI = 4, CPT = C / EPI;          // epilogue warps per 32 lanes, channels of a thread
+constexpr int THREADS = 64 + 4 * EPI * 32;
+constexpr int BOX_B = 2 * 32 * C * 2;          // 2 KB: 32 positions at two t, staged for a store
+constexpr int STAGE_B = 2 * BOX_B;             // a staging buffer
+
+struct T16Params {
+  FFDims dm;
+  const uint32_t* img;     // matrix of the w axis: hi [128][64] cells, then lo
+  float mat[T][T / 2];     // mat[k][i] = C[k][i], i < 8
+  int group, group_start;  // heads of the launch, the first one's place in the caller's tensor
+  int nchunk, nh, hpt;     // channel chunks, groups of h positions, h positions of a group (128 / W)
+  int* status;
+};
+
+struct T16Shared {
+  uint64_t full[NSLOT], empty[NSLOT], acc_full[NACC], acc_empty[NACC];
+  uint64_t stg_full[4], stg_free[4];           // per four epilogue warps
+  uint32_t tmem_base;
+  int abort_flag;
+};
+
+// Shared-memory descriptor of an MN-major operand stored as rows of 16 bf16 with the 32-byte swizzle: 8-row groups 256 bytes
+// apart, tiles of 16 channels (along N) TILE_B apart.
+__device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t smem_addr) {
+  return (uint64_t)((smem_addr & 0x3FFFF) >> 4) | (uint64_t)(TILE_B >> 4) << 16 | (uint64_t)(256 >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)6 << 61;
+}
+
+// 32 lanes x 4 columns
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&r)[4]) {
+  uint32_t v[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(taddr)
+               : "memory");
+#pragma unroll
+  for (int i = 0; i < 4; ++i) r[i] = __uint_as_float(v[i]);
+}
+__device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
+
+// A thread's channels -> eight bytes.
+__device__ __forceinline__ void stage4(uint8_t* dst, const float (&y)[CPT]) {
+  *(uint2*)dst = make_uint2(bf16_pair(__float_as_uint(y[0]), __float_as_uint(y[1])), bf16_pair(__float_as_uint(y[2]), __float_as_uint(y[3])));
+}
+
+// map_hi, map_lo: the pair of grids; map_out: the caller's tensor, box = 32 positions at two t.
+__global__ void __launch_bounds__(THREADS, 1)
+dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
+               const __grid_constant__ CUtensorMap map_out, const __grid_constant__ T16Params P) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const FFDims& dm = P.dm;
+  constexpr uint32_t COL_ACC = 128;
+  uint8_t* sIn = smem;
+  uint8_t* sStage = smem + 2 * LO_OFF;                      // four lane quarters x two buffers
+  T16Shared& sh = *(T16Shared*)(sStage + 4 * 2 * STAGE_B);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int total = P.group * P.nh * P.nchunk;
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < NSLOT; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 1); }
+    for (int i = 0; i < NACC; ++i) { mbar_init(&sh.acc_full[i], 1); mbar_init(&sh.acc_empty[i], 4 * EPI * 32); }
+    for (int i = 0; i < 4; ++i) { mbar_init(&sh.stg_full[i], EPI * 32); mbar_init(&sh.stg_free[i], 1); }
+    sh.abort_flag = 0;
+    fence_mbar_init();
+  }
+  if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tm = sh.tmem_base;
+  volatile int* abort_flag = &sh.abort_flag;
+  if (warp >= 2 && warp < 6) {
+    // the matrix into tensor memory: a thread loads the row of its lane
+    const int quarter = warp & 3, row = quarter * 32 + lane;
+    const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+#pragma unroll 1
+    for (int c0 = 0; c0 < 128; c0 += 32) {
+      const uint32_t* src = P.img + (size_t)(c0 >> 6) * FF_IMAGE_PART + (size_t)row * 64 + (c0 & 63);
+      uint32_t r[32];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint4 v = *(const uint4*)(src + 4 * i);
+        r[4 * i] = v.x; r[4 * i + 1] = v.y; r[4 * i + 2] = v.z; r[4 * i + 3] = v.w;
+      }
+      tmem_st32(tm + lane_addr + c0, r);
+    }
+    tmem_wait_st();
+  }
+  // (the next launch comes in when this one's blocks end: let in at the start, its blocks slowed the last third of this
+  // launch down, 16K tokens, six heads: 30.6 us instead of 22.3)
+  ff_pdl_join();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+
+  // Item: chunk fastest (CTAs that run side by side read neighbouring pieces of the same rows), then h, then the head.
+  if (warp == 0) {
+    if (lane == 0) {
+      tma_prefetch_desc(&map_hi); tma_prefetch_desc(&map_lo);
+      unsigned n = 0;
+      bool ok = true;
+      for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
+        const int chunk = it % P.nchunk, rest = it / P.nchunk, h0 = rest % P.nh * P.hpt, gi = rest / P.nh;
+        for (int k = 0; k < T / 2 && ok; ++k, ++n) {
+          const int slot = n % NSLOT;
+          if (n >= (unsigned)NSLOT) ok = mbar_wait(&sh.empty[slot], ((n / NSLOT) - 1) & 1, abort_flag);
+          if (!ok) break;
+          uint8_t* dst = sIn + slot * SLOT_B;
+          mbar_arrive_expect_tx(&sh.full[slot], 2 * SLOT_B);
+          tma_load_5d(dst, &map_hi, &sh.full[slot], chunk * C, 0, h0, 2 * k, gi);
+          tma_load_5d(dst + LO_OFF, &map_lo, &sh.full[slot], chunk * C, 0, h0, 2 * k, gi);
+        }
+      }
+    }
+  } else if (warp == 1) {
+    const uint32_t idesc = idesc_bf16_f32(ROWS, 128, /*a_mn_major=*/false, /*b_mn_major=*/true);
+    const uint32_t in_base = smem_u32(sIn);
+    unsigned nb = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
+      for (int half = 0; half < 2 && ok; ++half, ++nb) {
+        const int ab = nb % NACC, s0 = nb * BATCH % NSLOT;
+        for (int i = 0; i < BATCH && ok; ++i) ok = mbar_wait_warp(&sh.full[s0 + i], (nb * BATCH / NSLOT) & 1, abort_flag);
+        if (ok && nb >= NACC) ok = mbar_wait_warp(&sh.acc_empty[ab], ((nb / NACC) - 1) & 1, abort_flag);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t xh = smem_desc_sw32(in_base + s0 * SLOT_B), xl = smem_desc_sw32(in_base + s0 * SLOT_B + LO_OFF);
+        const uint32_t d_tm = tm + COL_ACC + ab * 128;
+#pragma unroll
+        for (int ks = 0; ks < ROWS / 16; ++ks) {           // (16 rows of K: 512 bytes, 32 in a descriptor's address field)
+          umma_ts(d_tm, tm + ks * 8, xh + (uint64_t)(ks * 32), idesc, ks > 0 ? 1u : 0u);
+          umma_ts(d_tm, tm + 64 + ks * 8, xh + (uint64_t)(ks * 32), idesc, 1u);
+          umma_ts(d_tm, tm + ks * 8, xl + (uint64_t)(ks * 32), idesc, 1u);
+        }
+        for (int i = 0; i < BATCH; ++i) umma_commit(&sh.empty[s0 + i]);
+        umma_commit(&sh.acc_full[ab]);
+      }
+    }
+  } else {
+    const int quarter = warp & 3, part = (warp - 2) >> 2;  // TMEM lanes; which four channels
+    const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
+    const int p0 = quarter * 32;                           // the warp's first position: w fastest, then h
+    const int w0 = p0 % dm.W, hq = p0 / dm.W;
+    uint8_t* stage = sStage + quarter * 2 * STAGE_B;
+    // the channels' place in row `lane` of a box, under the 32-byte swizzle (rows 32 on have the same pattern)
+    const uint32_t at = (uint32_t)(lane * 32 + (((part >> 1) ^ ((lane >> 2) & 1)) << 4) + (part & 1) * 8);
+    const bool issuer = part == 0 && lane == 0;
+    unsigned nb = 0, nq = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
+      const int chunk = it % P.nchunk, rest = it / P.nchunk, h0 = rest % P.nh * P.hpt + hq, gi = rest / P.nh;
+      float x[T][CPT];
+#pragma unroll
+      for (int b = 0; b < 2; ++b, ++nb) {
+        const int ab = nb % NACC;
+        if (ok) ok = mbar_wait_warp(&sh.acc_full[ab], (nb / NACC) & 1, abort_flag);
+        tc_fence_after();
+        if (ok) {
+#pragma unroll
+          for (int i = 0; i < T / 2; ++i) tmem_ld4(tm + lane_addr + COL_ACC + ab * 128 + i * C + part * CPT, x[b * 8 + i]);
+          tmem_wait_ld();
+        }
+        tc_fence_before();
+        mbar_arrive(&sh.acc_empty[ab]);
+      }
+      if (!ok) break;
+      // four t positions at a time, two boxes: 2 q, 2 q + 1 and 14 - 2 q, 15 - 2 q
+#pragma unroll
+      for (int q = 0; q < 4; ++q, ++nq) {
+        uint8_t* buf = stage + (nq & 1) * STAGE_B;
+        if (nq >= 2) {                                     // the buffer's previous stores have read it
+          if (issuer) { bulk_wait_read1(); mbar_arrive(&sh.stg_free[quarter]); }
+          ok = mbar_wait_warp(&sh.stg_free[quarter], nq & 1, abort_flag);
+          if (!ok) break;
+        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const int i = 2 * q + j;
+          float e[CPT] = {}, o[CPT] = {};
+#pragma unroll
+          for (int k = 0; k < T; k += 2)
+#pragma unroll
+            for (int c = 0; c < CPT; ++c) { e[c] = fmaf(P.mat[k][i], x[k][c], e[c]); o[c] = fmaf(P.mat[k + 1][i], x[k + 1][c], o[c]); }
+          float y[CPT], z[CPT];
+#pragma unroll
+          for (int c = 0; c < CPT; ++c) { y[c] = e[c] + o[c]; z[c] = e[c] - o[c]; }
+          stage4(buf + j * (BOX_B / 2) + at, y);
+          stage4(buf + BOX_B + (1 - j) * (BOX_B / 2) + at, z);
+        }
+        fence_proxy_async();
+        mbar_arrive(&sh.stg_full[quarter]);
+        if (part == 0) {
+          ok = mbar_wait_warp(&sh.stg_full[quarter], nq & 1, abort_flag);
+          if (!ok) break;
+          if (lane == 0) {
+            tma_store_5d(buf, &map_out, chunk * C, w0, h0, 2 * q, P.group_start + gi);
+            tma_store_5d(buf + BOX_B, &map_out, chunk * C, w0, h0, 14 - 2 * q, P.group_start + gi);
+            bulk_commit();
+          }
+          __syncwarp();
+        }
+      }
+    }
+    if (issuer) bulk_wait0();
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (sh.abort_flag) {
+    if (threadIdx.x == 0) atomicExch(P.status, FF_ERR_TIMEOUT | 0x700);   // low byte: status, next byte: which kernel
+    const long long t0 = clock64();
+    while (clock64() - t0 < 2000000) { }
+    __syncthreads();
+  }
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tm, 512);
+  }
+}
+
+// 5-D map over a [slices][T][H][W][d] bf16 grid: the box of 16 channels of two tiles (load), or of 32 positions at two t (store).
+bool grid_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, bool store) {
+  const FFDims& dm = p->dm;
+  return p->maps.get(map, base, store ? 49 : 48, slices, [&] {
+    const cuuint64_t ch = (cuuint64_t)dm.d, W = (cuuint64_t)dm.W;
+    const cuuint64_t dims[5] = {ch, W, (cuuint64_t)dm.H, (cuuint64_t)dm.T, (cuuint64_t)slices};
+    const cuuint64_t strides[4] = {ch * 2, W * ch * 2, dm.H * W * ch * 2, (cuuint64_t)dm.N * ch * 2};
+    const cuuint32_t w = (cuuint32_t)(store && dm.W > 32 ? 32 : dm.W);
+    const cuuint32_t box[5] = {C, w, (cuuint32_t)(store ? 32 : ROWS) / w, 2, 1};
+    return ff_encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_32B,
+                         store ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
+  });
+}
+
+// (the swizzles are functions of the address: 1024-byte alignment)
+constexpr size_t SMEM = 1024 + (size_t)2 * LO_OFF + 4 * 2 * STAGE_B + sizeof(T16Shared);
+
+}  // namespace
+
+cudaError_t ffk_dct_t16_init() {
+  return cudaFuncSetAttribute(dct_t16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
+}
+
+// Where it takes the place of the two-axis launch: t is that launch's second axis, 16 positions, and folds.
+bool ffk_dct_t16_supported(const ff_plan* p) {
+  return p->dct2_ok && p->dct2_axis2 == 0 && p->dm.T == T && p->cfg.transform == FF_TRANSFORM_DCT;
+}
+
+// Hi/lo grids of heads [h0, h0 + g) -> w and t inverse transform -> out.
+cudaError_t ffk_dct_t16_inverse(ff_plan* p, const void* in_hi, const void* in_lo, int h0, int g, void* out, cudaStream_t st) {
+  const FFDims& dm = p->dm;
+  CUtensorMap mh, ml, mo;
+  if (!grid_map(p, &mh, in_hi, p->dct_group, false) || !grid_map(p, &ml, in_lo, p->dct_group, false) || !grid_map(p, &mo, out, dm.BH, true))
+    return cudaErrorInvalidValue;
+  T16Params P{};
+  P.dm = dm; P.status = p->buf.status;
+  P.img = p->dct2_images + (size_t)(3 + 2) * FF_IMAGE_CELLS;
+  memcpy(P.mat, p->t16_mat, sizeof(P.mat));
+  P.group = g; P.group_start = h0;
+  P.nchunk = dm.d / C; P.hpt = ROWS / dm.W; P.nh = dm.H / P.hpt;
+  const int items = g * P.nh * P.nchunk;
+  const cudaError_t e = ff_launch(dct_t16_kernel, dim3((unsigned)(items < p->sm_count ? items : p->sm_count)), dim3(THREADS), SMEM, st, mh, ml, mo, P);
+  if (e == cudaSuccess) p->launches += 1;
+  return e;
+}

@@ -913,7 +913,7 @@ cudaError_t ffk_inverse_transform_tc(ff_plan* p, int h0, int g, void* out, cudaS
   P.image = matrix_image(p, first_axis, 1);
   cudaError_t e = launch_pass(p, m_in, m_inl, m_inl, obh, obl, P, form, st);
   if (e != cudaSuccess) return e;
-  if (fused) return ffk_dct2_inverse(p, sc.b_hi, sc.b_lo, h0, g, out, st);
+  if (fused) return (p->t16 ? ffk_dct_t16_inverse : ffk_dct2_inverse)(p, sc.b_hi, sc.b_lo, h0, g, out, st);
   P.reverse = 0; P.axis = 1; P.image = matrix_image(p, 1, 1);
   e = launch_pass(p, mbh, mbl, mbl, oah, oal, P, form, st);
   if (e != cudaSuccess) return e;

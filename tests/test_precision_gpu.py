@@ -45,12 +45,14 @@ def test_fp32_between_the_axes_of_any_other_grid(grid, d):
 
 
 # Planes of 2048 positions go in chunks of 16 channels: every number of coefficients a phase-2 tile can hold (128 / n2 =
-# 1, 2, 4, 8), against fp64 and against the separate passes.  The latter hand on one byte-form intermediate (2^-16 of the low
-# coefficients' norm); the 16-bit taps differ where a value lies that close to the middle of two bf16 numbers, by a bf16
-# step: share 2^-8 of the values at most, 2^-8 sqrt(2^-8) = 2.5e-4 of the norm.
-@pytest.mark.parametrize("grid", [(128, 128, 16), (64, 64, 32), (32, 64, 64), (16, 32, 128)], ids=lambda g: "x".join(map(str, g)))
+# 1, 2, 4, 8); a t axis of 16 has an inverse launch of its own: every W.  Against fp64 and against the separate passes.  The
+# latter hand on one byte-form intermediate (2^-16 of the low coefficients' norm); the 16-bit taps differ where a value lies
+# that close to the middle of two bf16 numbers, by a bf16 step: share 2^-8 of the values at most, 2^-8 sqrt(2^-8) = 2.5e-4
+# of the norm.
+@pytest.mark.parametrize("grid", [(128, 128, 16), (64, 64, 32), (32, 64, 64), (16, 32, 128),
+                                  (16, 32, 16), (16, 64, 32), (16, 32, 64)], ids=lambda g: "x".join(map(str, g)))
 @pytest.mark.parametrize("d", [64, 128])
-def test_planes_of_2048_positions(grid, d):
+def test_two_axes_in_one_launch(grid, d):
     import torch
     from paper_2604_22808_b200 import binding as B
     low, mid = tuple(n // 8 for n in grid), tuple(n // 8 + n // 2 for n in grid)
