@@ -199,7 +199,7 @@ __device__ __forceinline__ void attention_tc_body(const CUtensorMap& map_a, cons
     fence_mbar_init();
   }
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
-  ff_pdl_wait();
+  ff_pdl_join();
   if (threadIdx.x == 0) { sh.n_units = P.work[0]; sh.total = P.work[1]; }
   __syncthreads();
   for (int i = threadIdx.x; i <= sh.n_units; i += TC_THREADS) {

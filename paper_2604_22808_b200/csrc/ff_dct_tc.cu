@@ -213,7 +213,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     }
     tmem_wait_st();
   }
-  ff_pdl_wait();
+  if (RAG) ff_pdl_wait(); else ff_pdl_join();              // (any other grid: level)
   if (!CONVERT && P.clear && blockIdx.x == 0) for (int i = threadIdx.x; i < dm.B * 3 * CH; i += THREADS) P.clear[i] = 0.0;
   tc_fence_before();
   __syncthreads();

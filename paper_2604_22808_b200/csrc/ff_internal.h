@@ -84,6 +84,12 @@ __device__ __forceinline__ void ff_pdl_wait() {
 
 // The two halves on their own, for a kernel that does not depend on the one before it (but on the ones before that):
 // it starts with the trigger and ends with the wait, so that whoever waits for it has waited for both.
+//
+// A kernel with the join alone lets the next one in when its own blocks have ended.  The one-axis passes of the grids with
+// 16, 32, 64 or 128 positions an axis, the statistics with a router and the attention do: what follows them has little to do
+// ahead of its wait, and let in early it cost more than the start-up it hid (layers, us, with the trigger at the start /
+// without: six heads of 16K tokens 214.2 / 203.1, 24 of 64K 2815 / 2770, 16 of 64K with head_dim 64 1010 / 990, fp32
+// 7 x 16 x 12, six heads, 111 / 100).  The summaries keep it (16K tokens: 211, without 218), the two-axis launch too (203, 206).
 __device__ __forceinline__ void ff_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void ff_pdl_join() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
