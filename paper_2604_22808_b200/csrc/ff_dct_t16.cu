@@ -26,6 +26,7 @@
 #include "ff_clocks.cuh"
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
+#include "ff_two_buffers.h"
 
 using namespace sm100;
 
@@ -41,7 +42,7 @@ constexpr int NACC = 3;                        // accumulator buffers of 128 col
 constexpr int EPI = 4, CPT = C / EPI;          // epilogue warps per 32 lanes, channels of a thread
 constexpr int THREADS = 64 + 4 * EPI * 32;
 constexpr int BOX_B = 2 * 32 * C * 2;          // 2 KB: 32 positions at two t, staged for a store
-constexpr int STAGE_B = 2 * BOX_B;             // a staging buffer
+constexpr int STAGE_B = 2 * BOX_B;             // a staging buffer (two per lane quarter)
 
 struct T16Params {
   FFDims dm;
@@ -52,9 +53,15 @@ struct T16Params {
   int* status;
 };
 
+// Nobody arrives twice in one phase of any of these: a second arrival always lies behind a wait for the first one's phase.
+//   full       the producer, again for a slot behind empty, which the issuer commits behind its wait for full
+//   empty      the issuer's commit, again behind full, which the producer arms behind its wait for empty
+//   acc_full   the issuer's commit, again for a buffer behind acc_empty, where all epilogue threads arrive behind acc_full
+//   acc_empty  an epilogue thread, again behind acc_full, which the issuer commits behind its wait for acc_empty
+//   stg_*      ff_two_buffers.h
 struct T16Shared {
   uint64_t full[NSLOT], empty[NSLOT], acc_full[NACC], acc_empty[NACC];
-  uint64_t stg_full[4], stg_free[4];           // per four epilogue warps
+  uint64_t stg_full[4][FFTwoBuffers::FULL], stg_free[4];           // per four epilogue warps
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -99,7 +106,10 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
   if (threadIdx.x == 0) {
     for (int i = 0; i < NSLOT; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 1); }
     for (int i = 0; i < NACC; ++i) { mbar_init(&sh.acc_full[i], 1); mbar_init(&sh.acc_empty[i], 4 * EPI * 32); }
-    for (int i = 0; i < 4; ++i) { mbar_init(&sh.stg_full[i], EPI * 32); mbar_init(&sh.stg_free[i], 1); }
+    for (int i = 0; i < 4; ++i) {
+      for (int b = 0; b < FFTwoBuffers::FULL; ++b) mbar_init(&sh.stg_full[i][b], EPI * 32);
+      mbar_init(&sh.stg_free[i], 1);
+    }
     sh.abort_flag = 0;
     fence_mbar_init();
   }
@@ -181,7 +191,7 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const int p0 = quarter * 32;                           // the warp's first position: w fastest, then h
     const int w0 = p0 % dm.W, hq = p0 / dm.W;
-    uint8_t* stage = sStage + quarter * 2 * STAGE_B;
+    uint8_t* stage = sStage + quarter * FFTwoBuffers::BUFFERS * STAGE_B;
     // the channels' place in row `lane` of a box, under the 32-byte swizzle (rows 32 on have the same pattern)
     const uint32_t at = (uint32_t)(lane * 32 + (((part >> 1) ^ ((lane >> 2) & 1)) << 4) + (part & 1) * 8);
     const bool issuer = part == 0 && lane == 0;
@@ -207,10 +217,11 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
       // four t positions at a time, two boxes: 2 q, 2 q + 1 and 14 - 2 q, 15 - 2 q
 #pragma unroll
       for (int q = 0; q < 4; ++q, ++nq) {
-        uint8_t* buf = stage + (nq & 1) * STAGE_B;
-        if (nq >= 2) {                                     // the buffer's previous stores have read it
+        uint8_t* buf = stage + FFTwoBuffers::buffer(nq) * STAGE_B;
+        uint64_t* filled = &sh.stg_full[quarter][FFTwoBuffers::full(nq)];
+        if (FFTwoBuffers::waits_free(nq)) {                // the buffer's previous stores have read it
           if (issuer) { bulk_wait_read1(); mbar_arrive(&sh.stg_free[quarter]); }
-          ok = mbar_wait_warp(&sh.stg_free[quarter], nq & 1, abort_flag);
+          ok = mbar_wait_warp(&sh.stg_free[quarter], FFTwoBuffers::free_parity(nq), abort_flag);
           if (!ok) break;
         }
 #pragma unroll
@@ -228,9 +239,9 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
           stage4(buf + BOX_B + (1 - j) * (BOX_B / 2) + at, z);
         }
         fence_proxy_async();
-        mbar_arrive(&sh.stg_full[quarter]);
+        mbar_arrive(filled);
         if (part == 0) {
-          ok = mbar_wait_warp(&sh.stg_full[quarter], nq & 1, abort_flag);
+          ok = mbar_wait_warp(filled, FFTwoBuffers::full_parity(nq), abort_flag);
           if (!ok) break;
           if (lane == 0) {
             tma_store_5d(buf, &map_out, chunk * C, w0, h0, 2 * q, P.group_start + gi);
