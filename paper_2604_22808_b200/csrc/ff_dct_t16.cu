@@ -155,6 +155,8 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
           const int slot = n % NSLOT;
           if (n >= (unsigned)NSLOT) ok = mbar_wait(&sh.empty[slot], ((n / NSLOT) - 1) & 1, abort_flag);
           if (!ok) break;
+          // (debug build) the box lies inside the grid; a refused item ends in the bounded wait of its consumer
+          if (!FF_DBG_OK((chunk + 1) * C <= dm.d && h0 + P.hpt <= dm.H && gi < P.group, P.status, 7)) continue;
           uint8_t* dst = sIn + slot * SLOT_B;
           mbar_arrive_expect_tx(&sh.full[slot], 2 * SLOT_B);
           tma_load_5d(dst, &map_hi, &sh.full[slot], chunk * C, 0, h0, 2 * k, gi);
@@ -243,7 +245,9 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
         if (part == 0) {
           ok = mbar_wait_warp(filled, FFTwoBuffers::full_parity(nq), abort_flag);
           if (!ok) break;
-          if (lane == 0) {
+          // (debug build) its 32 positions are whole lines of the plane, or lie in one
+          if (lane == 0 && FF_DBG_OK((chunk + 1) * C <= dm.d && w0 + (dm.W < 32 ? dm.W : 32) <= dm.W &&
+                                         h0 + (dm.W < 32 ? 32 / dm.W : 1) <= dm.H && P.group_start + gi < dm.BH, P.status, 7)) {
             tma_store_5d(buf, &map_out, chunk * C, w0, h0, 2 * q, P.group_start + gi);
             tma_store_5d(buf + BOX_B, &map_out, chunk * C, w0, h0, 14 - 2 * q, P.group_start + gi);
             bulk_commit();
