@@ -308,7 +308,7 @@ class Plan:
     def kernel_info(self) -> dict:
         info = (C.c_int32 * 4)()
         _check(library().ff_plan_kernel_info(self.handle, info), self.handle)
-        return {"transform_fused": bool(info[0]), "transform_cluster": int(info[1]), "attention_tensor_core": bool(info[2]),
+        return {"transform_fused": bool(info[0]), "inverse_t_in_registers": bool(info[1]), "attention_tensor_core": bool(info[2]),
                 "low_band_tensor_core": bool(info[3])}
 
     def last_launches(self) -> int:

@@ -11,7 +11,7 @@ import harness as Hn
 pytestmark = pytest.mark.gpu
 
 CONFIGS = [C.TINY, C.R64K.scaled("two_axes", heads=3),
-           C.R64K.scaled("cta_pairs", H=16, W=128, low_cut=(2, 2, 16), mid_cut=(10, 10, 80), heads=3),
+           C.R64K.scaled("planes_of_2048", H=16, W=128, low_cut=(2, 2, 16), mid_cut=(10, 10, 80), heads=3),
            C.R64K.scaled("ragged", T=5, H=33, W=20, low_cut=(1, 4, 2), mid_cut=(3, 20, 12), heads=3)]
 
 
