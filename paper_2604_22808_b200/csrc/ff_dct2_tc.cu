@@ -48,7 +48,7 @@ constexpr int GROUP_B = ROWS * GCOLS * 2;     // 8 KB as bf16
 constexpr int NSTG = 8;                       // input ring: at most 8 groups (64 KB: 8 bf16 groups or 4 hi/lo pairs)
 constexpr int RING_B = NSTG * GROUP_B;
 constexpr int MAX_GPI = 8;                    // groups of an item (128 KB of hi/lo buffer)
-constexpr int D2_THREADS = 640;                 // TMA, MMA 1, release, MMA 2, 8 phase-1 and 8 phase-2 epilogue warps
+constexpr int D2_THREADS = 640;                 // TMA, MMA 1, idle, MMA 2, 8 phase-1 and 8 phase-2 epilogue warps
 constexpr int ACC_GROUPS = 4;                 // groups that fit a phase's 128 accumulator columns: one batch of 4, or 2 of 2
 constexpr int IMG_CELLS = 64;                 // 32-bit tensor-memory cells per matrix row: two bf16 K elements each
 constexpr int STG_B = 32 * GCOLS * 2;         // bytes an epilogue warp stages at a time (its 32 rows of a group), hi or lo

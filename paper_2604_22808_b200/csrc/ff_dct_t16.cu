@@ -136,7 +136,7 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
     }
     tmem_wait_st();
   }
-  // (the next launch comes in when this one's blocks end: let in at the start, its blocks slowed the last third of this
+  // (the next launch comes in when this one's blocks end: let in earlier, its blocks slowed the last third of this
   // launch down, 16K tokens, six heads: 30.6 us instead of 22.3)
   ff_pdl_join();
   tc_fence_before();

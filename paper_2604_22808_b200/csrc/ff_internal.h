@@ -74,22 +74,24 @@ inline FFFastDiv ff_fast_div(unsigned d) {
 }
 #if defined(__CUDACC__)
 // Programmatic dependent launch.  Every kernel of the path is launched with the attribute, does what does not
-// depend on earlier kernels (barriers, tensor memory, matrices of the plan), then waits here until the kernel
-// before it in the stream has finished and its writes are visible, and lets the next kernel start its own
-// prologue.  It reads or writes nothing another kernel touches before the wait.
+// depend on earlier kernels (barriers, tensor memory, matrices of the plan), then waits until the kernel
+// before it in the stream has finished and its writes are visible.  It reads or writes nothing another kernel
+// touches before the wait.  Here it then lets the next kernel start its own prologue.
 __device__ __forceinline__ void ff_pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// The two halves on their own, for a kernel that does not depend on the one before it (but on the ones before that):
-// it starts with the trigger and ends with the wait, so that whoever waits for it has waited for both.
+// The two halves on their own.  The exchange of the mid and high bands starts with the trigger and ends with the join: it
+// does not depend on the launch before it, the low band's exchange, but on the ones before that, and whoever waits for it
+// has waited for both.  That holds only while the launch before it triggers behind its own wait, or not at all.
 //
 // A kernel with the join alone lets the next one in when its own blocks have ended.  The one-axis passes of the grids with
-// 16, 32, 64 or 128 positions an axis, the statistics with a router and the attention do: what follows them has little to do
-// ahead of its wait, and let in early it cost more than the start-up it hid (layers, us, with the trigger at the start /
-// without: six heads of 16K tokens 214.2 / 203.1, 24 of 64K 2815 / 2770, 16 of 64K with head_dim 64 1010 / 990, fp32
-// 7 x 16 x 12, six heads, 111 / 100).  The summaries keep it (16K tokens: 211, without 218), the two-axis launch too (203, 206).
+// 16, 32, 64 or 128 positions an axis, the inverse launch with t in registers, the statistics with a router and the attention
+// do: what follows them has little to do ahead of its wait, and let in early it cost more than the start-up it hid (layers, us,
+// with the trigger behind the wait / without: six heads of 16K tokens 214.2 / 203.1, 24 of 64K 2815 / 2770, 16 of 64K with
+// head_dim 64 1010 / 990, fp32 7 x 16 x 12, six heads, 111 / 100).  The summaries keep it (16K tokens: 211, without 218), the
+// two-axis launch too (203, 206).
 __device__ __forceinline__ void ff_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void ff_pdl_join() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
