@@ -19,6 +19,9 @@ NAMES = {
     "transform_pass": {16 * m + i: f"{mode}, {what}" for m, mode in enumerate(("first pass", "middle pass", "band split", "last pass"))
                        for i, what in _PASS.items()},
     "transform_plane": {16 * s + i: f"{('forward', 'inverse')[s]}, {what}" for s in range(2) for i, what in _PLANE.items()},
+    "transform_t16": {0: "copies: wait for a slot", 1: "issuer: wait for input", 2: "issuer: wait for accumulators",
+                      3: "epilogue: wait for accumulators", 4: "epilogue: wait for staging", 5: "epilogue: wait for the other warps",
+                      6: "epilogue: fold, stage and send an item", 7: "whole kernel"},
     "exchange": {0: "copies: wait for a slot", 1: "issuer: wait for tokens", 2: "issuer: wait for P", 3: "issuer: wait for the update buffer",
                  4: "issuer: wait for summaries", 6: "softmax: wait for scores", 7: "softmax: work", 9: "store: wait for the update",
                  10: "store: work", 14: "store: look up positions"},

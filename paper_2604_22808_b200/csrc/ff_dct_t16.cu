@@ -18,7 +18,8 @@
 //                thread sends two t positions at a time out with tensor stores
 // Every wait is bounded.
 //
-// Bound by its rows of 32 bytes.  24 heads of 64K tokens, at 1.6 GHz under the power limit: 334 us with ff_dct2_tc.cu, 254
+// Bound by its epilogue, which by its clocks folds, stages and sends rows of 32 bytes for 8300 of an item's 9700 cycles, and
+// behind it by the loads (six heads of 64K tokens alone: 64.7 us, DRAM 49%, L2 57%, issue slots 49%).  24 heads of 64K tokens, at 1.6 GHz under the power limit: 334 us with ff_dct2_tc.cu, 254
 // here (1.2 GB at 4.7 TB/s); six heads of 16K tokens 28 and 22 us.  The forward launch stays with ff_dct2_tc.cu: it writes a
 // hi/lo pair, and with twice as many 32-byte rows out as in it took 1130 to 1160 instead of 883 us.
 #include <cuda.h>
@@ -143,6 +144,7 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
   __syncthreads();
   tc_fence_after();
 
+  FF_CLOCK(t_all);
   // Item: chunk fastest (CTAs that run side by side read neighbouring pieces of the same rows), then h, then the head.
   if (warp == 0) {
     if (lane == 0) {
@@ -153,7 +155,9 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
         const int chunk = it % P.nchunk, rest = it / P.nchunk, h0 = rest % P.nh * P.hpt, gi = rest / P.nh;
         for (int k = 0; k < T / 2 && ok; ++k, ++n) {
           const int slot = n % NSLOT;
+          FF_CLOCK(tp);
           if (n >= (unsigned)NSLOT) ok = mbar_wait(&sh.empty[slot], ((n / NSLOT) - 1) & 1, abort_flag);
+          FF_CLOCK_ADD(true, 0, tp);
           if (!ok) break;
           // (debug build) the box lies inside the grid; a refused item ends in the bounded wait of its consumer
           if (!FF_DBG_OK((chunk + 1) * C <= dm.d && h0 + P.hpt <= dm.H && gi < P.group, P.status, 7)) continue;
@@ -172,8 +176,12 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
     for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
       for (int half = 0; half < 2 && ok; ++half, ++nb) {
         const int ab = nb % NACC, s0 = nb * BATCH % NSLOT;
+        FF_CLOCK(ti);
         for (int i = 0; i < BATCH && ok; ++i) ok = mbar_wait_warp(&sh.full[s0 + i], (nb * BATCH / NSLOT) & 1, abort_flag);
+        FF_CLOCK_ADD(lane == 0, 1, ti);
+        FF_CLOCK(ta);
         if (ok && nb >= NACC) ok = mbar_wait_warp(&sh.acc_empty[ab], ((nb / NACC) - 1) & 1, abort_flag);
+        FF_CLOCK_ADD(lane == 0, 2, ta);
         if (!ok) break;
         tc_fence_after();
         const uint64_t xh = smem_desc_sw32(in_base + s0 * SLOT_B), xl = smem_desc_sw32(in_base + s0 * SLOT_B + LO_OFF);
@@ -205,7 +213,9 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
 #pragma unroll
       for (int b = 0; b < 2; ++b, ++nb) {
         const int ab = nb % NACC;
+        FF_CLOCK(te);
         if (ok) ok = mbar_wait_warp(&sh.acc_full[ab], (nb / NACC) & 1, abort_flag);
+        FF_CLOCK_ADD(issuer && quarter == 0, 3, te);
         tc_fence_after();
         if (ok) {
 #pragma unroll
@@ -216,14 +226,17 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
         mbar_arrive(&sh.acc_empty[ab]);
       }
       if (!ok) break;
+      FF_CLOCK(tw);
       // four t positions at a time, two boxes: 2 q, 2 q + 1 and 14 - 2 q, 15 - 2 q
 #pragma unroll
       for (int q = 0; q < 4; ++q, ++nq) {
         uint8_t* buf = stage + FFTwoBuffers::buffer(nq) * STAGE_B;
         uint64_t* filled = &sh.stg_full[quarter][FFTwoBuffers::full(nq)];
         if (FFTwoBuffers::waits_free(nq)) {                // the buffer's previous stores have read it
+          FF_CLOCK(tb);
           if (issuer) { bulk_wait_read1(); mbar_arrive(&sh.stg_free[quarter]); }
           ok = mbar_wait_warp(&sh.stg_free[quarter], FFTwoBuffers::free_parity(nq), abort_flag);
+          FF_CLOCK_ADD(issuer && quarter == 0, 4, tb);
           if (!ok) break;
         }
 #pragma unroll
@@ -243,7 +256,9 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
         fence_proxy_async();
         mbar_arrive(filled);
         if (part == 0) {
+          FF_CLOCK(tf);
           ok = mbar_wait_warp(filled, FFTwoBuffers::full_parity(nq), abort_flag);
+          FF_CLOCK_ADD(issuer && quarter == 0, 5, tf);
           if (!ok) break;
           // (debug build) its 32 positions are whole lines of the plane, or lie in one
           if (lane == 0 && FF_DBG_OK((chunk + 1) * C <= dm.d && w0 + (dm.W < 32 ? dm.W : 32) <= dm.W &&
@@ -255,8 +270,10 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
           __syncwarp();
         }
       }
+      FF_CLOCK_ADD(issuer && quarter == 0, 6, tw);
     }
     if (issuer) bulk_wait0();
+    FF_CLOCK_ADD(issuer && quarter == 0, 7, t_all);
   }
 
   tc_fence_before();
@@ -318,3 +335,5 @@ cudaError_t ffk_dct_t16_inverse(ff_plan* p, const void* in_hi, const void* in_lo
   if (e == cudaSuccess) p->launches += 1;
   return e;
 }
+
+FF_CLOCKS_READ(transform_t16)
