@@ -418,6 +418,7 @@ static ff_status_t transform_and_route(ff_plan* p, const void* Q, const void* K,
                                        const uint8_t* alloc_in, cudaStream_t st) {
   FF_CUDA(p, mark(p, 0, st));
   const bool route = alloc_in == nullptr;
+  p->masks_given = !route;
   if (route) {
     if (!p->has_router) return fail(p, FF_ERR_NOT_ROUTED, "the plan was created without router weights%s");
     if (!timestep) return fail(p, FF_ERR_NOT_ROUTED, "neither an allocation nor a timestep was given%s");

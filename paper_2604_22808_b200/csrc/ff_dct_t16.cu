@@ -19,9 +19,10 @@
 // Every wait is bounded.
 //
 // Bound by its epilogue, which by its clocks folds, stages and sends rows of 32 bytes for 8300 of an item's 9700 cycles, and
-// behind it by the loads (six heads of 64K tokens alone: 64.7 us, DRAM 49%, L2 57%, issue slots 49%).  24 heads of 64K tokens, at 1.6 GHz under the power limit: 334 us with ff_dct2_tc.cu, 254
-// here (1.2 GB at 4.7 TB/s); six heads of 16K tokens 28 and 22 us.  The forward launch stays with ff_dct2_tc.cu: it writes a
-// hi/lo pair, and with twice as many 32-byte rows out as in it took 1130 to 1160 instead of 883 us.
+// behind it by the loads (six heads of 64K tokens alone: 64.7 us, DRAM 49%, L2 57%, issue slots 49%).  24 heads of 64K
+// tokens, at 1.6 GHz under the power limit: 334 us with ff_dct2_tc.cu, 254 here (1.2 GB at 4.7 TB/s); six heads of 16K tokens
+// 28 and 22 us.  The forward launch stays with ff_dct2_tc.cu: it writes a hi/lo pair, and with twice as many 32-byte rows out
+// as in it took 1130 to 1160 instead of 883 us.
 #include <cuda.h>
 
 #include "ff_clocks.cuh"

@@ -114,6 +114,7 @@ struct DctTcParams {
   int in_split;            // input is a hi/lo pair of grids (map0 = hi, map1 = lo)
   int out_lo8;             // the lo part of the output pair is one byte per value (see "Three-byte intermediates")
   int nstage;              // ring depth
+  int early;               // the next launch comes in behind this one's wait, not when its blocks end
   int reverse;             // walk the tiles from the last to the first (what the previous launch wrote last is still in L2)
   __nv_bfloat16* spec_mid; __nv_bfloat16* spec_high;
   float* spec_low;         // MODE_SPLIT: [3 BH][N_low][d] fp32
@@ -213,7 +214,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     }
     tmem_wait_st();
   }
-  if (RAG) ff_pdl_wait(); else ff_pdl_join();              // (any other grid: level)
+  if (P.early) ff_pdl_wait(); else ff_pdl_join();
   if (!CONVERT && P.clear && blockIdx.x == 0) for (int i = threadIdx.x; i < dm.B * 3 * CH; i += THREADS) P.clear[i] = 0.0;
   tc_fence_before();
   __syncthreads();
@@ -749,6 +750,8 @@ cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1
   int nstage = (int)((232448 - 256 - fixed) / stage);   // 227 KB of shared memory per CTA
   if (nstage > MAX_STAGE) nstage = MAX_STAGE;
   P.nstage = nstage;
+  // (see ff_internal.h; any other grid: level)
+  P.early = ff_fp32_grid(P.dm) || p->masks_given;
   const size_t smem = nstage * stage + fixed;
   P.g = ff_pass_shape(P.dm, P.axis);
   P.by_tiles = ff_fast_div((unsigned)P.g.tiles); P.by_inner = ff_fast_div((unsigned)P.g.tiles_inner);

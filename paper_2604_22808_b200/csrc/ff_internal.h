@@ -87,11 +87,14 @@ __device__ __forceinline__ void ff_pdl_wait() {
 // has waited for both.  That holds only while the launch before it triggers behind its own wait, or not at all.
 //
 // A kernel with the join alone lets the next one in when its own blocks have ended.  The one-axis passes of the grids with
-// 16, 32, 64 or 128 positions an axis, the inverse launch with t in registers, the statistics with a router and the attention
-// do: what follows them has little to do ahead of its wait, and let in early it cost more than the start-up it hid (layers, us,
+// 16, 32, 64 or 128 positions an axis and the statistics, both in a routed call, the inverse launch with t in registers and the
+// attention do: what follows them has little to do ahead of its wait, and let in early it cost more than the start-up it hid (layers, us,
 // with the trigger behind the wait / without: six heads of 16K tokens 214.2 / 203.1, 24 of 64K 2815 / 2770, 16 of 64K with
 // head_dim 64 1010 / 990, fp32 7 x 16 x 12, six heads, 111 / 100).  The summaries keep it (16K tokens: 211, without 218), the
-// two-axis launch too (203, 206).
+// two-axis launch too (203, 206).  With masks given there is no router to wait for, and the passes let the next launch in behind
+// their wait (all bands, when their blocks end / behind the wait: six heads of 16 x 16 x 16 110.7 / 106.9, four of 16 x 16 x 32
+// 130.1 / 127.2, of 16 x 32 x 32 with head_dim 64 135.1 / 131.6, six of 64 x 16 x 64 901 / 889, of 16 x 32 x 32 228.0 / 229.7,
+// four of 64 x 64 x 64 3368 / 3358; routed calls lose by it: six of 16 x 32 x 32 217 / 224, of 64 x 16 x 64 681 / 695).
 __device__ __forceinline__ void ff_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void ff_pdl_join() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -220,6 +223,7 @@ struct ff_plan {
   alignas(64) unsigned char tmap_low[128];     // ... over the pooled low band (bf16 copy), when low_tc_ok
   bool low_tc_ok;                              // the low branch runs in the tensor-core attention launch
   long long launches;
+  bool masks_given;                            // the call has the caller's masks (set by every call before its first launch)
   // ff_forward_host on the tensor-core path: copies run on a second stream, one event per launch
   // group of the forward transform (host -> device) and of the inverse transform (device -> host)
   cudaStream_t copy_stream;
