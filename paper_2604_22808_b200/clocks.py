@@ -15,13 +15,14 @@ _PLANE = {0: "phase 1 epilogue: wait for accumulators", 1: "phase 1 epilogue: wa
           6: "phase 1 epilogue: hand-over", 7: "issuer 1: wait for input", 8: "issuer 1: wait for accumulators",
           9: "issuer 2: wait for rows", 10: "issuer 2: wait for accumulators", 11: "issuer 2: wait for the second half",
           12: "copies: wait for a slot", 15: "whole kernel"}
+_T16 = {0: "copies: wait for a slot", 1: "issuer: wait for input", 2: "issuer: wait for accumulators",
+        3: "epilogue: wait for accumulators", 4: "epilogue: wait for staging", 5: "epilogue: wait for the other warps",
+        6: "epilogue: fold, stage and send an item", 7: "whole kernel"}
 NAMES = {
     "transform_pass": {16 * m + i: f"{mode}, {what}" for m, mode in enumerate(("first pass", "middle pass", "band split", "last pass"))
                        for i, what in _PASS.items()},
     "transform_plane": {16 * s + i: f"{('forward', 'inverse')[s]}, {what}" for s in range(2) for i, what in _PLANE.items()},
-    "transform_t16": {0: "copies: wait for a slot", 1: "issuer: wait for input", 2: "issuer: wait for accumulators",
-                      3: "epilogue: wait for accumulators", 4: "epilogue: wait for staging", 5: "epilogue: wait for the other warps",
-                      6: "epilogue: fold, stage and send an item", 7: "whole kernel"},
+    "transform_t16": {16 * f + i: f"{('inverse', 'forward')[f]}, {what}" for f in range(2) for i, what in _T16.items()},
     "exchange": {0: "copies: wait for a slot", 1: "issuer: wait for tokens", 2: "issuer: wait for P", 3: "issuer: wait for the update buffer",
                  4: "issuer: wait for summaries", 6: "softmax: wait for scores", 7: "softmax: work", 9: "store: wait for the update",
                  10: "store: work", 14: "store: look up positions"},

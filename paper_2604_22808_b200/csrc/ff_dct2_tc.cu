@@ -626,7 +626,7 @@ bool ffk_dct2_supported(const FFDims& dm, int* axis2, int* chunk) {
 bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat, int n) {
   const size_t per = FF_IMAGE_CELLS;
   const int parts = ff_fp32_grid(p->dm) ? 3 : 2;        // (the third is read on those grids only)
-  if (!p->dct2_images && cudaMalloc((void**)&p->dct2_images, 6 * per * sizeof(uint32_t)) != cudaSuccess) return false;
+  if (!p->dct2_images && cudaMalloc((void**)&p->dct2_images, FF_IMAGES * per * sizeof(uint32_t)) != cudaSuccess) return false;
   const FFPassShape g = ff_pass_shape(p->dm, axis);
   const int kf = g.kf;
   const bool seq = axis == 2;

@@ -144,6 +144,7 @@ FF_HD bool ff_fp32_grid(const FFDims& dm) { return !(ff_tile_axis(dm.T) && ff_ti
 // Transform matrix of an axis as tensor-memory operand images: [3 parts][128 rows][64 cells of two bf16]; the first two
 // parts are the bf16 pair, all three the fp32 value.
 constexpr size_t FF_IMAGE_PART = (size_t)128 * 64, FF_IMAGE_CELLS = 3 * FF_IMAGE_PART;
+constexpr int FF_IMAGES = 7;
 
 // SMs for the rules that shape the workspace: its size is a function of the configuration alone (it is asked for without
 // a device).  Rules that shape only a launch take the device's count.
@@ -211,11 +212,12 @@ struct ff_plan {
   unsigned* tickets;                           // "last block" counters, zero between launches (plan-owned)
   int* pos_table;                              // rank -> flat coefficient index of the mid, then the high band (plan-owned)
   alignas(64) unsigned char tmap_x[4][128];    // CUtensorMaps of the exchange kernel (Y / V~ of the mid and high bands)
-  uint32_t* dct2_images;                       // 6 transform matrices as tensor-memory operand images (plan-owned)
+  uint32_t* dct2_images;                       // transform matrices as tensor-memory operand images (plan-owned): three axes forward,
+                                               // inverse, and the folded one of ff_dct_t16.cu
   FFMapCache maps;                             // tensor maps of the transform passes, by shape
   bool dct2_ok;                                // the fused two-axis launch covers this configuration
   int dct2_axis2;                              // its second axis (1 = h, 0 = t); the remaining axis gets a pass of its own
-  bool t16;                                    // ... and the inverse one is ff_dct_t16.cu
+  bool t16, t16_forward;                       // ... and the inverse, the forward one is ff_dct_t16.cu
   float t16_mat[16][8];                        // C_T[k][i], i < 8
   int dct2_chunk;                              // channels of its work items: 32, or 16 for the larger planes
   alignas(64) unsigned char tmap_mid[128];     // CUtensorMap over the mid-band / high-band coefficient buffers
@@ -281,6 +283,10 @@ cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, i
 // ---- the same with a t axis of 16 positions in registers (ff_dct_t16.cu) ------------------------------
 cudaError_t ffk_dct_t16_init();
 bool ffk_dct_t16_supported(const ff_plan* p);
+bool ffk_dct_t16_forward_supported(const ff_plan* p);
+bool ffk_dct_t16_build_image(ff_plan* p, const float* mat_host);
+cudaError_t ffk_dct_t16_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
+                                bool clear_energy, cudaStream_t st);
 cudaError_t ffk_dct_t16_inverse(ff_plan* p, const void* in_hi, const void* in_lo, int h0, int g, void* out, cudaStream_t st);
 // ---- projections around the path (ff_proj_tc.cu) -------------------------------------------------------
 bool ffk_proj_supported(const FFDims& dm);
