@@ -16,8 +16,8 @@ _PLANE = {0: "phase 1 epilogue: wait for accumulators", 1: "phase 1 epilogue: wa
           9: "issuer 2: wait for rows", 10: "issuer 2: wait for accumulators", 11: "issuer 2: wait for the second half",
           12: "copies: wait for a slot", 15: "whole kernel"}
 _T16 = {0: "copies: wait for a slot", 1: "issuer: wait for input", 2: "issuer: wait for accumulators",
-        3: "epilogue: wait for accumulators", 4: "epilogue: wait for staging", 5: "epilogue: wait for the other warps",
-        6: "epilogue: fold, stage and send an item", 7: "whole kernel"}
+        3: "epilogue: wait for accumulators", 4: "epilogue: wait for staging", 6: "epilogue: stage and send an item",
+        7: "whole kernel"}
 NAMES = {
     "transform_pass": {16 * m + i: f"{mode}, {what}" for m, mode in enumerate(("first pass", "middle pass", "band split", "last pass"))
                        for i, what in _PASS.items()},

@@ -3,8 +3,8 @@
 //
 // A 16 x 16 matrix is too small for the tensor core: as Mat kron I it fills an eighth of the 128 x 128 operand that
 // ff_dct2_tc.cu multiplies with, three times over for the hi/lo parts, and its input has to go from the accumulators through
-// registers and shared memory to become an operand.  Here a thread takes all 16 t coefficients of a (h, w) position and four
-// channels from the accumulators of the w axis and folds them (C[k][15 - i] = (-1)^k C[k][i]: even and odd k apart), eight
+// registers and shared memory to become an operand.  Here a thread takes all 16 t coefficients of a (h, w) position from the
+// accumulators of the w axis and folds them (C[k][15 - i] = (-1)^k C[k][i]: even and odd k apart), eight
 // FMA and one addition a value, in fp32.  On long runs every launch of this path meets the board's power limit; three of six
 // tensor products and the plane's way through shared memory are energy, too.
 //
@@ -14,14 +14,14 @@
 // columns, so that nothing crosses lanes; 256 columns an item and 128 more for the first half of the next.
 //   warp 0       TMA producer (ring of twelve slots: two tiles as a hi/lo pair)
 //   warp 1       tcgen05.mma issuer; owns the tensor-memory allocation
-//   warps 2..17  epilogue: four warps per 32 lanes, four channels each; they stage rows of 16 channels together and one
-//                thread sends two t positions at a time out with tensor stores
+//   warps 2..17  epilogue: four warps per 32 lanes; a warp makes four of the 16 t positions (two pairs i, 15 - i) for all
+//                channels, stages its rows and sends two t positions at a time out with a tensor store
 // Every wait is bounded.
 //
-// Bound by its epilogue, which by its clocks folds, stages and sends rows of 32 bytes for 8300 of an item's 9700 cycles, and
-// behind it by the loads (six heads of 64K tokens alone: 64.7 us, DRAM 49%, L2 57%, issue slots 49%).  24 heads of 64K
-// tokens, at 1.6 GHz under the power limit: 334 us with ff_dct2_tc.cu, 254 here (1.2 GB at 4.7 TB/s); six heads of 16K tokens
-// 28 and 22 us.  The forward launch has a kernel of its own, below.
+// Bound by its epilogue and the loads: six heads of 64K tokens alone 62 us, 0.3 GB at 4.9 TB/s, issue slots 50%.  The four
+// warps of 32 lanes share a scheduler; when each made all t positions of four channels and they staged whole rows together, the
+// scheduler stood still at every hand-over: 69 us, six heads of 16K tokens 193 -> 190 for the whole layer.  With ff_dct2_tc.cu in
+// this launch's place it took 334 us for 24 heads of 64K tokens at 1.6 GHz, with the shared staging 254.  The forward launch has a kernel of its own, below.
 #include <cuda.h>
 
 #include <vector>
@@ -29,7 +29,6 @@
 #include "ff_clocks.cuh"
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
-#include "ff_two_buffers.h"
 
 using namespace sm100;
 
@@ -42,10 +41,9 @@ constexpr int SLOT_B = 2 * TILE_B;             // two t positions
 constexpr int BATCH = 4;                       // slots of an instruction batch: N = 8 tiles of 16 channels
 constexpr int NSLOT = 12, LO_OFF = NSLOT * SLOT_B;     // ring: three batches, the hi parts, behind them their lo parts (192 KB)
 constexpr int NACC = 3;                        // accumulator buffers of 128 columns, behind the matrix (2 x 64)
-constexpr int EPI = 4, CPT = C / EPI;          // epilogue warps per 32 lanes, channels of a thread
+constexpr int EPI = 4;                         // epilogue warps per 32 lanes
 constexpr int THREADS = 64 + 4 * EPI * 32;
-constexpr int BOX_B = 2 * 32 * C * 2;          // 2 KB: 32 positions at two t, staged for a store
-constexpr int STAGE_B = 2 * BOX_B;             // a staging buffer (two per lane quarter)
+constexpr int BOX_B = 2 * 32 * C * 2;          // 2 KB: 32 positions at two t, staged for a store (an area per epilogue warp)
 
 struct T16Params {
   FFDims dm;
@@ -62,10 +60,8 @@ struct T16Params {
 //   empty      the issuer's commit, again behind full, which the producer arms behind its wait for empty
 //   acc_full   the issuer's commit, again for a buffer behind acc_empty, where all epilogue threads arrive behind acc_full
 //   acc_empty  an epilogue thread, again behind acc_full, which the issuer commits behind its wait for acc_empty
-//   stg_*      ff_two_buffers.h
 struct T16Shared {
   uint64_t full[NSLOT], empty[NSLOT], acc_full[NACC], acc_empty[NACC];
-  uint64_t stg_full[4][FFTwoBuffers::FULL], stg_free[4];           // per four epilogue warps
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -75,18 +71,6 @@ struct T16Shared {
 __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t smem_addr) {
   return (uint64_t)((smem_addr & 0x3FFFF) >> 4) | (uint64_t)(TILE_B >> 4) << 16 | (uint64_t)(256 >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)6 << 61;
 }
-
-// 32 lanes x 4 columns
-__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&r)[4]) {
-  uint32_t v[4];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-               : "r"(taddr)
-               : "memory");
-#pragma unroll
-  for (int i = 0; i < 4; ++i) r[i] = __uint_as_float(v[i]);
-}
-__device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 
 // The matrix (hi, then lo part) into tensor memory by four warps: a thread loads the row of its lane.
 __device__ __forceinline__ void matrix_to_tmem(const uint32_t* img, uint32_t tm, int quarter, int lane) {
@@ -106,11 +90,6 @@ __device__ __forceinline__ void matrix_to_tmem(const uint32_t* img, uint32_t tm,
   tmem_wait_st();
 }
 
-// A thread's channels -> eight bytes.
-__device__ __forceinline__ void stage4(uint8_t* dst, const float (&y)[CPT]) {
-  *(uint2*)dst = make_uint2(bf16_pair(__float_as_uint(y[0]), __float_as_uint(y[1])), bf16_pair(__float_as_uint(y[2]), __float_as_uint(y[3])));
-}
-
 // map_hi, map_lo: the pair of grids; map_out: the caller's tensor, box = 32 positions at two t.
 __global__ void __launch_bounds__(THREADS, 1)
 dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant__ CUtensorMap map_lo,
@@ -120,18 +99,14 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
   const FFDims& dm = P.dm;
   constexpr uint32_t COL_ACC = 128;
   uint8_t* sIn = smem;
-  uint8_t* sStage = smem + 2 * LO_OFF;                      // four lane quarters x two buffers
-  T16Shared& sh = *(T16Shared*)(sStage + 4 * 2 * STAGE_B);
+  uint8_t* sStage = smem + 2 * LO_OFF;                      // an area per epilogue warp
+  T16Shared& sh = *(T16Shared*)(sStage + 4 * EPI * BOX_B);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int total = P.group * P.nh * P.nchunk;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < NSLOT; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 1); }
     for (int i = 0; i < NACC; ++i) { mbar_init(&sh.acc_full[i], 1); mbar_init(&sh.acc_empty[i], 4 * EPI * 32); }
-    for (int i = 0; i < 4; ++i) {
-      for (int b = 0; b < FFTwoBuffers::FULL; ++b) mbar_init(&sh.stg_full[i][b], EPI * 32);
-      mbar_init(&sh.stg_free[i], 1);
-    }
     sh.abort_flag = 0;
     fence_mbar_init();
   }
@@ -202,83 +177,78 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
       }
     }
   } else {
-    const int quarter = warp & 3, part = (warp - 2) >> 2;  // TMEM lanes; which four channels
+    const int quarter = warp & 3, part = (warp - 2) >> 2;  // TMEM lanes; which t: 2 part, 2 part + 1 and 14 - 2 part, 15 - 2 part
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const int p0 = quarter * 32;                           // the warp's first position: w fastest, then h
     const int w0 = p0 % dm.W, hq = p0 / dm.W;
-    uint8_t* stage = sStage + quarter * FFTwoBuffers::BUFFERS * STAGE_B;
-    // the channels' place in row `lane` of a box, under the 32-byte swizzle (rows 32 on have the same pattern)
-    const uint32_t at = (uint32_t)(lane * 32 + (((part >> 1) ^ ((lane >> 2) & 1)) << 4) + (part & 1) * 8);
-    const bool issuer = part == 0 && lane == 0;
-    unsigned nb = 0, nq = 0;
+    const int i0 = __shfl_sync(0xffffffffu, 2 * part, 0);
+    uint8_t* stage = sStage + (warp - 2) * BOX_B;
+    unsigned nb = 0;
     bool ok = true;
     for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
       const int chunk = it % P.nchunk, rest = it / P.nchunk, h0 = rest % P.nh * P.hpt + hq, gi = rest / P.nh;
-      float x[T][CPT];
-#pragma unroll
+      float e[2][C] = {}, o[2][C] = {};
+#pragma unroll 1
       for (int b = 0; b < 2; ++b, ++nb) {
         const int ab = nb % NACC;
         FF_CLOCK(te);
-        if (ok) ok = mbar_wait_warp(&sh.acc_full[ab], (nb / NACC) & 1, abort_flag);
-        FF_CLOCK_ADD(issuer && quarter == 0, 3, te);
+        ok = mbar_wait_warp(&sh.acc_full[ab], (nb / NACC) & 1, abort_flag);
+        FF_CLOCK_ADD(threadIdx.x == 64, 3, te);
+        if (!ok) break;
         tc_fence_after();
-        if (ok) {
+#pragma unroll 1
+        for (int k2 = 0; k2 < T / 2; k2 += 2)
 #pragma unroll
-          for (int i = 0; i < T / 2; ++i) tmem_ld4(tm + lane_addr + COL_ACC + ab * 128 + i * C + part * CPT, x[b * 8 + i]);
-          tmem_wait_ld();
-        }
+          for (int odd = 0; odd < 2; ++odd) {
+            const int k = k2 + odd;
+            uint32_t x[C];
+            tmem_ld16(tm + lane_addr + COL_ACC + ab * 128 + k * C, x);
+            const float2 m = *(const float2*)(P.mat[b * 8 + k] + i0);
+            tmem_wait_ld();
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+              float& f0 = odd ? o[0][c] : e[0][c];
+              float& f1 = odd ? o[1][c] : e[1][c];
+              f0 = fmaf(m.x, __uint_as_float(x[c]), f0);
+              f1 = fmaf(m.y, __uint_as_float(x[c]), f1);
+            }
+          }
         tc_fence_before();
         mbar_arrive(&sh.acc_empty[ab]);
       }
       if (!ok) break;
       FF_CLOCK(tw);
-      // four t positions at a time, two boxes: 2 q, 2 q + 1 and 14 - 2 q, 15 - 2 q
 #pragma unroll
-      for (int q = 0; q < 4; ++q, ++nq) {
-        uint8_t* buf = stage + FFTwoBuffers::buffer(nq) * STAGE_B;
-        uint64_t* filled = &sh.stg_full[quarter][FFTwoBuffers::full(nq)];
-        if (FFTwoBuffers::waits_free(nq)) {                // the buffer's previous stores have read it
-          FF_CLOCK(tb);
-          if (issuer) { bulk_wait_read1(); mbar_arrive(&sh.stg_free[quarter]); }
-          ok = mbar_wait_warp(&sh.stg_free[quarter], FFTwoBuffers::free_parity(nq), abort_flag);
-          FF_CLOCK_ADD(issuer && quarter == 0, 4, tb);
-          if (!ok) break;
-        }
+      for (int back = 0; back < 2; ++back) {               // the two t of one end, then those of the other
+        uint32_t v[2][C / 2];
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int i = 2 * q + j;
-          float e[CPT] = {}, o[CPT] = {};
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
-          for (int k = 0; k < T; k += 2)
+          for (int c = 0; c < C; c += 2)
+            v[j][c / 2] = back ? bf16_pair(__float_as_uint(e[1 - j][c] - o[1 - j][c]), __float_as_uint(e[1 - j][c + 1] - o[1 - j][c + 1]))
+                               : bf16_pair(__float_as_uint(e[j][c] + o[j][c]), __float_as_uint(e[j][c + 1] + o[j][c + 1]));
+        FF_CLOCK(tb);
+        if (lane == 0) bulk_wait_read0();                  // the warp's previous store has read the area
+        __syncwarp();
+        FF_CLOCK_ADD(threadIdx.x == 64, 4, tb);
 #pragma unroll
-            for (int c = 0; c < CPT; ++c) { e[c] = fmaf(P.mat[k][i], x[k][c], e[c]); o[c] = fmaf(P.mat[k + 1][i], x[k + 1][c], o[c]); }
-          float y[CPT], z[CPT];
+        for (int j = 0; j < 2; ++j)
 #pragma unroll
-          for (int c = 0; c < CPT; ++c) { y[c] = e[c] + o[c]; z[c] = e[c] - o[c]; }
-          stage4(buf + j * (BOX_B / 2) + at, y);
-          stage4(buf + BOX_B + (1 - j) * (BOX_B / 2) + at, z);
-        }
+          for (int c = 0; c < 2; ++c)                      // (32-byte swizzle)
+            *(uint4*)(stage + j * (BOX_B / 2) + lane * 32 + ((c ^ ((lane >> 2) & 1)) << 4)) = make_uint4(v[j][4 * c], v[j][4 * c + 1], v[j][4 * c + 2], v[j][4 * c + 3]);
         fence_proxy_async();
-        mbar_arrive(filled);
-        if (part == 0) {
-          FF_CLOCK(tf);
-          ok = mbar_wait_warp(filled, FFTwoBuffers::full_parity(nq), abort_flag);
-          FF_CLOCK_ADD(issuer && quarter == 0, 5, tf);
-          if (!ok) break;
-          // (debug build) its 32 positions are whole lines of the plane, or lie in one
-          if (lane == 0 && FF_DBG_OK((chunk + 1) * C <= dm.d && w0 + (dm.W < 32 ? dm.W : 32) <= dm.W &&
-                                         h0 + (dm.W < 32 ? 32 / dm.W : 1) <= dm.H && P.group_start + gi < dm.BH, P.status, 7)) {
-            tma_store_5d(buf, &map_out, chunk * C, w0, h0, 2 * q, P.group_start + gi);
-            tma_store_5d(buf + BOX_B, &map_out, chunk * C, w0, h0, 14 - 2 * q, P.group_start + gi);
-            bulk_commit();
-          }
-          __syncwarp();
+        __syncwarp();
+        // (debug build) its 32 positions are whole lines of the plane, or lie in one
+        if (lane == 0 && FF_DBG_OK((chunk + 1) * C <= dm.d && w0 + (dm.W < 32 ? dm.W : 32) <= dm.W &&
+                                       h0 + (dm.W < 32 ? 32 / dm.W : 1) <= dm.H && P.group_start + gi < dm.BH, P.status, 7)) {
+          tma_store_5d(stage, &map_out, chunk * C, w0, h0, back ? 14 - i0 : i0, P.group_start + gi);
+          bulk_commit();
         }
       }
-      FF_CLOCK_ADD(issuer && quarter == 0, 6, tw);
+      FF_CLOCK_ADD(threadIdx.x == 64, 6, tw);
     }
-    if (issuer) bulk_wait0();
-    FF_CLOCK_ADD(issuer && quarter == 0, 7, t_all);
+    if (lane == 0) bulk_wait0();
+    FF_CLOCK_ADD(threadIdx.x == 64, 7, t_all);
   }
 
   tc_fence_before();
@@ -535,7 +505,7 @@ bool grid_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, bool s
 }
 
 // (the swizzles are functions of the address: 1024-byte alignment)
-constexpr size_t SMEM = 1024 + (size_t)2 * LO_OFF + 4 * 2 * STAGE_B + sizeof(T16Shared);
+constexpr size_t SMEM = 1024 + (size_t)2 * LO_OFF + 4 * EPI * BOX_B + sizeof(T16Shared);
 
 }  // namespace
 
