@@ -33,11 +33,18 @@
 // clipped by the copies.  Grids with an axis other than 16, 32, 64 or 128 ran on fp32 kernels, and the precision stays
 // that of fp32 numbers: the passes hand on fp32 grids (FORM_EXACT1 and FORM_EXACT), matrix and data are three bf16 parts
 // each, which hold all 24 bits, and six of their nine products are summed, the small ones first (the others are below
-// 2^-24).  The parts of the data are made by the four warps that expand bytes in FORM_BYTES: truncations, so that they
+// 2^-24).  The parts of the data are made by warps of their own: truncations, so that they
 // add up to the value.  A pass moves 4 bytes per value like a bf16 pair, and 48 instructions a tile keep the tensor core
 // below the copies' time.  21 x 45 x 80 tokens, 16 heads: forward transform 1.94 ms and inverse with the exchange 0.94
-// (fp32 kernels: 4.46 and 2.83; 16-bit intermediates: 1.54 and 0.67); the passes run at 4.1 - 5.9 TB/s, the later ones
-// below the first because two stages of 96 KB are all that fit.
+// (fp32 kernels: 4.46 and 2.83; 16-bit intermediates: 1.54 and 0.67).
+// What bounds the passes that read fp32 is the way of a tile through its stage: copy, parts, instructions, 10 300 cycles
+// with 128 channels.  A stage there holds only the rows in use and no third part, which lives from its making to the
+// instructions and has two slots: three stages of 96 rows or less fit where two of 96 KB did, two of 128 rows still.  And eight
+// warps make the parts instead of four (not beside the band split, whose epilogue needs the registers).  The first pass waited for
+// its one staging area: it has two, and a stage less.  Six heads of that grid, the passes alone, us: w 176 -> 172 (6.1 TB/s),
+// h 296 -> 245 (5.7), t with the band split 271 -> 264 (4.0), inverse t 96 -> 94, h 107 -> 89, w 107 -> 96; layers (16 heads 3640 ->
+// 3474, eight of 7 x 90 x 127 tokens 1970 -> 1873).  With 64 channels none of it gained (20 x 30 x 52 tokens, eight heads, 484 -> 490):
+// they keep four stages of whole tiles.
 //
 // Order of the tiles.  A pass that reads what the previous launch wrote walks its tiles from the last to the
 // first (P.reverse), the next one forward again: the end of the previous launch's output is still in L2.
@@ -46,7 +53,7 @@
 //   warp 1      tcgen05.mma issuer (A from tensor memory), 3 accumulator buffers of 128 TMEM columns (2 beside three
 //               matrix parts)
 //   warps 2..9  epilogue: tcgen05.ld, convert to the output's form, store; a thread owns one output position
-//   warps 10..13  (FORM_BYTES, FORM_EXACT) operands of an arriving tile
+//   warps 10..13  (FORM_BYTES, FORM_EXACT) operands of an arriving tile; FORM_EXACT with 128 channels: 10..17
 // Output path (FIRST, MIDDLE, LAST): an epilogue warp's 32 rows are 32 grid positions that form a
 // box of the grid, so the warp writes 32 channels of them (64 bytes per row, 64-byte swizzle, no
 // bank conflicts) into its own staging area and one lane sends them out with a tensor store; the
@@ -68,6 +75,7 @@
 #include "ff_internal.h"
 #include "ff_sm100.cuh"
 #include "ff_three_byte.cuh"
+#include "ff_two_buffers.h"
 
 using namespace sm100;
 
@@ -87,12 +95,16 @@ enum {
   FORM_PAIR,      // bf16: the caller's tensor, or a hi/lo pair of grids
   FORM_BYTES,     // a pair in the three-byte form
   FORM_EXACT1,    // any grid: the caller's bf16 tensor, handed on as fp32
-  FORM_EXACT      // any grid: an fp32 grid
+  FORM_EXACT,     // any grid: an fp32 grid
+  FORM_EXACT_SPLIT   // ... and the band split follows (128 channels; with 64 it is a mode of FORM_EXACT)
 };
-template <int FORM> struct Shape {
+template <int CH, int FORM> struct Shape {
   static constexpr bool any_grid = FORM >= FORM_EXACT1;
-  static constexpr bool convert = FORM == FORM_BYTES || FORM == FORM_EXACT;
-  static constexpr int threads = convert ? 448 : 320;      // TMA warp, MMA warp, 8 epilogue warps; 4 that make operands of the data
+  static constexpr bool convert = FORM == FORM_BYTES || FORM >= FORM_EXACT;
+  // TMA warp, MMA warp, 8 epilogue warps; then those that make operands of the data: 128 threads, and of fp32 numbers as many
+  // for every 64 channels
+  static constexpr int makers = !convert ? 0 : (FORM == FORM_EXACT ? 2 * CH : 128);
+  static constexpr int threads = 320 + makers;
   static constexpr int parts = any_grid ? 3 : 2;           // of the matrix, 64 tensor-memory columns each
   static constexpr uint32_t col_acc = parts * 64;          // accumulator buffers of 128 columns behind them
   static constexpr int nacc = any_grid ? 2 : NACC_MAX;
@@ -127,7 +139,8 @@ constexpr int STG_PITCH = 64;                       // bytes per staged row piec
 
 struct DctShared {
   uint64_t full[MAX_STAGE], empty[MAX_STAGE], acc_full[NACC_MAX], acc_empty[NACC_MAX], conv[MAX_STAGE];
-  uint64_t stg_full[2], stg_free[2];       // (any grid) staging area of four epilogue warps: written / read by its store
+  uint64_t third_empty[2];                 // (F32) a slot of the third part has been read
+  uint64_t stg_full[2][FFTwoBuffers::FULL], stg_free[2];       // (any grid) staging areas of four epilogue warps: written / read by the store
   uint32_t tmem_base;
   int abort_flag;
   int e_sample;            // (SPLIT) sample of the CTA's last tile
@@ -135,6 +148,9 @@ struct DctShared {
   // into stores where four lanes cover a row's 64 contiguous bytes
   alignas(1024) uint8_t stage[8][2][32 * STG_PITCH];
 };
+
+// (F32) rows of a tile in shared memory: whole k-steps.
+__host__ __device__ constexpr int exact_rows(int rows) { return (rows + 15) / 16 * 16; }
 
 // First line of tile `u` of a tensor-head: index along the inner extent and along the outer one.
 __device__ __forceinline__ void tile_origin(const DctTcParams& P, unsigned u, int& i0, int& o0) {
@@ -150,41 +166,50 @@ __device__ __forceinline__ void tile_origin(const DctTcParams& P, unsigned u, in
 // are clipped by the stores.  32 rows are then no box of the grid, so the four warps of a channel half stage a
 // whole tile (32 channels) and one thread stores it.
 template <int CH, int FORM>
-__global__ void __launch_bounds__(Shape<FORM>::threads, 1)
+__global__ void __launch_bounds__(Shape<CH, FORM>::threads, 1)
 dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
               const __grid_constant__ CUtensorMap map2, const __grid_constant__ CUtensorMap map_oh,
               const __grid_constant__ CUtensorMap map_ol, const DctTcParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  constexpr bool LO8 = FORM == FORM_BYTES, F32 = FORM == FORM_EXACT, RAG = Shape<FORM>::any_grid, CONVERT = Shape<FORM>::convert;
-  constexpr int NACC = Shape<FORM>::nacc, THREADS = Shape<FORM>::threads;
-  constexpr uint32_t COL_ACC = Shape<FORM>::col_acc;
+  constexpr bool LO8 = FORM == FORM_BYTES, F32 = FORM >= FORM_EXACT, RAG = Shape<CH, FORM>::any_grid, CONVERT = Shape<CH, FORM>::convert;
+  constexpr int NACC = Shape<CH, FORM>::nacc, THREADS = Shape<CH, FORM>::threads;
+  constexpr uint32_t COL_ACC = Shape<CH, FORM>::col_acc;
   const FFDims& dm = P.dm;
   const int n = P.g.n, kf = P.g.kf;                       // axis length, lines per tile
   const bool seq = P.g.seq;                               // lines follow one another (w axis) or interleave
   const int rows = RAG ? P.g.rows : TILE_ROWS;
   const int NSTAGE = P.nstage;
-  const bool split = !LO8 && FORM != FORM_EXACT1 && P.mode == MODE_SPLIT;     // (the band-split pass never reads the byte form)
+  const bool split = FORM == FORM_EXACT_SPLIT || ((FORM == FORM_PAIR || (FORM == FORM_EXACT && CH == 64)) && P.mode == MODE_SPLIT);     // (the band-split pass never reads the byte form)
   const bool tma_out = !split;
   constexpr int TB = TILE_ROWS * CH * 2;                  // bytes of one data tile (16 KB for 64 channels)
   constexpr int LO8_OFF = CH == 128 ? TB : 2 * TB;         // where a stage takes the lo bytes
-  const int STAGE_BYTES = LO8 ? LO8_OFF + TB / 2 + (CH == 128 ? TB / 2 : 0) : (F32 ? 3 * TB : (P.in_split ? 2 * TB : TB));   // hi tile, lo tile
+  // (F32) blocks of 128-byte rows, as many as the instructions read; the third part of the data has two slots of its own, or
+  // lies behind the other two (64 channels: stages of whole tiles are small enough)
+  constexpr bool SLOTS = F32 && CH == 128;
+  const int RB = SLOTS ? exact_rows(rows) * 128 : HALF_BYTES, THIRD_BYTES = SLOTS ? RB * (CH / 64) : 0;
+  const int STAGE_BYTES = LO8 ? LO8_OFF + TB / 2 + (CH == 128 ? TB / 2 : 0) : (SLOTS ? RB * (CH / 32) : F32 ? 3 * TB : (P.in_split ? 2 * TB : TB));   // hi tile, lo tile
   uint8_t* sData = smem;                                  // NSTAGE x STAGE_BYTES
-  DctShared& sh = *(DctShared*)(smem + NSTAGE * STAGE_BYTES);
+  uint8_t* sThird = smem + NSTAGE * STAGE_BYTES;
+  DctShared& sh = *(DctShared*)(sThird + 2 * THIRD_BYTES);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const unsigned tiles_per_th = (unsigned)P.g.tiles;
   const int total_tiles = P.group * P.g.tiles;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < NSTAGE; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 1); mbar_init(&sh.conv[i], 128); }
+    for (int i = 0; i < NSTAGE; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 1); mbar_init(&sh.conv[i], CONVERT ? Shape<CH, FORM>::makers : 1); }
     for (int i = 0; i < NACC; ++i) { mbar_init(&sh.acc_full[i], 1); mbar_init(&sh.acc_empty[i], 256); }
-    if (RAG) for (int i = 0; i < 2; ++i) { mbar_init(&sh.stg_full[i], 128); mbar_init(&sh.stg_free[i], 1); }
+    if (RAG)
+      for (int i = 0; i < 2; ++i) {
+        for (int b = 0; b < FFTwoBuffers::FULL; ++b) mbar_init(&sh.stg_full[i][b], 128);
+        mbar_init(&sh.stg_free[i], 1); mbar_init(&sh.third_empty[i], 1);
+      }
     sh.abort_flag = 0;
     fence_mbar_init();
   }
   if (warp == 1) { tmem_alloc(&sh.tmem_base, 512); tmem_relinquish(); }
   if (RAG) {                                              // rows that no copy writes must not hold NaN patterns
-    for (int i = threadIdx.x * 16; i < NSTAGE * STAGE_BYTES; i += blockDim.x * 16) *(uint4*)(sData + i) = make_uint4(0, 0, 0, 0);
+    for (int i = threadIdx.x * 16; i < NSTAGE * STAGE_BYTES + 2 * THIRD_BYTES; i += blockDim.x * 16) *(uint4*)(sData + i) = make_uint4(0, 0, 0, 0);
     fence_proxy_async();
   }
   tc_fence_before();
@@ -199,7 +224,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
     const int quarter = warp & 3, row = quarter * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
 #pragma unroll 1
-    for (int im = 0; im < Shape<FORM>::parts; ++im) {
+    for (int im = 0; im < Shape<CH, FORM>::parts; ++im) {
       const uint32_t* src = P.image + (size_t)im * FF_IMAGE_PART + (size_t)row * IMG_CELLS;
 #pragma unroll
       for (int c0 = 0; c0 < IMG_CELLS; c0 += 32) {
@@ -246,7 +271,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
         mbar_arrive_expect_tx(&sh.full[slot], (uint32_t)(rows * CH) * (LO8 ? 3u : (F32 || P.in_split ? 4u : 2u)));
         if (F32) {                                         // blocks of 32 channels: rows of 128 bytes
 #pragma unroll
-          for (int b = 0; b < CH / 32; ++b) tma_load_5d(dst + b * HALF_BYTES, map, &sh.full[slot], 32 * b, i0, 0, o0, slice);
+          for (int b = 0; b < CH / 32; ++b) tma_load_5d(dst + b * RB, map, &sh.full[slot], 32 * b, i0, 0, o0, slice);
           continue;
         }
         tma_load_5d(dst, map, &sh.full[slot], 0, i0, 0, o0, slice);
@@ -286,8 +311,8 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
         };
         if (F32) {
           // (the halves of 64 channels of the first two parts alternate, those of the third follow one another)
-          const uint64_t x0 = smem_desc_sw128(dbase, 2 * HALF_BYTES, 1024), x1 = smem_desc_sw128(dbase + HALF_BYTES, 2 * HALF_BYTES, 1024);
-          const uint64_t x2 = smem_desc_sw128(dbase + 2 * TB, HALF_BYTES, 1024);
+          const uint64_t x0 = smem_desc_sw128(dbase, 2 * RB, 1024), x1 = smem_desc_sw128(dbase + RB, 2 * RB, 1024);
+          const uint64_t x2 = smem_desc_sw128(SLOTS ? smem_u32(sThird + (it & 1) * THIRD_BYTES) : dbase + 2 * TB, RB, 1024);
           product(2, x0, true);
           product(1, x1, false);
           product(0, x2, false);
@@ -309,34 +334,46 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
           }
         }
         umma_commit(&sh.empty[slot]);
+        if (SLOTS) umma_commit(&sh.third_empty[it & 1]);
         umma_commit(&sh.acc_full[ab]);
       }
     }
   } else if (F32 && warp >= 10) {
     // ------------------------------------------------------------------ fp32 -> three bf16 parts, in place
-    // A thread owns a row of the tile.  64 channels at a time: they arrive in two blocks of 32 channels, the first and the
-    // second part go where they were (64 channels a block), the third part behind the tile; all with the 128-byte swizzle.
-    const int r0 = threadIdx.x - 320;
+    // A thread owns 64 channels of a row of the tile: they arrive in two blocks of 32 channels, the first and the
+    // second part go where they were (64 channels a block), the third part into its slot; all with the 128-byte swizzle.
+    const int r0 = (threadIdx.x - 320) & 127, h0 = (threadIdx.x - 320) >> 7;
     unsigned it = 0;
     bool ok = true;
     for (int sl = blockIdx.x; sl < total_tiles && ok; sl += gridDim.x, ++it) {
       const int slot = it % NSTAGE;
       FF_CLOCK(pc0);
       ok = __all_sync(0xffffffffu, mbar_wait(&sh.full[slot], (it / NSTAGE) & 1, abort_flag));
+      if (SLOTS && ok && it >= 2) ok = mbar_wait_warp(&sh.third_empty[it & 1], ((it >> 1) - 1) & 1, abort_flag);
       FF_CLOCK_ADD(threadIdx.x == 320, P.mode * 16 + 0, pc0);
       if (!ok) break;
       FF_CLOCK(pc1);
       if (r0 < rows) {
 #pragma unroll 1
-        for (int h = 0; h < CH / 64; ++h) {
-          uint8_t* b0 = sData + slot * STAGE_BYTES + h * 2 * HALF_BYTES + r0 * 128;
-          uint8_t* b2 = sData + slot * STAGE_BYTES + 2 * TB + h * HALF_BYTES + r0 * 128;
-          uint4 x[16];                                     // four channels each
+        for (int h = h0; h < CH / 64; h += Shape<CH, FORM>::makers / 128) {
+          uint8_t* b0 = sData + slot * STAGE_BYTES + h * 2 * RB + r0 * 128;
+          uint8_t* b2 = (SLOTS ? sThird + (it & 1) * THIRD_BYTES : sData + slot * STAGE_BYTES + 2 * TB) + h * RB + r0 * 128;
+          // The first 32 channels go to registers.  Then eight channels at a time, those of the second block from its end, so
+          // that no chunk is written before it has been read.
+          uint4 x[8];                                      // four channels each
 #pragma unroll
-          for (int c = 0; c < 16; ++c) x[c] = *(const uint4*)(b0 + (c >> 3) * HALF_BYTES + (((c & 7) ^ (r0 & 7)) << 4));
+          for (int c = 0; c < 8; ++c) x[c] = *(const uint4*)(b0 + ((c ^ (r0 & 7)) << 4));
 #pragma unroll
-          for (int c = 0; c < 8; ++c) {                    // eight channels: a 16-byte chunk of each part
-            const uint32_t v[8] = {x[2 * c].x, x[2 * c].y, x[2 * c].z, x[2 * c].w, x[2 * c + 1].x, x[2 * c + 1].y, x[2 * c + 1].z, x[2 * c + 1].w};
+          for (int k = 0; k < 8; ++k) {
+            const int c = k < 4 ? 7 - k : k - 4;           // 16-byte chunk of each part
+            uint4 xa, xb;
+            if (c >= 4) {
+              xa = *(const uint4*)(b0 + RB + (((2 * c - 8) ^ (r0 & 7)) << 4));
+              xb = *(const uint4*)(b0 + RB + (((2 * c - 7) ^ (r0 & 7)) << 4));
+            } else {
+              xa = x[2 * (c & 3)]; xb = x[2 * (c & 3) + 1];
+            }
+            const uint32_t v[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
             uint32_t p0[4], p1[4], p2[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -350,7 +387,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
             }
             const uint32_t off = (uint32_t)((c ^ (r0 & 7)) << 4);
             *(uint4*)(b0 + off) = make_uint4(p0[0], p0[1], p0[2], p0[3]);
-            *(uint4*)(b0 + HALF_BYTES + off) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
+            *(uint4*)(b0 + RB + off) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
             *(uint4*)(b2 + off) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
           }
         }
@@ -521,18 +558,26 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       const int out_slice = P.mode == MODE_LAST ? th : gi;
       const unsigned nonlow_rows = __ballot_sync(0xffffffffu, band > 0), mid_rows = __ballot_sync(0xffffffffu, band == 1);
       // both 32-channel chunks of the row at once; the accumulator buffer is free as soon as they are read
-      uint32_t rr2[NQ][32];
-      FF_CLOCK(pl);
+      constexpr bool EACH = FORM == FORM_EXACT_SPLIT;      // (for want of registers one after the other)
+      uint32_t rr2[EACH ? 1 : NQ][32];
+      if (!EACH) {
+        FF_CLOCK(pl);
 #pragma unroll
-      for (int qi = 0; qi < NQ; ++qi) tmem_ld32(tm + lane_addr + COL_ACC + ab * 128 + (q_lo + qi) * 32, rr2[qi]);
-      tmem_wait_ld();
-      FF_CLOCK_ADD(threadIdx.x == 64, P.mode * 16 + 8, pl);
-      tc_fence_before();
-      mbar_arrive(&sh.acc_empty[ab]);
+        for (int qi = 0; qi < NQ; ++qi) tmem_ld32(tm + lane_addr + COL_ACC + ab * 128 + (q_lo + qi) * 32, rr2[EACH ? 0 : qi]);
+        tmem_wait_ld();
+        FF_CLOCK_ADD(threadIdx.x == 64, P.mode * 16 + 8, pl);
+        tc_fence_before();
+        mbar_arrive(&sh.acc_empty[ab]);
+      }
 #pragma unroll
       for (int qi = 0; qi < NQ; ++qi) {
         const int q = q_lo + qi;
-        uint32_t (&r)[32] = rr2[qi];
+        uint32_t (&r)[32] = rr2[EACH ? 0 : qi];
+        if (EACH) {
+          tmem_ld32(tm + lane_addr + COL_ACC + ab * 128 + q * 32, r);
+          tmem_wait_ld();
+          if (qi == NQ - 1) { tc_fence_before(); mbar_arrive(&sh.acc_empty[ab]); }
+        }
         if (!LO8 && row_f32) {
 #pragma unroll
           for (int i = 0; i < 8; ++i)
@@ -541,12 +586,18 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
         if (RAG && tma_out) {
           // four warps stage one tile, 32 channels of 128 rows: fp32 in rows of 128 bytes (128-byte swizzle), or the caller's
           // bf16 in rows of 64 (64-byte swizzle).  (Two areas of half the size in turn: 3470 against 3300 us for the
-          // 76K-token layer.)
+          // 76K-token layer; two whole ones for the bf16 rows: 96 -> 103 us.)
           const int grp = ew >> 2;
-          uint8_t* area = sh.stage[grp * 4][0];
-          if (nchunk > 0) {
-            if (quarter == 0 && lane == 0) { bulk_wait_read0(); mbar_arrive(&sh.stg_free[grp]); }
-            ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_free[grp], (nchunk - 1) & 1, abort_flag));
+          // The first pass has two areas in turn (the second pair behind the barriers) and five instead of six stages.
+          constexpr bool TWO = FORM == FORM_EXACT1 && CH == 128;
+          uint8_t* area = TWO && FFTwoBuffers::buffer(nchunk) ? (uint8_t*)(&sh + 1) + grp * HALF_BYTES : sh.stage[grp * 4][0];
+          uint64_t* filled = &sh.stg_full[grp][TWO ? FFTwoBuffers::full(nchunk) : 0];
+          if (TWO ? FFTwoBuffers::waits_free(nchunk) : nchunk > 0) {
+            if (quarter == 0 && lane == 0) {
+              if (TWO) bulk_wait_read1(); else bulk_wait_read0();
+              mbar_arrive(&sh.stg_free[grp]);
+            }
+            ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_free[grp], TWO ? FFTwoBuffers::free_parity(nchunk) : (nchunk - 1) & 1, abort_flag));
             if (!ok) break;
           }
           if (FORM == FORM_EXACT1 || P.mode == MODE_MIDDLE) {
@@ -563,9 +614,9 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
             }
           }
           fence_proxy_async();
-          mbar_arrive(&sh.stg_full[grp]);
+          mbar_arrive(filled);
           if (quarter == 0) {
-            ok = __all_sync(0xffffffffu, mbar_wait(&sh.stg_full[grp], nchunk & 1, abort_flag));
+            ok = __all_sync(0xffffffffu, mbar_wait(filled, TWO ? FFTwoBuffers::full_parity(nchunk) : nchunk & 1, abort_flag));
             if (!ok) break;
             if (lane == 0) {
               tma_store_5d(area, &map_oh, q * 32, i0, 0, o0, out_slice);
@@ -744,28 +795,30 @@ bool store_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, int a
 // `form`: what the pass reads.
 cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1, const CUtensorMap& m2,
                         const CUtensorMap& moh, const CUtensorMap& mol, DctTcParams& P, int form, cudaStream_t st) {
-  const size_t tile = (size_t)TILE_ROWS * P.dm.d * 2;
-  const size_t stage = form == FORM_EXACT ? 3 * tile : (form == FORM_BYTES ? (P.dm.d == 128 ? 2 * tile : 2 * tile + tile / 2) : (size_t)(P.in_split ? 2 : 1) * tile);
-  const size_t fixed = sizeof(DctShared) + 1024;
+  P.g = ff_pass_shape(P.dm, P.axis);
+  const size_t tile = (size_t)TILE_ROWS * P.dm.d * 2, third = form >= FORM_EXACT && P.dm.d == 128 ? (size_t)exact_rows(P.g.rows) * P.dm.d * 2 : 0;
+  const size_t stage = third ? 2 * third : form >= FORM_EXACT ? 3 * tile : (form == FORM_BYTES ? (P.dm.d == 128 ? 2 * tile : 2 * tile + tile / 2) : (size_t)(P.in_split ? 2 : 1) * tile);
+  const size_t second = form == FORM_EXACT1 && P.dm.d == 128 ? 2 * HALF_BYTES : 0;      // the second pair of staging areas
+  const size_t fixed = sizeof(DctShared) + 1024 + 2 * third + second;
   int nstage = (int)((232448 - 256 - fixed) / stage);   // 227 KB of shared memory per CTA
   if (nstage > MAX_STAGE) nstage = MAX_STAGE;
   P.nstage = nstage;
   // (see ff_internal.h; any other grid: level)
   P.early = ff_fp32_grid(P.dm) || p->masks_given;
   const size_t smem = nstage * stage + fixed;
-  P.g = ff_pass_shape(P.dm, P.axis);
   P.by_tiles = ff_fast_div((unsigned)P.g.tiles); P.by_inner = ff_fast_div((unsigned)P.g.tiles_inner);
   P.by_line = ff_fast_div((unsigned)(P.axis == 2 ? P.dm.H : P.dm.W));
   const int tiles = P.group * P.g.tiles;
   const int grid = tiles < p->sm_count ? tiles : p->sm_count;
   cudaError_t e;
-#define FF_DCT(D, F) e = ff_launch(dct_tc_kernel<D, F>, dim3(grid), dim3(Shape<F>::threads), smem, st, m0, m1, m2, moh, mol, P)
+#define FF_DCT(D, F) e = ff_launch(dct_tc_kernel<D, F>, dim3(grid), dim3(Shape<D, F>::threads), smem, st, m0, m1, m2, moh, mol, P)
 #define FF_DCT_D(F) do { if (P.dm.d == 128) FF_DCT(128, F); else FF_DCT(64, F); } while (0)
   switch (form) {
     case FORM_PAIR: FF_DCT_D(FORM_PAIR); break;
     case FORM_BYTES: FF_DCT_D(FORM_BYTES); break;
     case FORM_EXACT1: FF_DCT_D(FORM_EXACT1); break;
-    default: FF_DCT_D(FORM_EXACT);
+    case FORM_EXACT: FF_DCT_D(FORM_EXACT); break;
+    default: FF_DCT(128, FORM_EXACT_SPLIT);
   }
 #undef FF_DCT_D
 #undef FF_DCT
@@ -781,7 +834,8 @@ cudaError_t ffk_dct_tc_init(const FFDims& dm) {
 #define FF_DCT(D, F) \
   if (e == cudaSuccess && dm.d == D) e = cudaFuncSetAttribute(dct_tc_kernel<D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 256)
   if (!ffk_dct_tc_supported(dm)) return e;
-  if (ff_fp32_grid(dm)) { FF_DCT(128, FORM_EXACT1); FF_DCT(128, FORM_EXACT); FF_DCT(64, FORM_EXACT1); FF_DCT(64, FORM_EXACT); }
+  if (ff_fp32_grid(dm)) { FF_DCT(128, FORM_EXACT1); FF_DCT(128, FORM_EXACT); FF_DCT(64, FORM_EXACT1); FF_DCT(64, FORM_EXACT);
+                           FF_DCT(128, FORM_EXACT_SPLIT); }
   else { FF_DCT(128, FORM_PAIR); FF_DCT(128, FORM_BYTES); FF_DCT(64, FORM_PAIR); FF_DCT(64, FORM_BYTES); }
 #undef FF_DCT
   return e;
@@ -878,7 +932,7 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
     if (e != cudaSuccess) return e;
     P.in_split = 1; P.out_lo8 = 0; P.reverse = 0;
     P.mode = MODE_SPLIT; P.axis = 0; P.image = matrix_image(p, 0, 0);
-    e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, exact ? FORM_EXACT : FORM_PAIR, st);    // (no tensor stores in this mode)
+    e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, exact ? (dm.d == 128 ? FORM_EXACT_SPLIT : FORM_EXACT) : FORM_PAIR, st);    // (no tensor stores in this mode)
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
