@@ -229,7 +229,7 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
   // orthonormal Haar wavelets (row 0 constant; row 2^j + q is +-sqrt(2^j / n) on the halves of the q-th block of
   // n / 2^j positions), rows from the coarsest scale to the finest.
   const int n[3] = {c->T, c->H, c->W};
-  std::vector<float> w_matrix;
+  std::vector<float> mats[3];
   for (int a = 0; a < 3 && s == FF_OK; ++a) {
     std::vector<float> C((size_t)n[a] * n[a]), Ct((size_t)n[a] * n[a]);
     for (int k = 0; k < n[a]; ++k)
@@ -253,7 +253,7 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
       }
     if (a == 0 && c->T == 16)
       for (int k = 0; k < 16; ++k) for (int i = 0; i < 8; ++i) p->t16_mat[k][i] = C[(size_t)k * 16 + i];
-    if (a == 2) w_matrix = C;
+    mats[a] = C;
     s = upload(p, &p->basis[a], C.data(), C.size());
     if (s == FF_OK) s = upload(p, &p->basis_t[a], Ct.data(), Ct.size());
     if (s == FF_OK && ffk_dct_tc_supported(p->dm) &&
@@ -262,9 +262,12 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
   }
   p->dct2_ok = s == FF_OK && p->dct2_images && ffk_dct2_supported(p->dm, &p->dct2_axis2, &p->dct2_chunk);
   p->t16 = ffk_dct_t16_supported(p);
-  p->t16_forward = ffk_dct_t16_forward_supported(p);
-  if (p->t16_forward && !ffk_dct_t16_build_image(p, w_matrix.data()))
-    s = fail(p, FF_ERR_CUDA, "could not upload the transform matrix images%s");
+  p->fold = ffk_dct_fold_supported(p);
+  if (p->fold) {
+    const int n2 = n[p->dct2_axis2 ? 1 : 0];
+    for (int k = 0; k < n2; ++k) for (int i = 0; i < n2 / 2; ++i) p->fold_mat[k * (n2 / 2) + i] = mats[p->dct2_axis2 ? 1 : 0][(size_t)k * n2 + i];
+    if (!ffk_dct_fold_build_image(p, mats[2].data())) s = fail(p, FF_ERR_CUDA, "could not upload the transform matrix images%s");
+  }
   const size_t d = c->head_dim, hid = c->router_hidden, nin = 3 * d + c->t_embed_dim;
   if (s == FF_OK && w && w->W1 && w->b1 && w->W2 && w->b2) {
     s = upload(p, &p->W1, w->W1, hid * nin);

@@ -1,5 +1,6 @@
-// The first launch of the forward and the last one of the inverse transform ("Separable spectral decomposition",
-// "Reconstruction") where the t axis has 16 positions: the w axis on the tensor cores, t in fp32 registers.  bf16 storage, DCT-II.
+// Two axis passes in one launch with the second axis in fp32 registers instead of on the tensor cores ("Separable spectral
+// decomposition", "Reconstruction"): the last launch of the inverse where the t axis has 16 positions, and, below, the first
+// launch of the forward where the second axis, t or h, has 16 or 32.  bf16 storage, DCT-II.
 //
 // A 16 x 16 matrix is too small for the tensor core: as Mat kron I it fills an eighth of the 128 x 128 operand that
 // ff_dct2_tc.cu multiplies with, three times over for the hi/lo parts, and its input has to go from the accumulators through
@@ -50,8 +51,7 @@ struct T16Params {
   const uint32_t* img;     // matrix of the w axis: hi [128][64] cells, then lo
   alignas(16) float mat[T][T / 2];     // mat[k][i] = C[k][i], i < 8
   int group, group_start;  // heads of the launch, the first one's place in the caller's tensor
-  int nchunk, nh, hpt;     // channel chunks, groups of h positions, h positions of a group (128 / W; forward: 64 / W)
-  double* clear;           // (forward) band energies to clear for the sums that follow (first launch of a routed forward), or NULL
+  int nchunk, nh, hpt;     // channel chunks, groups of h positions, h positions of a group (128 / W)
   int* status;
 };
 
@@ -266,55 +266,90 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
 }
 
 // ------------------------------------------------------------------------------------------------------------------
-// Forward.  w on the tensor cores, t in fp32 registers, and the fold of t on the tensor cores, too: a tile is 64 positions at
-// t = i over the same 64 at t = 15 - i, the operand [[M, M], [M, -M]] with M = I kron C_w.  Lanes 0..63 then hold the w transform
-// of x[i] + x[15 - i], lanes 64..127 that of x[i] - x[15 - i], and a thread makes the eight even or the eight odd t coefficients
-// of its position from eight numbers a channel: an item of 32 channels takes the 256 accumulator columns that one of 16 would
-// take unfolded, and rows of 64 bytes go in and out.
-//   warp 0       TMA producer (ring of five batches of four tiles)
+// Forward.  w on the tensor cores, the second axis (t, or h where h is shorter; n2 = 16 or 32 positions) in fp32 registers, and
+// its fold on the tensor cores, too: a tile is 64 positions at i over the same 64 at n2 - 1 - i of the second axis, the operand
+// [[M, M], [M, -M]] with M = I kron C_w.  Lanes 0..63 then hold the w transform of x[i] + x[n2 - 1 - i], lanes 64..127 that of the
+// difference, and a thread makes the even or the odd coefficients of its position from n2 / 2 numbers a channel.  An item is
+// 64 positions at all n2, 32 channels (n2 = 16, rows of 64 bytes) or 16 (n2 = 32, rows of 32): n2 / 2 tiles, 256 accumulator columns.
+//   warp 0       TMA producer (ring of five batches: half an item, 32 KB)
 //   warp 1       tcgen05.mma issuer; owns the tensor-memory allocation
-//   warps 2..17  epilogue: four warps per 32 lanes, two coefficients each; a warp stages and sends its rows by itself.  (The
-//                four warps of 32 lanes share a scheduler: when they shared the staging area, too, eight channels each, it stood
-//                still at every hand-over.)
+//   warps 2..17  epilogue: four warps per 32 lanes, two or four coefficients each: 64 sums a thread, to which it adds the
+//                accumulators as they come; a warp stages and sends its rows by itself.  (The four warps of 32 lanes share a
+//                scheduler: when they shared the staging area, too, a quarter of the channels each, it stood still at every hand-over.)
 // Every wait is bounded.
 //
-// Bound by HBM and, close behind, by the epilogue: six heads of 64K tokens alone 163 us, 0.9 GB at 5.6 TB/s, issue slots 62%.
-// ff_dct2_tc.cu sends the intermediate through shared memory as a bf16 pair and multiplies t with a 128 x 128 operand that is
-// seven eighths zeros.  Layers before and after (us, 24 heads of 64K tokens at 1.6 GHz 2850 / 2711; all bands 3575 / 3417; 16 heads
-// with head_dim 64 1025 / 967; six heads of 16K 206 / 193, four of 8K 126 / 118, six of 128K 1581 / 1501).  A line of 128
-// positions does not fit twice into the operand: that grid keeps the two-axis launch.  Variants (six heads of 64K): eight channels a
-// thread, staged by four warps together, coefficients as constants of unrolled code 201 us (instruction cache), in a loop 177; packed
-// FMA 181; without its stores that form took 155, without its FMA 163.
-constexpr int FC = 32, FPOS = 64;                          // channels, positions of an item
-constexpr int F_TILE_B = 2 * FPOS * FC * 2;                // 8 KB
-constexpr int F_NSLOT = 5, F_SLOT_B = 4 * F_TILE_B;        // ring
-constexpr int F_BOX_B = 32 * FC * 2;                       // 2 KB: 32 positions at one t, hi or lo
-constexpr int F_STAGE_B = 2 * F_BOX_B;                     // staging area of an epilogue warp
+// n2 = 16: bound by HBM and, close behind, by the epilogue: six heads of 64K tokens alone 163 us, 0.9 GB at 5.6 TB/s, issue slots
+// 62%.  n2 = 32: by its rows of 32 bytes and the epilogue: six heads of 32 x 64 x 64 tokens 365 us, 1.8 GB at 5.0 TB/s, issue slots
+// 57% (75% and 384 us without packed FMA, which with n2 = 16 gain nothing: 724 -> 732 us for six heads of 64 x 16 x 64); stores of 32
+// bytes from the registers 494.
+// ff_dct2_tc.cu sends the intermediate through shared memory as a bf16 pair and multiplies the second axis with a 128 x 128
+// operand of which 128 / n2 - 1 parts are zeros.  Layers before and after (us, at 1.6 GHz): 24 heads of 64K tokens 2850 / 2562; all
+// bands 3575 / 3417; 16 heads with head_dim 64 1025 / 935; six heads of 16K 206 / 193 (190 / 189 with the inverse below), four of 8K
+// 126 / 118, six of 64 x 16 x 64 784 / 724; n2 = 32: two samples of 24 heads of 32 x 64 x 64 10570 / 10300, 12 heads 3115 / 3040, eight
+// with head_dim 64 1205 / 1185, eight of 32 x 64 x 32 998 / 986.  A line of 128 positions does not fit twice into the operand: those
+// grids keep the two-axis launch.  Variants (n2 = 16, six heads of 64K): a quarter of the channels a thread, staged by four warps together,
+// coefficients as constants of unrolled code 201 us (instruction cache), in a loop 177; packed FMA 181; without its stores that form
+// took 155, without its FMA 163.
+constexpr int FPOS = 64;                                   // positions of an item
+template <int N2> struct Fold {
+  static constexpr int C = 512 / N2;                       // channels of an item
+  static constexpr int TILE_B = 2 * FPOS * C * 2, BATCH = 128 / C;       // 8 or 4 KB; tiles of a batch
+  static constexpr int KPW = N2 / 8;                       // coefficients of an epilogue warp
+  static constexpr int BOX_B = 32 * C * 2;                 // 32 positions at one coefficient, hi or lo
+  static constexpr int KPS = N2 / 16;                      // coefficients staged at a time
+  static constexpr int UNROLL = N2 == 32 ? BATCH : 1;      // (what leaves no register spilled)
+};
+constexpr int F_NSLOT = 5, F_SLOT_B = 32 * 1024;           // ring: batches
+constexpr int F_STAGE_B = 4 * 1024;                        // staging area of an epilogue warp
 
-struct T16ForwardShared {
+struct FoldParams {
+  FFDims dm;
+  const uint32_t* img;     // [[M, M], [M, -M]]: hi [128][64] cells, then lo
+  alignas(16) float mat[2][16][16];      // [parity][i][k / 2]: C[k][i] of the second axis
+  int axis2;               // 0 = t, 1 = h
+  int group, group_start;  // tensor-heads of the launch, the first one
+  int nchunk, n3, lines;   // channel chunks; items along the remaining axis, w lines of an item (64 / W)
+  double* clear;           // band energies to clear for the sums that follow (first launch of a routed forward), or NULL
+  int* status;
+};
+
+struct FoldShared {
   uint64_t full[F_NSLOT], empty[F_NSLOT], acc_full[NACC], acc_empty[NACC];
   uint32_t tmem_base;
   int abort_flag;
 };
 
-// Descriptor of an MN-major operand stored as rows of 32 bf16 with the 64-byte swizzle, tiles F_TILE_B apart along N.
-__device__ __forceinline__ uint64_t smem_desc_sw64(uint32_t smem_addr) {
-  return (uint64_t)((smem_addr & 0x3FFFF) >> 4) | (uint64_t)(F_TILE_B >> 4) << 16 | (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)4 << 61;
+// Descriptor of an MN-major operand stored as rows of C bf16 with the swizzle of that width, tiles one after the other along N.
+template <int C>
+__device__ __forceinline__ uint64_t smem_desc_rows(uint32_t smem_addr) {
+  return (uint64_t)((smem_addr & 0x3FFFF) >> 4) | (uint64_t)(2 * FPOS * C * 2 >> 4) << 16 | (uint64_t)(8 * C * 2 >> 4) << 32 | (uint64_t)1 << 46 |
+         (uint64_t)(C == 32 ? 4 : 6) << 61;
 }
-// map0..map2: Q, K, V; map_oh, map_ol: the pair of grids, box = 32 positions at one t.
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, const uint32_t (&v)[4]) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]) : "memory");
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(*(uint64_t*)&d) : "l"(*(uint64_t*)&a), "l"(*(uint64_t*)&b), "l"(*(uint64_t*)&c));
+  return d;
+}
+// map0..map2: Q, K, V; map_oh, map_ol: the pair of grids, box = 32 positions at one coefficient.
+template <int N2>
 __global__ void __launch_bounds__(THREADS, 1)
-dct_t16_forward_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
+dct_fold_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ CUtensorMap map1,
                        const __grid_constant__ CUtensorMap map2, const __grid_constant__ CUtensorMap map_oh,
-                       const __grid_constant__ CUtensorMap map_ol, const __grid_constant__ T16Params P) {
+                       const __grid_constant__ CUtensorMap map_ol, const __grid_constant__ FoldParams P) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const FFDims& dm = P.dm;
+  using F = Fold<N2>;
+  constexpr int FC = F::C;
   constexpr uint32_t COL_ACC = 128;
   uint8_t* sIn = smem;
   uint8_t* sStage = smem + F_NSLOT * F_SLOT_B;              // an area per epilogue warp
-  T16ForwardShared& sh = *(T16ForwardShared*)(sStage + 4 * EPI * F_STAGE_B);
+  FoldShared& sh = *(FoldShared*)(sStage + 4 * EPI * F_STAGE_B);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int total = P.group * P.nh * P.nchunk;
+  const int total = P.group * P.n3 * P.nchunk;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < F_NSLOT; ++i) { mbar_init(&sh.full[i], 1); mbar_init(&sh.empty[i], 1); }
@@ -336,14 +371,14 @@ dct_t16_forward_kernel(const __grid_constant__ CUtensorMap map0, const __grid_co
   tc_fence_after();
 
   FF_CLOCK(t_all);
-  // Item: chunk fastest (CTAs that run side by side read neighbouring pieces of the same rows), then 64 positions, then the tensor-head.
+  // Item: chunk fastest (CTAs that run side by side read neighbouring pieces of the same rows), then the remaining axis, then the tensor-head.
   if (warp == 0) {
     if (lane == 0) {
       tma_prefetch_desc(&map0);
       unsigned n = 0;
       bool ok = true;
       for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
-        const int chunk = it % P.nchunk, rest = it / P.nchunk, p0 = rest % P.nh * FPOS, gi = rest / P.nh;
+        const int chunk = it % P.nchunk, rest = it / P.nchunk, o0 = rest % P.n3 * P.lines, gi = rest / P.n3;
         const int th = P.group_start + gi, tensor = (th >= dm.BH) + (th >= 2 * dm.BH);
         const CUtensorMap* map = tensor == 0 ? &map0 : (tensor == 1 ? &map1 : &map2);
         for (int b = 0; b < 2 && ok; ++b, ++n) {
@@ -355,10 +390,10 @@ dct_t16_forward_kernel(const __grid_constant__ CUtensorMap map0, const __grid_co
           uint8_t* dst = sIn + slot * F_SLOT_B;
           mbar_arrive_expect_tx(&sh.full[slot], F_SLOT_B);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const int i = b * 4 + k;
-            tma_load_5d(dst + k * F_TILE_B, map, &sh.full[slot], chunk * FC, p0, i, th - tensor * dm.BH, 0);
-            tma_load_5d(dst + k * F_TILE_B + F_TILE_B / 2, map, &sh.full[slot], chunk * FC, p0, 15 - i, th - tensor * dm.BH, 0);
+          for (int k = 0; k < F::BATCH; ++k) {
+            const int i = b * F::BATCH + k, j = N2 - 1 - i;
+            tma_load_5d(dst + k * F::TILE_B, map, &sh.full[slot], chunk * FC, 0, P.axis2 ? i : o0, P.axis2 ? o0 : i, th - tensor * dm.BH);
+            tma_load_5d(dst + k * F::TILE_B + F::TILE_B / 2, map, &sh.full[slot], chunk * FC, 0, P.axis2 ? j : o0, P.axis2 ? o0 : j, th - tensor * dm.BH);
           }
         }
       }
@@ -379,27 +414,26 @@ dct_t16_forward_kernel(const __grid_constant__ CUtensorMap map0, const __grid_co
         FF_CLOCK_ADD(lane == 0, 18, ta);
         if (!ok) break;
         tc_fence_after();
-        const uint64_t x = smem_desc_sw64(in_base + slot * F_SLOT_B);
+        const uint64_t x = smem_desc_rows<FC>(in_base + slot * F_SLOT_B);
         const uint32_t d_tm = tm + COL_ACC + ab * 128;
 #pragma unroll
-        for (int ks = 0; ks < ROWS / 16; ++ks) {           // (16 rows of K: 1024 bytes, 64 in a descriptor's address field)
-          umma_ts(d_tm, tm + ks * 8, x + (uint64_t)(ks * 64), idesc, ks > 0 ? 1u : 0u);
-          umma_ts(d_tm, tm + 64 + ks * 8, x + (uint64_t)(ks * 64), idesc, 1u);
+        for (int ks = 0; ks < ROWS / 16; ++ks) {           // (16 rows of K)
+          umma_ts(d_tm, tm + ks * 8, x + (uint64_t)(ks * FC * 2), idesc, ks > 0 ? 1u : 0u);
+          umma_ts(d_tm, tm + 64 + ks * 8, x + (uint64_t)(ks * FC * 2), idesc, 1u);
         }
         umma_commit(&sh.empty[slot]);
         umma_commit(&sh.acc_full[ab]);
       }
     }
   } else {
-    const int quarter = warp & 3, part = (warp - 2) >> 2;  // TMEM lanes; which two of the lanes' eight coefficients
+    const int quarter = warp & 3, part = (warp - 2) >> 2;  // TMEM lanes; which of the lanes' coefficients
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
-    const int k0 = __shfl_sync(0xffffffffu, 4 * part + (quarter >> 1), 0);       // coefficients k0 and k0 + 2
-    uint8_t* stage = sStage + (warp - 2) * F_STAGE_B;
+    const int parity = __shfl_sync(0xffffffffu, quarter >> 1, 0), k0 = __shfl_sync(0xffffffffu, F::KPW * part, 0);
+    const uint32_t stage = smem_u32(sStage) + (warp - 2) * F_STAGE_B;
     unsigned nb = 0;
     bool ok = true;
     for (int it = blockIdx.x; it < total && ok; it += gridDim.x) {
-      const int chunk = it % P.nchunk, rest = it / P.nchunk, p0 = rest % P.nh * FPOS + (quarter & 1) * 32, gi = rest / P.nh;
-      float y[2][FC] = {};
+      float y[F::KPW][FC] = {};
 #pragma unroll 1
       for (int b = 0; b < 2; ++b, ++nb) {
         const int ab = nb % NACC;
@@ -408,50 +442,74 @@ dct_t16_forward_kernel(const __grid_constant__ CUtensorMap map0, const __grid_co
         FF_CLOCK_ADD(threadIdx.x == 64, 19, te);
         if (!ok) break;
         tc_fence_after();
-        const float4 ma = *(const float4*)(P.mat[k0] + 4 * b), mb = *(const float4*)(P.mat[k0 + 2] + 4 * b);
-        const float m[2][4] = {{ma.x, ma.y, ma.z, ma.w}, {mb.x, mb.y, mb.z, mb.w}};
+#pragma unroll F::UNROLL
+        for (int i = 0; i < F::BATCH; ++i) {
+          float m[F::KPW];
+          const float* row = P.mat[parity][b * F::BATCH + i] + k0;
+          if (F::KPW == 2) { const float2 v = *(const float2*)row; m[0] = v.x; m[1] = v.y; }
+          else { const float4 v = *(const float4*)row; m[0] = v.x; m[1] = v.y; m[2] = v.z; m[3] = v.w; }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
+          for (int h = 0; h < FC / 16; ++h) {
             uint32_t x[16];
             tmem_ld16(tm + lane_addr + COL_ACC + ab * 128 + i * FC + h * 16, x);
             tmem_wait_ld();
 #pragma unroll
-            for (int j = 0; j < 2; ++j)
+            for (int j = 0; j < F::KPW; ++j)
 #pragma unroll
-              for (int c = 0; c < 16; ++c) y[j][h * 16 + c] = fmaf(m[j][i], __uint_as_float(x[c]), y[j][h * 16 + c]);
+              for (int c = 0; c < 16; c += 2) {
+                if (N2 == 32) {
+                  const float2 v = fma2(make_float2(m[j], m[j]), make_float2(__uint_as_float(x[c]), __uint_as_float(x[c + 1])),
+                                        make_float2(y[j][h * 16 + c], y[j][h * 16 + c + 1]));
+                  y[j][h * 16 + c] = v.x; y[j][h * 16 + c + 1] = v.y;
+                } else {
+                  y[j][h * 16 + c] = fmaf(m[j], __uint_as_float(x[c]), y[j][h * 16 + c]);
+                  y[j][h * 16 + c + 1] = fmaf(m[j], __uint_as_float(x[c + 1]), y[j][h * 16 + c + 1]);
+                }
+              }
           }
+        }
         tc_fence_before();
         mbar_arrive(&sh.acc_empty[ab]);
       }
       if (!ok) break;
       FF_CLOCK(tw);
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        uint32_t hi[16], lo[16];
-#pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          hi[c] = bf16_pair(__float_as_uint(y[j][2 * c]), __float_as_uint(y[j][2 * c + 1]));
-          lo[c] = bf16_pair(__float_as_uint(y[j][2 * c] - __uint_as_float(hi[c] << 16)), __float_as_uint(y[j][2 * c + 1] - __uint_as_float(hi[c] & 0xffff0000u)));
-        }
+      for (int j0 = 0; j0 < F::KPW; j0 += F::KPS) {
         FF_CLOCK(tb);
         if (lane == 0) bulk_wait_read0();                  // the warp's previous stores have read the area
         __syncwarp();
         FF_CLOCK_ADD(threadIdx.x == 64, 20, tb);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {                      // (64-byte swizzle)
-          uint8_t* at = stage + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4);
-          *(uint4*)at = make_uint4(hi[4 * c], hi[4 * c + 1], hi[4 * c + 2], hi[4 * c + 3]);
-          *(uint4*)(at + F_BOX_B) = make_uint4(lo[4 * c], lo[4 * c + 1], lo[4 * c + 2], lo[4 * c + 3]);
+        for (int j = j0; j < j0 + F::KPS; ++j) {
+          const uint32_t box = stage + (j - j0) * 2 * F::BOX_B;
+#pragma unroll
+          for (int p = 0; p < FC / 8; ++p) {               // 16-byte pieces of the row, under the swizzle
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const float a = y[j][8 * p + 2 * c], e = y[j][8 * p + 2 * c + 1];
+              hi[c] = bf16_pair(__float_as_uint(a), __float_as_uint(e));
+              lo[c] = bf16_pair(__float_as_uint(a - __uint_as_float(hi[c] << 16)), __float_as_uint(e - __uint_as_float(hi[c] & 0xffff0000u)));
+            }
+            const uint32_t at = box + lane * FC * 2 + ((FC == 32 ? p ^ ((lane >> 1) & 3) : p ^ ((lane >> 2) & 1)) << 4);
+            st_shared_v4(at, hi);
+            st_shared_v4(at + F::BOX_B, lo);
+          }
         }
         fence_proxy_async();
         __syncwarp();
         if (lane == 0) {
-          // (debug build) the box lies inside the grid
-          if (FF_DBG_OK((chunk + 1) * FC <= dm.d && p0 + 32 <= dm.H * dm.W && k0 + 2 * j < T && gi < P.group, P.status, 7)) {
-            tma_store_5d(stage, &map_oh, chunk * FC, p0, k0 + 2 * j, gi, 0);
-            tma_store_5d(stage + F_BOX_B, &map_ol, chunk * FC, p0, k0 + 2 * j, gi, 0);
+          const int chunk = it % P.nchunk, rest = it / P.nchunk, gi = rest / P.n3;
+          const int p0 = (quarter & 1) * 32, w0 = p0 % dm.W, o0 = rest % P.n3 * P.lines + p0 / dm.W;      // the warp's first position
+#pragma unroll
+          for (int j = j0; j < j0 + F::KPS; ++j) {
+            const uint8_t* box = sStage + (warp - 2) * F_STAGE_B + (j - j0) * 2 * F::BOX_B;
+            const int k = 2 * (k0 + j) + parity, ch = P.axis2 ? k : o0, ct = P.axis2 ? o0 : k;
+            // (debug build) the box lies inside the grid
+            if (FF_DBG_OK((chunk + 1) * FC <= dm.d && w0 + (dm.W < 32 ? dm.W : 32) <= dm.W && ch < dm.H && ct < dm.T && gi < P.group, P.status, 7)) {
+              tma_store_5d(box, &map_oh, chunk * FC, w0, ch, ct, gi);
+              tma_store_5d(box + F::BOX_B, &map_ol, chunk * FC, w0, ch, ct, gi);
+            }
           }
           bulk_commit();
         }
@@ -476,19 +534,23 @@ dct_t16_forward_kernel(const __grid_constant__ CUtensorMap map0, const __grid_co
   }
 }
 
-// Map over the same grid seen as [slices][t][h w][d]: 32 channels of 64 positions (load) or 32 (store) at one t.
-bool forward_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, bool store) {
+int fold_length(const FFDims& dm, int axis2) { return axis2 ? dm.H : dm.T; }
+
+// Map over a [slices][T][H][W][d] grid: a chunk's channels of 64 positions (load) or 32 (store) at one position of the second axis.
+bool fold_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, bool store) {
   const FFDims& dm = p->dm;
   return p->maps.get(map, base, store ? 51 : 50, slices, [&] {
-    const cuuint64_t ch = (cuuint64_t)dm.d, hw = (cuuint64_t)dm.H * dm.W, plane = hw * ch * 2;
-    const cuuint64_t dims[5] = {ch, hw, T, (cuuint64_t)slices, 1};
-    const cuuint64_t strides[4] = {ch * 2, plane, plane * T, plane * T * slices};
-    const cuuint32_t box[5] = {FC, (cuuint32_t)(store ? 32 : FPOS), 1, 1, 1};
-    return ff_encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_64B,
+    const cuuint64_t ch = (cuuint64_t)dm.d, W = (cuuint64_t)dm.W;
+    const cuuint64_t dims[5] = {ch, W, (cuuint64_t)dm.H, (cuuint64_t)dm.T, (cuuint64_t)slices};
+    const cuuint64_t strides[4] = {ch * 2, W * ch * 2, dm.H * W * ch * 2, (cuuint64_t)dm.N * ch * 2};
+    const cuuint32_t C = (cuuint32_t)(512 / fold_length(dm, p->dct2_axis2)), positions = store ? 32 : FPOS, w = (cuuint32_t)dm.W < positions ? (cuuint32_t)dm.W : positions;
+    cuuint32_t box[5] = {C, w, 1, 1, 1};
+    box[p->dct2_axis2 ? 3 : 2] = positions / w;
+    return ff_encode_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, base, dims, strides, box, C == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
                          store ? CU_TENSOR_MAP_L2_PROMOTION_NONE : CU_TENSOR_MAP_L2_PROMOTION_L2_256B);
   });
 }
-constexpr size_t F_SMEM = 1024 + (size_t)F_NSLOT * F_SLOT_B + 4 * EPI * F_STAGE_B + sizeof(T16ForwardShared);
+constexpr size_t F_SMEM = 1024 + (size_t)F_NSLOT * F_SLOT_B + 4 * EPI * F_STAGE_B + sizeof(FoldShared);
 
 // 5-D map over a [slices][T][H][W][d] bf16 grid: the box of 16 channels of two tiles (load), or of 32 positions at two t (store).
 bool grid_map(ff_plan* p, CUtensorMap* map, const void* base, int slices, bool store) {
@@ -511,7 +573,9 @@ constexpr size_t SMEM = 1024 + (size_t)2 * LO_OFF + 4 * EPI * BOX_B + sizeof(T16
 
 cudaError_t ffk_dct_t16_init() {
   const cudaError_t e = cudaFuncSetAttribute(dct_t16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(dct_t16_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM);
+  if (e != cudaSuccess) return e;
+  const cudaError_t f = cudaFuncSetAttribute(dct_fold_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM);
+  return f != cudaSuccess ? f : cudaFuncSetAttribute(dct_fold_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F_SMEM);
 }
 
 // Where it takes the place of the two-axis launch: t is that launch's second axis, 16 positions, and folds.
@@ -537,32 +601,40 @@ cudaError_t ffk_dct_t16_inverse(ff_plan* p, const void* in_hi, const void* in_lo
   return e;
 }
 
-// Forward: Q, K, V of tensor-heads [g0, g0 + g) -> w and t transform -> hi/lo grids.
-bool ffk_dct_t16_forward_supported(const ff_plan* p) { return ffk_dct_t16_supported(p) && p->dm.W <= FPOS; }
+// Where it takes the place of the two-axis launch.  With 32 positions from 20 items an SM on, all tensor-heads together: four
+// heads of 32 x 64 x 32 tokens (20) take the same time, of 32 x 64 x 64 (41) 1347 -> 1330 us, of 32 x 32 x 16 (5) 170 -> 179.
+bool ffk_dct_fold_supported(const ff_plan* p) {
+  const FFDims& dm = p->dm;
+  const int n2 = fold_length(dm, p->dct2_axis2);
+  if (!p->dct2_ok || p->cfg.transform != FF_TRANSFORM_DCT || dm.W > FPOS || (n2 != 16 && n2 != 32)) return false;
+  return n2 == 16 || 3LL * dm.BH * (dm.N / n2 / FPOS) * (dm.d / Fold<32>::C) >= 20LL * p->sm_count;
+}
 
-cudaError_t ffk_dct_t16_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
-                                bool clear_energy, cudaStream_t st) {
+// Forward: Q, K, V of tensor-heads [g0, g0 + g) -> transform along w and the second axis -> hi/lo grids.
+cudaError_t ffk_dct_fold_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
+                                 bool clear_energy, cudaStream_t st) {
   const FFDims& dm = p->dm;
   CUtensorMap mq, mk, mv, oh, ol;
-  if (!forward_map(p, &mq, Q, dm.BH, false) || !forward_map(p, &mk, K, dm.BH, false) || !forward_map(p, &mv, V, dm.BH, false) ||
-      !forward_map(p, &oh, out_hi, p->dct_group, true) || !forward_map(p, &ol, out_lo, p->dct_group, true))
+  if (!fold_map(p, &mq, Q, dm.BH, false) || !fold_map(p, &mk, K, dm.BH, false) || !fold_map(p, &mv, V, dm.BH, false) ||
+      !fold_map(p, &oh, out_hi, p->dct_group, true) || !fold_map(p, &ol, out_lo, p->dct_group, true))
     return cudaErrorInvalidValue;
-  T16Params P{};
+  FoldParams P{};
+  const int n2 = fold_length(dm, p->dct2_axis2);
   P.dm = dm; P.status = p->buf.status;
   P.img = p->dct2_images + (size_t)6 * FF_IMAGE_CELLS;
-  memcpy(P.mat, p->t16_mat, sizeof(P.mat));
-  P.group = g; P.group_start = g0;
-  P.nchunk = dm.d / FC; P.hpt = FPOS / dm.W; P.nh = dm.H / P.hpt;
+  for (int k = 0; k < n2; ++k) for (int i = 0; i < n2 / 2; ++i) P.mat[k & 1][i][k >> 1] = p->fold_mat[k * (n2 / 2) + i];
+  P.axis2 = p->dct2_axis2; P.group = g; P.group_start = g0;
+  P.nchunk = dm.d / (512 / n2); P.lines = FPOS / dm.W; P.n3 = (P.axis2 ? dm.T : dm.H) / P.lines;
   P.clear = clear_energy ? p->buf.energy : nullptr;
-  const int items = g * P.nh * P.nchunk;
-  const cudaError_t e = ff_launch(dct_t16_forward_kernel, dim3((unsigned)(items < p->sm_count ? items : p->sm_count)), dim3(THREADS), F_SMEM, st,
-                                  mq, mk, mv, oh, ol, P);
+  const int items = g * P.n3 * P.nchunk;
+  const cudaError_t e = ff_launch(n2 == 16 ? dct_fold_kernel<16> : dct_fold_kernel<32>, dim3((unsigned)(items < p->sm_count ? items : p->sm_count)),
+                                  dim3(THREADS), F_SMEM, st, mq, mk, mv, oh, ol, P);
   if (e == cudaSuccess) p->launches += 1;
   return e;
 }
 
 // Its matrix as the tensor-memory A operand, hi and lo parts: [[M, M], [M, -M]], M = I kron C_w over 64 positions.
-bool ffk_dct_t16_build_image(ff_plan* p, const float* mat) {
+bool ffk_dct_fold_build_image(ff_plan* p, const float* mat) {
   const int n = p->dm.W;
   std::vector<uint32_t> img(2 * FF_IMAGE_PART);
   for (int j = 0; j < ROWS; ++j)

@@ -914,7 +914,7 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
       if (e != cudaSuccess) return e;
     }
     if (fused) {
-      e = (p->t16_forward ? ffk_dct_t16_forward : ffk_dct2_forward)(p, Q, K, V, g0, g, sc.a_hi, sc.a_lo, want_energy && g0 == 0, st);
+      e = (p->fold ? ffk_dct_fold_forward : ffk_dct2_forward)(p, Q, K, V, g0, g, sc.a_hi, sc.a_lo, want_energy && g0 == 0, st);
       if (e != cudaSuccess) return e;
       P.in_split = 1; P.out_lo8 = 0; P.reverse = 1;
       P.mode = MODE_SPLIT; P.axis = last_axis; P.image = matrix_image(p, last_axis, 0);

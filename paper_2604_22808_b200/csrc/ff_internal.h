@@ -217,8 +217,9 @@ struct ff_plan {
   FFMapCache maps;                             // tensor maps of the transform passes, by shape
   bool dct2_ok;                                // the fused two-axis launch covers this configuration
   int dct2_axis2;                              // its second axis (1 = h, 0 = t); the remaining axis gets a pass of its own
-  bool t16, t16_forward;                       // ... and the inverse, the forward one is ff_dct_t16.cu
+  bool t16, fold;                              // ... and the inverse, the forward one is ff_dct_t16.cu
   float t16_mat[16][8];                        // C_T[k][i], i < 8
+  float fold_mat[32 * 16];                     // C[k][i] of the second axis, i < n2 / 2
   int dct2_chunk;                              // channels of its work items: 32, or 16 for the larger planes
   alignas(64) unsigned char tmap_mid[128];     // CUtensorMap over the mid-band / high-band coefficient buffers
   alignas(64) unsigned char tmap_high[128];
@@ -280,13 +281,13 @@ bool ffk_dct2_build_image(ff_plan* p, int axis, int inverse, const float* mat_ho
 cudaError_t ffk_dct2_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
                              bool clear_energy, cudaStream_t st);
 cudaError_t ffk_dct2_inverse(ff_plan* p, const void* in_hi, const void* in_lo, int h0, int g, void* out, cudaStream_t st);
-// ---- the same with a t axis of 16 positions in registers (ff_dct_t16.cu) ------------------------------
+// ---- the same with the second axis in registers (ff_dct_t16.cu): inverse with t = 16, forward with 16 or 32 positions --
 cudaError_t ffk_dct_t16_init();
 bool ffk_dct_t16_supported(const ff_plan* p);
-bool ffk_dct_t16_forward_supported(const ff_plan* p);
-bool ffk_dct_t16_build_image(ff_plan* p, const float* mat_host);
-cudaError_t ffk_dct_t16_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
-                                bool clear_energy, cudaStream_t st);
+bool ffk_dct_fold_supported(const ff_plan* p);
+bool ffk_dct_fold_build_image(ff_plan* p, const float* mat_host);
+cudaError_t ffk_dct_fold_forward(ff_plan* p, const void* Q, const void* K, const void* V, int g0, int g, void* out_hi, void* out_lo,
+                                 bool clear_energy, cudaStream_t st);
 cudaError_t ffk_dct_t16_inverse(ff_plan* p, const void* in_hi, const void* in_lo, int h0, int g, void* out, cudaStream_t st);
 // ---- projections around the path (ff_proj_tc.cu) -------------------------------------------------------
 bool ffk_proj_supported(const FFDims& dm);

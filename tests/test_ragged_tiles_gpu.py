@@ -9,8 +9,7 @@ from paper_2604_22808_b200 import configs as C
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("grid", [(21, 45, 80), (40, 33, 50), (9, 100, 66), (48, 24, 60)], ids=lambda g: "x".join(map(str, g)))
-@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("grid,d", [((21, 45, 80), 128), ((9, 100, 66), 128), ((40, 33, 50), 64), ((48, 24, 60), 128)], ids=str)
 def test_many_tiles(grid, d):
     import torch
     from paper_2604_22808_b200 import binding as B
