@@ -56,7 +56,7 @@ struct TcParams {
 };
 
 // (ff_high_attention_noalloc only; the plan's worklist is built where its allocation is decided)
-__global__ void build_worklist_kernel(TcParams P) { build_worklist(P.dm, P.alloc, 0, P.work); }
+__global__ void build_worklist_kernel(TcParams P) { build_worklist(P.dm, P.alloc, 0, 0, P.work); }
 
 struct Item {
   int band, bh, c;

@@ -5,7 +5,10 @@
 // The router needs the energies of every block, so the block that finishes last (a ticket counter owned by the plan)
 // runs it.  What these steps cost is latency, not work: as five launches (low-band energy, router, pooling, worklist
 // and the fp32 path's energies) they took 53 us of a 16K-token layer, the router alone 29 us with its second layer
-// read by three threads.
+// read by three threads.  By clocks of the last block (six heads of 16K tokens, 27 000 cycles) the hidden layer took 9400, its
+// weights read in rounds of eight inputs and then one by one, the second layer 2800, e(t) 2300 before the launch's wait, which
+// nothing overlaps there: now the weights are asked for ahead, e(t) is made beside the energies.  The launch alone 14.6 -> 10.2 us,
+// layers 188.5 -> 184.8 (four heads of 8K 118.5 -> 115.4, 256 fp32 tokens 29.6 -> 28.7).
 #include "ff_bands.cuh"
 #include "ff_internal.h"
 #include "ff_worklist.cuh"
@@ -13,6 +16,8 @@
 namespace {
 
 constexpr int ST_THREADS = 512;
+constexpr int ST_MASKS = 512;            // band masks kept in shared memory for the worklist
+constexpr int ST_ROWS = 8;               // rows of a pooled token that a thread reads at a time
 constexpr int ST_STEPS = 8;              // rows per thread of a mid / high block
 
 struct StatsParams {
@@ -26,6 +31,7 @@ struct StatsParams {
   const uint8_t* alloc_in;               // the caller's masks, or NULL to route
   uint8_t* alloc; float* pi;
   int* work; int low_on;                 // attention worklist (NULL: the tensor-core kernel does not run)
+  int mid_items;                         // items of one head's mid band in it
   unsigned* ticket;
   int n_low, n_mid;                      // blocks of the low and of the mid band (the rest: high band); 0: not covered
   int low_steps;                         // pooled tokens per thread of a low block
@@ -40,10 +46,10 @@ __device__ __forceinline__ void prefetch_line(const float* p, int line, int n) {
   if (line < (n + 31) / 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + line * 32));
 }
 
-// Sinusoidal embedding of the sample's timestep into et[dt]: double-precision sines that depend on no other kernel.
+// Sinusoidal embedding of the sample's timestep into et[dt], in double precision; by the block's last warp if it is that short.
 __device__ void embed_timestep(const StatsParams& P, int sample, float* et) {
-  const int half = P.dm.dt / 2;
-  for (int k = threadIdx.x; k < half; k += ST_THREADS) {
+  const int half = P.dm.dt / 2, threads = half <= 32 ? 32 : ST_THREADS;
+  for (int k = (int)threadIdx.x - (ST_THREADS - threads); k >= 0 && k < half; k += threads) {
     const double t = (double)(P.timestep ? P.timestep[sample] : P.ts[sample]);
     const double om = exp2(-(double)k / (double)half * 13.287712379549449);     // 10000^(-k/half); log2(10000)
     double sn, cs;
@@ -53,9 +59,11 @@ __device__ void embed_timestep(const StatsParams& P, int sample, float* et) {
   }
 }
 
-// z = W2 relu(W1 [g; e(t)] + b1) + b2, pi = softmax(z), largest-remainder quota, one-hot masks; a whole block.  e(t) is
-// in place already.
-__device__ void route_sample(const StatsParams& P, int sample, float* sm) {
+// z = W2 relu(W1 [g; e(t)] + b1) + b2, pi = softmax(z), largest-remainder quota, one-hot masks; a whole block.  A chain of
+// latencies: everything that does not depend on the step before is under way by then (the weights of a layer, e(t) on a warp of
+// its own).
+constexpr int ST_AHEAD = 7;              // inputs of a hidden unit that a lane holds weights of at a time
+__device__ void route_sample(const StatsParams& P, int sample, float* sm, uint8_t* masks) {
   const FFDims& dm = P.dm;
   const int d = dm.d, nin = 3 * d + dm.dt, hid = dm.hid;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -63,6 +71,21 @@ __device__ void route_sample(const StatsParams& P, int sample, float* sm) {
   float* h = sm + nin;      // [hid]
   __shared__ float z[3];
   __shared__ int first[4];  // first head of each band
+  // hidden layer: four units per warp at a time, lanes stride over the inputs (coalesced rows of W1)
+  float w[4][ST_AHEAD];
+  auto weights = [&](int j0, int i0) {
+#pragma unroll
+    for (int t = 0; t < ST_AHEAD; ++t) {
+      const int i = i0 + 32 * t + lane;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w[k][t] = i < nin && j0 + k < hid ? P.W1[(size_t)(j0 + k) * nin + i] : 0.f;
+    }
+  };
+  weights(warp * 4, 0);
+  const float w2 = warp < 3 && lane < hid ? P.W2[warp * hid + lane] : 0.f, w2b = warp < 3 && lane + 32 < hid ? P.W2[warp * hid + lane + 32] : 0.f;
+  const float bias2 = warp < 3 ? P.b2[warp] : 0.f;
+  float bias1 = lane < 4 && warp * 4 + lane < hid ? P.b1[warp * 4 + lane] : 0.f;
+  embed_timestep(P, sample, x + 3 * d);
   for (int i = tid; i < 3 * d; i += ST_THREADS) {
     const int band = i / d;
     const long long cnt = band == 0 ? dm.Nlow : (band == 1 ? dm.Nmid : dm.Nhigh);
@@ -70,27 +93,32 @@ __device__ void route_sample(const StatsParams& P, int sample, float* sm) {
     x[i] = (float)log1p(__ldcg(P.energy + (size_t)sample * 3 * d + i) / terms);
   }
   __syncthreads();
-  // hidden layer: four units per warp at a time, lanes stride over the inputs (coalesced rows of W1)
   for (int j0 = warp * 4; j0 < hid; j0 += (ST_THREADS / 32) * 4) {
     float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-    for (int i = lane; i < nin; i += 32) {
+    for (int i0 = 0; i0 < nin; i0 += 32 * ST_AHEAD) {
+      if (i0 > 0 || j0 != warp * 4) weights(j0, i0);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) acc[k] = fmaf(P.W1[(size_t)(j0 + k < hid ? j0 + k : j0) * nin + i], x[i], acc[k]);
+      for (int t = 0; t < ST_AHEAD; ++t) {
+        const float v = i0 + 32 * t + lane < nin ? x[i0 + 32 * t + lane] : 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[k] = fmaf(w[k][t], v, acc[k]);
+      }
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[k] = warp_sum(acc[k]);
     if (lane < 4 && j0 + lane < hid) {
       const float v = lane == 0 ? acc[0] : (lane == 1 ? acc[1] : (lane == 2 ? acc[2] : acc[3]));
-      h[j0 + lane] = fmaxf(v + P.b1[j0 + lane], 0.f);
+      if (j0 != warp * 4) bias1 = P.b1[j0 + lane];
+      h[j0 + lane] = fmaxf(v + bias1, 0.f);
     }
   }
   __syncthreads();
   if (warp < 3) {
-    float acc = 0.f;
-    for (int j = lane; j < hid; j += 32) acc = fmaf(P.W2[warp * hid + j], h[j], acc);
+    float acc = lane < hid ? w2 * h[lane] : 0.f;
+    if (lane + 32 < hid) acc = fmaf(w2b, h[lane + 32], acc);
+    for (int j = lane + 64; j < hid; j += 32) acc = fmaf(P.W2[warp * hid + j], h[j], acc);
     acc = warp_sum(acc);
-    if (lane == 0) z[warp] = acc + P.b2[warp];
+    if (lane == 0) z[warp] = acc + bias2;
   }
   __syncthreads();
   if (tid == 0) {
@@ -114,15 +142,19 @@ __device__ void route_sample(const StatsParams& P, int sample, float* sm) {
     first[0] = 0; first[1] = base[0]; first[2] = base[0] + base[1]; first[3] = 0;
   }
   __syncthreads();
-  for (int hix = tid; hix < dm.heads; hix += ST_THREADS)
-    P.alloc[sample * dm.heads + hix] = hix < first[1] ? FF_BAND_LOW : (hix < first[2] ? FF_BAND_MID : FF_BAND_HIGH);
+  for (int hix = tid; hix < dm.heads; hix += ST_THREADS) {
+    const uint8_t mask = hix < first[1] ? FF_BAND_LOW : (hix < first[2] ? FF_BAND_MID : FF_BAND_HIGH);
+    P.alloc[sample * dm.heads + hix] = mask;
+    if (sample * dm.heads + hix < ST_MASKS) masks[sample * dm.heads + hix] = mask;
+  }
   __syncthreads();                                          // (the next sample reuses the shared memory; the worklist reads the masks)
 }
 
 template <typename ST>
-__global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_constant__ StatsParams P) {
+__global__ void __launch_bounds__(ST_THREADS, 2) band_stats_kernel(const __grid_constant__ StatsParams P) {
   extern __shared__ float sm[];
   __shared__ bool last;
+  __shared__ uint8_t masks[ST_MASKS];
   const FFDims& dm = P.dm;
   // (any block may turn out to be the one that routes; the sums below use other shared memory)
   float* mlp = sm + (ST_THREADS / (dm.d / 4)) * dm.d;
@@ -134,7 +166,6 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
     prefetch_line(P.W2, line, 3 * dm.hid);
     prefetch_line(P.b1, line, dm.hid);
     prefetch_line(P.b2, line, 3);
-    if (!P.timestep) embed_timestep(P, 0, mlp + 3 * dm.d);
   }
   // (a router keeps one block busy long after the others: let in early, the next launch's blocks settle unevenly meanwhile.
   // With masks given there is little to wait for: 4 x 19 x 16 fp32 tokens, six heads, all bands, 55.6 us, let in late 61.1)
@@ -153,11 +184,15 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
         const float* src = P.spec_low + ((size_t)th * dm.Nlow + p0) * d + vec * 4;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
         const int n = (int)(p1 - p0);
-#pragma unroll 4
-        for (int i = 0; i < n; ++i) {
-          const float4 x = ld4(src + (size_t)i * d);
-          acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
-          add_squares(e, x);
+        for (int i0 = 0; i0 < n; i0 += ST_ROWS) {
+          float4 x[ST_ROWS];
+#pragma unroll
+          for (int i = 0; i < ST_ROWS; ++i) x[i] = i0 + i < n ? ld4(src + (size_t)(i0 + i) * d) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int i = 0; i < ST_ROWS; ++i) {
+            acc.x += x[i].x; acc.y += x[i].y; acc.z += x[i].z; acc.w += x[i].w;
+            add_squares(e, x[i]);
+          }
         }
         const float fn = (float)n;
         acc = make_float4(acc.x / fn, acc.y / fn, acc.z / fn, acc.w / fn);
@@ -192,7 +227,7 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
     if (blockIdx.x == 0 && blockIdx.y == 0) {
       for (int i = threadIdx.x; i < dm.BH; i += ST_THREADS) P.alloc[i] = P.alloc_in[i];
       __syncthreads();
-      if (P.work && threadIdx.x < 32) build_worklist(dm, P.alloc, P.low_on, P.work);
+      if (P.work && threadIdx.x < 32) build_worklist(dm, P.alloc, P.low_on, P.mid_items, P.work);
     }
     return;
   }
@@ -204,10 +239,9 @@ __global__ void __launch_bounds__(ST_THREADS) band_stats_kernel(const __grid_con
   __threadfence();
   if (threadIdx.x == 0) *P.ticket = 0;
   for (int sample = 0; sample < dm.B; ++sample) {
-    if (sample > 0 || P.timestep) embed_timestep(P, sample, mlp + 3 * d);
-    route_sample(P, sample, mlp);
+    route_sample(P, sample, mlp, masks);
   }
-  if (P.work && threadIdx.x < 32) build_worklist(dm, P.alloc, P.low_on, P.work);
+  if (P.work && threadIdx.x < 32) build_worklist(dm, dm.BH <= ST_MASKS ? masks : P.alloc, P.low_on, P.mid_items, P.work);
 }
 
 // More timesteps than fit the statistics' arguments, in launches of their own: a copy from the caller's memory would be
@@ -256,6 +290,7 @@ cudaError_t ffk_band_stats(ff_plan* p, const uint8_t* alloc_in, const float* tim
   P.ticket = p->tickets;
   const bool tc = p->tc_ok && !(p->attn_impl & 1);
   P.work = tc ? p->buf.work : nullptr; P.low_on = p->low_tc_ok ? 1 : 0;
+  P.mid_items = mid_shape(dm).items;
   if (!alloc_in) {
     P.energy = p->buf.energy;
     P.W1 = p->W1; P.b1 = p->b1; P.W2 = p->W2; P.b2 = p->b2;

@@ -33,8 +33,8 @@ __host__ __device__ __forceinline__ MidShape mid_shape(const FFDims& dm) {
 #if defined(__CUDACC__)
 // One unit per (head, band) that the allocation executes, called by a whole warp: the low band's units first (when
 // `low_on`), then the mid band's (their items are the long ones), then the high band's.  The units of a band have
-// equally many items, so a unit's number and first item follow from a ballot.
-__device__ __forceinline__ void build_worklist(const FFDims& dm, const uint8_t* alloc, int low_on, int* work) {
+// equally many items (`mid_items` of the mid band), so a unit's number and first item follow from a ballot.
+__device__ __forceinline__ void build_worklist(const FFDims& dm, const uint8_t* alloc, int low_on, int mid_items, int* work) {
   const int lane = threadIdx.x & 31;
   int* offsets = work + 2;
   int* desc = offsets + FF_MAX_UNITS + 1;
@@ -44,7 +44,7 @@ __device__ __forceinline__ void build_worklist(const FFDims& dm, const uint8_t* 
     // (the anchor pattern of the mid band is not a union of dense classes: those heads run on the generic kernel)
     if (band == 1 && dm.pattern != FF_MID_STRIDED) continue;
     const int nt = band == 1 ? 0 : (int)(((band == 0 ? dm.Nbar : dm.Nhigh) + FF_TILE - 1) / FF_TILE);
-    const int items = band == 1 ? mid_shape(dm).items : (nt + 1) / 2;
+    const int items = band == 1 ? mid_items : (nt + 1) / 2;
     for (int base = 0; base < dm.BH; base += 32) {
       const int bh = base + lane;
       const bool has = bh < dm.BH && (alloc[bh] & (1 << band));
