@@ -184,9 +184,12 @@ cudaError_t launch_dct_pass(ff_plan* p, DctPassParams& P, int group, cudaStream_
 // All three axes of a small grid in one launch: a block holds eight channels of a tensor-head's whole grid in shared
 // memory and transforms it in place, axis by axis (lines are handled in rounds: everything a round reads is in
 // registers before any of it is overwritten).  Small grids are bound by launches and latency: 4 x 8 x 8 tokens take
-// one launch of 6 us instead of three of 5.
+// one launch of 6 us instead of three of 5.  Up to 256 positions a thread computes two outputs instead of eight: eight keep a quarter
+// of the threads or fewer busy (layers, us, eight / two: 4 x 8 x 8 routed 28.7 / 27.55, 2 x 10 x 12 33.6 / 32.25, 2 x 2 x 64 33.9 / 32.0,
+// 2 x 6 x 8 30.3 / 28.9; 5 x 9 x 10, 450 positions, 40.7 / 41.2, 4 x 16 x 8 42.3 / 42.8).
 // ------------------------------------------------------------------------------------------------
 constexpr int VOL_CH = 8, VOL_THREADS = 256;
+constexpr int VOL_FINE = 256;            // positions, up to which a thread computes two outputs of a line instead of eight
 constexpr int VOL_MAX = 2304;            // positions: 72 KB, so that three blocks share an SM
 
 struct VolParams {
@@ -199,7 +202,8 @@ struct VolParams {
   double* clear;
 };
 
-template <typename ST, bool INVERSE>
+// OUT: outputs (of four channels each) that a thread computes of a line.
+template <typename ST, bool INVERSE, int OUT>
 __global__ void __launch_bounds__(VOL_THREADS) dct_volume_kernel(const __grid_constant__ VolParams P) {
   extern __shared__ float4 vol[];                      // [N][2]
   const FFDims& dm = P.dm;
@@ -224,10 +228,10 @@ __global__ void __launch_bounds__(VOL_THREADS) dct_volume_kernel(const __grid_co
   for (int step = 0; step < 3; ++step) {
     const int axis = INVERSE ? step : 2 - step;
     const int n = axis == 2 ? dm.W : (axis == 1 ? dm.H : dm.T), stride = axis == 2 ? 1 : (axis == 1 ? dm.W : dm.H * dm.W);
-    const int npad = (n + 7) & ~7, groups = npad / 8;
+    const int npad = (n + 7) & ~7, groups = OUT == 8 ? npad / 8 : (n + OUT - 1) / OUT;
     const int at = axis == 0 ? 0 : dm.T * ((dm.T + 7) & ~7) + (axis == 1 ? 0 : dm.H * ((dm.H + 7) & ~7));
     const float* mt = mats + at;
-    const int upl = 2 * groups, lines = N / n;           // units (8 outputs x 4 channels) of a line
+    const int upl = 2 * groups, lines = N / n;           // units (OUT outputs x 4 channels) of a line
     const int lpr = VOL_THREADS / upl;                   // lines per round
     const int l = tid / upl, u = tid - l * upl, cg = u & 1, g = u >> 1;
     for (int l0 = 0; l0 < lines; l0 += lpr) {
@@ -235,22 +239,27 @@ __global__ void __launch_bounds__(VOL_THREADS) dct_volume_kernel(const __grid_co
       const bool on = l < lpr && line < lines;
       const int base = axis == 0 ? line : (line / stride) * stride * n + line % stride;
       float4* x = vol + 2 * base + cg;
-      float4 acc[8];
+      float4 acc[OUT];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int i = 0; i < OUT; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (on)
 #pragma unroll 4
         for (int b = 0; b < n; ++b) {
           const float4 v = x[2 * b * stride];
-          const float4 m0 = *(const float4*)(mt + b * npad + g * 8), m1 = *(const float4*)(mt + b * npad + g * 8 + 4);
-          fma4(acc[0], m0.x, v); fma4(acc[1], m0.y, v); fma4(acc[2], m0.z, v); fma4(acc[3], m0.w, v);
-          fma4(acc[4], m1.x, v); fma4(acc[5], m1.y, v); fma4(acc[6], m1.z, v); fma4(acc[7], m1.w, v);
+          if (OUT == 2) {
+            const float2 m = *(const float2*)(mt + b * npad + g * 2);
+            fma4(acc[0], m.x, v); fma4(acc[1], m.y, v);
+          } else {
+            const float4 m0 = *(const float4*)(mt + b * npad + g * 8), m1 = *(const float4*)(mt + b * npad + g * 8 + 4);
+            fma4(acc[0], m0.x, v); fma4(acc[1], m0.y, v); fma4(acc[2 % OUT], m0.z, v); fma4(acc[3 % OUT], m0.w, v);
+            fma4(acc[4 % OUT], m1.x, v); fma4(acc[5 % OUT], m1.y, v); fma4(acc[6 % OUT], m1.z, v); fma4(acc[7 % OUT], m1.w, v);
+          }
         }
       __syncthreads();
       if (on)
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          if (g * 8 + i < n) x[2 * (g * 8 + i) * stride] = acc[i];
+        for (int i = 0; i < OUT; ++i)
+          if (g * OUT + i < n) x[2 * (g * OUT + i) * stride] = acc[i];
     }
     __syncthreads();
   }
@@ -707,7 +716,7 @@ static cudaError_t forward_transform_t(ff_plan* p, const void* Q, const void* K,
     P.spec_low = p->buf.spec_low; P.spec_mid = p->buf.spec_mid; P.spec_high = p->buf.spec_high;
     P.clear = want_energy ? p->buf.energy : nullptr;
     p->launches += 1;
-    return ff_launch(dct_volume_kernel<ST, false>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)(3 * dm.BH)), dim3(VOL_THREADS),
+    return ff_launch(dm.N <= VOL_FINE ? dct_volume_kernel<ST, false, 2> : dct_volume_kernel<ST, false, 8>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)(3 * dm.BH)), dim3(VOL_THREADS),
                      vol_smem(dm), st, P);
   }
   const int total = 3 * dm.BH, G = p->lay.group;
@@ -845,7 +854,7 @@ static cudaError_t exchange_inverse_t(ff_plan* p, void* out, cudaStream_t st) {
       P.src[0] = p->buf.scratchA; P.out = out; P.dm = dm; P.group_start = h0;
       for (int a = 0; a < 3; ++a) P.mat_t[a] = p->basis[a];
       p->launches += 1;
-      e = ff_launch(dct_volume_kernel<ST, true>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)g), dim3(VOL_THREADS), vol_smem(dm), st, P);
+      e = ff_launch(dm.N <= VOL_FINE ? dct_volume_kernel<ST, true, 2> : dct_volume_kernel<ST, true, 8>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)g), dim3(VOL_THREADS), vol_smem(dm), st, P);
       if (e != cudaSuccess) return e;
       continue;
     }
@@ -879,7 +888,8 @@ cudaError_t ffk_simt_init() {
   FF_SET(attention_simt_kernel<T, D>); FF_SET(exchange_recombine_kernel<T, D, float>)
 #define FF_SET_T(T)                                                                            \
   FF_SET(dct_pass_kernel<T, 0>); FF_SET(dct_pass_kernel<T, 1>); FF_SET(dct_pass_kernel<T, 2>); FF_SET(dct_pass_kernel<T, 3>); \
-  FF_SET(dct_volume_kernel<T, false>); FF_SET(dct_volume_kernel<T, true>);                     \
+  FF_SET(dct_volume_kernel<T, false, 2>); FF_SET(dct_volume_kernel<T, true, 2>);               \
+  FF_SET(dct_volume_kernel<T, false, 8>); FF_SET(dct_volume_kernel<T, true, 8>);               \
   FF_SET_D(T, 1); FF_SET_D(T, 2); FF_SET_D(T, 3); FF_SET_D(T, 4)
   FF_SET_T(float); FF_SET_T(__nv_bfloat16);
   FF_SET(exchange_recombine_kernel<__nv_bfloat16, 2, __nv_bfloat16>); FF_SET(exchange_recombine_kernel<__nv_bfloat16, 4, __nv_bfloat16>);
