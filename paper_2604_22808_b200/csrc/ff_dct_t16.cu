@@ -72,13 +72,14 @@ __device__ __forceinline__ uint64_t smem_desc_sw32(uint32_t smem_addr) {
   return (uint64_t)((smem_addr & 0x3FFFF) >> 4) | (uint64_t)(TILE_B >> 4) << 16 | (uint64_t)(256 >> 4) << 32 | (uint64_t)1 << 46 | (uint64_t)6 << 61;
 }
 
-// The matrix (hi, then lo part) into tensor memory by four warps: a thread loads the row of its lane.
+// The matrix (hi part, the lo part LO cells behind it) into tensor memory by four warps: a thread loads the row of its lane.
+template <size_t LO>
 __device__ __forceinline__ void matrix_to_tmem(const uint32_t* img, uint32_t tm, int quarter, int lane) {
   const int row = quarter * 32 + lane;
   const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
 #pragma unroll 1
   for (int c0 = 0; c0 < 128; c0 += 32) {
-    const uint32_t* src = img + (size_t)(c0 >> 6) * FF_IMAGE_PART + (size_t)row * 64 + (c0 & 63);
+    const uint32_t* src = img + (size_t)(c0 >> 6) * LO + (size_t)row * 64 + (c0 & 63);
     uint32_t r[32];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -116,7 +117,7 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
   tc_fence_after();
   const uint32_t tm = sh.tmem_base;
   volatile int* abort_flag = &sh.abort_flag;
-  if (warp >= 2 && warp < 6) matrix_to_tmem(P.img, tm, warp & 3, lane);
+  if (warp >= 2 && warp < 6) matrix_to_tmem<FF_IMAGE_PART>(P.img, tm, warp & 3, lane);
   // (the next launch comes in when this one's blocks end: let in earlier, its blocks slowed the last third of this
   // launch down, 16K tokens, six heads: 30.6 us instead of 22.3)
   ff_pdl_join();
@@ -299,12 +300,13 @@ template <int N2> struct Fold {
   static constexpr int KPS = N2 / 16;                      // coefficients staged at a time
   static constexpr int UNROLL = N2 == 32 ? BATCH : 1;      // (what leaves no register spilled)
 };
+constexpr size_t FOLD_IMAGE = 2 * FF_IMAGE_PART;           // hi and lo: the third parts of the first two images, which these grids leave unused
 constexpr int F_NSLOT = 5, F_SLOT_B = 32 * 1024;           // ring: batches
 constexpr int F_STAGE_B = 4 * 1024;                        // staging area of an epilogue warp
 
 struct FoldParams {
   FFDims dm;
-  const uint32_t* img;     // [[M, M], [M, -M]]: hi [128][64] cells, then lo
+  const uint32_t* img;     // [[M, M], [M, -M]]: hi [128][64] cells, lo FF_IMAGE_CELLS behind it
   alignas(16) float mat[2][16][16];      // [parity][i][k / 2]: C[k][i] of the second axis
   int axis2;               // 0 = t, 1 = h
   int group, group_start;  // tensor-heads of the launch, the first one
@@ -363,7 +365,7 @@ dct_fold_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant_
   tc_fence_after();
   const uint32_t tm = sh.tmem_base;
   volatile int* abort_flag = &sh.abort_flag;
-  if (warp >= 2 && warp < 6) matrix_to_tmem(P.img, tm, warp & 3, lane);
+  if (warp >= 2 && warp < 6) matrix_to_tmem<FF_IMAGE_CELLS>(P.img, tm, warp & 3, lane);
   ff_pdl_wait();
   if (P.clear && blockIdx.x == 0) for (int i = threadIdx.x; i < dm.B * 3 * dm.d; i += THREADS) P.clear[i] = 0.0;
   tc_fence_before();
@@ -606,7 +608,7 @@ cudaError_t ffk_dct_t16_inverse(ff_plan* p, const void* in_hi, const void* in_lo
 bool ffk_dct_fold_supported(const ff_plan* p) {
   const FFDims& dm = p->dm;
   const int n2 = fold_length(dm, p->dct2_axis2);
-  if (!p->dct2_ok || p->cfg.transform != FF_TRANSFORM_DCT || dm.W > FPOS || (n2 != 16 && n2 != 32)) return false;
+  if (!p->dct2_ok || ff_fp32_grid(dm) || p->cfg.transform != FF_TRANSFORM_DCT || dm.W > FPOS || (n2 != 16 && n2 != 32)) return false;
   return n2 == 16 || 3LL * dm.BH * (dm.N / n2 / FPOS) * (dm.d / Fold<32>::C) >= 20LL * p->sm_count;
 }
 
@@ -621,7 +623,7 @@ cudaError_t ffk_dct_fold_forward(ff_plan* p, const void* Q, const void* K, const
   FoldParams P{};
   const int n2 = fold_length(dm, p->dct2_axis2);
   P.dm = dm; P.status = p->buf.status;
-  P.img = p->dct2_images + (size_t)6 * FF_IMAGE_CELLS;
+  P.img = p->dct2_images + FOLD_IMAGE;
   for (int k = 0; k < n2; ++k) for (int i = 0; i < n2 / 2; ++i) P.mat[k & 1][i][k >> 1] = p->fold_mat[k * (n2 / 2) + i];
   P.axis2 = p->dct2_axis2; P.group = g; P.group_start = g0;
   P.nchunk = dm.d / (512 / n2); P.lines = FPOS / dm.W; P.n3 = (P.axis2 ? dm.T : dm.H) / P.lines;
@@ -637,21 +639,20 @@ cudaError_t ffk_dct_fold_forward(ff_plan* p, const void* Q, const void* K, const
 bool ffk_dct_fold_build_image(ff_plan* p, const float* mat) {
   const int n = p->dm.W;
   std::vector<uint32_t> img(2 * FF_IMAGE_PART);
-  for (int j = 0; j < ROWS; ++j)
-    for (int r = 0; r < ROWS; ++r) {
-      const int a = j % FPOS, b = r % FPOS;
-      if (a / n != b / n) continue;
-      float v = mat[(a % n) * n + b % n];
-      if (j >= FPOS && r >= FPOS) v = -v;
-      size_t cell = (size_t)j * 64 + (r >> 1);
-      for (int part = 0; part < 2; ++part, cell += FF_IMAGE_PART) {
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        const uint32_t hb = *(const uint16_t*)&h;
-        img[cell] |= (r & 1) ? hb << 16 : hb;
-        v -= __bfloat162float(h);
+  for (int a = 0; a < n; ++a)
+    for (int b = 0; b < n; b += 2) {
+      float v[2] = {mat[a * n + b], mat[a * n + b + 1]};
+      for (int part = 0; part < 2; ++part) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v[0], v[1]);
+        const uint32_t cell = *(const uint32_t*)&h;
+        v[0] -= __low2float(h); v[1] -= __high2float(h);
+        for (int l = 0; l < ROWS; l += n)                // the lines of the rows, and the same line in both halves of the columns
+          for (int r = l % FPOS; r < ROWS; r += FPOS)
+            img[part * FF_IMAGE_PART + (size_t)(l + a) * 64 + ((r + b) >> 1)] = l >= FPOS && r >= FPOS ? cell ^ 0x80008000u : cell;
       }
     }
-  return cudaMemcpy(p->dct2_images + (size_t)6 * FF_IMAGE_CELLS, img.data(), img.size() * sizeof(uint32_t), cudaMemcpyHostToDevice) == cudaSuccess;
+  const size_t row = FF_IMAGE_PART * sizeof(uint32_t);
+  return cudaMemcpy2D(p->dct2_images + FOLD_IMAGE, FF_IMAGE_CELLS * sizeof(uint32_t), img.data(), row, row, 2, cudaMemcpyHostToDevice) == cudaSuccess;
 }
 
 FF_CLOCKS_READ(transform_t16)

@@ -144,7 +144,7 @@ FF_HD bool ff_fp32_grid(const FFDims& dm) { return !(ff_tile_axis(dm.T) && ff_ti
 // Transform matrix of an axis as tensor-memory operand images: [3 parts][128 rows][64 cells of two bf16]; the first two
 // parts are the bf16 pair, all three the fp32 value.
 constexpr size_t FF_IMAGE_PART = (size_t)128 * 64, FF_IMAGE_CELLS = 3 * FF_IMAGE_PART;
-constexpr int FF_IMAGES = 7;
+constexpr int FF_IMAGES = 6;
 
 // SMs for the rules that shape the workspace: its size is a function of the configuration alone (it is asked for without
 // a device).  Rules that shape only a launch take the device's count.
@@ -213,7 +213,7 @@ struct ff_plan {
   int* pos_table;                              // rank -> flat coefficient index of the mid, then the high band (plan-owned)
   alignas(64) unsigned char tmap_x[4][128];    // CUtensorMaps of the exchange kernel (Y / V~ of the mid and high bands)
   uint32_t* dct2_images;                       // transform matrices as tensor-memory operand images (plan-owned): three axes forward,
-                                               // inverse, and the folded one of ff_dct_t16.cu
+                                               // inverse; in unused parts the folded one of ff_dct_t16.cu
   FFMapCache maps;                             // tensor maps of the transform passes, by shape
   bool dct2_ok;                                // the fused two-axis launch covers this configuration
   int dct2_axis2;                              // its second axis (1 = h, 0 = t); the remaining axis gets a pass of its own
