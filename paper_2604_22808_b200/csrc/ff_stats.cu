@@ -258,10 +258,11 @@ size_t router_bytes(const FFDims& dm) { return (size_t)(3 * dm.d + dm.dt + dm.hi
 
 }  // namespace
 
-// (routers up to what a block can have; a wider one fails where it is used, with the launch's error)
+// (routers up to what a block can have; a wider one fails where it is used, with the launch's error.  The 48 KB of a launch that asked
+// for nothing hold the kernel's static arrays, too: 544 bytes)
 cudaError_t ffk_stats_init(const FFDims& dm) {
-  const size_t most = 226 * 1024, need = sums_bytes(dm) + router_bytes(dm);
-  if (need <= 48 * 1024) return cudaSuccess;
+  const size_t most = 226 * 1024, beside = 1024, need = sums_bytes(dm) + router_bytes(dm);     // (of 227 KB)
+  if (need + beside <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(dm.fp32 ? band_stats_kernel<float> : band_stats_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)(need < most ? need : most));
 }

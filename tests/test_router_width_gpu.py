@@ -1,5 +1,9 @@
 """Routers wider than the shared memory a block has by default, and one wider than it can have: the layer runs under a given
 allocation all the same."""
+import os
+import subprocess
+import sys
+
 import pytest
 
 from paper_2604_22808_b200 import configs as C
@@ -26,3 +30,23 @@ def test_wider_than_shared_memory():
         plan.forward(x, x, x, torch.empty_like(x), timesteps=[500.0])
     assert e.value.status == 4
     plan.destroy()
+
+
+EDGES = r"""
+import sys
+sys.path.insert(0, %r); sys.path.insert(0, %r)
+from paper_2604_22808_b200 import configs as C
+from test_parity_gpu import _run
+for n in (9944, 9946, 10000, 10072, 10080, 10082):
+    _run(C.TINY.scaled("edge", t_embed_dim=n))
+    print("ran", n)
+"""
+
+
+def test_around_the_default_shared_memory():
+    """8192 + 4 (3 x 32 + t_embed_dim + 64) bytes of dynamic shared memory, from 544 below the 48 KB that a launch has without asking
+    to just above them: what the kernel declares statically counts, too.  In a process of its own: a wider router asks for more
+    and leaves it to all that come later."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", EDGES % (root, os.path.join(root, "tests"))], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.split("\n")[-2] == "ran 10082", r.stdout[-500:] + r.stderr[-2000:]
