@@ -259,12 +259,13 @@ size_t router_bytes(const FFDims& dm) { return (size_t)(3 * dm.d + dm.dt + dm.hi
 }  // namespace
 
 // (routers up to what a block can have; a wider one fails where it is used, with the launch's error.  The 48 KB of a launch that asked
-// for nothing hold the kernel's static arrays, too: 544 bytes)
+// for nothing hold the kernel's static arrays, too: 544 bytes.  The most and not this plan's need: the attribute is the kernel's, and
+// a plan made later must not take it back from an earlier, wider one.)
 cudaError_t ffk_stats_init(const FFDims& dm) {
-  const size_t most = 226 * 1024, beside = 1024, need = sums_bytes(dm) + router_bytes(dm);     // (of 227 KB)
-  if (need + beside <= 48 * 1024) return cudaSuccess;
+  constexpr size_t most = 226 * 1024, beside = 1024;       // (of 227 KB)
+  if (sums_bytes(dm) + router_bytes(dm) + beside <= 48 * 1024) return cudaSuccess;
   return cudaFuncSetAttribute(dm.fp32 ? band_stats_kernel<float> : band_stats_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)(need < most ? need : most));
+                              (int)most);
 }
 
 cudaError_t ffk_set_timesteps(ff_plan* p, const float* host, cudaStream_t st) {
