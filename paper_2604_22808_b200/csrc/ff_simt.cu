@@ -289,8 +289,8 @@ bool vol_fits(const FFDims& dm) { return dm.N <= VOL_MAX; }
 // 128 FMA (4 x 4 scores per thread were bound by those reads: 233 us), then 8 rows x d / 16 output channels.  Rows lie
 // as they are in memory, padded by 16 bytes against bank conflicts, so copies are asynchronous: the next keys arrive
 // during the softmax and P V, the values during Q K.  P is only read by the half warp that wrote it.  64 keys a tile up
-// to head_dim 64, 32 above (three blocks, two blocks per SM; fewer by a rule of the launch).  Measured there: 196 us with three blocks,
-// 178 with two; packed pairs of FMA gained nothing (204 us).
+// to head_dim 64, 32 above (three blocks, two blocks per SM).  Measured there: 196 us, 70% of the issue slots; packed
+// pairs of FMA gained nothing (204 us).
 // ------------------------------------------------------------------------------------------------
 constexpr int AT = 64, AT_THREADS = 128, AT_PITCH = AT + 4;
 
@@ -751,38 +751,6 @@ cudaError_t ffk_forward_transform(ff_plan* p, const void* Q, const void* K, cons
                     : forward_transform_t<__nv_bfloat16>(p, Q, K, V, want_energy, st);
 }
 
-// Head_dim 64: two blocks per SM instead of three where the longest item, at a third of its SM's rate, would outlast the mean SM's
-// work (both in key tiles, as if every head ran every band): its blocks end the launch, alone on their SMs.  Layers, three / two
-// blocks, us (longest item, mean of an SM): 9 x 30 x 40 tokens, four heads, all bands 325.8 / 307.4 (15, 33); 5 x 33 x 32, six,
-// routed 190.9 / 175.2 (7, 19.3); 8 x 24 x 32, six 224.6 / 215.5 (10, 20.8).  With no more items than two an SM
-// there is no third block, and the shared memory only keeps the next launch out: 8 x 19 x 16, four 87.1 / 87.8.  On the other side
-// 10 x 30 x 40, six 465.0 / 527.9 (18, 62), 16 x 64 x 64, four 1968 / 2111 (31, 270), 9 x 40 x 60, four 854 / 839 (31, 121).
-// Head_dim 32 gains less and lost 1.7% at 12 x 10 x 33 tokens, four heads (6, 6): three blocks there.
-constexpr size_t AT_SMEM_TWO = 80 * 1024;              // two of them fit an SM, three do not
-
-static bool long_items(const FFDims& dm, int band_bits, int sm_count) {
-  constexpr int KT = AtShape<2>::KT;
-  auto tiles = [](long long n, int size) { return (n + size - 1) / size; };
-  long long longest = 0, total = 0, all = 0;
-  auto add = [&](long long items, long long steps) {
-    if (items > 0 && steps > longest) longest = steps;
-    total += items * steps * dm.BH;
-    all += items * dm.BH;
-  };
-  if (band_bits & FF_BAND_LOW) add(tiles(dm.Nbar, AT), tiles(dm.Nbar, KT));
-  if ((band_bits & FF_BAND_MID) && dm.Nmid > 0) {
-    const long long per = dm.nb / dm.s, rem = dm.nb % dm.s, b = dm.b < dm.Nmid ? dm.b : dm.Nmid;
-    if (dm.pattern == FF_MID_STRIDED) {
-      add(rem * tiles((per + 1) * b, AT), tiles((per + 1) * b, KT));
-      add((dm.s - rem) * tiles(per * b, AT), tiles(per * b, KT));
-    } else {
-      add(tiles(dm.Nmid, AT), tiles(dm.Nmid, KT));
-    }
-  }
-  if (band_bits & FF_BAND_HIGH) add(tiles(dm.Nhigh, AT), tiles(dm.Nhigh < 2LL * dm.R + AT ? dm.Nhigh : 2LL * dm.R + AT, KT));
-  return all > 2LL * sm_count && 3 * longest * sm_count > total;
-}
-
 template <typename ST>
 static cudaError_t attention_simt_t(ff_plan* p, int band_bits, cudaStream_t st) {
   const FFDims& dm = p->dm;
@@ -816,10 +784,9 @@ static cudaError_t attention_simt_t(ff_plan* p, int band_bits, cudaStream_t st) 
     }
   }
   const dim3 grid((unsigned)most, (unsigned)dm.BH, bands);
-  const size_t smem2 = AtShape<2>::smem < AT_SMEM_TWO && long_items(dm, band_bits, p->sm_count) ? AT_SMEM_TWO : AtShape<2>::smem;
   switch (dm.d / 32) {
     case 1: return ff_launch(attention_simt_kernel<ST, 1>, grid, dim3(AT_THREADS), AtShape<1>::smem, st, p->buf, dm, band_bits);
-    case 2: return ff_launch(attention_simt_kernel<ST, 2>, grid, dim3(AT_THREADS), smem2, st, p->buf, dm, band_bits);
+    case 2: return ff_launch(attention_simt_kernel<ST, 2>, grid, dim3(AT_THREADS), AtShape<2>::smem, st, p->buf, dm, band_bits);
     case 3: return ff_launch(attention_simt_kernel<ST, 3>, grid, dim3(AT_THREADS), AtShape<3>::smem, st, p->buf, dm, band_bits);
     default: return ff_launch(attention_simt_kernel<ST, 4>, grid, dim3(AT_THREADS), AtShape<4>::smem, st, p->buf, dm, band_bits);
   }

@@ -1,5 +1,5 @@
-"""The fp32 attention at head_dim 64 on both sides of the rule that puts two instead of three blocks on an SM: one long mid item
-among few, the anchor pattern, bf16 storage, and more work than the rule takes."""
+"""The fp32 attention at head_dim 64 with few items (less than one an SM) and with several an SM: strided and anchor pattern, fp32 and
+bf16 storage, mid items longer than the others."""
 import pytest
 
 from paper_2604_22808_b200 import configs as C
