@@ -215,7 +215,7 @@ extern "C" ff_status_t ff_plan_create(const ff_config_t* c, const ff_weights_t* 
   ce = ffk_simt_init();
   if (ce == cudaSuccess) ce = ffk_attention_tc_init();
   if (ce == cudaSuccess) ce = ffk_exchange_tc_init(p->dm);
-  if (ce == cudaSuccess) ce = ffk_dct_tc_init(p->dm);
+  if (ce == cudaSuccess) ce = ffk_dct_tc_init(p->dm, p->sm_count);
   if (ce == cudaSuccess) ce = ffk_dct2_init();
   if (ce == cudaSuccess) ce = ffk_dct_t16_init();
   if (ce == cudaSuccess) ce = ffk_proj_init();

@@ -44,7 +44,8 @@
 // its one staging area: it has two, and a stage less.  Six heads of that grid, the passes alone, us: w 176 -> 172 (6.1 TB/s),
 // h 296 -> 245 (5.7), t with the band split 271 -> 264 (4.0), inverse t 96 -> 94, h 107 -> 89, w 107 -> 96; layers (16 heads 3640 ->
 // 3474, eight of 7 x 90 x 127 tokens 1970 -> 1873).  With 64 channels none of it gained (20 x 30 x 52 tokens, eight heads, 484 -> 490):
-// they keep four stages of whole tiles.
+// they keep four stages of whole tiles.  With few tiles a launch whose code no SM has run yet costs more than eight warps gain: the
+// middle pass and the band split then share theirs, four warps in both (rule: FEW_TILES).
 //
 // Order of the tiles.  A pass that reads what the previous launch wrote walks its tiles from the last to the
 // first (P.reverse), the next one forward again: the end of the previous launch's output is still in L2.
@@ -96,13 +97,14 @@ enum {
   FORM_BYTES,     // a pair in the three-byte form
   FORM_EXACT1,    // any grid: the caller's bf16 tensor, handed on as fp32
   FORM_EXACT,     // any grid: an fp32 grid
-  FORM_EXACT_SPLIT   // ... and the band split follows (128 channels; with 64 it is a mode of FORM_EXACT)
+  FORM_EXACT_SPLIT,  // ... and the band split follows (128 channels; with 64 it is a mode of FORM_EXACT)
+  FORM_EXACT_FEW     // ... either of them (128 channels, few tiles)
 };
 template <int CH, int FORM> struct Shape {
   static constexpr bool any_grid = FORM >= FORM_EXACT1;
   static constexpr bool convert = FORM == FORM_BYTES || FORM >= FORM_EXACT;
-  // TMA warp, MMA warp, 8 epilogue warps; then those that make operands of the data: 128 threads, and of fp32 numbers as many
-  // for every 64 channels
+  // TMA warp, MMA warp, 8 epilogue warps; then those that make operands of the data: 128 threads, with FORM_EXACT as many for
+  // every 64 channels
   static constexpr int makers = !convert ? 0 : (FORM == FORM_EXACT ? 2 * CH : 128);
   static constexpr int threads = 320 + makers;
   static constexpr int parts = any_grid ? 3 : 2;           // of the matrix, 64 tensor-memory columns each
@@ -180,7 +182,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
   const bool seq = P.g.seq;                               // lines follow one another (w axis) or interleave
   const int rows = RAG ? P.g.rows : TILE_ROWS;
   const int NSTAGE = P.nstage;
-  const bool split = FORM == FORM_EXACT_SPLIT || ((FORM == FORM_PAIR || (FORM == FORM_EXACT && CH == 64)) && P.mode == MODE_SPLIT);     // (the band-split pass never reads the byte form)
+  const bool split = FORM == FORM_EXACT_SPLIT || ((FORM == FORM_PAIR || FORM == FORM_EXACT_FEW || (FORM == FORM_EXACT && CH == 64)) && P.mode == MODE_SPLIT);     // (the band-split pass never reads the byte form)
   const bool tma_out = !split;
   constexpr int TB = TILE_ROWS * CH * 2;                  // bytes of one data tile (16 KB for 64 channels)
   constexpr int LO8_OFF = CH == 128 ? TB : 2 * TB;         // where a stage takes the lo bytes
@@ -558,7 +560,7 @@ dct_tc_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant__ 
       const int out_slice = P.mode == MODE_LAST ? th : gi;
       const unsigned nonlow_rows = __ballot_sync(0xffffffffu, band > 0), mid_rows = __ballot_sync(0xffffffffu, band == 1);
       // both 32-channel chunks of the row at once; the accumulator buffer is free as soon as they are read
-      constexpr bool EACH = FORM == FORM_EXACT_SPLIT;      // (for want of registers one after the other)
+      constexpr bool EACH = FORM >= FORM_EXACT_SPLIT;      // (for want of registers one after the other)
       uint32_t rr2[EACH ? 1 : NQ][32];
       if (!EACH) {
         FF_CLOCK(pl);
@@ -818,7 +820,8 @@ cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1
     case FORM_BYTES: FF_DCT_D(FORM_BYTES); break;
     case FORM_EXACT1: FF_DCT_D(FORM_EXACT1); break;
     case FORM_EXACT: FF_DCT_D(FORM_EXACT); break;
-    default: FF_DCT(128, FORM_EXACT_SPLIT);
+    case FORM_EXACT_SPLIT: FF_DCT(128, FORM_EXACT_SPLIT); break;
+    default: FF_DCT(128, FORM_EXACT_FEW);
   }
 #undef FF_DCT_D
 #undef FF_DCT
@@ -829,14 +832,24 @@ cudaError_t launch_pass(ff_plan* p, const CUtensorMap& m0, const CUtensorMap& m1
 
 }  // namespace
 
-cudaError_t ffk_dct_tc_init(const FFDims& dm) {
+// Any grid, 128 channels: tiles an SM of the middle pass, all tensor-heads together, up to which it and the band split run the
+// same code.  Layers, us, each its own / the same (tiles): 5 x 33 x 20 tokens, eight heads, all bands 159.5 / 154.0 (6); 12 x 40 x 100,
+// one 231.7 / 222.9 (8), two 354.4 / 350.1 (16); 21 x 45 x 80, one 297.2 / 285.9 (17).  10 x 50 x 110, two 403.6 / 399.2 (22),
+// 48 x 24 x 60, two 490.1 / 494.0 (23), 21 x 45 x 80, two, routed 471.2 / 476.7 (34), four 994.5 / 1004.7 (68).
+constexpr int FEW_TILES = 20;
+static bool few_tiles(const FFDims& dm, int sm_count) {
+  return dm.d == 128 && 3LL * dm.BH * ff_pass_shape(dm, 1).tiles <= (long long)FEW_TILES * sm_count;
+}
+
+cudaError_t ffk_dct_tc_init(const FFDims& dm, int sm_count) {
   cudaError_t e = cudaSuccess;
 #define FF_DCT(D, F) \
   if (e == cudaSuccess && dm.d == D) e = cudaFuncSetAttribute(dct_tc_kernel<D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 256)
   if (!ffk_dct_tc_supported(dm)) return e;
-  if (ff_fp32_grid(dm)) { FF_DCT(128, FORM_EXACT1); FF_DCT(128, FORM_EXACT); FF_DCT(64, FORM_EXACT1); FF_DCT(64, FORM_EXACT);
-                           FF_DCT(128, FORM_EXACT_SPLIT); }
-  else { FF_DCT(128, FORM_PAIR); FF_DCT(128, FORM_BYTES); FF_DCT(64, FORM_PAIR); FF_DCT(64, FORM_BYTES); }
+  if (ff_fp32_grid(dm)) {
+    FF_DCT(128, FORM_EXACT1); FF_DCT(128, FORM_EXACT); FF_DCT(64, FORM_EXACT1); FF_DCT(64, FORM_EXACT);
+    if (few_tiles(dm, sm_count)) { FF_DCT(128, FORM_EXACT_FEW); } else { FF_DCT(128, FORM_EXACT_SPLIT); }
+  } else { FF_DCT(128, FORM_PAIR); FF_DCT(128, FORM_BYTES); FF_DCT(64, FORM_PAIR); FF_DCT(64, FORM_BYTES); }
 #undef FF_DCT
   return e;
 }
@@ -900,6 +913,7 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
     return cudaErrorInvalidValue;
   if (exact) { o0l = o0h; m1l = m1h; o1l = o1h; m2l = m2h; }     // (not used)
   const int total = 3 * dm.BH;
+  const bool few = few_tiles(dm, p->sm_count);
   DctTcParams P{};
   P.dm = dm; P.status = p->buf.status;
   P.spec_mid = (__nv_bfloat16*)p->buf.spec_mid; P.spec_high = (__nv_bfloat16*)p->buf.spec_high;
@@ -928,11 +942,11 @@ cudaError_t ffk_forward_transform_tc(ff_plan* p, const void* Q, const void* K, c
     if (e != cudaSuccess) return e;
     P.clear = nullptr;
     P.mode = MODE_MIDDLE; P.in_split = 1; P.out_lo8 = 0; P.reverse = 1; P.axis = 1; P.image = matrix_image(p, 1, 0);
-    e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, exact ? FORM_EXACT : FORM_BYTES, st);
+    e = launch_pass(p, m1h, m1l, m1l, o1h, o1l, P, exact ? (few ? FORM_EXACT_FEW : FORM_EXACT) : FORM_BYTES, st);
     if (e != cudaSuccess) return e;
     P.in_split = 1; P.out_lo8 = 0; P.reverse = 0;
     P.mode = MODE_SPLIT; P.axis = 0; P.image = matrix_image(p, 0, 0);
-    e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, exact ? (dm.d == 128 ? FORM_EXACT_SPLIT : FORM_EXACT) : FORM_PAIR, st);    // (no tensor stores in this mode)
+    e = launch_pass(p, m2h, m2l, m2l, m2h, m2l, P, exact ? (few ? FORM_EXACT_FEW : dm.d == 128 ? FORM_EXACT_SPLIT : FORM_EXACT) : FORM_PAIR, st);    // (no tensor stores in this mode)
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -251,7 +251,7 @@ void ff_compute_layout(const FFDims& dm, bool with_staging, FFLayout* lay);
 cudaError_t ffk_simt_init();
 cudaError_t ffk_attention_tc_init();
 cudaError_t ffk_exchange_tc_init(const FFDims& dm);
-cudaError_t ffk_dct_tc_init(const FFDims& dm);
+cudaError_t ffk_dct_tc_init(const FFDims& dm, int sm_count);
 cudaError_t ffk_dct2_init();
 cudaError_t ffk_proj_init();
 cudaError_t ffk_stats_init(const FFDims& dm);

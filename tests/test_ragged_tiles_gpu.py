@@ -11,16 +11,26 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("grid,d", [((21, 45, 80), 128), ((9, 100, 66), 128), ((40, 33, 50), 64), ((48, 24, 60), 128)], ids=str)
 def test_many_tiles(grid, d):
+    _both(grid, d, 4)
+
+
+# (the middle pass and the band split share their code up to 20 tiles an SM: 6 and 16 of them here, and 25)
+@pytest.mark.parametrize("grid,heads", [((5, 33, 20), 8), ((12, 40, 100), 2), ((12, 40, 100), 3)], ids=str)
+def test_few_tiles(grid, heads):
+    _both(grid, 128, heads)
+
+
+def _both(grid, d, heads):
     import torch
     from paper_2604_22808_b200 import binding as B
     low, mid = tuple(max(1, n // 8) for n in grid), tuple(n // 8 + n // 2 for n in grid)
-    cfg = C.FFConfig(name="tiles", batch=1, T=grid[0], H=grid[1], W=grid[2], heads=4, head_dim=d, dtype="bf16", low_cut=low, mid_cut=mid,
+    cfg = C.FFConfig(name="tiles", batch=1, T=grid[0], H=grid[1], W=grid[2], heads=heads, head_dim=d, dtype="bf16", low_cut=low, mid_cut=mid,
                      r=8, b=64, s=8, R=64, m=0, seed=93, timesteps=(500.0,))
     plan = B.Plan(cfg)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(7)
-    q, k, v, other = (torch.randn((1, 4) + grid + (d,), generator=gen, device="cuda").to(torch.bfloat16) for _ in range(4))
-    alloc, out = torch.zeros(4, dtype=torch.uint8, device="cuda"), torch.empty_like(q)
+    q, k, v, other = (torch.randn((1, heads) + grid + (d,), generator=gen, device="cuda").to(torch.bfloat16) for _ in range(4))
+    alloc, out = torch.zeros(heads, dtype=torch.uint8, device="cuda"), torch.empty_like(q)
     taps, got = (B.TAP_SPEC_LOW, B.TAP_SPEC_MID, B.TAP_SPEC_HIGH), {}
     for impl in (2, 0, 0, 0):
         plan.set_attention_impl(impl)
