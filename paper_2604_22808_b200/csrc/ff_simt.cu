@@ -184,12 +184,10 @@ cudaError_t launch_dct_pass(ff_plan* p, DctPassParams& P, int group, cudaStream_
 // All three axes of a small grid in one launch: a block holds eight channels of a tensor-head's whole grid in shared
 // memory and transforms it in place, axis by axis (lines are handled in rounds: everything a round reads is in
 // registers before any of it is overwritten).  Small grids are bound by launches and latency: 4 x 8 x 8 tokens take
-// one launch of 6 us instead of three of 5.  Up to 256 positions a thread computes two outputs instead of eight: eight keep a quarter
-// of the threads or fewer busy (layers, us, eight / two: 4 x 8 x 8 routed 28.7 / 27.55, 2 x 10 x 12 33.6 / 32.25, 2 x 2 x 64 33.9 / 32.0,
-// 2 x 6 x 8 30.3 / 28.9; 5 x 9 x 10, 450 positions, 40.7 / 41.2, 4 x 16 x 8 42.3 / 42.8).
+// one launch of 6 us instead of three of 5.  On the smallest grids a thread computes two outputs instead of eight, which keep a
+// quarter of the threads or fewer busy (rule: vol_fine).
 // ------------------------------------------------------------------------------------------------
 constexpr int VOL_CH = 8, VOL_THREADS = 256;
-constexpr int VOL_FINE = 256;            // positions, up to which a thread computes two outputs of a line instead of eight
 constexpr int VOL_MAX = 2304;            // positions: 72 KB, so that three blocks share an SM
 
 struct VolParams {
@@ -277,6 +275,25 @@ size_t vol_smem(const FFDims& dm) {
   return (size_t)dm.N * VOL_CH * sizeof(float) + m * sizeof(float);
 }
 bool vol_fits(const FFDims& dm) { return dm.N <= VOL_MAX; }
+
+// Two outputs a thread, both ways (a layer of this size is bound by fetching code, too), where they cover the axes in one round, up
+// to an eighth of the steps.  Layers, fp32, all bands, us, eight / two: 4 x 8 x 8 tokens, two heads of 32 channels 27.3 / 26.2, 24 of
+// 64 59.4 / 58.2, 96 of 64 125.3 / 112.2; 3 x 5 x 7, twelve of 64 29.3 / 27.2; 2 x 3 x 40 (two rounds of h), 24 of 64 65.5 / 62.2.  In more
+// rounds they gain once there are blocks enough to fill the SMs: 3 x 9 x 9, four heads of 64, routed 32.6 / 33.8, 24 of 128 (2.6 blocks
+// an SM, inverse) 74.7 / 76.8, 48 of 128 122.5 / 113.9; 5 x 9 x 10, 450 positions, 40.7 / 41.2.  And not where every SM has one block or
+// two of the inverse launch, of more than half of 256 positions: 4 x 8 x 8, nine heads of 128 (0.97 an SM) 36.6 / 38.5, 36 of 32
+// 48.3 / 52.4, 24 of 96 (1.95) 59.8 / 62.5, 30 of 64 (1.6) 61.5 / 63.4; 42 of 64 (2.3) 71.9 / 69.2.
+bool vol_fine(const FFDims& dm, int sm_count) {
+  if (dm.N > VOL_THREADS) return false;
+  const double blocks = (double)dm.BH * (dm.d / VOL_CH) / sm_count;
+  int steps = 0, more = 0;
+  for (const int n : {dm.T, dm.H, dm.W}) {
+    const int per_round = VOL_THREADS / ((n + 1) / 2 * 2), rounds = ((int)(dm.N / n) + per_round - 1) / per_round;
+    steps += n; more += (rounds - 1) * n;
+  }
+  if (8 * more > steps) return blocks > 4;
+  return dm.N <= VOL_THREADS / 2 || !((blocks > 0.875 && blocks < 1.2) || (blocks > 1.5 && blocks < 2.2));
+}
 
 // ------------------------------------------------------------------------------------------------
 // Band operators ("Hierarchical frequency-domain attention") in fp32: a block takes 64 query rows of one (head, band)
@@ -716,7 +733,7 @@ static cudaError_t forward_transform_t(ff_plan* p, const void* Q, const void* K,
     P.spec_low = p->buf.spec_low; P.spec_mid = p->buf.spec_mid; P.spec_high = p->buf.spec_high;
     P.clear = want_energy ? p->buf.energy : nullptr;
     p->launches += 1;
-    return ff_launch(dm.N <= VOL_FINE ? dct_volume_kernel<ST, false, 2> : dct_volume_kernel<ST, false, 8>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)(3 * dm.BH)), dim3(VOL_THREADS),
+    return ff_launch(vol_fine(dm, p->sm_count) ? dct_volume_kernel<ST, false, 2> : dct_volume_kernel<ST, false, 8>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)(3 * dm.BH)), dim3(VOL_THREADS),
                      vol_smem(dm), st, P);
   }
   const int total = 3 * dm.BH, G = p->lay.group;
@@ -854,7 +871,7 @@ static cudaError_t exchange_inverse_t(ff_plan* p, void* out, cudaStream_t st) {
       P.src[0] = p->buf.scratchA; P.out = out; P.dm = dm; P.group_start = h0;
       for (int a = 0; a < 3; ++a) P.mat_t[a] = p->basis[a];
       p->launches += 1;
-      e = ff_launch(dm.N <= VOL_FINE ? dct_volume_kernel<ST, true, 2> : dct_volume_kernel<ST, true, 8>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)g), dim3(VOL_THREADS), vol_smem(dm), st, P);
+      e = ff_launch(vol_fine(dm, p->sm_count) ? dct_volume_kernel<ST, true, 2> : dct_volume_kernel<ST, true, 8>, dim3((unsigned)(dm.d / VOL_CH), (unsigned)g), dim3(VOL_THREADS), vol_smem(dm), st, P);
       if (e != cudaSuccess) return e;
       continue;
     }
