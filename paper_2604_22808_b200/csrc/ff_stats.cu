@@ -46,9 +46,9 @@ __device__ __forceinline__ void prefetch_line(const float* p, int line, int n) {
   if (line < (n + 31) / 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + line * 32));
 }
 
-// Sinusoidal embedding of the sample's timestep into et[dt], in double precision; by the block's last warp if it is that short.
+// Sinusoidal embedding of the sample's timestep into et[dt], in double precision; by as many of the block's last warps as it takes.
 __device__ void embed_timestep(const StatsParams& P, int sample, float* et) {
-  const int half = P.dm.dt / 2, threads = half <= 32 ? 32 : ST_THREADS;
+  const int half = P.dm.dt / 2, threads = half < ST_THREADS ? (half + 31) / 32 * 32 : ST_THREADS;
   for (int k = (int)threadIdx.x - (ST_THREADS - threads); k >= 0 && k < half; k += threads) {
     const double t = (double)(P.timestep ? P.timestep[sample] : P.ts[sample]);
     const double om = exp2(-(double)k / (double)half * 13.287712379549449);     // 10000^(-k/half); log2(10000)
@@ -60,10 +60,12 @@ __device__ void embed_timestep(const StatsParams& P, int sample, float* et) {
 }
 
 // z = W2 relu(W1 [g; e(t)] + b1) + b2, pi = softmax(z), largest-remainder quota, one-hot masks; a whole block.  A chain of
-// latencies: everything that does not depend on the step before is under way by then (the weights of a layer, e(t) on a warp of
-// its own).
-constexpr int ST_AHEAD = 7;              // inputs of a hidden unit that a lane holds weights of at a time
-__device__ void route_sample(const StatsParams& P, int sample, float* sm, uint8_t* masks) {
+// latencies: under way before the step that needs them are the weights of the first 224 inputs of the first 64 hidden units (all of
+// them with head_dim 32 and an embedding of up to 128), those of the second layer's first 64, and e(t) on warps of its own.  The other
+// weights are loaded eight inputs at a time, without a test where eight are left: in chunks of seven tested ones layers took, us,
+// 256 fp32 tokens, 1024 hidden units 52.4 for 44.2, 512 with t_embed_dim 512 45.7 for 39.7, head_dim 128 with 256 38.8 for 38.4.
+constexpr int ST_AHEAD = 7;              // inputs of a hidden unit that a lane holds weights of (28 registers of 64)
+__device__ void route_sample(const StatsParams& P, int sample, bool embedded, float* sm, uint8_t* masks) {
   const FFDims& dm = P.dm;
   const int d = dm.d, nin = 3 * d + dm.dt, hid = dm.hid;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -73,19 +75,14 @@ __device__ void route_sample(const StatsParams& P, int sample, float* sm, uint8_
   __shared__ int first[4];  // first head of each band
   // hidden layer: four units per warp at a time, lanes stride over the inputs (coalesced rows of W1)
   float w[4][ST_AHEAD];
-  auto weights = [&](int j0, int i0) {
 #pragma unroll
-    for (int t = 0; t < ST_AHEAD; ++t) {
-      const int i = i0 + 32 * t + lane;
+  for (int t = 0; t < ST_AHEAD; ++t)
 #pragma unroll
-      for (int k = 0; k < 4; ++k) w[k][t] = i < nin && j0 + k < hid ? P.W1[(size_t)(j0 + k) * nin + i] : 0.f;
-    }
-  };
-  weights(warp * 4, 0);
+    for (int k = 0; k < 4; ++k) w[k][t] = 32 * t + lane < nin && warp * 4 + k < hid ? P.W1[(size_t)(warp * 4 + k) * nin + 32 * t + lane] : 0.f;
   const float w2 = warp < 3 && lane < hid ? P.W2[warp * hid + lane] : 0.f, w2b = warp < 3 && lane + 32 < hid ? P.W2[warp * hid + lane + 32] : 0.f;
   const float bias2 = warp < 3 ? P.b2[warp] : 0.f;
   float bias1 = lane < 4 && warp * 4 + lane < hid ? P.b1[warp * 4 + lane] : 0.f;
-  embed_timestep(P, sample, x + 3 * d);
+  if (!embedded) embed_timestep(P, sample, x + 3 * d);
   for (int i = tid; i < 3 * d; i += ST_THREADS) {
     const int band = i / d;
     const long long cnt = band == 0 ? dm.Nlow : (band == 1 ? dm.Nmid : dm.Nhigh);
@@ -93,17 +90,29 @@ __device__ void route_sample(const StatsParams& P, int sample, float* sm, uint8_
     x[i] = (float)log1p(__ldcg(P.energy + (size_t)sample * 3 * d + i) / terms);
   }
   __syncthreads();
+  // (the first units' inputs so far; from there on as many loads at a time as fit)
+  float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int t = 0; t < ST_AHEAD; ++t) {
+    const float v = 32 * t + lane < nin ? x[32 * t + lane] : 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = fmaf(w[k][t], v, acc[k]);
+  }
+  int i0 = 32 * ST_AHEAD;
   for (int j0 = warp * 4; j0 < hid; j0 += (ST_THREADS / 32) * 4) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int i0 = 0; i0 < nin; i0 += 32 * ST_AHEAD) {
-      if (i0 > 0 || j0 != warp * 4) weights(j0, i0);
+    const float* row = P.W1 + (size_t)j0 * nin + lane;
+    const int o1 = j0 + 1 < hid ? nin : 0, o2 = j0 + 2 < hid ? 2 * nin : 0, o3 = j0 + 3 < hid ? 3 * nin : 0;
+    auto add = [&](int i, bool on) {
+      const float v = on ? x[i + lane] : 0.f;
+      acc[0] = fmaf(on ? row[i] : 0.f, v, acc[0]); acc[1] = fmaf(on ? row[i + o1] : 0.f, v, acc[1]);
+      acc[2] = fmaf(on ? row[i + o2] : 0.f, v, acc[2]); acc[3] = fmaf(on ? row[i + o3] : 0.f, v, acc[3]);
+    };
+    for (; i0 + 32 * 8 <= nin; i0 += 32 * 8)
 #pragma unroll
-      for (int t = 0; t < ST_AHEAD; ++t) {
-        const float v = i0 + 32 * t + lane < nin ? x[i0 + 32 * t + lane] : 0.f;
+      for (int t = 0; t < 8; ++t) add(i0 + 32 * t, true);
+    if (i0 < nin)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] = fmaf(w[k][t], v, acc[k]);
-      }
-    }
+      for (int t = 0; t < 8; ++t) add(i0 + 32 * t, i0 + 32 * t + lane < nin);
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[k] = warp_sum(acc[k]);
     if (lane < 4 && j0 + lane < hid) {
@@ -111,6 +120,9 @@ __device__ void route_sample(const StatsParams& P, int sample, float* sm, uint8_
       if (j0 != warp * 4) bias1 = P.b1[j0 + lane];
       h[j0 + lane] = fmaxf(v + bias1, 0.f);
     }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc[k] = 0.f;
+    i0 = 0;
   }
   __syncthreads();
   if (warp < 3) {
@@ -158,6 +170,8 @@ __global__ void __launch_bounds__(ST_THREADS, 2) band_stats_kernel(const __grid_
   const FFDims& dm = P.dm;
   // (any block may turn out to be the one that routes; the sums below use other shared memory)
   float* mlp = sm + (ST_THREADS / (dm.d / 4)) * dm.d;
+  // (an embedding that takes more than half of the threads is not overlapped with the energies: 1024, 33.1 us a layer, here 32.3)
+  const bool early = !P.timestep && dm.dt > ST_THREADS;
   if (!P.alloc_in) {
     // A transform that has gone through L2 leaves none of the router's weights there: the first blocks ask for them while
     // the sums are made.
@@ -166,6 +180,7 @@ __global__ void __launch_bounds__(ST_THREADS, 2) band_stats_kernel(const __grid_
     prefetch_line(P.W2, line, 3 * dm.hid);
     prefetch_line(P.b1, line, dm.hid);
     prefetch_line(P.b2, line, 3);
+    if (early) embed_timestep(P, 0, mlp + 3 * dm.d);
   }
   // (a router keeps one block busy long after the others: let in early, the next launch's blocks settle unevenly meanwhile.
   // With masks given there is little to wait for: 4 x 19 x 16 fp32 tokens, six heads, all bands, 55.6 us, let in late 61.1)
@@ -239,7 +254,7 @@ __global__ void __launch_bounds__(ST_THREADS, 2) band_stats_kernel(const __grid_
   __threadfence();
   if (threadIdx.x == 0) *P.ticket = 0;
   for (int sample = 0; sample < dm.B; ++sample) {
-    route_sample(P, sample, mlp, masks);
+    route_sample(P, sample, early && sample == 0, mlp, masks);
   }
   if (P.work && threadIdx.x < 32) build_worklist(dm, dm.BH <= ST_MASKS ? masks : P.alloc, P.low_on, P.mid_items, P.work);
 }

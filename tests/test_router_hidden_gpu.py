@@ -12,3 +12,10 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("hidden,head_dim,t_embed_dim", [(1, 32, 2), (37, 32, 64), (64, 32, 128), (65, 64, 34), (130, 128, 70)])
 def test_hidden_layer(hidden, head_dim, t_embed_dim):
     _run(C.TINY.scaled("hidden", router_hidden=hidden, head_dim=head_dim, t_embed_dim=t_embed_dim, heads=3))
+
+
+# (units beyond the first 64 with just one load of eight inputs a lane, one input less, and with one behind what is held; an
+# embedding as wide as the block and wider)
+@pytest.mark.parametrize("hidden,head_dim,t_embed_dim", [(70, 64, 64), (70, 64, 62), (66, 32, 384), (66, 32, 386), (96, 32, 1024), (33, 32, 1040)])
+def test_inputs_behind_those_held(hidden, head_dim, t_embed_dim):
+    _run(C.TINY.scaled("inputs", router_hidden=hidden, head_dim=head_dim, t_embed_dim=t_embed_dim, heads=3))
