@@ -31,9 +31,10 @@ METRIC = "freqformer_attn_layer_tokens_per_s"
 # dram__bytes_read.sum + dram__bytes_write.sum of the transform kernels per token and head, from the ncu
 # capture of the 6-head 64K case (forward: the passes over Q, K and V; inverse: the passes over one tensor).
 FP32_FMA_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12      # 74.5: plain fp32 FMA rate of the GPU (unit counts x max clock)
-# [0]: three separate axis passes; [1]: two axes in one launch (64K-class grids); [2]: the same, inverse with t = 16 in registers
-NCU_DRAM_BYTES_PER_TOKEN_HEAD = {"transform": (6554.0, 4388.0), "inverse": (2345.0, 1985.0, 1938.0)}
-TRANSFORM_KERNELS = {"transform": ("dct_tc_kernel x3 (transform stage)", "dct_fold_kernel (second axis of 16 or 32) or dct2_tc_kernel + dct_tc_kernel (transform stage)"),
+# [0]: three separate axis passes; [1]: two axes in one launch (64K-class grids); [2]: the same with the second axis in registers
+NCU_DRAM_BYTES_PER_TOKEN_HEAD = {"transform": (6554.0, 4380.0, 4388.0), "inverse": (2345.0, 1985.0, 1938.0)}
+TRANSFORM_KERNELS = {"transform": ("dct_tc_kernel x3 (transform stage)", "dct2_tc_kernel + dct_tc_kernel (transform stage)",
+                                   "dct_fold_kernel + dct_tc_kernel (transform stage)"),
                      "inverse": ("exchange_tc_kernel + dct_tc_kernel x3 (inverse stage)",
                                  "exchange_tc_kernel + dct_tc_kernel + dct2_tc_kernel (inverse stage)",
                                  "exchange_tc_kernel + dct_tc_kernel + dct_t16_kernel (inverse stage)")}
@@ -527,7 +528,7 @@ def run_cuda(args, cfg):
             # DRAM bytes per token-head and stage from the ncu capture of the 6-head 64K case; the traffic is
             # proportional to tokens x heads
             fused = int(kinfo["transform_fused"])
-            label = fused + int(top == "inverse" and kinfo["inverse_t_in_registers"])
+            label = fused + int(kinfo["inverse_t_in_registers" if top == "inverse" else "forward_axis_in_registers"])
             per_token_head = NCU_DRAM_BYTES_PER_TOKEN_HEAD[top][label] * cfg.head_dim / 128.0
             roof = {"bound": "hbm", "achieved": st["gbs"], "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": st["frac"],
                     "traffic": per_token_head * cfg.N * heads_total / n_launch if tensor_core_path else None,

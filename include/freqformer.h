@@ -210,9 +210,9 @@ ff_status_t ff_plan_selftest_bounded_wait(ff_plan_t *plan, int64_t limit_cycles,
                                           int32_t *waiters_released, void *cuda_stream);
 
 /* Which kernels the plan's forward runs with the workspace it has (benchmarks label their numbers with it):
- *   info[0]  1: the transform runs two axes in one launch (intermediate in shared memory), 0: three passes
- *   info[1]  1: that launch runs forward only, the last inverse launch keeps a t axis of 16 positions in registers
- *            (0: it runs both ways, or is unused)
+ *   info[0]  bit 0: the transform runs two axes in one launch (0: three passes); bit 1: the forward one keeps the second
+ *            axis, of 16 or 32 positions, in registers (0: its intermediate goes through shared memory)
+ *   info[1]  1: the last inverse launch keeps a t axis of 16 positions in registers (0: through shared memory, or three passes)
  *   info[2]  1: the band operators run on the tensor-core kernel, 0: generic kernels
  *   info[3]  1: the pooled low band is part of the tensor-core attention launch */
 ff_status_t ff_plan_kernel_info(const ff_plan_t *plan, int32_t info[4]);

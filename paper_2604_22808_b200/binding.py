@@ -308,8 +308,8 @@ class Plan:
     def kernel_info(self) -> dict:
         info = (C.c_int32 * 4)()
         _check(library().ff_plan_kernel_info(self.handle, info), self.handle)
-        return {"transform_fused": bool(info[0]), "inverse_t_in_registers": bool(info[1]), "attention_tensor_core": bool(info[2]),
-                "low_band_tensor_core": bool(info[3])}
+        return {"transform_fused": bool(info[0] & 1), "forward_axis_in_registers": bool(info[0] & 2),
+                "inverse_t_in_registers": bool(info[1]), "attention_tensor_core": bool(info[2]), "low_band_tensor_core": bool(info[3])}
 
     def last_launches(self) -> int:
         n = C.c_int64()

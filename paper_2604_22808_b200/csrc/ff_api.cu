@@ -360,7 +360,7 @@ extern "C" ff_status_t ff_plan_set_attention_impl(ff_plan_t* p, int32_t impl) {
 extern "C" ff_status_t ff_plan_kernel_info(const ff_plan_t* p, int32_t info[4]) {
   if (!p || !info) return fail(nullptr, FF_ERR_INVALID_ARG, "plan or info is NULL%s");
   const bool fused = p->dct_tc_ok && p->dct2_ok && !(p->attn_impl & 6);
-  info[0] = fused ? 1 : 0; info[1] = fused && p->t16 ? 1 : 0;
+  info[0] = fused ? (p->fold ? 3 : 1) : 0; info[1] = fused && p->t16 ? 1 : 0;
   info[2] = (p->tc_ok && !(p->attn_impl & 1)) ? 1 : 0; info[3] = (info[2] && p->low_tc_ok) ? 1 : 0;
   return FF_OK;
 }

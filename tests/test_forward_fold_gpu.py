@@ -22,6 +22,7 @@ def test_forward_fold(grid, heads, d):
     cfg = C.FFConfig(name="fold", batch=1, T=grid[0], H=grid[1], W=grid[2], heads=heads, head_dim=d, dtype="bf16", low_cut=low, mid_cut=mid,
                      r=8, b=64, s=8, R=64, m=0, seed=92, timesteps=(500.0,))
     plan = B.Plan(cfg)
+    assert plan.kernel_info()["forward_axis_in_registers"]
     gen = torch.Generator(device="cuda")
     gen.manual_seed(6)
     q, k, v, other = (torch.randn((1, heads) + grid + (d,), generator=gen, device="cuda").to(torch.bfloat16) for _ in range(4))
@@ -43,4 +44,19 @@ def test_forward_fold(grid, heads, d):
             assert np.linalg.norm(low_got - bands[0]) < 2.0 ** -17 * np.linalg.norm(bands[0])
             for got, ref in zip(want[1:], bands[1:]):
                 Hn.assert_close(got[t, h].float().cpu().numpy(), ref, "bf16", f"tensor {t} head {h}")
+    plan.destroy()
+
+
+@pytest.mark.parametrize("grid,heads,more,folds", [((16, 32, 16), 1, {}, True), ((32, 64, 32), 3, {}, False), ((32, 64, 32), 4, {}, True),
+                                                   ((16, 32, 128), 4, {}, False), ((64, 64, 16), 4, {}, False),
+                                                   ((16, 32, 32), 4, {"transform": "haar"}, False), ((16, 32, 48), 4, {}, False)], ids=str)
+def test_which_plans_take_it(grid, heads, more, folds):
+    from paper_2604_22808_b200 import binding as B
+    low, mid = tuple(n // 8 for n in grid), tuple(n // 8 + n // 2 for n in grid)
+    plan = B.Plan(C.FFConfig(name="fold", batch=1, T=grid[0], H=grid[1], W=grid[2], heads=heads, head_dim=128, dtype="bf16", low_cut=low,
+                             mid_cut=mid, r=8, b=64, s=8, R=64, m=0, seed=92, timesteps=(500.0,), **more))
+    assert plan.kernel_info()["forward_axis_in_registers"] == folds
+    for impl in (2, 4):                                        # generic transform; three passes
+        plan.set_attention_impl(impl)
+        assert not plan.kernel_info()["forward_axis_in_registers"]
     plan.destroy()
