@@ -389,6 +389,9 @@ dct_fold_kernel(const __grid_constant__ CUtensorMap map0, const __grid_constant_
           if (n >= (unsigned)F_NSLOT) ok = mbar_wait(&sh.empty[slot], ((n / F_NSLOT) - 1) & 1, abort_flag);
           FF_CLOCK_ADD(true, 16, tp);
           if (!ok) break;
+          // (debug build) the boxes lie inside the grid; a refused batch ends in the bounded wait of its consumer
+          if (!FF_DBG_OK((chunk + 1) * FC <= dm.d && o0 + P.lines <= (P.axis2 ? dm.T : dm.H) && N2 <= (P.axis2 ? dm.H : dm.T) && th < 3 * dm.BH,
+                         P.status, 7)) continue;
           uint8_t* dst = sIn + slot * F_SLOT_B;
           mbar_arrive_expect_tx(&sh.full[slot], F_SLOT_B);
 #pragma unroll
