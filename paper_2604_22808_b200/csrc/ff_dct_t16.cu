@@ -20,7 +20,7 @@
 // Every wait is bounded.
 //
 // Bound by its epilogue and the loads: six heads of 64K tokens alone 62 us, 0.3 GB at 4.9 TB/s, issue slots 50%.  The four
-// warps of 32 lanes share a scheduler; when each made all t positions of four channels and they staged whole rows together, the
+// warps of 32 lanes share a scheduler; when each made all t positions of four channels and they staged whole rows together in two areas, the
 // scheduler stood still at every hand-over: 69 us, six heads of 16K tokens 193 -> 190 for the whole layer.  With ff_dct2_tc.cu in
 // this launch's place it took 334 us for 24 heads of 64K tokens at 1.6 GHz, with the shared staging 254.  The forward launch has a kernel of its own, below.
 #include <cuda.h>
@@ -284,11 +284,11 @@ dct_t16_kernel(const __grid_constant__ CUtensorMap map_hi, const __grid_constant
 // 57% (75% and 384 us without packed FMA, which with n2 = 16 gain nothing: 724 -> 732 us for six heads of 64 x 16 x 64); stores of 32
 // bytes from the registers 494.
 // ff_dct2_tc.cu sends the intermediate through shared memory as a bf16 pair and multiplies the second axis with a 128 x 128
-// operand of which 128 / n2 - 1 parts are zeros.  Layers before and after (us, at 1.6 GHz): 24 heads of 64K tokens 2850 / 2562; all
-// bands 3575 / 3417; 16 heads with head_dim 64 1025 / 935; six heads of 16K 206 / 193 (190 / 189 with the inverse below), four of 8K
-// 126 / 118, six of 64 x 16 x 64 784 / 724; n2 = 32: two samples of 24 heads of 32 x 64 x 64 10570 / 10300, 12 heads 3115 / 3040, eight
-// with head_dim 64 1205 / 1185, eight of 32 x 64 x 32 998 / 986.  A line of 128 positions does not fit twice into the operand: those
-// grids keep the two-axis launch.  Variants (n2 = 16, six heads of 64K): a quarter of the channels a thread, staged by four warps together,
+// operand of which 128 / n2 - 1 parts are zeros.  Layers with that launch / with this one, all else equal, in turn on one box (us,
+// under the power limit): 24 heads of 64K tokens 2745 / 2528; all bands 3427 / 3309; 16 heads with head_dim 64 993 / 937; six heads of
+// 16K 197 / 185, four of 8K 120 / 116, six of 64 x 16 x 64 765 / 730; n2 = 32: two samples of 24 heads of 32 x 64 x 64 10375 / 9998,
+// 12 heads 3059 / 2984, eight with head_dim 64 1197 / 1171, eight of 32 x 64 x 32 979 / 970.  A line of 128 positions does not fit twice
+// into the operand: those grids keep the two-axis launch.  Variants (n2 = 16, six heads of 64K): a quarter of the channels a thread, staged by four warps together,
 // coefficients as constants of unrolled code 201 us (instruction cache), in a loop 177; packed FMA 181; without its stores that form
 // took 155, without its FMA 163.
 constexpr int FPOS = 64;                                   // positions of an item
@@ -606,8 +606,10 @@ cudaError_t ffk_dct_t16_inverse(ff_plan* p, const void* in_hi, const void* in_lo
   return e;
 }
 
-// Where it takes the place of the two-axis launch.  With 32 positions from 20 items an SM on, all tensor-heads together: four
-// heads of 32 x 64 x 32 tokens (20) take the same time, of 32 x 64 x 64 (41) 1347 -> 1330 us, of 32 x 32 x 16 (5) 170 -> 179.
+// Where it takes the place of the two-axis launch.  With 32 positions from 20 items an SM on, all tensor-heads together: layers, us,
+// with that launch / with this one, long runs: four heads of 32 x 64 x 32 tokens (20) 513 / 512, of 32 x 64 x 64 (41) 1050 / 1033, six
+// (62) 1529 / 1498; of 32 x 32 x 16 (5) 170 / 179.  In bursts of some ms after a pause, at full clock, the line lies higher: four of
+// 32 x 64 x 64 938 / 955, six 1949 / 1962 (all bands), twelve (124) 2735 / 2720.
 bool ffk_dct_fold_supported(const ff_plan* p) {
   const FFDims& dm = p->dm;
   const int n2 = fold_length(dm, p->dct2_axis2);

@@ -43,8 +43,8 @@
 // warps make the parts instead of four (not beside the band split, whose epilogue needs the registers).  The first pass waited for
 // its one staging area: it has two, and a stage less.  Six heads of that grid, the passes alone, us: w 176 -> 172 (6.1 TB/s),
 // h 296 -> 245 (5.7), t with the band split 271 -> 264 (4.0), inverse t 96 -> 94, h 107 -> 89, w 107 -> 96; layers (16 heads 3640 ->
-// 3474, eight of 7 x 90 x 127 tokens 1970 -> 1873).  With 64 channels none of it gained (20 x 30 x 52 tokens, eight heads, 484 -> 490):
-// they keep four stages of whole tiles.  With few tiles a launch whose code no SM has run yet costs more than eight warps gain: the
+// 3474, eight of 7 x 90 x 127 tokens 1970 -> 1873).  With 64 channels the smaller stages lost (20 x 30 x 52 tokens, eight heads, 481 ->
+// 501, 16 x 45 x 80, four, 487 -> 502; and two staging areas, 504 and 508): they keep four stages of whole tiles.  With few tiles a launch whose code no SM has run yet costs more than eight warps gain: the
 // middle pass and the band split then share theirs, four warps in both (rule: FEW_TILES).
 //
 // Order of the tiles.  A pass that reads what the previous launch wrote walks its tiles from the last to the
